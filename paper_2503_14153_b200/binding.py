@@ -362,7 +362,7 @@ class SpecDecoder:
         mt = 16 if m <= 16 else (32 if m <= 32 else (64 if m <= 64 else 128))
         if self.query(Q_CLUSTER_GATE_UP):
             return f"gemm_cluster<{mt},swiglu>"
-        return "gemm_wide" if m > 128 and self.query(Q_WIDE_GEMM) else f"gemm_stream<{mt}>"
+        return "gemm_pair<swiglu>" if m > 128 and self.query(Q_WIDE_GEMM) else f"gemm_stream<{mt}>"
 
     def query(self, what: int) -> int:
         return int(self.lib.spec_query(self._ctx, what))

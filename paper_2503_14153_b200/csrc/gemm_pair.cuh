@@ -1,0 +1,453 @@
+// bf16 linear for passes of many rows (batched verification, prompt processing), where the projections are
+// compute-bound: y = x W^T on the 5th-generation tensor cores, two SMs per output tile, with the element-wise step
+// that follows the projection applied in the epilogue.
+//
+// Operands are swapped as in gemm_stream (weight rows are the MMA's M). A cluster of two CTAs owns an output tile
+// of [256 weight rows] x [NT activation rows] and issues tcgen05.mma.cta_group::2 (M 256, N NT): each CTA holds
+// the accumulator of its own 128 weight rows and brings in those 128 weight rows and half of the activation rows.
+// Why pairs: a 64-wide K chunk of a 128 x 256 tile in one CTA writes 48 KB into shared memory and reads 48 KB out
+// of it in the 512 cycles its MMAs take at full rate, 192 bytes per cycle where an SM moves 128; the pair's chunk
+// is 32 KB in and 32 KB out per CTA, 128 bytes per cycle. Two accumulators of NT tensor-memory columns alternate, so
+// that the epilogue of one tile runs under the MMAs of the next. No split K. Persistent: cluster c takes tiles
+// c, c + clusters, ...; tile = weight pair * m_tiles + activation tile, so the clusters that share weights run side
+// by side and the weights cross HBM once.
+//
+// Modes:
+//  * GP_PLAIN     float32 sums to out[m][ld] (columns below n_cols only)
+//  * GP_RESIDUAL  x[m][n] += sum, in place (output and down projections)
+//  * GP_SWIGLU    act[m][n] = bf16(SiLU(gate) * up): a CTA's 128 weight rows are 64 rows of the gate and the same 64
+//                 rows of the up matrix
+//  * GP_ROPE      stacked q, k, v: rotates q and k, writes bf16 q rows and the cache rows
+// In the last two modes an output needs two weight rows of the tile, which sit in different tensor-memory lanes: the
+// threads swap halves of their activation rows through 16 KB of shared memory, 32 rows at a time.
+//
+// Measured on the 7B shape at M = 1024 (inside a step, launch to end, per layer), against a kernel with 128 x 256 tiles per
+// CTA that wrote float32 sums for separate glue kernels: gate+up 175 -> 141 us (1.31 PFLOP/s) and the 33 us SwiGLU kernel
+// gone, q/k/v 107 -> 91 us and the 23 us RoPE / store kernel gone, output 41 -> 39, down 92 -> 84 us; a step of 16
+// sequences through 8 layers 5.58 -> 4.56 ms.
+//
+// Warp roles (both CTAs): warp 0 feeds a ring of 32 KB stages (TMA, completing on the leader CTA's barrier), warp
+// 1 of the leader issues the MMAs, warps 2..9 drain: two warps per SM quarter, one for each half of the tile's
+// activation rows. Every wait is bounded; a CTA whose wait ran out still takes part in the closing cluster barrier.
+#pragma once
+#include <cuda.h>
+
+#include "common.cuh"
+#include "gemm_cluster.cuh"
+#include "gemm_stream.cuh"
+
+namespace spec {
+
+constexpr int GP_PLAIN = 0, GP_RESIDUAL = 1, GP_SWIGLU = 2, GP_ROPE = 3;
+constexpr int GP_THREADS = 320;
+
+struct PairGemmParams {
+  int M, KC;                                // activation rows, K / 64
+  int n_mats;
+  int mat_tile0[GS_MAX_MATS + 1];           // first 128-row weight tile of each stacked matrix
+  int n_tiles, w_pairs, m_tiles;            // weight tiles (all matrices), pairs of them, activation tiles of NT rows
+  int packed;                               // 1: the tensor maps view pre-tiled images, 0: row-major matrices
+  int n_cols;                               // GP_PLAIN: columns stored; GP_RESIDUAL / GP_SWIGLU: weight rows of one matrix
+  size_t ld;                                // GP_PLAIN: row pitch of out
+  float* out;                               // GP_PLAIN: sums; GP_RESIDUAL: residual stream [M][n_cols]
+  bf16* act;                                // GP_SWIGLU: [M][n_cols]
+  // GP_ROPE
+  int H, layer;
+  Rows rows;
+  const float2* cs;                         // [position][head_dim / 2] (cos, sin)
+  bf16* q;                                  // [M][H * head_dim]
+  bf16* pool;
+  KVGeom g;
+  const int* page_table;
+  int* status;
+  unsigned long long* trace;
+};
+
+template <int NT> struct PairCfg {
+  static constexpr int BK = 64;
+  static constexpr int A_BYTES = 128 * BK * 2;
+  static constexpr int B_BYTES = (NT / 2) * BK * 2;
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int STAGES = 6;
+  static constexpr int EX_COLS = 16;                              // activation rows swapped in one direction at a time
+  static constexpr int EX_BYTES = 2 * 2 * 64 * EX_COLS * 4;       // [half][direction][column][64 pairs] float32
+  static constexpr int META_BYTES = NT * 16;                      // GP_ROPE: (cache offset, position, swizzle row) of a row
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EX_BYTES + META_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
+  static constexpr int TMEM_COLS = 2 * NT;
+};
+
+// ---- cta_group::2 forms ----
+__device__ __forceinline__ void tmem_alloc2(uint32_t* smem_dst, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(ncols) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void tc_mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrives on the barrier at this offset in both CTAs once all MMAs issued so far by this thread are complete.
+__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+               ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+// 2D tiled TMA load into this CTA's shared memory that completes on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const void* tmap, int x, int y, uint32_t cluster_bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(smem_u32(smem_dst)), "l"(tmap), "r"(cluster_bar), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// Barriers of one half's four epilogue warps; group_and also tells whether `v` holds in all of them.
+__device__ __forceinline__ void group_bar(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ bool group_and(int id, bool v) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %2, 0;\n\tbar.red.and.pred q, %1, 128, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"(id), "r"((uint32_t)v) : "memory");
+  return r != 0;
+}
+
+struct PairRowMeta {
+  long long kv;      // element offset of the row's slot within its (layer, head) K|V blocks; -1: row not in use
+  int pos, prow;
+};
+
+template <int MODE, int NT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
+gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
+  using Cfg = PairCfg<NT>;
+  constexpr int STAGES = Cfg::STAGES;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  uint8_t* tiles = smem_raw + (((raw + 1023u) & ~1023u) - raw);
+  float* exch = reinterpret_cast<float*>(tiles + STAGES * Cfg::STAGE_BYTES);
+  PairRowMeta* meta = reinterpret_cast<PairRowMeta*>(tiles + STAGES * Cfg::STAGE_BYTES + Cfg::EX_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + STAGES * Cfg::STAGE_BYTES + Cfg::EX_BYTES + Cfg::META_BYTES);
+  uint64_t* full = bars;                    // leader's: both CTAs' operands of a stage have landed
+  uint64_t* empty = bars + STAGES;          // each CTA's: the stage has been read
+  uint64_t* acc_full = bars + 2 * STAGES;   // each CTA's
+  uint64_t* acc_empty = bars + 2 * STAGES + 2;   // leader's: drained by the eight warps of both CTAs
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
+
+  KTrace kt(p.trace);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank();
+  const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+  const int KC = p.KC;
+  const int total_tiles = p.w_pairs * p.m_tiles;
+  const int my_tiles = cl < total_tiles ? (total_tiles - 1 - cl) / ncl + 1 : 0;
+
+  pdl_launch_dependents();
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    mbar_init(&acc_full[0], 1); mbar_init(&acc_full[1], 1);
+    mbar_init(&acc_empty[0], 16); mbar_init(&acc_empty[1], 16);
+    mbar_fence_init();
+    for (int i = 0; i < p.n_mats; ++i) tma_prefetch_desc(&tm.a[i]);
+    tma_prefetch_desc(&tm.b);
+  }
+  if (warp == 1) tmem_alloc2(tmem_slot, Cfg::TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();                       // the peer's barriers are set up
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  // weight tile of this CTA in pair wp (a last odd tile is computed twice and stored once)
+  auto mat_of = [&](int nt) {
+    int mat = 0;
+#pragma unroll
+    for (int i = 1; i < GS_MAX_MATS; ++i)
+      if (i < p.n_mats && nt >= p.mat_tile0[i]) mat = i;
+    return mat;
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- producer: this CTA's weight rows and its half of the activation rows ----
+      struct At { int i, kc, wp, mt; };
+      auto at_tile = [&](At& a) {
+        const int tau = cl + a.i * ncl;
+        a.wp = tau / p.m_tiles; a.mt = tau - a.wp * p.m_tiles;
+      };
+      auto next = [&](At& a) { if (++a.kc == KC) { a.kc = 0; ++a.i; at_tile(a); } };
+      auto load_a = [&](uint8_t* dst, const At& a, uint32_t bar) {
+        if (MODE == GP_SWIGLU) {
+          const int row = (p.packed ? (a.wp * KC + a.kc) * 128 : a.wp * 128) + rank * 64, x = p.packed ? 0 : a.kc * Cfg::BK;
+          tma_load_2d_pair(dst, &tm.a[0], x, row, bar);
+          tma_load_2d_pair(dst + Cfg::A_BYTES / 2, &tm.a[1], x, row, bar);
+        } else {
+          const int nt = min(2 * a.wp + rank, p.n_tiles - 1), mat = mat_of(nt), t = nt - p.mat_tile0[mat];
+          tma_load_2d_pair(dst, &tm.a[mat], p.packed ? 0 : a.kc * Cfg::BK, p.packed ? (t * KC + a.kc) * 128 : t * 128, bar);
+        }
+      };
+      auto load_b = [&](uint8_t* dst, const At& a, uint32_t bar) {
+        tma_load_2d_pair(dst, &tm.b, a.kc * Cfg::BK, a.mt * NT + rank * (NT / 2), bar);
+      };
+      const int n_units = my_tiles * KC;
+      const int n_pre = n_units < STAGES ? n_units : STAGES;
+      const uint32_t full0 = dsmem_addr(smem_u32(full), 0);            // the leader's barriers
+      At a{0, 0, 0, 0};
+      at_tile(a);
+      At b = a;
+      // weights do not depend on the kernel before this one
+      for (int i = 0; i < n_pre; ++i, next(a)) {
+        if (rank == 0) mbar_expect_tx(&full[i], 2 * Cfg::STAGE_BYTES);
+        load_a(tiles + i * Cfg::STAGE_BYTES, a, full0 + 8 * i);
+      }
+      pdl_wait();
+      for (int i = 0; i < n_pre; ++i, next(b)) load_b(tiles + i * Cfg::STAGE_BYTES + Cfg::A_BYTES, b, full0 + 8 * i);
+      bool ok = true;
+      int issued = n_pre, st = 0;
+      uint32_t ph = 0;
+      for (; issued < n_units; ++issued, next(a)) {
+        if (!mbar_wait(&empty[st], ph, p.status, 40)) { ok = false; break; }
+        uint8_t* dst = tiles + st * Cfg::STAGE_BYTES;
+        if (rank == 0) mbar_expect_tx(&full[st], 2 * Cfg::STAGE_BYTES);
+        load_a(dst, a, full0 + 8 * st);
+        load_b(dst + Cfg::A_BYTES, a, full0 + 8 * st);
+        if (++st == STAGES) { st = 0; ph ^= 1; }
+      }
+      if (!ok && rank == 0) {
+        for (int i = issued > STAGES ? issued - STAGES : 0; i < issued; ++i)
+          mbar_wait(&full[i % STAGES], (i / STAGES) & 1, p.status, 43);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      // ---- MMA issuer of the pair ----
+      const uint32_t idesc = make_idesc_bf16(256, NT);
+      bool ok = true;
+      int st = 0;
+      uint32_t ph = 0;
+      for (int i = 0; i < my_tiles && ok; ++i) {
+        const int buf = i & 1;
+        if (!mbar_wait(&acc_empty[buf], ((i >> 1) & 1) ^ 1, p.status, 44)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d_addr = tmem_base + (uint32_t)(buf * NT);
+        for (int kc = 0; kc < KC; ++kc) {
+          if (!mbar_wait(&full[st], ph, p.status, 41)) { ok = false; break; }
+          if (i == 0 && kc == 0) trace_mark_min(p.trace, 2);
+          tc_fence_after();
+          const uint32_t a_addr = smem_u32(tiles + st * Cfg::STAGE_BYTES);
+          const uint64_t adesc = make_kmajor_sw128_desc(a_addr);
+          const uint64_t bdesc = make_kmajor_sw128_desc(a_addr + Cfg::A_BYTES);
+#pragma unroll
+          for (int k = 0; k < Cfg::BK / 16; ++k)
+            tc_mma_f16_pair(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kc > 0 || k > 0) ? 1u : 0u);
+          tc_commit_pair(&empty[st]);
+          if (++st == STAGES) { st = 0; ph ^= 1; }
+        }
+        if (!ok) break;
+        tc_commit_pair(&acc_full[buf]);
+      }
+      trace_mark_max(p.trace, 3);
+    }
+  } else {
+    // ---- epilogue: warp w may touch tensor-memory lanes [32 (w % 4), +32); warps 2..5 take the first half of the
+    // tile's activation rows, warps 6..9 the second ----
+    constexpr int HC = NT / 2;
+    const int q = warp & 3, hf = warp >= 6 ? 1 : 0;
+    const int wl = q * 32 + lane;                             // weight row within the CTA's 128
+    const uint32_t acc_empty0 = dsmem_addr(smem_u32(acc_empty), 0);
+    pdl_wait();
+    for (int i = 0; i < my_tiles; ++i) {
+      const int buf = i & 1;
+      const int tau = cl + i * ncl;
+      const int wp = tau / p.m_tiles, mt = tau - wp * p.m_tiles;
+      const int nt = 2 * wp + rank;
+      const int m0 = mt * NT + hf * HC;                       // this warp's first activation row
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * NT + hf * HC);
+      bool fine;
+      if (MODE == GP_PLAIN) {
+        fine = mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42);
+        if (!fine) break;
+        tc_fence_after();
+        const int col = nt * 128 + wl;
+        float* dst = p.out + col;
+        const bool on = nt < p.n_tiles && col < p.n_cols;
+#pragma unroll 2
+        for (int g = 0; g < HC / 32; ++g) {
+          uint32_t r[32];
+          tmem_ld32(taddr + g * 32, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const int m = m0 + g * 32 + j;
+            if (on && m < p.M) dst[(size_t)m * p.ld] = __uint_as_float(r[j]);
+          }
+        }
+      } else if (MODE == GP_RESIDUAL) {
+        // old values of the next 32 rows are fetched while 32 rows are finished, the first ones under the MMAs
+        const int col = nt * 128 + wl;
+        const bool on = nt < p.n_tiles && col < p.n_cols;
+        float* dst = p.out + col;
+        float xo[2][32];
+        auto fetch = [&](int g, float (&v)[32]) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const int m = m0 + g * 32 + j;
+            v[j] = (on && m < p.M) ? dst[(size_t)m * p.n_cols] : 0.f;
+          }
+        };
+        fetch(0, xo[0]);
+        fine = mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42);
+        if (!fine) break;
+        tc_fence_after();
+#pragma unroll
+        for (int g = 0; g < HC / 32; ++g) {
+          uint32_t r[32];
+          tmem_ld32(taddr + g * 32, r);
+          if (g + 1 < HC / 32) fetch(g + 1, xo[(g + 1) & 1]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const int m = m0 + g * 32 + j;
+            if (on && m < p.M) dst[(size_t)m * p.n_cols] = xo[g & 1][j] + __uint_as_float(r[j]);
+          }
+        }
+      } else {
+        // outputs that need two weight rows of the tile: row pairs (lower, upper) = (gate, up) or a rotation pair
+        const int D = p.g.head_dim;
+        const int nt_c = min(nt, p.n_tiles - 1);
+        const int mat = MODE == GP_ROPE ? mat_of(nt_c) : 0;
+        const int hp = MODE == GP_ROPE ? D >> 1 : 64;           // distance between the rows of a pair
+        const bool lower = (wl & hp) == 0;
+        const int pr = hp == 64 ? (wl & 63) : ((wl & 31) | ((wl >> 6) << 5));   // pair 0..63
+        float* ex_lo = exch + hf * (2 * 64 * Cfg::EX_COLS);      // written by the lower rows' threads
+        float* ex_up = ex_lo + 64 * Cfg::EX_COLS;
+        PairRowMeta* mrow = meta + hf * HC;
+        const int e = threadIdx.x - 64 - hf * 128;
+        if (MODE == GP_ROPE) {
+          group_bar(1 + hf);                                     // everybody is through with the previous tile's rows
+          if (e < HC) {
+            PairRowMeta v{-1, 0, 0};
+            const int m = m0 + e;
+            if (m < p.M) {
+              const int b = m / p.rows.R, ri = m - b * p.rows.R;
+              if (ri < p.rows.cnt[b]) {
+                const int slot = p.rows.slot[m];
+                const int page = p.page_table[b * p.g.pages_per_seq + slot / p.g.page_size];
+                v.prow = slot % p.g.page_size;
+                v.pos = p.rows.pos[m];
+                v.kv = (long long)page * 2 * (long long)p.g.block_elems() + (long long)v.prow * D;
+              }
+            }
+            mrow[e] = v;
+          }
+          group_bar(1 + hf);
+        }
+        fine = mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42);
+        // (the group stays together: all of its threads give up when one of them does)
+        if (!group_and(1 + hf, fine)) break;
+        tc_fence_after();
+        if (MODE == GP_SWIGLU) {
+          const int col = nt * 64 + pr;
+          const bool on = col < p.n_cols;
+#pragma unroll 1
+          for (int g = 0; g < HC / 32; ++g) {
+            uint32_t r[32];
+            tmem_ld32(taddr + g * 32, r);
+            tmem_ld_wait();
+            if (g) group_bar(1 + hf);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              if (lower) ex_lo[j * 64 + pr] = __uint_as_float(r[16 + j]);
+              else ex_up[j * 64 + pr] = __uint_as_float(r[j]);
+            }
+            group_bar(1 + hf);
+            const int mb = m0 + g * 32 + (lower ? 0 : 16);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float gt = lower ? __uint_as_float(r[j]) : ex_lo[j * 64 + pr];
+              const float up = lower ? ex_up[j * 64 + pr] : __uint_as_float(r[16 + j]);
+              if (on && mb + j < p.M) p.act[(size_t)(mb + j) * p.n_cols + col] = __float2bfloat16_rn(silu_f(gt) * up);
+            }
+          }
+          group_bar(1 + hf);
+        } else {
+          const int n_rows_mat = (mat == 0 ? p.H : p.g.n_kv_heads) * D;
+          const int row = (nt_c - p.mat_tile0[mat]) * 128 + wl;  // weight row within its matrix
+          const bool on = nt < p.n_tiles && row < n_rows_mat;
+          const int head = row / D, dim = row - head * D;
+          const int half = D >> 1;
+          const size_t lh = ((size_t)p.layer * p.g.n_kv_heads + head) * p.g.pool_pages() * 2 * p.g.block_elems();
+          if (mat == 2) {
+            bf16* dst = p.pool + lh + p.g.block_elems();
+#pragma unroll 1
+            for (int g = 0; g < HC / 32; ++g) {
+              uint32_t r[32];
+              tmem_ld32(taddr + g * 32, r);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 32; ++j) {
+                const PairRowMeta v = mrow[g * 32 + j];
+                if (on && v.kv >= 0) dst[v.kv + kv_elem<bf16>(v.prow, dim, D, p.g.page_size)] = __float2bfloat16_rn(__uint_as_float(r[j]));
+              }
+            }
+          } else {
+            const int di = dim & (half - 1);                     // the pair's place in its head
+#pragma unroll 1
+            for (int g = 0; g < HC / 32; ++g) {
+              uint32_t r[32];
+              tmem_ld32(taddr + g * 32, r);
+              const int jb = g * 32 + (lower ? 0 : 16);
+              float2 t[16];
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const PairRowMeta v = mrow[jb + j];
+                t[j] = p.cs[(size_t)v.pos * half + di];          // (position 0 for rows not in use)
+              }
+              tmem_ld_wait();
+              if (g) group_bar(1 + hf);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                if (lower) ex_lo[j * 64 + pr] = __uint_as_float(r[16 + j]);
+                else ex_up[j * 64 + pr] = __uint_as_float(r[j]);
+              }
+              group_bar(1 + hf);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const PairRowMeta v = mrow[jb + j];
+                if (!on || v.kv < 0) continue;
+                const float a = lower ? __uint_as_float(r[j]) : ex_lo[j * 64 + pr];
+                const float c = lower ? ex_up[j * 64 + pr] : __uint_as_float(r[16 + j]);
+                const bf16 lo = __float2bfloat16_rn(a * t[j].x - c * t[j].y), hi = __float2bfloat16_rn(c * t[j].x + a * t[j].y);
+                if (mat == 0) {
+                  bf16* dst = p.q + (size_t)(m0 + jb + j) * p.H * D + head * D + di;
+                  dst[0] = lo;
+                  dst[half] = hi;
+                } else {
+                  bf16* dst = p.pool + lh + v.kv;
+                  dst[kv_elem<bf16>(v.prow, di, D, p.g.page_size)] = lo;
+                  dst[kv_elem<bf16>(v.prow, di + half, D, p.g.page_size)] = hi;
+                }
+              }
+            }
+            group_bar(1 + hf);
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();                       // nobody leaves while the pair's MMAs, copies or arrivals may still reach it
+  if (warp == 1) { tc_fence_after(); tmem_dealloc2(tmem_base, Cfg::TMEM_COLS); }
+}
+
+}  // namespace spec

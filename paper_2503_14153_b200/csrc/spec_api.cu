@@ -22,7 +22,7 @@
 #include "common.cuh"
 #include "gemm_cluster.cuh"
 #include "gemm_stream.cuh"
-#include "gemm_wide.cuh"
+#include "gemm_pair.cuh"
 #include "glue_tc.cuh"
 #include "kernels_simple.cuh"
 #include "labels.cuh"
@@ -61,8 +61,9 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-// bf16 row-major [rows][cols] matrix, box = box_rows x 64 columns (128 bytes), 128-byte swizzle.
-bool make_tmap(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+// bf16 row-major [rows][cols] matrix, box = box_rows x 64 columns (128 bytes), 128-byte swizzle. With `image` the
+// matrix is a pre-tiled image seen as rows of 64 columns: its bytes are in shared-memory order already, no swizzle.
+bool make_tmap(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows, bool image = false) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {cols, rows};
@@ -70,8 +71,8 @@ bool make_tmap(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, u
   cuuint32_t box[2] = {64, box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, image ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 
@@ -228,7 +229,7 @@ struct spec_ctx {
   float2* d_rope;
   void *d_u, *d_q, *d_attn, *d_act, *d_hq, *d_hq_last, *d_r, *d_pool;
   size_t part_floats;
-  std::map<std::tuple<const void*, uint64_t, uint64_t, uint32_t>, CUtensorMap> tmaps;
+  std::map<std::tuple<const void*, uint64_t, uint64_t, uint32_t, bool>, CUtensorMap> tmaps;
   long long launches = 0;
   // optional device timeline of the last step: four stamps per launch (see KTrace)
   bool trace_on = false;
@@ -281,12 +282,12 @@ struct spec_ctx {
   std::string err = "no error";
 
   int fail(int code, const std::string& msg) { err = msg; return code; }
-  const CUtensorMap* tmap(const void* p, uint64_t rows, uint64_t cols, uint32_t box_rows) {
-    auto key = std::make_tuple(p, rows, cols, box_rows);
+  const CUtensorMap* tmap(const void* p, uint64_t rows, uint64_t cols, uint32_t box_rows, bool image = false) {
+    auto key = std::make_tuple(p, rows, cols, box_rows, image);
     auto it = tmaps.find(key);
     if (it != tmaps.end()) return &it->second;
     CUtensorMap tm;
-    if (!make_tmap(&tm, p, rows, cols, box_rows)) return nullptr;
+    if (!make_tmap(&tm, p, rows, cols, box_rows, image)) return nullptr;
     return &tmaps.emplace(key, tm).first->second;
   }
 };
@@ -480,6 +481,63 @@ int aligned_ctas(int n_tiles, int cap) {
   return cap;
 }
 
+// ---- many rows: the two-SM kernel, the step after the projection in its epilogue ----
+constexpr int GP_NT = 256;            // activation rows per tile
+constexpr int GP_MAX_CLUSTERS = SM_SLOTS / 4;   // one CTA per SM, two CTAs per cluster
+
+bool pair_gemm_ok(const spec_ctx* c, int M, int K) { return c->wide_gemm && M > 128 && K % 64 == 0; }
+
+template <int MODE>
+cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, const PairGemmParams& p) {
+  static bool attr_set_dev[kAttrDevices] = {};
+  bool& attr_set = *attr_flag(attr_set_dev);
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
+  const int grid = 2 * std::min(p.w_pairs * p.m_tiles, GP_MAX_CLUSTERS);
+  return launch_k(pdl, gemm_pair<MODE, GP_NT>, dim3(grid), dim3(GP_THREADS), (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
+}
+
+// x[M,K] * [mats]^T with the epilogue of `mode`; the caller has filled in the fields its mode uses.
+int run_gemm_pair(spec_ctx* c, int mode, const void* x, int M, int K, int n_mats, const void* const* mats, const int* rows,
+                  PairGemmParams* w, int kind) {
+  StreamTmaps tm{};
+  w->M = M; w->KC = K / 64; w->n_mats = n_mats; w->packed = c->packed;
+  const uint32_t box = mode == GP_SWIGLU ? 64 : 128;      // SwiGLU: 64 gate rows and 64 up rows make a CTA's tile
+  int t0 = 0;
+  for (int i = 0; i < n_mats; ++i) {
+    const int t = (rows[i] + 127) / 128;
+    w->mat_tile0[i] = t0;
+    t0 += t;
+    const CUtensorMap* ta = c->packed ? c->tmap(mats[i], (uint64_t)t * w->KC * 128, 64, box, true) : c->tmap(mats[i], rows[i], K, box);
+    if (!ta) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (weights)");
+    tm.a[i] = *ta;
+  }
+  for (int i = n_mats; i <= GS_MAX_MATS; ++i) w->mat_tile0[i] = t0;
+  w->n_tiles = mode == GP_SWIGLU ? w->mat_tile0[1] : t0;
+  w->w_pairs = mode == GP_SWIGLU ? w->n_tiles : (w->n_tiles + 1) / 2;
+  w->m_tiles = (M + GP_NT - 1) / GP_NT;
+  const CUtensorMap* tb = c->tmap(x, round_up(M, 16), K, GP_NT / 2);
+  if (!tb) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (activations)");
+  tm.b = *tb;
+  w->status = c->d_status; w->trace = c->next_trace(gemm_kind_name(kind));
+  cudaError_t e;
+  {
+    ProfScope ps(c, kind);
+    switch (mode) {
+      case GP_RESIDUAL: e = launch_gp<GP_RESIDUAL>(c->stream, c->pdl, tm, *w); break;
+      case GP_SWIGLU: e = launch_gp<GP_SWIGLU>(c->stream, c->pdl, tm, *w); break;
+      case GP_ROPE: e = launch_gp<GP_ROPE>(c->stream, c->pdl, tm, *w); break;
+      default: e = launch_gp<GP_PLAIN>(c->stream, c->pdl, tm, *w); break;
+    }
+    c->launches++;
+  }
+  if (e != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("gemm_pair launch: ") + cudaGetErrorString(e));
+  return SPEC_OK;
+}
+
 // ---- tensor-core linear (bf16): partial sums of x[M,K] * [mats]^T ----
 // kind: SPEC_PROFILE_* of the call site. On success *view describes the partial sums.
 int run_gemm(spec_ctx* c, const void* x, int M, int K, int n_mats, const void* const* mats, const int* rows, int kind,
@@ -487,43 +545,19 @@ int run_gemm(spec_ctx* c, const void* x, int M, int K, int n_mats, const void* c
   GemmPlan g;
   int tiles_all = 0;
   for (int i = 0; i < n_mats; ++i) tiles_all += (rows[i] + 127) / 128;
-  if (M > 128 && c->wide_gemm && K % 64 == 0 && n_mats <= GS_MAX_MATS) {
+  if (pair_gemm_ok(c, M, K)) {
     // many rows: the compute-bound kernel, whole tiles (one "slot" of finished sums)
-    WideGemmParams w{};
-    w.M = M; w.K = K; w.KC = K / 64; w.n_mats = n_mats;
-    int t0 = 0;
-    StreamTmaps tmw{};
-    for (int i = 0; i < n_mats; ++i) {
-      w.mat_tile0[i] = t0;
-      t0 += (rows[i] + 127) / 128;
-      if (c->packed) { w.packed[i] = static_cast<const uint8_t*>(mats[i]); continue; }
-      const CUtensorMap* t = c->tmap(mats[i], rows[i], K, 128);
-      if (!t) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (weights)");
-      tmw.a[i] = *t;
-    }
-    for (int i = n_mats; i <= GS_MAX_MATS; ++i) w.mat_tile0[i] = t0;
-    w.n_tiles = tiles_all; w.m_tiles = (M + GW_NT - 1) / GW_NT;
-    const long long total = (long long)w.n_tiles * w.m_tiles * w.KC;
+    PairGemmParams w{};
+    const long long total = (long long)tiles_all * ((M + GP_NT - 1) / GP_NT) * (K / 64);
     if ((size_t)M * tiles_all * 128 > c->part_floats) return c->fail(SPEC_E_NOMEM, "partial-sum scratch too small");
-    if (total > 0x3fffffff || (total + 1) * (long long)(w.n_tiles * w.m_tiles) >= 0x7fffffffLL) return c->fail(SPEC_E_BADARG, "unsupported linear shape");
-    const CUtensorMap* tb = c->tmap(x, std::max<size_t>(round_up(M, 16), GW_NT), K, GW_NT);
-    if (!tb) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (activations)");
-    tmw.b = *tb;
-    w.part = c->d_part; w.status = c->d_status; w.trace = c->next_trace(gemm_kind_name(kind));
-    const int grid = std::min(w.n_tiles * w.m_tiles, SM_SLOTS / 2);
-    {
-      ProfScope ps(c, kind);
-      static bool set_dev[kAttrDevices] = {};
-      bool& set_ = *attr_flag(set_dev);
-      if (!set_) { CUDA_OK(cudaFuncSetAttribute(gemm_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, WideCfg::SMEM_BYTES)); set_ = true; }
-      cudaError_t e = launch_k(c->pdl, gemm_wide, dim3(grid), dim3(GW_THREADS), (size_t)WideCfg::SMEM_BYTES, c->stream, tmw, w);
-      c->launches++;
-      if (e != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("gemm_wide launch: ") + cudaGetErrorString(e));
-    }
-    // the consumers see one finished slot per tile: a dealing of the units with one CTA per (weight tile, 256-row tile)
+    if (total > 0x3fffffff || (total + 1) * (long long)(tiles_all * ((M + GP_NT - 1) / GP_NT)) >= 0x7fffffffLL) return c->fail(SPEC_E_BADARG, "unsupported linear shape");
+    w.out = c->d_part; w.ld = (size_t)tiles_all * 128; w.n_cols = tiles_all * 128;
+    int r = run_gemm_pair(c, GP_PLAIN, x, M, K, n_mats, mats, rows, &w, kind);
+    if (r) return r;
+    // the consumers see one finished slot per tile: a dealing of the units with one CTA per (weight tile, activation tile)
     PartView v{};
     v.part = c->d_part; v.slot_stride = (size_t)M * tiles_all * 128; v.ld = tiles_all * 128;
-    v.seg.KC = w.KC; v.seg.m_tiles = w.m_tiles; v.seg.G = w.n_tiles * w.m_tiles; v.seg.total = (int)total;
+    v.seg.KC = K / 64; v.seg.m_tiles = w.m_tiles; v.seg.G = w.n_tiles * w.m_tiles; v.seg.total = (int)total;
     v.mt_shift = 8;
     v.single = 1;
     *view = v;
@@ -841,7 +875,12 @@ int forward_layers_tc(spec_ctx* c, int R, bool chain, const int* n_hi_pass, cons
     {
       const void* mats[3] = {c->wq[l], c->wk[l], c->wv[l]};
       int rws[3] = {HD, KD, KD};
-      if (cluster_gemm_ok(c, GC_ROPE, M, d)) {
+      if (pair_gemm_ok(c, M, d)) {
+        PairGemmParams w{};
+        w.H = H; w.layer = l; w.rows = rows; w.cs = c->d_rope; w.q = static_cast<bf16*>(c->d_q);
+        w.pool = static_cast<bf16*>(c->d_pool); w.g = c->geom; w.page_table = c->d_page_table;
+        if ((r = run_gemm_pair(c, GP_ROPE, u, M, d, 3, mats, rws, &w, SPEC_PROFILE_QKV))) return r;
+      } else if (cluster_gemm_ok(c, GC_ROPE, M, d)) {
         // the clusters rotate q and k and store q and the cache rows themselves
         if ((r = run_gemm_cluster(c, GC_ROPE, u, M, d, mats, 0, nullptr, nullptr, SPEC_PROFILE_QKV, l, &rows))) return r;
       } else {
@@ -856,7 +895,11 @@ int forward_layers_tc(spec_ctx* c, int R, bool chain, const int* n_hi_pass, cons
     {
       const void* mats[1] = {c->wo[l]};
       int rws[1] = {d};
-      if (cluster_gemm_ok(c, GC_RESIDUAL, M, HD)) {
+      if (pair_gemm_ok(c, M, HD)) {
+        PairGemmParams w{};
+        w.out = c->d_x; w.n_cols = d;
+        if ((r = run_gemm_pair(c, GP_RESIDUAL, c->d_attn, M, HD, 1, mats, rws, &w, SPEC_PROFILE_WO))) return r;
+      } else if (cluster_gemm_ok(c, GC_RESIDUAL, M, HD)) {
         // the cluster adds its split-K sums and the residual stream itself: nothing left for the norm kernel to add
         if ((r = run_gemm_cluster(c, GC_RESIDUAL, c->d_attn, M, HD, mats, d, c->d_x, nullptr, SPEC_PROFILE_WO))) return r;
         ss_ready = true;
@@ -869,7 +912,11 @@ int forward_layers_tc(spec_ctx* c, int R, bool chain, const int* n_hi_pass, cons
     {
       const void* mats[2] = {c->wg[l], c->wu[l]};
       int rws[2] = {F, F};
-      if (cluster_gemm_ok(c, GC_SWIGLU, M, d)) {
+      if (pair_gemm_ok(c, M, d)) {
+        PairGemmParams w{};
+        w.act = act; w.n_cols = F;
+        if ((r = run_gemm_pair(c, GP_SWIGLU, u, M, d, 2, mats, rws, &w, SPEC_PROFILE_GATE_UP))) return r;
+      } else if (cluster_gemm_ok(c, GC_SWIGLU, M, d)) {
         if ((r = run_gemm_cluster(c, GC_SWIGLU, u, M, d, mats, F, nullptr, act, SPEC_PROFILE_GATE_UP))) return r;
       } else {
         PartView vg{};
@@ -883,7 +930,11 @@ int forward_layers_tc(spec_ctx* c, int R, bool chain, const int* n_hi_pass, cons
       const void* mats[1] = {c->wd[l]};
       int rws[1] = {d};
       pend = PartView{};
-      if (cluster_gemm_ok(c, GC_RESIDUAL, M, F)) {
+      if (pair_gemm_ok(c, M, F)) {
+        PairGemmParams w{};
+        w.out = c->d_x; w.n_cols = d;
+        if ((r = run_gemm_pair(c, GP_RESIDUAL, act, M, F, 1, mats, rws, &w, SPEC_PROFILE_DOWN))) return r;
+      } else if (cluster_gemm_ok(c, GC_RESIDUAL, M, F)) {
         if ((r = run_gemm_cluster(c, GC_RESIDUAL, act, M, F, mats, d, c->d_x, nullptr, SPEC_PROFILE_DOWN))) return r;
         ss_ready = true;
       } else {
