@@ -109,7 +109,7 @@ attention_tc(const AttnTcArgs a, unsigned long long* tr) {
   constexpr int row0 = 0;                                        // the CTA owns all query rows of its sequence
   const int H = a.H, kvh = h / (H / a.g.n_kv_heads);
   const bool single = a.nsplit == 1;          // one split: its tiles start at 0 whatever the length
-  const int* pt = a.page_table + b * a.g.pages_per_seq;
+  const int* pt = a.page_table + a.rows.sequence(b) * a.g.pages_per_seq;
   if (threadIdx.x == 0) {
     for (int i = 0; i < ST; ++i) mbar_init(&full[i], 1);
     mbar_fence_init();
@@ -492,7 +492,7 @@ attention_rows(const AttnTcArgs a, unsigned long long* tr) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.x, b = blockIdx.z, row0 = blockIdx.y * 16;
   const int H = a.H, kvh = h / (H / a.g.n_kv_heads);
-  const int* pt = a.page_table + b * a.g.pages_per_seq;
+  const int* pt = a.page_table + a.rows.sequence(b) * a.g.pages_per_seq;
   if (threadIdx.x == 0) {
     for (int i = 0; i < W * NB; ++i) mbar_init(&full[i], 1);
     mbar_fence_init();
@@ -787,7 +787,7 @@ attention_shared(const AttnTcArgs a, unsigned long long* tr) {
   const int h = blockIdx.x, sp = blockIdx.y, b = blockIdx.z / halves, half = blockIdx.z % halves;
   const int row0 = half * (AS_RB * 16);
   const int H = a.H, kvh = h / (H / a.g.n_kv_heads);
-  const int* pt = a.page_table + b * a.g.pages_per_seq;
+  const int* pt = a.page_table + a.rows.sequence(b) * a.g.pages_per_seq;
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
   const int R = a.rows.R, cnt = a.rows.cnt[b], n = a.rows.n[b];

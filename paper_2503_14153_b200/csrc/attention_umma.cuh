@@ -113,6 +113,7 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
   const int ncl = (int)gridDim.y;                              // key splits = the cluster; split sp owns tiles sp, sp + ncl, ...
   // ---- producer's loads: two K slabs and two V slabs per tile, K one tile ahead of V (K is released by the
   // score MMAs, long before the tile's V is released by the P V MMAs) ----
+  const int seq = a.rows.sequence(b);
   const int lh = a.layer * a.g.n_kv_heads + kvh;             // slab rows of a page's pair: K dims 0..63, K 64..127, V, V
   auto load_k = [&](int t) -> bool {
     const int st = t & 1;
@@ -120,8 +121,8 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
     uint8_t* dst = kv_s + st * 65536;
     mbar_expect_tx(&k_full[st], 32768);
     const int page0 = (sp + t * ncl) * (AU_KT / 16);
-    tma_load_5d(dst, &tm_kv, 0, 0, b, page0, lh, &k_full[st]);
-    tma_load_5d(dst + 16384, &tm_kv, 0, 16, b, page0, lh, &k_full[st]);
+    tma_load_5d(dst, &tm_kv, 0, 0, seq, page0, lh, &k_full[st]);
+    tma_load_5d(dst + 16384, &tm_kv, 0, 16, seq, page0, lh, &k_full[st]);
     return true;
   };
   auto load_v = [&](int t) -> bool {
@@ -130,8 +131,8 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
     uint8_t* dst = kv_s + st * 65536 + 32768;
     mbar_expect_tx(&v_full[st], 32768);
     const int page0 = (sp + t * ncl) * (AU_KT / 16);
-    tma_load_5d(dst, &tm_kv, 0, 32, b, page0, lh, &v_full[st]);
-    tma_load_5d(dst + 16384, &tm_kv, 0, 48, b, page0, lh, &v_full[st]);
+    tma_load_5d(dst, &tm_kv, 0, 32, seq, page0, lh, &v_full[st]);
+    tma_load_5d(dst + 16384, &tm_kv, 0, 48, seq, page0, lh, &v_full[st]);
     return true;
   };
   // The producer thread sets up the barriers itself and at once asks for its first two tiles where they lie

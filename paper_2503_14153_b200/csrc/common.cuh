@@ -91,7 +91,10 @@ struct Rows {
   int R, B;
   int *tok, *pos, *slot;  // [B*R]
   int *n, *cnt;           // [B]
+  const int* seq;         // [B] the sequence whose cache a group of R rows belongs to, or nullptr: group b is sequence b
+                          // (prompt processing takes several 128-row chunks of one sequence in a pass)
   const uint32_t* anc;    // [R][4] ancestor bitsets (bit u of anc[i]: row i sees row u)
+  __device__ __forceinline__ int sequence(int b) const { return seq ? seq[b] : b; }
 };
 
 // ------------------------------------------------------------------ PTX wrappers

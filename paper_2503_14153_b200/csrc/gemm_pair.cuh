@@ -337,7 +337,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
               const int b = m / p.rows.R, ri = m - b * p.rows.R;
               if (ri < p.rows.cnt[b]) {
                 const int slot = p.rows.slot[m];
-                const int page = p.page_table[b * p.g.pages_per_seq + slot / p.g.page_size];
+                const int page = p.page_table[p.rows.sequence(b) * p.g.pages_per_seq + slot / p.g.page_size];
                 v.prow = slot % p.g.page_size;
                 v.pos = p.rows.pos[m];
                 v.kv = (long long)page * 2 * (long long)p.g.block_elems() + (long long)v.prow * D;

@@ -328,7 +328,7 @@ rope_store_tc(const PartView pv, int qp0, int kp0, int vp0, Rows rows, const flo
         *reinterpret_cast<uint2*>(dst) = lo;
         *reinterpret_cast<uint2*>(dst + half) = hi;
       } else {
-        const int page = page_table[b * g.pages_per_seq + slot / g.page_size], prow = slot % g.page_size;
+        const int page = page_table[rows.sequence(b) * g.pages_per_seq + slot / g.page_size], prow = slot % g.page_size;
         bf16* dst = pool + g.block_offset(page, layer, 0, head - H) + (size_t)prow * D;
         *reinterpret_cast<uint2*>(dst + kv_elem<bf16>(prow, e, D, g.page_size)) = lo;
         *reinterpret_cast<uint2*>(dst + kv_elem<bf16>(prow, e + half, D, g.page_size)) = hi;
@@ -336,7 +336,7 @@ rope_store_tc(const PartView pv, int qp0, int kp0, int vp0, Rows rows, const flo
     } else {
       const int iv = it - n_rot;
       const int kh = iv / (D >> 2), e = (iv % (D >> 2)) * 4;
-      const int page = page_table[b * g.pages_per_seq + slot / g.page_size], prow = slot % g.page_size;
+      const int page = page_table[rows.sequence(b) * g.pages_per_seq + slot / g.page_size], prow = slot % g.page_size;
       bf16* dst = pool + g.block_offset(page, layer, 1, kh) + (size_t)prow * D;
       *reinterpret_cast<uint2*>(dst + kv_elem<bf16>(prow, e, D, g.page_size)) = pack4_bf16(a.x, a.y, a.z, a.w);
     }

@@ -9,6 +9,23 @@
 namespace spec {
 
 // ------------------------------------------------------------------ row preparation
+// Embedding row `e` of d elements (or zeros) into the residual stream; 16-byte loads where the type allows.
+template <typename T>
+__device__ __forceinline__ void embed_row(const T* __restrict__ e, float* __restrict__ x, int d, bool on) {
+  if (sizeof(T) == 2 && d % 8 == 0) {
+    for (int c8 = threadIdx.x; c8 < (d >> 3); c8 += blockDim.x) {
+      const uint4 raw = on ? *reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(e) + c8 * 8) : make_uint4(0, 0, 0, 0);
+      const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&raw);
+      const float2 f0 = __bfloat1622float2(hp[0]), f1 = __bfloat1622float2(hp[1]), f2 = __bfloat1622float2(hp[2]), f3 = __bfloat1622float2(hp[3]);
+      float* dst = x + c8 * 8;
+      *reinterpret_cast<float4*>(dst) = make_float4(f0.x, f0.y, f1.x, f1.y);
+      *reinterpret_cast<float4*>(dst + 4) = make_float4(f2.x, f2.y, f3.x, f3.y);
+    }
+  } else {
+    for (int c = threadIdx.x; c < d; c += blockDim.x) x[c] = on ? to_f<T>(e[c]) : 0.f;
+  }
+}
+
 // Verify pass: tree node i of sequence b carries candidate rank[i] of head depth[i]
 // (head 0 = the base model's own next token) and sits at position n[b] + depth[i].
 template <typename T>
@@ -36,30 +53,17 @@ __global__ void prepare_verify_rows(Rows rows, const int* __restrict__ cand, int
     rows.slot[m] = n + i;
     if (i == 0) rows.cnt[b] = ok ? rows.R : 0;
   }
-  const T* e = embed + (size_t)t * d;
-  if (sizeof(T) == 2 && d % 8 == 0) {
-    // 16-byte loads of the embedding row, all in flight at once
-    for (int c8 = threadIdx.x; c8 < (d >> 3); c8 += blockDim.x) {
-      const uint4 raw = *reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(e) + c8 * 8);
-      const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&raw);
-      const float2 f0 = __bfloat1622float2(hp[0]), f1 = __bfloat1622float2(hp[1]), f2 = __bfloat1622float2(hp[2]), f3 = __bfloat1622float2(hp[3]);
-      float* dst = x + (size_t)m * d + c8 * 8;
-      *reinterpret_cast<float4*>(dst) = make_float4(f0.x, f0.y, f1.x, f1.y);
-      *reinterpret_cast<float4*>(dst + 4) = make_float4(f2.x, f2.y, f3.x, f3.y);
-    }
-  } else {
-    for (int c = threadIdx.x; c < d; c += blockDim.x) x[(size_t)m * d + c] = to_f<T>(e[c]);
-  }
+  embed_row<T>(embed + (size_t)t * d, x + (size_t)m * d, d, true);
 }
 
-// Prefill pass number `chunk`: row i of sequence b is prompt token chunk*R + i.
+// Prompt processing: row group v of the pass is prompt tokens [chunk_pos[v], + R) of sequence rows.seq[v].
 template <typename T>
 __global__ void prepare_prefill_rows(Rows rows, const int* __restrict__ prompt, const int* __restrict__ offsets,
-                                     int chunk, const T* __restrict__ embed, float* __restrict__ x, int d,
+                                     const int* __restrict__ chunk_pos, const T* __restrict__ embed, float* __restrict__ x, int d,
                                      int vocab, int* status) {
-  int m = blockIdx.x, b = m / rows.R, i = m % rows.R;
-  int len = offsets[b + 1] - offsets[b];
-  int p = chunk * rows.R + i;
+  const int m = blockIdx.x, v = m / rows.R, i = m % rows.R, b = rows.seq[v];
+  const int start = chunk_pos[v], len = offsets[b + 1] - offsets[b];
+  const int p = start + i;
   int t = 0;
   if (p < len) {
     t = prompt[offsets[b] + p];
@@ -70,32 +74,31 @@ __global__ void prepare_prefill_rows(Rows rows, const int* __restrict__ prompt, 
     rows.pos[m] = p;
     rows.slot[m] = p;
     if (i == 0) {
-      int c = len - chunk * rows.R;
-      rows.cnt[b] = c < 0 ? 0 : (c > rows.R ? rows.R : c);
-      rows.n[b] = chunk * rows.R < len ? chunk * rows.R : len;
+      const int c = len - start;
+      rows.cnt[v] = c < 0 ? 0 : (c > rows.R ? rows.R : c);
+      rows.n[v] = start;
     }
   }
-  const T* e = embed + (size_t)t * d;
-  for (int c = threadIdx.x; c < d; c += blockDim.x) x[(size_t)m * d + c] = (p < len) ? to_f<T>(e[c]) : 0.f;
+  embed_row<T>(embed + (size_t)t * d, x + (size_t)m * d, d, p < len);
 }
 
 // After a prefill pass: sequences whose last prompt token is in this pass keep that row's
 // final hidden state (float32 and operand type) for the first step's heads and lm_head.
 template <typename T>
-__global__ void prefill_keep_last(Rows rows, const int* __restrict__ offsets, int chunk,
+__global__ void prefill_keep_last(Rows rows, const int* __restrict__ offsets, const int* __restrict__ chunk_pos,
                                   const float* __restrict__ hid, float* __restrict__ h_last,
-                                  T* __restrict__ hq_last, int d) {
-  int b = blockIdx.x;
-  int len = offsets[b + 1] - offsets[b];
-  int last = len - 1;
-  if (last / rows.R != chunk) return;
-  int m = b * rows.R + last % rows.R;
+                                  T* __restrict__ hq_last, int* __restrict__ n_seq, int d) {
+  const int v = blockIdx.x, b = rows.seq[v];
+  const int len = offsets[b + 1] - offsets[b];
+  const int i = len - 1 - chunk_pos[v];
+  if (i < 0 || i >= rows.R) return;
+  const int m = v * rows.R + i;
   for (int c = threadIdx.x; c < d; c += blockDim.x) {
     float v = hid[(size_t)m * d + c];
     h_last[(size_t)b * d + c] = v;
     hq_last[(size_t)b * d + c] = from_f<T>(v);
   }
-  if (threadIdx.x == 0) rows.n[b] = len;
+  if (threadIdx.x == 0) n_seq[b] = len;
 }
 
 // ------------------------------------------------------------------ RMSNorm (+ residual)
@@ -205,7 +208,7 @@ __global__ void rope_store(const float* __restrict__ qkv, int nsplit, size_t spl
   int D = g.head_dim, half = D >> 1, Hkv = g.n_kv_heads;
   int nq = H * D, nk = Hkv * D, ld = nq + 2 * nk;
   int pos = rows.pos[m], slot = rows.slot[m];
-  int page = page_table[b * g.pages_per_seq + slot / g.page_size], prow = slot % g.page_size;
+  int page = page_table[rows.sequence(b) * g.pages_per_seq + slot / g.page_size], prow = slot % g.page_size;
   const float* src = qkv + (size_t)m * ld;
   // q and k pairs
   int npairs = (H + Hkv) * half;
@@ -257,7 +260,7 @@ __global__ void attention_simple(const T* __restrict__ q, T* __restrict__ out, c
   for (int e = 0; e < EPL; ++e) qv[e] = to_f<T>(q[(size_t)m * H * D + h * D + lane * EPL + e]);
   uint32_t a[4];
   for (int w = 0; w < 4; ++w) a[w] = rows.anc[i * 4 + w];
-  const int* pt = page_table + b * g.pages_per_seq;
+  const int* pt = page_table + rows.sequence(b) * g.pages_per_seq;
 
   float mx = -INFINITY;
   for (int j = 0; j < S; ++j) {

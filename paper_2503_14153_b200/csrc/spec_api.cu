@@ -33,7 +33,12 @@ namespace {
 
 thread_local std::string g_create_error = "no error";
 
-constexpr int PREFILL_ROWS = 128;   // rows per sequence in one prefill pass
+constexpr int PREFILL_ROWS = 128;   // rows of one chunk of a prompt (a chunk's causal mask is one ancestor set per row)
+// Chunks a prompt-processing pass takes at most on the tensor-core path: 18 chunks = 2304 rows = 9 activation tiles, with
+// which the tiles of all four projections of the 7B shape fill the 74 CTA pairs to 95-97% of whole waves (16 chunks: 86-93%).
+// A 2048-token prompt through 8 layers of that shape: 17.6 ms at 128 rows a pass, 7.1 ms in one; eight ragged prompts of
+// 128..1024 tokens through 4 layers: 14.2 ms in passes of one chunk a prompt (mostly padding at the end), 7.5 ms.
+constexpr int PREFILL_CHUNKS = 18;
 constexpr int TRACE_CAP = 1024;     // launches of one step the timeline can hold
 constexpr int SM_SLOTS = 296;       // 148 SMs x 2 co-resident GEMM CTAs
 constexpr int N_COPY_EVERY = 4;         // enqueue-only steps between two copies of the committed lengths to the host
@@ -222,6 +227,8 @@ struct spec_ctx {
   int *d_n, *d_cnt, *d_n_old, *d_root, *d_count, *d_path, *d_out_tok, *d_gen_cnt, *d_gen_log, *d_cand, *d_cand_ov;
   int *d_tok, *d_pos, *d_slot, *d_am, *d_edge, *d_parent, *d_depth, *d_rank, *d_page_table, *d_prompt, *d_offsets;
   int *d_status, *d_pidx, *d_pk_idx, *d_draws;
+  int chunk_cap;                       // prompt chunks the row buffers hold in one pass
+  int *d_chunk_seq, *d_chunk_pos, *d_chunk_n, *d_chunk_cnt;   // [max_batch * ceil(max_seq / 128)]: sequence and first token; [chunk_cap]
   uint32_t *d_anc_tree, *d_anc_chain;
   const void **d_mw, **d_mb;
   float *d_x, *d_hid, *d_h_last, *d_part, *d_logits, *d_pval, *d_part_o, *d_part_ml, *d_pk_val;
@@ -334,6 +341,9 @@ bool validate_config(const spec_config* c, std::string* why) {
   return true;
 }
 
+// KV splits of an attention launch over `groups` row groups: as many as fit beside each other, at most `most`.
+int attn_splits(int most, int n_heads, int groups) { return std::max(1, std::min(most, (SM_SLOTS / 2) / (n_heads * groups))); }
+
 // Lays the workspace out; with base == nullptr only measures it.
 size_t carve(spec_ctx* c, void* base) {
   const spec_config& f = c->cfg;
@@ -341,7 +351,9 @@ size_t carve(spec_ctx* c, void* base) {
   int B = f.max_batch, T = c->T, K = c->K, d = f.d_model, F = f.d_ffn, V = f.vocab;
   int HD = f.n_heads * f.head_dim;
   c->Nqkv = HD + 2 * f.n_kv_heads * f.head_dim;
-  c->Mcap = (int)round_up((size_t)B * (T > PREFILL_ROWS ? T : PREFILL_ROWS), 128);
+  const int max_chunks = B * (int)((f.max_seq + PREFILL_ROWS - 1) / PREFILL_ROWS);   // of the longest possible prompts
+  c->chunk_cap = c->tc ? std::max(B, std::min(PREFILL_CHUNKS, max_chunks)) : B;
+  c->Mcap = (int)round_up((size_t)std::max(B * std::max(T, PREFILL_ROWS), c->chunk_cap * PREFILL_ROWS), 128);
   c->cap = (int)round_up((size_t)f.max_seq + T, f.page_size);
   if (64 % f.page_size == 0) c->cap = (int)round_up(c->cap, 64);   // whole 64-key attention tiles
   c->pages_per_seq = c->cap / f.page_size;
@@ -356,7 +368,7 @@ size_t carve(spec_ctx* c, void* base) {
 
   c->d_status = b.take<int>(4);
   c->d_trace = b.take<unsigned long long>((size_t)TRACE_CAP * 4);
-  c->d_attn_arrive = b.take<unsigned int>((size_t)B * f.n_heads * 2);
+  c->d_attn_arrive = b.take<unsigned int>((size_t)c->chunk_cap * f.n_heads * 2);
   c->d_row_arrive = b.take<unsigned int>(c->Mcap);
   c->d_pval2 = b.take<float>(c->Mcap); c->d_pidx2 = b.take<int>(c->Mcap);
   c->d_draws = b.take<int>(B);
@@ -369,6 +381,8 @@ size_t carve(spec_ctx* c, void* base) {
   c->d_parent = b.take<int>(SPEC_MAX_NODES); c->d_depth = b.take<int>(SPEC_MAX_NODES); c->d_rank = b.take<int>(SPEC_MAX_NODES);
   c->d_anc_tree = b.take<uint32_t>(SPEC_MAX_NODES * 4); c->d_anc_chain = b.take<uint32_t>(PREFILL_ROWS * 4);
   c->d_page_table = b.take<int>((size_t)B * c->pages_per_seq);
+  c->d_chunk_seq = b.take<int>(max_chunks); c->d_chunk_pos = b.take<int>(max_chunks);
+  c->d_chunk_n = b.take<int>(c->chunk_cap); c->d_chunk_cnt = b.take<int>(c->chunk_cap);
   c->d_prompt = b.take<int>((size_t)B * f.max_seq); c->d_offsets = b.take<int>(B + 1);
   c->d_mw = b.take<const void*>(SPEC_MAX_HEADS); c->d_mb = b.take<const void*>(SPEC_MAX_HEADS);
   c->d_x = b.take<float>(M * d, 1024); c->d_hid = b.take<float>(M * d, 1024); c->d_h_last = b.take<float>((size_t)B * d);
@@ -399,8 +413,12 @@ size_t carve(spec_ctx* c, void* base) {
   c->d_part = b.take<float>(pf, 1024);
   c->d_logits = c->keep_logits ? b.take<float>((size_t)Mlog * V, 1024) : nullptr;
   c->d_pval = b.take<float>((size_t)c->ntile_lm * M, 1024); c->d_pidx = b.take<int>((size_t)c->ntile_lm * M, 1024);
-  c->d_part_o = c->tc ? b.take<float>((size_t)c->nsplit_attn * M * HD, 1024) : nullptr;
-  c->d_part_ml = c->tc ? b.take<float>((size_t)c->nsplit_attn * M * f.n_heads * 2) : nullptr;
+  // partial outputs of the KV splits: rows times splits, over the passes that use more than one split
+  size_t split_rows = (size_t)c->nsplit_attn * B * std::max(T, PREFILL_ROWS);
+  for (int g = 1; g <= c->chunk_cap; ++g)
+    split_rows = std::max(split_rows, (size_t)attn_splits(c->nsplit_attn, f.n_heads, g) * g * PREFILL_ROWS);
+  c->d_part_o = c->tc ? b.take<float>(split_rows * HD, 1024) : nullptr;
+  c->d_part_ml = c->tc ? b.take<float>(split_rows * f.n_heads * 2) : nullptr;
   c->d_ss_part = c->tc ? b.take<float>((size_t)128 * ((d + 127) / 128) * GC_RES_CLUSTER) : nullptr;
   c->d_pk_val = b.take<float>((size_t)c->topk_blocks * B * (K ? K : 1) * c->kmax);
   c->d_pk_idx = b.take<int>((size_t)c->topk_blocks * B * (K ? K : 1) * c->kmax);
@@ -453,6 +471,7 @@ Rows make_rows(spec_ctx* c, int R, bool chain) {
   Rows r;
   r.R = R; r.B = c->B;
   r.tok = c->d_tok; r.pos = c->d_pos; r.slot = c->d_slot; r.n = c->d_n; r.cnt = c->d_cnt;
+  r.seq = nullptr;
   r.anc = chain ? c->d_anc_chain : c->d_anc_tree;
   return r;
 }
@@ -704,32 +723,33 @@ int linear_simple(spec_ctx* c, const T* x, int ldx, const T* W, float* y, int ld
 
 // Passes with several 16-row blocks whose (sequence, head, row block) CTAs fit the SMs in one wave
 // use the kernel that needs no merge across CTAs and no length-dependent launch shape.
-bool attn_rows_mode(const spec_ctx* c, int R) {
+bool attn_rows_mode(const spec_ctx* c, int R, int groups) {
   const int nw = (R + 15) / 16;
-  return nw > 1 && c->cfg.n_heads * c->B * nw <= SM_SLOTS / 2;
+  return nw > 1 && c->cfg.n_heads * groups * nw <= SM_SLOTS / 2;
 }
 
 // Context length from which a pass of R rows goes to the long-context kernels: the option's value, but at most
 // ATTN_WAVES_KEYS for passes of more than 32 rows whose (sequence, head, 16-row block) CTAs do not fit one wave
 // (batched verification): there the tcgen05 kernel, one CTA per (sequence, head, 64 rows), already wins.
 constexpr int ATTN_WAVES_KEYS = 512;
-int attn_long_threshold(const spec_ctx* c, int R) {
+int attn_long_threshold(const spec_ctx* c, int R, int groups) {
   const bool umma = c->attn_umma && c->tm_kv_ok && c->cfg.head_dim == 128;
-  if (c->long_attn_keys > 0 && umma && R > 32 && !attn_rows_mode(c, R)) return std::min(c->long_attn_keys, ATTN_WAVES_KEYS);
+  if (c->long_attn_keys > 0 && umma && R > 32 && !attn_rows_mode(c, R, groups)) return std::min(c->long_attn_keys, ATTN_WAVES_KEYS);
   return c->long_attn_keys;
 }
 // Passes of more than 32 rows (any pass with the tcgen05 kernel) over a context that may exceed that length.
-bool attn_long_mode(const spec_ctx* c, int R, int keys_hi) {
+bool attn_long_mode(const spec_ctx* c, int R, int groups, int keys_hi) {
   const bool umma = c->attn_umma && c->tm_kv_ok && c->cfg.head_dim == 128;
-  const int thr = attn_long_threshold(c, R);
+  const int thr = attn_long_threshold(c, R, groups);
   return thr > 0 && (R > 32 || umma) && keys_hi > thr;
 }
 
 // n_hi_pass / n_lo_pass: host bounds of the cached length the pass's rows sit on, per sequence
 // (n_lo_pass may be null: nothing is fetched before the dependency wait).
-int launch_attention_tc(spec_ctx* c, const Rows& rows, int R, int l, const int* n_hi_pass, const int* n_lo_pass) {
+// len_now: the lengths as well as the host knows them (what the longest-first order goes by).
+int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pass, const int* n_lo_pass, const int* len_now) {
   const spec_config& f = c->cfg;
-  int H = f.n_heads, D = f.head_dim;
+  const int H = f.n_heads, D = f.head_dim, R = rows.R, B = rows.B;
   AttnTcArgs a{};
   a.q = static_cast<const bf16*>(c->d_q); a.part_o = c->d_part_o; a.part_ml = c->d_part_ml;
   a.pool = static_cast<const bf16*>(c->d_pool); a.g = c->geom; a.page_table = c->d_page_table; a.rows = rows;
@@ -737,25 +757,23 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int R, int l, const int* 
   a.out = static_cast<bf16*>(c->d_attn); a.arrive = c->d_attn_arrive;
   a.status = c->d_status;
   int tiles_hi = 1;
-  for (int b = 0; b < c->B; ++b) {
+  for (int b = 0; b < B; ++b) {
     tiles_hi = std::max(tiles_hi, (n_hi_pass[b] + R + 63) / 64);
     if (b < ATTN_MAX_SEQS) a.n_lo[b] = n_lo_pass ? n_lo_pass[b] : 0;
   }
   const int nw = (R + 15) / 16;
-  if (attn_long_mode(c, R, tiles_hi * 64) && c->attn_umma && c->tm_kv_ok && D == 128) {
+  if (attn_long_mode(c, R, B, tiles_hi * 64) && c->attn_umma && c->tm_kv_ok && D == 128) {
     // long contexts: scores and P V on tcgen05, a CTA per (head, 64 rows, key split)
     const int halves = (R + AU_ROWS - 1) / AU_ROWS;
-    if (c->B <= ATTN_MAX_SEQS) {
+    if (B <= ATTN_MAX_SEQS) {
       int idx[ATTN_MAX_SEQS];
-      for (int b = 0; b < c->B; ++b) idx[b] = b;
-      // (the host's current bounds, not the bounds the launch is planned for: those are the same for all)
-      const int* len = (int)c->n_hi.size() >= c->B ? c->n_hi.data() : n_hi_pass;
-      std::stable_sort(idx, idx + c->B, [&](int x, int y) { return len[x] > len[y]; });
-      for (int b = 0; b < c->B; ++b) a.order[b] = (unsigned char)idx[b];
+      for (int b = 0; b < B; ++b) idx[b] = b;
+      std::stable_sort(idx, idx + B, [&](int x, int y) { return len_now[x] > len_now[y]; });
+      for (int b = 0; b < B; ++b) a.order[b] = (unsigned char)idx[b];
     }
     // the key splits of a (sequence, row half, head) are one cluster: one CTA per SM, at most a wave of them
-    a.nsplit = std::max(1, std::min(std::min(c->nsplit_attn, AU_MAX_CLUSTER), (SM_SLOTS / 2) / (H * c->B * halves)));
-    dim3 grid(H, a.nsplit, c->B * halves);
+    a.nsplit = std::max(1, std::min(std::min(c->nsplit_attn, AU_MAX_CLUSTER), (SM_SLOTS / 2) / (H * B * halves)));
+    dim3 grid(H, a.nsplit, B * halves);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     static bool set_dev[kAttrDevices] = {};
     bool& set_ = *attr_flag(set_dev);
@@ -780,12 +798,12 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int R, int l, const int* 
     if (e_ != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("attention_umma: ") + cudaGetErrorString(e_));
     return SPEC_OK;
   }
-  if (attn_long_mode(c, R, tiles_hi * 64) && R > 32) {
+  if (attn_long_mode(c, R, B, tiles_hi * 64) && R > 32) {
     // long contexts, more than 32 rows: K/V tiles shared by the row blocks of a CTA, keys split across CTAs
     const int halves = (R + AS_RB * 16 - 1) / (AS_RB * 16);
-    a.nsplit = std::max(1, std::min(c->nsplit_attn, (SM_SLOTS / 2) / (H * c->B * halves)));
+    a.nsplit = std::max(1, std::min(c->nsplit_attn, (SM_SLOTS / 2) / (H * B * halves)));
     a.stages = AS_NB; a.split_tiles = AS_SPLIT_SUB;
-    dim3 grid(H, a.nsplit, c->B * halves);
+    dim3 grid(H, a.nsplit, B * halves);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     static bool set_dev[2][kAttrDevices] = {};
     bool& set_ = *attr_flag(set_dev[D == 128 ? 0 : 1]);
@@ -798,10 +816,10 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int R, int l, const int* 
     }
     return SPEC_OK;
   }
-  if (attn_rows_mode(c, R)) {
+  if (attn_rows_mode(c, R, B)) {
     // few sequences: a CTA per (head, 16 query rows) walks the whole context, whatever its length
     a.nsplit = 1; a.stages = 2; a.split_tiles = 1;
-    dim3 grid(H, nw, c->B);
+    dim3 grid(H, nw, B);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     if (D == 128) {
       static bool set_dev[kAttrDevices] = {};
@@ -819,11 +837,11 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int R, int l, const int* 
   // more sequences: one CTA per (sequence, head) and KV split, all query rows. Short contexts (host
   // bound of at most ATTN_SINGLE_TILES tiles) get one split and no merge step; longer ones as many
   // split CTAs as fit beside each other, of which the kernel uses min(that, tiles / split_tiles)
-  const int slots1 = std::max(1, std::min(c->nsplit_attn, (SM_SLOTS / 2) / (H * c->B)));
+  const int slots1 = attn_splits(c->nsplit_attn, H, B);
   a.nsplit = tiles_hi <= ATTN_SINGLE_TILES ? 1 : slots1;
   a.split_tiles = ATTN_SPLIT_TILES;
   a.stages = 4;
-  dim3 grid(H, a.nsplit, c->B);
+  dim3 grid(H, a.nsplit, B);
 #define ATTN_CASE(HDV, NWV, KGV)                                                                         \
   {                                                                                                    \
     size_t sm = attention_tc_smem(HDV, NWV, a.stages);                                                 \
@@ -845,13 +863,12 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int R, int l, const int* 
   return SPEC_OK;
 }
 
-// One pass of the base model over M = B*R rows whose tokens/positions/slots are prepared and
+// One pass of the base model over M = groups * R rows whose tokens/positions/slots are prepared and
 // whose embeddings are in d_x: bf16 tensor-core path. Leaves the final hidden state in d_hid
 // (float32) and d_hq (bf16).
-int forward_layers_tc(spec_ctx* c, int R, bool chain, const int* n_hi_pass, const int* n_lo_pass) {
+int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const int* n_lo_pass, const int* len_now) {
   const spec_config& f = c->cfg;
-  Rows rows = make_rows(c, R, chain);
-  const int M = c->B * R, d = f.d_model, F = f.d_ffn, H = f.n_heads, D = f.head_dim, HD = H * D, KD = f.n_kv_heads * D;
+  const int M = rows.B * rows.R, d = f.d_model, F = f.d_ffn, H = f.n_heads, D = f.head_dim, HD = H * D, KD = f.n_kv_heads * D;
   bf16* u = static_cast<bf16*>(c->d_u);
   bf16* act = static_cast<bf16*>(c->d_act);
   const int kp0 = (HD + 127) / 128 * 128, vp0 = kp0 + (KD + 127) / 128 * 128;   // padded columns of k and v in the QKV partials
@@ -890,7 +907,7 @@ int forward_layers_tc(spec_ctx* c, int R, bool chain, const int* n_hi_pass, cons
                 static_cast<bf16*>(c->d_q), static_cast<bf16*>(c->d_pool), c->geom, c->d_page_table, l, H);
       }
     }
-    if ((r = launch_attention_tc(c, rows, R, l, n_hi_pass, n_lo_pass))) return r;
+    if ((r = launch_attention_tc(c, rows, l, n_hi_pass, n_lo_pass, len_now))) return r;
     PartView vo{};
     {
       const void* mats[1] = {c->wo[l]};
@@ -950,11 +967,11 @@ int forward_layers_tc(spec_ctx* c, int R, bool chain, const int* n_hi_pass, cons
 
 // The same pass with the plain CUDA-core kernels (float32 configurations and the bf16 debug mode).
 template <typename T>
-int forward_layers(spec_ctx* c, int R, bool chain, const int* n_hi_pass, const int* n_lo_pass) {
-  if (c->tc) return forward_layers_tc(c, R, chain, n_hi_pass, n_lo_pass);
+int forward_layers(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const int* n_lo_pass, const int* len_now) {
+  if (c->tc) return forward_layers_tc(c, rows, n_hi_pass, n_lo_pass, len_now);
   const spec_config& f = c->cfg;
-  Rows rows = make_rows(c, R, chain);
-  int M = c->B * R, d = f.d_model, F = f.d_ffn, H = f.n_heads, D = f.head_dim, HD = H * D;
+  const int R = rows.R;
+  int M = rows.B * R, d = f.d_model, F = f.d_ffn, H = f.n_heads, D = f.head_dim, HD = H * D;
   T* u = static_cast<T*>(c->d_u);
   T* q = static_cast<T*>(c->d_q);
   T* attn = static_cast<T*>(c->d_attn);
@@ -971,7 +988,7 @@ int forward_layers(spec_ctx* c, int R, bool chain, const int* n_hi_pass, const i
     rope_store<T><<<M, 256, 0, c->stream>>>(c->d_part, 1, (size_t)M * c->Nqkv, rows, c->d_rope, q, pool, c->geom, c->d_page_table, l, H);
     LAUNCH_CHECK("rope_store");
     {
-      dim3 grid(H, c->B, (R + 3) / 4);
+      dim3 grid(H, rows.B, (R + 3) / 4);
       attention_simple<T><<<grid, 128, 0, c->stream>>>(q, attn, pool, c->geom, c->d_page_table, rows, l, H, 1.0f / sqrtf((float)D));
       LAUNCH_CHECK("attention_simple");
     }
@@ -1097,20 +1114,32 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   CUDA_OK(cudaMemcpyAsync(c->d_offsets, off.data(), (batch + 1) * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_OK(cudaMemsetAsync(c->d_gen_cnt, 0, batch * sizeof(int), c->stream));
   CUDA_OK(cudaMemsetAsync(c->d_draws, 0, batch * sizeof(int), c->stream));
-  CUDA_OK(cudaStreamSynchronize(c->stream));   // host staging vector goes out of scope below
-  int R = PREFILL_ROWS, M = batch * R;
-  Rows rows = make_rows(c, R, true);
-  int chunks = (maxlen + R - 1) / R;
-  for (int ch = 0; ch < chunks; ++ch) {
-    prepare_prefill_rows<T><<<M, 128, 0, c->stream>>>(rows, c->d_prompt, c->d_offsets, ch, static_cast<const T*>(c->embed), c->d_x,
-                                                    f.d_model, f.vocab, c->d_status);
+  // The prompts are cut into chunks of R tokens and the chunks of all prompts, one prompt after another, are dealt to as
+  // few passes as the row buffers allow, evenly. A chunk sees the chunks before it in the cache whether they belong to an
+  // earlier pass or to this one: a layer stores the keys and values of all its rows before its attention starts.
+  // (without the many-row projection kernel a pass takes as many chunks as there are sequences)
+  const int cap = c->tc && !c->wide_gemm ? f.max_batch : c->chunk_cap;
+  const int R = std::min(PREFILL_ROWS, (int)round_up(maxlen, 16));
+  std::vector<int> cseq, cpos;
+  for (int b = 0; b < batch; ++b)
+    for (int p = 0; p < off[b + 1] - off[b]; p += R) { cseq.push_back(b); cpos.push_back(p); }
+  const int chunks = (int)cseq.size(), passes = (chunks + cap - 1) / cap;
+  CUDA_OK(cudaMemcpyAsync(c->d_chunk_seq, cseq.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  CUDA_OK(cudaMemcpyAsync(c->d_chunk_pos, cpos.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  CUDA_OK(cudaStreamSynchronize(c->stream));   // the host staging vectors go out of scope
+  for (int pass = 0, ch = 0; pass < passes; ++pass) {
+    const int g = (chunks - ch + passes - pass - 1) / (passes - pass);    // chunks of this pass
+    Rows rows = make_rows(c, R, true);
+    rows.B = g; rows.seq = c->d_chunk_seq + ch; rows.n = c->d_chunk_n; rows.cnt = c->d_chunk_cnt;
+    prepare_prefill_rows<T><<<g * R, 128, 0, c->stream>>>(rows, c->d_prompt, c->d_offsets, c->d_chunk_pos + ch, static_cast<const T*>(c->embed),
+                                                        c->d_x, f.d_model, f.vocab, c->d_status);
     LAUNCH_CHECK("prepare_prefill_rows");
-    std::vector<int> n_pass(batch);
-    for (int b = 0; b < batch; ++b) n_pass[b] = std::min(offsets[b + 1] - offsets[b], ch * R);
-    int r = forward_layers<T>(c, R, true, n_pass.data(), nullptr);
+    int r = forward_layers<T>(c, rows, cpos.data() + ch, nullptr, cpos.data() + ch);
     if (r) return r;
-    prefill_keep_last<T><<<batch, 256, 0, c->stream>>>(rows, c->d_offsets, ch, c->d_hid, c->d_h_last, static_cast<T*>(c->d_hq_last), f.d_model);
+    prefill_keep_last<T><<<g, 256, 0, c->stream>>>(rows, c->d_offsets, c->d_chunk_pos + ch, c->d_hid, c->d_h_last, static_cast<T*>(c->d_hq_last),
+                                                   c->d_n, f.d_model);
     LAUNCH_CHECK("prefill_keep_last");
+    ch += g;
   }
   int r = lm_head_argmax<T>(c, static_cast<const T*>(c->d_hq_last), batch);
   if (r) return r;
@@ -1175,7 +1204,9 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
           (const int*)c->d_depth, (const int*)c->d_rank, c->cap, static_cast<const T*>(c->embed), c->d_x, d, f.vocab, c->d_status);
   step_event(c, 2);
   // (3) verification forward
-  int r = forward_layers<T>(c, T_, false, n_hi_plan, n_lo_plan);
+  // (the order the attention CTAs are handed out in goes by the host's current bounds, not by the bounds the launch is
+  // planned for: those are the same for all sequences)
+  int r = forward_layers<T>(c, rows, n_hi_plan, n_lo_plan, c->n_hi.data());
   if (r) return r;
   r = lm_head_argmax<T>(c, static_cast<const T*>(c->d_hq), M);
   if (r) return r;
@@ -1231,9 +1262,9 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     // below it the CTA-per-16-rows kernel serves every length up to the threshold, and the split kernel is planned
     // for at most ATTN_SINGLE_TILES tiles or for any length
     int bound;
-    if (attn_long_mode(c, T_, c->n_hi[b] + T_)) bound = c->cap;
-    else if (attn_rows_mode(c, T_)) bound = attn_long_mode(c, T_, 1 << 30) ? std::min(attn_long_threshold(c, T_) / 64 * 64, c->cap) : c->cap;
-    else if (c->n_hi[b] + T_ > ATTN_SINGLE_TILES * 64) bound = attn_long_mode(c, T_, 1 << 30) ? std::min(std::max(attn_long_threshold(c, T_) / 64 * 64, ATTN_SINGLE_TILES * 64), c->cap) : c->cap;
+    if (attn_long_mode(c, T_, B, c->n_hi[b] + T_)) bound = c->cap;
+    else if (attn_rows_mode(c, T_, B)) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(attn_long_threshold(c, T_, B) / 64 * 64, c->cap) : c->cap;
+    else if (c->n_hi[b] + T_ > ATTN_SINGLE_TILES * 64) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(std::max(attn_long_threshold(c, T_, B) / 64 * 64, ATTN_SINGLE_TILES * 64), c->cap) : c->cap;
     else bound = std::min(ATTN_SINGLE_TILES * 64, c->cap);
     n_hi_plan[b] = bound - T_;
     n_lo_plan[b] = c->n_lo[b];
@@ -1412,7 +1443,7 @@ int spec_create(const spec_config* cfg, const spec_weights* w, const spec_tree* 
   up(c->d_mw, c->mw.data(), c->mw.size() * sizeof(void*));
   up(c->d_mb, c->mb.data(), c->mb.size() * sizeof(void*));
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), c->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_attn_arrive, 0, (size_t)cfg->max_batch * cfg->n_heads * 2 * sizeof(unsigned int), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_attn_arrive, 0, (size_t)c->chunk_cap * cfg->n_heads * 2 * sizeof(unsigned int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_row_arrive, 0, (size_t)c->Mcap * sizeof(unsigned int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_cand, 0, (size_t)cfg->max_batch * (c->K + 1) * c->kmax * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

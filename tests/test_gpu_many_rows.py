@@ -46,3 +46,31 @@ def test_many_row_projections_vs_oracle(torch, heads, kv, hd, ffn, T, batch):
     gpu.close()
     for b in oracles:
         assert reps[b].steps == 3
+
+
+@pytest.mark.parametrize("hd,lengths", [
+    (128, (2500,)),               # 20 chunks of one prompt: two passes, the second sees the first pass's chunks in the cache
+    (64, (1300,)),                # 11 chunks in one pass, the mma.sync attention
+    (128, (300, 5, 129, 700)),    # chunks of several prompts in a pass, last chunks of 44, 5, 1 and 60 rows
+    (64, (17, 33)),               # short prompts: a chunk each, no longer than the longest prompt
+])
+def test_prompts_in_chunks_vs_oracle(torch, hd, lengths):
+    """Prompt processing deals the 128-token chunks of all prompts to shared passes: the first root, the hidden state and
+    the cache rows after it, and two steps on top, against an oracle for each prompt."""
+    from oracle.decoder import OracleModel
+    from oracle.spec import OracleSpecDecoder
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from tests_lockstep import run_lockstep_batch
+    from paper_2503_14153_b200 import binding as B
+    cfg = BASE.with_(n_heads=4, n_kv_heads=2, head_dim=hd, tree_nodes=32, seed=51)
+    w = draw_weights(cfg)
+    prompts = [draw_prompt(cfg.with_(seed=70 + i), n) for i, n in enumerate(lengths)]
+    tree = build_tree(cfg.topk, 32)
+    room = max(lengths) + 40
+    gpu = SpecDecoder(cfg, upload_weights(cfg, w), tree, room, max_batch=len(lengths), flags=B.FLAG_KEEP_LOGITS)
+    model = OracleModel(cfg, w)
+    oracles = {b: OracleSpecDecoder(model, tree, room) for b in range(len(lengths))}
+    reps = run_lockstep_batch(cfg, gpu, oracles, prompts, 2, TOL_BF16, TIE_GAP)
+    gpu.close()
+    for b in oracles:
+        assert reps[b].steps == 2
