@@ -465,8 +465,7 @@ argmax_partials_tc(const PartView pv, int V, float* __restrict__ logits, float* 
   const int per = (v4 + nsl - 1) / nsl;
   const int c_lo = blockIdx.y * per, c_hi = min(v4, c_lo + per);
   float bv = -INFINITY; int bi = 0x7fffffff;
-  for (int c4 = c_lo + threadIdx.x; c4 < c_hi; c4 += blockDim.x) {
-    const float4 a = part_sum4(pv, m, c4 * 4);
+  auto take = [&](int c4, const float4& a) {
     const float z[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -476,6 +475,19 @@ argmax_partials_tc(const PartView pv, int V, float* __restrict__ logits, float* 
         if (better(z[j], n, bv, bi)) { bv = z[j]; bi = n; }
       }
     }
+  };
+  if (pv.single) {
+    // passes of many rows (finished sums, 131 MB at 1024 rows): bound by bandwidth, so a thread keeps four loads in flight
+    constexpr int U = 4;
+    for (int c0 = c_lo + threadIdx.x; c0 < c_hi; c0 += U * blockDim.x) {
+      float4 a[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) if (c0 + k * (int)blockDim.x < c_hi) a[k] = part_one4(pv, m, (c0 + k * (int)blockDim.x) * 4);
+#pragma unroll
+      for (int k = 0; k < U; ++k) if (c0 + k * (int)blockDim.x < c_hi) take(c0 + k * (int)blockDim.x, a[k]);
+    }
+  } else {
+    for (int c4 = c_lo + threadIdx.x; c4 < c_hi; c4 += blockDim.x) take(c4, part_sum4(pv, m, c4 * 4));
   }
   __shared__ float sv[8];
   __shared__ int si[8];
@@ -526,32 +538,17 @@ topk_slices_tc(const PartView pv, int V, int rows_total, int slice, int kmax, fl
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
   extern __shared__ float zs[];
   const int row = blockIdx.y, n0 = blockIdx.x * slice, n1 = min(n0 + slice, V);    // slice % 4 == 0
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int c4 = threadIdx.x; c4 * 4 < n1 - n0; c4 += blockDim.x) {
     const float4 a = part_sum4(pv, row, n0 + c4 * 4);
     zs[c4 * 4] = a.x; zs[c4 * 4 + 1] = a.y; zs[c4 * 4 + 2] = a.z; zs[c4 * 4 + 3] = a.w;
   }
   __syncthreads();
-  __shared__ float sv[8];
-  __shared__ int si[8];
-  for (int t = 0; t < kmax; ++t) {
-    float bv = -INFINITY; int bi = 0x7fffffff;
-    for (int c = threadIdx.x; c < n1 - n0; c += blockDim.x) if (better(zs[c], n0 + c, bv, bi)) { bv = zs[c]; bi = n0 + c; }
-    warp_argmax(bv, bi);
-    if (lane == 0) { sv[warp] = bv; si[warp] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < nw; ++w) if (better(sv[w], si[w], bv, bi)) { bv = sv[w]; bi = si[w]; }
-      const size_t o = ((size_t)row * gridDim.x + blockIdx.x) * kmax + t;
-      pk_val[o] = bv;
-      pk_idx[o] = bi;
-      if (bi != 0x7fffffff) zs[bi - n0] = -INFINITY;
-    }
-    __syncthreads();
-  }
+  const size_t list = ((size_t)row * gridDim.x + blockIdx.x) * kmax;
+  block_topk(zs, nullptr, n0, n1 - n0, kmax, [&](int t, float v, int i) { pk_val[list + t] = v; pk_idx[list + t] = i; });
+  __threadfence();                                           // every writer's list entries, before the arrival below
+  __syncthreads();
   __shared__ int last_s;
   if (threadIdx.x == 0) {
-    __threadfence();
     const unsigned int old = atomicAdd(arrive + row, 1u);
     last_s = old == gridDim.x - 1;
     if (last_s) arrive[row] = 0u;

@@ -319,52 +319,70 @@ __global__ void argmax_rows(const float* __restrict__ logits, int V, float* __re
 
 // ------------------------------------------------------------------ typical acceptance
 // Eq. 1: a node passes iff p_base(token | prefix ending at its parent) >
-// min(eps, delta * exp(-H(p_base))). One block per node v; it reduces its parent's logits
-// row (softmax at the given temperature, entropy in nats).
-__global__ void typical_edges(const float* __restrict__ logits, int V, Rows rows, const int* __restrict__ parent,
-                              float eps, float delta, float inv_temp, int* __restrict__ edge_ok) {
-  int m = blockIdx.x, b = m / rows.R, v = m % rows.R;
-  if (v >= rows.cnt[b]) return;
-  if (v == 0) { if (threadIdx.x == 0) edge_ok[m] = 1; return; }
-  const float* z = logits + (size_t)(b * rows.R + parent[v]) * V;
-  __shared__ float red[32];
-  __shared__ float bc[2];
-  float mx = -INFINITY;
-  for (int c = threadIdx.x; c < V; c += blockDim.x) mx = fmaxf(mx, z[c] * inv_temp);
-  mx = warp_max(mx);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    float t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : -INFINITY;
-    t = warp_max(t);
-    if (threadIdx.x == 0) bc[0] = t;
+// min(eps, delta * exp(-H(p_base))). One block per row that is some node's parent: it reduces the row's logits
+// (softmax at the given temperature, entropy in nats) and decides all the row's children. A thread fetches its
+// TYP_CACHE float4 of the row (all of it for vocabularies of up to 32768) before it uses the first and keeps them for
+// the second pass; on the 7B shape 6.8 us for 64 nodes. (One block per node and
+// two passes over memory before: this kernel and sample_root took 107 us of a step together, now 13.)
+constexpr int TYP_THREADS = 1024, TYP_CACHE = 8;
+__global__ void __launch_bounds__(TYP_THREADS)
+typical_edges(const float* __restrict__ logits, int V, Rows rows, const int* __restrict__ parent,
+              float eps, float delta, float inv_temp, int* __restrict__ edge_ok, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  __shared__ float red[32], red2[32];
+  const int m = blockIdx.x, b = m / rows.R, u = m % rows.R, tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  // the tree is fixed at set-up: its parents are read before the dependency wait (R <= 128 threads hold a node each)
+  const bool child = tid > 0 && tid < rows.R && parent[tid] == u;
+  const int any = __syncthreads_or(child);
+  pdl_wait();
+  if (tid == 0) trace_mark_min(tr, 2);
+  const int cnt = rows.cnt[b];
+  if (u == 0 && tid == 0 && cnt > 0) edge_ok[m] = 1;
+  if (!any || u >= cnt) return;
+  const float* z = logits + (size_t)m * V;
+  const bool vec = (V & 3) == 0;
+  const int v4 = vec ? V >> 2 : 0;
+  float4 keep[TYP_CACHE];
+#pragma unroll
+  for (int k = 0; k < TYP_CACHE; ++k) {
+    const int c = tid + k * TYP_THREADS;
+    keep[k] = c < v4 ? *reinterpret_cast<const float4*>(z + 4 * c) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   }
+  const int rest0 = vec ? 4 * TYP_CACHE * TYP_THREADS : 0;     // elements from here on are read twice
+  float mx = -INFINITY;
+#pragma unroll
+  for (int k = 0; k < TYP_CACHE; ++k)
+    mx = fmaxf(fmaxf(mx, fmaxf(keep[k].x * inv_temp, keep[k].y * inv_temp)), fmaxf(keep[k].z * inv_temp, keep[k].w * inv_temp));
+  for (int c = rest0 + tid; c < V; c += TYP_THREADS) mx = fmaxf(mx, z[c] * inv_temp);
+  mx = warp_max(mx);
+  if (lane == 0) red[warp] = mx;
   __syncthreads();
-  mx = bc[0];
+  mx = warp_max(red[lane]);
+  __syncthreads();
   float se = 0.f, sez = 0.f;   // sum e, sum e * (z - mx)
-  for (int c = threadIdx.x; c < V; c += blockDim.x) {
-    float t = z[c] * inv_temp - mx;
-    float e = expf(t);
+  auto add = [&](float x) {
+    const float t = x * inv_temp - mx;
+    const float e = expf(t);
     se += e;
     sez += e * t;
-  }
+  };
+#pragma unroll
+  for (int k = 0; k < TYP_CACHE; ++k)
+    if (tid + k * TYP_THREADS < v4) { add(keep[k].x); add(keep[k].y); add(keep[k].z); add(keep[k].w); }
+  for (int c = rest0 + tid; c < V; c += TYP_THREADS) add(z[c]);
   se = warp_sum(se);
   sez = warp_sum(sez);
-  __shared__ float red2[32];
+  if (lane == 0) { red[warp] = se; red2[warp] = sez; }
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5] = se; red2[threadIdx.x >> 5] = sez; }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    int nw = blockDim.x >> 5;
-    float a = threadIdx.x < nw ? red[threadIdx.x] : 0.f, c = threadIdx.x < nw ? red2[threadIdx.x] : 0.f;
-    a = warp_sum(a);
-    c = warp_sum(c);
-    if (threadIdx.x == 0) {
-      float H = logf(a) - c / a;                 // -sum p log p with p = e / a
-      float thr = fminf(eps, delta * expf(-H));
-      float p = expf(z[rows.tok[m]] * inv_temp - mx) / a;
-      edge_ok[m] = p > thr ? 1 : 0;
-    }
+  se = warp_sum(red[lane]);
+  sez = warp_sum(red2[lane]);
+  if (child && tid < cnt) {
+    const float H = logf(se) - sez / se;                        // -sum p log p with p = e / se
+    const float thr = fminf(eps, delta * expf(-H));
+    const float p = expf(z[rows.tok[b * rows.R + tid]] * inv_temp - mx) / se;
+    edge_ok[b * rows.R + tid] = p > thr ? 1 : 0;
   }
 }
 
@@ -385,74 +403,88 @@ __device__ __forceinline__ void philox4x32_10(uint32_t (&c)[4], uint32_t k0, uin
 // token that follows the accepted span is drawn from softmax(logits / temperature) of the last
 // accepted node by inverting the cumulative distribution in token order at the uniform
 // u = top 24 bits of philox(counter = (draw index, sequence, 0, 0), key = seed) * 2^-24.
-// One block per sequence; thread t owns a contiguous chunk of the vocabulary, the chunks' weights
-// are summed in double precision, a prefix over the chunks finds the chunk that holds u * total
-// and its owner scans it. prefill != 0: the row is the sequence's last prompt position (row b).
-__global__ void __launch_bounds__(256)
-sample_root(const float* __restrict__ logits, int V, int R, int K, const int* __restrict__ path,
+// A cluster of SAMPLE_CLUSTER CTAs per sequence; every thread owns a contiguous run of the vocabulary and adds its
+// weights in double precision, relative to the row's largest logit (row_max, left by the argmax). Prefix sums over the
+// threads of a CTA and over the CTAs (distributed shared memory) give the weight before each run; the one thread whose
+// run holds u * total scans it. prefill != 0: the row is the sequence's last prompt position (row b). Bound by the
+// double-precision exponentials of 32016 tokens: 4096 threads with 8 each take 6.3 us (one CTA
+// of 256 threads with 126 each, reading them twice, and 512 additions by one thread before).
+constexpr int SAMPLE_CLUSTER = 8, SAMPLE_THREADS = 512;
+__global__ void __cluster_dims__(SAMPLE_CLUSTER, 1, 1) __launch_bounds__(SAMPLE_THREADS)
+sample_root(const float* __restrict__ logits, const float* __restrict__ row_max, int V, int R, int K, const int* __restrict__ path,
             const int* __restrict__ count, float temperature, uint32_t seed_lo, uint32_t seed_hi,
-            int* __restrict__ draws, int* __restrict__ root_tok, int prefill) {
-  const int b = blockIdx.x;
+            int* __restrict__ draws, int* __restrict__ root_tok, int prefill, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  __shared__ double wsum[SAMPLE_THREADS / 32];
+  __shared__ double total_s;                 // weight of this CTA's tokens, read by the whole cluster
+  __shared__ int pick_s;                     // rank 0: the drawn token, the last one until a run claims it
+  const int b = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int row = b;
+  bool on = true;
   if (!prefill) {
     const int len = count[b];
-    if (len < 1) return;
-    row = b * R + path[b * (K + 1) + len - 1];
+    on = len >= 1;                           // the same for every CTA of the cluster
+    if (on) row = b * R + path[b * (K + 1) + len - 1];
   }
   const float* z = logits + (size_t)row * V;
   const double inv_t = 1.0 / (double)temperature;
-  __shared__ double red[256];
-  __shared__ double mx_s;
-  __shared__ int chunk_s;
-  __shared__ double target_s, before_s;
-  const int per = (V + blockDim.x - 1) / blockDim.x;
-  const int c0 = threadIdx.x * per, c1 = min(V, c0 + per);
-  double mx = -INFINITY;
-  for (int c = c0; c < c1; ++c) mx = fmax(mx, (double)z[c] * inv_t);
-  red[threadIdx.x] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = -INFINITY;
-    for (int t = 0; t < (int)blockDim.x; ++t) m = fmax(m, red[t]);
-    mx_s = m;
-  }
-  __syncthreads();
-  mx = mx_s;
+  const double mx = (double)row_max[row] * inv_t;
+  const int runs = SAMPLE_CLUSTER * SAMPLE_THREADS, per = (V + runs - 1) / runs;
+  const int run = rank * SAMPLE_THREADS + tid;
+  const int c0 = min(V, run * per), c1 = min(V, c0 + per);
   double sum = 0.0;
-  for (int c = c0; c < c1; ++c) sum += exp((double)z[c] * inv_t - mx);
-  __syncthreads();
-  red[threadIdx.x] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t ctr[4] = {(uint32_t)draws[b], (uint32_t)b, 0u, 0u};
-    philox4x32_10(ctr, seed_lo, seed_hi);
-    const double u = (double)(ctr[0] >> 8) * (1.0 / 16777216.0);
-    double total = 0.0;
-    for (int t = 0; t < (int)blockDim.x; ++t) total += red[t];
-    const double target = u * total;
-    // total was added in this order, so the last non-empty chunk always exceeds the target (u < 1)
-    double acc = 0.0;
-    int chunk = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      chunk = t;
-      if (acc + red[t] > target) break;
-      acc += red[t];
-    }
-    chunk_s = chunk; target_s = target; before_s = acc;
-    draws[b] += 1;
+  if (on) for (int c = c0; c < c1; ++c) sum += exp((double)z[c] * inv_t - mx);
+  double incl = sum;                         // inclusive prefix over the warp, then over the CTA
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
   }
+  if (lane == 31) wsum[warp] = incl;
   __syncthreads();
-  if ((int)threadIdx.x == chunk_s) {
-    // (the scan adds the chunk's weights one by one onto the prefix; should rounding keep it from
-    // passing the target, the chunk's last token is the answer)
-    double acc = before_s;
+  double before = incl - sum, cta = 0.0;
+#pragma unroll
+  for (int w = 0; w < SAMPLE_THREADS / 32; ++w) {
+    if (w < warp) before += wsum[w];
+    cta += wsum[w];
+  }
+  if (tid == 0) { total_s = cta; if (rank == 0) pick_s = V - 1; }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  double total = 0.0;
+#pragma unroll
+  for (int r = 0; r < SAMPLE_CLUSTER; ++r) {
+    uint32_t remote;
+    double v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&total_s)), "r"(r));
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(remote) : "memory");
+    if (r < rank) before += v;
+    total += v;
+  }
+  uint32_t ctr[4] = {(uint32_t)draws[b], (uint32_t)b, 0u, 0u};
+  philox4x32_10(ctr, seed_lo, seed_hi);
+  const double u = (double)(ctr[0] >> 8) * (1.0 / 16777216.0);
+  const double target = u * total;
+  // The first run whose end passes the target holds the token: of every warp the lowest such run is scanned and the
+  // lowest token wins (should rounding keep all runs below the target, the last token is the answer).
+  const unsigned past = __ballot_sync(0xffffffffu, on && c0 < c1 && before + sum > target);
+  if (past && lane == __ffs(past) - 1) {
+    double acc = before;
     int pick = c1 - 1;
     for (int c = c0; c < c1; ++c) {
       acc += exp((double)z[c] * inv_t - mx);
-      if (acc > target_s) { pick = c; break; }
+      if (acc > target) { pick = c; break; }
     }
-    root_tok[b] = pick;
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&pick_s)), "r"(0));
+    asm volatile("red.relaxed.cluster.shared::cluster.min.s32 [%0], %1;" ::"r"(remote), "r"(pick) : "memory");
   }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (on && rank == 0 && tid == 0) { root_tok[b] = pick_s; draws[b] += 1; }
 }
 
 // ------------------------------------------------------------------ bounded-wait self test
@@ -743,20 +775,94 @@ __global__ void medusa_lmhead_topk(const T* __restrict__ r, const T* __restrict_
   }
 }
 
+// Top-k of `n` pairs (v[c], ix[c]) (ix == nullptr: index base + c) in shared memory by a CTA of 256 threads, ordered (value
+// desc, index asc): the first kmax <= 16 go to emit(rank, value, index), absent ones as (-inf, 0x7fffffff). NaN never
+// wins. `v` and `ix` are scratch afterwards. Called by all threads.
+// Selection instead of kmax rounds of a block-wide argmax (two barriers each): the kmax-th largest of the maxima of 64
+// groups of four threads is a lower bound of the kmax-th largest value, only a few times kmax values reach it, and those
+// are ranked against each other. Where more than TOPK_CAP reach it (many equal values), the rounds do the work. For the four
+// heads of a batch-1 7B step this and fewer, wider slices took the kernel from 26 to 10 us, for 64 rows from 183 to 32 us.
+constexpr int TOPK_CAP = 256;
+template <typename Emit>
+__device__ __forceinline__ void block_topk(float* v, int* ix, int base, int n, int kmax, Emit emit) {
+  __shared__ float gv[64], cv[TOPK_CAP];
+  __shared__ int gi[64], ci[TOPK_CAP];
+  __shared__ float tau_v;
+  __shared__ int tau_i, count;
+  const int tid = threadIdx.x;
+  constexpr int NONE = 0x7fffffff;
+  float bv = -INFINITY; int bi = NONE;
+  for (int c = tid; c < n; c += 256) {
+    const float x = v[c]; const int i = ix ? ix[c] : base + c;
+    if (better(x, i, bv, bi)) { bv = x; bi = i; }
+  }
+#pragma unroll
+  for (int o = 1; o <= 2; o <<= 1) {
+    const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (better(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+  }
+  if ((tid & 3) == 0) { gv[tid >> 2] = bv; gi[tid >> 2] = bi; }
+  if (tid == 0) { tau_v = -INFINITY; tau_i = NONE - 1; count = 0; }   // fewer than kmax groups hold a value: all values pass
+  __syncthreads();
+  if (tid < 64 && gi[tid] != NONE) {
+    const float x = gv[tid]; const int i = gi[tid];
+    int rank = 0;
+#pragma unroll 16
+    for (int j = 0; j < 64; ++j) rank += better(gv[j], gi[j], x, i) ? 1 : 0;
+    if (rank == kmax - 1) { tau_v = x; tau_i = i; }
+  }
+  __syncthreads();
+  const float tv = tau_v; const int ti = tau_i;
+  for (int c = tid; c < n; c += 256) {
+    const float x = v[c]; const int i = ix ? ix[c] : base + c;
+    if (x >= tv && i != NONE && !better(tv, ti, x, i)) {
+      const int at = atomicAdd(&count, 1);
+      if (at < TOPK_CAP) { cv[at] = x; ci[at] = i; }
+    }
+  }
+  __syncthreads();
+  const int nc = count;
+  if (nc <= TOPK_CAP) {
+    if (tid < nc) {
+      const float x = cv[tid]; const int i = ci[tid];
+      int rank = 0;
+      for (int j = 0; j < nc; ++j) rank += better(cv[j], ci[j], x, i) ? 1 : 0;
+      if (rank < kmax) emit(rank, x, i);
+    }
+    if (tid >= nc && tid < kmax) emit(tid, -INFINITY, NONE);
+    return;
+  }
+  // many equal values: kmax rounds of a block-wide argmax, the owner of the winner taking it out (a value taken out is NaN)
+  const int warp = tid >> 5;
+  for (int t = 0; t < kmax; ++t) {
+    bv = -INFINITY; bi = NONE;
+    int bc = -1;
+    for (int c = tid; c < n; c += 256) {
+      const float x = v[c]; const int i = ix ? ix[c] : base + c;
+      if (better(x, i, bv, bi)) { bv = x; bi = i; bc = c; }
+    }
+    const float mv = bv; const int mi = bi;
+    warp_argmax(bv, bi);
+    if ((tid & 31) == 0) { cv[warp] = bv; ci[warp] = bi; }
+    __syncthreads();
+    bv = cv[0]; bi = ci[0];
+    for (int w = 1; w < 8; ++w) if (better(cv[w], ci[w], bv, bi)) { bv = cv[w]; bi = ci[w]; }
+    if (bc >= 0 && mi == bi && mv == bv) v[bc] = __int_as_float(0x7fc00000);
+    if (tid == 0) emit(t, bv, bi);
+    __syncthreads();
+  }
+}
+
 // Merges the partial lists of one (sequence, head) row into cand[b][k+1][0..kmax) and applies
-// the optional override table; the row of head 0 of each sequence also writes cand[b][0][0] = root.
-// The row's nblocks * kmax candidates sit in shared memory (ms: nblocks * kmax * 8 bytes), every
-// thread looking after each blockDim-th of them; kmax rounds of a block-wide argmax (value desc,
-// index asc), the owner of the winner taking it out. Called by all threads of a CTA of at most 8
-// warps; the lists are read around L1 (another CTA of the same launch may have written them).
+// the override table; the row of head 0 of each sequence also writes cand[b][0][0] = root.
+// The row's nblocks * kmax candidates sit in shared memory (ms: nblocks * kmax * 8 bytes). Called by all threads of a
+// CTA of 256; the lists are read around L1 (another CTA of the same launch may have written them).
 __device__ __forceinline__ void topk_merge_row(const float* pk_val, const int* pk_idx, int nblocks, int row, int K, int kmax,
                                                const int* __restrict__ root_tok, const int* __restrict__ cand_override,
                                                int* __restrict__ cand, float* ms) {
-  __shared__ float wv[8];
-  __shared__ int wi[8], wc[8];
   const int b = row / K, k = row % K;
   const int total = nblocks * kmax;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   float* v = ms;
   int* ix = reinterpret_cast<int*>(ms + total);
   for (int c = threadIdx.x; c < total; c += blockDim.x) {
@@ -764,34 +870,13 @@ __device__ __forceinline__ void topk_merge_row(const float* pk_val, const int* p
     v[c] = __ldcg(pk_val + o);
     ix[c] = __ldcg(pk_idx + o);
   }
-  // the override entries do not depend on the lists: one load per round, issued up front
-  int ovr = -1;
-  if (cand_override && threadIdx.x < kmax) ovr = cand_override[((size_t)b * K + k) * kmax + threadIdx.x];
   __syncthreads();
   int* out = cand + ((size_t)b * (K + 1) + k + 1) * kmax;
-  for (int t = 0; t < kmax; ++t) {
-    float bv = -INFINITY; int bi = 0x7fffffff, bc = -1;
-    for (int c = threadIdx.x; c < total; c += blockDim.x)
-      if (better(v[c], ix[c], bv, bi)) { bv = v[c]; bi = ix[c]; bc = c; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o), oc = __shfl_xor_sync(0xffffffffu, bc, o);
-      if (better(ov, oi, bv, bi)) { bv = ov; bi = oi; bc = oc; }
-    }
-    if (lane == 0) { wv[warp] = bv; wi[warp] = bi; wc[warp] = bc; }
-    __syncthreads();
-    bv = wv[0]; bi = wi[0]; bc = wc[0];
-    for (int w = 1; w < nw; ++w)
-      if (better(wv[w], wi[w], bv, bi)) { bv = wv[w]; bi = wi[w]; bc = wc[w]; }
-    // every thread holds the winner; its owner takes it out, thread t publishes rank t
-    if (bc >= 0 && bc % (int)blockDim.x == (int)threadIdx.x) { v[bc] = -INFINITY; ix[bc] = 0x7fffffff; }
-    if ((int)threadIdx.x == t) {
-      const int tokv = ovr >= 0 ? ovr : bi;
-      out[t] = (tokv == 0x7fffffff) ? 0 : tokv;
-    }
-    __syncthreads();
-  }
+  block_topk(v, ix, 0, total, kmax, [&](int t, float, int i) {
+    const int ovr = cand_override ? cand_override[((size_t)b * K + k) * kmax + t] : -1;
+    const int tokv = ovr >= 0 ? ovr : i;
+    out[t] = (tokv == 0x7fffffff) ? 0 : tokv;
+  });
   if (k == 0 && threadIdx.x == 0) cand[(size_t)b * (K + 1) * kmax] = root_tok[b];
 }
 

@@ -1039,10 +1039,14 @@ int heads_tc(spec_ctx* c, const int* ov) {
     if (r) return r;
   }
   // the row's last-arriving CTA merges the slices' lists: no merge kernel
-  const size_t sm_topk = std::max((size_t)c->topk_slice * sizeof(float), (size_t)c->topk_blocks * kmax * 8);
+  // about 296 CTAs whatever the number of rows, at least four a row: more slices would only lengthen the lists to merge
+  // (and at least as many as let a slice fit 40 KB)
+  const int want = std::min(c->topk_blocks, std::max(std::max(4, (f.vocab + 10239) / 10240), SM_SLOTS / rows_total));
+  const int slice = (int)round_up((f.vocab + want - 1) / want, 4), blocks = (f.vocab + slice - 1) / slice;
+  const size_t sm_topk = std::max((size_t)slice * sizeof(float), (size_t)blocks * kmax * 8);
   if (sm_topk > 48 * 1024) return c->fail(SPEC_E_BADARG, "top-k lists do not fit the merge's shared memory");
-  KLAUNCH("topk_slices_tc", topk_slices_tc, dim3(c->topk_blocks, rows_total), dim3(256), sm_topk,
-          pl, f.vocab, rows_total, c->topk_slice, kmax, c->d_pk_val, c->d_pk_idx, c->d_row_arrive, K, (const int*)c->d_root, ov, c->d_cand);
+  KLAUNCH("topk_slices_tc", topk_slices_tc, dim3(blocks, rows_total), dim3(256), sm_topk,
+          pl, f.vocab, rows_total, slice, kmax, c->d_pk_val, c->d_pk_idx, c->d_row_arrive, K, (const int*)c->d_root, ov, c->d_cand);
   return SPEC_OK;
 }
 
@@ -1146,9 +1150,8 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   AcceptArgs a = make_accept(c, 1, 1);
   KLAUNCH("accept_kernel", accept_kernel, dim3(batch), dim3(256), 0, a);
   if (f.sampling) {
-    sample_root<<<batch, 256, 0, c->stream>>>(c->d_logits, f.vocab, 1, c->K, c->d_path, c->d_count, f.temperature, f.seed_lo,
-                                              f.seed_hi, c->d_draws, c->d_root, 1);
-    LAUNCH_CHECK("sample_root");
+    KLAUNCH("sample_root", sample_root, dim3(SAMPLE_CLUSTER, batch), dim3(SAMPLE_THREADS), 0, (const float*)c->d_logits, a.pval, f.vocab, 1, c->K,
+            (const int*)c->d_path, (const int*)c->d_count, f.temperature, f.seed_lo, f.seed_hi, c->d_draws, c->d_root, 1);
   }
   r = check_status(c);
   if (r) return r;
@@ -1214,16 +1217,14 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
   // (4) acceptance
   AcceptArgs a = make_accept(c, T_, 0);
   if (f.accept_mode == 1) {
-    typical_edges<<<M, 256, 0, c->stream>>>(c->d_logits, f.vocab, rows, c->d_parent, f.typ_eps, f.typ_delta,
-                                            1.0f / (f.temperature > 0.f ? f.temperature : 1.0f), c->d_edge);
-    LAUNCH_CHECK("typical_edges");
+    KLAUNCH("typical_edges", typical_edges, dim3(M), dim3(TYP_THREADS), 0, (const float*)c->d_logits, f.vocab, rows, (const int*)c->d_parent,
+            f.typ_eps, f.typ_delta, 1.0f / (f.temperature > 0.f ? f.temperature : 1.0f), c->d_edge);
     a.edge_ok = c->d_edge;
   }
   KLAUNCH("accept_kernel", accept_kernel, dim3(B), dim3(256), 0, a);
   if (f.sampling) {
-    sample_root<<<B, 256, 0, c->stream>>>(c->d_logits, f.vocab, T_, K, c->d_path, c->d_count, f.temperature, f.seed_lo,
-                                          f.seed_hi, c->d_draws, c->d_root, 0);
-    LAUNCH_CHECK("sample_root");
+    KLAUNCH("sample_root", sample_root, dim3(SAMPLE_CLUSTER, B), dim3(SAMPLE_THREADS), 0, (const float*)c->d_logits, a.pval, f.vocab, T_, K,
+            (const int*)c->d_path, (const int*)c->d_count, f.temperature, f.seed_lo, f.seed_hi, c->d_draws, c->d_root, 0);
   }
   step_event(c, 4);
   // (5) KV compaction
