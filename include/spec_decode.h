@@ -157,7 +157,7 @@ enum { SPEC_Q_KMAX = 0, SPEC_Q_KERNEL_LAUNCHES = 1, SPEC_Q_N_NODES = 2, SPEC_Q_B
        SPEC_Q_ALGO_BYTES_PER_STEP = 4 /* weights + lm_head (twice) + heads, in KiB */,
        SPEC_Q_GRAPH_CAPTURES = 5 /* times a step was recorded into a CUDA graph */,
        SPEC_Q_CLUSTER_GATE_UP = 6 /* 1 if a step's gate+up projection runs as the cluster kernel with the SwiGLU inside */,
-       SPEC_Q_WIDE_GEMM = 7 /* 1 if passes of more than 128 rows use the 128 x 256-tile kernel */ };
+       SPEC_Q_WIDE_GEMM = 7 /* 1 if passes of more than 128 rows use the kernel that runs a tile on two SMs */ };
 int64_t spec_query(const spec_ctx *ctx, int32_t what);
 
 /* Tuning knobs of a context (defaults in brackets). SPEC_OPT_PDL [1]: launch the kernels of
@@ -183,8 +183,8 @@ int64_t spec_query(const spec_ctx *ctx, int32_t what);
  * store). A projection whose bit is clear leaves partial sums for a separate kernel (other summation
  * order, same rounding points). All three are on by default: on the 7B shape they shorten a step by 2.2%,
  * 2% and 4.4%. SPEC_OPT_WIDE_GEMM [1]: passes of more than
- * 128 rows (batched verification, batched prompt processing) run their projections as whole
- * [128 weight rows] x [256 activation rows] tiles that keep a weight tile for 256 rows at a time;
+ * 128 rows (batched verification, prompt processing) run their projections as whole
+ * [256 weight rows] x [256 activation rows] tiles on pairs of SMs, with the step that follows in the epilogue;
  * 0 = the weight-streaming kernel, which re-reads the weights for every 128 rows.
  * SPEC_OPT_LONG_ATTN_KEYS [2048]: passes whose context may exceed this many positions run a long-context
  * attention kernel, in which a CTA reads a head's K/V once for 64 query rows and the keys are split across
@@ -274,7 +274,9 @@ int spec_pack_weight(const void *w, int32_t rows, int32_t cols, void *packed, vo
  * dealt in equal contiguous runs to `ctas` persistent CTAs, runs that end inside a tile leave
  * float32 partial sums in `scratch` (DEVICE, spec_op_linear_scratch_floats() + 4 floats; the
  * last four hold the call's status word) and a second kernel adds a tile's partial sums in CTA
- * order into y. float32 runs the CUDA-core row kernel (ctas and scratch ignored).
+ * order into y. More than 128 rows of bf16 run as whole output tiles on pairs of SMs (at most `ctas` CTAs, at least
+ * two), which write y themselves; of scratch only the status word is used then. float32 runs the CUDA-core row kernel
+ * (ctas and scratch ignored).
  * M <= 2048; for bf16 K % 64 == 0, M % 16 == 0, N >= 128, 1 <= ctas <= 1024.
  * Synchronises in bf16 mode. */
 size_t spec_op_linear_scratch_floats(int32_t M, int32_t N, int32_t K, int32_t ctas);

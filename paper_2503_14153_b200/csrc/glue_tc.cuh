@@ -461,6 +461,7 @@ argmax_partials_tc(const PartView pv, int V, float* __restrict__ logits, float* 
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
   const int m = blockIdx.x, nsl = gridDim.y;
+  const bool vec = (pv.ld & 3) == 0;                           // (rows of any length come from the float32 path only)
   const int v4 = (V + 3) >> 2;
   const int per = (v4 + nsl - 1) / nsl;
   const int c_lo = blockIdx.y * per, c_hi = min(v4, c_lo + per);
@@ -476,7 +477,11 @@ argmax_partials_tc(const PartView pv, int V, float* __restrict__ logits, float* 
       }
     }
   };
-  if (pv.single) {
+  if (pv.single && !vec) {
+    const float* z = pv.part + (size_t)m * pv.ld;
+    for (int n = c_lo * 4 + threadIdx.x; n < min(V, c_hi * 4); n += blockDim.x)
+      if (better(__ldcg(z + n), n, bv, bi)) { bv = __ldcg(z + n); bi = n; }
+  } else if (pv.single) {
     // passes of many rows (finished sums, 131 MB at 1024 rows): bound by bandwidth, so a thread keeps four loads in flight
     constexpr int U = 4;
     for (int c0 = c_lo + threadIdx.x; c0 < c_hi; c0 += U * blockDim.x) {

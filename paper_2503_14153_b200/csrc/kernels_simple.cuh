@@ -4,6 +4,8 @@
 // Templated on the operand type T (float or bf16): operands are rounded to T exactly where
 // a tensor-core kernel would consume them; accumulation is float32.
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace spec {
@@ -102,19 +104,19 @@ __global__ void prefill_keep_last(Rows rows, const int* __restrict__ offsets, co
 }
 
 // ------------------------------------------------------------------ RMSNorm (+ residual)
-// x[m] += sum_s part[s][m] (s in slice order) when nsplit > 0; u[m] = T(x / rms(x) * g);
-// optionally the unrounded normed row goes to hid (final norm).
+// u[m] = T(x[m] / rms(x[m]) * g); optionally the unrounded normed row goes to hid (final norm).
 template <typename T>
-__global__ void rmsnorm_rows(float* __restrict__ x, const float* __restrict__ part, int nsplit, size_t split_stride,
-                             const float* __restrict__ gain, float eps, T* __restrict__ u,
-                             float* __restrict__ hid, int d) {
+__global__ void rmsnorm_rows(const float* __restrict__ x, const float* __restrict__ gain, float eps, T* __restrict__ u,
+                             float* __restrict__ hid, int d, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
   int m = blockIdx.x;
-  float* xr = x + (size_t)m * d;
+  const float* xr = x + (size_t)m * d;
   float ss = 0.f;
   for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    float v = xr[c];
-    for (int s = 0; s < nsplit; ++s) v += part[s * split_stride + (size_t)m * d + c];
-    if (nsplit > 0) xr[c] = v;
+    const float v = xr[c];
     ss += v * v;
   }
   __shared__ float red[32];
@@ -141,14 +143,14 @@ __global__ void rmsnorm_rows(float* __restrict__ x, const float* __restrict__ pa
 template <typename T> struct Vec16;
 template <> struct Vec16<float> {
   static constexpr int N = 4;
-  __device__ static void load(const float* p, float (&o)[8]) {
+  template <int S> __device__ static void load(const float* p, float (&o)[S]) {
     float4 v = *reinterpret_cast<const float4*>(p);
     o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
   }
 };
 template <> struct Vec16<bf16> {
   static constexpr int N = 8;
-  __device__ static void load(const bf16* p, float (&o)[8]) {
+  template <int S> __device__ static void load(const bf16* p, float (&o)[S]) {
     uint4 v = *reinterpret_cast<const uint4*>(p);
     const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
@@ -156,53 +158,148 @@ template <> struct Vec16<bf16> {
   }
 };
 
-template <typename T, int MC>
-__global__ void linear_rows(const T* __restrict__ x, int ldx, const T* __restrict__ W, float* __restrict__ y,
-                            int ldy, int M, int N, int K) {
-  constexpr int VN = Vec16<T>::N;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int n = blockIdx.x * (blockDim.x >> 5) + warp;
-  int m0 = blockIdx.y * MC;
-  if (n >= N) return;
-  float acc[MC];
-#pragma unroll
-  for (int i = 0; i < MC; ++i) acc[i] = 0.f;
-  const T* wr = W + (size_t)n * K;
-  for (int k = lane * VN; k < K; k += 32 * VN) {
-    float wv[8], xv[8];
-    Vec16<T>::load(wr + k, wv);
-#pragma unroll
-    for (int i = 0; i < MC; ++i) {
-      if (m0 + i < M) {
-        Vec16<T>::load(x + (size_t)(m0 + i) * ldx + k, xv);
-#pragma unroll
-        for (int e = 0; e < VN; ++e) acc[i] = fmaf(wv[e], xv[e], acc[i]);
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < MC; ++i) {
-    float v = warp_sum(acc[i]);
-    if (lane == 0 && m0 + i < M) y[(size_t)(m0 + i) * ldy + n] = v;
-  }
+// A warp computes LR_N outputs of LR_M rows: per step of the inner dimension it fetches LR_N pieces of weight rows and LR_M
+// of activation rows and does LR_N * LR_M products with each, and the 32 sums are reduced over the lanes by halving (31
+// shuffles; lane l ends up with sum l). Bound by latency at the widths of the float32 configuration, so the first
+// weights are fetched before the dependency wait and, where that still leaves the chip half empty, `ks` warps share a
+// group of outputs and split the inner dimension. The other warps of a CTA take `ms` groups of rows of the same outputs, which
+// then come out of L2 once: at lm_head (32016 x 256, 16 rows) the weights crossing L2 are the bound. What follows the
+// projection is done in place of a kernel of its own.
+constexpr int LR_N = 4, LR_M = 8, LR_WARPS = 4;
+constexpr int LR_PLAIN = 0, LR_SWIGLU = 1, LR_RESIDUAL = 2;
+template <typename T> struct RowLinear {
+  const T* w[3];          // stacked matrices (LR_SWIGLU: gate, up)
+  int rows[3];            // their rows
+  int group0[3];          // first group of LR_N outputs of each (LR_SWIGLU: groups of LR_N / 2 columns, one range)
+  int n_mats;
+};
+
+// Warps that share a group of outputs: as many as have a step of the inner dimension each, while there are few warps.
+template <typename T> inline int linear_rows_split(int groups, int M, int K) {
+  const long long warps = (long long)groups * ((M + LR_M - 1) / LR_M);
+  const int steps = K / (32 * Vec16<T>::N);
+  return steps >= 4 && warps * 4 <= 2400 ? 4 : (steps >= 2 && warps * 2 <= 2400 ? 2 : 1);
 }
 
-// act = T(SiLU(g) * u)
-template <typename T>
-__global__ void swiglu_rows(const float* __restrict__ g, const float* __restrict__ up, T* __restrict__ act,
-                            size_t total) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < total) act[i] = from_f<T>(silu_f(g[i]) * up[i]);
+struct RowLinearShape {
+  int ks, ms;
+  dim3 grid;
+};
+template <typename T> inline RowLinearShape linear_rows_shape(int groups, int M, int K) {
+  RowLinearShape s;
+  const int mg = (M + LR_M - 1) / LR_M;
+  s.ks = linear_rows_split<T>(groups, M, K);
+  s.ms = 1;
+  while (s.ms * 2 <= LR_WARPS / s.ks && s.ms < mg) s.ms *= 2;
+  const int per = LR_WARPS / (s.ks * s.ms);
+  s.grid = dim3((groups + per - 1) / per, (mg + s.ms - 1) / s.ms);
+  // many outputs: four CTAs per SM walk over the groups, each fetching its next weights ahead
+  if (s.ks == 1) s.grid.x = std::min(s.grid.x, std::max(1u, 4u * 148u / s.grid.y));
+  return s;
+}
+
+template <typename T, int MODE>
+__global__ void __launch_bounds__(LR_WARPS * 32, 4)
+linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y, size_t ldy, T* __restrict__ act, int M, int K, int groups, int ks, int ms,
+            unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  constexpr int VN = Vec16<T>::N;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kpart = warp % ks, mpart = (warp / ks) % ms;
+  const int per = LR_WARPS / (ks * ms), m0 = (blockIdx.y * ms + mpart) * LR_M;
+  int g = blockIdx.x * per + warp / (ks * ms);
+  // where the current group's outputs are: its matrix, first row there, first column of y
+  const T *wa, *wb;
+  int N, n0, col0;
+  auto locate = [&](int gg) {
+    if (MODE == LR_SWIGLU) { wa = w.w[0]; wb = w.w[1]; N = w.rows[0]; n0 = gg * (LR_N / 2); col0 = 0; return; }
+    const int mat = w.n_mats > 2 && gg >= w.group0[2] ? 2 : (w.n_mats > 1 && gg >= w.group0[1] ? 1 : 0);
+    wa = wb = mat == 0 ? w.w[0] : (mat == 1 ? w.w[1] : w.w[2]);
+    N = mat == 0 ? w.rows[0] : (mat == 1 ? w.rows[1] : w.rows[2]);
+    n0 = (gg - (mat == 0 ? 0 : (mat == 1 ? w.group0[1] : w.group0[2]))) * LR_N;
+    col0 = mat == 0 ? 0 : (mat == 1 ? w.rows[0] : w.rows[0] + w.rows[1]);
+  };
+  float wv[LR_N][VN], xv[LR_M][VN];
+  // (rows past the end of a matrix repeat its last row and are not stored)
+  auto load_w = [&](int k) {
+#pragma unroll
+    for (int j = 0; j < LR_N; ++j) {
+      const int n = min(MODE == LR_SWIGLU ? n0 + (j & 1) : n0 + j, N - 1);
+      Vec16<T>::load((j < 2 ? wa : wb) + (size_t)n * K + k, wv[j]);
+    }
+  };
+  const int k0 = (kpart * 32 + lane) * VN;
+  locate(g);
+  if (k0 < K) load_w(k0);
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  for (;;) {
+    float v[LR_N * LR_M];
+#pragma unroll
+    for (int i = 0; i < LR_N * LR_M; ++i) v[i] = 0.f;
+    const int n_this = n0, N_this = N, col_this = col0;
+    g += gridDim.x * per;
+    const bool more = g < groups;
+    for (int k = k0; k < K;) {
+#pragma unroll
+      for (int i = 0; i < LR_M; ++i) Vec16<T>::load(x + (size_t)min(m0 + i, M - 1) * K + k, xv[i]);
+#pragma unroll
+      for (int j = 0; j < LR_N; ++j)
+#pragma unroll
+        for (int i = 0; i < LR_M; ++i)
+#pragma unroll
+          for (int e = 0; e < VN; ++e) v[j * LR_M + i] = fmaf(wv[j][e], xv[i][e], v[j * LR_M + i]);
+      k += ks * 32 * VN;
+      if (k < K) load_w(k);
+    }
+    // the next group's first weights are on their way while this one's sums are reduced
+    if (more) { locate(g); if (k0 < K) load_w(k0); }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const bool hi = (lane & o) != 0;
+#pragma unroll
+      for (int t = 0; t < o; ++t) {
+        const float send = hi ? v[t] : v[t + o], keep = hi ? v[t + o] : v[t];
+        v[t] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+    if (ks > 1) {                                             // (one group a warp: the loop ends here)
+      __shared__ float parts[LR_WARPS][32];
+      if (kpart) parts[warp][lane] = v[0];
+      __syncthreads();
+      if (kpart) return;
+      for (int i = 1; i < ks; ++i) v[0] += parts[warp + i][lane];
+    }
+    const int j = lane / LR_M, m = m0 + lane % LR_M;
+    if (MODE == LR_SWIGLU) {
+      const float up = __shfl_xor_sync(0xffffffffu, v[0], 16);
+      const int n = n_this + (j & 1);
+      if (j < 2 && m < M && n < N_this) act[(size_t)m * N_this + n] = from_f<T>(silu_f(v[0]) * up);
+    } else {
+      const int n = n_this + j;
+      if (m < M && n < N_this) {
+        float* dst = y + (size_t)m * ldy + col_this + n;
+        if (MODE == LR_RESIDUAL) *dst += v[0];
+        else *dst = v[0];
+      }
+    }
+    if (!more || ks > 1) return;
+  }
 }
 
 // ------------------------------------------------------------------ RoPE + cache store
-// qkv: float32 [nsplit][M][(H+2Hkv)*D] partial sums. Rotate-half RoPE (element i pairs with
+// qkv: float32 [M][(H+2Hkv)*D]. Rotate-half RoPE (element i pairs with
 // i + D/2, angle pos * base^(-2i/D), table cs[pos][i] = (cos, sin)) on q and k; q -> T
 // [M][H*D]; k, v -> T into the paged cache at the row's slot.
 template <typename T>
-__global__ void rope_store(const float* __restrict__ qkv, int nsplit, size_t split_stride, Rows rows,
+__global__ void rope_store(const float* __restrict__ qkv, Rows rows,
                            const float2* __restrict__ cs, T* __restrict__ q, T* __restrict__ pool, KVGeom g,
-                           const int* __restrict__ page_table, int layer, int H) {
+                           const int* __restrict__ page_table, int layer, int H, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
   int m = blockIdx.x, b = m / rows.R, i = m % rows.R;
   if (i >= rows.cnt[b]) return;
   int D = g.head_dim, half = D >> 1, Hkv = g.n_kv_heads;
@@ -215,11 +312,7 @@ __global__ void rope_store(const float* __restrict__ qkv, int nsplit, size_t spl
   for (int p = threadIdx.x; p < npairs; p += blockDim.x) {
     int head = p / half, e = p % half;
     int col = head * D + e;
-    float a = 0.f, c = 0.f;
-    for (int s = 0; s < max(nsplit, 1); ++s) {
-      a += src[s * split_stride + col];
-      c += src[s * split_stride + col + half];
-    }
+    const float a = src[col], c = src[col + half];
     float2 t = cs[(size_t)pos * half + e];
     float r0 = a * t.x - c * t.y, r1 = c * t.x + a * t.y;
     if (head < H) {
@@ -234,87 +327,158 @@ __global__ void rope_store(const float* __restrict__ qkv, int nsplit, size_t spl
   }
   for (int p = threadIdx.x; p < nk; p += blockDim.x) {
     int kh = p / D, e = p % D;
-    float a = 0.f;
-    for (int s = 0; s < max(nsplit, 1); ++s) a += src[s * split_stride + nq + nk + p];
+    const float a = src[nq + nk + p];
     T* dst = pool + g.block_offset(page, layer, 1, kh) + (size_t)prow * D;
     dst[kv_elem<T>(prow, e, D, g.page_size)] = from_f<T>(a);
   }
 }
 
 // ------------------------------------------------------------------ plain tree attention
-// One warp per (row, head). Row i of sequence b sees every cached position < n[b] and row u
-// of the same pass iff bit u of anc[i] is set. Two passes over the keys: maximum, then
-// exp / sum / value accumulation with the probabilities rounded to T before the product.
-template <typename T>
-__global__ void attention_simple(const T* __restrict__ q, T* __restrict__ out, const T* __restrict__ pool, KVGeom g,
-                                 const int* __restrict__ page_table, Rows rows, int layer, int H, float scale) {
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int h = blockIdx.x, b = blockIdx.y;
-  int i = blockIdx.z * (blockDim.x >> 5) + warp;
-  if (i >= rows.cnt[b]) return;
-  int m = b * rows.R + i;
-  int D = g.head_dim, EPL = D >> 5;   // D in {32,64,128,256}
-  int kvh = h / (H / g.n_kv_heads);
-  int n = rows.n[b], S = n + rows.cnt[b];
-  float qv[8];
-  for (int e = 0; e < EPL; ++e) qv[e] = to_f<T>(q[(size_t)m * H * D + h * D + lane * EPL + e]);
-  uint32_t a[4];
-  for (int w = 0; w < 4; ++w) a[w] = rows.anc[i * 4 + w];
+// Row i of sequence b sees every cached position < n[b] and row u of the same pass iff bit u of anc[i] is set. A CTA takes
+// AP_ROWS query rows of one head, a warp each, and stages tiles of KT keys and values in shared memory (all of them in
+// one tile for the contexts of the float32 configuration); within a group of 32 keys a lane owns a key for the scores and
+// every 32nd dimension for the values. Two passes over the keys: maximum, then exp / sum / value accumulation with the
+// probabilities rounded to T before the product; with one tile the scores stay in registers in between. (With a warp that
+// walked the keys one by one out of L2, twice, a 16-node step of the two-layer configuration at 60 positions took 320 us in
+// all; with this, the row linear above and their fused steps 138. This kernel is 8.8 us of it per layer.)
+constexpr int AP_ROWS = 8, AP_GROUPS = 4;       // at most AP_GROUPS * 32 keys a tile
+__host__ __device__ inline int attention_plain_tile(int D) { return D <= 64 ? 128 : (D <= 128 ? 64 : 32); }
+inline size_t attention_plain_smem(int D) { return ((size_t)2 * attention_plain_tile(D) * (D + 4) + (size_t)AP_ROWS * D) * sizeof(float); }
+
+template <typename T, int EPL>
+__global__ void __launch_bounds__(AP_ROWS * 32)
+attention_plain(const T* __restrict__ q, T* __restrict__ out, const T* __restrict__ pool, KVGeom g,
+                const int* __restrict__ page_table, Rows rows, int layer, int H, float scale, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  extern __shared__ __align__(16) float sm_plain[];
+  constexpr int D = EPL * 32, P = D + 4, KT = D <= 64 ? 128 : (D <= 128 ? 64 : 32);
+  float* ks = sm_plain;
+  float* vs = ks + KT * P;
+  float* qs = vs + KT * P;
+  __shared__ long long ko[AP_GROUPS * 32];     // a key's offset in the pool, -1 past the end, and its row in its page
+  __shared__ int kr_s[AP_GROUPS * 32];
+  __shared__ __align__(16) float ps[AP_ROWS][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int h = blockIdx.x, b = blockIdx.y, i0 = blockIdx.z * AP_ROWS;
+  const int kvh = h / (H / g.n_kv_heads);
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  const int cnt = rows.cnt[b], n = rows.n[b];
+  if (i0 >= cnt) return;
+  const int S = n + cnt;
   const int* pt = page_table + rows.sequence(b) * g.pages_per_seq;
-
-  float mx = -INFINITY;
-  for (int j = 0; j < S; ++j) {
-    if (j >= n && !((a[(j - n) >> 5] >> ((j - n) & 31)) & 1u)) continue;
-    int prow = j % g.page_size;
-    const T* kr = pool + g.block_offset(pt[j / g.page_size], layer, 0, kvh) + (size_t)prow * D;
-    float s = 0.f;
-    for (int e = 0; e < EPL; ++e) s = fmaf(qv[e], to_f<T>(kr[kv_elem<T>(prow, lane * EPL + e, D, g.page_size)]), s);
-    s = warp_sum(s) * scale;
-    mx = fmaxf(mx, s);
+  const int i = i0 + warp;
+  const bool on = i < cnt;
+  const size_t m = (size_t)b * rows.R + i;
+  uint32_t a[4];
+#pragma unroll
+  for (int w = 0; w < 4; ++w) a[w] = on ? rows.anc[i * 4 + w] : 0u;
+  if (on) for (int e = lane; e < D; e += 32) qs[warp * D + e] = to_f<T>(q[m * H * D + h * D + e]);
+  // keys [k0, k0 + KT) and, where asked, their values; rows past the end (up to a whole group of 32) are zeros. The
+  // divisions by the page size are done once a key; D / 4 lanes (or the warp) then copy a row.
+  constexpr int per = D / 4, rpw = per <= 32 ? 32 / per : 1;
+  const int sub = per <= 32 ? lane / per : 0, e0 = per <= 32 ? lane - sub * per : lane;
+  auto stage = [&](int k0, bool values) {
+    const int live = min(KT, (S - k0 + 31) & ~31);
+    for (int r = threadIdx.x; r < live; r += AP_ROWS * 32) {
+      const int j = k0 + r;
+      long long o = -1;
+      if (j < S) {
+        const int pg = j / g.page_size, prow = j - pg * g.page_size;
+        o = (long long)(g.block_offset(pt[pg], layer, 0, kvh) + (size_t)prow * D);
+        kr_s[r] = prow;
+      }
+      ko[r] = o;
+    }
+    __syncthreads();
+    for (int r = warp * rpw + sub; sub < rpw && r < live; r += AP_ROWS * rpw) {
+      const long long o = ko[r];
+      const T* kr = pool + o;
+      const T* vr = kr + g.block_elems();
+      const int prow = kr_s[r];
+      for (int c = e0; c < per; c += 32) {
+        float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
+        if (o >= 0) {
+          const int e = kv_elem<T>(prow, c * 4, D, g.page_size);   // four neighbouring elements stay together
+          if (sizeof(T) == 4) {
+            kv = *reinterpret_cast<const float4*>(kr + e);
+            if (values) vv = *reinterpret_cast<const float4*>(vr + e);
+          } else {
+            kv = make_float4(to_f<T>(kr[e]), to_f<T>(kr[e + 1]), to_f<T>(kr[e + 2]), to_f<T>(kr[e + 3]));
+            if (values) vv = make_float4(to_f<T>(vr[e]), to_f<T>(vr[e + 1]), to_f<T>(vr[e + 2]), to_f<T>(vr[e + 3]));
+          }
+        }
+        *reinterpret_cast<float4*>(ks + r * P + c * 4) = kv;
+        if (values) *reinterpret_cast<float4*>(vs + r * P + c * 4) = vv;
+      }
+    }
+  };
+  auto score = [&](int k0, int gr) {
+    const int j = k0 + gr * 32 + lane;
+    const int u = j - n;                                          // node of this pass, or negative
+    const uint32_t word = u < 64 ? (u < 32 ? a[0] : a[1]) : (u < 96 ? a[2] : a[3]);
+    const bool vis = on && j < S && (u < 0 || ((word >> (u & 31)) & 1u));
+    const float4* kr = reinterpret_cast<const float4*>(ks + (gr * 32 + lane) * P);
+    const float4* qr = reinterpret_cast<const float4*>(qs + warp * D);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int e = 0; e < D / 4; ++e) {
+      const float4 kv = kr[e], qv = qr[e];
+      s.x = fmaf(qv.x, kv.x, s.x); s.y = fmaf(qv.y, kv.y, s.y); s.z = fmaf(qv.z, kv.z, s.z); s.w = fmaf(qv.w, kv.w, s.w);
+    }
+    return vis ? ((s.x + s.y) + (s.z + s.w)) * scale : -INFINITY;
+  };
+  constexpr int groups = KT / 32;
+  const int tiles = (S + KT - 1) / KT;
+  float keep[AP_GROUPS], mx = -INFINITY;
+  for (int t = 0; t < tiles; ++t) {
+    __syncthreads();
+    stage(t * KT, tiles == 1);
+    __syncthreads();
+#pragma unroll
+    for (int gr = 0; gr < AP_GROUPS; ++gr) {
+      keep[gr] = -INFINITY;
+      if (gr < groups && t * KT + gr * 32 < S) keep[gr] = score(t * KT, gr);
+      mx = fmaxf(mx, keep[gr]);
+    }
   }
-  float l = 0.f, acc[8];
+  mx = warp_max(mx);
+  float l = 0.f, acc[EPL];
+#pragma unroll
   for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-  for (int j = 0; j < S; ++j) {
-    if (j >= n && !((a[(j - n) >> 5] >> ((j - n) & 31)) & 1u)) continue;
-    int prow = j % g.page_size;
-    int page = pt[j / g.page_size];
-    const T* kr = pool + g.block_offset(page, layer, 0, kvh) + (size_t)prow * D;
-    const T* vr = pool + g.block_offset(page, layer, 1, kvh) + (size_t)prow * D;
-    float s = 0.f;
-    for (int e = 0; e < EPL; ++e) s = fmaf(qv[e], to_f<T>(kr[kv_elem<T>(prow, lane * EPL + e, D, g.page_size)]), s);
-    s = warp_sum(s) * scale;
-    float p = expf(s - mx);
-    l += p;
-    float pq = quant<T>(p);
-    for (int e = 0; e < EPL; ++e) acc[e] = fmaf(pq, to_f<T>(vr[kv_elem<T>(prow, lane * EPL + e, D, g.page_size)]), acc[e]);
+  for (int t = 0; t < tiles; ++t) {
+    if (tiles > 1) {
+      __syncthreads();
+      stage(t * KT, true);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int gr = 0; gr < AP_GROUPS; ++gr) {
+      if (gr >= groups || t * KT + gr * 32 >= S) continue;
+      const float s = tiles > 1 ? score(t * KT, gr) : keep[gr];
+      const float p = s == -INFINITY ? 0.f : expf(s - mx);       // (keys a row does not see carry no weight)
+      l += p;
+      __syncwarp();
+      ps[warp][lane] = quant<T>(p);
+      __syncwarp();
+      const float* vr = vs + gr * 32 * P + lane;
+#pragma unroll
+      for (int k4 = 0; k4 < 8; ++k4) {
+        const float4 p4 = *reinterpret_cast<const float4*>(&ps[warp][k4 * 4]);
+        const float pk[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+          for (int e = 0; e < EPL; ++e)                          // (a key without weight is left out whatever its values are)
+            acc[e] = fmaf(pk[kk], pk[kk] != 0.f ? vr[(k4 * 4 + kk) * P + e * 32] : 0.f, acc[e]);
+      }
+    }
   }
-  float inv = 1.f / l;
-  for (int e = 0; e < EPL; ++e) out[(size_t)m * H * D + h * D + lane * EPL + e] = from_f<T>(acc[e] * inv);
-}
-
-// ------------------------------------------------------------------ argmax over vocabulary
-// One block per row; lowest index wins ties. Writes one (value, index) partial per row.
-__global__ void argmax_rows(const float* __restrict__ logits, int V, float* __restrict__ pval, int* __restrict__ pidx) {
-  int m = blockIdx.x;
-  const float* z = logits + (size_t)m * V;
-  float bv = -INFINITY;
-  int bi = 0x7fffffff;
-  for (int c = threadIdx.x; c < V; c += blockDim.x) {
-    float v = z[c];
-    if (better(v, c, bv, bi)) { bv = v; bi = c; }
-  }
-  __shared__ float sv[32];
-  __shared__ int si[32];
-  warp_argmax(bv, bi);
-  if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = bv; si[threadIdx.x >> 5] = bi; }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    int nw = blockDim.x >> 5;
-    bv = threadIdx.x < nw ? sv[threadIdx.x] : -INFINITY;
-    bi = threadIdx.x < nw ? si[threadIdx.x] : 0x7fffffff;
-    warp_argmax(bv, bi);
-    if (threadIdx.x == 0) { pval[m] = bv; pidx[m] = bi; }
-  }
+  if (!on) return;
+  const float inv = 1.f / warp_sum(l);
+#pragma unroll
+  for (int e = 0; e < EPL; ++e) out[m * H * D + h * D + lane + e * 32] = from_f<T>(acc[e] * inv);
 }
 
 // ------------------------------------------------------------------ typical acceptance
@@ -717,64 +881,6 @@ __global__ void medusa_resblock(const float* __restrict__ h_last, const T* const
   }
 }
 
-// z[row][n] = W_lm[n] . r[row] for MC rows (row = b*K + k) over this block's slice of the
-// vocabulary, kept in shared memory; then each row's kmax best (value desc, index asc) of
-// the slice go to the partial lists pk_val/pk_idx [row][block][kmax].
-template <typename T, int MC>
-__global__ void medusa_lmhead_topk(const T* __restrict__ r, const T* __restrict__ Wlm, int rows_total, int V, int d,
-                                   int slice, int kmax, float* __restrict__ pk_val, int* __restrict__ pk_idx,
-                                   unsigned long long* tr) {
-  KTrace kt(tr);
-  pdl_launch_dependents();
-  pdl_wait();
-  if (threadIdx.x == 0) trace_mark_min(tr, 2);
-  constexpr int VN = Vec16<T>::N;
-  extern __shared__ float zs[];   // [MC][slice]
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  int n0 = blockIdx.x * slice, r0 = blockIdx.y * MC;
-  int n1 = min(n0 + slice, V);
-  for (int n = n0 + warp; n < n1; n += nw) {
-    const T* wr = Wlm + (size_t)n * d;
-    float acc[MC];
-#pragma unroll
-    for (int j = 0; j < MC; ++j) acc[j] = 0.f;
-    for (int c = lane * VN; c < d; c += 32 * VN) {
-      float wv[8], xv[8];
-      Vec16<T>::load(wr + c, wv);
-#pragma unroll
-      for (int j = 0; j < MC; ++j) {
-        if (r0 + j < rows_total) {
-          Vec16<T>::load(r + (size_t)(r0 + j) * d + c, xv);
-#pragma unroll
-          for (int e = 0; e < VN; ++e) acc[j] = fmaf(wv[e], xv[e], acc[j]);
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < MC; ++j) {
-      float v = warp_sum(acc[j]);
-      if (lane == 0) zs[j * slice + (n - n0)] = v;
-    }
-  }
-  __syncthreads();
-  for (int j = warp; j < MC; j += nw) {
-    if (r0 + j >= rows_total) continue;
-    float* z = zs + j * slice;
-    for (int t = 0; t < kmax; ++t) {
-      float bv = -INFINITY; int bi = 0x7fffffff;
-      for (int c = lane; c < n1 - n0; c += 32) if (better(z[c], n0 + c, bv, bi)) { bv = z[c]; bi = n0 + c; }
-      warp_argmax(bv, bi);
-      if (lane == 0) {
-        size_t o = ((size_t)(r0 + j) * gridDim.x + blockIdx.x) * kmax + t;
-        pk_val[o] = bv;
-        pk_idx[o] = bi;
-        if (bi != 0x7fffffff) z[bi - n0] = -INFINITY;
-      }
-      __syncwarp();
-    }
-  }
-}
-
 // Top-k of `n` pairs (v[c], ix[c]) (ix == nullptr: index base + c) in shared memory by a CTA of 256 threads, ordered (value
 // desc, index asc): the first kmax <= 16 go to emit(rank, value, index), absent ones as (-inf, 0x7fffffff). NaN never
 // wins. `v` and `ix` are scratch afterwards. Called by all threads.
@@ -878,19 +984,6 @@ __device__ __forceinline__ void topk_merge_row(const float* pk_val, const int* p
     out[t] = (tokv == 0x7fffffff) ? 0 : tokv;
   });
   if (k == 0 && threadIdx.x == 0) cand[(size_t)b * (K + 1) * kmax] = root_tok[b];
-}
-
-// The merge as a kernel of its own (one CTA per row; dynamic shared memory nblocks * kmax * 8 bytes).
-__global__ void __launch_bounds__(256)
-topk_merge(const float* __restrict__ pk_val, const int* __restrict__ pk_idx, int nblocks,
-           int rows_total, int K, int kmax, const int* __restrict__ root_tok,
-           const int* __restrict__ cand_override, int* __restrict__ cand, unsigned long long* tr) {
-  KTrace kt(tr);
-  pdl_launch_dependents();
-  pdl_wait();
-  if (threadIdx.x == 0) trace_mark_min(tr, 2);
-  extern __shared__ float ms[];     // values [nblocks*kmax], indices [nblocks*kmax]
-  topk_merge_row(pk_val, pk_idx, nblocks, blockIdx.x, K, kmax, root_tok, cand_override, cand, ms);
 }
 
 }  // namespace spec

@@ -201,7 +201,7 @@ struct spec_ctx {
   int T, K, kmax, B;                   // tree nodes, heads, candidates per head, current batch
   bool tc;                             // bf16 tensor-core path
   size_t esz;                          // operand element size
-  int Mcap, cap, pages_per_seq, gen_cap, nsplit_attn, Nqkv, ntile_lm, topk_slice, topk_blocks;
+  int Mcap, cap, pages_per_seq, gen_cap, nsplit_attn, Nqkv, n_argmax, topk_slice, topk_blocks;
   bool qkv_fused, keep_logits;
   bool packed = false;                 // linear weights are pre-tiled images (SPEC_FLAG_PACKED_WEIGHTS)
   bool pdl = true;                     // programmatic dependent launch between the kernels of a step
@@ -358,7 +358,7 @@ size_t carve(spec_ctx* c, void* base) {
   if (64 % f.page_size == 0) c->cap = (int)round_up(c->cap, 64);   // whole 64-key attention tiles
   c->pages_per_seq = c->cap / f.page_size;
   c->gen_cap = f.max_seq + K + 1;
-  c->ntile_lm = c->tc ? 8 : 1;   // argmax partials per row (vocabulary slices)
+  c->n_argmax = 8;                // argmax partials per row (vocabulary slices)
   c->topk_slice = ((V + SM_SLOTS - 1) / SM_SLOTS + 3) / 4 * 4;
   c->topk_blocks = (V + c->topk_slice - 1) / c->topk_slice;
   c->nsplit_attn = c->tc ? std::max(1, std::min(16, (SM_SLOTS / 2) / (f.n_heads * B))) : 1;   // most KV splits a launch may use
@@ -405,14 +405,14 @@ size_t carve(spec_ctx* c, void* base) {
         int r_hd[GS_MAX_MATS] = {d, d, d, d};
         if (plan_gemm((int)m, d, GS_MAX_MATS, r_hd, SM_SLOTS, &g)) pf = std::max(pf, plan_part_floats(g));
       } else {
-        pf = std::max(pf, std::max(m * (size_t)c->Nqkv, 2 * m * (size_t)F));
+        pf = std::max(pf, std::max(m * (size_t)c->Nqkv, (size_t)B * K * round_up(V, 4)));   // q, k, v; the heads' logits
       }
     }
   }
   c->part_floats = pf;
   c->d_part = b.take<float>(pf, 1024);
   c->d_logits = c->keep_logits ? b.take<float>((size_t)Mlog * V, 1024) : nullptr;
-  c->d_pval = b.take<float>((size_t)c->ntile_lm * M, 1024); c->d_pidx = b.take<int>((size_t)c->ntile_lm * M, 1024);
+  c->d_pval = b.take<float>((size_t)c->n_argmax * M, 1024); c->d_pidx = b.take<int>((size_t)c->n_argmax * M, 1024);
   // partial outputs of the KV splits: rows times splits, over the passes that use more than one split
   size_t split_rows = (size_t)c->nsplit_attn * B * std::max(T, PREFILL_ROWS);
   for (int g = 1; g <= c->chunk_cap; ++g)
@@ -507,7 +507,7 @@ constexpr int GP_MAX_CLUSTERS = SM_SLOTS / 4;   // one CTA per SM, two CTAs per 
 bool pair_gemm_ok(const spec_ctx* c, int M, int K) { return c->wide_gemm && M > 128 && K % 64 == 0; }
 
 template <int MODE>
-cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, const PairGemmParams& p) {
+cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, const PairGemmParams& p, int max_clusters = GP_MAX_CLUSTERS) {
   static bool attr_set_dev[kAttrDevices] = {};
   bool& attr_set = *attr_flag(attr_set_dev);
   if (!attr_set) {
@@ -515,7 +515,7 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, const Pa
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  const int grid = 2 * std::min(p.w_pairs * p.m_tiles, GP_MAX_CLUSTERS);
+  const int grid = 2 * std::min(p.w_pairs * p.m_tiles, std::min(GP_MAX_CLUSTERS, max_clusters));
   return launch_k(pdl, gemm_pair<MODE, GP_NT>, dim3(grid), dim3(GP_THREADS), (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
 }
 
@@ -705,21 +705,30 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
   return SPEC_OK;
 }
 
-template <typename T>
-int linear_simple(spec_ctx* c, const T* x, int ldx, const T* W, float* y, int ldy, int M, int N, int K) {
-  constexpr int MC = 8;
-  dim3 grid((N + 7) / 8, (M + MC - 1) / MC);
-  linear_rows<T, MC><<<grid, 256, 0, c->stream>>>(x, ldx, W, y, ldy, M, N, K);
-  LAUNCH_CHECK("linear_rows");
-  return SPEC_OK;
-}
-
 #define KLAUNCH(name, kernel, grid, block, smem, ...)                                            \
   do {                                                                                         \
     cudaError_t e_ = launch_k(c->pdl, kernel, grid, block, smem, c->stream, __VA_ARGS__, c->next_trace(name)); \
     c->launches++;                                                                             \
     if (e_ != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string(name) + ": " + cudaGetErrorString(e_)); \
   } while (0)
+
+// y[M, rows of all matrices] = x * [mats]^T on the CUDA cores, act = SiLU(x W_0^T) * (x W_1^T) (LR_SWIGLU, float32 y unused)
+// or y += x * W_0^T (LR_RESIDUAL). ldy: row pitch of y.
+template <typename T, int MODE>
+int linear_simple(spec_ctx* c, const char* name, const T* x, int n_mats, const void* const* mats, const int* rows, float* y, size_t ldy, T* act,
+                  int M, int K) {
+  RowLinear<T> w{};
+  w.n_mats = n_mats;
+  int groups = 0;
+  for (int i = 0; i < n_mats; ++i) {
+    w.w[i] = static_cast<const T*>(mats[i]); w.rows[i] = rows[i]; w.group0[i] = groups;
+    if (MODE != LR_SWIGLU) groups += (rows[i] + LR_N - 1) / LR_N;
+  }
+  if (MODE == LR_SWIGLU) groups = (rows[0] + LR_N / 2 - 1) / (LR_N / 2);
+  const RowLinearShape sh = linear_rows_shape<T>(groups, M, K);
+  KLAUNCH(name, (linear_rows<T, MODE>), sh.grid, dim3(LR_WARPS * 32), 0, x, w, y, ldy, act, M, K, groups, sh.ks, sh.ms);
+  return SPEC_OK;
+}
 
 // Passes with several 16-row blocks whose (sequence, head, row block) CTAs fit the SMs in one wave
 // use the kernel that needs no merge across CTAs and no length-dependent launch shape.
@@ -965,52 +974,92 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
   return SPEC_OK;
 }
 
+template <typename T, int EPL>
+int launch_attention_plain(spec_ctx* c, const Rows& rows, int l) {
+  static bool set_dev[kAttrDevices] = {};
+  bool& set_ = *attr_flag(set_dev);
+  const size_t sm = attention_plain_smem(EPL * 32);
+  if (!set_) { CUDA_OK(cudaFuncSetAttribute(attention_plain<T, EPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); set_ = true; }
+  KLAUNCH("attention_plain", (attention_plain<T, EPL>), dim3(c->cfg.n_heads, rows.B, (rows.R + AP_ROWS - 1) / AP_ROWS), dim3(AP_ROWS * 32), sm,
+          static_cast<const T*>(c->d_q), static_cast<T*>(c->d_attn), static_cast<const T*>(c->d_pool), c->geom, (const int*)c->d_page_table, rows, l,
+          c->cfg.n_heads, 1.0f / sqrtf((float)c->cfg.head_dim));
+  return SPEC_OK;
+}
+
 // The same pass with the plain CUDA-core kernels (float32 configurations and the bf16 debug mode).
 template <typename T>
 int forward_layers(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const int* n_lo_pass, const int* len_now) {
   if (c->tc) return forward_layers_tc(c, rows, n_hi_pass, n_lo_pass, len_now);
   const spec_config& f = c->cfg;
-  const int R = rows.R;
-  int M = rows.B * R, d = f.d_model, F = f.d_ffn, H = f.n_heads, D = f.head_dim, HD = H * D;
+  const int R = rows.R, M = rows.B * R, d = f.d_model, F = f.d_ffn, H = f.n_heads, D = f.head_dim, HD = H * D, KD = f.n_kv_heads * D;
   T* u = static_cast<T*>(c->d_u);
   T* q = static_cast<T*>(c->d_q);
   T* attn = static_cast<T*>(c->d_attn);
   T* act = static_cast<T*>(c->d_act);
   T* pool = static_cast<T*>(c->d_pool);
-  int pending = 0;              // 1: the previous down-projection output is still to be added to x
   for (int l = 0; l < f.n_layers; ++l) {
-    rmsnorm_rows<T><<<M, 256, 0, c->stream>>>(c->d_x, c->d_part, pending, (size_t)M * d, c->an[l], f.rms_eps, u, nullptr, d);
-    LAUNCH_CHECK("rmsnorm_rows");
-    int nk = f.n_kv_heads * D, r;
-    if ((r = linear_simple<T>(c, u, d, static_cast<const T*>(c->wq[l]), c->d_part, c->Nqkv, M, HD, d))) return r;
-    if ((r = linear_simple<T>(c, u, d, static_cast<const T*>(c->wk[l]), c->d_part + HD, c->Nqkv, M, nk, d))) return r;
-    if ((r = linear_simple<T>(c, u, d, static_cast<const T*>(c->wv[l]), c->d_part + HD + nk, c->Nqkv, M, nk, d))) return r;
-    rope_store<T><<<M, 256, 0, c->stream>>>(c->d_part, 1, (size_t)M * c->Nqkv, rows, c->d_rope, q, pool, c->geom, c->d_page_table, l, H);
-    LAUNCH_CHECK("rope_store");
+    int r;
+    KLAUNCH("rmsnorm_rows", rmsnorm_rows<T>, dim3(M), dim3(256), 0, (const float*)c->d_x, c->an[l], f.rms_eps, u, (float*)nullptr, d);
     {
-      dim3 grid(H, rows.B, (R + 3) / 4);
-      attention_simple<T><<<grid, 128, 0, c->stream>>>(q, attn, pool, c->geom, c->d_page_table, rows, l, H, 1.0f / sqrtf((float)D));
-      LAUNCH_CHECK("attention_simple");
+      const void* mats[3] = {c->wq[l], c->wk[l], c->wv[l]};
+      const int rws[3] = {HD, KD, KD};
+      if ((r = linear_simple<T, LR_PLAIN>(c, "linear_qkv", u, 3, mats, rws, c->d_part, c->Nqkv, nullptr, M, d))) return r;
     }
-    if ((r = linear_simple<T>(c, attn, HD, static_cast<const T*>(c->wo[l]), c->d_part, d, M, d, HD))) return r;
-    rmsnorm_rows<T><<<M, 256, 0, c->stream>>>(c->d_x, c->d_part, 1, (size_t)M * d, c->fn[l], f.rms_eps, u, nullptr, d);
-    LAUNCH_CHECK("rmsnorm_rows");
+    KLAUNCH("rope_store", rope_store<T>, dim3(M), dim3(256), 0, (const float*)c->d_part, rows, (const float2*)c->d_rope, q, pool, c->geom,
+            (const int*)c->d_page_table, l, H);
+    switch (D / 32) {
+      case 1: r = launch_attention_plain<T, 1>(c, rows, l); break;
+      case 2: r = launch_attention_plain<T, 2>(c, rows, l); break;
+      case 3: r = launch_attention_plain<T, 3>(c, rows, l); break;
+      case 4: r = launch_attention_plain<T, 4>(c, rows, l); break;
+      case 5: r = launch_attention_plain<T, 5>(c, rows, l); break;
+      case 6: r = launch_attention_plain<T, 6>(c, rows, l); break;
+      case 7: r = launch_attention_plain<T, 7>(c, rows, l); break;
+      default: r = launch_attention_plain<T, 8>(c, rows, l); break;
+    }
+    if (r) return r;
     {
-      float* g = c->d_part;
-      float* up = c->d_part + (size_t)M * F;
-      if ((r = linear_simple<T>(c, u, d, static_cast<const T*>(c->wg[l]), g, F, M, F, d))) return r;
-      if ((r = linear_simple<T>(c, u, d, static_cast<const T*>(c->wu[l]), up, F, M, F, d))) return r;
-      size_t total = (size_t)M * F;
-      swiglu_rows<T><<<(unsigned)((total + 255) / 256), 256, 0, c->stream>>>(g, up, act, total);
-      LAUNCH_CHECK("swiglu_rows");
+      const void* mats[1] = {c->wo[l]};
+      if ((r = linear_simple<T, LR_RESIDUAL>(c, "linear_wo", attn, 1, mats, &d, c->d_x, d, nullptr, M, HD))) return r;
     }
-    if ((r = linear_simple<T>(c, act, F, static_cast<const T*>(c->wd[l]), c->d_part, d, M, d, F))) return r;
-    pending = 1;
+    KLAUNCH("rmsnorm_rows", rmsnorm_rows<T>, dim3(M), dim3(256), 0, (const float*)c->d_x, c->fn[l], f.rms_eps, u, (float*)nullptr, d);
+    {
+      const void* mats[2] = {c->wg[l], c->wu[l]};
+      const int rws[2] = {F, F};
+      if ((r = linear_simple<T, LR_SWIGLU>(c, "linear_gate_up", u, 2, mats, rws, nullptr, 0, act, M, d))) return r;
+    }
+    {
+      const void* mats[1] = {c->wd[l]};
+      if ((r = linear_simple<T, LR_RESIDUAL>(c, "linear_down", act, 1, mats, &d, c->d_x, d, nullptr, M, F))) return r;
+    }
   }
   // final norm: hidden (float32) and its operand-typed copy
-  rmsnorm_rows<T><<<M, 256, 0, c->stream>>>(c->d_x, c->d_part, pending, (size_t)M * d, c->final_norm, f.rms_eps,
-                                            static_cast<T*>(c->d_hq), c->d_hid, d);
-  LAUNCH_CHECK("rmsnorm_rows");
+  KLAUNCH("rmsnorm_rows", rmsnorm_rows<T>, dim3(M), dim3(256), 0, (const float*)c->d_x, c->final_norm, f.rms_eps, static_cast<T*>(c->d_hq), c->d_hid, d);
+  return SPEC_OK;
+}
+
+// A [rows][ld] matrix of finished float32 values seen as one slot of partial sums.
+PartView plain_view(const float* p, int rows, int ld) {
+  PartView v{};
+  v.part = p; v.slot_stride = (size_t)rows * ld; v.ld = ld;
+  v.seg.KC = 1; v.seg.m_tiles = 1; v.seg.G = v.seg.total = (ld + 127) / 128;
+  v.mt_shift = 30;                     // all rows are one activation tile
+  v.single = 1;
+  return v;
+}
+
+// Per-head top-k over the heads' logits into the candidate table.
+int heads_top_k(spec_ctx* c, const PartView& pl, int rows_total, const int* ov) {
+  const int kmax = c->kmax, V = c->cfg.vocab;
+  // the row's last-arriving CTA merges the slices' lists: no merge kernel
+  // about 296 CTAs whatever the number of rows, at least four a row: more slices would only lengthen the lists to merge
+  // (and at least as many as let a slice fit 40 KB)
+  const int want = std::min(c->topk_blocks, std::max(std::max(4, (V + 10239) / 10240), SM_SLOTS / rows_total));
+  const int slice = (int)round_up((V + want - 1) / want, 4), blocks = (V + slice - 1) / slice;
+  const size_t sm_topk = std::max((size_t)slice * sizeof(float), (size_t)blocks * kmax * 8);
+  if (sm_topk > 44 * 1024) return c->fail(SPEC_E_BADARG, "top-k lists do not fit the merge's shared memory");
+  KLAUNCH("topk_slices_tc", topk_slices_tc, dim3(blocks, rows_total), dim3(256), sm_topk,
+          pl, V, rows_total, slice, kmax, c->d_pk_val, c->d_pk_idx, c->d_row_arrive, c->K, (const int*)c->d_root, ov, c->d_cand);
   return SPEC_OK;
 }
 
@@ -1018,7 +1067,7 @@ int forward_layers(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const in
 // output dimension, up to four per launch), shared lm_head, per-head top-k.
 int heads_tc(spec_ctx* c, const int* ov) {
   const spec_config& f = c->cfg;
-  const int B = c->B, K = c->K, d = f.d_model, kmax = c->kmax, rows_total = B * K;
+  const int B = c->B, K = c->K, d = f.d_model, rows_total = B * K;
   const int dpad = (d + 127) / 128 * 128;
   for (int k0 = 0; k0 < K; k0 += GS_MAX_MATS) {
     const int nk = std::min(GS_MAX_MATS, K - k0);
@@ -1038,44 +1087,33 @@ int heads_tc(spec_ctx* c, const int* ov) {
     int r = run_gemm(c, c->d_r, rows_total, d, 1, mats, rws, SPEC_PROFILE_OFF, &pl);
     if (r) return r;
   }
-  // the row's last-arriving CTA merges the slices' lists: no merge kernel
-  // about 296 CTAs whatever the number of rows, at least four a row: more slices would only lengthen the lists to merge
-  // (and at least as many as let a slice fit 40 KB)
-  const int want = std::min(c->topk_blocks, std::max(std::max(4, (f.vocab + 10239) / 10240), SM_SLOTS / rows_total));
-  const int slice = (int)round_up((f.vocab + want - 1) / want, 4), blocks = (f.vocab + slice - 1) / slice;
-  const size_t sm_topk = std::max((size_t)slice * sizeof(float), (size_t)blocks * kmax * 8);
-  if (sm_topk > 48 * 1024) return c->fail(SPEC_E_BADARG, "top-k lists do not fit the merge's shared memory");
-  KLAUNCH("topk_slices_tc", topk_slices_tc, dim3(blocks, rows_total), dim3(256), sm_topk,
-          pl, f.vocab, rows_total, slice, kmax, c->d_pk_val, c->d_pk_idx, c->d_row_arrive, K, (const int*)c->d_root, ov, c->d_cand);
-  return SPEC_OK;
+  return heads_top_k(c, pl, rows_total, ov);
 }
 
 // lm_head over `M` operand rows at `src`, leaving per-row argmax partials (and logits).
 template <typename T>
 int lm_head_argmax(spec_ctx* c, const T* src, int M) {
   const spec_config& f = c->cfg;
+  PartView pl{};
+  const void* mats[1] = {c->lm_head};
+  int rws[1] = {f.vocab};
   if (c->tc) {
-    PartView pl{};
-    const void* mats[1] = {c->lm_head};
-    int rws[1] = {f.vocab};
     int r = run_gemm(c, src, M, f.d_model, 1, mats, rws, SPEC_PROFILE_OFF, &pl);
     if (r) return r;
-    const int NSL = c->ntile_lm;
-    KLAUNCH("argmax_partials_tc", argmax_partials_tc, dim3(M, NSL), dim3(256), 0, pl, f.vocab,
-            c->keep_logits ? c->d_logits : (float*)nullptr, c->d_pval, c->d_pidx, c->d_row_arrive, c->d_pval2, c->d_pidx2);
   } else {
-    int r = linear_simple<T>(c, src, f.d_model, static_cast<const T*>(c->lm_head), c->d_logits, f.vocab, M, f.vocab, f.d_model);
+    int r = linear_simple<T, LR_PLAIN>(c, "linear_lm_head", src, 1, mats, rws, c->d_logits, f.vocab, nullptr, M, f.d_model);
     if (r) return r;
-    argmax_rows<<<M, 256, 0, c->stream>>>(c->d_logits, f.vocab, c->d_pval, c->d_pidx);
-    LAUNCH_CHECK("argmax_rows");
+    pl = plain_view(c->d_logits, M, f.vocab);
   }
+  KLAUNCH("argmax_partials_tc", argmax_partials_tc, dim3(M, c->n_argmax), dim3(256), 0, pl, f.vocab,
+          c->tc && c->keep_logits ? c->d_logits : (float*)nullptr, c->d_pval, c->d_pidx, c->d_row_arrive, c->d_pval2, c->d_pidx2);
   return SPEC_OK;
 }
 
 AcceptArgs make_accept(spec_ctx* c, int R, int mode) {
   AcceptArgs a{};
   a.rows = make_rows(c, R, false);
-  a.pval = c->tc ? c->d_pval2 : c->d_pval; a.pidx = c->tc ? c->d_pidx2 : c->d_pidx; a.ntile = 1;
+  a.pval = c->d_pval2; a.pidx = c->d_pidx2; a.ntile = 1;
   a.hq_last = c->tc ? static_cast<bf16*>(c->d_hq_last) : nullptr;
   a.parent = c->d_parent; a.depth = c->d_depth; a.edge_ok = nullptr;
   a.K = c->K; a.frag_token = c->cfg.frag_token; a.d = c->cfg.d_model; a.mode = mode;
@@ -1187,15 +1225,11 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
     dim3 g1((K * d + 7) / 8, (B + MC - 1) / MC);
     KLAUNCH("medusa_resblock", (medusa_resblock<T, MC>), g1, dim3(256), 0, (const float*)c->d_h_last,
             reinterpret_cast<const T* const*>(c->d_mw), reinterpret_cast<const T* const*>(c->d_mb), static_cast<T*>(c->d_r), B, K, d);
-    int rows_total = B * K;
-    dim3 g2(c->topk_blocks, (rows_total + MC - 1) / MC);
-    size_t sm = (size_t)MC * c->topk_slice * sizeof(float);
-    KLAUNCH("medusa_lmhead_topk", (medusa_lmhead_topk<T, MC>), g2, dim3(256), sm, static_cast<const T*>(c->d_r),
-            static_cast<const T*>(c->lm_head), rows_total, f.vocab, d, c->topk_slice, kmax, c->d_pk_val, c->d_pk_idx);
-    // partial lists of the row chunks are laid out per block over all rows
-    size_t sm2 = (size_t)c->topk_blocks * kmax * 8 + (size_t)c->topk_blocks * 4;
-    KLAUNCH("topk_merge", topk_merge, dim3(rows_total), dim3(256), sm2, (const float*)c->d_pk_val, (const int*)c->d_pk_idx,
-            c->topk_blocks, rows_total, K, kmax, (const int*)c->d_root, ov, c->d_cand);
+    const void* mats[1] = {c->lm_head};
+    const int ldz = (int)round_up(f.vocab, 4);
+    int r = linear_simple<T, LR_PLAIN>(c, "linear_heads", static_cast<const T*>(c->d_r), 1, mats, &f.vocab, c->d_part, ldz, nullptr, B * K, d);
+    if (r) return r;
+    if ((r = heads_top_k(c, plain_view(c->d_part, B * K, ldz), B * K, ov))) return r;
   } else {
     CUDA_OK(cudaMemcpyAsync(c->d_cand, c->d_root, B * sizeof(int), cudaMemcpyDeviceToDevice, c->stream));
   }
@@ -1705,6 +1739,13 @@ int spec_debug_read_kv(spec_ctx* c, int32_t seq, int32_t layer, int32_t slot0, i
 }
 
 namespace {
+// Waits for the call's kernels and reads their status word.
+int op_linear_status(const int* status, cudaStream_t st) {
+  int stw[4];
+  if (cudaMemcpyAsync(stw, status, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+    return SPEC_E_CUDA;
+  return stw[0] == 0 ? SPEC_OK : SPEC_E_TIMEOUT;
+}
 // Shared body of the two stand-alone linear entry points (bf16): scratch holds the partial
 // sums followed by the four-int status word.
 int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, int ctas, float* scratch,
@@ -1713,6 +1754,19 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
   int rws[1] = {N};
   if (!plan_gemm(M, K, 1, rws, ctas, &g)) return SPEC_E_BADARG;
   StreamTmaps tm{};
+  if (M > 128) {
+    // many rows: whole tiles on pairs of SMs, finished sums straight into y (at M = 1008, N = 11008, K = 4096 the call takes
+    // 116 us; weight streaming, which fetches the weights once per 128 rows, took 127 us, adding up its partial sums 34, the call 204)
+    PairGemmParams p{};
+    if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, GP_NT / 2)) return SPEC_E_CUDA;
+    p.M = M; p.KC = K / 64; p.n_mats = 1;
+    p.n_tiles = g.p.n_tiles; p.w_pairs = (g.p.n_tiles + 1) / 2; p.m_tiles = (M + GP_NT - 1) / GP_NT;
+    for (int i = 1; i <= GS_MAX_MATS; ++i) p.mat_tile0[i] = p.n_tiles;
+    p.out = y; p.ld = (size_t)N; p.n_cols = N;
+    p.status = reinterpret_cast<int*>(scratch + scratch_floats);
+    if (cudaMemsetAsync(p.status, 0, 16, st) != cudaSuccess || launch_gp<GP_PLAIN>(st, false, tm, p, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
+    return op_linear_status(p.status, st);
+  }
   if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, g.MT)) return SPEC_E_CUDA;
   g.p.part = scratch;
   g.p.slot_stride = (size_t)M * g.p.n_tiles * 128;
@@ -1722,12 +1776,17 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
   if (cudaMemsetAsync(g.p.status, 0, 16, st) != cudaSuccess) return SPEC_E_CUDA;
   if (launch_gs(st, false, g, tm) != cudaSuccess) return SPEC_E_CUDA;
   size_t total = (size_t)M * ((N + 3) / 4);
-  part_sum_rows<<<(unsigned)std::min<size_t>((total + 255) / 256, 4096), 256, 0, st>>>(plan_view(g), y, M, N);
-  if (cudaGetLastError() != cudaSuccess) return SPEC_E_CUDA;
-  int stw[4];
-  if (cudaMemcpyAsync(stw, g.p.status, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+  if (launch_k(true, part_sum_rows, dim3((unsigned)std::min<size_t>((total + 255) / 256, 4096)), dim3(256), 0, st, plan_view(g), y, M, N) != cudaSuccess)
     return SPEC_E_CUDA;
-  return stw[0] == 0 ? SPEC_OK : SPEC_E_TIMEOUT;
+  return op_linear_status(g.p.status, st);
+}
+int op_linear_f32(const void* x, const void* w, float* y, int M, int N, int K, cudaStream_t st) {
+  RowLinear<float> rl{};
+  rl.w[0] = static_cast<const float*>(w); rl.rows[0] = N; rl.n_mats = 1;
+  const int groups = (N + LR_N - 1) / LR_N;
+  const RowLinearShape sh = linear_rows_shape<float>(groups, M, K);
+  linear_rows<float, LR_PLAIN><<<sh.grid, LR_WARPS * 32, 0, st>>>(static_cast<const float*>(x), rl, y, (size_t)N, nullptr, M, K, groups, sh.ks, sh.ms, nullptr);
+  return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_E_CUDA;
 }
 bool op_linear_args_ok(int32_t dtype, const void* x, const void* w, const float* y, int M, int N, int K, int ctas) {
   if (!x || !w || !y || M < 1 || N < 1 || K < 8 || K % 8 || M > 2048) return false;
@@ -1779,10 +1838,7 @@ int spec_op_linear(int32_t dtype, const void* x, const void* w, float* y, int32_
   if (!op_linear_args_ok(dtype, x, w, y, M, N, K, ctas)) return SPEC_E_BADARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (dtype == 0) {
-    constexpr int MC = 8;
-    dim3 grid((N + 7) / 8, (M + MC - 1) / MC);
-    linear_rows<float, MC><<<grid, 256, 0, st>>>(static_cast<const float*>(x), K, static_cast<const float*>(w), y, N, M, N, K);
-    return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_E_CUDA;
+    return op_linear_f32(x, w, y, M, N, K, st);
   }
   if (!scratch) return SPEC_E_BADARG;
   return op_linear_bf16(x, w, y, M, N, K, ctas, scratch, spec_op_linear_scratch_floats(M, N, K, ctas), st);
@@ -1805,10 +1861,7 @@ extern "C" int spec_op_linear_static(int32_t dtype, const void* x, const void* w
   if (!op_linear_args_ok(dtype, x, w, y, M, N, K, ctas)) { g_create_error = "spec_op_linear_static: bad argument"; return SPEC_E_BADARG; }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (dtype == 0) {
-    constexpr int MC = 8;
-    dim3 grid((N + 7) / 8, (M + MC - 1) / MC);
-    linear_rows<float, MC><<<grid, 256, 0, st>>>(static_cast<const float*>(x), K, static_cast<const float*>(w), y, N, M, N, K);
-    return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_E_CUDA;
+    return op_linear_f32(x, w, y, M, N, K, st);
   }
   const size_t need = spec_op_linear_scratch_floats(M, N, K, ctas);
   if (need == 0) { g_create_error = "spec_op_linear_static: bad argument"; return SPEC_E_BADARG; }

@@ -1,0 +1,48 @@
+"""The float32 kernels at the edges of their tiles: projections (split inner dimension, ragged rows and columns) and
+attention (every head width, one tile of keys and several)."""
+import pytest
+
+from synthetic import draw_prompt, draw_weights, get_config
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    t = pytest.importorskip("torch")
+    if not t.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    return t
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (1, 1, 8),           # one output, most lanes without a piece of the inner dimension
+    (7, 301, 96),        # ragged rows and columns, less than one step of 128
+    (3, 9, 2048),        # four warps split the inner dimension
+    (9, 130, 264),       # two warps split it, the last step is not full
+    (16, 32016, 256),    # a CTA's warps walk over the outputs, two row groups beside each other
+    (100, 3000, 1024),   # 13 row groups
+])
+def test_op_linear_f32(torch, M, N, K):
+    """Bound: K accumulations in float32, each off by at most half a unit in the last place of the running sum."""
+    from paper_2503_14153_b200 import spec_op_linear
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    x, w = torch.randn((M, K), generator=g, device="cuda"), torch.randn((N, K), generator=g, device="cuda")
+    y = spec_op_linear(x, w)
+    want, size = x.double() @ w.double().T, x.double().abs() @ w.double().abs().T
+    assert ((y.double() - want).abs() <= K * 2.0 ** -24 * size).all()
+
+
+@pytest.mark.parametrize("hd,heads,kv,prompt_len,dtype", [
+    (32, 4, 4, 150, "fp32"), (64, 4, 2, 140, "fp32"), (96, 2, 2, 70, "fp32"), (128, 2, 1, 63, "fp32"), (160, 2, 2, 33, "fp32"),
+    (256, 2, 2, 100, "fp32"), (256, 1, 1, 1, "fp32"), (64, 4, 2, 140, "bf16"),
+])
+def test_plain_attention_vs_oracle(torch, hd, heads, kv, prompt_len, dtype):
+    """Decoding on the CUDA-core kernels (bf16: the debug mode of the 16-bit path) with contexts of one key tile, several, and
+    a last group of keys that is not full, grouped heads among them."""
+    from paper_2503_14153_b200 import FLAG_SIMPLE_KERNELS, build_tree
+    from tests_lockstep import run_lockstep
+    cfg = get_config("c0", name="plain", n_heads=heads, n_kv_heads=kv, head_dim=hd, dtype=dtype, vocab=2000, seed=hd, norm_gain="random")
+    rep = run_lockstep(cfg, draw_weights(cfg), build_tree(cfg.topk, cfg.tree_nodes), draw_prompt(cfg, prompt_len), 10,
+                       1e-4 if dtype == "fp32" else 2e-2, 1e-2, flags=FLAG_SIMPLE_KERNELS if dtype == "bf16" else 0)
+    assert rep.steps > 0

@@ -74,3 +74,20 @@ def test_prompts_in_chunks_vs_oracle(torch, hd, lengths):
     gpu.close()
     for b in oracles:
         assert reps[b].steps == 2
+
+
+@pytest.mark.parametrize("M,N,K,ctas", [(144, 128, 64, 1), (272, 300, 64, 2), (1008, 1000, 704, 148), (2048, 129, 128, 296),
+                                        (512, 4096, 4096, 7)])
+def test_op_linear_many_rows(torch, M, N, K, ctas):
+    """More than 128 rows of the stand-alone projection: one weight tile (computed by both SMs of a pair, stored once), ragged
+    columns and activation tiles, more tiles than CTA pairs. Bound: K accumulations in float32, each off by at most one
+    unit in the last place of the running sum, against sum |x w|."""
+    from paper_2503_14153_b200 import spec_op_linear
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    x = torch.randn((M, K), generator=g, device="cuda", dtype=torch.bfloat16)
+    w = torch.randn((N, K), generator=g, device="cuda", dtype=torch.bfloat16)
+    y = spec_op_linear(x, w, ctas)
+    want, size = x.double() @ w.double().T, x.double().abs() @ w.double().abs().T
+    assert ((y.double() - want).abs() <= K * 2.0 ** -23 * size).all()
+    # the bound above is loose where K is large: a dropped or doubled 64-wide chunk would still show here
+    assert ((y.double() - want).norm() / want.norm()).item() < 2e-5
