@@ -422,7 +422,9 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
                 if (!on || v.kv < 0) continue;
                 const float a = lower ? __uint_as_float(r[j]) : ex_lo[j * 64 + pr];
                 const float c = lower ? ex_up[j * 64 + pr] : __uint_as_float(r[16 + j]);
-                const bf16 lo = __float2bfloat16_rn(a * t[j].x - c * t[j].y), hi = __float2bfloat16_rn(c * t[j].x + a * t[j].y);
+                                // (the rounding of the other kernels that rotate: one product rounded, the other fused into the sum)
+                const bf16 lo = __float2bfloat16_rn(__fmaf_rn(a, t[j].x, -__fmul_rn(c, t[j].y)));
+                const bf16 hi = __float2bfloat16_rn(__fmaf_rn(c, t[j].x, __fmul_rn(a, t[j].y)));
                 if (mat == 0) {
                   bf16* dst = p.q + (size_t)(m0 + jb + j) * p.H * D + head * D + di;
                   dst[0] = lo;
