@@ -173,7 +173,7 @@ int64_t spec_query(const spec_ctx *ctx, int32_t what);
  * record a device timeline of every step (see spec_trace_read). SPEC_OPT_GRAPH [1]: record the
  * kernel sequence of a step into a CUDA graph once and replay it on the following steps (a new
  * recording when a sequence grows past the 768 positions the single-split attention launch covers,
- * after a prefill and after an option change; steps that are traced or profiled are enqueued
+ * after a prefill whose sequences the recording was not planned for (shorter ones, above all) and after an option change; steps that are traced or profiled are enqueued
  * directly). Results do not depend on it. SPEC_OPT_PHASE_TIMING [0]: record an event at the five
  * phase boundaries of every step for spec_last_step_phase_ms (costs the programmatic overlap at
  * those boundaries: about 0.03 ms of a 7B step). SPEC_OPT_CLUSTER_EPILOGUE [7]: bit mask of the projections

@@ -226,6 +226,8 @@ struct spec_ctx {
   // device buffers (workspace)
   int *d_n, *d_cnt, *d_n_old, *d_root, *d_count, *d_path, *d_out_tok, *d_gen_cnt, *d_gen_log, *d_cand, *d_cand_ov;
   int *d_tok, *d_pos, *d_slot, *d_am, *d_edge, *d_parent, *d_depth, *d_rank, *d_page_table, *d_prompt, *d_offsets;
+  int *d_result;                       // [4 + B * (K + 3)]: d_status, d_n, d_count, d_out_tok
+  int* h_result = nullptr;             // the same in pinned host memory
   int *d_status, *d_pidx, *d_pk_idx, *d_draws;
   int chunk_cap;                       // prompt chunks the row buffers hold in one pass
   int *d_chunk_seq, *d_chunk_pos, *d_chunk_n, *d_chunk_cnt;   // [max_batch * ceil(max_seq / 128)]: sequence and first token; [chunk_cap]
@@ -265,9 +267,12 @@ struct spec_ctx {
     int B = 0;
     long long n_launches = 0;
     std::vector<int> n_hi_plan, n_lo_plan;
+    unsigned long long prefills = 0;   // the prompts it was recorded or last checked for
+    std::vector<int> order;            // sequences, longest first, where the recorded attention hands its CTAs out in that order
   };
   StepGraph step_graph[2];
   unsigned long long graph_epoch = 1;
+  unsigned long long prefills = 0;
   long long graph_captures = 0;
   bool prefilled = false;
   // timing: phase boundaries of the last step; optional per-launch timing of one kernel kind
@@ -366,14 +371,17 @@ size_t carve(spec_ctx* c, void* base) {
   c->keep_logits = !c->tc || (f.flags & SPEC_FLAG_KEEP_LOGITS) || f.accept_mode == 1;
   size_t M = c->Mcap;
 
-  c->d_status = b.take<int>(4);
+  // what a step hands to the host lies side by side, so that one copy brings it: status word, committed lengths, counts,
+  // emitted tokens
+  c->d_result = b.take<int>(4 + (size_t)B * (2 + K + 1));
+  c->d_status = c->d_result; c->d_n = c->d_result + 4; c->d_count = c->d_n + B; c->d_out_tok = c->d_count + B;
   c->d_trace = b.take<unsigned long long>((size_t)TRACE_CAP * 4);
   c->d_attn_arrive = b.take<unsigned int>((size_t)c->chunk_cap * f.n_heads * 2);
   c->d_row_arrive = b.take<unsigned int>(c->Mcap);
   c->d_pval2 = b.take<float>(c->Mcap); c->d_pidx2 = b.take<int>(c->Mcap);
   c->d_draws = b.take<int>(B);
-  c->d_n = b.take<int>(B); c->d_cnt = b.take<int>(B); c->d_n_old = b.take<int>(B); c->d_root = b.take<int>(B);
-  c->d_count = b.take<int>(B); c->d_path = b.take<int>((size_t)B * (K + 1)); c->d_out_tok = b.take<int>((size_t)B * (K + 1));
+  c->d_cnt = b.take<int>(B); c->d_n_old = b.take<int>(B); c->d_root = b.take<int>(B);
+  c->d_path = b.take<int>((size_t)B * (K + 1));
   c->d_gen_cnt = b.take<int>(B); c->d_gen_log = b.take<int>((size_t)B * c->gen_cap);
   c->d_cand = b.take<int>((size_t)B * (K + 1) * c->kmax); c->d_cand_ov = b.take<int>((size_t)B * (K ? K : 1) * c->kmax);
   c->d_tok = b.take<int>(M); c->d_pos = b.take<int>(M); c->d_slot = b.take<int>(M); c->d_am = b.take<int>(M);
@@ -1123,15 +1131,19 @@ AcceptArgs make_accept(spec_ctx* c, int R, int mode) {
   return a;
 }
 
+int report_status(spec_ctx* c, const int* st) {
+  if (st[0] == ST_OK) return SPEC_OK;
+  char buf[128];
+  snprintf(buf, sizeof(buf), "device status %d at %d (detail %d)", st[0], st[1], st[2]);
+  return c->fail(st[0] == ST_TIMEOUT ? SPEC_E_TIMEOUT : (st[0] == ST_SEQLEN ? SPEC_E_SEQLEN : SPEC_E_BADARG), buf);
+}
+
 int check_status(spec_ctx* c) {
   int st[4];
   cudaError_t e = cudaMemcpyAsync(st, c->d_status, sizeof(st), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("status read: ") + cudaGetErrorString(e));
-  if (st[0] == ST_OK) return SPEC_OK;
-  char buf[128];
-  snprintf(buf, sizeof(buf), "device status %d at %d (detail %d)", st[0], st[1], st[2]);
-  return c->fail(st[0] == ST_TIMEOUT ? SPEC_E_TIMEOUT : (st[0] == ST_SEQLEN ? SPEC_E_SEQLEN : SPEC_E_BADARG), buf);
+  return report_status(c, st);
 }
 
 template <typename T>
@@ -1147,7 +1159,7 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   }
   c->B = batch;
   c->prefilled = false;
-  c->graph_epoch++;   // recorded steps were planned for the previous sequences
+  c->prefills++;      // a recorded step stays valid while its plan covers the new sequences (step_t looks)
   std::vector<int> off(batch + 1);
   for (int b = 0; b <= batch; ++b) off[b] = offsets[b] - offsets[0];
   CUDA_OK(cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), c->stream));
@@ -1302,7 +1314,8 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     else if (c->n_hi[b] + T_ > ATTN_SINGLE_TILES * 64) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(std::max(attn_long_threshold(c, T_, B) / 64 * 64, ATTN_SINGLE_TILES * 64), c->cap) : c->cap;
     else bound = std::min(ATTN_SINGLE_TILES * 64, c->cap);
     n_hi_plan[b] = bound - T_;
-    n_lo_plan[b] = c->n_lo[b];
+    // the attention kernels fetch ahead of their dependency wait what lies below this bound, at most the first 1024 positions
+    n_lo_plan[b] = std::min(c->n_lo[b], 1024);
   }
   const bool use_graph = c->graph_on && !c->trace_on && c->profile_kind == 0;
   if (!use_graph) {
@@ -1312,6 +1325,16 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     spec_ctx::StepGraph& g = c->step_graph[ov ? 1 : 0];
     bool valid = g.exec && g.epoch == c->graph_epoch && g.B == B;
     for (int b = 0; valid && b < B; ++b) valid = c->n_hi[b] <= g.n_hi_plan[b] && c->n_lo[b] >= g.n_lo_plan[b];
+    // after a prefill: the same launch shape as a new recording would get (a shorter bound may choose another kernel) and the
+    // same order of the sequences
+    std::vector<int> order;
+    if (!valid || g.prefills != c->prefills) {
+      order.resize(B);
+      for (int b = 0; b < B; ++b) order[b] = b;
+      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return c->n_hi[x] > c->n_hi[y]; });
+      if (valid) valid = g.n_hi_plan == n_hi_plan && g.order == order;
+      if (valid) g.prefills = c->prefills;
+    }
     if (!valid) {
       // record the step once, then replay it until a sequence outgrows the planned bound
       cudaGraph_t graph = nullptr;
@@ -1335,6 +1358,7 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
       if (e != cudaSuccess) { g.exec = nullptr; c->launches = l0; return c->fail(SPEC_E_CUDA, std::string("step graph instantiate: ") + cudaGetErrorString(e)); }
       g.epoch = c->graph_epoch; g.B = B; g.n_launches = c->launches - l0;
       g.n_hi_plan = n_hi_plan; g.n_lo_plan = n_lo_plan;
+      g.prefills = c->prefills; g.order = order;
       c->launches = l0;
       c->graph_captures++;
     }
@@ -1350,11 +1374,14 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     }
   }
   if (out_tokens || out_counts) {
-    if (out_tokens) CUDA_OK(cudaMemcpyAsync(out_tokens, c->d_out_tok, (size_t)B * (K + 1) * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    if (out_counts) CUDA_OK(cudaMemcpyAsync(out_counts, c->d_count, (size_t)B * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    std::vector<int> nn(B);
-    CUDA_OK(cudaMemcpyAsync(nn.data(), c->d_n, B * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    int r = check_status(c);   // synchronises
+    // one copy of the whole result block and one wait (four copies of a few bytes each cost a short step 15 us more)
+    const int cap = f.max_batch;
+    CUDA_OK(cudaMemcpyAsync(c->h_result, c->d_result, (4 + (size_t)cap * (K + 3)) * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_OK(cudaStreamSynchronize(c->stream));
+    const int *nn = c->h_result + 4, *counts = nn + cap, *toks = counts + cap;
+    if (out_tokens) memcpy(out_tokens, toks, (size_t)B * (K + 1) * sizeof(int));
+    if (out_counts) memcpy(out_counts, counts, (size_t)B * sizeof(int));
+    int r = report_status(c, c->h_result);
     if (r) return r;
     for (int b = 0; b < B; ++b) c->n_hi[b] = c->n_lo[b] = nn[b];
     c->n_copy_pending = false;
@@ -1483,6 +1510,9 @@ int spec_create(const spec_config* cfg, const spec_weights* w, const spec_tree* 
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_cand, 0, (size_t)cfg->max_batch * (c->K + 1) * c->kmax * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) { g_create_error = std::string("set-up copies: ") + cudaGetErrorString(e); delete c; return SPEC_E_CUDA; }
+  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_result), (4 + (size_t)cfg->max_batch * (c->K + 3)) * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+    g_create_error = "pinned host memory for a step's result"; delete c; return SPEC_E_CUDA;
+  }
   if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_n_pinned), (size_t)cfg->max_batch * sizeof(int), cudaHostAllocDefault) != cudaSuccess) c->h_n_pinned = nullptr;
   if (cudaEventCreateWithFlags(&c->n_ev, cudaEventDisableTiming) != cudaSuccess) c->n_ev = nullptr;
   cudaGetLastError();
@@ -1549,6 +1579,7 @@ int spec_destroy(spec_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->n_ev) cudaEventDestroy(c->n_ev);
   if (c->h_n_pinned) cudaFreeHost(c->h_n_pinned);
+  if (c->h_result) cudaFreeHost(c->h_result);
   delete c;
   return SPEC_OK;
 }
