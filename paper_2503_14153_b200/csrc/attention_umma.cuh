@@ -1,8 +1,11 @@
 // Tree-masked attention on the 5th-generation tensor cores (tcgen05, accumulators in tensor memory) for
-// passes of up to 64 query rows per CTA over long contexts, and for batched passes.
+// passes over long contexts, for batched passes and for prompt processing.
 //
-// A CTA owns one head, up to 64 query rows (a "row half": a 128-row pass takes two CTAs per head) and one
-// split of the keys, and walks its keys in tiles of 128. A warp can read only the 32 tensor-memory lanes of
+// A CTA owns one head, ROWS = 64 or 128 query rows and one split of the keys, and walks its keys in tiles of 128.
+// With 128 rows (prompt chunks, trees of more than 64 nodes) a thread of a softmax group owns a row of the tile. Taking
+// 128 rows at a time instead of two CTAs of 64, each reading the keys, shortens a layer's attention over a 2048-token
+// prompt (16 chunks, 32 heads) from 146 to 118 us. What follows describes 64 rows.
+// A warp can read only the 32 tensor-memory lanes of
 // its own SM quarter, and lane = MMA row, so to put all four quarters to work the 64 query rows are given
 // twice to the 128-row MMA: rows 0..63 ("low stream") take care of keys 0..63 of every tile, rows 64..127
 // (the same queries again, "high stream") of keys 64..127.
@@ -38,7 +41,6 @@
 namespace spec {
 
 constexpr int AU_KT = 128;        // keys per tile
-constexpr int AU_ROWS = 64;       // query rows per CTA
 constexpr int AU_THREADS = 320;   // warps 0..3: softmax group 0; warps 4..7: group 1; warp 8: producer; warp 9: MMA
 constexpr float AU_RESCALE_LOG2 = 8.f;   // a stream's reference is raised when a tile's maximum exceeds it by more than this
 constexpr int AU_MAX_CLUSTER = 8; // most key splits (portable cluster size)
@@ -81,10 +83,13 @@ __device__ __forceinline__ float2 dsmem_ld2(uint32_t addr) {
 }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-template <int HD>
+template <int HD, int ROWS>
 __global__ void __launch_bounds__(AU_THREADS, 1)
 attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, unsigned long long* tr) {
   static_assert(HD == 128, "two 64-dim slabs per row");
+  static_assert(ROWS == 64 || ROWS == 128, "query rows per CTA");
+  constexpr int AU_ROWS = ROWS;
+  constexpr int STREAMS = 256 / ROWS;         // softmax streams a query row has: two groups, times two key halves with 64 rows
   KTrace kt(tr);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -152,8 +157,8 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
     }
   }
   if (warp == 9) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
-  // the P operands' off-diagonal blocks stay zero for the whole kernel
-  for (int c = threadIdx.x; c < 65536 / 16; c += AU_THREADS) reinterpret_cast<uint4*>(p_s)[c] = make_uint4(0, 0, 0, 0);
+  // with 64 rows the P operands' off-diagonal blocks stay zero for the whole kernel
+  if (ROWS == 64) for (int c = threadIdx.x; c < 65536 / 16; c += AU_THREADS) reinterpret_cast<uint4*>(p_s)[c] = make_uint4(0, 0, 0, 0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -177,21 +182,22 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
         if (pre < 1) load_v(0);
       }
     } else if (warp < 8) {
-      // Q rows of this CTA into the two K-major slabs, each row at r and at r + 64 (rows beyond cnt are zeros);
-      // a thread fetches its four pieces before it stores the first
-      uint4 v[4];
+      // Q rows of this CTA into the two K-major slabs, with 64 rows each row at r and at r + 64 (rows beyond cnt are
+      // zeros); a thread fetches its pieces before it stores the first
+      constexpr int PIECES = ROWS * (HD / 8) / 256;
+      uint4 v[PIECES];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < PIECES; ++k) {
         const int c = threadIdx.x + 256 * k, qr = c / (HD / 8), ch = c % (HD / 8);
         v[k] = make_uint4(0, 0, 0, 0);
         if (row0 + qr < cnt) v[k] = *reinterpret_cast<const uint4*>(a.q + (size_t)(b * R + row0 + qr) * H * HD + h * HD + ch * 8);
       }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < PIECES; ++k) {
         const int c = threadIdx.x + 256 * k, qr = c / (HD / 8), ch = c % (HD / 8);
         uint8_t* dst = q_s + (ch >> 3) * 16384 + qr * 128 + (((ch & 7) ^ (qr & 7)) << 4);   // (qr + 64) & 7 == qr & 7
         *reinterpret_cast<uint4*>(dst) = v[k];
-        *reinterpret_cast<uint4*>(dst + AU_ROWS * 128) = v[k];
+        if (ROWS == 64) *reinterpret_cast<uint4*>(dst + 64 * 128) = v[k];
       }
     }
   } else if (pre > 0 && threadIdx.x == 8 * 32) {
@@ -207,7 +213,8 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
   const int grp = warp >> 2;                                   // softmax group of warps 0..3 / 4..7
   const int q4 = warp & 3;                                     // SM quarter = tensor-memory lanes [32 q4, +32)
   const int mrow = q4 * 32 + lane;                             // this thread's MMA row (tensor-memory lane)
-  const int qrow = mrow & (AU_ROWS - 1), kh = mrow >> 6;       // its query row within the CTA and key half of every tile
+  const int qrow = mrow & (AU_ROWS - 1);                       // its query row within the CTA
+  const int kh = ROWS == 64 ? mrow >> 6 : 0;                   // 64 rows: its key half of every tile
   float m_ref = -INFINITY, l_run = 0.f;
   int my_tiles = 0;
   bool ok = true;
@@ -275,39 +282,18 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
 #pragma unroll
       for (int w = 0; w < 4; ++w) anc[w] = i_row < cnt ? a.rows.anc[i_row * 4 + w] : 0u;
       const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
-      for (int t = grp; t < nt; t += 2) {
+      // Raises the stream's reference to the tile's maximum `tmax` (unscaled) where it has to and returns what the sums so far
+      // are multiplied by; the group's previous tile must be through the tensor cores by then (its P operand and
+      // accumulator are reused), which is awaited here.
+      auto raise_reference = [&](float tmax, int t) -> float {
         const int bf = t & 1;
-        if (!mbar_wait(&s_full[bf], (t >> 1) & 1, a.status, 54)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t s_addr = tmem + lane_base + (uint32_t)(bf * 128 + kh * 64);
-        const int k0 = (sp + t * ncl) * AU_KT + kh * 64;       // first key of this thread's half
-        uint32_t r0[32], r1[32];
-        tmem_ld32(s_addr, r0);
-        tmem_ld32(s_addr + 32, r1);
-        uint32_t vis0 = 0xffffffffu, vis1 = 0xffffffffu;
-        if (k0 + 64 > n) {                                      // the half reaches into the tree rows or past the end
-          const unsigned long long v = attn_vis64(anc, k0, n);
-          vis0 = (uint32_t)v; vis1 = (uint32_t)(v >> 32);
-        }
-        tmem_ld_wait();
-        float tmax = -INFINITY;
-        if ((vis0 & vis1) == 0xffffffffu) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) tmax = fmaxf(tmax, fmaxf(__uint_as_float(r0[j]), __uint_as_float(r1[j])));
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if ((vis0 >> j) & 1u) tmax = fmaxf(tmax, __uint_as_float(r0[j]));
-            if ((vis1 >> j) & 1u) tmax = fmaxf(tmax, __uint_as_float(r1[j]));
-          }
-        }
         tmax *= a.scale_log2;
         // raise the reference only when it is too low by more than 2^AU_RESCALE_LOG2 (or not set yet)
         const bool raise = tmax > m_ref + AU_RESCALE_LOG2 || (m_ref == -INFINITY && tmax > -INFINITY);
         const float m_new = raise ? tmax : m_ref;
         const float alpha = raise ? exp2f(m_ref - m_new) : 1.f;   // 0 the first time
         // the group's previous tile must be through the tensor cores: its P operand and accumulator are reused
-        if (t >= 2 && !mbar_wait(&o_done[bf], ((t >> 1) - 1) & 1, a.status, 55)) { ok = false; break; }
+        if (t >= 2 && !mbar_wait(&o_done[bf], ((t >> 1) - 1) & 1, a.status, 55)) { ok = false; return 1.f; }
         if (__any_sync(0xffffffffu, raise && my_tiles > 0)) {
           // rescale this lane's accumulator row (other lanes of the warp multiply by one)
           tc_fence_after();
@@ -323,33 +309,120 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
           }
           tmem_st_wait();
         }
-        l_run *= alpha;
         m_ref = m_new;
-        const float base = (m_new == -INFINITY) ? 0.f : m_new;
-        // probabilities of this thread's 64 keys, rounded to bf16, into row `mrow` of slab `kh` of the P operand
-        float l0 = 0.f, l1 = 0.f;
-        uint8_t* p_row = p_s + bf * 32768 + kh * 16384 + mrow * 128;
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const uint32_t (&r)[32] = c ? r1 : r0;
-          const uint32_t vc = c ? vis1 : vis0;
-          uint32_t pk[16];
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            float p0 = exp2f(fmaf(__uint_as_float(r[j]), a.scale_log2, -base));
-            float p1 = exp2f(fmaf(__uint_as_float(r[j + 1]), a.scale_log2, -base));
-            if (!((vc >> j) & 1u)) p0 = 0.f;
-            if (!((vc >> (j + 1)) & 1u)) p1 = 0.f;
-            l0 += p0; l1 += p1;
-            pk[j >> 1] = pack_bf16(p0, p1);
+        return alpha;
+      };
+      for (int t = grp; t < nt; t += 2) {
+        const int bf = t & 1;
+        if (!mbar_wait(&s_full[bf], (t >> 1) & 1, a.status, 54)) { ok = false; break; }
+        tc_fence_after();
+        if constexpr (ROWS == 128) {
+          // a thread has all 128 keys of the tile: 32 scores at a time, read out of tensor memory once for the maximum and
+          // once for the probabilities (128 of them would not stay in registers)
+          const uint32_t s_addr = tmem + lane_base + (uint32_t)(bf * 128);
+          const int k0 = (sp + t * ncl) * AU_KT;
+          uint32_t vis[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
+          const bool whole = k0 + AU_KT <= n;                     // no tree row, nothing past the end
+          if (!whole) {
+            const unsigned long long v0 = attn_vis64(anc, k0, n), v1 = attn_vis64(anc, k0 + 64, n);
+            vis[0] = (uint32_t)v0; vis[1] = (uint32_t)(v0 >> 32); vis[2] = (uint32_t)v1; vis[3] = (uint32_t)(v1 >> 32);
           }
+          float tmax = -INFINITY;
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const int ch = c * 4 + g;
-            *reinterpret_cast<uint4*>(p_row + ((ch ^ (mrow & 7)) << 4)) = make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
+          for (int c = 0; c < 4; ++c) {
+            uint32_t r[32];
+            tmem_ld32(s_addr + c * 32, r);
+            tmem_ld_wait();
+            if (whole) {
+#pragma unroll
+              for (int j = 0; j < 32; ++j) tmax = fmaxf(tmax, __uint_as_float(r[j]));
+            } else {
+#pragma unroll
+              for (int j = 0; j < 32; ++j) if ((vis[c] >> j) & 1u) tmax = fmaxf(tmax, __uint_as_float(r[j]));
+            }
           }
+          const float alpha = raise_reference(tmax, t);
+          if (!ok) break;
+          const float base = (m_ref == -INFINITY) ? 0.f : m_ref;
+          l_run *= alpha;
+          uint8_t* p_row = p_s + bf * 32768 + mrow * 128;
+          float l0 = 0.f, l1 = 0.f;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            uint32_t r[32], pk[16];
+            tmem_ld32(s_addr + c * 32, r);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+              float p0 = exp2f(fmaf(__uint_as_float(r[j]), a.scale_log2, -base));
+              float p1 = exp2f(fmaf(__uint_as_float(r[j + 1]), a.scale_log2, -base));
+              if (!whole) {
+                if (!((vis[c] >> j) & 1u)) p0 = 0.f;
+                if (!((vis[c] >> (j + 1)) & 1u)) p1 = 0.f;
+              }
+              l0 += p0; l1 += p1;
+              pk[j >> 1] = pack_bf16(p0, p1);
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              const int ch = (c & 1) * 4 + g;
+              *reinterpret_cast<uint4*>(p_row + (c >> 1) * 16384 + ((ch ^ (mrow & 7)) << 4)) =
+                  make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
+            }
+          }
+          l_run += l0 + l1;
+        } else {
+          const uint32_t s_addr = tmem + lane_base + (uint32_t)(bf * 128 + kh * 64);
+          const int k0 = (sp + t * ncl) * AU_KT + kh * 64;       // first key of this thread's half
+          uint32_t r0[32], r1[32];
+          tmem_ld32(s_addr, r0);
+          tmem_ld32(s_addr + 32, r1);
+          uint32_t vis0 = 0xffffffffu, vis1 = 0xffffffffu;
+          if (k0 + 64 > n) {                                      // the half reaches into the tree rows or past the end
+            const unsigned long long v = attn_vis64(anc, k0, n);
+            vis0 = (uint32_t)v; vis1 = (uint32_t)(v >> 32);
+          }
+          tmem_ld_wait();
+          float tmax = -INFINITY;
+          if ((vis0 & vis1) == 0xffffffffu) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) tmax = fmaxf(tmax, fmaxf(__uint_as_float(r0[j]), __uint_as_float(r1[j])));
+          } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              if ((vis0 >> j) & 1u) tmax = fmaxf(tmax, __uint_as_float(r0[j]));
+              if ((vis1 >> j) & 1u) tmax = fmaxf(tmax, __uint_as_float(r1[j]));
+            }
+          }
+          const float alpha = raise_reference(tmax, t);
+          if (!ok) break;
+          l_run *= alpha;
+          const float base = (m_ref == -INFINITY) ? 0.f : m_ref;
+          // probabilities of this thread's 64 keys, rounded to bf16, into row `mrow` of slab `kh` of the P operand
+          float l0 = 0.f, l1 = 0.f;
+          uint8_t* p_row = p_s + bf * 32768 + kh * 16384 + mrow * 128;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const uint32_t (&r)[32] = c ? r1 : r0;
+            const uint32_t vc = c ? vis1 : vis0;
+            uint32_t pk[16];
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+              float p0 = exp2f(fmaf(__uint_as_float(r[j]), a.scale_log2, -base));
+              float p1 = exp2f(fmaf(__uint_as_float(r[j + 1]), a.scale_log2, -base));
+              if (!((vc >> j) & 1u)) p0 = 0.f;
+              if (!((vc >> (j + 1)) & 1u)) p1 = 0.f;
+              l0 += p0; l1 += p1;
+              pk[j >> 1] = pack_bf16(p0, p1);
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              const int ch = c * 4 + g;
+              *reinterpret_cast<uint4*>(p_row + ((ch ^ (mrow & 7)) << 4)) = make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
+            }
+          }
+          l_run += l0 + l1;
         }
-        l_run += l0 + l1;
         ++my_tiles;
         fence_proxy_async_smem();
         tc_fence_before();
@@ -368,13 +441,13 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
     if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem, 512); }
     return;
   }
-  // ---- the four streams of a query row (two groups x two key halves), staged in shared memory ----
-  float* ex = reinterpret_cast<float*>(sm);                    // [4 streams][64 rows][AU_EXP]; stream 0 becomes the CTA's partial
-  float* ml = ex + 4 * AU_ROWS * AU_EXP;                       // [4 streams][64 rows] (reference, sum)
-  float* cml = ml + 4 * AU_ROWS * 2;                           // [64 rows] of the CTA's partial
+  // ---- the streams of a query row (two groups, with 64 rows times two key halves), staged in shared memory ----
+  float* ex = reinterpret_cast<float*>(sm);                    // [STREAMS][ROWS][AU_EXP]; stream 0 becomes the CTA's partial
+  float* ml = ex + STREAMS * AU_ROWS * AU_EXP;                 // [STREAMS][ROWS] (reference, sum)
+  float* cml = ml + STREAMS * AU_ROWS * 2;                     // [ROWS] of the CTA's partial
   const bool work = active && ok;
   if (warp < 8) {
-    const int sid = grp * 2 + kh;
+    const int sid = ROWS == 64 ? grp * 2 + kh : grp;
     float* my = ex + ((size_t)sid * AU_ROWS + qrow) * AU_EXP;
     tc_fence_after();
     if (work && my_tiles > 0) {
@@ -399,11 +472,11 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
   __syncthreads();
   if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem, 512); }
   if (warp < 8) {
-    // thread = (row, every fourth 4-dim chunk): merge the four streams
-    const int row = threadIdx.x >> 2, qd = threadIdx.x & 3;
-    float ms[4], ls[4], mm = -INFINITY;
+    // thread = (row, every STREAMS-th 4-dim chunk): merge the streams
+    const int row = threadIdx.x / STREAMS, qd = threadIdx.x % STREAMS;
+    float ms[STREAMS], ls[STREAMS], mm = -INFINITY;
 #pragma unroll
-    for (int s2 = 0; s2 < 4; ++s2) {
+    for (int s2 = 0; s2 < STREAMS; ++s2) {
       const float2 v = *reinterpret_cast<const float2*>(ml + ((size_t)s2 * AU_ROWS + row) * 2);
       ms[s2] = v.x; ls[s2] = v.y;
       mm = fmaxf(mm, v.x);
@@ -411,16 +484,16 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
     const float base = (mm == -INFINITY) ? 0.f : mm;
     float L = 0.f;
 #pragma unroll
-    for (int s2 = 0; s2 < 4; ++s2) { ms[s2] = exp2f(ms[s2] - base); L += ms[s2] * ls[s2]; }
+    for (int s2 = 0; s2 < STREAMS; ++s2) { ms[s2] = exp2f(ms[s2] - base); L += ms[s2] * ls[s2]; }
     const float inv = 1.f / L;
     const size_t m = (size_t)b * R + row0 + row;
     const bool valid = row0 + row < cnt;
 #pragma unroll
-    for (int j = 0; j < HD / 16; ++j) {
-      const int d = (j * 4 + qd) * 4;
+    for (int j = 0; j < HD / (4 * STREAMS); ++j) {
+      const int d = (j * STREAMS + qd) * 4;
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int s2 = 0; s2 < 4; ++s2) {
+      for (int s2 = 0; s2 < STREAMS; ++s2) {
         const float4 v = *reinterpret_cast<const float4*>(ex + ((size_t)s2 * AU_ROWS + row) * AU_EXP + d);
         acc.x += ms[s2] * v.x; acc.y += ms[s2] * v.y; acc.z += ms[s2] * v.z; acc.w += ms[s2] * v.w;
       }

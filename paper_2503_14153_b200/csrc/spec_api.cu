@@ -781,7 +781,10 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
   const int nw = (R + 15) / 16;
   if (attn_long_mode(c, R, B, tiles_hi * 64) && c->attn_umma && c->tm_kv_ok && D == 128) {
     // long contexts: scores and P V on tcgen05, a CTA per (head, 64 rows, key split)
-    const int halves = (R + AU_ROWS - 1) / AU_ROWS;
+    // passes of more than 64 rows (prompt chunks, trees of up to 128 nodes): a CTA takes 128 rows and reads the keys once for
+    // them; 64 rows or fewer fill the 128-row MMAs twice, with two halves of the keys
+    const bool tall = R > 64;
+    const int halves = tall ? (R + 127) / 128 : 1;
     if (B <= ATTN_MAX_SEQS) {
       int idx[ATTN_MAX_SEQS];
       for (int b = 0; b < B; ++b) idx[b] = b;
@@ -794,7 +797,11 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     static bool set_dev[kAttrDevices] = {};
     bool& set_ = *attr_flag(set_dev);
-    if (!set_) { CUDA_OK(cudaFuncSetAttribute(attention_umma<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_umma_smem())); set_ = true; }
+    if (!set_) {
+      CUDA_OK(cudaFuncSetAttribute(attention_umma<128, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_umma_smem()));
+      CUDA_OK(cudaFuncSetAttribute(attention_umma<128, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_umma_smem()));
+      set_ = true;
+    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = dim3(AU_THREADS); cfg.dynamicSmemBytes = attention_umma_smem(); cfg.stream = c->stream;
     cudaLaunchAttribute at[2];
@@ -810,7 +817,7 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
       ++n_at;
     }
     cfg.attrs = at; cfg.numAttrs = (unsigned)n_at;
-    cudaError_t e_ = cudaLaunchKernelEx(&cfg, attention_umma<128>, c->tm_kv, a, c->next_trace("attention_tc"));
+    cudaError_t e_ = cudaLaunchKernelEx(&cfg, tall ? attention_umma<128, 128> : attention_umma<128, 64>, c->tm_kv, a, c->next_trace("attention_tc"));
     c->launches++;
     if (e_ != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("attention_umma: ") + cudaGetErrorString(e_));
     return SPEC_OK;
