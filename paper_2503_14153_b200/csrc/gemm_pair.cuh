@@ -8,9 +8,14 @@
 // Why pairs: a 64-wide K chunk of a 128 x 256 tile in one CTA writes 48 KB into shared memory and reads 48 KB out
 // of it in the 512 cycles its MMAs take at full rate, 192 bytes per cycle where an SM moves 128; the pair's chunk
 // is 32 KB in and 32 KB out per CTA, 128 bytes per cycle. Two accumulators of NT tensor-memory columns alternate, so
-// that the epilogue of one tile runs under the MMAs of the next. No split K. Persistent: cluster c takes tiles
+// that the epilogue of one tile runs under the MMAs of the next. Persistent: cluster c takes tiles
 // c, c + clusters, ...; tile = weight pair * m_tiles + activation tile, so the clusters that share weights run side
-// by side and the weights cross HBM once.
+// by side and the weights cross HBM once. Where there are tiles for less than half of the clusters (a 256-row pass has
+// 16 tiles of an output projection for 74 clusters), every tile's K chunks are dealt to `parts` clusters: each leaves float32
+// partial sums, and the CTA of a tile that arrives last (arrival counter, nobody waits) adds them in order, so that the sum
+// does not depend on who that is, and does the tile's epilogue. (Dealing the last wave's tiles to all clusters where whole
+// tiles leave some of them idle does not pay: the clusters share the L2's bandwidth, so that fewer of them run faster; at 2048
+// rows the output and down projections took 184 us instead of 120.)
 //
 // Modes:
 //  * GP_PLAIN     float32 sums to out[m][ld] (columns below n_cols only)
@@ -46,6 +51,9 @@ struct PairGemmParams {
   int n_mats;
   int mat_tile0[GS_MAX_MATS + 1];           // first 128-row weight tile of each stacked matrix
   int n_tiles, w_pairs, m_tiles;            // weight tiles (all matrices), pairs of them, activation tiles of NT rows
+  int parts;                                // clusters that share a tile's K chunks (1: tiles are whole)
+  float* part;                              // parts > 1: [tile][part][CTA of the pair][NT][128] float32
+  unsigned int* arrive;                     // parts > 1: [tile][CTA of the pair], zero between launches
   int packed;                               // 1: the tensor maps view pre-tiled images, 0: row-major matrices
   int n_cols;                               // GP_PLAIN: columns stored; GP_RESIDUAL / GP_SWIGLU: weight rows of one matrix
   size_t ld;                                // GP_PLAIN: row pitch of out
@@ -107,12 +115,12 @@ __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const void* tma
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
-// Barriers of one half's four epilogue warps; group_and also tells whether `v` holds in all of them.
+// Barrier of one half's four epilogue warps; epilogue_and: of all eight, telling whether `v` holds in all of their threads.
 __device__ __forceinline__ void group_bar(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
-__device__ __forceinline__ bool group_and(int id, bool v) {
+__device__ __forceinline__ bool epilogue_and(bool v) {
   uint32_t r;
-  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %2, 0;\n\tbar.red.and.pred q, %1, 128, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
-               : "=r"(r) : "r"(id), "r"((uint32_t)v) : "memory");
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.and.pred q, 3, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"((uint32_t)v) : "memory");
   return r != 0;
 }
 
@@ -137,14 +145,18 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   uint64_t* acc_full = bars + 2 * STAGES;   // each CTA's
   uint64_t* acc_empty = bars + 2 * STAGES + 2;   // leader's: drained by the eight warps of both CTAs
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
+  volatile uint32_t* last_slot = reinterpret_cast<volatile uint32_t*>(bars + 2 * STAGES + 5);   // this CTA completes a split tile
 
   KTrace kt(p.trace);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
   const int KC = p.KC;
-  const int total_tiles = p.w_pairs * p.m_tiles;
-  const int my_tiles = cl < total_tiles ? (total_tiles - 1 - cl) / ncl + 1 : 0;
+  // this cluster's work: tiles cl, cl + ncl, ..., or with parts > 1 one part of one tile
+  const int total_tiles = p.w_pairs * p.m_tiles, parts = p.parts;
+  const int my_tiles = cl < total_tiles * parts ? (parts > 1 ? 1 : (total_tiles - 1 - cl) / ncl + 1) : 0;
+  const int k_lo = parts > 1 ? cl % parts * KC / parts : 0, k_hi = parts > 1 ? (cl % parts + 1) * KC / parts : KC;
+  auto tile_of = [&](int i) { return parts > 1 ? cl / parts : cl + i * ncl; };
 
   pdl_launch_dependents();
 
@@ -177,10 +189,10 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       // ---- producer: this CTA's weight rows and its half of the activation rows ----
       struct At { int i, kc, wp, mt; };
       auto at_tile = [&](At& a) {
-        const int tau = cl + a.i * ncl;
+        const int tau = tile_of(a.i);
         a.wp = tau / p.m_tiles; a.mt = tau - a.wp * p.m_tiles;
       };
-      auto next = [&](At& a) { if (++a.kc == KC) { a.kc = 0; ++a.i; at_tile(a); } };
+      auto next = [&](At& a) { if (++a.kc == k_hi) { a.kc = k_lo; ++a.i; at_tile(a); } };
       auto load_a = [&](uint8_t* dst, const At& a, uint32_t bar) {
         if (MODE == GP_SWIGLU) {
           const int row = (p.packed ? (a.wp * KC + a.kc) * 128 : a.wp * 128) + rank * 64, x = p.packed ? 0 : a.kc * Cfg::BK;
@@ -194,10 +206,10 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       auto load_b = [&](uint8_t* dst, const At& a, uint32_t bar) {
         tma_load_2d_pair(dst, &tm.b, a.kc * Cfg::BK, a.mt * NT + rank * (NT / 2), bar);
       };
-      const int n_units = my_tiles * KC;
+      const int n_units = my_tiles * (k_hi - k_lo);
       const int n_pre = n_units < STAGES ? n_units : STAGES;
       const uint32_t full0 = dsmem_addr(smem_u32(full), 0);            // the leader's barriers
-      At a{0, 0, 0, 0};
+      At a{0, k_lo, 0, 0};
       at_tile(a);
       At b = a;
       // weights do not depend on the kernel before this one
@@ -235,16 +247,16 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         if (!mbar_wait(&acc_empty[buf], ((i >> 1) & 1) ^ 1, p.status, 44)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_addr = tmem_base + (uint32_t)(buf * NT);
-        for (int kc = 0; kc < KC; ++kc) {
+        for (int kc = k_lo; kc < k_hi; ++kc) {
           if (!mbar_wait(&full[st], ph, p.status, 41)) { ok = false; break; }
-          if (i == 0 && kc == 0) trace_mark_min(p.trace, 2);
+          if (i == 0 && kc == k_lo) trace_mark_min(p.trace, 2);
           tc_fence_after();
           const uint32_t a_addr = smem_u32(tiles + st * Cfg::STAGE_BYTES);
           const uint64_t adesc = make_kmajor_sw128_desc(a_addr);
           const uint64_t bdesc = make_kmajor_sw128_desc(a_addr + Cfg::A_BYTES);
 #pragma unroll
           for (int k = 0; k < Cfg::BK / 16; ++k)
-            tc_mma_f16_pair(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kc > 0 || k > 0) ? 1u : 0u);
+            tc_mma_f16_pair(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kc > k_lo || k > 0) ? 1u : 0u);
           tc_commit_pair(&empty[st]);
           if (++st == STAGES) { st = 0; ph ^= 1; }
         }
@@ -263,24 +275,108 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
     pdl_wait();
     for (int i = 0; i < my_tiles; ++i) {
       const int buf = i & 1;
-      const int tau = cl + i * ncl;
+      const int tau = tile_of(i);
       const int wp = tau / p.m_tiles, mt = tau - wp * p.m_tiles;
       const int nt = 2 * wp + rank;
       const int m0 = mt * NT + hf * HC;                       // this warp's first activation row
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * NT + hf * HC);
-      bool fine;
+      const bool split = parts > 1;
+      // (what the epilogue needs besides the sums is fetched while the tile's MMAs run)
+      // GP_RESIDUAL: old values of the first rows
+      float xo[2][32];
+      const int rcol = nt * 128 + wl;
+      const bool ron = MODE == GP_RESIDUAL && nt < p.n_tiles && rcol < p.n_cols;
+      auto fetch_x = [&](int g, float (&v)[32]) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int m = m0 + g * 32 + j;
+          v[j] = (ron && m < p.M) ? p.out[(size_t)m * p.n_cols + rcol] : 0.f;
+        }
+      };
+      if (MODE == GP_RESIDUAL && !split) fetch_x(0, xo[0]);
+      // GP_ROPE: the rows' positions and cache slots
+      PairRowMeta* mrow = meta + hf * HC;
+      if (MODE == GP_ROPE) {
+        const int e = threadIdx.x - 64 - hf * 128;
+        group_bar(1 + hf);                                     // everybody is through with the previous tile's rows
+        if (e < HC) {
+          PairRowMeta v{-1, 0, 0};
+          const int m = m0 + e;
+          if (m < p.M) {
+            const int b = m / p.rows.R, ri = m - b * p.rows.R;
+            if (ri < p.rows.cnt[b]) {
+              const int slot = p.rows.slot[m];
+              const int page = p.page_table[p.rows.sequence(b) * p.g.pages_per_seq + slot / p.g.page_size];
+              v.prow = slot % p.g.page_size;
+              v.pos = p.rows.pos[m];
+              v.kv = (long long)page * 2 * (long long)p.g.block_elems() + (long long)v.prow * p.g.head_dim;
+            }
+          }
+          mrow[e] = v;
+        }
+        group_bar(1 + hf);
+      }
+      // (all eight warps give up when one of them does: barriers follow)
+      if (!epilogue_and(mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42))) break;
+      tc_fence_after();
+      // partial sums of this warp's rows, part k at parts_at + k * PART
+      constexpr size_t PART = (size_t)2 * NT * 128;
+      const float* parts_at = p.part + ((size_t)tau * parts * 2 + rank) * (NT * 128) + (size_t)hf * HC * 128 + wl;
+      if (split) {
+        float* mine = const_cast<float*>(parts_at) + (cl % parts) * PART;
+#pragma unroll 1
+        for (int g = 0; g < HC / 32; ++g) {
+          uint32_t r[32];
+          tmem_ld32(taddr + g * 32, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) __stcg(mine + (g * 32 + j) * 128, __uint_as_float(r[j]));
+        }
+        tc_fence_before();
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);
+        asm volatile("bar.sync 3, 256;" ::: "memory");        // every warp's part precedes the arrival
+        if (threadIdx.x == 64) {
+          unsigned int* ctr = p.arrive + 2 * tau + rank;
+          const bool last = atomicAdd(ctr, 1u) == (unsigned)(parts - 1);
+          if (last) *ctr = 0u;
+          *last_slot = last;
+        }
+        asm volatile("bar.sync 3, 256;" ::: "memory");
+        const bool last = *last_slot != 0;
+        asm volatile("bar.sync 3, 256;" ::: "memory");        // everybody has read it
+        if (!last) continue;
+        __threadfence();
+        if (MODE == GP_RESIDUAL) fetch_x(0, xo[0]);
+      }
+      // sums of this thread's weight row for activation rows [g * 32, +32) of the warp's half
+      auto acc = [&](int g, uint32_t (&r)[32]) {
+        if (!split) {
+          tmem_ld32(taddr + g * 32, r);
+          tmem_ld_wait();
+          return;
+        }
+        const float* src = parts_at + g * 32 * 128;
+        float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = __ldcg(src + j * 128);
+        for (int k = 1; k < parts; ++k) {
+          src += PART;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] += __ldcg(src + j * 128);
+        }
+#pragma unroll
+        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(v[j]);
+      };
       if (MODE == GP_PLAIN) {
-        fine = mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42);
-        if (!fine) break;
-        tc_fence_after();
         const int col = nt * 128 + wl;
         float* dst = p.out + col;
         const bool on = nt < p.n_tiles && col < p.n_cols;
 #pragma unroll 2
         for (int g = 0; g < HC / 32; ++g) {
           uint32_t r[32];
-          tmem_ld32(taddr + g * 32, r);
-          tmem_ld_wait();
+          acc(g, r);
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const int m = m0 + g * 32 + j;
@@ -288,32 +384,17 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           }
         }
       } else if (MODE == GP_RESIDUAL) {
-        // old values of the next 32 rows are fetched while 32 rows are finished, the first ones under the MMAs
-        const int col = nt * 128 + wl;
-        const bool on = nt < p.n_tiles && col < p.n_cols;
-        float* dst = p.out + col;
-        float xo[2][32];
-        auto fetch = [&](int g, float (&v)[32]) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int m = m0 + g * 32 + j;
-            v[j] = (on && m < p.M) ? dst[(size_t)m * p.n_cols] : 0.f;
-          }
-        };
-        fetch(0, xo[0]);
-        fine = mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42);
-        if (!fine) break;
-        tc_fence_after();
+        // old values of the next 32 rows are fetched while 32 rows are finished
+        float* dst = p.out + rcol;
 #pragma unroll
         for (int g = 0; g < HC / 32; ++g) {
           uint32_t r[32];
-          tmem_ld32(taddr + g * 32, r);
-          if (g + 1 < HC / 32) fetch(g + 1, xo[(g + 1) & 1]);
-          tmem_ld_wait();
+          if (g + 1 < HC / 32) fetch_x(g + 1, xo[(g + 1) & 1]);
+          acc(g, r);
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const int m = m0 + g * 32 + j;
-            if (on && m < p.M) dst[(size_t)m * p.n_cols] = xo[g & 1][j] + __uint_as_float(r[j]);
+            if (ron && m < p.M) dst[(size_t)m * p.n_cols] = xo[g & 1][j] + __uint_as_float(r[j]);
           }
         }
       } else {
@@ -326,39 +407,13 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         const int pr = hp == 64 ? (wl & 63) : ((wl & 31) | ((wl >> 6) << 5));   // pair 0..63
         float* ex_lo = exch + hf * (2 * 64 * Cfg::EX_COLS);      // written by the lower rows' threads
         float* ex_up = ex_lo + 64 * Cfg::EX_COLS;
-        PairRowMeta* mrow = meta + hf * HC;
-        const int e = threadIdx.x - 64 - hf * 128;
-        if (MODE == GP_ROPE) {
-          group_bar(1 + hf);                                     // everybody is through with the previous tile's rows
-          if (e < HC) {
-            PairRowMeta v{-1, 0, 0};
-            const int m = m0 + e;
-            if (m < p.M) {
-              const int b = m / p.rows.R, ri = m - b * p.rows.R;
-              if (ri < p.rows.cnt[b]) {
-                const int slot = p.rows.slot[m];
-                const int page = p.page_table[p.rows.sequence(b) * p.g.pages_per_seq + slot / p.g.page_size];
-                v.prow = slot % p.g.page_size;
-                v.pos = p.rows.pos[m];
-                v.kv = (long long)page * 2 * (long long)p.g.block_elems() + (long long)v.prow * D;
-              }
-            }
-            mrow[e] = v;
-          }
-          group_bar(1 + hf);
-        }
-        fine = mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42);
-        // (the group stays together: all of its threads give up when one of them does)
-        if (!group_and(1 + hf, fine)) break;
-        tc_fence_after();
         if (MODE == GP_SWIGLU) {
           const int col = nt * 64 + pr;
           const bool on = col < p.n_cols;
 #pragma unroll 1
           for (int g = 0; g < HC / 32; ++g) {
             uint32_t r[32];
-            tmem_ld32(taddr + g * 32, r);
-            tmem_ld_wait();
+            acc(g, r);
             if (g) group_bar(1 + hf);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
@@ -387,8 +442,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
 #pragma unroll 1
             for (int g = 0; g < HC / 32; ++g) {
               uint32_t r[32];
-              tmem_ld32(taddr + g * 32, r);
-              tmem_ld_wait();
+              acc(g, r);
 #pragma unroll
               for (int j = 0; j < 32; ++j) {
                 const PairRowMeta v = mrow[g * 32 + j];
@@ -400,7 +454,6 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
 #pragma unroll 1
             for (int g = 0; g < HC / 32; ++g) {
               uint32_t r[32];
-              tmem_ld32(taddr + g * 32, r);
               const int jb = g * 32 + (lower ? 0 : 16);
               float2 t[16];
 #pragma unroll
@@ -408,7 +461,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
                 const PairRowMeta v = mrow[jb + j];
                 t[j] = p.cs[(size_t)v.pos * half + di];          // (position 0 for rows not in use)
               }
-              tmem_ld_wait();
+              acc(g, r);
               if (g) group_bar(1 + hf);
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
@@ -440,6 +493,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           }
         }
       }
+      if (split) continue;                                    // (its accumulator was given back above)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);

@@ -48,6 +48,12 @@ constexpr int ATTN_SPLIT_TILES = 8;       // fewest KV tiles a split of attentio
 constexpr int ATTN_SINGLE_TILES = 12;   // contexts of at most this many 64-key tiles use one KV split
 constexpr int ATTN_LONG_KEYS = 2048;    // default context length from which passes of more than 32 rows use the shared-K/V kernel
 
+constexpr int GP_NT = 256;              // activation rows per tile of the many-row projection kernel
+constexpr int GP_MAX_CLUSTERS = SM_SLOTS / 4;   // its clusters: two CTAs each, one CTA per SM
+constexpr int GP_SPLIT_KC = 64;         // see pair_parts
+constexpr size_t GP_PART_FLOATS = (size_t)GP_MAX_CLUSTERS * 2 * GP_NT * 128;   // a part of a tile per cluster
+constexpr int GP_ARRIVE = GP_MAX_CLUSTERS;   // at most half as many shared tiles as clusters, two CTAs each
+
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -244,6 +250,7 @@ struct spec_ctx {
   bool trace_on = false;
   unsigned long long* d_trace = nullptr;
   unsigned int* d_attn_arrive = nullptr;
+  unsigned int* d_pair_arrive = nullptr;  // [GP_ARRIVE] arrival counters of the split tiles, zero between launches
   unsigned int* d_row_arrive = nullptr;   // [Mcap] arrival counters of the per-row finishing steps, zero between launches
   float* d_pval2 = nullptr;            // finished per-row argmax (tensor-core path)
   int* d_pidx2 = nullptr;
@@ -378,6 +385,7 @@ size_t carve(spec_ctx* c, void* base) {
   c->d_trace = b.take<unsigned long long>((size_t)TRACE_CAP * 4);
   c->d_attn_arrive = b.take<unsigned int>((size_t)c->chunk_cap * f.n_heads * 2);
   c->d_row_arrive = b.take<unsigned int>(c->Mcap);
+  c->d_pair_arrive = b.take<unsigned int>(GP_ARRIVE);
   c->d_pval2 = b.take<float>(c->Mcap); c->d_pidx2 = b.take<int>(c->Mcap);
   c->d_draws = b.take<int>(B);
   c->d_cnt = b.take<int>(B); c->d_n_old = b.take<int>(B); c->d_root = b.take<int>(B);
@@ -417,6 +425,8 @@ size_t carve(spec_ctx* c, void* base) {
       }
     }
   }
+  // (split tiles of the many-row projections leave their partial sums here too)
+  if (c->tc && c->Mcap > 128 && std::max(d, std::max(HD, F)) >= 64 * GP_SPLIT_KC) pf = std::max(pf, GP_PART_FLOATS);
   c->part_floats = pf;
   c->d_part = b.take<float>(pf, 1024);
   c->d_logits = c->keep_logits ? b.take<float>((size_t)Mlog * V, 1024) : nullptr;
@@ -509,13 +519,20 @@ int aligned_ctas(int n_tiles, int cap) {
 }
 
 // ---- many rows: the two-SM kernel, the step after the projection in its epilogue ----
-constexpr int GP_NT = 256;            // activation rows per tile
-constexpr int GP_MAX_CLUSTERS = SM_SLOTS / 4;   // one CTA per SM, two CTAs per cluster
-
 bool pair_gemm_ok(const spec_ctx* c, int M, int K) { return c->wide_gemm && M > 128 && K % 64 == 0; }
 
+// Clusters that share each tile of a launch (PairGemmParams::parts): as many as there are for it where the tiles employ less than
+// half of the clusters, at most four, eight for a long inner dimension (the CTA that finishes a tile adds the parts up, about
+// 1 us each). A tile of fewer than GP_SPLIT_KC chunks is short (16 chunks: 6 us) and the exchange takes most of what
+// sharing saves; it stays whole and keeps one order of the sums for every number of rows.
+int pair_parts(int tiles, int KC, int clusters) {
+  if (KC < GP_SPLIT_KC || tiles * 2 > clusters) return 1;
+  return std::min(clusters / tiles, KC >= 2 * GP_SPLIT_KC ? 8 : 4);
+}
+
 template <int MODE>
-cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, const PairGemmParams& p, int max_clusters = GP_MAX_CLUSTERS) {
+cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemmParams p, float* part, unsigned int* arrive,
+                      int max_clusters = GP_MAX_CLUSTERS) {
   static bool attr_set_dev[kAttrDevices] = {};
   bool& attr_set = *attr_flag(attr_set_dev);
   if (!attr_set) {
@@ -523,7 +540,11 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, const Pa
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  const int grid = 2 * std::min(p.w_pairs * p.m_tiles, std::min(GP_MAX_CLUSTERS, max_clusters));
+  const int clusters = std::min(GP_MAX_CLUSTERS, max_clusters);
+  const int tiles = p.w_pairs * p.m_tiles;
+  p.parts = part && arrive ? pair_parts(tiles, p.KC, clusters) : 1;
+  p.part = part; p.arrive = arrive;
+  const int grid = 2 * (p.parts > 1 ? tiles * p.parts : std::min(tiles, clusters));
   return launch_k(pdl, gemm_pair<MODE, GP_NT>, dim3(grid), dim3(GP_THREADS), (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
 }
 
@@ -551,13 +572,14 @@ int run_gemm_pair(spec_ctx* c, int mode, const void* x, int M, int K, int n_mats
   tm.b = *tb;
   w->status = c->d_status; w->trace = c->next_trace(gemm_kind_name(kind));
   cudaError_t e;
+  float* part = c->part_floats >= GP_PART_FLOATS ? c->d_part : nullptr;
   {
     ProfScope ps(c, kind);
     switch (mode) {
-      case GP_RESIDUAL: e = launch_gp<GP_RESIDUAL>(c->stream, c->pdl, tm, *w); break;
-      case GP_SWIGLU: e = launch_gp<GP_SWIGLU>(c->stream, c->pdl, tm, *w); break;
-      case GP_ROPE: e = launch_gp<GP_ROPE>(c->stream, c->pdl, tm, *w); break;
-      default: e = launch_gp<GP_PLAIN>(c->stream, c->pdl, tm, *w); break;
+      case GP_RESIDUAL: e = launch_gp<GP_RESIDUAL>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
+      case GP_SWIGLU: e = launch_gp<GP_SWIGLU>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
+      case GP_ROPE: e = launch_gp<GP_ROPE>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
+      default: e = launch_gp<GP_PLAIN>(c->stream, c->pdl, tm, *w, nullptr, nullptr);   // (writes the scratch itself) break;
     }
     c->launches++;
   }
@@ -1173,6 +1195,7 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   CUDA_OK(cudaMemsetAsync(c->d_pool, 0, (size_t)f.max_batch * c->pages_per_seq * c->geom.page_elems() * c->esz, c->stream));
   CUDA_OK(cudaMemcpyAsync(c->d_prompt, tokens + offsets[0], (size_t)off[batch] * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_OK(cudaMemcpyAsync(c->d_offsets, off.data(), (batch + 1) * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  CUDA_OK(cudaMemsetAsync(c->d_pair_arrive, 0, GP_ARRIVE * sizeof(unsigned int), c->stream));   // (a wait that ran out may have left some set)
   CUDA_OK(cudaMemsetAsync(c->d_gen_cnt, 0, batch * sizeof(int), c->stream));
   CUDA_OK(cudaMemsetAsync(c->d_draws, 0, batch * sizeof(int), c->stream));
   // The prompts are cut into chunks of R tokens and the chunks of all prompts, one prompt after another, are dealt to as
@@ -1802,7 +1825,11 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     for (int i = 1; i <= GS_MAX_MATS; ++i) p.mat_tile0[i] = p.n_tiles;
     p.out = y; p.ld = (size_t)N; p.n_cols = N;
     p.status = reinterpret_cast<int*>(scratch + scratch_floats);
-    if (cudaMemsetAsync(p.status, 0, 16, st) != cudaSuccess || launch_gp<GP_PLAIN>(st, false, tm, p, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
+    // partial sums of split tiles at the start of the scratch where it is large enough, arrival counters before the status word
+    const bool room = scratch_floats >= GP_PART_FLOATS + GP_ARRIVE;
+    unsigned int* arrive = room ? reinterpret_cast<unsigned int*>(p.status) - GP_ARRIVE : nullptr;
+    if (cudaMemsetAsync(room ? (void*)arrive : (void*)p.status, 0, 16 + (room ? GP_ARRIVE * 4 : 0), st) != cudaSuccess ||
+        launch_gp<GP_PLAIN>(st, false, tm, p, room ? scratch : nullptr, arrive, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
     return op_linear_status(p.status, st);
   }
   if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, g.MT)) return SPEC_E_CUDA;

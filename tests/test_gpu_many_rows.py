@@ -77,7 +77,11 @@ def test_prompts_in_chunks_vs_oracle(torch, hd, lengths):
 
 
 @pytest.mark.parametrize("M,N,K,ctas", [(144, 128, 64, 1), (272, 300, 64, 2), (1008, 1000, 704, 148), (2048, 129, 128, 296),
-                                        (512, 4096, 4096, 7)])
+                                        (512, 4096, 4096, 7),
+                                        # inner dimensions long enough to split the last tiles between clusters: four equal parts
+                                        # a tile, few tiles with eight parts, runs that cross tiles, runs longer than a tile
+                                        (256, 4096, 4096, 296), (272, 300, 8192, 296), (512, 5000, 4096, 296),
+                                        (1008, 11008, 4096, 296)])
 def test_op_linear_many_rows(torch, M, N, K, ctas):
     """More than 128 rows of the stand-alone projection: one weight tile (computed by both SMs of a pair, stored once), ragged
     columns and activation tiles, more tiles than CTA pairs. Bound: K accumulations in float32, each off by at most one
