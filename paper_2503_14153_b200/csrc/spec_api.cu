@@ -1207,7 +1207,11 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   std::vector<int> cseq, cpos;
   for (int b = 0; b < batch; ++b)
     for (int p = 0; p < off[b + 1] - off[b]; p += R) { cseq.push_back(b); cpos.push_back(p); }
-  const int chunks = (int)cseq.size(), passes = (chunks + cap - 1) / cap;
+  const int chunks = (int)cseq.size();
+  // A lone prompt of two chunks goes chunk by chunk, through the projections that stream the weights: on the 7B shape that takes
+  // 8.5 ms instead of 7.1, the weights being read twice, but in the order of sums that the prompt of one chunk and the
+  // verification steps have, so that a short prompt's first tokens do not depend on which side of 128 its length lies.
+  const int passes = batch == 1 && chunks == 2 ? 2 : (chunks + cap - 1) / cap;
   CUDA_OK(cudaMemcpyAsync(c->d_chunk_seq, cseq.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_OK(cudaMemcpyAsync(c->d_chunk_pos, cpos.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_OK(cudaStreamSynchronize(c->stream));   // the host staging vectors go out of scope
