@@ -129,7 +129,8 @@ struct PairRowMeta {
   int pos, prow;
 };
 
-template <int MODE, int NT>
+// SPLIT: p.parts > 1.
+template <int MODE, int NT, bool SPLIT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
 gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   using Cfg = PairCfg<NT>;
@@ -153,10 +154,10 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
   const int KC = p.KC;
   // this cluster's work: tiles cl, cl + ncl, ..., or with parts > 1 one part of one tile
-  const int total_tiles = p.w_pairs * p.m_tiles, parts = p.parts;
-  const int my_tiles = cl < total_tiles * parts ? (parts > 1 ? 1 : (total_tiles - 1 - cl) / ncl + 1) : 0;
-  const int k_lo = parts > 1 ? cl % parts * KC / parts : 0, k_hi = parts > 1 ? (cl % parts + 1) * KC / parts : KC;
-  auto tile_of = [&](int i) { return parts > 1 ? cl / parts : cl + i * ncl; };
+  const int total_tiles = p.w_pairs * p.m_tiles, parts = SPLIT ? p.parts : 1;
+  const int my_tiles = cl < total_tiles * parts ? (SPLIT ? 1 : (total_tiles - 1 - cl) / ncl + 1) : 0;
+  const int k_lo = SPLIT ? cl % parts * KC / parts : 0, k_hi = SPLIT ? (cl % parts + 1) * KC / parts : KC;
+  auto tile_of = [&](int i) { return SPLIT ? cl / parts : cl + i * ncl; };
 
   pdl_launch_dependents();
 
@@ -280,7 +281,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       const int nt = 2 * wp + rank;
       const int m0 = mt * NT + hf * HC;                       // this warp's first activation row
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * NT + hf * HC);
-      const bool split = parts > 1;
+      constexpr bool split = SPLIT;
       // (what the epilogue needs besides the sums is fetched while the tile's MMAs run)
       // GP_RESIDUAL: old values of the first rows
       float xo[2][32];

@@ -536,7 +536,8 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemm
   static bool attr_set_dev[kAttrDevices] = {};
   bool& attr_set = *attr_flag(attr_set_dev);
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
@@ -545,7 +546,8 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemm
   p.parts = part && arrive ? pair_parts(tiles, p.KC, clusters) : 1;
   p.part = part; p.arrive = arrive;
   const int grid = 2 * (p.parts > 1 ? tiles * p.parts : std::min(tiles, clusters));
-  return launch_k(pdl, gemm_pair<MODE, GP_NT>, dim3(grid), dim3(GP_THREADS), (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
+  return launch_k(pdl, p.parts > 1 ? gemm_pair<MODE, GP_NT, true> : gemm_pair<MODE, GP_NT, false>, dim3(grid), dim3(GP_THREADS),
+                  (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
 }
 
 // x[M,K] * [mats]^T with the epilogue of `mode`; the caller has filled in the fields its mode uses.
@@ -1283,7 +1285,7 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
   // (2) candidate tree -> rows
   int M = B * T_;
   Rows rows = make_rows(c, T_, false);
-  KLAUNCH("prepare_verify_rows", prepare_verify_rows<T>, dim3(M), dim3(128), 0, rows, (const int*)c->d_cand, (K + 1) * kmax, kmax,
+  KLAUNCH("prepare_verify_rows", prepare_verify_rows<T>, dim3(M), dim3(256), 0, rows, (const int*)c->d_cand, (K + 1) * kmax, kmax,
           (const int*)c->d_depth, (const int*)c->d_rank, c->cap, static_cast<const T*>(c->embed), c->d_x, d, f.vocab, c->d_status);
   step_event(c, 2);
   // (3) verification forward
@@ -1308,8 +1310,8 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
   }
   step_event(c, 4);
   // (5) KV compaction
-  dim3 gc(f.n_layers * 2 * f.n_kv_heads, B);
-  KLAUNCH("compact_kv", compact_kv<T>, gc, dim3(64), 0, static_cast<T*>(c->d_pool), c->geom, (const int*)c->d_page_table,
+  dim3 gc(f.n_layers * 2 * ((f.n_kv_heads + COMPACT_HEADS - 1) / COMPACT_HEADS), B);
+  KLAUNCH("compact_kv", compact_kv<T>, gc, dim3(128), 0, static_cast<T*>(c->d_pool), c->geom, (const int*)c->d_page_table,
           (const int*)c->d_path, (const int*)c->d_count, (const int*)c->d_n_old, K);
   step_event(c, 5);
   return SPEC_OK;
