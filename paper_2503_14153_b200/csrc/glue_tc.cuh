@@ -19,7 +19,7 @@ struct PartView {
   int ld;
   SegMap seg;                  // how the GEMM dealt its units: gives the slots of a tile
   int mt_shift;                // log2 of the activation rows per tile
-  int single;                  // 1: every tile is one finished slot (the 128 x 256-tile GEMM): read it directly
+  int single;                  // 1: every tile is one finished slot (gemm_pair, plain matrices): read it directly
 };
 
 constexpr int PV_UNROLL = 12;
