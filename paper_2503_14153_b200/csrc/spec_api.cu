@@ -218,7 +218,7 @@ struct spec_ctx {
   bool attn_umma = true;               // SPEC_OPT_ATTN_UMMA: the long-context kernel is the tcgen05 one (head_dim 128)
   CUtensorMap tm_kv;                   // 5-D view of the page pool for its TMA loads
   bool tm_kv_ok = false;
-  bool wide_gemm = true;               // SPEC_OPT_WIDE_GEMM: passes of more than 128 rows use the 128 x 256-tile kernel
+  bool wide_gemm = true;               // SPEC_OPT_WIDE_GEMM: passes of more than 128 rows use the two-SM kernel (gemm_pair)
   int cluster_epilogue = 7;            // SPEC_OPT_CLUSTER_EPILOGUE: which projections finish their split-K sums inside a cluster
                                        // (bits: 1 output/down, 2 gate+up, 4 q/k/v; measured on the 7B shape: only gate+up pays)
   int small_gemm_ctas = 288;           // CTAs of GEMMs with at most 48 weight tiles (Wo, down); 288 since the weights are pre-tiled (192 before)
@@ -286,7 +286,7 @@ struct spec_ctx {
   cudaEvent_t phase_ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   // enqueue-only steps: the committed lengths are copied to pinned host memory now and then, so
   // the host's bounds on them stay tight without a synchronisation
-  int* h_n_pinned = nullptr;           // [max_batch], cudaHostAlloc
+  int* h_n_pinned = nullptr;           // [max_batch], behind h_result
   cudaEvent_t n_ev = nullptr;
   bool n_copy_pending = false;
   int n_copy_steps_after = 0;          // steps enqueued after the pending copy
@@ -1205,7 +1205,9 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   // earlier pass or to this one: a layer stores the keys and values of all its rows before its attention starts.
   // (without the many-row projection kernel a pass takes as many chunks as there are sequences)
   const int cap = c->tc && !c->wide_gemm ? f.max_batch : c->chunk_cap;
-  const int R = std::min(PREFILL_ROWS, (int)round_up(maxlen, 16));
+  // The 16-bit path keeps whole chunks also for shorter prompts: fewer rows would take other kernels, and a prompt's results
+  // would depend on the lengths it is batched with. (The float32 rows are computed one by one.)
+  const int R = c->tc ? PREFILL_ROWS : std::min(PREFILL_ROWS, (int)round_up(maxlen, 16));
   std::vector<int> cseq, cpos;
   for (int b = 0; b < batch; ++b)
     for (int p = 0; p < off[b + 1] - off[b]; p += R) { cseq.push_back(b); cpos.push_back(p); }
@@ -1546,10 +1548,11 @@ int spec_create(const spec_config* cfg, const spec_weights* w, const spec_tree* 
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_cand, 0, (size_t)cfg->max_batch * (c->K + 1) * c->kmax * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) { g_create_error = std::string("set-up copies: ") + cudaGetErrorString(e); delete c; return SPEC_E_CUDA; }
-  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_result), (4 + (size_t)cfg->max_batch * (c->K + 3)) * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+  // one pinned block: a step's result, then the copy of the committed lengths
+  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_result), (4 + (size_t)cfg->max_batch * (c->K + 4)) * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
     g_create_error = "pinned host memory for a step's result"; delete c; return SPEC_E_CUDA;
   }
-  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_n_pinned), (size_t)cfg->max_batch * sizeof(int), cudaHostAllocDefault) != cudaSuccess) c->h_n_pinned = nullptr;
+  c->h_n_pinned = c->h_result + 4 + (size_t)cfg->max_batch * (c->K + 3);
   if (cudaEventCreateWithFlags(&c->n_ev, cudaEventDisableTiming) != cudaSuccess) c->n_ev = nullptr;
   cudaGetLastError();
   if (c->tc && cfg->head_dim == 128 && cfg->page_size == 16) {
@@ -1614,7 +1617,6 @@ int spec_destroy(spec_ctx* c) {
   for (auto& g : c->step_graph) if (g.exec) cudaGraphExecDestroy(g.exec);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->n_ev) cudaEventDestroy(c->n_ev);
-  if (c->h_n_pinned) cudaFreeHost(c->h_n_pinned);
   if (c->h_result) cudaFreeHost(c->h_result);
   delete c;
   return SPEC_OK;

@@ -52,7 +52,7 @@ def test_many_row_projections_vs_oracle(torch, heads, kv, hd, ffn, T, batch):
     (128, (2500,)),               # 20 chunks of one prompt: two passes, the second sees the first pass's chunks in the cache
     (64, (1300,)),                # 11 chunks in one pass, the mma.sync attention
     (128, (300, 5, 129, 700)),    # chunks of several prompts in a pass, last chunks of 44, 5, 1 and 60 rows
-    (64, (17, 33)),               # short prompts: a chunk each, no longer than the longest prompt
+    (64, (17, 33)),               # short prompts: a chunk each that is mostly empty
 ])
 def test_prompts_in_chunks_vs_oracle(torch, hd, lengths):
     """Prompt processing deals the 128-token chunks of all prompts to shared passes: the first root, the hidden state and
