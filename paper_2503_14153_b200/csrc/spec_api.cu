@@ -1823,7 +1823,9 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
   int rws[1] = {N};
   if (!plan_gemm(M, K, 1, rws, ctas, &g)) return SPEC_E_BADARG;
   StreamTmaps tm{};
-  if (M > 128) {
+  if (M > 128 && (long long)g.p.n_tiles * g.p.seg.m_tiles >= 2LL * g.grid) {
+    // (With fewer than two tiles a CTA the streaming kernel cuts the inner dimension into several separately rounded sums: there it
+    // is as fast, 67 us against 65 in one case, and closer to the exact result, 1.7e-6 against 2.7e-6.)
     // many rows: whole tiles on pairs of SMs, finished sums straight into y (at M = 1008, N = 11008, K = 4096 the call takes
     // 116 us; weight streaming, which fetches the weights once per 128 rows, took 127 us, adding up its partial sums 34, the call 204)
     PairGemmParams p{};
