@@ -18,7 +18,13 @@
 // rows the output and down projections took 184 us instead of 120.)
 //
 // Modes:
-//  * GP_PLAIN     float32 sums to out[m][ld] (columns below n_cols only)
+//  * GP_PLAIN     float32 sums to out[m][ld] (columns below n_cols only). The only mode whose sums are results as they stand:
+//                 the two halves of the inner dimension go to the two accumulators and are added in registers, because the error
+//                 of a running sum in the tensor cores grows with its length (K 4096: 4.4e-6 of the result in one accumulator,
+//                 2.1e-6 in two halves; the weight streamer, which cuts about every other tile, 3.9e-6 at M = 1008). The first
+//                 half is taken out of tensor memory under the MMAs of the second, and both accumulators are given back
+//                 before the stores, so that the next tile's MMAs run under them: 112 us instead of 114 at M = 1008, N = 11008,
+//                 K = 4096; 98 instead of 94 at M = 2048, K = 1024, where the stores take longer than the MMAs.
 //  * GP_RESIDUAL  x[m][n] += sum, in place (output and down projections)
 //  * GP_SWIGLU    act[m][n] = bf16(SiLU(gate) * up): a CTA's 128 weight rows are 64 rows of the gate and the same 64
 //                 rows of the up matrix
@@ -157,6 +163,8 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   const int total_tiles = p.w_pairs * p.m_tiles, parts = SPLIT ? p.parts : 1;
   const int my_tiles = cl < total_tiles * parts ? (SPLIT ? 1 : (total_tiles - 1 - cl) / ncl + 1) : 0;
   const int k_lo = SPLIT ? cl % parts * KC / parts : 0, k_hi = SPLIT ? (cl % parts + 1) * KC / parts : KC;
+  static_assert(MODE != GP_PLAIN || !SPLIT, "plain sums are not shared between clusters");
+  const int halves = MODE == GP_PLAIN && KC > 1 ? 2 : 1;    // accumulators a tile's inner dimension is cut into
   auto tile_of = [&](int i) { return SPLIT ? cl / parts : cl + i * ncl; };
 
   pdl_launch_dependents();
@@ -243,12 +251,14 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       bool ok = true;
       int st = 0;
       uint32_t ph = 0;
-      for (int i = 0; i < my_tiles && ok; ++i) {
+      for (int i = 0; i < my_tiles * halves && ok; ++i) {        // (accumulator fills: tiles, or halves of tiles in turn)
         const int buf = i & 1;
         if (!mbar_wait(&acc_empty[buf], ((i >> 1) & 1) ^ 1, p.status, 44)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_addr = tmem_base + (uint32_t)(buf * NT);
-        for (int kc = k_lo; kc < k_hi; ++kc) {
+        const int mid = (k_lo + k_hi) >> 1;
+        const int k_first = halves == 2 && buf ? mid : k_lo, k_end = halves == 2 && !buf ? mid : k_hi;
+        for (int kc = k_first; kc < k_end; ++kc) {
           if (!mbar_wait(&full[st], ph, p.status, 41)) { ok = false; break; }
           if (i == 0 && kc == k_lo) trace_mark_min(p.trace, 2);
           tc_fence_after();
@@ -257,7 +267,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           const uint64_t bdesc = make_kmajor_sw128_desc(a_addr + Cfg::A_BYTES);
 #pragma unroll
           for (int k = 0; k < Cfg::BK / 16; ++k)
-            tc_mma_f16_pair(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kc > k_lo || k > 0) ? 1u : 0u);
+            tc_mma_f16_pair(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kc > k_first || k > 0) ? 1u : 0u);
           tc_commit_pair(&empty[st]);
           if (++st == STAGES) { st = 0; ph ^= 1; }
         }
@@ -275,7 +285,8 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
     const uint32_t acc_empty0 = dsmem_addr(smem_u32(acc_empty), 0);
     pdl_wait();
     for (int i = 0; i < my_tiles; ++i) {
-      const int buf = i & 1;
+      const int buf = halves == 2 ? 1 : i & 1;                // the accumulator that completes the tile
+      const uint32_t acc_ph = halves == 2 ? i & 1 : (i >> 1) & 1;
       const int tau = tile_of(i);
       const int wp = tau / p.m_tiles, mt = tau - wp * p.m_tiles;
       const int nt = 2 * wp + rank;
@@ -317,8 +328,27 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         }
         group_bar(1 + hf);
       }
+      // GP_PLAIN: the sums over the first half of the inner dimension, kept in registers
+      float first[MODE == GP_PLAIN ? HC : 1];
+      if constexpr (MODE == GP_PLAIN) {
+#pragma unroll
+        for (int j = 0; j < HC; ++j) first[j] = 0.f;
+        if (halves == 2) {
+          if (!epilogue_and(mbar_wait(&acc_full[0], acc_ph, p.status, 42))) break;
+          tc_fence_after();
+          uint32_t r[HC / 32][32];
+#pragma unroll
+          for (int g = 0; g < HC / 32; ++g) tmem_ld32(taddr - NT + g * 32, r[g]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < HC; ++j) first[j] = __uint_as_float(r[j / 32][j % 32]);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(acc_empty0);
+        }
+      }
       // (all eight warps give up when one of them does: barriers follow)
-      if (!epilogue_and(mbar_wait(&acc_full[buf], (i >> 1) & 1, p.status, 42))) break;
+      if (!epilogue_and(mbar_wait(&acc_full[buf], acc_ph, p.status, 42))) break;
       tc_fence_after();
       // partial sums of this warp's rows, part k at parts_at + k * PART
       constexpr size_t PART = (size_t)2 * NT * 128;
@@ -370,21 +400,30 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(v[j]);
       };
-      if (MODE == GP_PLAIN) {
+      if constexpr (MODE == GP_PLAIN) {
         const int col = nt * 128 + wl;
-        float* dst = p.out + col;
+        float* dst = p.out + (size_t)m0 * p.ld + col;
         const bool on = nt < p.n_tiles && col < p.n_cols;
-#pragma unroll 2
-        for (int g = 0; g < HC / 32; ++g) {
-          uint32_t r[32];
-          acc(g, r);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int m = m0 + g * 32 + j;
-            if (on && m < p.M) dst[(size_t)m * p.ld] = __uint_as_float(r[j]);
-          }
+        for (int g = 0; g < HC / 16; ++g) {                    // (16 columns at a time: registers)
+          uint32_t r[16];
+          tmem_ld16(taddr + g * 16, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) first[g * 16 + j] += __uint_as_float(r[j]);
         }
-      } else if (MODE == GP_RESIDUAL) {
+        // (given back before the stores: the next tile's MMAs run under them)
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);
+        const int live = on ? p.M - m0 : 0;
+#pragma unroll
+        for (int j = 0; j < HC; ++j) {                         // (a running pointer: 128 separate addresses cost 2-3 us a tile)
+          if (j < live) *dst = first[j];
+          dst += p.ld;
+        }
+        continue;
+      } else if constexpr (MODE == GP_RESIDUAL) {
         // old values of the next 32 rows are fetched while 32 rows are finished
         float* dst = p.out + rcol;
 #pragma unroll

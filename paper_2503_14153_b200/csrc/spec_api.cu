@@ -537,17 +537,20 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemm
   bool& attr_set = *attr_flag(attr_set_dev);
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+    if constexpr (MODE != GP_PLAIN)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   const int clusters = std::min(GP_MAX_CLUSTERS, max_clusters);
   const int tiles = p.w_pairs * p.m_tiles;
-  p.parts = part && arrive ? pair_parts(tiles, p.KC, clusters) : 1;
+  p.parts = MODE != GP_PLAIN && part ? pair_parts(tiles, p.KC, clusters) : 1;
   p.part = part; p.arrive = arrive;
   const int grid = 2 * (p.parts > 1 ? tiles * p.parts : std::min(tiles, clusters));
-  return launch_k(pdl, p.parts > 1 ? gemm_pair<MODE, GP_NT, true> : gemm_pair<MODE, GP_NT, false>, dim3(grid), dim3(GP_THREADS),
-                  (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
+  auto kernel = gemm_pair<MODE, GP_NT, false>;
+  if constexpr (MODE != GP_PLAIN)
+    if (p.parts > 1) kernel = gemm_pair<MODE, GP_NT, true>;
+  return launch_k(pdl, kernel, dim3(grid), dim3(GP_THREADS), (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
 }
 
 // x[M,K] * [mats]^T with the epilogue of `mode`; the caller has filled in the fields its mode uses.
@@ -581,7 +584,7 @@ int run_gemm_pair(spec_ctx* c, int mode, const void* x, int M, int K, int n_mats
       case GP_RESIDUAL: e = launch_gp<GP_RESIDUAL>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
       case GP_SWIGLU: e = launch_gp<GP_SWIGLU>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
       case GP_ROPE: e = launch_gp<GP_ROPE>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
-      default: e = launch_gp<GP_PLAIN>(c->stream, c->pdl, tm, *w, nullptr, nullptr);   // (writes the scratch itself) break;
+      default: e = launch_gp<GP_PLAIN>(c->stream, c->pdl, tm, *w, nullptr, nullptr); break;   // (its sums go to the scratch)
     }
     c->launches++;
   }
@@ -1824,10 +1827,10 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
   if (!plan_gemm(M, K, 1, rws, ctas, &g)) return SPEC_E_BADARG;
   StreamTmaps tm{};
   if (M > 128 && (long long)g.p.n_tiles * g.p.seg.m_tiles >= 2LL * g.grid) {
-    // (With fewer than two tiles a CTA the streaming kernel cuts the inner dimension into several separately rounded sums: there it
-    // is as fast, 67 us against 65 in one case, and closer to the exact result, 1.7e-6 against 2.7e-6.)
     // many rows: whole tiles on pairs of SMs, finished sums straight into y (at M = 1008, N = 11008, K = 4096 the call takes
-    // 116 us; weight streaming, which fetches the weights once per 128 rows, took 127 us, adding up its partial sums 34, the call 204)
+    // 112 us; weight streaming, which fetches the weights once per 128 rows, took 127 us, adding up its partial sums 34, the call 204)
+    // With fewer than two tiles a CTA the streaming kernel is as fast (67 us against 65 in one case) and closer to the exact
+    // result, since it cuts the inner dimension into several separately rounded sums where this kernel adds two.
     PairGemmParams p{};
     if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, GP_NT / 2)) return SPEC_E_CUDA;
     p.M = M; p.KC = K / 64; p.n_mats = 1;
@@ -1835,11 +1838,8 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     for (int i = 1; i <= GS_MAX_MATS; ++i) p.mat_tile0[i] = p.n_tiles;
     p.out = y; p.ld = (size_t)N; p.n_cols = N;
     p.status = reinterpret_cast<int*>(scratch + scratch_floats);
-    // partial sums of split tiles at the start of the scratch where it is large enough, arrival counters before the status word
-    const bool room = scratch_floats >= GP_PART_FLOATS + GP_ARRIVE;
-    unsigned int* arrive = room ? reinterpret_cast<unsigned int*>(p.status) - GP_ARRIVE : nullptr;
-    if (cudaMemsetAsync(room ? (void*)arrive : (void*)p.status, 0, 16 + (room ? GP_ARRIVE * 4 : 0), st) != cudaSuccess ||
-        launch_gp<GP_PLAIN>(st, false, tm, p, room ? scratch : nullptr, arrive, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
+    if (cudaMemsetAsync(p.status, 0, 16, st) != cudaSuccess ||
+        launch_gp<GP_PLAIN>(st, false, tm, p, nullptr, nullptr, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
     return op_linear_status(p.status, st);
   }
   if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, g.MT)) return SPEC_E_CUDA;
