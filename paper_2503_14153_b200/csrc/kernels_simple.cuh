@@ -175,11 +175,15 @@ template <typename T> struct RowLinear {
   int n_mats;
 };
 
-// Warps that share a group of outputs: as many as have a step of the inner dimension each, while there are few warps.
-template <typename T> inline int linear_rows_split(int groups, int M, int K) {
-  const long long warps = (long long)groups * ((M + LR_M - 1) / LR_M);
-  const int steps = K / (32 * Vec16<T>::N);
-  return steps >= 4 && warps * 4 <= 2400 ? 4 : (steps >= 2 && warps * 2 <= 2400 ? 2 : 1);
+// Warps that share a group of outputs: as many as have a step of the inner dimension each, while 16 rows (the verification
+// pass of a small tree) leave the chip's resident warps, LR_WARPS * 4 an SM, room for them. The number of rows is left out on
+// purpose: the split decides the order of a row's sums, and a row's result must not depend on what it is computed with.
+// (Choosing by the rows of the call as well gained nothing up to 128 rows: a 24-step request of the two-layer configuration takes
+// 3.1 ms either way. From 512 rows a narrow projection is slower for it: 768 x 256 at 512 rows 23 us instead of 16.)
+template <typename T> inline int linear_rows_split(int groups, int K) {
+  constexpr int RESIDENT = 148 * LR_WARPS * 4, ROW_GROUPS = 16 / LR_M;
+  const int steps = K / (32 * Vec16<T>::N), warps = groups * ROW_GROUPS;
+  return steps >= 4 && warps * 4 <= RESIDENT ? 4 : (steps >= 2 && warps * 2 <= RESIDENT ? 2 : 1);
 }
 
 struct RowLinearShape {
@@ -189,7 +193,7 @@ struct RowLinearShape {
 template <typename T> inline RowLinearShape linear_rows_shape(int groups, int M, int K) {
   RowLinearShape s;
   const int mg = (M + LR_M - 1) / LR_M;
-  s.ks = linear_rows_split<T>(groups, M, K);
+  s.ks = linear_rows_split<T>(groups, K);
   s.ms = 1;
   while (s.ms * 2 <= LR_WARPS / s.ks && s.ms < mg) s.ms *= 2;
   const int per = LR_WARPS / (s.ks * s.ms);

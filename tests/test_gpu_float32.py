@@ -33,6 +33,17 @@ def test_op_linear_f32(torch, M, N, K):
     assert ((y.double() - want).abs() <= K * 2.0 ** -24 * size).all()
 
 
+@pytest.mark.parametrize("N,K", [(768, 256), (1000, 1024), (3000, 1024), (256, 688), (130, 264)])
+def test_rows_do_not_depend_on_the_number_of_rows(torch, N, K):
+    """A row's float32 sums are the same, bit for bit, whatever other rows the call has."""
+    from paper_2503_14153_b200 import spec_op_linear
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    x, w = torch.randn((300, K), generator=g, device="cuda"), torch.randn((N, K), generator=g, device="cuda")
+    whole = spec_op_linear(x, w)
+    for m in (1, 4, 16, 33, 128):
+        assert torch.equal(spec_op_linear(x[:m].contiguous(), w), whole[:m]), m
+
+
 @pytest.mark.parametrize("hd,heads,kv,prompt_len,dtype", [
     (32, 4, 4, 150, "fp32"), (64, 4, 2, 140, "fp32"), (96, 2, 2, 70, "fp32"), (128, 2, 1, 63, "fp32"), (160, 2, 2, 33, "fp32"),
     (256, 2, 2, 100, "fp32"), (256, 1, 1, 1, "fp32"), (64, 4, 2, 140, "bf16"),
