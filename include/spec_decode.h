@@ -103,10 +103,13 @@ typedef struct {
 } spec_weights;
 
 /* Bytes of DEVICE workspace spec_create needs for this shape and tree (KV page pool, page
- * tables, activations, split-K and split-KV scratch, status word). 0 on invalid input. */
+ * tables, activations, split-K and split-KV scratch, status word). 0 on invalid input. On the bf16
+ * tensor-core path that includes activations for prompt passes of up to 18 chunks of 128 tokens (2304 rows;
+ * 220 MB more than one chunk's at the 7B shape). spec_create takes a smaller workspace too, as far down as
+ * one chunk a sequence: the passes then take as many chunks as there is room for, and prompts take longer. */
 size_t spec_workspace_bytes(const spec_config *cfg, const spec_tree *tree);
 
-/* Builds a context. `workspace` is a DEVICE buffer of at least spec_workspace_bytes(),
+/* Builds a context. `workspace` is a DEVICE buffer of spec_workspace_bytes() (or less, see there),
  * 1024-byte aligned, zero-filled or not (the library initialises what it needs).
  * `cuda_stream` is a cudaStream_t (NULL = default stream); all work is enqueued on it.
  * The q, k and v projections of a layer run as one launch (bf16) whether or not the three

@@ -530,11 +530,11 @@ argmax_partials_tc(const PartView pv, int V, float* __restrict__ logits, float* 
 
 // Per-head top-k straight from the partial sums of the heads' lm_head GEMM (no materialised logits): each
 // row's kmax best (value desc, index asc) of this block's slice of the vocabulary go to the partial lists
-// pk_val / pk_idx [row][block][kmax]; grid (slices, rows). The CTA of a row that arrives last (arrive[row],
+// pk_val / pk_idx [row][block][kmax]; grid (slices, rows), the view's first row being row `row0` of the lists. The CTA of a row that arrives last (arrive[row],
 // zero between launches) merges the row's lists itself (topk_merge_row: the result does not depend on who
 // that is). Dynamic shared memory: the larger of slice * 4 and gridDim.x * kmax * 8 bytes.
 __global__ void __launch_bounds__(256)
-topk_slices_tc(const PartView pv, int V, int rows_total, int slice, int kmax, float* pk_val, int* pk_idx,
+topk_slices_tc(const PartView pv, int V, int row0, int slice, int kmax, float* pk_val, int* pk_idx,
                unsigned int* __restrict__ arrive, int K, const int* __restrict__ root_tok,
                const int* __restrict__ cand_override, int* __restrict__ cand, unsigned long long* tr) {
   KTrace kt(tr);
@@ -542,9 +542,9 @@ topk_slices_tc(const PartView pv, int V, int rows_total, int slice, int kmax, fl
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
   extern __shared__ float zs[];
-  const int row = blockIdx.y, n0 = blockIdx.x * slice, n1 = min(n0 + slice, V);    // slice % 4 == 0
+  const int row = row0 + blockIdx.y, n0 = blockIdx.x * slice, n1 = min(n0 + slice, V);    // slice % 4 == 0
   for (int c4 = threadIdx.x; c4 * 4 < n1 - n0; c4 += blockDim.x) {
-    const float4 a = part_sum4(pv, row, n0 + c4 * 4);
+    const float4 a = part_sum4(pv, blockIdx.y, n0 + c4 * 4);
     zs[c4 * 4] = a.x; zs[c4 * 4 + 1] = a.y; zs[c4 * 4 + 2] = a.z; zs[c4 * 4 + 3] = a.w;
   }
   __syncthreads();

@@ -235,6 +235,7 @@ struct spec_ctx {
   int *d_result;                       // [4 + B * (K + 3)]: d_status, d_n, d_count, d_out_tok
   int* h_result = nullptr;             // the same in pinned host memory
   int *d_status, *d_pidx, *d_pk_idx, *d_draws;
+  int head_rows;                       // rows of the heads' logits computed at a time (without tensor cores)
   int chunk_cap;                       // prompt chunks the row buffers hold in one pass
   int *d_chunk_seq, *d_chunk_pos, *d_chunk_n, *d_chunk_cnt;   // [max_batch * ceil(max_seq / 128)]: sequence and first token; [chunk_cap]
   uint32_t *d_anc_tree, *d_anc_chain;
@@ -250,7 +251,7 @@ struct spec_ctx {
   bool trace_on = false;
   unsigned long long* d_trace = nullptr;
   unsigned int* d_attn_arrive = nullptr;
-  unsigned int* d_pair_arrive = nullptr;  // [GP_ARRIVE] arrival counters of the split tiles, zero between launches
+  unsigned int* d_pair_arrive = nullptr;  // [GP_ARRIVE] arrival counters of the shared tiles, zero between launches
   unsigned int* d_row_arrive = nullptr;   // [Mcap] arrival counters of the per-row finishing steps, zero between launches
   float* d_pval2 = nullptr;            // finished per-row argmax (tensor-core path)
   int* d_pidx2 = nullptr;
@@ -356,15 +357,22 @@ bool validate_config(const spec_config* c, std::string* why) {
 // KV splits of an attention launch over `groups` row groups: as many as fit beside each other, at most `most`.
 int attn_splits(int most, int n_heads, int groups) { return std::max(1, std::min(most, (SM_SLOTS / 2) / (n_heads * groups))); }
 
-// Lays the workspace out; with base == nullptr only measures it.
-size_t carve(spec_ctx* c, void* base) {
+int max_prompt_chunks(const spec_config& f) { return f.max_batch * (int)((f.max_seq + PREFILL_ROWS - 1) / PREFILL_ROWS); }   // of the longest prompts
+// Chunks a prompt-processing pass takes where the workspace has room for them.
+int full_chunk_cap(const spec_ctx* c) {
+  return c->tc ? std::max(c->cfg.max_batch, std::min(PREFILL_CHUNKS, max_prompt_chunks(c->cfg))) : c->cfg.max_batch;
+}
+
+// Lays the workspace out; with base == nullptr only measures it. chunk_cap: prompt chunks of a pass, at least one a sequence;
+// share_tiles: with scratch for the partial sums of gemm_pair's shared tiles even if no other use asks for that much.
+size_t carve(spec_ctx* c, void* base, int chunk_cap, bool share_tiles) {
   const spec_config& f = c->cfg;
   Bump b(base);
   int B = f.max_batch, T = c->T, K = c->K, d = f.d_model, F = f.d_ffn, V = f.vocab;
   int HD = f.n_heads * f.head_dim;
   c->Nqkv = HD + 2 * f.n_kv_heads * f.head_dim;
-  const int max_chunks = B * (int)((f.max_seq + PREFILL_ROWS - 1) / PREFILL_ROWS);   // of the longest possible prompts
-  c->chunk_cap = c->tc ? std::max(B, std::min(PREFILL_CHUNKS, max_chunks)) : B;
+  const int max_chunks = max_prompt_chunks(f);
+  c->chunk_cap = chunk_cap;
   c->Mcap = (int)round_up((size_t)std::max(B * std::max(T, PREFILL_ROWS), c->chunk_cap * PREFILL_ROWS), 128);
   c->cap = (int)round_up((size_t)f.max_seq + T, f.page_size);
   if (64 % f.page_size == 0) c->cap = (int)round_up(c->cap, 64);   // whole 64-key attention tiles
@@ -384,21 +392,25 @@ size_t carve(spec_ctx* c, void* base) {
   c->d_status = c->d_result; c->d_n = c->d_result + 4; c->d_count = c->d_n + B; c->d_out_tok = c->d_count + B;
   c->d_trace = b.take<unsigned long long>((size_t)TRACE_CAP * 4);
   c->d_attn_arrive = b.take<unsigned int>((size_t)c->chunk_cap * f.n_heads * 2);
-  c->d_row_arrive = b.take<unsigned int>(c->Mcap);
-  c->d_pair_arrive = b.take<unsigned int>(GP_ARRIVE);
+  // (the projections' shared tiles and the selections' rows are never counted at the same time: a kernel touches its counters
+  // after its dependency wait and leaves them at zero)
+  static_assert(GP_ARRIVE <= PREFILL_ROWS, "Mcap is at least PREFILL_ROWS");
+  c->d_row_arrive = c->d_pair_arrive = b.take<unsigned int>(c->Mcap);
   c->d_pval2 = b.take<float>(c->Mcap); c->d_pidx2 = b.take<int>(c->Mcap);
   c->d_draws = b.take<int>(B);
   c->d_cnt = b.take<int>(B); c->d_n_old = b.take<int>(B); c->d_root = b.take<int>(B);
   c->d_path = b.take<int>((size_t)B * (K + 1));
-  c->d_gen_cnt = b.take<int>(B); c->d_gen_log = b.take<int>((size_t)B * c->gen_cap);
+  c->d_gen_cnt = b.take<int>(B);
+  // (the log of generated tokens is empty while prompts are processed: the chunks' bookkeeping lies there)
+  c->d_gen_log = b.take<int>(std::max((size_t)B * c->gen_cap, 2 * (size_t)max_chunks + 2 * (size_t)chunk_cap));
+  c->d_chunk_seq = c->d_gen_log; c->d_chunk_pos = c->d_chunk_seq + max_chunks;
+  c->d_chunk_n = c->d_chunk_pos + max_chunks; c->d_chunk_cnt = c->d_chunk_n + chunk_cap;
   c->d_cand = b.take<int>((size_t)B * (K + 1) * c->kmax); c->d_cand_ov = b.take<int>((size_t)B * (K ? K : 1) * c->kmax);
   c->d_tok = b.take<int>(M); c->d_pos = b.take<int>(M); c->d_slot = b.take<int>(M); c->d_am = b.take<int>(M);
   c->d_edge = b.take<int>(M);
   c->d_parent = b.take<int>(SPEC_MAX_NODES); c->d_depth = b.take<int>(SPEC_MAX_NODES); c->d_rank = b.take<int>(SPEC_MAX_NODES);
   c->d_anc_tree = b.take<uint32_t>(SPEC_MAX_NODES * 4); c->d_anc_chain = b.take<uint32_t>(PREFILL_ROWS * 4);
   c->d_page_table = b.take<int>((size_t)B * c->pages_per_seq);
-  c->d_chunk_seq = b.take<int>(max_chunks); c->d_chunk_pos = b.take<int>(max_chunks);
-  c->d_chunk_n = b.take<int>(c->chunk_cap); c->d_chunk_cnt = b.take<int>(c->chunk_cap);
   c->d_prompt = b.take<int>((size_t)B * f.max_seq); c->d_offsets = b.take<int>(B + 1);
   c->d_mw = b.take<const void*>(SPEC_MAX_HEADS); c->d_mb = b.take<const void*>(SPEC_MAX_HEADS);
   c->d_x = b.take<float>(M * d, 1024); c->d_hid = b.take<float>(M * d, 1024); c->d_h_last = b.take<float>((size_t)B * d);
@@ -421,15 +433,18 @@ size_t carve(spec_ctx* c, void* base) {
         int r_hd[GS_MAX_MATS] = {d, d, d, d};
         if (plan_gemm((int)m, d, GS_MAX_MATS, r_hd, SM_SLOTS, &g)) pf = std::max(pf, plan_part_floats(g));
       } else {
-        pf = std::max(pf, std::max(m * (size_t)c->Nqkv, (size_t)B * K * round_up(V, 4)));   // q, k, v; the heads' logits
+        pf = std::max(pf, m * (size_t)c->Nqkv);
       }
     }
   }
   // (split tiles of the many-row projections leave their partial sums here too)
-  if (c->tc && c->Mcap > 128 && std::max(d, std::max(HD, F)) >= 64 * GP_SPLIT_KC) pf = std::max(pf, GP_PART_FLOATS);
+  if (share_tiles && c->tc && c->Mcap > 128 && std::max(d, std::max(HD, F)) >= 64 * GP_SPLIT_KC) pf = std::max(pf, GP_PART_FLOATS);
   c->part_floats = pf;
   c->d_part = b.take<float>(pf, 1024);
+  // (without tensor cores the heads' logits lie here too, `head_rows` at a time: they are used up before the verification pass
+  // writes its own)
   c->d_logits = c->keep_logits ? b.take<float>((size_t)Mlog * V, 1024) : nullptr;
+  c->head_rows = (int)std::min((size_t)B * K, (size_t)Mlog * V / round_up(V, 4));
   c->d_pval = b.take<float>((size_t)c->n_argmax * M, 1024); c->d_pidx = b.take<int>((size_t)c->n_argmax * M, 1024);
   // partial outputs of the KV splits: rows times splits, over the passes that use more than one split
   size_t split_rows = (size_t)c->nsplit_attn * B * std::max(T, PREFILL_ROWS);
@@ -1090,18 +1105,18 @@ PartView plain_view(const float* p, int rows, int ld) {
   return v;
 }
 
-// Per-head top-k over the heads' logits into the candidate table.
-int heads_top_k(spec_ctx* c, const PartView& pl, int rows_total, const int* ov) {
+// Per-head top-k over the logits of `rows` (sequence, head) rows from `row0` on into the candidate table.
+int heads_top_k(spec_ctx* c, const PartView& pl, int row0, int rows, const int* ov) {
   const int kmax = c->kmax, V = c->cfg.vocab;
   // the row's last-arriving CTA merges the slices' lists: no merge kernel
   // about 296 CTAs whatever the number of rows, at least four a row: more slices would only lengthen the lists to merge
   // (and at least as many as let a slice fit 40 KB)
-  const int want = std::min(c->topk_blocks, std::max(std::max(4, (V + 10239) / 10240), SM_SLOTS / rows_total));
+  const int want = std::min(c->topk_blocks, std::max(std::max(4, (V + 10239) / 10240), SM_SLOTS / rows));
   const int slice = (int)round_up((V + want - 1) / want, 4), blocks = (V + slice - 1) / slice;
   const size_t sm_topk = std::max((size_t)slice * sizeof(float), (size_t)blocks * kmax * 8);
   if (sm_topk > 44 * 1024) return c->fail(SPEC_E_BADARG, "top-k lists do not fit the merge's shared memory");
-  KLAUNCH("topk_slices_tc", topk_slices_tc, dim3(blocks, rows_total), dim3(256), sm_topk,
-          pl, V, rows_total, slice, kmax, c->d_pk_val, c->d_pk_idx, c->d_row_arrive, c->K, (const int*)c->d_root, ov, c->d_cand);
+  KLAUNCH("topk_slices_tc", topk_slices_tc, dim3(blocks, rows), dim3(256), sm_topk,
+          pl, V, row0, slice, kmax, c->d_pk_val, c->d_pk_idx, c->d_row_arrive, c->K, (const int*)c->d_root, ov, c->d_cand);
   return SPEC_OK;
 }
 
@@ -1129,7 +1144,7 @@ int heads_tc(spec_ctx* c, const int* ov) {
     int r = run_gemm(c, c->d_r, rows_total, d, 1, mats, rws, SPEC_PROFILE_OFF, &pl);
     if (r) return r;
   }
-  return heads_top_k(c, pl, rows_total, ov);
+  return heads_top_k(c, pl, 0, rows_total, ov);
 }
 
 // lm_head over `M` operand rows at `src`, leaving per-row argmax partials (and logits).
@@ -1280,9 +1295,13 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
             reinterpret_cast<const T* const*>(c->d_mw), reinterpret_cast<const T* const*>(c->d_mb), static_cast<T*>(c->d_r), B, K, d);
     const void* mats[1] = {c->lm_head};
     const int ldz = (int)round_up(f.vocab, 4);
-    int r = linear_simple<T, LR_PLAIN>(c, "linear_heads", static_cast<const T*>(c->d_r), 1, mats, &f.vocab, c->d_part, ldz, nullptr, B * K, d);
-    if (r) return r;
-    if ((r = heads_top_k(c, plain_view(c->d_part, B * K, ldz), B * K, ov))) return r;
+    for (int r0 = 0; r0 < B * K; r0 += c->head_rows) {
+      const int rows_now = std::min(c->head_rows, B * K - r0);
+      int r = linear_simple<T, LR_PLAIN>(c, "linear_heads", static_cast<const T*>(c->d_r) + (size_t)r0 * d, 1, mats, &f.vocab, c->d_logits, ldz, nullptr,
+                                         rows_now, d);
+      if (r) return r;
+      if ((r = heads_top_k(c, plain_view(c->d_logits, rows_now, ldz), r0, rows_now, ov))) return r;
+    }
   } else {
     CUDA_OK(cudaMemcpyAsync(c->d_cand, c->d_root, B * sizeof(int), cudaMemcpyDeviceToDevice, c->stream));
   }
@@ -1468,7 +1487,7 @@ size_t spec_workspace_bytes(const spec_config* cfg, const spec_tree* tree) {
   tmp.T = tree->n_nodes; tmp.K = cfg->n_medusa;
   tmp.tc = cfg->dtype == 1 && !(cfg->flags & SPEC_FLAG_SIMPLE_KERNELS);
   tmp.esz = cfg->dtype == 1 ? 2 : 4;
-  return carve(&tmp, nullptr);
+  return carve(&tmp, nullptr, full_chunk_cap(&tmp), true);
 }
 
 int spec_create(const spec_config* cfg, const spec_weights* w, const spec_tree* tree, void* workspace,
@@ -1490,7 +1509,11 @@ int spec_create(const spec_config* cfg, const spec_weights* w, const spec_tree* 
   c->tc = cfg->dtype == 1 && !(cfg->flags & SPEC_FLAG_SIMPLE_KERNELS);
   c->packed = (cfg->flags & SPEC_FLAG_PACKED_WEIGHTS) != 0;
   c->esz = cfg->dtype == 1 ? 2 : 4;
-  size_t need = carve(c, workspace);
+  // a smaller workspace than spec_workspace_bytes: prompts in passes of fewer chunks, at least one a sequence
+  int chunks = full_chunk_cap(c);
+  size_t need = carve(c, workspace, chunks, true);
+  while (need > workspace_bytes && chunks > cfg->max_batch) need = carve(c, workspace, --chunks, true);
+  if (need > workspace_bytes) need = carve(c, workspace, chunks, false);
   if (need > workspace_bytes) { g_create_error = "workspace too small"; delete c; return SPEC_E_NOMEM; }
   c->h_parent.assign(tree->parent, tree->parent + c->T);
   c->h_depth.assign(tree->depth, tree->depth + c->T);

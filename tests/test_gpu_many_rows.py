@@ -76,6 +76,35 @@ def test_prompts_in_chunks_vs_oracle(torch, hd, lengths):
         assert reps[b].steps == 2
 
 
+@pytest.mark.parametrize("hd,lengths,nbytes", [(128, (1300,), 18661376), (64, (300, 5, 129, 700), 44637184)])
+def test_prompts_in_a_smaller_workspace(torch, monkeypatch, hd, lengths, nbytes):
+    """A workspace that holds the activations of one chunk a sequence and no more (the sizes that sufficed when a pass took no
+    more than that) is accepted and gives the same tokens; one that does not even hold those is refused."""
+    from oracle.decoder import OracleModel
+    from oracle.spec import OracleSpecDecoder
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from tests_lockstep import run_lockstep_batch
+    from paper_2503_14153_b200 import binding as B
+    cfg = BASE.with_(n_heads=4, n_kv_heads=2, head_dim=hd, tree_nodes=32, seed=51)
+    w = draw_weights(cfg)
+    dw = upload_weights(cfg, w)
+    prompts = [draw_prompt(cfg.with_(seed=70 + i), n) for i, n in enumerate(lengths)]
+    tree = build_tree(cfg.topk, 32)
+    room = max(lengths) + 40
+    size = {"n": nbytes}
+    monkeypatch.setattr(B.load_library(), "spec_workspace_bytes", lambda *a: size["n"])
+    gpu = SpecDecoder(cfg, dw, tree, room, max_batch=len(lengths), flags=B.FLAG_KEEP_LOGITS)
+    model = OracleModel(cfg, w)
+    oracles = {b: OracleSpecDecoder(model, tree, room) for b in range(len(lengths))}
+    reps = run_lockstep_batch(cfg, gpu, oracles, prompts, 2, TOL_BF16, TIE_GAP)
+    gpu.close()
+    for b in oracles:
+        assert reps[b].steps == 2
+    size["n"] = nbytes // 2
+    with pytest.raises(B.SpecError, match="workspace too small"):
+        SpecDecoder(cfg, dw, tree, room, max_batch=len(lengths), flags=B.FLAG_KEEP_LOGITS)
+
+
 @pytest.mark.parametrize("M,N,K,ctas", [(144, 128, 64, 1), (272, 300, 64, 2), (1008, 1000, 704, 148), (2048, 129, 128, 296),
                                         (512, 4096, 4096, 7),
                                         (256, 4096, 4096, 296), (272, 300, 8192, 296), (512, 5000, 4096, 296),

@@ -37,6 +37,29 @@ def test_top_k_and_argmax_with_equal_logits(torch, dtype, vocab, batch, period):
     dec.close()
 
 
+@pytest.mark.parametrize("vocab", [1001, 3000])
+def test_head_rows_in_several_passes(torch, vocab):
+    """Without tensor cores the heads' logits share the verification pass's buffer: 24 (sequence, head) rows where it holds 16
+    (or 15, padded to whole vectors) are selected from in two passes, with each sequence's own candidates."""
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = get_config("c0", name="head_rows", vocab=vocab, seed=9)
+    dw, tree = upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, 2)
+
+    def candidates(prompts):
+        dec = SpecDecoder(cfg, dw, tree, 64, max_batch=len(prompts))
+        dec.prefill(prompts)
+        dec.step()
+        cand = dec.debug(B.DBG_CAND).copy()
+        dec.close()
+        return cand
+
+    prompts = [draw_prompt(cfg.with_(seed=20 + b), 5 + b) for b in range(8)]
+    together = candidates(prompts)
+    for b, p in enumerate(prompts):
+        assert np.array_equal(together[b], candidates([p])[0]), b
+
+
 @pytest.mark.parametrize("vocab", [1001, 4096 * 8 + 4, 40003])
 def test_sampled_decoding_vocabulary_sizes(torch, vocab):
     """Typical acceptance and sampling where the row does not fill a thread's share evenly: fewer tokens than threads, just
