@@ -467,17 +467,18 @@ attention_tc(const AttnTcArgs a, unsigned long long* tr) {
 // loop. The warps' softmax states are merged through shared memory at the end and warp 0
 // writes the normalised bf16 rows. Sub-tiles below the host's lower bound of the committed
 // length are requested before the wait on the previous kernel.
+constexpr int ATTN_ROWS_SUB = 32;             // keys per sub-tile
+constexpr int ATTN_ROWS_BUFS = 2;             // buffers per warp
 __host__ __device__ inline size_t attention_rows_smem(int head_dim, int warps) {
   const size_t rowb = (size_t)head_dim * 2;
-  return 16 * rowb + (size_t)warps * 2 * 2 * 32 * rowb + 8 * (size_t)warps * 2 + 4 * ATTN_PT_CACHE;
+  return 16 * rowb + (size_t)warps * 2 * ATTN_ROWS_BUFS * ATTN_ROWS_SUB * rowb + 8 * (size_t)warps * 2 + 4 * ATTN_PT_CACHE;
 }
 
 template <int HD, int W>
 __global__ void __launch_bounds__(W * 32)
 attention_rows(const AttnTcArgs a, unsigned long long* tr) {
   KTrace kt(tr);
-  constexpr int SK = 32;                      // keys per sub-tile
-  constexpr int NB = 2;                       // buffers per warp
+  constexpr int SK = ATTN_ROWS_SUB, NB = ATTN_ROWS_BUFS;
   constexpr int ROWB = HD * 2;                // bytes per row
   constexpr int SUB_BYTES = SK * ROWB;        // one operand of a sub-tile
   constexpr int PAGE_BYTES = 16 * ROWB;

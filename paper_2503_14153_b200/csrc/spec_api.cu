@@ -45,6 +45,7 @@ constexpr int N_COPY_EVERY = 4;         // enqueue-only steps between two copies
 constexpr int MAX_STEPS_AHEAD = 8;      // enqueue-only steps the host may run ahead of the device
 constexpr int ATTN_ROWS_WARPS = 6;      // warps of the CTA-per-16-rows attention kernel
 constexpr int ATTN_SPLIT_TILES = 8;       // fewest KV tiles a split of attention_tc gets (2..8 measured alike)
+constexpr int ATTN_STAGES = 4;          // tiles attention_tc has in flight
 constexpr int ATTN_SINGLE_TILES = 12;   // contexts of at most this many 64-key tiles use one KV split
 constexpr int ATTN_LONG_KEYS = 2048;    // default context length from which passes of more than 32 rows use the shared-K/V kernel
 
@@ -803,6 +804,23 @@ bool attn_long_mode(const spec_ctx* c, int R, int groups, int keys_hi) {
   return thr > 0 && (R > 32 || umma) && keys_hi > thr;
 }
 
+// Key splits of the tcgen05 kernel = its cluster: one CTA per SM, at most a wave of them.
+int attn_umma_splits(const spec_ctx* c, int R, int groups) {
+  const int halves = R > 64 ? (R + 127) / 128 : 1;
+  return std::max(1, std::min(std::min(c->nsplit_attn, AU_MAX_CLUSTER), (SM_SLOTS / 2) / (c->cfg.n_heads * groups * halves)));
+}
+// First positions of a sequence that the attention kernel of such a pass may fetch ahead of its dependency wait, where they
+// lie below the host's lower bound of the committed length. A bound beyond them makes no difference to the kernel.
+int attn_fetch_ahead(const spec_ctx* c, int R, int groups, int keys_hi) {
+  if (!c->tc) return 0;
+  if (attn_long_mode(c, R, groups, keys_hi)) {
+    if (c->attn_umma && c->tm_kv_ok && c->cfg.head_dim == 128) return 2 * attn_umma_splits(c, R, groups) * AU_KT;   // two tiles a split
+    if (R > 32) return 0;
+  }
+  if (attn_rows_mode(c, R, groups)) return ATTN_ROWS_WARPS * ATTN_ROWS_BUFS * ATTN_ROWS_SUB;
+  return keys_hi <= ATTN_SINGLE_TILES * 64 ? ATTN_STAGES * 64 : 0;
+}
+
 // n_hi_pass / n_lo_pass: host bounds of the cached length the pass's rows sit on, per sequence
 // (n_lo_pass may be null: nothing is fetched before the dependency wait).
 // len_now: the lengths as well as the host knows them (what the longest-first order goes by).
@@ -833,8 +851,8 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
       std::stable_sort(idx, idx + B, [&](int x, int y) { return len_now[x] > len_now[y]; });
       for (int b = 0; b < B; ++b) a.order[b] = (unsigned char)idx[b];
     }
-    // the key splits of a (sequence, row half, head) are one cluster: one CTA per SM, at most a wave of them
-    a.nsplit = std::max(1, std::min(std::min(c->nsplit_attn, AU_MAX_CLUSTER), (SM_SLOTS / 2) / (H * B * halves)));
+    // the key splits of a (sequence, row half, head) are one cluster
+    a.nsplit = attn_umma_splits(c, R, B);
     dim3 grid(H, a.nsplit, B * halves);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     static bool set_dev[kAttrDevices] = {};
@@ -906,7 +924,7 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
   const int slots1 = attn_splits(c->nsplit_attn, H, B);
   a.nsplit = tiles_hi <= ATTN_SINGLE_TILES ? 1 : slots1;
   a.split_tiles = ATTN_SPLIT_TILES;
-  a.stages = 4;
+  a.stages = ATTN_STAGES;
   dim3 grid(H, a.nsplit, B);
 #define ATTN_CASE(HDV, NWV, KGV)                                                                         \
   {                                                                                                    \
@@ -1374,9 +1392,10 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     else if (c->n_hi[b] + T_ > ATTN_SINGLE_TILES * 64) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(std::max(attn_long_threshold(c, T_, B) / 64 * 64, ATTN_SINGLE_TILES * 64), c->cap) : c->cap;
     else bound = std::min(ATTN_SINGLE_TILES * 64, c->cap);
     n_hi_plan[b] = bound - T_;
-    // the attention kernels fetch ahead of their dependency wait what lies below this bound, at most the first 1024 positions
-    n_lo_plan[b] = std::min(c->n_lo[b], 1024);
   }
+  // a recorded step serves every sequence that is at least as long as the part it fetches ahead
+  const int ahead = attn_fetch_ahead(c, T_, B, (*std::max_element(n_hi_plan.begin(), n_hi_plan.end()) + T_ + 63) / 64 * 64);
+  for (int b = 0; b < B; ++b) n_lo_plan[b] = std::min(c->n_lo[b], ahead);
   const bool use_graph = c->graph_on && !c->trace_on && c->profile_kind == 0;
   if (!use_graph) {
     int r = step_body<T>(c, ov, n_hi_plan.data(), n_lo_plan.data());

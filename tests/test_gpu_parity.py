@@ -398,8 +398,8 @@ def test_timeline_and_options(torch):
 def test_step_graph_replay(torch):
     """The step is recorded into a CUDA graph once and replayed: one recording serves the steps until a
     sequence passes the 768-position bound of the single-split attention launch, then one more is made
-    (for every longer length); a new prefill and an option change also start a new recording; the
-    tokens are those of direct enqueue."""
+    (for every longer length); an option change and a prompt that the recording is not planned for (here: one below that
+    bound again) also start a new recording; the tokens are those of direct enqueue."""
     from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
     from paper_2503_14153_b200 import binding as B
     cfg = SMALL_BF16
@@ -435,6 +435,42 @@ def test_step_graph_replay(torch):
     d1.step()
     assert d1.query(B.Q_GRAPH_CAPTURES) == 4
     d1.close()
+
+
+def test_recording_kept_over_a_prefill(torch):
+    """A recorded step serves the next prompts too where its plan covers them: the same launch shape and order of the sequences,
+    and no sequence shorter than the part the recorded attention fetches ahead of its dependency wait (at most the first 384
+    positions of attention_rows, two tiles of 128 for each of the eight key splits of attention_umma with four heads). The
+    tokens are those of a fresh decoder that enqueues directly."""
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = SMALL_BF16_D128.with_(n_heads=4, n_kv_heads=2, vocab=3000, seed=24)
+    dw, tree = upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, cfg.tree_nodes)
+
+    def tokens(dec, lengths):
+        dec.prefill([draw_prompt(cfg.with_(seed=100 + n), n) for n in lengths])
+        out = [[] for _ in lengths]
+        for _ in range(3):
+            tok, cnt = dec.step()
+            for b in range(len(lengths)):
+                out[b].extend(int(t) for t in tok[b][: int(cnt[b])])
+        return out
+
+    for batch, cases in ((1, [((700,), 1), ((500,), 1), ((900,), 1),      # attention_rows, all longer than what it fetches ahead
+                              ((100,), 2), ((300,), 2),                   # shorter; longer than the shorter one
+                              ((3000,), 3), ((2000,), 4), ((2500,), 4)]), # attention_umma: 2000 is shorter than 2048
+                         (3, [((900, 800, 700), 1), ((950, 850, 400), 1),
+                              ((700, 900, 800), 2),                       # another order
+                              ((700, 900), 3)])):                         # fewer sequences
+        dec = SpecDecoder(cfg, dw, tree, 3200, max_batch=batch)
+        for lengths, captures in cases:
+            got = tokens(dec, lengths)
+            assert dec.query(B.Q_GRAPH_CAPTURES) == captures, lengths
+            fresh = SpecDecoder(cfg, dw, tree, 3200, max_batch=batch)
+            fresh.set_option(B.OPT_GRAPH, 0)
+            assert got == tokens(fresh, lengths), lengths
+            fresh.close()
+        dec.close()
 
 
 def test_packed_weight_image_and_equivalence(torch):
