@@ -48,6 +48,40 @@ def test_many_row_projections_vs_oracle(torch, heads, kv, hd, ffn, T, batch):
         assert reps[b].steps == 3
 
 
+@pytest.mark.parametrize("d,heads,kv,hd,ffn,T,batch", [
+    # d 4096: q/k/v in 3 tiles of 4 parts each (heads of 128) and in 2 of 4 (heads of 64), gate/up in 2 tiles of 4, 129 rows
+    (4096, 2, 2, 128, 256, 43, 3), (4096, 4, 2, 64, 128, 43, 3),
+    # grouped heads at 256 rows: q/k/v in 24 tiles of 3, output in 16 of 4, gate/up in 32 of 2, down in 16 of 4
+    (4096, 32, 8, 128, 4096, 64, 4),
+    # 768 rows: down in 24 tiles of 3; 320 rows, the second activation tile a quarter full: down in 16 tiles of 4
+    (2048, 4, 2, 64, 4096, 128, 6), (2048, 4, 2, 64, 4160, 64, 5),
+    # an inner dimension of 8192 and few tiles: down in 2 tiles of 8; the output projection (4096) in 2 of 4
+    (256, 32, 2, 128, 8192, 60, 5),
+])
+def test_shared_tiles_vs_oracle(torch, d, heads, kv, hd, ffn, T, batch):
+    """Projections with tiles for less than half of the CTA pairs and an inner dimension of 4096 or more: the K chunks of a tile
+    are shared between clusters, and the last to arrive adds the parts and does the tile's epilogue. Three steps in a
+    row also show that the arrival counters are back at zero."""
+    from oracle.decoder import OracleModel
+    from oracle.spec import OracleSpecDecoder
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    from tests_lockstep import run_lockstep_batch
+    cfg = BASE.with_(n_layers=1, d_model=d, n_heads=heads, n_kv_heads=kv, head_dim=hd, d_ffn=ffn, n_medusa=2, topk=(10, 16), tree_nodes=T,
+                     seed=91 + T)
+    w = draw_weights(cfg)
+    prompts = [draw_prompt(cfg.with_(seed=60 + i), 9 + 37 * i) for i in range(batch)]
+    tree = build_tree(cfg.topk, T)
+    room = max(len(p) for p in prompts) + 40
+    gpu = SpecDecoder(cfg, upload_weights(cfg, w), tree, room, max_batch=batch, flags=B.FLAG_KEEP_LOGITS)
+    model = OracleModel(cfg, w)
+    oracles = {b: OracleSpecDecoder(model, tree, room) for b in (0, batch - 1)}
+    reps = run_lockstep_batch(cfg, gpu, oracles, prompts, 3, TOL_BF16, TIE_GAP, tie_from_row_error=True)
+    gpu.close()
+    for b in oracles:
+        assert reps[b].steps == 3
+
+
 @pytest.mark.parametrize("hd,lengths", [
     (128, (2500,)),               # 20 chunks of one prompt: two passes, the second sees the first pass's chunks in the cache
     (64, (1300,)),                # 11 chunks in one pass, the mma.sync attention
