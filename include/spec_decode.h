@@ -190,7 +190,7 @@ int64_t spec_query(const spec_ctx *ctx, int32_t what);
  * [256 weight rows] x [256 activation rows] tiles on pairs of SMs, with the step that follows in the epilogue;
  * 0 = the weight-streaming kernel, which re-reads the weights for every 128 rows.
  * SPEC_OPT_LONG_ATTN_KEYS [2048]: passes whose context may exceed this many positions run a long-context
- * attention kernel, in which a CTA reads a head's K/V once for 64 query rows and the keys are split across
+ * attention kernel, in which a CTA reads a head's K/V once for 64 query rows (passes of more than 64 rows: 128) and the keys are split across
  * the CTAs of a cluster (0 = never; batched passes that need more than one wave of CTAs switch at 512
  * positions already). SPEC_OPT_ATTN_UMMA [1]: that kernel computes scores and P V on tcgen05 with
  * accumulators in tensor memory (head_dim 128, 16-row pages); 0 = the mma.sync kernel that shares K/V tiles

@@ -19,7 +19,7 @@ struct PartView {
   int ld;
   SegMap seg;                  // how the GEMM dealt its units: gives the slots of a tile
   int mt_shift;                // log2 of the activation rows per tile
-  int single;                  // 1: every tile is one finished slot (gemm_pair, plain matrices): read it directly
+  int single;                  // 1: every tile is one finished slot (gemm_pair's plain sums, the float32 logits): read it directly
 };
 
 constexpr int PV_UNROLL = 12;
@@ -226,7 +226,6 @@ norm_rows_wide(float* __restrict__ x, const PartView pv, const float* __restrict
   }
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
-  auto part4 = [&](int c4) { return pv.single ? part_one4(pv, m, c4 * 4) : part_sum4(pv, m, c4 * 4); };
   float4 keep[NORMW_CACHE], add[NORMW_CACHE];
 #pragma unroll
   for (int k = 0; k < NORMW_CACHE; ++k) {
@@ -234,7 +233,7 @@ norm_rows_wide(float* __restrict__ x, const PartView pv, const float* __restrict
     keep[k] = add[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c4 < n4) {
       keep[k] = *reinterpret_cast<const float4*>(xr + c4 * 4);
-      if (pv.part) add[k] = part4(c4);
+      if (pv.part) add[k] = part_sum4(pv, m, c4 * 4);
     }
   }
   float ss = 0.f;
@@ -253,7 +252,7 @@ norm_rows_wide(float* __restrict__ x, const PartView pv, const float* __restrict
   for (int c4 = threadIdx.x + NORMW_CACHE * NORMW_THREADS; c4 < n4; c4 += NORMW_THREADS) {
     float4 v = *reinterpret_cast<const float4*>(xr + c4 * 4);
     if (pv.part) {
-      const float4 a = part4(c4);
+      const float4 a = part_sum4(pv, m, c4 * 4);
       v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
       *reinterpret_cast<float4*>(xr + c4 * 4) = v;
     }
@@ -341,29 +340,6 @@ rope_store_tc(const PartView pv, int qp0, int kp0, int vp0, Rows rows, const flo
       *reinterpret_cast<uint2*>(dst + kv_elem<bf16>(prow, e, D, g.page_size)) = pack4_bf16(a.x, a.y, a.z, a.w);
     }
   };
-  if (pv.single) {
-    // passes of many rows (finished sums): a thread keeps the loads of four items in flight
-    constexpr int U = 4;
-    for (int it0 = tid; it0 < n_rot + n_v; it0 += U * nthr) {
-      float4 a[U], c[U];
-#pragma unroll
-      for (int k = 0; k < U; ++k) {
-        const int it = it0 + k * nthr;
-        a[k] = c[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (it < n_rot + n_v) {
-          const int colp = item_col(it);
-          a[k] = part_one4(pv, m, colp);
-          if (it < n_rot) c[k] = part_one4(pv, m, colp + half);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < U; ++k) {
-        const int it = it0 + k * nthr;
-        if (it < n_rot + n_v) finish(it, a[k], c[k]);
-      }
-    }
-    return;
-  }
   for (int it = tid; it < n_rot + n_v; it += nthr) {
     const int colp = item_col(it);
     const float4 a = part_sum4(pv, m, colp);
@@ -383,34 +359,6 @@ swiglu_reduce_tc(const PartView pv, int gp0, int up0, bf16* __restrict__ act, in
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
   const int f4 = F >> 2;
   const size_t total = (size_t)M * f4;
-  if (pv.single) {
-    // passes of many rows (finished sums, hundreds of MB): bandwidth-bound, so a thread keeps the loads of four
-    // items in flight
-    constexpr int U = 4;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t idx0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx0 < total; idx0 += U * stride) {
-      float4 gt[U], up[U];
-#pragma unroll
-      for (int k = 0; k < U; ++k) {
-        const size_t idx = idx0 + k * stride;
-        if (idx < total) {
-          const int m = (int)(idx / f4), f = (int)(idx % f4) * 4;
-          gt[k] = part_one4(pv, m, gp0 + f);
-          up[k] = part_one4(pv, m, up0 + f);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < U; ++k) {
-        const size_t idx = idx0 + k * stride;
-        if (idx < total) {
-          const int m = (int)(idx / f4), f = (int)(idx % f4) * 4;
-          *reinterpret_cast<uint2*>(act + (size_t)m * F + f) =
-              pack4_bf16(silu_f(gt[k].x) * up[k].x, silu_f(gt[k].y) * up[k].y, silu_f(gt[k].z) * up[k].z, silu_f(gt[k].w) * up[k].w);
-        }
-      }
-    }
-    return;
-  }
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
     const int m = (int)(idx / f4), f = (int)(idx % f4) * 4;
     const float4 gt = part_sum4(pv, m, gp0 + f), up = part_sum4(pv, m, up0 + f);

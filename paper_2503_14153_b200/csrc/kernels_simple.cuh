@@ -671,9 +671,7 @@ __global__ void wait_probe(int* status, unsigned long long limit_ns) {
 // ------------------------------------------------------------------ acceptance walk
 struct AcceptArgs {
   Rows rows;
-  const float* pval;   // [row][ntile]
-  const int* pidx;
-  int ntile;
+  const int* pidx;             // [row] argmax of the base logits
   const int *parent, *depth;   // tree arrays [R]
   const int* edge_ok;          // typical mode: per-row pass flag; NULL = greedy token match
   int K, frag_token, d, mode;  // mode 0 = verify step, 1 = prefill (row b is sequence b)
@@ -684,8 +682,7 @@ struct AcceptArgs {
   int *gen_log, *gen_cnt, gen_cap;
 };
 
-// One block per sequence: finishes the per-node argmax from the partials (pval/pidx
-// [row][ntile], a warp per row), walks the tree (a node is accepted iff its parent is and its
+// One block per sequence: takes the nodes' argmax, walks the tree (a node is accepted iff its parent is and its
 // token is the argmax at the parent, or its Eq. 1 flag is set), takes the deepest accepted node
 // (lowest index on ties), applies the fragment-integrity rule, and publishes the step's result
 // and the next step's state.
@@ -695,50 +692,19 @@ __global__ void __launch_bounds__(256) accept_kernel(AcceptArgs a, unsigned long
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
   const int b = blockIdx.x, R = a.rows.R;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   __shared__ int am_s[SPEC_MAX_NODES], tok_s[SPEC_MAX_NODES], par_s[SPEC_MAX_NODES], dep_s[SPEC_MAX_NODES];
   __shared__ int edge_s[SPEC_MAX_NODES];
   __shared__ int last_s, len_s, best_s;
   if (a.mode == 1) {
-    if (warp == 0) {
-      float bv = -INFINITY; int bi = 0x7fffffff;
-      for (int t = lane; t < a.ntile; t += 32) {
-        float v = a.pval[(size_t)b * a.ntile + t]; int i = a.pidx[(size_t)b * a.ntile + t];
-        if (better(v, i, bv, bi)) { bv = v; bi = i; }
-      }
-      warp_argmax(bv, bi);
-      if (lane == 0) {
-        a.am[b] = bi;
-        a.root_tok[b] = bi;
-        a.gen_cnt[b] = 0;
-      }
+    if (threadIdx.x == 0) {
+      a.am[b] = a.root_tok[b] = a.pidx[b];
+      a.gen_cnt[b] = 0;
     }
     return;
   }
   const int cnt = a.rows.cnt[b], m0 = b * R;
-  if (a.ntile <= 4) {
-    // few partial results per row: a thread per row, every row's loads in one trip
-    for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-      float bv = -INFINITY; int bi = 0x7fffffff;
-      for (int t = 0; t < a.ntile; ++t) {
-        const float v = a.pval[(size_t)(m0 + i) * a.ntile + t]; const int idx = a.pidx[(size_t)(m0 + i) * a.ntile + t];
-        if (better(v, idx, bv, bi)) { bv = v; bi = idx; }
-      }
-      am_s[i] = bi; a.am[m0 + i] = bi;
-    }
-  } else
-  for (int i = warp; i < cnt; i += nw) {
-    float bv = -INFINITY; int bi = 0x7fffffff;
-    const float* pv = a.pval + (size_t)(m0 + i) * a.ntile;
-    const int* pi = a.pidx + (size_t)(m0 + i) * a.ntile;
-    for (int t = lane; t < a.ntile; t += 32) {
-      float v = pv[t]; int idx = pi[t];
-      if (better(v, idx, bv, bi)) { bv = v; bi = idx; }
-    }
-    warp_argmax(bv, bi);
-    if (lane == 0) { am_s[i] = bi; a.am[m0 + i] = bi; }
-  }
   for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+    am_s[i] = a.am[m0 + i] = a.pidx[m0 + i];
     tok_s[i] = a.rows.tok[m0 + i];
     par_s[i] = a.parent[i];
     dep_s[i] = a.depth[i];

@@ -1188,7 +1188,7 @@ int lm_head_argmax(spec_ctx* c, const T* src, int M) {
 AcceptArgs make_accept(spec_ctx* c, int R, int mode) {
   AcceptArgs a{};
   a.rows = make_rows(c, R, false);
-  a.pval = c->d_pval2; a.pidx = c->d_pidx2; a.ntile = 1;
+  a.pidx = c->d_pidx2;
   a.hq_last = c->tc ? static_cast<bf16*>(c->d_hq_last) : nullptr;
   a.parent = c->d_parent; a.depth = c->d_depth; a.edge_ok = nullptr;
   a.K = c->K; a.frag_token = c->cfg.frag_token; a.d = c->cfg.d_model; a.mode = mode;
@@ -1241,16 +1241,17 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   // earlier pass or to this one: a layer stores the keys and values of all its rows before its attention starts.
   // (without the many-row projection kernel a pass takes as many chunks as there are sequences)
   const int cap = c->tc && !c->wide_gemm ? f.max_batch : c->chunk_cap;
-  // The 16-bit path keeps whole chunks also for shorter prompts: fewer rows would take other kernels, and a prompt's results
-  // would depend on the lengths it is batched with. (The float32 rows are computed one by one.)
+  // The 16-bit path keeps whole chunks also for shorter prompts: the projections' kernels go by the number of rows, here a multiple
+  // of 128 whatever the lengths. (In float32 a row's sums do not depend on the others.)
   const int R = c->tc ? PREFILL_ROWS : std::min(PREFILL_ROWS, (int)round_up(maxlen, 16));
   std::vector<int> cseq, cpos;
   for (int b = 0; b < batch; ++b)
     for (int p = 0; p < off[b + 1] - off[b]; p += R) { cseq.push_back(b); cpos.push_back(p); }
   const int chunks = (int)cseq.size();
-  // A lone prompt of two chunks goes chunk by chunk, through the projections that stream the weights: on the 7B shape that takes
-  // 8.5 ms instead of 7.1, the weights being read twice, but in the order of sums that the prompt of one chunk and the
-  // verification steps have, so that a short prompt's first tokens do not depend on which side of 128 its length lies.
+  // A lone prompt of two chunks goes chunk by chunk, through the projections that stream the weights, in the order of sums that the
+  // prompt of one chunk and a lone sequence's verification steps have. On the 7B shape that takes 8.5 ms instead of 7.1, the
+  // weights being read twice. Nothing more is promised: prompts of more chunks, and any prompt processed together with
+  // others, take the many-row projections, whose order of sums is another one (and, up to 512 rows, depends on the rows).
   const int passes = batch == 1 && chunks == 2 ? 2 : (chunks + cap - 1) / cap;
   CUDA_OK(cudaMemcpyAsync(c->d_chunk_seq, cseq.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_OK(cudaMemcpyAsync(c->d_chunk_pos, cpos.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
@@ -1274,7 +1275,7 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   AcceptArgs a = make_accept(c, 1, 1);
   KLAUNCH("accept_kernel", accept_kernel, dim3(batch), dim3(256), 0, a);
   if (f.sampling) {
-    KLAUNCH("sample_root", sample_root, dim3(SAMPLE_CLUSTER, batch), dim3(SAMPLE_THREADS), 0, (const float*)c->d_logits, a.pval, f.vocab, 1, c->K,
+    KLAUNCH("sample_root", sample_root, dim3(SAMPLE_CLUSTER, batch), dim3(SAMPLE_THREADS), 0, (const float*)c->d_logits, (const float*)c->d_pval2, f.vocab, 1, c->K,
             (const int*)c->d_path, (const int*)c->d_count, f.temperature, f.seed_lo, f.seed_hi, c->d_draws, c->d_root, 1);
   }
   r = check_status(c);
@@ -1347,7 +1348,7 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
   }
   KLAUNCH("accept_kernel", accept_kernel, dim3(B), dim3(256), 0, a);
   if (f.sampling) {
-    KLAUNCH("sample_root", sample_root, dim3(SAMPLE_CLUSTER, B), dim3(SAMPLE_THREADS), 0, (const float*)c->d_logits, a.pval, f.vocab, T_, K,
+    KLAUNCH("sample_root", sample_root, dim3(SAMPLE_CLUSTER, B), dim3(SAMPLE_THREADS), 0, (const float*)c->d_logits, (const float*)c->d_pval2, f.vocab, T_, K,
             (const int*)c->d_path, (const int*)c->d_count, f.temperature, f.seed_lo, f.seed_hi, c->d_draws, c->d_root, 0);
   }
   step_event(c, 4);
@@ -1362,7 +1363,7 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
 template <typename T>
 int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t* cand_override) {
   const spec_config& f = c->cfg;
-  int B = c->B, K = c->K, T_ = c->T, d = f.d_model, kmax = c->kmax;
+  int B = c->B, K = c->K, T_ = c->T, kmax = c->kmax;
   for (int b = 0; b < B; ++b)
     if (c->n_hi[b] + K + 1 > f.max_seq) return c->fail(SPEC_E_SEQLEN, "sequence would exceed max_seq");
   for (int i = 0; i < 6; ++i)

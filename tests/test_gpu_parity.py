@@ -134,8 +134,8 @@ def test_long_context_attention_kernels_batched_ragged(torch, umma, wide):
     """The long-context attention kernels on a batch of four ragged sequences (17 to 530 cached positions: less
     than one 128-key tile up to several tiles with a ragged tail; sequence b's pages interleave with the others'
     in the pool), every sequence in lock step with an oracle of its own for three steps. The passes have 256 rows
-    (512 in the prompt): the projections run as 128 x 256 tiles (wide = 1) or on the weight streamer (wide = 0),
-    and the glue kernels take their many-row forms on finished sums or on partial sums."""
+    (512 in the prompt): the projections run on the two-SM kernel with the following step in its epilogue
+    (wide = 1) or on the weight streamer (wide = 0), whose partial sums the many-row glue kernels take."""
     from oracle.decoder import OracleModel
     from oracle.spec import OracleSpecDecoder
     from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
