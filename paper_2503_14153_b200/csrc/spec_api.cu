@@ -374,6 +374,8 @@ size_t carve(spec_ctx* c, void* base, int chunk_cap, bool share_tiles) {
   c->Nqkv = HD + 2 * f.n_kv_heads * f.head_dim;
   const int max_chunks = max_prompt_chunks(f);
   c->chunk_cap = chunk_cap;
+  // a workspace with less than full room: buffers that are never in use at the same time share their place
+  const bool spare = chunk_cap < full_chunk_cap(c) || !share_tiles;
   c->Mcap = (int)round_up((size_t)std::max(B * std::max(T, PREFILL_ROWS), c->chunk_cap * PREFILL_ROWS), 128);
   c->cap = (int)round_up((size_t)f.max_seq + T, f.page_size);
   if (64 % f.page_size == 0) c->cap = (int)round_up(c->cap, 64);   // whole 64-key attention tiles
@@ -396,22 +398,29 @@ size_t carve(spec_ctx* c, void* base, int chunk_cap, bool share_tiles) {
   // (the projections' shared tiles and the selections' rows are never counted at the same time: a kernel touches its counters
   // after its dependency wait and leaves them at zero)
   static_assert(GP_ARRIVE <= PREFILL_ROWS, "Mcap is at least PREFILL_ROWS");
-  c->d_row_arrive = c->d_pair_arrive = b.take<unsigned int>(c->Mcap);
+  c->d_row_arrive = b.take<unsigned int>(c->Mcap);
+  c->d_pair_arrive = spare ? c->d_row_arrive : b.take<unsigned int>(GP_ARRIVE);
   c->d_pval2 = b.take<float>(c->Mcap); c->d_pidx2 = b.take<int>(c->Mcap);
   c->d_draws = b.take<int>(B);
   c->d_cnt = b.take<int>(B); c->d_n_old = b.take<int>(B); c->d_root = b.take<int>(B);
   c->d_path = b.take<int>((size_t)B * (K + 1));
   c->d_gen_cnt = b.take<int>(B);
-  // (the log of generated tokens is empty while prompts are processed: the chunks' bookkeeping lies there)
+  // (the log of generated tokens is empty while prompts are processed: in a small workspace the chunks' bookkeeping lies there)
   c->d_gen_log = b.take<int>(std::max((size_t)B * c->gen_cap, 2 * (size_t)max_chunks + 2 * (size_t)chunk_cap));
-  c->d_chunk_seq = c->d_gen_log; c->d_chunk_pos = c->d_chunk_seq + max_chunks;
-  c->d_chunk_n = c->d_chunk_pos + max_chunks; c->d_chunk_cnt = c->d_chunk_n + chunk_cap;
+  if (spare) {
+    c->d_chunk_seq = c->d_gen_log; c->d_chunk_pos = c->d_chunk_seq + max_chunks;
+    c->d_chunk_n = c->d_chunk_pos + max_chunks; c->d_chunk_cnt = c->d_chunk_n + chunk_cap;
+  }
   c->d_cand = b.take<int>((size_t)B * (K + 1) * c->kmax); c->d_cand_ov = b.take<int>((size_t)B * (K ? K : 1) * c->kmax);
   c->d_tok = b.take<int>(M); c->d_pos = b.take<int>(M); c->d_slot = b.take<int>(M); c->d_am = b.take<int>(M);
   c->d_edge = b.take<int>(M);
   c->d_parent = b.take<int>(SPEC_MAX_NODES); c->d_depth = b.take<int>(SPEC_MAX_NODES); c->d_rank = b.take<int>(SPEC_MAX_NODES);
   c->d_anc_tree = b.take<uint32_t>(SPEC_MAX_NODES * 4); c->d_anc_chain = b.take<uint32_t>(PREFILL_ROWS * 4);
   c->d_page_table = b.take<int>((size_t)B * c->pages_per_seq);
+  if (!spare) {
+    c->d_chunk_seq = b.take<int>(max_chunks); c->d_chunk_pos = b.take<int>(max_chunks);
+    c->d_chunk_n = b.take<int>(c->chunk_cap); c->d_chunk_cnt = b.take<int>(c->chunk_cap);
+  }
   c->d_prompt = b.take<int>((size_t)B * f.max_seq); c->d_offsets = b.take<int>(B + 1);
   c->d_mw = b.take<const void*>(SPEC_MAX_HEADS); c->d_mb = b.take<const void*>(SPEC_MAX_HEADS);
   c->d_x = b.take<float>(M * d, 1024); c->d_hid = b.take<float>(M * d, 1024); c->d_h_last = b.take<float>((size_t)B * d);
