@@ -1,11 +1,19 @@
 // Weight-streaming bf16 linear whose split-K partial sums never leave the chip: the CTAs that
 // share an output tile form a thread-block cluster and exchange their float32 accumulators through
 // distributed shared memory, so the kernel writes finished results and the element-wise step that
-// used to follow in a kernel of its own runs in the epilogue. The residual and SwiGLU modes push: once
-// every CTA's MMAs are complete (first cluster barrier; every ring is free then) a thread sends the
-// values of its weight row with remote stores, which nobody waits for, into the shared memory of the
-// CTA that finishes that column; after the second barrier each CTA reads only its own shared memory.
-// (Reading the parts out of the other CTAs' shared memory instead cost 3 us more per kernel.)
+// used to follow in a kernel of its own runs in the epilogue.
+//
+// The exchange: once its MMAs are complete a CTA announces that its ring is free (cluster barrier, arrive only), puts its
+// accumulators into its own shared memory, a block of columns (or rows) per CTA that finishes them, and when every ring of
+// the cluster is free (the barrier's wait) sends each block with one bulk copy that completes on the receiver's mbarrier.
+// A CTA exits only after everybody has received (another arrive / wait pair, under the finishing work). Only the pass's
+// rows travel, not the MT rows of the MMA.
+// The tail, last MMA to the end of the kernel, is what bounds these kernels beside the weight stream. On the 7B shape with 64
+// rows it was 7.1 us for gate+up, 3.6 and 3.5 for the output and down projections and 2.8 for q/k/v with four epilogue warps that sent
+// single values with remote stores (q/k/v: read them), and is 4.1, 2.5, 2.9 and 1.6; a layer 96.4 -> 93.2 us. In-kernel
+// timestamps of gate+up: draining 2.0 -> 0.7 us and finishing 3.0 -> 1.2 with eight warps; 0.5 us for each barrier.cluster.arrive with release
+// semantics where nothing has to be published (now .relaxed); the copies themselves, 48 KB out of the middle CTA with two CTAs an
+// SM, 1.7 us.
 //
 // Three modes (operands swapped as in gemm_stream: 128 weight rows are the MMA's M, the MT activation
 // rows its N; MT covers all rows of the pass):
@@ -16,18 +24,18 @@
 //    that follows needs the row's mean square) in ss_part[m][tile * 8 + r].
 //  * GC_SWIGLU (gate and up projections): a cluster of 3 CTAs per pair (gate tile t, up tile t); the
 //    2 KC units of the pair are cut into three equal runs, so CTA 0 holds a gate part, CTA 1 a gate
-//    and an up part (two accumulators) and CTA 2 an up part. Once every CTA's MMAs are complete (first
-//    barrier) each thread sends the values of its weight row into the shared memory of the CTA that finishes
-//    that column (remote stores); after the second barrier each CTA finishes a third of the tile's columns
-//    from its own shared memory: gate = G0 + G1, up = U1 + U2, act = bf16(SiLU(gate) * up).
+//    and an up part (two accumulators) and CTA 2 an up part. Each CTA finishes a share of the tile's columns (48, 32 and 48):
+//    gate = G0 + G1, up = U1 + U2, act = bf16(SiLU(gate) * up).
+//  * GC_SWIGLU8 (the same projections where there are few tiles): a cluster of 8 per pair (gate tile t, up tile t), CTAs 0 to 3
+//    streaming a quarter of the gate tile's K chunks each, 4 to 7 the up tile's; columns as in GC_RESIDUAL.
 //  * GC_ROPE (query, key and value projections, stacked): a cluster of 2 CTAs per 128-row tile of the
 //    stacked matrices, each streaming half of the K chunks (96 pairs on the 7B shape: all co-resident, which
 //    96 clusters of 3 are not). A tile holds whole heads (head_dim 64 or
-//    128), so after the barrier the cluster rotates the query / key pairs (i, i + head_dim / 2) by the
+//    128), so after the exchange the cluster rotates the query / key pairs (i, i + head_dim / 2) by the
 //    row's position, writes the bf16 query rows and puts the bf16 key and value rows into the paged cache
-//    at the row's slot; CTA r takes every second activation row.
+//    at the row's slot; each CTA takes half of the activation rows.
 // Sums are added in a fixed order: results are bit-reproducible. Every wait is bounded; a CTA whose
-// wait ran out still arrives at both cluster barriers, so its cluster mates never wait for it.
+// wait ran out still sends its blocks and arrives at the cluster barriers, so its cluster mates never wait for it.
 #pragma once
 #include <cuda.h>
 
@@ -36,16 +44,17 @@
 
 namespace spec {
 
-constexpr int GC_RESIDUAL = 0, GC_SWIGLU = 1, GC_ROPE = 2;
+constexpr int GC_RESIDUAL = 0, GC_SWIGLU = 1, GC_ROPE = 2, GC_SWIGLU8 = 3;
+constexpr int GC_THREADS = 320, GC_EPI = GC_THREADS - 64;     // producer, MMA issuer, eight epilogue warps (two per SM quarter)
 constexpr int GC_RES_CLUSTER = 8, GC_GLU_CLUSTER = 3, GC_ROPE_CLUSTER = 2;
 
 struct ClusterGemmParams {
   int M, K, KC;                 // activation rows (<= MT), inner size, K / 64
   int N;                        // weight rows of one matrix (output columns)
-  const uint8_t* packed[3];     // pre-tiled images (GC_RESIDUAL: [0]; GC_SWIGLU: gate, up; GC_ROPE: q, k, v) or nullptr -> tensor maps a[i]
+  const uint8_t* packed[3];     // pre-tiled images (GC_RESIDUAL: [0]; GC_SWIGLU(8): gate, up; GC_ROPE: q, k, v) or nullptr -> tensor maps a[i]
   float* x;                     // GC_RESIDUAL: [M][N] float32 residual stream, updated in place
   float* ss_part;               // GC_RESIDUAL: [M][ceil(N/128) * 8] sums of squares of the updated pieces, or nullptr
-  bf16* act;                    // GC_SWIGLU: [M][N] bf16
+  bf16* act;                    // GC_SWIGLU(8): [M][N] bf16
   // GC_ROPE: tiles [0, tile0[1]) belong to q, [tile0[1], tile0[2]) to k, the rest to v
   int tile0[3];
   int H;                        // query heads
@@ -66,8 +75,6 @@ template <int MT> struct ClusterCfg {
   static constexpr int B_BYTES = MT * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = (MT <= 32) ? 5 : (MT == 64 ? 4 : 3);
-  static constexpr int PITCH = 132;                          // floats per staged activation row: 128 weight rows + 4 (16-byte aligned rows, banks shifted by 4)
-  static constexpr int STAGING_FLOATS = MT * PITCH;          // one accumulator, staged as [activation row][weight row]
   static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
   static constexpr int SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
 };
@@ -80,6 +87,9 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint32_t dsmem_addr(uint32_t local_smem_addr, uint32_t rank) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local_smem_addr), "r"(rank));
@@ -93,11 +103,47 @@ __device__ __forceinline__ float4 dsmem_ld4(uint32_t addr) {
 __device__ __forceinline__ void dsmem_st(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
+// Bulk copy from this CTA's shared memory into another CTA's, completing on that CTA's barrier (16-byte aligned, size
+// a multiple of 16).
+__device__ __forceinline__ void bulk_push(uint32_t dst_cluster, const void* src, uint32_t bytes, uint32_t bar_cluster) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst_cluster), "r"(smem_u32(src)), "r"(bytes), "r"(bar_cluster) : "memory");
+}
+// Generic-proxy writes to shared memory become visible to bulk copies that read it.
+__device__ __forceinline__ void fence_smem_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// Rows of one accumulator (or of a stretch of at most MT of its columns) at `taddr`, in groups of 16 of which the two epilogue warps of an SM quarter take every
+// second one: put(row, value) in the thread that owns the weight row, for rows below M.
+template <int MT, typename F>
+__device__ __forceinline__ void tmem_rows(uint32_t taddr, int hf, int M, F&& put) {
+  constexpr int NG = MT >= 32 ? MT / 32 : 1, U = NG < 2 ? NG : 2;   // (two groups at a time: registers)
+  if (MT == 16 && hf) return;
+#pragma unroll
+  for (int k0 = 0; k0 < NG; k0 += U) {
+    uint32_t r[U][16];
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if ((2 * (k0 + k) + hf) * 16 < M) tmem_ld16(taddr + (2 * (k0 + k) + hf) * 16, r[k]);      // (the same in the whole warp)
+    tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int m0 = (2 * (k0 + k) + hf) * 16;
+      if (m0 + 16 <= M) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) put(m0 + j, __uint_as_float(r[k][j]));
+      } else if (m0 < M) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (m0 + j < M) put(m0 + j, __uint_as_float(r[k][j]));
+      }
+    }
+  }
 }
 
 // One run of K chunks of one weight tile, accumulated into one tensor-memory buffer.
@@ -106,14 +152,13 @@ struct GcSeg {
 };
 
 template <int MT, int MODE>
-__global__ void __launch_bounds__(192, 2)
+__global__ void __launch_bounds__(GC_THREADS, 2)
 gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) {
   using Cfg = ClusterCfg<MT>;
   constexpr int STAGES = Cfg::STAGES;
-  constexpr int CS = MODE == GC_RESIDUAL ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER);
+  constexpr bool EIGHT = MODE == GC_RESIDUAL || MODE == GC_SWIGLU8;      // eight CTAs, each finishing 16 columns
+  constexpr int CS = EIGHT ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER);
   constexpr int TMEM_COLS = ((MODE == GC_SWIGLU ? 2 : 1) * MT < 32) ? 32 : (MODE == GC_SWIGLU ? 2 : 1) * MT;   // 32, 64 or 128
-  static_assert(MODE != GC_SWIGLU || 2 * Cfg::STAGING_FLOATS * 4 <= Cfg::RING_BYTES, "two staged accumulators must fit the ring");
-  static_assert(Cfg::STAGING_FLOATS * 4 <= Cfg::RING_BYTES, "a staged accumulator must fit the ring");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* tiles = smem_raw + (((raw + 1023u) & ~1023u) - raw);
@@ -121,7 +166,8 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   uint64_t* full = bars;
   uint64_t* empty = bars + STAGES;
   uint64_t* acc_full = bars + 2 * STAGES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
+  uint64_t* part_full = bars + 2 * STAGES + 1;               // the other CTAs' parts of this CTA's outputs have landed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
   float* staging = reinterpret_cast<float*>(tiles);          // reuses the ring once every MMA is complete
 
   KTrace kt(p.trace);
@@ -136,7 +182,10 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   // this CTA's runs
   GcSeg seg[2];
   int nseg = 0;
-  if (MODE != GC_SWIGLU) {
+  if (MODE == GC_SWIGLU8) {
+    seg[0] = GcSeg{rank >> 2, (rank & 3) * KC / 4, ((rank & 3) + 1) * KC / 4};
+    nseg = 1;
+  } else if (MODE != GC_SWIGLU) {
     seg[0] = GcSeg{rope_mat, rank * KC / CS, (rank + 1) * KC / CS};
     nseg = 1;
   } else {
@@ -146,13 +195,41 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   }
   const int n_units = (seg[0].kc1 - seg[0].kc0) + (nseg > 1 ? seg[1].kc1 - seg[1].kc0 : 0);
 
+  // ---- layout of the exchange, in the ring: `in`, the parts of this CTA's outputs, then `out`, what it sends ----
+  const int M = p.M;
+  // GC_ROPE: CTA 0 finishes activation rows [0, r_half), CTA 1 the rest
+  const int r_half = (M + 1) / 2, r_row0 = rank * r_half, r_rows = MODE == GC_ROPE ? (rank ? M - r_half : r_half) : 0;
+  // GC_SWIGLU: the tile's columns in groups of 16, of which CTA 0 finishes 0..2, CTA 1 3 and 4, CTA 2 5..7
+  constexpr int GLU_FIRST[4] = {0, 3, 5, 8};
+  const int glu_g0 = GLU_FIRST[rank % 3], glu_ng = GLU_FIRST[rank % 3 + 1] - glu_g0;
+  // ... and more than 64 rows in two rounds, because the ring does not hold all of them staged and arriving at once
+  constexpr int ROUNDS = MODE == GC_SWIGLU && MT > 64 ? 2 : 1, RT = MODE == GC_SWIGLU && MT > 64 ? 64 : MT;
+  const int rr = ROUNDS == 2 ? (M + 31) / 32 * 16 : M;       // rows of a round (at most RT)
+  // GC_RESIDUAL: rows that travel as bulk copies; the ring of MT = 128 has no room for the staged copy of all rows beside the
+  // arriving ones when there are more than about 100, and the others are sent straight from tensor memory
+  const int S = EIGHT ? min(M, (Cfg::RING_BYTES - GC_RES_CLUSTER * M * 64) / ((GC_RES_CLUSTER - 1) * 64) - 1) : rr;
+  const int in_pitch = EIGHT ? M * 16 : (rr | 1) * 16;       // floats of a group of 16 columns (odd: banks)
+  const int out_pitch = (S | 1) * 16;
+  float* in = staging;
+  float* out = staging + (EIGHT ? GC_RES_CLUSTER * in_pitch : MODE == GC_SWIGLU ? 4 * glu_ng * in_pitch : 2 * r_rows * 128);
+  static_assert(!EIGHT || Cfg::RING_BYTES >= GC_RES_CLUSTER * MT * 64 + (GC_RES_CLUSTER - 1) * 64 * 17, "in, and 16 rows of out");
+  static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 3 + 5) * (RT | 1) * 64, "CTA 0 and 2: four parts of three groups, five groups to send");
+  static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 2 + 2 * 6) * (RT | 1) * 64, "CTA 1: four parts of two groups, six groups of two accumulators");
+  static_assert(MODE != GC_ROPE || Cfg::RING_BYTES >= 3 * ((MT + 1) / 2) * 512, "own and arriving rows, rows to send");
+  // bytes that arrive in a round of `rows` rows
+  auto in_bytes = [&](int rows) -> uint32_t {
+    return EIGHT ? (GC_RES_CLUSTER - 1) * S * 64 : MODE == GC_SWIGLU ? (rank == 1 ? 2 : 3) * glu_ng * rows * 64 : r_rows * 512;
+  };
+
   pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(acc_full, 1);
+    mbar_init(part_full, 1);
     mbar_fence_init();
-    for (int i = 0; i < (MODE == GC_RESIDUAL ? 1 : (MODE == GC_SWIGLU ? 2 : 3)); ++i) if (!p.packed[i]) tma_prefetch_desc(&tm.a[i]);
+    mbar_expect_tx(part_full, in_bytes(rr));                 // (the first copy comes after the first cluster barrier)
+    for (int i = 0; i < (MODE == GC_RESIDUAL ? 1 : (MODE == GC_ROPE ? 3 : 2)); ++i) if (!p.packed[i]) tma_prefetch_desc(&tm.a[i]);
     tma_prefetch_desc(&tm.b);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, TMEM_COLS); tmem_relinquish(); }
@@ -167,16 +244,21 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
     if (i < n0) { s = 0; kc = seg[0].kc0 + i; } else { s = 1; kc = seg[1].kc0 + (i - n0); }
   };
 
+  // GC_RESIDUAL: a finishing thread's items (row, group of four columns) and their old values
+  constexpr int X_PER = EIGHT ? (MT * 4 + GC_EPI - 1) / GC_EPI : 1;
+  float4 xo[X_PER];
+  bool x_on[X_PER];
+
   // GC_ROPE: what a finishing thread needs to know about its items (row bookkeeping, cos / sin, destination) is
   // fetched by the epilogue warps while the MMAs run, not after the cluster barrier
   constexpr int R_ROWS_MAX = (MT + GC_ROPE_CLUSTER - 1) / GC_ROPE_CLUSTER, R_ITEMS = R_ROWS_MAX * 16;
-  constexpr int R_PER = MODE == GC_ROPE ? (R_ITEMS + 127) / 128 : 1;
+  constexpr int R_PER = MODE == GC_ROPE ? (R_ITEMS + GC_EPI - 1) / GC_EPI : 1;
   bool r_on[R_PER];
   int r_mrow[R_PER], r_lo_c[R_PER];
   float4 r_cs01[R_PER], r_cs23[R_PER];
   bf16* r_dst[R_PER];
   auto rope_meta = [&]() {
-    constexpr int ITEMS = R_ITEMS, PER = R_PER;
+    constexpr int PER = R_PER;
     const int e = threadIdx.x - 64;
     const int D = p.g.head_dim, half = D >> 1, gph = half >> 2;       // pair groups per head
     const int n_rows_mat = rope_mat == 0 ? p.H * D : p.g.n_kv_heads * D;
@@ -186,13 +268,13 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
     bf16* (&dst)[R_PER] = r_dst;
 #pragma unroll
       for (int k = 0; k < PER; ++k) {
-        const int it = e + 128 * k, ml = it >> 4, pg = it & 15;
-        const int m = rank + CS * ml;
+        const int it = e + GC_EPI * k, ml = it >> 4, pg = it & 15;
+        const int m = r_row0 + ml;
         const int hh = pg / gph, g = pg % gph;
         lo_c[k] = hh * D + 4 * g;
-        mrow[k] = m;
+        mrow[k] = ml;
         const int row_lo = t_in_mat * 128 + lo_c[k];                      // weight row within its matrix
-        on[k] = it < ITEMS && m < p.M && row_lo < n_rows_mat;
+        on[k] = ml < r_rows && row_lo < n_rows_mat;
         cs01[k] = cs23[k] = make_float4(1.f, 0.f, 1.f, 0.f);
         dst[k] = nullptr;
         if (on[k]) {
@@ -287,244 +369,213 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
       trace_mark_max(p.trace, 3);
     }
   } else {
-    // ---- epilogue, part 1: accumulators -> staged float32 rows [weight row][activation row] ----
-    const int q = warp & 3;
+    // ---- epilogue: what it needs besides the sums is fetched while the MMAs run ----
     pdl_wait();
     if (MODE == GC_ROPE) rope_meta();
-    if (MODE == GC_SWIGLU || MODE == GC_RESIDUAL) {
-      // the accumulators stay in tensor memory until every CTA of the cluster has finished its MMAs (below)
-      if (n_units > 0) mbar_wait(acc_full, 0, p.status, 32);
-    } else if (n_units > 0 && mbar_wait(acc_full, 0, p.status, 32)) {
-      tc_fence_after();
-      for (int s = 0; s < nseg; ++s) {
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(s * MT);
-        // thread = weight row q * 32 + lane; a warp writes 32 neighbouring floats of one activation row at a time
-        float* dst = staging + (size_t)s * Cfg::STAGING_FLOATS + (q * 32 + lane);
-        if (MT >= 32) {
+    if (MODE == GC_RESIDUAL) {
 #pragma unroll
-          for (int g = 0; g < MT / 32; ++g) {
-            uint32_t r[32];
-            tmem_ld32(taddr + g * 32, r);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 32; ++j) dst[(size_t)(g * 32 + j) * Cfg::PITCH] = __uint_as_float(r[j]);
-          }
-        } else {
-          uint32_t r[16];
-          tmem_ld16(taddr, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) dst[(size_t)j * Cfg::PITCH] = __uint_as_float(r[j]);
-        }
+      for (int k = 0; k < X_PER; ++k) {
+        const int it = (int)threadIdx.x - 64 + GC_EPI * k, m = it >> 2, col = t * 128 + rank * 16 + (it & 3) * 4;
+        x_on[k] = m < M && col < p.N;
+        xo[k] = x_on[k] ? *reinterpret_cast<const float4*>(p.x + (size_t)m * p.N + col) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      tc_fence_before();
     }
+    mbar_wait(acc_full, 0, p.status, 32);
   }
 
-  // ---- every thread of every CTA of the cluster: the staged accumulators are complete (GC_SWIGLU: every CTA's
-  // MMAs are complete, so every ring is free) ----
-  __syncwarp();
-  cluster_sync_all();
-
-  if (MODE == GC_RESIDUAL) {
-    // Pushed like the gate+up parts below: a thread sends the MT values of its weight row w into the shared memory
-    // of the CTA that finishes column w (CTA w / 16), buffer [source CTA][activation row][16 columns]; after the
-    // second barrier CTA `rank` adds the eight parts of its columns [16 rank, +16) in rank order, adds the residual
-    // stream in place (its old values were fetched during the exchange) and leaves the sums of squares.
-    constexpr int CP = 16;
-    static_assert(CS * MT * CP * 4 <= Cfg::RING_BYTES, "the parts of a CTA's columns must fit the ring");
-    constexpr int ITEMS = MT * 4, PER = (ITEMS + 127) / 128;   // (row m, group of four columns c4)
-    const int e = threadIdx.x - 64;
-    const bool fin = warp >= 2 && n_units > 0;
-    float4 xo[PER];
-    bool on[PER];
-    if (fin) {
-#pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        const int it = e + 128 * k, m = it >> 2, c4 = it & 3;
-        const int col = t * 128 + rank * 16 + c4 * 4;
-        on[k] = it < ITEMS && m < p.M && col < p.N;
-        xo[k] = on[k] ? *reinterpret_cast<const float4*>(p.x + (size_t)m * p.N + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+  // ---- exchange: this CTA's MMAs are complete, its ring is free. Its accumulators go to shared memory (`out`, or `in` where
+  // the columns are its own) while the others finish theirs ----
+  const int e = (int)threadIdx.x - 64;                       // epilogue thread
+  const bool epi = warp >= 2;
+  const int q = warp & 3, hf = warp >= 6 ? 1 : 0, w = q * 32 + lane;   // its tensor-memory lane = weight row of the tile
+  const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+  const int grp = w >> 4;                                    // its group of 16 columns
+#pragma unroll 1
+  for (int rd = 0; rd < ROUNDS; ++rd) {
+    const int m0 = rd * rr, Mr = min(rr, M - m0);            // rows of this round
+    __syncwarp();
+    if (rd == 0) {
+      if (warp == 0) cluster_arrive();                       // (its first thread has set up the barrier the copies complete on)
+      else cluster_arrive_relaxed();                         // (a ring is free once its MMAs are complete; nothing else to publish)
+    } else {
+      // everybody has received the first round (so `out` may be overwritten) and is through with it (`in`)
+      if (epi) {
+        asm volatile("bar.sync 5, %0;" ::"n"(GC_EPI) : "memory");
+        if (e == 0) mbar_expect_tx(part_full, in_bytes(Mr));
+        __syncwarp();
       }
-      const int q = warp & 3, w = q * 32 + lane;
-      const uint32_t dst = dsmem_addr(smem_u32(staging), (uint32_t)(w >> 4)) + (uint32_t)((rank * MT * CP + (w & 15)) * 4);
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+      if (warp == 2) cluster_arrive();
+      else cluster_arrive_relaxed();
+      cluster_wait();
+    }
+    if (epi) {
       tc_fence_after();
-      if (MT >= 32) {
-#pragma unroll
-        for (int g = 0; g < MT / 32; ++g) {
-          uint32_t r[32];
-          tmem_ld32(taddr + g * 32, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) dsmem_st(dst + (uint32_t)((g * 32 + j) * CP * 4), __uint_as_float(r[j]));
+      if (EIGHT) {
+        const bool own = grp == rank;
+        float* dst = (own ? in + rank * in_pitch : out + (grp - (grp > rank)) * out_pitch) + (w & 15);
+        const int rows = own ? M : S;
+        tmem_rows<RT>(taddr, hf, M, [&](int m, float v) { if (MT < 128 || m < rows) dst[m * 16] = v; });
+      } else if (MODE == GC_SWIGLU) {
+        const bool own = grp >= glu_g0 && grp < glu_g0 + glu_ng;
+        for (int s = 0; s < nseg; ++s) {
+          const int slot = seg[s].mat == 0 ? rank : rank + 1;  // gate parts of CTA 0 and 1, up parts of CTA 1 and 2
+          float* dst = (own ? in + (slot * glu_ng + grp - glu_g0) * in_pitch
+                            : out + (s * (8 - glu_ng) + (grp < glu_g0 ? grp : grp - glu_ng)) * out_pitch) + (w & 15);
+          tmem_rows<RT>(taddr + (uint32_t)(s * MT + m0), hf, Mr, [&](int m, float v) { dst[m * 16] = v; });
         }
       } else {
-        uint32_t r[16];
-        tmem_ld16(taddr, r);
-        tmem_ld_wait();
-#pragma unroll
-        for (int j = 0; j < 16; ++j) dsmem_st(dst + (uint32_t)(j * CP * 4), __uint_as_float(r[j]));
+        // the other CTA's rows to `out`, its own beside the place where the other's part arrives; both [warp][row][32 columns]
+        float* mine = in + (size_t)r_rows * 128 + q * r_rows * 32 + lane;
+        float* theirs = out + q * (M - r_rows) * 32 + lane;
+        const int there0 = rank ? 0 : r_half;
+        tmem_rows<RT>(taddr, hf, M, [&](int m, float v) { *(((m < r_half) == (rank == 0)) ? mine + (m - r_row0) * 32 : theirs + (m - there0) * 32) = v; });
       }
       tc_fence_before();
+      fence_smem_async();
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");   // the two warps of a quarter have staged its columns
+    }
+    if (rd == 0) cluster_wait();                             // every ring of the cluster is free
+    if (epi && hf == 0) {
+      // the first of a quarter's warps sends its columns
+      if (MODE == GC_ROPE) {
+        const int n = M - r_rows;                            // (all four warps' blocks lie in the other CTA's `in`)
+        if (lane == 0 && n > 0)
+          bulk_push(dsmem_addr(smem_u32(in + q * n * 32), (uint32_t)(rank ^ 1)), out + q * n * 32, n * 128, dsmem_addr(smem_u32(part_full), (uint32_t)(rank ^ 1)));
+      } else if ((lane & 15) == 0) {
+        const int to = EIGHT ? grp : (grp < GLU_FIRST[1] ? 0 : (grp < GLU_FIRST[2] ? 1 : 2));
+        if (to != rank) {
+          const uint32_t bar = dsmem_addr(smem_u32(part_full), (uint32_t)to), there = dsmem_addr(smem_u32(in), (uint32_t)to);
+          if (EIGHT) {
+            bulk_push(there + (uint32_t)(rank * in_pitch * 4), out + (grp - (grp > rank)) * out_pitch, S * 64, bar);
+          } else {
+            const int g0 = GLU_FIRST[to], ng = GLU_FIRST[to + 1] - g0;
+            for (int s = 0; s < nseg; ++s) {
+              const int slot = seg[s].mat == 0 ? rank : rank + 1;
+              bulk_push(there + (uint32_t)((slot * ng + grp - g0) * in_pitch * 4), out + (s * (8 - glu_ng) + (grp < glu_g0 ? grp : grp - glu_ng)) * out_pitch,
+                        Mr * 64, bar);
+            }
+          }
+        }
+      }
+    }
+    if (EIGHT && S < M) {                                    // (the same in every CTA of the cluster)
+      if (epi) {
+        const uint32_t dst = dsmem_addr(smem_u32(in + rank * in_pitch + (w & 15)), (uint32_t)grp);
+        tmem_rows<RT>(taddr, hf, M, [&](int m, float v) { if (m >= S && grp != rank) dsmem_st(dst + (uint32_t)(m * 64), v); });
+        tc_fence_before();
+      }
+      __syncwarp();
+      cluster_sync_all();
+    }
+    if (epi) {
+      asm volatile("bar.sync 5, %0;" ::"n"(GC_EPI) : "memory");   // the own parts, written by the other warps
+      mbar_wait(part_full, rd, p.status, 34);
     }
     __syncwarp();
-    cluster_sync_all();                                       // the parts have arrived (release / acquire)
-    if (fin) {
-      float ss[PER];
+    if (rd == ROUNDS - 1) cluster_arrive_relaxed();          // this CTA reads nobody's shared memory but its own from here on
+
+    if (epi) {
+      if (MODE == GC_RESIDUAL) {
+        // the eight parts of columns [16 rank, +16) in rank order, the residual stream in place and the sums of squares
 #pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        const int it = e + 128 * k, m = it >> 2, c4 = it & 3;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (it < ITEMS) {
-          const float* src = staging + m * CP + c4 * 4;
+        for (int k = 0; k < X_PER; ++k) {
+          const int it = e + GC_EPI * k, m = it >> 2, c4 = it & 3;
+          float ss = 0.f;
+          if (m < M) {
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float* src = in + m * 16 + c4 * 4;
 #pragma unroll
-          for (int rr = 0; rr < CS; ++rr) add4(acc, *reinterpret_cast<const float4*>(src + rr * MT * CP));   // rank order
+            for (int rr = 0; rr < CS; ++rr) add4(acc, *reinterpret_cast<const float4*>(src + rr * in_pitch));
+            add4(xo[k], acc);
+            if (x_on[k]) {
+              ss = xo[k].x * xo[k].x + xo[k].y * xo[k].y + xo[k].z * xo[k].z + xo[k].w * xo[k].w;
+              *reinterpret_cast<float4*>(p.x + (size_t)m * p.N + t * 128 + rank * 16 + c4 * 4) = xo[k];
+            }
+          }
+          if (p.ss_part) {
+            // the four column groups of a row sit in four neighbouring lanes
+            ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+            ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+            if (c4 == 0 && m < M) p.ss_part[(size_t)m * (((p.N + 127) >> 7) * CS) + t * CS + rank] = ss;
+          }
         }
-        add4(xo[k], acc);
-        ss[k] = xo[k].x * xo[k].x + xo[k].y * xo[k].y + xo[k].z * xo[k].z + xo[k].w * xo[k].w;
-        if (on[k]) *reinterpret_cast<float4*>(p.x + (size_t)m * p.N + t * 128 + rank * 16 + c4 * 4) = xo[k];
-      }
-      if (p.ss_part) {
-        // the four column groups of a row sit in four neighbouring lanes
+      } else if (MODE == GC_SWIGLU8) {
+        // the four gate parts and the four up parts of columns [16 rank, +16), each in rank order
+#pragma unroll
+        for (int k = 0; k < X_PER; ++k) {
+          const int it = e + GC_EPI * k, m = it >> 2, col = t * 128 + rank * 16 + (it & 3) * 4;
+          if (m < M && col < p.N) {
+            const float* src = in + m * 16 + (it & 3) * 4;
+            float4 ga = *reinterpret_cast<const float4*>(src), ua = *reinterpret_cast<const float4*>(src + 4 * in_pitch);
+#pragma unroll
+            for (int rr8 = 1; rr8 < 4; ++rr8) {
+              add4(ga, *reinterpret_cast<const float4*>(src + rr8 * in_pitch));
+              add4(ua, *reinterpret_cast<const float4*>(src + (4 + rr8) * in_pitch));
+            }
+            uint2 o;
+            o.x = pack_bf16x2(silu_f(ga.x) * ua.x, silu_f(ga.y) * ua.y);
+            o.y = pack_bf16x2(silu_f(ga.z) * ua.z, silu_f(ga.w) * ua.w);
+            *reinterpret_cast<uint2*>(p.act + (size_t)m * p.N + col) = o;
+          }
+        }
+      } else if (MODE == GC_SWIGLU) {
+        const int gpr = glu_ng * 4;                            // groups of four columns per row: 12 or 8
+        constexpr int PER = (RT * 12 + GC_EPI - 1) / GC_EPI;
+        const int part = glu_ng * in_pitch;
+        float4 ga[PER], ua[PER];
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-          float v = on[k] ? ss[k] : 0.f;
-          v += __shfl_xor_sync(0xffffffffu, v, 1);
-          v += __shfl_xor_sync(0xffffffffu, v, 2);
-          const int it = e + 128 * k, m = it >> 2;
-          if ((it & 3) == 0 && it < ITEMS && m < p.M)
-            p.ss_part[(size_t)m * (((p.N + 127) >> 7) * CS) + t * CS + rank] = v;
+          const int it = min(e + GC_EPI * k, Mr * gpr - 1), m = glu_ng == 3 ? it / 12 : it >> 3, w4 = it - m * gpr;
+          const float* src = in + (w4 >> 2) * in_pitch + m * 16 + (w4 & 3) * 4;
+          ga[k] = *reinterpret_cast<const float4*>(src);
+          ua[k] = *reinterpret_cast<const float4*>(src + 2 * part);
+          add4(ga[k], *reinterpret_cast<const float4*>(src + part));
+          add4(ua[k], *reinterpret_cast<const float4*>(src + 3 * part));
         }
-      }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
-    return;
-  }
-
-  if (MODE == GC_SWIGLU) {
-    // Push instead of pull: a thread owns weight row w of its CTA's accumulators and sends its MT values
-    // straight into the shared memory of the CTA that finishes column w (rows 0..43 -> CTA 0, 44..83 -> CTA 1,
-    // 84..127 -> CTA 2) with remote stores, which nobody waits for; after the next barrier each CTA reads only
-    // its own shared memory. Four compact buffers [MT][GLU_PITCH] per CTA: gate parts of CTA 0 and CTA 1, up
-    // parts of CTA 1 and CTA 2. (Reading the parts through distributed shared memory instead took 4.4 us.)
-    constexpr int CP = 48;                                    // floats per staged row (44 columns at most)
-    static_assert(4 * MT * CP * 4 <= Cfg::RING_BYTES, "four compact buffers must fit the ring");
-    if (warp >= 2 && n_units > 0) {
-      const int q = warp & 3, w = q * 32 + lane;
-      const int own = w < 44 ? 0 : (w < 84 ? 1 : 2);
-      const int col = w - (own == 0 ? 0 : (own == 1 ? 44 : 84));
-      const uint32_t dst0 = dsmem_addr(smem_u32(staging), (uint32_t)own);
-      tc_fence_after();
-      for (int s2 = 0; s2 < nseg; ++s2) {
-        const int slot = seg[s2].mat == 0 ? rank : rank + 1;
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(s2 * MT);
-        const uint32_t dst = dst0 + (uint32_t)((slot * MT * CP + col) * 4);
-        if (MT >= 32) {
 #pragma unroll
-          for (int g = 0; g < MT / 32; ++g) {
-            uint32_t r[32];
-            tmem_ld32(taddr + g * 32, r);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 32; ++j) dsmem_st(dst + (uint32_t)((g * 32 + j) * CP * 4), __uint_as_float(r[j]));
-          }
-        } else {
-          uint32_t r[16];
-          tmem_ld16(taddr, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) dsmem_st(dst + (uint32_t)(j * CP * 4), __uint_as_float(r[j]));
-        }
-      }
-      tc_fence_before();
-    }
-    __syncwarp();
-    cluster_sync_all();                                       // the parts have arrived (release / acquire)
-    if (warp >= 2 && n_units > 0) {
-      const int e = threadIdx.x - 64;
-      const int lo = rank == 0 ? 0 : (rank == 1 ? 44 : 84), hi = rank == 0 ? 44 : (rank == 1 ? 84 : 128);
-      const int gpr = (hi - lo) >> 2;                        // groups of four columns per row: 11, 10, 11
-      constexpr int PER = (MT * 11 + 127) / 128;
-      const float* b0 = staging;
-#pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        const int it = e + 128 * k, m = it / gpr, w4 = it % gpr;
-        const int col = t * 128 + lo + 4 * w4;
-        if (m < MT && m < p.M && col < p.N) {
-          const float* src = b0 + m * CP + 4 * w4;
-          float4 ga = *reinterpret_cast<const float4*>(src), ua = *reinterpret_cast<const float4*>(src + 2 * MT * CP);
-          add4(ga, *reinterpret_cast<const float4*>(src + MT * CP));
-          add4(ua, *reinterpret_cast<const float4*>(src + 3 * MT * CP));
+        for (int k = 0; k < PER; ++k) {
+          const int it = e + GC_EPI * k, m = glu_ng == 3 ? it / 12 : it >> 3, w4 = it - m * gpr;
+          const int col = t * 128 + glu_g0 * 16 + 4 * w4;
           uint2 o;
-          o.x = pack_bf16x2(silu_f(ga.x) * ua.x, silu_f(ga.y) * ua.y);
-          o.y = pack_bf16x2(silu_f(ga.z) * ua.z, silu_f(ga.w) * ua.w);
-          *reinterpret_cast<uint2*>(p.act + (size_t)m * p.N + col) = o;
+          o.x = pack_bf16x2(silu_f(ga[k].x) * ua[k].x, silu_f(ga[k].y) * ua[k].y);
+          o.y = pack_bf16x2(silu_f(ga[k].z) * ua[k].z, silu_f(ga[k].w) * ua[k].w);
+          if (m < Mr && col < p.N) *reinterpret_cast<uint2*>(p.act + (size_t)(m0 + m) * p.N + col) = o;
+        }
+      } else {
+        // the tile holds 128 / D whole heads; an item is (row, group of four rotation pairs): columns [lo, lo + 4) and
+        // [lo + D/2, lo + D/2 + 4) of one head
+        const int half = p.g.head_dim >> 1;
+        const float* first = rank ? in : in + (size_t)r_rows * 128;         // CTA 0's part, then CTA 1's
+        const float* second = rank ? in + (size_t)r_rows * 128 : in;
+#pragma unroll
+        for (int k = 0; k < R_PER; ++k) {
+          if (!r_on[k]) continue;
+          const int lo = r_lo_c[k] & 0xffff, hi = lo + half;
+          const int o_lo = ((lo >> 5) * r_rows + r_mrow[k]) * 32 + (lo & 31), o_hi = ((hi >> 5) * r_rows + r_mrow[k]) * 32 + (hi & 31);
+          float4 a = *reinterpret_cast<const float4*>(first + o_lo), c = *reinterpret_cast<const float4*>(first + o_hi);
+          add4(a, *reinterpret_cast<const float4*>(second + o_lo));
+          add4(c, *reinterpret_cast<const float4*>(second + o_hi));
+          const float4 t01 = r_cs01[k], t23 = r_cs23[k];
+          uint2 lo_o, hi_o;
+          if (rope_mat < 2) {
+            lo_o.x = pack_bf16x2(a.x * t01.x - c.x * t01.y, a.y * t01.z - c.y * t01.w);
+            lo_o.y = pack_bf16x2(a.z * t23.x - c.z * t23.y, a.w * t23.z - c.w * t23.w);
+            hi_o.x = pack_bf16x2(c.x * t01.x + a.x * t01.y, c.y * t01.z + a.y * t01.w);
+            hi_o.y = pack_bf16x2(c.z * t23.x + a.z * t23.y, c.w * t23.z + a.w * t23.w);
+          } else {
+            lo_o.x = pack_bf16x2(a.x, a.y); lo_o.y = pack_bf16x2(a.z, a.w);
+            hi_o.x = pack_bf16x2(c.x, c.y); hi_o.y = pack_bf16x2(c.z, c.w);
+          }
+          const int up = rope_mat == 0 ? half : (r_lo_c[k] >> 16);
+          *reinterpret_cast<uint2*>(r_dst[k]) = lo_o;
+          *reinterpret_cast<uint2*>(r_dst[k] + up) = hi_o;
         }
       }
     }
-    // nobody writes to or reads from another CTA's shared memory after the second barrier: no third one
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
-    return;
   }
-
-  if (warp >= 2 && n_units > 0) {
-    // Every finishing thread issues all its loads (distributed shared memory, residual stream) before it
-    // uses the first one: the step costs about one round trip, not one per item.
-    const int e = threadIdx.x - 64;                        // 0..127
-    const uint32_t stage_local = smem_u32(staging);
-    if (MODE == GC_ROPE) {
-      // the tile holds 128 / D whole heads. CTA `rank` takes the activation rows rank, rank + cluster size, ...; an item is
-      // (row, group of four rotation pairs): columns [lo, lo + 4) and [lo + D/2, lo + D/2 + 4) of one head
-      constexpr int ITEMS = R_ITEMS, PER = R_PER;
-      const int half = p.g.head_dim >> 1;
-      bool (&on)[R_PER] = r_on;
-      int (&mrow)[R_PER] = r_mrow, (&lo_c)[R_PER] = r_lo_c;
-      float4 (&cs01)[R_PER] = r_cs01, (&cs23)[R_PER] = r_cs23;
-      bf16* (&dst)[R_PER] = r_dst;
-      uint32_t sb[CS];
-#pragma unroll
-      for (int r = 0; r < CS; ++r) sb[r] = dsmem_addr(stage_local, (uint32_t)r);
-      float4 a[PER], c[PER];
-#pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        const int lo = lo_c[k] & 0xffff;
-        const uint32_t o_lo = (uint32_t)((mrow[k] * Cfg::PITCH + lo) * 4), o_hi = o_lo + (uint32_t)(half * 4);
-        const bool ld = (e + 128 * k) < ITEMS && mrow[k] < MT;
-        a[k] = ld ? dsmem_ld4(sb[0] + o_lo) : make_float4(0.f, 0.f, 0.f, 0.f);
-        c[k] = ld ? dsmem_ld4(sb[0] + o_hi) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int r = 1; r < CS; ++r)
-          if (ld) { add4(a[k], dsmem_ld4(sb[r] + o_lo)); add4(c[k], dsmem_ld4(sb[r] + o_hi)); }
-      }
-#pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        if (!on[k]) continue;
-        const float4 t01 = cs01[k], t23 = cs23[k];
-        uint2 lo_o, hi_o;
-        if (rope_mat < 2) {
-          lo_o.x = pack_bf16x2(a[k].x * t01.x - c[k].x * t01.y, a[k].y * t01.z - c[k].y * t01.w);
-          lo_o.y = pack_bf16x2(a[k].z * t23.x - c[k].z * t23.y, a[k].w * t23.z - c[k].w * t23.w);
-          hi_o.x = pack_bf16x2(c[k].x * t01.x + a[k].x * t01.y, c[k].y * t01.z + a[k].y * t01.w);
-          hi_o.y = pack_bf16x2(c[k].z * t23.x + a[k].z * t23.y, c[k].w * t23.z + a[k].w * t23.w);
-        } else {
-          lo_o.x = pack_bf16x2(a[k].x, a[k].y); lo_o.y = pack_bf16x2(a[k].z, a[k].w);
-          hi_o.x = pack_bf16x2(c[k].x, c[k].y); hi_o.y = pack_bf16x2(c[k].z, c[k].w);
-        }
-        const int up = rope_mat == 0 ? half : (lo_c[k] >> 16);
-        *reinterpret_cast<uint2*>(dst[k]) = lo_o;
-        *reinterpret_cast<uint2*>(dst[k] + up) = hi_o;
-      }
-    }
-  }
-
-  // nobody leaves (and gives up its shared memory) before every CTA of the cluster has read it
+  // nobody leaves while a copy out of its shared memory may still be on its way
   __syncwarp();
-  cluster_sync_all();
+  cluster_wait();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
