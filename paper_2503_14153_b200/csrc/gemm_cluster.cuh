@@ -57,6 +57,7 @@ struct ClusterGemmParams {
   bf16* act;                    // GC_SWIGLU(8): [M][N] bf16
   // GC_ROPE: tiles [0, tile0[1]) belong to q, [tile0[1], tile0[2]) to k, the rest to v
   int tile0[3];
+  int tile_first;               // first tile of the launch (a prompt's last layer takes k and v, or q, alone)
   int H;                        // query heads
   int layer;
   Rows rows;
@@ -173,7 +174,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   KTrace kt(p.trace);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
-  const int t = blockIdx.x / CS;                             // weight tile (GC_SWIGLU: tile pair; GC_ROPE: of the stacked q, k, v)
+  const int t = blockIdx.x / CS + (MODE == GC_ROPE ? p.tile_first : 0);   // weight tile (GC_SWIGLU: tile pair; GC_ROPE: of the stacked q, k, v)
   const int KC = p.KC;
   int rope_mat = 0;
   if (MODE == GC_ROPE) rope_mat = t >= p.tile0[2] ? 2 : (t >= p.tile0[1] ? 1 : 0);

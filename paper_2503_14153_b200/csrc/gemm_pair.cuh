@@ -66,6 +66,7 @@ struct PairGemmParams {
   float* out;                               // GP_PLAIN: sums; GP_RESIDUAL: residual stream [M][n_cols]
   bf16* act;                                // GP_SWIGLU: [M][n_cols]
   // GP_ROPE
+  int kind0;                                // what the first matrix is: 0 q, 1 k (a prompt's last layer projects k and v alone)
   int H, layer;
   Rows rows;
   const float2* cs;                         // [position][head_dim / 2] (cos, sin)
@@ -471,13 +472,14 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           }
           group_bar(1 + hf);
         } else {
-          const int n_rows_mat = (mat == 0 ? p.H : p.g.n_kv_heads) * D;
+          const int kind = mat + p.kind0;                        // 0 q, 1 k, 2 v
+          const int n_rows_mat = (kind == 0 ? p.H : p.g.n_kv_heads) * D;
           const int row = (nt_c - p.mat_tile0[mat]) * 128 + wl;  // weight row within its matrix
           const bool on = nt < p.n_tiles && row < n_rows_mat;
           const int head = row / D, dim = row - head * D;
           const int half = D >> 1;
           const size_t lh = ((size_t)p.layer * p.g.n_kv_heads + head) * p.g.pool_pages() * 2 * p.g.block_elems();
-          if (mat == 2) {
+          if (kind == 2) {
             bf16* dst = p.pool + lh + p.g.block_elems();
 #pragma unroll 1
             for (int g = 0; g < HC / 32; ++g) {
@@ -518,7 +520,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
                                 // (the rounding of the other kernels that rotate: one product rounded, the other fused into the sum)
                 const bf16 lo = __float2bfloat16_rn(__fmaf_rn(a, t[j].x, -__fmul_rn(c, t[j].y)));
                 const bf16 hi = __float2bfloat16_rn(__fmaf_rn(c, t[j].x, __fmul_rn(a, t[j].y)));
-                if (mat == 0) {
+                if (kind == 0) {
                   bf16* dst = p.q + (size_t)(m0 + jb + j) * p.H * D + head * D + di;
                   dst[0] = lo;
                   dst[half] = hi;

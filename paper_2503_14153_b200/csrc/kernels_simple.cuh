@@ -104,6 +104,37 @@ __global__ void prefill_keep_last(Rows rows, const int* __restrict__ offsets, co
   if (threadIdx.x == 0) n_seq[b] = len;
 }
 
+// Rows of a pass that are last tokens of prompts, for the rest of the last layer: residual stream and normed operand of row
+// end_row[g] of the pass to row g, and the sequence's length.
+__global__ void __launch_bounds__(256)
+gather_prompt_ends(const int* __restrict__ end_row, const int* __restrict__ end_pos, const float* __restrict__ x, const bf16* __restrict__ u,
+                   float* __restrict__ x_end, bf16* __restrict__ u_end, int* __restrict__ n_seq, int d, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  const int g = blockIdx.x;
+  const size_t m = end_row[g];
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  for (int c = threadIdx.x; c < (d >> 2); c += blockDim.x) {
+    reinterpret_cast<float4*>(x_end + (size_t)g * d)[c] = reinterpret_cast<const float4*>(x + m * d)[c];
+    reinterpret_cast<uint2*>(u_end + (size_t)g * d)[c] = reinterpret_cast<const uint2*>(u + m * d)[c];
+  }
+  if (threadIdx.x == 0) n_seq[g] = end_pos[g] + 1;
+}
+
+// Before prompts are processed: zeros in every cache slot that they do not fill, from the page of a sequence's first free slot on
+// (attention reads whole tiles of keys; what lies past a sequence's end has weight zero but must be finite). A sequence's pages
+// that its prompt fills are left alone: clearing the whole pool took 45 us for a 2048-token prompt and 8 layers of the 7B shape.
+__global__ void __launch_bounds__(256)
+clear_free_pages(uint4* __restrict__ pool, const int* __restrict__ offsets, int batch, int pages_per_seq, int max_batch, int page_size,
+                 int pair_vecs, int share) {
+  // grid (sequences times the CTAs that share one's pages, layers * heads); pool page p * max_batch + b is page p of sequence b
+  const int b = blockIdx.x / share, len = b < batch ? offsets[b + 1] - offsets[b] : 0;
+  uint4* base = pool + ((size_t)blockIdx.y * pages_per_seq * max_batch + b) * pair_vecs;
+  for (int p = len / page_size + blockIdx.x % share; p < pages_per_seq; p += share)
+    for (int i = threadIdx.x; i < pair_vecs; i += blockDim.x) base[(size_t)p * max_batch * pair_vecs + i] = make_uint4(0, 0, 0, 0);
+}
+
 // ------------------------------------------------------------------ RMSNorm (+ residual)
 // u[m] = T(x[m] / rms(x[m]) * g); optionally the unrounded normed row goes to hid (final norm).
 template <typename T>

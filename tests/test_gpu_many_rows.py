@@ -174,3 +174,36 @@ def test_op_linear_many_rows_error(torch, M, N, K, streamed):
     y = spec_op_linear(x, w).double()
     want = x.double() @ w.double().T
     assert ((y - want).norm() / want.norm()).item() <= 1.005 * streamed
+
+
+@pytest.mark.parametrize("lens,layers,hd,batch", [
+    ([129], 2, 128, 1),             # two chunks in two passes: the first ends no prompt
+    ([256], 1, 64, 1),              # the only layer is the last one; the last row of a chunk
+    ([300], 2, 128, 1),             # one pass of three chunks
+    ([384, 1, 130, 128], 2, 64, 5), # ragged, a prompt of one token, whole chunks, a free sequence
+    ([2400, 7], 1, 128, 2),         # 20 chunks: the first pass ends no prompt, the second both
+])
+def test_last_layer_of_a_prompt_for_its_last_rows(torch, lens, layers, hd, batch):
+    """Prompt processing takes only the prompts' last tokens through the rest of the last layer: first token, hidden state, cache rows of
+    the whole prompts and the steps that follow against an oracle each. A second, shorter set of prompts in the same context finds
+    the slots behind it cleared."""
+    from oracle.decoder import OracleModel
+    from oracle.spec import OracleSpecDecoder
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    from tests_lockstep import run_lockstep_batch
+    cfg = BASE.with_(n_layers=layers, d_model=512, n_heads=512 // hd, n_kv_heads=512 // hd, head_dim=hd, d_ffn=1344, tree_nodes=16, seed=130 + len(lens))
+    w = draw_weights(cfg)
+    tree = build_tree(cfg.topk, 16)
+    room = max(lens) + 40
+    gpu = SpecDecoder(cfg, upload_weights(cfg, w), tree, room, max_batch=batch, flags=B.FLAG_KEEP_LOGITS)
+    model = OracleModel(cfg, w)
+    for k, sizes in enumerate((lens, [max(1, n // 2) for n in reversed(lens)])):
+        prompts = [draw_prompt(cfg.with_(seed=150 + 10 * k + i), n) for i, n in enumerate(sizes)]
+        oracles = {b: OracleSpecDecoder(model, tree, room) for b in {0, len(sizes) - 1}}
+        reps = run_lockstep_batch(cfg, gpu, oracles, prompts, 2, TOL_BF16, TIE_GAP, tie_from_row_error=True)
+        for b in oracles:
+            assert reps[b].steps == 2
+        k0, v0 = gpu.read_kv(0, layers - 1, len(prompts[0]) + 30, 2)
+        assert not k0.any() and not v0.any()          # nothing was written there since the prompts were processed
+    gpu.close()
