@@ -28,6 +28,9 @@
 //    gate = G0 + G1, up = U1 + U2, act = bf16(SiLU(gate) * up).
 //  * GC_SWIGLU8 (the same projections where there are few tiles): a cluster of 8 per pair (gate tile t, up tile t), CTAs 0 to 3
 //    streaming a quarter of the gate tile's K chunks each, 4 to 7 the up tile's; columns as in GC_RESIDUAL.
+//  * GC_PLAIN (a projection by itself; lm_head): a cluster of 1 to 8 per tile, CTA r streaming the r-th part of the K chunks, its
+//    first half into one accumulator and its second into another (the error of a running sum grows with its
+//    length), and finishing a block of rows: float32 sums, and where asked each row's largest in the tile.
 //  * GC_ROPE (query, key and value projections, stacked): a cluster of 2 CTAs per 128-row tile of the
 //    stacked matrices, each streaming half of the K chunks (96 pairs on the 7B shape: all co-resident, which
 //    96 clusters of 3 are not). A tile holds whole heads (head_dim 64 or
@@ -44,7 +47,7 @@
 
 namespace spec {
 
-constexpr int GC_RESIDUAL = 0, GC_SWIGLU = 1, GC_ROPE = 2, GC_SWIGLU8 = 3;
+constexpr int GC_RESIDUAL = 0, GC_SWIGLU = 1, GC_ROPE = 2, GC_SWIGLU8 = 3, GC_PLAIN = 4;
 constexpr int GC_THREADS = 320, GC_EPI = GC_THREADS - 64;     // producer, MMA issuer, eight epilogue warps (two per SM quarter)
 constexpr int GC_RES_CLUSTER = 8, GC_GLU_CLUSTER = 3, GC_ROPE_CLUSTER = 2;
 
@@ -55,6 +58,13 @@ struct ClusterGemmParams {
   float* x;                     // GC_RESIDUAL: [M][N] float32 residual stream, updated in place
   float* ss_part;               // GC_RESIDUAL: [M][ceil(N/128) * 8] sums of squares of the updated pieces, or nullptr
   bf16* act;                    // GC_SWIGLU(8): [M][N] bf16
+  // GC_PLAIN: sums to y[M][ldy], columns below N (y may be nullptr), and of every row's sums in this tile the largest and its column (value
+  // descending, column ascending) to best_val / best_idx [M][tiles] (may be nullptr); clear: four ints set to zero, or nullptr
+  float* y;
+  size_t ldy;
+  float* best_val;
+  int* best_idx;
+  int* clear;
   // GC_ROPE: tiles [0, tile0[1]) belong to q, [tile0[1], tile0[2]) to k, the rest to v
   int tile0[3];
   int tile_first;               // first tile of the launch (a prompt's last layer takes k and v, or q, alone)
@@ -83,6 +93,11 @@ template <int MT> struct ClusterCfg {
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_nctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
   return r;
 }
 __device__ __forceinline__ void cluster_sync_all() {
@@ -121,8 +136,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 
 // Rows of one accumulator (or of a stretch of at most MT of its columns) at `taddr`, in groups of 16 of which the two epilogue warps of an SM quarter take every
 // second one: put(row, value) in the thread that owns the weight row, for rows below M.
+// With `second` > 0 the accumulator that many columns further on is added.
 template <int MT, typename F>
-__device__ __forceinline__ void tmem_rows(uint32_t taddr, int hf, int M, F&& put) {
+__device__ __forceinline__ void tmem_rows(uint32_t taddr, int hf, int M, F&& put, int second = 0) {
   constexpr int NG = MT >= 32 ? MT / 32 : 1, U = NG < 2 ? NG : 2;   // (two groups at a time: registers)
   if (MT == 16 && hf) return;
 #pragma unroll
@@ -132,6 +148,17 @@ __device__ __forceinline__ void tmem_rows(uint32_t taddr, int hf, int M, F&& put
     for (int k = 0; k < U; ++k)
       if ((2 * (k0 + k) + hf) * 16 < M) tmem_ld16(taddr + (2 * (k0 + k) + hf) * 16, r[k]);      // (the same in the whole warp)
     tmem_ld_wait();
+    if (second) {
+      uint32_t r2[U][16];
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if ((2 * (k0 + k) + hf) * 16 < M) tmem_ld16(taddr + second + (2 * (k0 + k) + hf) * 16, r2[k]);
+      tmem_ld_wait();
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) r[k][j] = __float_as_uint(__uint_as_float(r[k][j]) + __uint_as_float(r2[k][j]));
+    }
 #pragma unroll
     for (int k = 0; k < U; ++k) {
       const int m0 = (2 * (k0 + k) + hf) * 16;
@@ -158,8 +185,9 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   using Cfg = ClusterCfg<MT>;
   constexpr int STAGES = Cfg::STAGES;
   constexpr bool EIGHT = MODE == GC_RESIDUAL || MODE == GC_SWIGLU8;      // eight CTAs, each finishing 16 columns
-  constexpr int CS = EIGHT ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER);
-  constexpr int TMEM_COLS = ((MODE == GC_SWIGLU ? 2 : 1) * MT < 32) ? 32 : (MODE == GC_SWIGLU ? 2 : 1) * MT;   // 32, 64 or 128
+  constexpr bool PLAIN = MODE == GC_PLAIN;
+  const int CS = PLAIN ? (int)cluster_nctarank() : (EIGHT ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER));
+  constexpr int TMEM_COLS = (MODE == GC_SWIGLU || PLAIN ? 2 : 1) * MT < 32 ? 32 : (MODE == GC_SWIGLU || PLAIN ? 2 : 1) * MT;   // 32 to 256
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* tiles = smem_raw + (((raw + 1023u) & ~1023u) - raw);
@@ -186,6 +214,10 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   if (MODE == GC_SWIGLU8) {
     seg[0] = GcSeg{rank >> 2, (rank & 3) * KC / 4, ((rank & 3) + 1) * KC / 4};
     nseg = 1;
+  } else if (PLAIN) {
+    const int k0 = rank * KC / CS, k1 = (rank + 1) * KC / CS, mid = (k0 + k1 + 1) >> 1;
+    seg[nseg++] = GcSeg{0, k0, mid};
+    if (mid < k1) seg[nseg++] = GcSeg{0, mid, k1};
   } else if (MODE != GC_SWIGLU) {
     seg[0] = GcSeg{rope_mat, rank * KC / CS, (rank + 1) * KC / CS};
     nseg = 1;
@@ -203,23 +235,26 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   // GC_SWIGLU: the tile's columns in groups of 16, of which CTA 0 finishes 0..2, CTA 1 3 and 4, CTA 2 5..7
   constexpr int GLU_FIRST[4] = {0, 3, 5, 8};
   const int glu_g0 = GLU_FIRST[rank % 3], glu_ng = GLU_FIRST[rank % 3 + 1] - glu_g0;
-  // ... and more than 64 rows in two rounds, because the ring does not hold all of them staged and arriving at once
-  constexpr int ROUNDS = MODE == GC_SWIGLU && MT > 64 ? 2 : 1, RT = MODE == GC_SWIGLU && MT > 64 ? 64 : MT;
+  // ... and more than 64 rows in two rounds, because the ring does not hold all of them staged and arriving at once (GC_PLAIN too)
+  constexpr int ROUNDS = (MODE == GC_SWIGLU || PLAIN) && MT > 64 ? 2 : 1, RT = ROUNDS == 2 ? 64 : MT;
   const int rr = ROUNDS == 2 ? (M + 31) / 32 * 16 : M;       // rows of a round (at most RT)
   // GC_RESIDUAL: rows that travel as bulk copies; the ring of MT = 128 has no room for the staged copy of all rows beside the
   // arriving ones when there are more than about 100, and the others are sent straight from tensor memory
   const int S = EIGHT ? min(M, (Cfg::RING_BYTES - GC_RES_CLUSTER * M * 64) / ((GC_RES_CLUSTER - 1) * 64) - 1) : rr;
+  // GC_PLAIN: CTA r finishes the r-th block of rows of a round
+  const int rb = PLAIN ? (rr + CS - 1) / CS : 0;
   const int in_pitch = EIGHT ? M * 16 : (rr | 1) * 16;       // floats of a group of 16 columns (odd: banks)
   const int out_pitch = (S | 1) * 16;
   float* in = staging;
-  float* out = staging + (EIGHT ? GC_RES_CLUSTER * in_pitch : MODE == GC_SWIGLU ? 4 * glu_ng * in_pitch : 2 * r_rows * 128);
+  float* out = staging + (EIGHT ? GC_RES_CLUSTER * in_pitch : MODE == GC_SWIGLU ? 4 * glu_ng * in_pitch : PLAIN ? CS * rb * 128 : 2 * r_rows * 128);
+  static_assert(!PLAIN || Cfg::RING_BYTES >= (2 * RT + 8) * 512, "a round's rows staged, and eight parts of this CTA's block");
   static_assert(!EIGHT || Cfg::RING_BYTES >= GC_RES_CLUSTER * MT * 64 + (GC_RES_CLUSTER - 1) * 64 * 17, "in, and 16 rows of out");
   static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 3 + 5) * (RT | 1) * 64, "CTA 0 and 2: four parts of three groups, five groups to send");
   static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 2 + 2 * 6) * (RT | 1) * 64, "CTA 1: four parts of two groups, six groups of two accumulators");
   static_assert(MODE != GC_ROPE || Cfg::RING_BYTES >= 3 * ((MT + 1) / 2) * 512, "own and arriving rows, rows to send");
   // bytes that arrive in a round of `rows` rows
   auto in_bytes = [&](int rows) -> uint32_t {
-    return EIGHT ? (GC_RES_CLUSTER - 1) * S * 64 : MODE == GC_SWIGLU ? (rank == 1 ? 2 : 3) * glu_ng * rows * 64 : r_rows * 512;
+    return EIGHT ? (GC_RES_CLUSTER - 1) * S * 64 : MODE == GC_SWIGLU ? (rank == 1 ? 2 : 3) * glu_ng * rows * 64 : PLAIN ? (CS - 1) * max(0, min(rb, rows - rank * rb)) * 512 : r_rows * 512;
   };
 
   pdl_launch_dependents();
@@ -230,7 +265,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
     mbar_init(part_full, 1);
     mbar_fence_init();
     mbar_expect_tx(part_full, in_bytes(rr));                 // (the first copy comes after the first cluster barrier)
-    for (int i = 0; i < (MODE == GC_RESIDUAL ? 1 : (MODE == GC_ROPE ? 3 : 2)); ++i) if (!p.packed[i]) tma_prefetch_desc(&tm.a[i]);
+    for (int i = 0; i < (MODE == GC_RESIDUAL || PLAIN ? 1 : (MODE == GC_ROPE ? 3 : 2)); ++i) if (!p.packed[i]) tma_prefetch_desc(&tm.a[i]);
     tma_prefetch_desc(&tm.b);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, TMEM_COLS); tmem_relinquish(); }
@@ -373,6 +408,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
     // ---- epilogue: what it needs besides the sums is fetched while the MMAs run ----
     pdl_wait();
     if (MODE == GC_ROPE) rope_meta();
+    if (PLAIN && p.clear && blockIdx.x == 0 && threadIdx.x < 68) p.clear[threadIdx.x - 64] = 0;
     if (MODE == GC_RESIDUAL) {
 #pragma unroll
       for (int k = 0; k < X_PER; ++k) {
@@ -424,6 +460,12 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
                             : out + (s * (8 - glu_ng) + (grp < glu_g0 ? grp : grp - glu_ng)) * out_pitch) + (w & 15);
           tmem_rows<RT>(taddr + (uint32_t)(s * MT + m0), hf, Mr, [&](int m, float v) { dst[m * 16] = v; });
         }
+      } else if (PLAIN) {
+        // rows of this CTA's block to its place in `in`, all others to `out`; the two halves of the run are added here
+        float* mine = in + w;                                  // (block `rank` of `in` starts at row rank * rb)
+        float* rest = out + w;
+        const int own0 = rank * rb, own1 = own0 + rb;
+        tmem_rows<RT>(taddr + (uint32_t)m0, hf, Mr, [&](int m, float v) { *((m >= own0 && m < own1 ? mine : rest) + m * 128) = v; }, nseg > 1 ? MT : 0);
       } else {
         // the other CTA's rows to `out`, its own beside the place where the other's part arrives; both [warp][row][32 columns]
         float* mine = in + (size_t)r_rows * 128 + q * r_rows * 32 + lane;
@@ -436,7 +478,15 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
       asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");   // the two warps of a quarter have staged its columns
     }
     if (rd == 0) cluster_wait();                             // every ring of the cluster is free
-    if (epi && hf == 0) {
+    if (PLAIN && CS > 1 && epi) {
+      asm volatile("bar.sync 6, %0;" ::"n"(GC_EPI) : "memory");   // all columns are staged
+      if (warp == 2 && lane < CS && lane != rank) {
+        const int rows = min(rb, Mr - lane * rb);
+        if (rows > 0)
+          bulk_push(dsmem_addr(smem_u32(in + (size_t)rank * rb * 128), (uint32_t)lane), out + (size_t)lane * rb * 128, rows * 512, dsmem_addr(smem_u32(part_full), (uint32_t)lane));
+      }
+    }
+    if (!PLAIN && epi && hf == 0) {
       // the first of a quarter's warps sends its columns
       if (MODE == GC_ROPE) {
         const int n = M - r_rows;                            // (all four warps' blocks lie in the other CTA's `in`)
@@ -498,6 +548,33 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
             ss += __shfl_xor_sync(0xffffffffu, ss, 1);
             ss += __shfl_xor_sync(0xffffffffu, ss, 2);
             if (c4 == 0 && m < M) p.ss_part[(size_t)m * (((p.N + 127) >> 7) * CS) + t * CS + rank] = ss;
+          }
+        }
+      } else if (PLAIN) {
+        // a warp has a row: 128 columns of it in every part, added in rank order
+        const int rows = min(rb, Mr - rank * rb), n0 = t * 128 + lane * 4;
+        const bool vec = (p.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 15) == 0 && n0 + 4 <= p.N;
+        for (int i = warp - 2; i < rows; i += GC_EPI / 32) {
+          const float* src = in + i * 128 + lane * 4;
+          float4 a = *reinterpret_cast<const float4*>(src);
+          for (int r = 1; r < CS; ++r) add4(a, *reinterpret_cast<const float4*>(src + (size_t)r * rb * 128));
+          const int m = m0 + rank * rb + i;
+          const float v[4] = {a.x, a.y, a.z, a.w};
+          if (p.y) {
+            float* dst = p.y + (size_t)m * p.ldy + n0;
+            if (vec) *reinterpret_cast<float4*>(dst) = a;
+            else
+              for (int j = 0; j < 4; ++j) if (n0 + j < p.N) dst[j] = v[j];
+          }
+          if (p.best_val) {
+            float bv = -INFINITY;
+            int bi = 0x7fffffff;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (n0 + j < p.N && better(v[j], n0 + j, bv, bi)) { bv = v[j]; bi = n0 + j; }
+            warp_argmax(bv, bi);
+            const int tiles_n = (p.N + 127) >> 7;
+            if (lane == 0) { p.best_val[(size_t)m * tiles_n + t] = bv; p.best_idx[(size_t)m * tiles_n + t] = bi; }
           }
         }
       } else if (MODE == GC_SWIGLU8) {

@@ -199,6 +199,44 @@ cudaError_t launch_gs(cudaStream_t st, bool pdl, const GemmPlan& g, const Stream
   }
 }
 
+template <int MT, int MODE>
+cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int grid, int cluster, const StreamTmaps& tm, const ClusterGemmParams& p, bool* attr_set) {
+  if (!*attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_cluster<MT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<MT>::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    *attr_set = true;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GC_THREADS); cfg.dynamicSmemBytes = (size_t)ClusterCfg<MT>::SMEM_BYTES; cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, gemm_cluster<MT, MODE>, tm, p);
+}
+
+// CTAs that share each tile of a GC_PLAIN launch: as many as let all clusters be resident at once (96 KB of shared memory a CTA) and have
+// two K chunks each; 0: more tiles than CTAs fit, the weight streamer deals them out evenly.
+int plain_cluster(int tiles, int KC, int max_ctas) {
+  constexpr int size[] = {8, 6, 4, 3, 2, 1}, most[] = {33, 45, 71, 93, 148, SM_SLOTS};
+  for (int i = 0; i < 6; ++i)
+    if (tiles <= most[i] && 2 * size[i] <= std::max(KC, 2) && (long long)tiles * size[i] <= max_ctas) return size[i];
+  return 0;
+}
+
+cudaError_t launch_gc_plain(cudaStream_t st, bool pdl, int tiles, int cluster, const StreamTmaps& tm, const ClusterGemmParams& p) {
+  static bool set[4][kAttrDevices] = {};
+  switch (mt_for_rows(p.M)) {
+    case 16: return launch_gc_mt<16, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[0]));
+    case 32: return launch_gc_mt<32, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[1]));
+    case 64: return launch_gc_mt<64, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[2]));
+    default: return launch_gc_mt<128, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[3]));
+  }
+}
+
 PartView plan_view(const GemmPlan& g) {
   PartView v{};
   v.part = g.p.part; v.slot_stride = g.p.slot_stride; v.ld = g.p.n_tiles * 128; v.seg = g.p.seg;
@@ -694,26 +732,6 @@ bool cluster_gemm_ok(const spec_ctx* c, int mode, int M, int K) {
   return KC >= GC_ROPE_CLUSTER && (c->cfg.head_dim == 64 || c->cfg.head_dim == 128);
 }
 
-template <int MT, int MODE>
-cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int grid, const StreamTmaps& tm, const ClusterGemmParams& p, bool* attr_set) {
-  if (!*attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_cluster<MT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<MT>::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    *attr_set = true;
-  }
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GC_THREADS); cfg.dynamicSmemBytes = (size_t)ClusterCfg<MT>::SMEM_BYTES; cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = MODE == GC_RESIDUAL || MODE == GC_SWIGLU8 ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER);
-  at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, gemm_cluster<MT, MODE>, tm, p);
-}
-
 constexpr int ROPE_ALL = 0, ROPE_Q = 1, ROPE_KV = 2;     // which of the stacked projections a GC_ROPE launch takes
 
 // x[M,N] += in[M,K] * W^T (GC_RESIDUAL, mats[0] = W), act_out[M,N] = bf16(SiLU(in W_g^T) * in W_u^T)
@@ -749,38 +767,38 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
   }
   p.trace = c->next_trace(gemm_kind_name(kind));
   if (mode == GC_SWIGLU && K / 64 >= 4 && n_tiles <= GC_GLU8_TILES) mode = GC_SWIGLU8;
-  const int grid = n_tiles * (mode == GC_SWIGLU ? GC_GLU_CLUSTER : mode == GC_ROPE ? GC_ROPE_CLUSTER : GC_RES_CLUSTER);
+  const int cs = mode == GC_SWIGLU ? GC_GLU_CLUSTER : mode == GC_ROPE ? GC_ROPE_CLUSTER : GC_RES_CLUSTER, grid = n_tiles * cs;
   cudaError_t e = cudaErrorInvalidValue;
   {
     ProfScope ps(c, kind);
     bool* as = c->gc_attr_set;
     if (mode == GC_RESIDUAL) {
       switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_RESIDUAL>(c->stream, c->pdl, grid, tm, p, as + 0); break;
-        case 32: e = launch_gc_mt<32, GC_RESIDUAL>(c->stream, c->pdl, grid, tm, p, as + 1); break;
-        case 64: e = launch_gc_mt<64, GC_RESIDUAL>(c->stream, c->pdl, grid, tm, p, as + 2); break;
-        default: e = launch_gc_mt<128, GC_RESIDUAL>(c->stream, c->pdl, grid, tm, p, as + 3); break;
+        case 16: e = launch_gc_mt<16, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 0); break;
+        case 32: e = launch_gc_mt<32, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 1); break;
+        case 64: e = launch_gc_mt<64, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 2); break;
+        default: e = launch_gc_mt<128, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 3); break;
       }
     } else if (mode == GC_SWIGLU8) {
       switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_SWIGLU8>(c->stream, c->pdl, grid, tm, p, as + 12); break;
-        case 32: e = launch_gc_mt<32, GC_SWIGLU8>(c->stream, c->pdl, grid, tm, p, as + 13); break;
-        case 64: e = launch_gc_mt<64, GC_SWIGLU8>(c->stream, c->pdl, grid, tm, p, as + 14); break;
-        default: e = launch_gc_mt<128, GC_SWIGLU8>(c->stream, c->pdl, grid, tm, p, as + 15); break;
+        case 16: e = launch_gc_mt<16, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 12); break;
+        case 32: e = launch_gc_mt<32, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 13); break;
+        case 64: e = launch_gc_mt<64, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 14); break;
+        default: e = launch_gc_mt<128, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 15); break;
       }
     } else if (mode == GC_SWIGLU) {
       switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_SWIGLU>(c->stream, c->pdl, grid, tm, p, as + 4); break;
-        case 32: e = launch_gc_mt<32, GC_SWIGLU>(c->stream, c->pdl, grid, tm, p, as + 5); break;
-        case 64: e = launch_gc_mt<64, GC_SWIGLU>(c->stream, c->pdl, grid, tm, p, as + 6); break;
-        default: e = launch_gc_mt<128, GC_SWIGLU>(c->stream, c->pdl, grid, tm, p, as + 11); break;
+        case 16: e = launch_gc_mt<16, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 4); break;
+        case 32: e = launch_gc_mt<32, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 5); break;
+        case 64: e = launch_gc_mt<64, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 6); break;
+        default: e = launch_gc_mt<128, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 11); break;
       }
     } else {
       switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_ROPE>(c->stream, c->pdl, grid, tm, p, as + 7); break;
-        case 32: e = launch_gc_mt<32, GC_ROPE>(c->stream, c->pdl, grid, tm, p, as + 8); break;
-        case 64: e = launch_gc_mt<64, GC_ROPE>(c->stream, c->pdl, grid, tm, p, as + 9); break;
-        default: e = launch_gc_mt<128, GC_ROPE>(c->stream, c->pdl, grid, tm, p, as + 10); break;
+        case 16: e = launch_gc_mt<16, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 7); break;
+        case 32: e = launch_gc_mt<32, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 8); break;
+        case 64: e = launch_gc_mt<64, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 9); break;
+        default: e = launch_gc_mt<128, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 10); break;
       }
     }
     c->launches++;
@@ -2014,6 +2032,16 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     return op_linear_status(p.status, st);
   }
   if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, g.MT)) return SPEC_E_CUDA;
+  const int cs = M <= 128 ? plain_cluster(g.p.n_tiles, K / 64, ctas) : 0;
+  if (2LL * g.p.n_tiles * cs >= g.grid) {
+    // few rows: the CTAs of a tile finish its sums on the chip. Not where their half runs would be longer than the streaming kernel's
+    // runs (few tiles and a long inner dimension): the error of a running sum grows with its length.
+    ClusterGemmParams p{};
+    p.M = M; p.K = K; p.KC = K / 64; p.N = N; p.y = y; p.ldy = (size_t)N;
+    p.status = reinterpret_cast<int*>(scratch + scratch_floats);
+    if (cudaMemsetAsync(p.status, 0, 16, st) != cudaSuccess || launch_gc_plain(st, false, g.p.n_tiles, cs, tm, p) != cudaSuccess) return SPEC_E_CUDA;
+    return op_linear_status(p.status, st);
+  }
   g.p.part = scratch;
   g.p.slot_stride = (size_t)M * g.p.n_tiles * 128;
   g.p.l2_prefetch = 0;

@@ -264,6 +264,27 @@ def test_op_linear_bf16_vs_oracle_matmul(torch, M, N, K, ctas):
     assert err < 1e-5, err
 
 
+@pytest.mark.parametrize("M,N,K", [(16, 128, 64), (32, 131, 128), (48, 1030, 192), (16, 4224, 1024), (64, 4225, 1024), (64, 5761, 768),
+                                   (80, 9088, 512), (112, 11904, 320), (128, 12001, 256), (64, 18944, 128), (96, 19000, 128), (128, 37888, 64)])
+def test_op_linear_few_rows_in_clusters(torch, M, N, K):
+    """Up to 128 rows the CTAs of a tile finish its sums on the chip: one to eight CTAs a tile, tiles that are not full, columns that are no
+    multiple of four (and rows of y off 16-byte boundaries), row blocks that do not divide, two rounds above 64 rows, one K chunk."""
+    from paper_2503_14153_b200 import spec_op_linear
+    from paper_2503_14153_b200.binding import spec_op_linear_static
+    g = torch.Generator().manual_seed(M + N + K)
+    x = torch.randn((M, K), generator=g).bfloat16().cuda()
+    w = (torch.randn((N, K), generator=g) * 0.02).bfloat16().cuda()
+    want = x.double() @ w.double().T
+    y = spec_op_linear(x, w)
+    # float32 sums of K products: K / 2 roundings of the running sum, each at most 2^-24 of the sum of the magnitudes
+    bound = (K / 2 + 8) * 2.0 ** -24 * (x.double().abs() @ w.double().abs().T)
+    assert ((y.double() - want).abs() <= bound).all()
+    if 8 * M * N + M * K < (1 << 20):                       # (the built-in scratch is limited)
+        flat = torch.full((M * N + 2,), 7.0, device="cuda")
+        spec_op_linear_static(x, w, flat[1:1 + M * N].view(M, N))
+        assert torch.equal(flat[1:1 + M * N].view(M, N), y) and flat[0] == 7 and flat[-1] == 7
+
+
 def test_op_linear_fp32_vs_oracle_matmul(torch):
     from paper_2503_14153_b200 import spec_op_linear
     rng = np.random.default_rng(3)
