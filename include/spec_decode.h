@@ -277,8 +277,9 @@ int spec_pack_weight(const void *w, int32_t rows, int32_t cols, void *packed, vo
  * dealt in equal contiguous runs to `ctas` persistent CTAs, runs that end inside a tile leave
  * float32 partial sums in `scratch` (DEVICE, spec_op_linear_scratch_floats() + 4 floats; the
  * last four hold the call's status word) and a second kernel adds a tile's partial sums in CTA
- * order into y. More than 128 rows of bf16 with two (128 x 128) tiles or more a CTA run as whole output tiles on pairs of SMs (at most `ctas` CTAs, at least
- * two), which write y themselves; of scratch only the status word is used then. float32 runs the CUDA-core row kernel
+ * order into y. Up to 128 rows, where a cluster of at most eight CTAs a tile employs at least half as many CTAs as that dealing would and
+ * at most `ctas`, the CTAs of a tile add their sums on the chip and write y themselves. More than 128 rows of bf16 with two (128 x 128) tiles or more a CTA run as whole output tiles on pairs of SMs (at most `ctas` CTAs, at least
+ * two), which write y themselves; of scratch only the status word is used in these cases. float32 runs the CUDA-core row kernel
  * (ctas and scratch ignored).
  * M <= 2048; for bf16 K % 64 == 0, M % 16 == 0, N >= 128, 1 <= ctas <= 1024.
  * Synchronises in bf16 mode. */

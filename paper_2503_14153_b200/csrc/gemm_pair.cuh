@@ -63,6 +63,7 @@ struct PairGemmParams {
   int packed;                               // 1: the tensor maps view pre-tiled images, 0: row-major matrices
   int n_cols;                               // GP_PLAIN: columns stored; GP_RESIDUAL / GP_SWIGLU: weight rows of one matrix
   size_t ld;                                // GP_PLAIN: row pitch of out
+  int* clear;                               // GP_PLAIN: four ints set to zero, or nullptr
   float* out;                               // GP_PLAIN: sums; GP_RESIDUAL: residual stream [M][n_cols]
   bf16* act;                                // GP_SWIGLU: [M][n_cols]
   // GP_ROPE
@@ -285,6 +286,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
     const int wl = q * 32 + lane;                             // weight row within the CTA's 128
     const uint32_t acc_empty0 = dsmem_addr(smem_u32(acc_empty), 0);
     pdl_wait();
+    if (MODE == GP_PLAIN && p.clear && blockIdx.x == 0 && threadIdx.x < 68) p.clear[threadIdx.x - 64] = 0;
     for (int i = 0; i < my_tiles; ++i) {
       const int buf = halves == 2 ? 1 : i & 1;                // the accumulator that completes the tile
       const uint32_t acc_ph = halves == 2 ? i & 1 : (i >> 1) & 1;

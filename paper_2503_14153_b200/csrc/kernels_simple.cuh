@@ -818,12 +818,14 @@ __global__ void __launch_bounds__(256) accept_kernel(AcceptArgs a, unsigned long
 // (path, page, row), whatever the path's length. A thread moves 16 bytes (a chunk of eight 16-bit or four 32-bit elements,
 // which the cache layout keeps together) of one row in COMPACT_HEADS neighbouring heads; rows beyond the block's share
 // follow in further rounds, in order. On the 7B shape 6.2 -> 2.1 us a step (one row after the other, two bytes a thread).
+// The step's result block also goes to pinned host memory from here, which saves a copy behind the step's last kernel.
 constexpr int COMPACT_HEADS = 4;
 template <typename T>
 __global__ void __launch_bounds__(128)
 compact_kv(T* __restrict__ pool, KVGeom g, const int* __restrict__ page_table,
            const int* __restrict__ path, const int* __restrict__ count,
-           const int* __restrict__ n_old, int K, unsigned long long* tr) {
+           const int* __restrict__ n_old, int K, const int* __restrict__ result, int* __restrict__ host_result, int n_result,
+           unsigned long long* tr) {
   KTrace kt(tr);
   pdl_launch_dependents();
   constexpr int EPC = 16 / sizeof(T);
@@ -836,6 +838,8 @@ compact_kv(T* __restrict__ pool, KVGeom g, const int* __restrict__ page_table,
   const int* pt = page_table + b * g.pages_per_seq;
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  if (blockIdx.x + blockIdx.y == 0)
+    for (int i = threadIdx.x; i < n_result; i += 128) host_result[i] = result[i];
   const int len = count[b], n0 = n_old[b];
   const size_t head_stride = g.pool_pages() * 2 * g.block_elems();
   for (int j1 = 0; j1 < len; j1 += rows) {

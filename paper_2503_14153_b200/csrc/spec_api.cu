@@ -278,7 +278,8 @@ struct spec_ctx {
   int *d_n, *d_cnt, *d_n_old, *d_root, *d_count, *d_path, *d_out_tok, *d_gen_cnt, *d_gen_log, *d_cand, *d_cand_ov;
   int *d_tok, *d_pos, *d_slot, *d_am, *d_edge, *d_parent, *d_depth, *d_rank, *d_page_table, *d_prompt, *d_offsets;
   int *d_result;                       // [4 + B * (K + 3)]: d_status, d_n, d_count, d_out_tok
-  int* h_result = nullptr;             // the same in pinned host memory
+  int* h_result = nullptr;             // the same in pinned host memory, written by the step's last kernel
+  int* h_result_dev = nullptr;         // its device address
   int *d_status, *d_pidx, *d_pk_idx, *d_draws;
   int head_rows;                       // rows of the heads' logits computed at a time (without tensor cores)
   int chunk_cap;                       // prompt chunks the row buffers hold in one pass
@@ -1323,11 +1324,10 @@ int report_status(spec_ctx* c, const int* st) {
 }
 
 int check_status(spec_ctx* c) {
-  int st[4];
-  cudaError_t e = cudaMemcpyAsync(st, c->d_status, sizeof(st), cudaMemcpyDeviceToHost, c->stream);
+  cudaError_t e = cudaMemcpyAsync(c->h_result, c->d_status, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("status read: ") + cudaGetErrorString(e));
-  return report_status(c, st);
+  return report_status(c, c->h_result);
 }
 
 template <typename T>
@@ -1501,7 +1501,7 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
   // (5) KV compaction
   dim3 gc(f.n_layers * 2 * ((f.n_kv_heads + COMPACT_HEADS - 1) / COMPACT_HEADS), B);
   KLAUNCH("compact_kv", compact_kv<T>, gc, dim3(128), 0, static_cast<T*>(c->d_pool), c->geom, (const int*)c->d_page_table,
-          (const int*)c->d_path, (const int*)c->d_count, (const int*)c->d_n_old, K);
+          (const int*)c->d_path, (const int*)c->d_count, (const int*)c->d_n_old, K, (const int*)c->d_result, c->h_result_dev, 4 + f.max_batch * (K + 3));
   step_event(c, 5);
   return SPEC_OK;
 }
@@ -1600,9 +1600,8 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     }
   }
   if (out_tokens || out_counts) {
-    // one copy of the whole result block and one wait (four copies of a few bytes each cost a short step 15 us more)
+    // (the step's last kernel has put the result block into host memory)
     const int cap = f.max_batch;
-    CUDA_OK(cudaMemcpyAsync(c->h_result, c->d_result, (4 + (size_t)cap * (K + 3)) * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
     const int *nn = c->h_result + 4, *counts = nn + cap, *toks = counts + cap;
     if (out_tokens) memcpy(out_tokens, toks, (size_t)B * (K + 1) * sizeof(int));
@@ -1741,7 +1740,9 @@ int spec_create(const spec_config* cfg, const spec_weights* w, const spec_tree* 
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) { g_create_error = std::string("set-up copies: ") + cudaGetErrorString(e); delete c; return SPEC_E_CUDA; }
   // one pinned block: a step's result, then the copy of the committed lengths
-  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_result), (4 + (size_t)cfg->max_batch * (c->K + 4)) * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_result), (4 + (size_t)cfg->max_batch * (c->K + 4)) * sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->h_result_dev), c->h_result, 0) != cudaSuccess) {
+    if (c->h_result) cudaFreeHost(c->h_result);
     g_create_error = "pinned host memory for a step's result"; delete c; return SPEC_E_CUDA;
   }
   c->h_n_pinned = c->h_result + 4 + (size_t)cfg->max_batch * (c->K + 3);
@@ -2000,12 +2001,28 @@ int spec_debug_read_kv(spec_ctx* c, int32_t seq, int32_t layer, int32_t slot0, i
 }
 
 namespace {
-// Waits for the call's kernels and reads their status word.
-int op_linear_status(const int* status, cudaStream_t st) {
-  int stw[4];
-  if (cudaMemcpyAsync(stw, status, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
-    return SPEC_E_CUDA;
-  return stw[0] == 0 ? SPEC_OK : SPEC_E_TIMEOUT;
+// The status word of a call lies in pinned host memory, where the kernels report a wait that ran out: nothing has to be cleared
+// before them and nothing copied after them (a memset and a 16-byte copy to pageable memory took 12 of the call's 53 us at 64 rows of 4096 x
+// 11008). A block a thread, given back when the thread ends; a call returns only after its kernels, so no other uses it.
+struct HostStatus {
+  int* word = nullptr;
+  ~HostStatus() { if (word) cudaFreeHost(word); }
+  int* clean() {
+    if (!word && cudaHostAlloc(reinterpret_cast<void**>(&word), 4 * sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      word = nullptr;
+    }
+    if (word) memset(word, 0, 4 * sizeof(int));
+    return word;
+  }
+};
+thread_local HostStatus t_status;
+// Waits for the call's kernels and looks at their status word; `words`, which the kernels have cleared, gets it where it is not zero.
+int op_linear_status(const int* status, int* words, cudaStream_t st) {
+  if (cudaStreamSynchronize(st) != cudaSuccess) return SPEC_E_CUDA;
+  if (*static_cast<const volatile int*>(status) == 0) return SPEC_OK;
+  cudaMemcpy(words, status, 4 * sizeof(int), cudaMemcpyHostToDevice);
+  return SPEC_E_TIMEOUT;
 }
 // Shared body of the two stand-alone linear entry points (bf16): scratch holds the partial
 // sums followed by the four-int status word.
@@ -2015,6 +2032,9 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
   int rws[1] = {N};
   if (!plan_gemm(M, K, 1, rws, ctas, &g)) return SPEC_E_BADARG;
   StreamTmaps tm{};
+  int* const words = reinterpret_cast<int*>(scratch + scratch_floats);
+  int *const host = t_status.clean(), *status = nullptr;
+  if (!host || cudaHostGetDevicePointer(reinterpret_cast<void**>(&status), host, 0) != cudaSuccess) return SPEC_E_CUDA;
   if (M > 128 && (long long)g.p.n_tiles * g.p.seg.m_tiles >= 2LL * g.grid) {
     // many rows: whole tiles on pairs of SMs, finished sums straight into y (at M = 1008, N = 11008, K = 4096 the call takes
     // 112 us; weight streaming, which fetches the weights once per 128 rows, took 127 us, adding up its partial sums 34, the call 204)
@@ -2026,10 +2046,9 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     p.n_tiles = g.p.n_tiles; p.w_pairs = (g.p.n_tiles + 1) / 2; p.m_tiles = (M + GP_NT - 1) / GP_NT;
     for (int i = 1; i <= GS_MAX_MATS; ++i) p.mat_tile0[i] = p.n_tiles;
     p.out = y; p.ld = (size_t)N; p.n_cols = N;
-    p.status = reinterpret_cast<int*>(scratch + scratch_floats);
-    if (cudaMemsetAsync(p.status, 0, 16, st) != cudaSuccess ||
-        launch_gp<GP_PLAIN>(st, false, tm, p, nullptr, nullptr, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
-    return op_linear_status(p.status, st);
+    p.status = status; p.clear = words;
+    if (launch_gp<GP_PLAIN>(st, false, tm, p, nullptr, nullptr, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
+    return op_linear_status(host, words, st);
   }
   if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, g.MT)) return SPEC_E_CUDA;
   const int cs = M <= 128 ? plain_cluster(g.p.n_tiles, K / 64, ctas) : 0;
@@ -2038,21 +2057,20 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     // runs (few tiles and a long inner dimension): the error of a running sum grows with its length.
     ClusterGemmParams p{};
     p.M = M; p.K = K; p.KC = K / 64; p.N = N; p.y = y; p.ldy = (size_t)N;
-    p.status = reinterpret_cast<int*>(scratch + scratch_floats);
-    if (cudaMemsetAsync(p.status, 0, 16, st) != cudaSuccess || launch_gc_plain(st, false, g.p.n_tiles, cs, tm, p) != cudaSuccess) return SPEC_E_CUDA;
-    return op_linear_status(p.status, st);
+    p.status = status; p.clear = words;
+    if (launch_gc_plain(st, false, g.p.n_tiles, cs, tm, p) != cudaSuccess) return SPEC_E_CUDA;
+    return op_linear_status(host, words, st);
   }
   g.p.part = scratch;
   g.p.slot_stride = (size_t)M * g.p.n_tiles * 128;
   g.p.l2_prefetch = 0;
-  g.p.status = reinterpret_cast<int*>(scratch + scratch_floats);
-  // the status word must start at zero; the partial sums are fully overwritten before they are read
-  if (cudaMemsetAsync(g.p.status, 0, 16, st) != cudaSuccess) return SPEC_E_CUDA;
+  g.p.status = status;
+  // (the partial sums are fully overwritten before they are read)
   if (launch_gs(st, false, g, tm) != cudaSuccess) return SPEC_E_CUDA;
   size_t total = (size_t)M * ((N + 3) / 4);
-  if (launch_k(true, part_sum_rows, dim3((unsigned)std::min<size_t>((total + 255) / 256, 4096)), dim3(256), 0, st, plan_view(g), y, M, N) != cudaSuccess)
+  if (launch_k(true, part_sum_rows, dim3((unsigned)std::min<size_t>((total + 255) / 256, 4096)), dim3(256), 0, st, plan_view(g), y, M, N, words) != cudaSuccess)
     return SPEC_E_CUDA;
-  return op_linear_status(g.p.status, st);
+  return op_linear_status(host, words, st);
 }
 int op_linear_f32(const void* x, const void* w, float* y, int M, int N, int K, cudaStream_t st) {
   RowLinear<float> rl{};
