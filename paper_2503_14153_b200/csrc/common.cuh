@@ -44,13 +44,14 @@ __device__ __forceinline__ float warp_max(float v) {
 __device__ __forceinline__ bool better(float v, int i, float ov, int oi) {
   return v > ov || (v == ov && i < oi);
 }
+// The warp's best pair in every lane (two warp-wide integer reductions; floats in an order-preserving integer form). A pair
+// without a value is (-inf, 0x7fffffff); NaN does not occur (`better` never lets it in).
 __device__ __forceinline__ void warp_argmax(float& v, int& i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    float ov = __shfl_xor_sync(0xffffffffu, v, o);
-    int oi = __shfl_xor_sync(0xffffffffu, i, o);
-    if (better(ov, oi, v, i)) { v = ov; i = oi; }
-  }
+  const uint32_t u = __float_as_uint(v + 0.f);               // (-0 and 0 are equal)
+  const uint32_t key = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  const uint32_t best = __reduce_max_sync(0xffffffffu, key);
+  i = (int)__reduce_min_sync(0xffffffffu, key == best ? (uint32_t)i : 0x7fffffffu);
+  v = __uint_as_float((best & 0x80000000u) ? (best & 0x7fffffffu) : ~best);
 }
 
 // ------------------------------------------------------------------ KV page layout

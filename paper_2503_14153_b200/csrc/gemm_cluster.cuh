@@ -554,27 +554,35 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
         // a warp has a row: 128 columns of it in every part, added in rank order
         const int rows = min(rb, Mr - rank * rb), n0 = t * 128 + lane * 4;
         const bool vec = (p.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 15) == 0 && n0 + 4 <= p.N;
-        for (int i = warp - 2; i < rows; i += GC_EPI / 32) {
-          const float* src = in + i * 128 + lane * 4;
-          float4 a = *reinterpret_cast<const float4*>(src);
-          for (int r = 1; r < CS; ++r) add4(a, *reinterpret_cast<const float4*>(src + (size_t)r * rb * 128));
-          const int m = m0 + rank * rb + i;
-          const float v[4] = {a.x, a.y, a.z, a.w};
-          if (p.y) {
-            float* dst = p.y + (size_t)m * p.ldy + n0;
-            if (vec) *reinterpret_cast<float4*>(dst) = a;
-            else
-              for (int j = 0; j < 4; ++j) if (n0 + j < p.N) dst[j] = v[j];
-          }
-          if (p.best_val) {
-            float bv = -INFINITY;
-            int bi = 0x7fffffff;
+        const int tiles_n = (p.N + 127) >> 7;
+        constexpr int U = MT > 64 ? 2 : 4, STEP = GC_EPI / 32; // rows in flight a warp
+        for (int i0 = warp - 2; i0 < rows; i0 += U * STEP) {
+          float4 a[U];
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-              if (n0 + j < p.N && better(v[j], n0 + j, bv, bi)) { bv = v[j]; bi = n0 + j; }
-            warp_argmax(bv, bi);
-            const int tiles_n = (p.N + 127) >> 7;
-            if (lane == 0) { p.best_val[(size_t)m * tiles_n + t] = bv; p.best_idx[(size_t)m * tiles_n + t] = bi; }
+          for (int k = 0; k < U; ++k) a[k] = *reinterpret_cast<const float4*>(in + min(i0 + k * STEP, rows - 1) * 128 + lane * 4);
+          for (int r = 1; r < CS; ++r)
+#pragma unroll
+            for (int k = 0; k < U; ++k) add4(a[k], *reinterpret_cast<const float4*>(in + ((size_t)r * rb + min(i0 + k * STEP, rows - 1)) * 128 + lane * 4));
+#pragma unroll
+          for (int k = 0; k < U; ++k) {
+            const int i = i0 + k * STEP, m = m0 + rank * rb + i;
+            if (i >= rows) continue;
+            const float v[4] = {a[k].x, a[k].y, a[k].z, a[k].w};
+            if (p.y) {
+              float* dst = p.y + (size_t)m * p.ldy + n0;
+              if (vec) *reinterpret_cast<float4*>(dst) = a[k];
+              else
+                for (int j = 0; j < 4; ++j) if (n0 + j < p.N) dst[j] = v[j];
+            }
+            if (p.best_val) {
+              float bv = -INFINITY;
+              int bi = 0x7fffffff;
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (n0 + j < p.N && better(v[j], n0 + j, bv, bi)) { bv = v[j]; bi = n0 + j; }
+              warp_argmax(bv, bi);
+              if (lane == 0) { p.best_val[(size_t)m * tiles_n + t] = bv; p.best_idx[(size_t)m * tiles_n + t] = bi; }
+            }
           }
         }
       } else if (MODE == GC_SWIGLU8) {

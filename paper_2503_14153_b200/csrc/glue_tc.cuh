@@ -476,6 +476,28 @@ argmax_partials_tc(const PartView pv, int V, float* __restrict__ logits, float* 
   }
 }
 
+// The best (value desc, index asc) of every row among its tiles' [M][tiles], a warp a row.
+__global__ void __launch_bounds__(256)
+argmax_tiles(const float* __restrict__ val, const int* __restrict__ idx, int M, int tiles, float* __restrict__ pval2, int* __restrict__ pidx2,
+             unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (m >= M) return;
+  float bv = -INFINITY;
+  int bi = 0x7fffffff;
+#pragma unroll 8
+  for (int t = lane; t < tiles; t += 32) {
+    const float v = __ldcg(val + (size_t)m * tiles + t);
+    const int i = __ldcg(idx + (size_t)m * tiles + t);
+    if (better(v, i, bv, bi)) { bv = v; bi = i; }
+  }
+  warp_argmax(bv, bi);
+  if (lane == 0) { pval2[m] = bv; pidx2[m] = bi; }
+}
+
 // Per-head top-k straight from the partial sums of the heads' lm_head GEMM (no materialised logits): each
 // row's kmax best (value desc, index asc) of this block's slice of the vocabulary go to the partial lists
 // pk_val / pk_idx [row][block][kmax]; grid (slices, rows), the view's first row being row `row0` of the lists. The CTA of a row that arrives last (arrive[row],
