@@ -30,15 +30,19 @@
 //                 rows of the up matrix
 //  * GP_ROPE      stacked q, k, v: rotates q and k, writes bf16 q rows and the cache rows
 // In the last two modes an output needs two weight rows of the tile, which sit in different tensor-memory lanes: the
-// threads swap halves of their activation rows through 16 KB of shared memory, 32 rows at a time.
+// threads swap halves of their activation rows through 16 KB of shared memory, 16 rows at a time.
 //
 // Measured on the 7B shape at M = 1024 (inside a step, launch to end, per layer), against a kernel with 128 x 256 tiles per
 // CTA that wrote float32 sums for separate glue kernels: gate+up 175 -> 141 us (1.31 PFLOP/s) and the 33 us SwiGLU kernel
 // gone, q/k/v 107 -> 91 us and the 23 us RoPE / store kernel gone, output 41 -> 39, down 92 -> 84 us; a step of 16
 // sequences through 8 layers 5.58 -> 4.56 ms.
 //
+// A tile's epilogue runs under the next tile's MMAs, but the last one of a CTA does not: with eight epilogue warps the time from
+// the last MMA to the end of the kernel was 10.0 us for q/k/v, 11.4 for the output, 10.3 for the gate+up and 13.8 for the down projection
+// (M = 1024), with sixteen, in half as long strides, it is 7.0, 7.0, 7.1 and 7.1; a step of 16 sequences through 8 layers 4.14 -> 4.04 ms.
+//
 // Warp roles (both CTAs): warp 0 feeds a ring of 32 KB stages (TMA, completing on the leader CTA's barrier), warp
-// 1 of the leader issues the MMAs, warps 2..9 drain: two warps per SM quarter, one for each half of the tile's
+// 1 of the leader issues the MMAs, warps 2..17 drain: four warps per SM quarter, one for each quarter of the tile's
 // activation rows. Every wait is bounded; a CTA whose wait ran out still takes part in the closing cluster barrier.
 #pragma once
 #include <cuda.h>
@@ -50,7 +54,8 @@
 namespace spec {
 
 constexpr int GP_PLAIN = 0, GP_RESIDUAL = 1, GP_SWIGLU = 2, GP_ROPE = 3;
-constexpr int GP_THREADS = 320;
+constexpr int GP_EPI = 512, GP_THREADS = 64 + GP_EPI;   // producer, MMA issuer, sixteen epilogue warps (four per SM quarter)
+constexpr int GP_QUARTERS = 4;                          // parts of a tile's activation rows that the epilogue warps share out
 
 struct PairGemmParams {
   int M, KC;                                // activation rows, K / 64
@@ -85,8 +90,8 @@ template <int NT> struct PairCfg {
   static constexpr int B_BYTES = (NT / 2) * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = 6;
-  static constexpr int EX_COLS = 16;                              // activation rows swapped in one direction at a time
-  static constexpr int EX_BYTES = 2 * 2 * 64 * EX_COLS * 4;       // [half][direction][column][64 pairs] float32
+  static constexpr int EX_COLS = 8;                               // activation rows swapped in one direction at a time
+  static constexpr int EX_BYTES = GP_QUARTERS * 2 * 64 * EX_COLS * 4;       // [part][direction][column][64 pairs] float32
   static constexpr int META_BYTES = NT * 16;                      // GP_ROPE: (cache offset, position, swizzle row) of a row
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EX_BYTES + META_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
   static constexpr int TMEM_COLS = 2 * NT;
@@ -123,12 +128,13 @@ __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const void* tma
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
-// Barrier of one half's four epilogue warps; epilogue_and: of all eight, telling whether `v` holds in all of their threads.
+// Barrier of one part's four epilogue warps; epilogue_bar, epilogue_and: of all sixteen, telling whether `v` holds in all of their threads.
 __device__ __forceinline__ void group_bar(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void epilogue_bar() { asm volatile("bar.sync 6, %0;" ::"n"(GP_EPI) : "memory"); }
 __device__ __forceinline__ bool epilogue_and(bool v) {
   uint32_t r;
-  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.and.pred q, 3, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
-               : "=r"(r) : "r"((uint32_t)v) : "memory");
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.and.pred q, 7, %2, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"((uint32_t)v), "n"(GP_EPI) : "memory");
   return r != 0;
 }
 
@@ -152,7 +158,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   uint64_t* full = bars;                    // leader's: both CTAs' operands of a stage have landed
   uint64_t* empty = bars + STAGES;          // each CTA's: the stage has been read
   uint64_t* acc_full = bars + 2 * STAGES;   // each CTA's
-  uint64_t* acc_empty = bars + 2 * STAGES + 2;   // leader's: drained by the eight warps of both CTAs
+  uint64_t* acc_empty = bars + 2 * STAGES + 2;   // leader's: drained by the sixteen warps of both CTAs
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
   volatile uint32_t* last_slot = reinterpret_cast<volatile uint32_t*>(bars + 2 * STAGES + 5);   // this CTA completes a split tile
 
@@ -174,7 +180,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(&acc_full[0], 1); mbar_init(&acc_full[1], 1);
-    mbar_init(&acc_empty[0], 16); mbar_init(&acc_empty[1], 16);
+    mbar_init(&acc_empty[0], 2 * GP_EPI / 32); mbar_init(&acc_empty[1], 2 * GP_EPI / 32);
     mbar_fence_init();
     for (int i = 0; i < p.n_mats; ++i) tma_prefetch_desc(&tm.a[i]);
     tma_prefetch_desc(&tm.b);
@@ -279,10 +285,10 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       trace_mark_max(p.trace, 3);
     }
   } else {
-    // ---- epilogue: warp w may touch tensor-memory lanes [32 (w % 4), +32); warps 2..5 take the first half of the
-    // tile's activation rows, warps 6..9 the second ----
-    constexpr int HC = NT / 2;
-    const int q = warp & 3, hf = warp >= 6 ? 1 : 0;
+    // ---- epilogue: warp w may touch tensor-memory lanes [32 (w % 4), +32); warps 2..5 take the first quarter of the
+    // tile's activation rows, warps 6..9 the second, ... ----
+    constexpr int HC = NT / GP_QUARTERS;
+    const int q = warp & 3, hf = (warp - 2) >> 2;
     const int wl = q * 32 + lane;                             // weight row within the CTA's 128
     const uint32_t acc_empty0 = dsmem_addr(smem_u32(acc_empty), 0);
     pdl_wait();
@@ -298,17 +304,19 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       constexpr bool split = SPLIT;
       // (what the epilogue needs besides the sums is fetched while the tile's MMAs run)
       // GP_RESIDUAL: old values of the first rows
-      float xo[2][32];
+      float xo[16];
       const int rcol = nt * 128 + wl;
       const bool ron = MODE == GP_RESIDUAL && nt < p.n_tiles && rcol < p.n_cols;
-      auto fetch_x = [&](int g, float (&v)[32]) {
+      auto fetch_x = [&](int g, float (&v)[16]) {
+        const float* src = p.out + (size_t)(m0 + g * 16) * p.n_cols + rcol;
+        const int live = ron ? p.M - m0 - g * 16 : 0;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int m = m0 + g * 32 + j;
-          v[j] = (ron && m < p.M) ? p.out[(size_t)m * p.n_cols + rcol] : 0.f;
+        for (int j = 0; j < 16; ++j) {                         // (a running pointer: registers)
+          v[j] = j < live ? *src : 0.f;
+          src += p.n_cols;
         }
       };
-      if (MODE == GP_RESIDUAL && !split) fetch_x(0, xo[0]);
+      if (MODE == GP_RESIDUAL && !split) fetch_x(0, xo);
       // GP_ROPE: the rows' positions and cache slots
       PairRowMeta* mrow = meta + hf * HC;
       if (MODE == GP_ROPE) {
@@ -350,7 +358,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           if (lane == 0) mbar_arrive_cluster(acc_empty0);
         }
       }
-      // (all eight warps give up when one of them does: barriers follow)
+      // (all warps give up when one of them does: barriers follow)
       if (!epilogue_and(mbar_wait(&acc_full[buf], acc_ph, p.status, 42))) break;
       tc_fence_after();
       // partial sums of this warp's rows, part k at parts_at + k * PART
@@ -370,38 +378,38 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         __threadfence();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);
-        asm volatile("bar.sync 3, 256;" ::: "memory");        // every warp's part precedes the arrival
+        epilogue_bar();        // every warp's part precedes the arrival
         if (threadIdx.x == 64) {
           unsigned int* ctr = p.arrive + 2 * tau + rank;
           const bool last = atomicAdd(ctr, 1u) == (unsigned)(parts - 1);
           if (last) *ctr = 0u;
           *last_slot = last;
         }
-        asm volatile("bar.sync 3, 256;" ::: "memory");
+        epilogue_bar();
         const bool last = *last_slot != 0;
-        asm volatile("bar.sync 3, 256;" ::: "memory");        // everybody has read it
+        epilogue_bar();        // everybody has read it
         if (!last) continue;
         __threadfence();
-        if (MODE == GP_RESIDUAL) fetch_x(0, xo[0]);
+        if (MODE == GP_RESIDUAL) fetch_x(0, xo);
       }
-      // sums of this thread's weight row for activation rows [g * 32, +32) of the warp's half
-      auto acc = [&](int g, uint32_t (&r)[32]) {
+      // sums of this thread's weight row for activation rows [g * 16, +16) of the warp's quarter
+      auto acc = [&](int g, uint32_t (&r)[16]) {
         if (!split) {
-          tmem_ld32(taddr + g * 32, r);
+          tmem_ld16(taddr + g * 16, r);
           tmem_ld_wait();
           return;
         }
-        const float* src = parts_at + g * 32 * 128;
-        float v[32];
+        const float* src = parts_at + g * 16 * 128;
+        float v[16];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = __ldcg(src + j * 128);
+        for (int j = 0; j < 16; ++j) v[j] = __ldcg(src + j * 128);
         for (int k = 1; k < parts; ++k) {
           src += PART;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] += __ldcg(src + j * 128);
+          for (int j = 0; j < 16; ++j) v[j] += __ldcg(src + j * 128);
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(v[j]);
+        for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(v[j]);
       };
       if constexpr (MODE == GP_PLAIN) {
         const int col = nt * 128 + wl;
@@ -427,18 +435,22 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         }
         continue;
       } else if constexpr (MODE == GP_RESIDUAL) {
-        // old values of the next 32 rows are fetched while 32 rows are finished
-        float* dst = p.out + rcol;
-#pragma unroll
-        for (int g = 0; g < HC / 32; ++g) {
-          uint32_t r[32];
-          if (g + 1 < HC / 32) fetch_x(g + 1, xo[(g + 1) & 1]);
+        // old values of the next 16 rows are fetched while 16 rows are finished
+#pragma unroll 1
+        for (int g = 0; g < HC / 16; ++g) {
+          uint32_t r[16];
+          float next[16];
+          if (g + 1 < HC / 16) fetch_x(g + 1, next);
           acc(g, r);
+          float* dst = p.out + (size_t)(m0 + g * 16) * p.n_cols + rcol;
+          const int live = ron ? p.M - m0 - g * 16 : 0;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int m = m0 + g * 32 + j;
-            if (ron && m < p.M) dst[(size_t)m * p.n_cols] = xo[g & 1][j] + __uint_as_float(r[j]);
+          for (int j = 0; j < 16; ++j) {
+            if (j < live) *dst = xo[j] + __uint_as_float(r[j]);
+            dst += p.n_cols;
           }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) xo[j] = next[j];
         }
       } else {
         // outputs that need two weight rows of the tile: row pairs (lower, upper) = (gate, up) or a rotation pair
@@ -454,21 +466,21 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           const int col = nt * 64 + pr;
           const bool on = col < p.n_cols;
 #pragma unroll 1
-          for (int g = 0; g < HC / 32; ++g) {
-            uint32_t r[32];
+          for (int g = 0; g < HC / 16; ++g) {
+            uint32_t r[16];
             acc(g, r);
             if (g) group_bar(1 + hf);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              if (lower) ex_lo[j * 64 + pr] = __uint_as_float(r[16 + j]);
+            for (int j = 0; j < 8; ++j) {
+              if (lower) ex_lo[j * 64 + pr] = __uint_as_float(r[8 + j]);
               else ex_up[j * 64 + pr] = __uint_as_float(r[j]);
             }
             group_bar(1 + hf);
-            const int mb = m0 + g * 32 + (lower ? 0 : 16);
+            const int mb = m0 + g * 16 + (lower ? 0 : 8);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
+            for (int j = 0; j < 8; ++j) {
               const float gt = lower ? __uint_as_float(r[j]) : ex_lo[j * 64 + pr];
-              const float up = lower ? ex_up[j * 64 + pr] : __uint_as_float(r[16 + j]);
+              const float up = lower ? ex_up[j * 64 + pr] : __uint_as_float(r[8 + j]);
               if (on && mb + j < p.M) p.act[(size_t)(mb + j) * p.n_cols + col] = __float2bfloat16_rn(silu_f(gt) * up);
             }
           }
@@ -484,41 +496,41 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           if (kind == 2) {
             bf16* dst = p.pool + lh + p.g.block_elems();
 #pragma unroll 1
-            for (int g = 0; g < HC / 32; ++g) {
-              uint32_t r[32];
+            for (int g = 0; g < HC / 16; ++g) {
+              uint32_t r[16];
               acc(g, r);
 #pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                const PairRowMeta v = mrow[g * 32 + j];
+              for (int j = 0; j < 16; ++j) {
+                const PairRowMeta v = mrow[g * 16 + j];
                 if (on && v.kv >= 0) dst[v.kv + kv_elem<bf16>(v.prow, dim, D, p.g.page_size)] = __float2bfloat16_rn(__uint_as_float(r[j]));
               }
             }
           } else {
             const int di = dim & (half - 1);                     // the pair's place in its head
 #pragma unroll 1
-            for (int g = 0; g < HC / 32; ++g) {
-              uint32_t r[32];
-              const int jb = g * 32 + (lower ? 0 : 16);
-              float2 t[16];
+            for (int g = 0; g < HC / 16; ++g) {
+              uint32_t r[16];
+              const int jb = g * 16 + (lower ? 0 : 8);
+              float2 t[8];
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < 8; ++j) {
                 const PairRowMeta v = mrow[jb + j];
                 t[j] = p.cs[(size_t)v.pos * half + di];          // (position 0 for rows not in use)
               }
               acc(g, r);
               if (g) group_bar(1 + hf);
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                if (lower) ex_lo[j * 64 + pr] = __uint_as_float(r[16 + j]);
+              for (int j = 0; j < 8; ++j) {
+                if (lower) ex_lo[j * 64 + pr] = __uint_as_float(r[8 + j]);
                 else ex_up[j * 64 + pr] = __uint_as_float(r[j]);
               }
               group_bar(1 + hf);
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < 8; ++j) {
                 const PairRowMeta v = mrow[jb + j];
                 if (!on || v.kv < 0) continue;
                 const float a = lower ? __uint_as_float(r[j]) : ex_lo[j * 64 + pr];
-                const float c = lower ? ex_up[j * 64 + pr] : __uint_as_float(r[16 + j]);
+                const float c = lower ? ex_up[j * 64 + pr] : __uint_as_float(r[8 + j]);
                                 // (the rounding of the other kernels that rotate: one product rounded, the other fused into the sum)
                 const bf16 lo = __float2bfloat16_rn(__fmaf_rn(a, t[j].x, -__fmul_rn(c, t[j].y)));
                 const bf16 hi = __float2bfloat16_rn(__fmaf_rn(c, t[j].x, __fmul_rn(a, t[j].y)));
