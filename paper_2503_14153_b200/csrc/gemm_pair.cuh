@@ -69,6 +69,8 @@ struct PairGemmParams {
   int n_cols;                               // GP_PLAIN: columns stored; GP_RESIDUAL / GP_SWIGLU: weight rows of one matrix
   size_t ld;                                // GP_PLAIN: row pitch of out
   int* clear;                               // GP_PLAIN: four ints set to zero, or nullptr
+  float* best_val;                          // GP_PLAIN: [4 * n_tiles][M] each row's largest of 32 columns and its column (value descending, column
+  int* best_idx;                            // ascending), or nullptr; out may then be nullptr
   float* out;                               // GP_PLAIN: sums; GP_RESIDUAL: residual stream [M][n_cols]
   bf16* act;                                // GP_SWIGLU: [M][n_cols]
   // GP_ROPE
@@ -427,11 +429,49 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);
-        const int live = on ? p.M - m0 : 0;
+        const int live = on && p.out ? p.M - m0 : 0;
 #pragma unroll
         for (int j = 0; j < HC; ++j) {                         // (a running pointer: 128 separate addresses cost 2-3 us a tile)
           if (j < live) *dst = first[j];
           dst += p.ld;
+        }
+        if (p.best_val) {
+          // 32 rows at a time, halved over the lanes (46 shuffles; 64 warp-wide reductions took longer than the tile's MMAs): lane l
+          // ends with row l and the lane its largest came from. Columns that are not there count as NaN, which never wins.
+#pragma unroll
+          for (int j = 0; j < HC; j += 32) {
+            int from[16];
+            auto wins = [](float v, int i, float ov, int oi) { return better(v, i, ov, oi) || (ov != ov && v == v); };
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const bool hi = (lane & 16) != 0;
+              float lo_v = on ? first[j + i] : __int_as_float(0x7fc00000), hi_v = on ? first[j + i + 16] : __int_as_float(0x7fc00000);
+              const float keep = hi ? hi_v : lo_v, got = __shfl_xor_sync(0xffffffffu, hi ? lo_v : hi_v, 16);
+              const bool take = wins(got, lane ^ 16, keep, lane);
+              first[j + i] = take ? got : keep;
+              from[i] = take ? lane ^ 16 : lane;
+            }
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) {
+              const bool hi = (lane & o) != 0;
+#pragma unroll
+              for (int i = 0; i < o; ++i) {
+                const float keep = hi ? first[j + i + o] : first[j + i];
+                const int keep_f = hi ? from[i + o] : from[i];
+                const float got = __shfl_xor_sync(0xffffffffu, hi ? first[j + i] : first[j + i + o], o);
+                const int got_f = __shfl_xor_sync(0xffffffffu, hi ? from[i] : from[i + o], o);
+                const bool take = wins(got, got_f, keep, keep_f);
+                first[j + i] = take ? got : keep;
+                from[i] = take ? got_f : keep_f;
+              }
+            }
+            const int m = m0 + j + lane;
+            const float best = first[j];
+            if (nt < p.n_tiles && m < p.M) {
+              p.best_val[(size_t)(nt * 4 + q) * p.M + m] = best == best ? best : -INFINITY;
+              p.best_idx[(size_t)(nt * 4 + q) * p.M + m] = best == best ? nt * 128 + q * 32 + from[0] : 0x7fffffff;
+            }
+          }
         }
         continue;
       } else if constexpr (MODE == GP_RESIDUAL) {

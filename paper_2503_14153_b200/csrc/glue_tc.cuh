@@ -498,6 +498,35 @@ argmax_tiles(const float* __restrict__ val, const int* __restrict__ idx, int M, 
   if (lane == 0) { pval2[m] = bv; pidx2[m] = bi; }
 }
 
+// The same among slots [slots][M] (passes of many rows): a CTA takes 32 rows, its warps every 32nd slot.
+__global__ void __launch_bounds__(1024)
+argmax_slots(const float* __restrict__ val, const int* __restrict__ idx, int M, int slots, float* __restrict__ pval2, int* __restrict__ pidx2,
+             unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  __shared__ float sv[32][33];
+  __shared__ int si[32][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m = blockIdx.x * 32 + lane;
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  float bv = -INFINITY;
+  int bi = 0x7fffffff;
+  if (m < M) {
+#pragma unroll 8
+    for (int t = warp; t < slots; t += 32) {
+      const float v = __ldcg(val + (size_t)t * M + m);
+      const int i = __ldcg(idx + (size_t)t * M + m);
+      if (better(v, i, bv, bi)) { bv = v; bi = i; }
+    }
+  }
+  sv[warp][lane] = bv; si[warp][lane] = bi;
+  __syncthreads();
+  bv = sv[lane][warp]; bi = si[lane][warp];                  // (row `warp` of the 32)
+  warp_argmax(bv, bi);
+  const int row = blockIdx.x * 32 + warp;
+  if (lane == 0 && row < M) { pval2[row] = bv; pidx2[row] = bi; }
+}
+
 // Per-head top-k straight from the partial sums of the heads' lm_head GEMM (no materialised logits): each
 // row's kmax best (value desc, index asc) of this block's slice of the vocabulary go to the partial lists
 // pk_val / pk_idx [row][block][kmax]; grid (slices, rows), the view's first row being row `row0` of the lists. The CTA of a row that arrives last (arrive[row],

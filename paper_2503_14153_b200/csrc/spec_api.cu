@@ -1245,9 +1245,9 @@ PartView plain_view(const float* p, int rows, int ld) {
 int heads_top_k(spec_ctx* c, const PartView& pl, int row0, int rows, const int* ov) {
   const int kmax = c->kmax, V = c->cfg.vocab;
   // the row's last-arriving CTA merges the slices' lists: no merge kernel
-  // about 296 CTAs whatever the number of rows, at least four a row: more slices would only lengthen the lists to merge
-  // (and at least as many as let a slice fit 40 KB)
-  const int want = std::min(c->topk_blocks, std::max(std::max(4, (V + 10239) / 10240), SM_SLOTS / rows));
+  // about 296 CTAs whatever the number of rows, and up to 1024 while that is at most 16 a row (64 rows with four slices each left the SMs at
+  // two CTAs: 27 us, now 21): more slices would only lengthen the lists to merge (and at least as many as let a slice fit 40 KB)
+  const int want = std::min(c->topk_blocks, std::max(std::max(std::max(4, std::min(16, 1024 / rows)), (V + 10239) / 10240), SM_SLOTS / rows));
   const int slice = (int)round_up((V + want - 1) / want, 4), blocks = (V + slice - 1) / slice;
   const size_t sm_topk = std::max((size_t)slice * sizeof(float), (size_t)blocks * kmax * 8);
   if (sm_topk > 44 * 1024) return c->fail(SPEC_E_BADARG, "top-k lists do not fit the merge's shared memory");
@@ -1331,6 +1331,18 @@ int lm_head_argmax(spec_ctx* c, const T* src, int M) {
     int r = run_lm_head(c, src, M, cs, c->keep_logits ? c->d_logits : nullptr, f.vocab, val, idx);
     if (r) return r;
     KLAUNCH("argmax_tiles", argmax_tiles, dim3((M + 7) / 8), dim3(256), 0, (const float*)val, (const int*)idx, M, tiles, c->d_pval2, c->d_pidx2);
+    return SPEC_OK;
+  }
+  if (c->tc && pair_gemm_ok(c, M, f.d_model)) {
+    // (the same with the projection of many rows, whose logits nobody else needs: written and read back they were 131 MB and a
+    // kernel of 53 us behind 195 for 16 sequences of 64 rows; now 14 behind 202)
+    const int slots = 4 * ((f.vocab + 127) / 128);
+    PairGemmParams w{};
+    w.out = c->keep_logits ? c->d_logits : nullptr; w.ld = (size_t)f.vocab; w.n_cols = f.vocab;
+    w.best_val = c->d_part; w.best_idx = reinterpret_cast<int*>(c->d_part + (size_t)slots * M);
+    int r = run_gemm_pair(c, GP_PLAIN, src, M, f.d_model, 1, mats, rws, &w, SPEC_PROFILE_OFF);
+    if (r) return r;
+    KLAUNCH("argmax_slots", argmax_slots, dim3((M + 31) / 32), dim3(1024), 0, (const float*)w.best_val, (const int*)w.best_idx, M, slots, c->d_pval2, c->d_pidx2);
     return SPEC_OK;
   }
   if (c->tc) {

@@ -70,3 +70,24 @@ def test_sampled_decoding_vocabulary_sizes(torch, vocab):
     rep = run_lockstep(cfg, draw_weights(cfg), build_tree(cfg.topk, cfg.tree_nodes), draw_prompt(cfg), 24, 1e-4, 1e-2,
                        accept_mode=1, typ=(0.09, 0.3, float(np.float32(0.8))), sampling=True, seed=11)
     assert rep.steps > 0
+
+
+@pytest.mark.parametrize("vocab,rows,batch", [(131, 33, 1), (2999, 64, 1), (4100, 128, 1), (131, 43, 3), (2999, 64, 4), (4100, 50, 6)])
+def test_row_maxima_out_of_the_projection(torch, vocab, rows, batch):
+    """lm_head compares its own tiles' tokens (up to 128 rows and more, vocabularies that fill no tile): every row's argmax is that of
+    the kept logits, and the same without them."""
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = get_config("c0", name="maxima", dtype="bf16", vocab=vocab, d_ffn=704, n_heads=2, n_kv_heads=2, head_dim=128, n_medusa=3, topk=(16, 8, 4),
+                     tree_nodes=rows, seed=5)
+    dw, tree = upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, rows)
+    got = []
+    for flags in (B.FLAG_KEEP_LOGITS, 0):
+        dec = SpecDecoder(cfg, dw, tree, 64, max_batch=batch, flags=flags)
+        dec.prefill([draw_prompt(cfg.with_(seed=30 + b), 5 + b) for b in range(batch)])
+        dec.step()
+        got.append(dec.debug(B.DBG_ARGMAX).copy())
+        if flags:
+            assert (dec.debug(B.DBG_LOGITS).argmax(-1) == got[0]).all()
+        dec.close()
+    assert (got[0] == got[1]).all()
