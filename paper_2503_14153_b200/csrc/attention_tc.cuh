@@ -44,7 +44,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 
 constexpr int ATTN_MAX_STAGES = 6;
 constexpr int ATTN_PT_CACHE = 256;
-constexpr int ATTN_MAX_SEQS = 16;
+constexpr int ATTN_MAX_SEQS = 32;
 
 struct AttnTcArgs {
   const bf16* q;        // [M][H*HD]

@@ -5,6 +5,12 @@
 // With 128 rows (prompt chunks, trees of more than 64 nodes) a thread of a softmax group owns a row of the tile. Taking
 // 128 rows at a time instead of two CTAs of 64, each reading the keys, shortens a layer's attention over a 2048-token
 // prompt (16 chunks, 32 heads) from 146 to 118 us. What follows describes 64 rows.
+// Where there are more (row group, head) items than SMs, a CTA takes one after another, the longest first, the next free one by a
+// counter: the query rows (TMA) and the first key tiles of the next item are on their way, and its first scores computed, while the
+// softmax warps finish the last one, and tensor memory and barriers are set up once. What remains exposed of an item is the merge
+// of its streams. A CTA an item spent about 10 us around 8 tiles of 1.4: with this and the merge below, 16 sequences of 64 rows at
+// 128..2048 keys 81 -> 76 us a layer (K and V alone take 44), eight ragged prompts through 4 layers 5.30 -> 5.02 ms; one
+// sequence of 8192 keys 33.6 -> 32.8.
 // A warp can read only the 32 tensor-memory lanes of
 // its own SM quarter, and lane = MMA row, so to put all four quarters to work the 64 query rows are given
 // twice to the 128-row MMA: rows 0..63 ("low stream") take care of keys 0..63 of every tile, rows 64..127
@@ -23,13 +29,15 @@
 // (K / V x dims 0..63 / 64..127) with four 5-dimensional TMA loads straight out of the page pool -- the
 // library places page p of sequence b at pool page p * max_batch + b and keeps the pages of a (layer, head)
 // side by side, so a sequence's pages are a strided dimension of the tensor map --; one thread issues all
-// MMAs. The four streams of a row (two groups x two key halves) are merged through shared memory. The key
-// splits of a (sequence, row half, head) form one thread-block cluster, split s owning tiles s, s + cluster
+// MMAs. Of the four streams of a row (two groups x two key halves) the groups' two sit in the same tensor-memory
+// lane, so each thread adds them straight from both accumulators; the key halves' are swapped through the blocks of
+// the P operands that are free between items (staging all four streams took 135 KB of shared memory, the next
+// item's tiles among it, and 2.3 us). The key
+// splits of a (sequence, head) form one thread-block cluster, split s owning tiles s, s + cluster
 // size, ... (which tiles does not depend on the length, so the first two can be asked for before the
 // dependency wait when they lie below the host's lower bound of the committed length): each CTA leaves its
 // merged partial in its own shared memory, and after a cluster barrier every CTA finishes a share of the
-// rows, reading all the partials through distributed shared memory -- no partial sums in HBM, no arrival
-// counter. Every mbarrier wait is bounded; a CTA whose wait ran out still joins the cluster barriers, so its
+// rows, reading all the partials through distributed shared memory -- no partial sums in HBM. Every mbarrier wait is bounded; a CTA whose wait ran out still joins the cluster barriers, so its
 // peers do not wait for it.
 #pragma once
 #include <cuda.h>
@@ -47,7 +55,7 @@ constexpr int AU_MAX_CLUSTER = 8; // most key splits (portable cluster size)
 constexpr int AU_EXP = 132;       // floats per staged output row: head_dim + 4 (16-byte aligned rows, banks shifted by 4)
 
 __host__ __device__ inline size_t attention_umma_smem() {
-  return 1024 /*alignment*/ + 32768 /*Q, twice*/ + 2 * 32768 /*P*/ + 2 * 65536 /*K/V stages*/ + 256 /*barriers*/;
+  return 1024 /*alignment*/ + 32768 /*Q, twice*/ + 2 * 32768 /*P*/ + 2 * 65536 /*K/V stages*/ + 512 /*barriers, items*/;
 }
 
 __device__ __forceinline__ void tma_load_5d(void* smem_dst, const void* tmap, int c0, int c1, int c2, int c3, int c4, uint64_t* bar) {
@@ -83,18 +91,32 @@ __device__ __forceinline__ float2 dsmem_ld2(uint32_t addr) {
 }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+constexpr int AU_ITEMS = 8;       // announced (row group, head) items a CTA can have in hand (its roles are at most six items apart)
+
+__device__ __forceinline__ float exp2_fast(float x) {        // (results below 2^-126 are zero; the others are exp2f's)
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// Barrier of the eight softmax warps, and the same telling whether `v` holds in all of their threads.
+__device__ __forceinline__ void softmax_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ bool softmax_and(bool v) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.and.pred q, 2, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"((uint32_t)v) : "memory");
+  return r != 0;
+}
+
 template <int HD, int ROWS>
 __global__ void __launch_bounds__(AU_THREADS, 1)
-attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, unsigned long long* tr) {
+attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant__ CUtensorMap tm_q, const AttnTcArgs a, unsigned long long* tr) {
   static_assert(HD == 128, "two 64-dim slabs per row");
   static_assert(ROWS == 64 || ROWS == 128, "query rows per CTA");
-  constexpr int AU_ROWS = ROWS;
-  constexpr int STREAMS = 256 / ROWS;         // softmax streams a query row has: two groups, times two key halves with 64 rows
   KTrace kt(tr);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  uint8_t* q_s = sm;                          // 2 slabs x [128 rows][128 B] (rows 64.. repeat rows 0..63)
+  uint8_t* q_s = sm;                          // 2 slabs x [128 rows][128 B] (64 rows: rows 64.. repeat rows 0..63)
   uint8_t* p_s = sm + 32768;                  // [2 buffers] x 2 slabs x [128 rows][128 B]; slab h = keys [64 h, +64) of the tile
   uint8_t* kv_s = sm + 32768 + 65536;         // [2 stages] x (K slab 0, K slab 1, V slab 0, V slab 1) x [128 keys][128 B]
   uint64_t* bars = reinterpret_cast<uint64_t*>(kv_s + 2 * 65536);
@@ -105,60 +127,61 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
   uint64_t* s_full = bars + 8;                // [2] scores of a tile are in tensor memory
   uint64_t* p_full = bars + 10;               // [2] P operand written (the group's four warps)
   uint64_t* o_done = bars + 12;               // [2] P V of a tile has been added to the group's accumulator
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 14);
+  uint64_t* q_full = bars + 14;               // an item's query rows have landed
+  uint64_t* q_empty = bars + 15;              // ... have been read by its score MMAs
+  uint64_t* item_full = bars + 16;            // [AU_ITEMS] an item is announced
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16 + AU_ITEMS);
+  int4* items = reinterpret_cast<int4*>(bars + 18 + AU_ITEMS);   // [AU_ITEMS] (row group or -1: no more, head, committed length, rows)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int halves = gridDim.z / a.rows.B;
-  // CTAs are handed out in grid order: with more CTAs than SMs the longest sequences go first, so that the
-  // launch does not end on a long sequence started last (the host sorts by its bounds of the lengths)
-  const int zb = blockIdx.z / halves;
-  const int h = blockIdx.x, sp = blockIdx.y, b = a.rows.B <= ATTN_MAX_SEQS ? (int)a.order[zb] : zb, half = blockIdx.z % halves;
-  const int row0 = half * AU_ROWS;
-  const int H = a.H, kvh = h / (H / a.g.n_kv_heads);
-  const int ncl = (int)gridDim.y;                              // key splits = the cluster; split sp owns tiles sp, sp + ncl, ...
-  // ---- producer's loads: two K slabs and two V slabs per tile, K one tile ahead of V (K is released by the
-  // score MMAs, long before the tile's V is released by the P V MMAs) ----
-  const int seq = a.rows.sequence(b);
-  const int lh = a.layer * a.g.n_kv_heads + kvh;             // slab rows of a page's pair: K dims 0..63, K 64..127, V, V
-  auto load_k = [&](int t) -> bool {
-    const int st = t & 1;
-    if (t >= 2 && !mbar_wait(&k_empty[st], ((t >> 1) - 1) & 1, a.status, 50)) return false;
-    uint8_t* dst = kv_s + st * 65536;
-    mbar_expect_tx(&k_full[st], 32768);
+  const int H = a.H, R = a.rows.R, n_items = H * a.rows.B;
+  const int sp = blockIdx.y, ncl = (int)gridDim.y;             // key split = rank in the cluster; split sp owns tiles sp, sp + ncl, ...
+  // Items are (row group, head) pairs, the longest sequences first (the host sorts by its bounds of the lengths). With one split
+  // a CTA begins with the item of its number and takes the next free one, by a counter, when it is through.
+  const int item0 = ncl == 1 ? (int)blockIdx.x : (int)(blockIdx.z * H + blockIdx.x);
+  auto group_of = [&](int item) { const int zb = item / H; return a.rows.B <= ATTN_MAX_SEQS ? (int)a.order[zb] : zb; };
+  auto tiles_of = [&](int n, int cnt) -> int {
+    const int total = cnt > 0 ? (n + cnt + AU_KT - 1) / AU_KT : 0;
+    return sp < total ? (total - sp + ncl - 1) / ncl : 0;
+  };
+  // ---- producer's loads of tile t of an item, the T-th of the CTA: two K slabs and two V slabs, K one tile ahead of V (K is
+  // released by the score MMAs, long before the tile's V is released by the P V MMAs) ----
+  auto load_half = [&](int T, int t, int seq, int lh, int v, uint64_t* fullb, uint64_t* emptyb, int where) -> bool {
+    const int st = T & 1;
+    if (T >= 2 && !mbar_wait(&emptyb[st], ((T >> 1) - 1) & 1, a.status, where)) return false;
+    uint8_t* dst = kv_s + st * 65536 + v * 32768;
+    mbar_expect_tx(&fullb[st], 32768);
     const int page0 = (sp + t * ncl) * (AU_KT / 16);
-    tma_load_5d(dst, &tm_kv, 0, 0, seq, page0, lh, &k_full[st]);
-    tma_load_5d(dst + 16384, &tm_kv, 0, 16, seq, page0, lh, &k_full[st]);
+    tma_load_5d(dst, &tm_kv, 0, 32 * v, seq, page0, lh, &fullb[st]);       // slab rows of a page's pair: K dims 0..63, K 64..127, V, V
+    tma_load_5d(dst + 16384, &tm_kv, 0, 32 * v + 16, seq, page0, lh, &fullb[st]);
     return true;
   };
-  auto load_v = [&](int t) -> bool {
-    const int st = t & 1;
-    if (t >= 2 && !mbar_wait(&v_empty[st], ((t >> 1) - 1) & 1, a.status, 56)) return false;
-    uint8_t* dst = kv_s + st * 65536 + 32768;
-    mbar_expect_tx(&v_full[st], 32768);
-    const int page0 = (sp + t * ncl) * (AU_KT / 16);
-    tma_load_5d(dst, &tm_kv, 0, 32, seq, page0, lh, &v_full[st]);
-    tma_load_5d(dst + 16384, &tm_kv, 0, 48, seq, page0, lh, &v_full[st]);
-    return true;
-  };
+  auto kv_head = [&](int h) { return a.layer * a.g.n_kv_heads + h / (H / a.g.n_kv_heads); };
+  auto load_k = [&](int T, int t, int seq, int lh) { return load_half(T, t, seq, lh, 0, k_full, k_empty, 50); };
+  auto load_v = [&](int T, int t, int seq, int lh) { return load_half(T, t, seq, lh, 1, v_full, v_empty, 56); };
   // The producer thread sets up the barriers itself and at once asks for its first two tiles where they lie
   // wholly below the host's lower bound of the committed length: those keys were written by earlier steps (no
   // kernel of this step starts before the kernels of the step before it have completed), so the loads need not
   // wait for the kernel before this one, and which tiles a split owns does not depend on the length.
   int pre = 0;                                                 // tiles whose loads went out before the dependency wait
   if (threadIdx.x == 8 * 32) {
-    for (int i = 0; i < 14; ++i) mbar_init(&bars[i], (i == 10 || i == 11) ? 4 : 1);
+    for (int i = 0; i < 16 + AU_ITEMS; ++i) mbar_init(&bars[i], (i == 10 || i == 11) ? 4 : 1);
     mbar_fence_init();
-    const int n_lo = b < ATTN_MAX_SEQS ? a.n_lo[b] : 0;
+    const int z = group_of(item0), n_lo = z < ATTN_MAX_SEQS ? a.n_lo[z] : 0;
     if ((sp + 1) * AU_KT <= n_lo) {
-      load_k(0);
+      const int seq = a.rows.sequence(z), lh = kv_head(item0 % H);
+      load_k(0, 0, seq, lh);
       pre = 1;
-      if ((sp + ncl + 1) * AU_KT <= n_lo) { load_k(1); pre = 2; }
-      load_v(0);
+      if ((sp + ncl + 1) * AU_KT <= n_lo) { load_k(1, 1, seq, lh); pre = 2; }
+      load_v(0, 0, seq, lh);
     }
   }
   if (warp == 9) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   // with 64 rows the P operands' off-diagonal blocks stay zero for the whole kernel
-  if (ROWS == 64) for (int c = threadIdx.x; c < 65536 / 16; c += AU_THREADS) reinterpret_cast<uint4*>(p_s)[c] = make_uint4(0, 0, 0, 0);
+  if (ROWS == 64) {
+    for (int c = threadIdx.x; c < 65536 / 16; c += AU_THREADS) reinterpret_cast<uint4*>(p_s)[c] = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -168,136 +191,168 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
   pdl_launch_dependents();
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
-  const int R = a.rows.R, cnt = a.rows.cnt[b], n = a.rows.n[b];
-  const int S = n + cnt;
-  const int total_tiles = (S + AU_KT - 1) / AU_KT;
-  const int nt = sp < total_tiles ? (total_tiles - sp + ncl - 1) / ncl : 0;   // (pre <= nt: the tiles asked for lie below n)
-  const bool active = row0 < cnt && nt > 0;
-  if (active) {
-    if (warp == 8) {
-      // the first tiles are on their way while the other warps stage Q
-      if (lane == 0) {
-        if (pre < 1) load_k(0);
-        if (pre < 2 && nt > 1) load_k(1);
-        if (pre < 1) load_v(0);
-      }
-    } else if (warp < 8) {
-      // Q rows of this CTA into the two K-major slabs, with 64 rows each row at r and at r + 64 (rows beyond cnt are
-      // zeros); a thread fetches its pieces before it stores the first
-      constexpr int PIECES = ROWS * (HD / 8) / 256;
-      uint4 v[PIECES];
+
+  // ---- cluster of key splits: what a CTA leaves for its peers, in the stages (all its tiles have been read by then) ----
+  float* ex = reinterpret_cast<float*>(kv_s);                  // [ROWS][AU_EXP]
+  float* cml = ex + ROWS * AU_EXP;                             // [ROWS] (reference, sum)
+
+  if (warp == 8) {
+    if (lane == 0) {
+      int T = 0, q_items = 0;
+      auto announce = [&](int k, int it) -> int4 {
+        int4 v = make_int4(-1, 0, 0, 0);
+        if (it < n_items) {
+          v.x = group_of(it); v.y = it % H;
+          v.z = a.rows.n[v.x]; v.w = a.rows.cnt[v.x];
+        }
+        items[k % AU_ITEMS] = v;
+        mbar_arrive(&item_full[k % AU_ITEMS]);
+        return v;
+      };
+      int4 cur = announce(0, item0);
+      bool ok = true;
+      for (int k = 0; cur.x >= 0 && ok; ++k) {
+        const int nt = tiles_of(cur.z, cur.w), seq = a.rows.sequence(cur.x), lh = kv_head(cur.y);
+        if (k) pre = 0;
+        int4 next = make_int4(-1, 0, 0, 0);
+        // the next item: from the counter, which the last to ask puts back to zero
+        auto ask = [&](bool go_on) {
+          int it = n_items;
+          if (ncl == 1)
+            do {
+              const unsigned int got = atomicAdd(a.arrive, 1u);
+              if (got == (unsigned)(n_items - 1)) *a.arrive = 0u;
+              it = (int)(gridDim.x + got);
+            } while (it < n_items && (!go_on || a.rows.cnt[group_of(it)] <= 0));     // (a group without rows has nothing to do)
+          next = announce(k + 1, it);
+        };
+        if (nt == 0) {
+          // a group without rows, or a split without tiles; loads asked for above must have landed before the CTA gives up its
+          // shared memory, and with them its stages are out of step: it takes no further item (an error of the pass)
+          if (pre > 0) { mbar_wait(&k_full[0], 0, a.status, 59); mbar_wait(&v_full[0], 0, a.status, 59); }
+          if (pre > 1) mbar_wait(&k_full[1], 0, a.status, 59);
+          ask(pre == 0);
+        } else {
+          if (q_items > 0 && !mbar_wait(q_empty, (q_items - 1) & 1, a.status, 53)) { ok = false; break; }
+          ++q_items;
+          // the query rows (with 64 of them each at r and at r + 64). Rows beyond the group's count bring whatever is there: a
+          // row's scores and output depend on no other row, and theirs are not stored.
+          mbar_expect_tx(q_full, 32768);
 #pragma unroll
-      for (int k = 0; k < PIECES; ++k) {
-        const int c = threadIdx.x + 256 * k, qr = c / (HD / 8), ch = c % (HD / 8);
-        v[k] = make_uint4(0, 0, 0, 0);
-        if (row0 + qr < cnt) v[k] = *reinterpret_cast<const uint4*>(a.q + (size_t)(b * R + row0 + qr) * H * HD + h * HD + ch * 8);
-      }
-#pragma unroll
-      for (int k = 0; k < PIECES; ++k) {
-        const int c = threadIdx.x + 256 * k, qr = c / (HD / 8), ch = c % (HD / 8);
-        uint8_t* dst = q_s + (ch >> 3) * 16384 + qr * 128 + (((ch & 7) ^ (qr & 7)) << 4);   // (qr + 64) & 7 == qr & 7
-        *reinterpret_cast<uint4*>(dst) = v[k];
-        if (ROWS == 64) *reinterpret_cast<uint4*>(dst + 64 * 128) = v[k];
+          for (int j = 0; j < 4; ++j)
+            tma_load_2d(q_s + (j & 1) * 16384 + (j >> 1) * 8192, &tm_q, cur.y * HD + (j & 1) * 64, cur.x * R + (ROWS == 128 ? (j >> 1) * 64 : 0), q_full);
+          if (pre < 1) ok = load_k(T, 0, seq, lh);
+          if (ok && pre < 2 && nt > 1) ok = load_k(T + 1, 1, seq, lh);
+          if (ok && pre < 1) ok = load_v(T, 0, seq, lh);
+          // (asking takes two trips to L2, in which this thread issues no loads: not before the second tile's are out)
+          if (nt == 1) ask(true);
+          for (int t = 1; t < nt && ok; ++t) {
+            if (t + 1 < nt) ok = load_k(T + t + 1, t + 1, seq, lh);
+            if (ok) ok = load_v(T + t, t, seq, lh);
+            if (t == 1) ask(true);
+          }
+          T += nt;
+        }
+        cur = next;
       }
     }
-  } else if (pre > 0 && threadIdx.x == 8 * 32) {
-    // rows beyond the pass's count: nothing to do, but the loads asked for above must have landed before the
-    // CTA gives up its shared memory
-    mbar_wait(&k_full[0], 0, a.status, 59);
-    mbar_wait(&v_full[0], 0, a.status, 59);
-    if (pre > 1) mbar_wait(&k_full[1], 0, a.status, 59);
-  }
-  fence_proxy_async_smem();
-  __syncthreads();
-
-  const int grp = warp >> 2;                                   // softmax group of warps 0..3 / 4..7
-  const int q4 = warp & 3;                                     // SM quarter = tensor-memory lanes [32 q4, +32)
-  const int mrow = q4 * 32 + lane;                             // this thread's MMA row (tensor-memory lane)
-  const int qrow = mrow & (AU_ROWS - 1);                       // its query row within the CTA
-  const int kh = ROWS == 64 ? mrow >> 6 : 0;                   // 64 rows: its key half of every tile
-  float m_ref = -INFINITY, l_run = 0.f;
-  int my_tiles = 0;
-  bool ok = true;
-
-  if (active) {
-    if (warp == 8) {
-      if (lane == 0) {
-        for (int t = 1; t < nt && ok; ++t) {
-          if (t + 1 < nt && !load_k(t + 1)) { ok = false; break; }
-          if (!load_v(t)) { ok = false; break; }
+  } else if (warp == 9) {
+    if (lane == 0) {
+      // ---- MMA issuer. Order S(0), S(1), then PV(T), S(T + 2) for T = 0, 1, ..., over all items: the scores of the next two tiles
+      // are always out before a group's probabilities are awaited, and no MMA waits behind a load it does not need ----
+      const uint32_t idesc_s = make_idesc_bf16(128, AU_KT);                  // A and B K-major
+      const uint32_t idesc_o = make_idesc_bf16(128, HD) | (1u << 16);        // B (V) MN-major
+      const uint32_t q_addr = smem_u32(q_s);
+      bool ok = true;
+      auto read_item = [&](int k) -> int4 {
+        if (!mbar_wait(&item_full[k % AU_ITEMS], (k / AU_ITEMS) & 1, a.status, 60)) { ok = false; return make_int4(-1, 0, 0, 0); }
+        return items[k % AU_ITEMS];
+      };
+      int s_item = 0, s_t = 0, s_nt = 0, s_T = 0, s_q = 0;
+      bool s_more = true;
+      auto score_next = [&]() {                                              // scores of the next tile, if there is one
+        while (s_more && s_t == s_nt) {
+          const int4 v = read_item(s_item++);
+          if (v.x < 0) { s_more = false; break; }
+          s_nt = tiles_of(v.z, v.w); s_t = 0;
         }
-      }
-    } else if (warp == 9) {
-      if (lane == 0) {
-        // ---- MMA issuer. Order S(0), S(1), then PV(t), S(t + 2) for t = 0, 1, ...: the scores of the next two tiles are
-        // always out before a group's probabilities are awaited, and no MMA waits behind a load it does not need ----
-        const uint32_t idesc_s = make_idesc_bf16(128, AU_KT);                  // A and B K-major
-        const uint32_t idesc_o = make_idesc_bf16(128, HD) | (1u << 16);        // B (V) MN-major
-        const uint32_t q_addr = smem_u32(q_s);
-        auto mma_s = [&](int t) -> bool {
-          const int bf = t & 1, st = t & 1;
-          if (!mbar_wait(&k_full[st], (t >> 1) & 1, a.status, 51)) return false;
-          tc_fence_after();
-          const uint32_t d_addr = tmem + (uint32_t)(bf * 128);
-          const uint32_t k_addr = smem_u32(kv_s + st * 65536);
+        if (!s_more || !ok) return;
+        if (s_t == 0 && !mbar_wait(q_full, s_q++ & 1, a.status, 61)) { ok = false; return; }
+        const int bf = s_T & 1;
+        if (!mbar_wait(&k_full[bf], (s_T >> 1) & 1, a.status, 51)) { ok = false; return; }
+        tc_fence_after();
+        const uint32_t d_addr = tmem + (uint32_t)(bf * 128);
+        const uint32_t k_addr = smem_u32(kv_s + bf * 65536);
 #pragma unroll
-          for (int j = 0; j < HD / 16; ++j) {                                 // k-steps of 16 dims
-            const uint64_t ad = make_kmajor_sw128_desc(q_addr + (j >> 2) * 16384) + 2 * (j & 3);
-            const uint64_t bd = make_kmajor_sw128_desc(k_addr + (j >> 2) * 16384) + 2 * (j & 3);
-            tc_mma_f16(d_addr, ad, bd, idesc_s, j > 0 ? 1u : 0u);
-          }
-          tc_commit(&s_full[bf]);
-          tc_commit(&k_empty[st]);
-          return true;
-        };
-        auto mma_pv = [&](int u) -> bool {
-          const int bf = u & 1, st = u & 1;
-          if (!mbar_wait(&p_full[bf], (u >> 1) & 1, a.status, 52)) return false;
-          if (!mbar_wait(&v_full[st], (u >> 1) & 1, a.status, 57)) return false;
+        for (int j = 0; j < HD / 16; ++j) {                                   // k-steps of 16 dims
+          const uint64_t ad = make_kmajor_sw128_desc(q_addr + (j >> 2) * 16384) + 2 * (j & 3);
+          const uint64_t bd = make_kmajor_sw128_desc(k_addr + (j >> 2) * 16384) + 2 * (j & 3);
+          tc_mma_f16(d_addr, ad, bd, idesc_s, j > 0 ? 1u : 0u);
+        }
+        tc_commit(&s_full[bf]);
+        tc_commit(&k_empty[bf]);
+        ++s_T;
+        if (++s_t == s_nt) tc_commit(q_empty);
+      };
+      score_next();
+      score_next();
+      if (ok) trace_mark_max(tr, 3);
+      int T = 0;
+      for (int k = 0; ok; ++k) {
+        const int4 v = read_item(k);
+        if (v.x < 0) break;
+        const int nt = tiles_of(v.z, v.w);
+        for (int t = 0; t < nt && ok; ++t, ++T) {
+          const int bf = T & 1;
+          if (!mbar_wait(&p_full[bf], (T >> 1) & 1, a.status, 52) || !mbar_wait(&v_full[bf], (T >> 1) & 1, a.status, 57)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t d_addr = tmem + 256u + (uint32_t)(bf * 128);            // the group's accumulator
-          const uint32_t p_addr = smem_u32(p_s + bf * 32768), v_addr = smem_u32(kv_s + st * 65536 + 32768);
+          const uint32_t d_addr = tmem + 256u + (uint32_t)(bf * 128);          // the group's accumulator
+          const uint32_t p_addr = smem_u32(p_s + bf * 32768), v_addr = smem_u32(kv_s + bf * 65536 + 32768);
 #pragma unroll
           for (int j = 0; j < AU_KT / 16; ++j) {                              // k-steps of 16 keys
             const uint64_t ad = make_kmajor_sw128_desc(p_addr + (j >> 2) * 16384) + 2 * (j & 3);
             const uint64_t bd = make_sw128_desc(v_addr + j * 2048, 16384, 1024);
-            tc_mma_f16(d_addr, ad, bd, idesc_o, (u >= 2 || j > 0) ? 1u : 0u);   // a group's first tile starts its accumulator
+            tc_mma_f16(d_addr, ad, bd, idesc_o, (t >= 2 || j > 0) ? 1u : 0u);   // a group's first tile of an item starts its accumulator
           }
           tc_commit(&o_done[bf]);
-          tc_commit(&v_empty[st]);
-          return true;
-        };
-        ok = mma_s(0);
-        if (ok && nt > 1) ok = mma_s(1);
-        if (ok) trace_mark_max(tr, 3);
-        for (int t = 0; t < nt && ok; ++t) {
-          if (!mma_pv(t)) { ok = false; break; }
-          if (t + 2 < nt && !mma_s(t + 2)) { ok = false; break; }
+          tc_commit(&v_empty[bf]);
+          score_next();
         }
       }
-    } else {
-      // ---- softmax groups: tiles grp, grp + 2, ...; a thread = one query row x one half of every tile's keys ----
-      const int i_row = row0 + qrow;
+    }
+  } else {
+    // ---- softmax groups: every second tile; a thread = one query row (64 rows: and one half of every tile's keys) ----
+    const int grp = warp >> 2;                                 // softmax group of warps 0..3 / 4..7
+    const int q4 = warp & 3;                                   // SM quarter = tensor-memory lanes [32 q4, +32)
+    const int mrow = q4 * 32 + lane;                           // this thread's MMA row (tensor-memory lane)
+    const int qrow = mrow & (ROWS - 1);                        // its query row
+    const int kh = ROWS == 64 ? mrow >> 6 : 0;                 // 64 rows: its key half of every tile
+    const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
+    int T0 = 0;                                                // the CTA's tiles before this item
+    for (int k = 0;; ++k) {
+      bool ok = mbar_wait(&item_full[k % AU_ITEMS], (k / AU_ITEMS) & 1, a.status, 62);
+      const volatile int* item = reinterpret_cast<const volatile int*>(items + k % AU_ITEMS);
+      if (!softmax_and(ok) || item[0] < 0) break;              // (the same in all 256 threads)
+      const int n = item[2], nt = tiles_of(n, item[3]);
+      float m_ref = -INFINITY, l_run = 0.f;
+      int my_tiles = 0;
       uint32_t anc[4];
 #pragma unroll
-      for (int w = 0; w < 4; ++w) anc[w] = i_row < cnt ? a.rows.anc[i_row * 4 + w] : 0u;
-      const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
+      for (int w = 0; w < 4; ++w) anc[w] = qrow < item[3] ? __ldg(a.rows.anc + qrow * 4 + w) : 0u;
       // Raises the stream's reference to the tile's maximum `tmax` (unscaled) where it has to and returns what the sums so far
       // are multiplied by; the group's previous tile must be through the tensor cores by then (its P operand and
       // accumulator are reused), which is awaited here.
-      auto raise_reference = [&](float tmax, int t) -> float {
-        const int bf = t & 1;
+      auto raise_reference = [&](float tmax, int t, int T) -> float {
         tmax *= a.scale_log2;
         // raise the reference only when it is too low by more than 2^AU_RESCALE_LOG2 (or not set yet)
         const bool raise = tmax > m_ref + AU_RESCALE_LOG2 || (m_ref == -INFINITY && tmax > -INFINITY);
         const float m_new = raise ? tmax : m_ref;
         const float alpha = raise ? exp2f(m_ref - m_new) : 1.f;   // 0 the first time
-        // the group's previous tile must be through the tensor cores: its P operand and accumulator are reused
-        if (t >= 2 && !mbar_wait(&o_done[bf], ((t >> 1) - 1) & 1, a.status, 55)) { ok = false; return 1.f; }
+        if (t >= 2 && !mbar_wait(&o_done[grp], ((T >> 1) - 1) & 1, a.status, 55)) { ok = false; return 1.f; }
         if (__any_sync(0xffffffffu, raise && my_tiles > 0)) {
           // rescale this lane's accumulator row (other lanes of the warp multiply by one)
           tc_fence_after();
-          const uint32_t o_addr = tmem + lane_base + 256u + (uint32_t)(bf * 128);
+          const uint32_t o_addr = tmem + lane_base + 256u + (uint32_t)(grp * 128);
 #pragma unroll 1
           for (int c = 0; c < 4; ++c) {
             uint32_t r[32];
@@ -312,9 +367,9 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
         m_ref = m_new;
         return alpha;
       };
-      for (int t = grp; t < nt; t += 2) {
-        const int bf = t & 1;
-        if (!mbar_wait(&s_full[bf], (t >> 1) & 1, a.status, 54)) { ok = false; break; }
+      for (int t = (T0 ^ grp) & 1; t < nt; t += 2) {
+        const int bf = grp;
+        if (!mbar_wait(&s_full[bf], ((T0 + t) >> 1) & 1, a.status, 54)) { ok = false; break; }
         tc_fence_after();
         if constexpr (ROWS == 128) {
           // a thread has all 128 keys of the tile: 32 scores at a time, read out of tensor memory once for the maximum and
@@ -341,7 +396,7 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
               for (int j = 0; j < 32; ++j) if ((vis[c] >> j) & 1u) tmax = fmaxf(tmax, __uint_as_float(r[j]));
             }
           }
-          const float alpha = raise_reference(tmax, t);
+          const float alpha = raise_reference(tmax, t, T0 + t);
           if (!ok) break;
           const float base = (m_ref == -INFINITY) ? 0.f : m_ref;
           l_run *= alpha;
@@ -354,8 +409,8 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
-              float p0 = exp2f(fmaf(__uint_as_float(r[j]), a.scale_log2, -base));
-              float p1 = exp2f(fmaf(__uint_as_float(r[j + 1]), a.scale_log2, -base));
+              float p0 = exp2_fast(fmaf(__uint_as_float(r[j]), a.scale_log2, -base));
+              float p1 = exp2_fast(fmaf(__uint_as_float(r[j + 1]), a.scale_log2, -base));
               if (!whole) {
                 if (!((vis[c] >> j) & 1u)) p0 = 0.f;
                 if (!((vis[c] >> (j + 1)) & 1u)) p1 = 0.f;
@@ -394,7 +449,7 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
               if ((vis1 >> j) & 1u) tmax = fmaxf(tmax, __uint_as_float(r1[j]));
             }
           }
-          const float alpha = raise_reference(tmax, t);
+          const float alpha = raise_reference(tmax, t, T0 + t);
           if (!ok) break;
           l_run *= alpha;
           const float base = (m_ref == -INFINITY) ? 0.f : m_ref;
@@ -408,8 +463,8 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
             uint32_t pk[16];
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
-              float p0 = exp2f(fmaf(__uint_as_float(r[j]), a.scale_log2, -base));
-              float p1 = exp2f(fmaf(__uint_as_float(r[j + 1]), a.scale_log2, -base));
+              float p0 = exp2_fast(fmaf(__uint_as_float(r[j]), a.scale_log2, -base));
+              float p1 = exp2_fast(fmaf(__uint_as_float(r[j + 1]), a.scale_log2, -base));
               if (!((vc >> j) & 1u)) p0 = 0.f;
               if (!((vc >> (j + 1)) & 1u)) p1 = 0.f;
               l0 += p0; l1 += p1;
@@ -430,89 +485,113 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
         if (lane == 0) mbar_arrive(&p_full[bf]);
       }
       // the group's last tile must be through the tensor cores before its accumulator is read
-      if (ok && my_tiles > 0) {
-        const int t_last = grp + 2 * (my_tiles - 1);
-        if (!mbar_wait(&o_done[t_last & 1], (t_last >> 1) & 1, a.status, 58)) ok = false;
-      }
-    }
-  }
-  ok = __syncthreads_and(ok);
-  if (row0 >= cnt) {                                           // the same for every CTA of the cluster
-    if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem, 512); }
-    return;
-  }
-  // ---- the streams of a query row (two groups, with 64 rows times two key halves), staged in shared memory ----
-  float* ex = reinterpret_cast<float*>(sm);                    // [STREAMS][ROWS][AU_EXP]; stream 0 becomes the CTA's partial
-  float* ml = ex + STREAMS * AU_ROWS * AU_EXP;                 // [STREAMS][ROWS] (reference, sum)
-  float* cml = ml + STREAMS * AU_ROWS * 2;                     // [ROWS] of the CTA's partial
-  const bool work = active && ok;
-  if (warp < 8) {
-    const int sid = ROWS == 64 ? grp * 2 + kh : grp;
-    float* my = ex + ((size_t)sid * AU_ROWS + qrow) * AU_EXP;
-    tc_fence_after();
-    if (work && my_tiles > 0) {
-      const uint32_t o_addr = tmem + ((uint32_t)(q4 * 32) << 16) + 256u + (uint32_t)(grp * 128);
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        uint32_t r[32];
-        tmem_ld32(o_addr + c * 32, r);
-        tmem_ld_wait();
+      const int t_last = nt - 1 - ((T0 + nt - 1 - grp) & 1);   // (negative: the group has none)
+      if (ok && t_last >= 0 && !mbar_wait(&o_done[grp], ((T0 + t_last) >> 1) & 1, a.status, 58)) ok = false;
+      // ---- the streams of a query row are merged: the two groups' (each thread reads both accumulators of its tensor-memory lane, group
+      // g half of the dims), with 64 rows also the two key halves', which sit in lanes 64 apart, through the diagonal blocks of the P
+      // operands (the others stay zero) ----
+      // (opaque: the addresses made from them would otherwise be kept in registers through the tiles' loop)
+      const int z = item[0], h = item[1], cnt = item[3];       // (read again: registers)
+      int mrow_ = mrow, qrow_ = qrow;
+      asm volatile("" : "+r"(mrow_), "+r"(qrow_));
+      auto ml = [&](int g) { return reinterpret_cast<float2*>(p_s + g * 32768); };   // [128 lanes] (reference, sum), in the group's own P operand
+      ml(grp)[mrow_] = ok && t_last >= 0 ? make_float2(m_ref, l_run) : make_float2(-INFINITY, 0.f);
+      tc_fence_before();
+      if (!softmax_and(ok)) break;                             // both groups' sums are there and their accumulators complete
+      tc_fence_after();
+      float2 st[4];
 #pragma unroll
-        for (int j = 0; j < 32; j += 4)
-          *reinterpret_cast<float4*>(my + c * 32 + j) =
-              make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+      for (int g = 0; g < 2; ++g) {
+        st[g] = ml(g)[mrow_];
+        st[2 + g] = ROWS == 64 ? ml(g)[mrow_ ^ 64] : make_float2(-INFINITY, 0.f);
       }
-    } else {
-#pragma unroll 4
-      for (int j = 0; j < HD; j += 4) *reinterpret_cast<float4*>(my + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+      const float mm = fmaxf(fmaxf(st[0].x, st[1].x), fmaxf(st[2].x, st[3].x)), base = mm == -INFINITY ? 0.f : mm;
+      const float w0 = exp2f(st[0].x - base), w1 = exp2f(st[1].x - base);
+      // (the same order of the sum in both halves of a row: low keys first)
+      const float own = w0 * st[0].y + w1 * st[1].y;
+      const float other = ROWS == 64 ? exp2f(st[2].x - base) * st[2].y + exp2f(st[3].x - base) * st[3].y : 0.f;
+      const float L = kh ? other + own : own + other;
+      const bool has0 = nt >= 2 || (nt == 1 && !(T0 & 1)), has1 = nt >= 2 || (nt == 1 && (T0 & 1));   // (a group without a tile has no accumulator)
+      // (16 dims at a time, and nothing spilled: with all of the SM's shared memory in use there is hardly any L1 to spill to)
+      auto dims16 = [&](int d, float (&v)[16]) {               // dims [d, +16) of this lane's two streams
+        uint32_t r[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = 0.f;
+        if (has0) {
+          tmem_ld16(tmem + lane_base + 256u + (uint32_t)d, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = w0 * __uint_as_float(r[j]);
+        }
+        if (has1) {
+          tmem_ld16(tmem + lane_base + 384u + (uint32_t)d, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] += w1 * __uint_as_float(r[j]);
+        }
+      };
+      const float inv = 1.f / L;
+      auto emit16 = [&](int d, const float (&v)[16]) {         // ... to the output, or to the cluster's exchange
+        if (ncl > 1) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 4)
+            *reinterpret_cast<float4*>(ex + (size_t)qrow_ * AU_EXP + d + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        } else if (qrow_ < cnt) {
+          uint4* dst = reinterpret_cast<uint4*>(a.out + ((size_t)z * R + qrow_) * H * HD + h * HD + d);
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            dst[j] = make_uint4(pack_bf16(v[8 * j] * inv, v[8 * j + 1] * inv), pack_bf16(v[8 * j + 2] * inv, v[8 * j + 3] * inv),
+                                pack_bf16(v[8 * j + 4] * inv, v[8 * j + 5] * inv), pack_bf16(v[8 * j + 6] * inv, v[8 * j + 7] * inv));
+        }
+      };
+      float v[16];
+      if constexpr (ROWS == 128) {
+#pragma unroll 1
+        for (int d = grp * 64; d < grp * 64 + 64; d += 16) {
+          dims16(d, v);
+          emit16(d, v);
+        }
+      } else {
+        // the thread of key half kh finishes dims [32 kh, +32) of the group's 64 and hands the other 32 over
+        softmax_bar();                                         // (the sums have been read: they lie in two of the blocks)
+        auto at = [&](int half, int c) {                       // 16-byte chunk c of this row in the block for the threads of `half`
+          return reinterpret_cast<float4*>(p_s + grp * 32768 + half * (16384 + 8192) + qrow_ * 128 + ((c ^ (qrow_ & 7)) << 4));
+        };
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          dims16(grp * 64 + (kh ^ 1) * 32 + i * 16, v);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) *at(kh ^ 1, i * 4 + j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        }
+        softmax_bar();
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          dims16(grp * 64 + kh * 32 + i * 16, v);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 o = *at(kh, i * 4 + j);
+            v[4 * j] += o.x; v[4 * j + 1] += o.y; v[4 * j + 2] += o.z; v[4 * j + 3] += o.w;
+          }
+          emit16(grp * 64 + kh * 32 + i * 16, v);
+        }
+      }
+      if (ncl > 1 && grp == 0 && kh == 0) *reinterpret_cast<float2*>(cml + qrow * 2) = make_float2(mm, L);
+      tc_fence_before();
+      softmax_bar();                                           // the accumulators and P operands may be written again
+      T0 += nt;
     }
-    *reinterpret_cast<float2*>(ml + ((size_t)sid * AU_ROWS + qrow) * 2) = work ? make_float2(m_ref, l_run) : make_float2(-INFINITY, 0.f);
-    tc_fence_before();
   }
+  tc_fence_before();
   __syncthreads();
   if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem, 512); }
-  if (warp < 8) {
-    // thread = (row, every STREAMS-th 4-dim chunk): merge the streams
-    const int row = threadIdx.x / STREAMS, qd = threadIdx.x % STREAMS;
-    float ms[STREAMS], ls[STREAMS], mm = -INFINITY;
-#pragma unroll
-    for (int s2 = 0; s2 < STREAMS; ++s2) {
-      const float2 v = *reinterpret_cast<const float2*>(ml + ((size_t)s2 * AU_ROWS + row) * 2);
-      ms[s2] = v.x; ls[s2] = v.y;
-      mm = fmaxf(mm, v.x);
-    }
-    const float base = (mm == -INFINITY) ? 0.f : mm;
-    float L = 0.f;
-#pragma unroll
-    for (int s2 = 0; s2 < STREAMS; ++s2) { ms[s2] = exp2f(ms[s2] - base); L += ms[s2] * ls[s2]; }
-    const float inv = 1.f / L;
-    const size_t m = (size_t)b * R + row0 + row;
-    const bool valid = row0 + row < cnt;
-#pragma unroll
-    for (int j = 0; j < HD / (4 * STREAMS); ++j) {
-      const int d = (j * STREAMS + qd) * 4;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int s2 = 0; s2 < STREAMS; ++s2) {
-        const float4 v = *reinterpret_cast<const float4*>(ex + ((size_t)s2 * AU_ROWS + row) * AU_EXP + d);
-        acc.x += ms[s2] * v.x; acc.y += ms[s2] * v.y; acc.z += ms[s2] * v.z; acc.w += ms[s2] * v.w;
-      }
-      if (ncl == 1) {
-        if (valid) *reinterpret_cast<uint2*>(a.out + m * H * HD + h * HD + d) =
-            make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
-      } else {
-        *reinterpret_cast<float4*>(ex + (size_t)row * AU_EXP + d) = acc;      // in place: only this thread touches it
-      }
-    }
-    if (ncl > 1 && qd == 0) *reinterpret_cast<float2*>(cml + row * 2) = make_float2(mm, L);
-  }
   if (ncl == 1) return;
-  // ---- the cluster's partials: CTA `rank` finishes rows [rank * rpc, +rpc) from everybody's shared memory ----
   __syncwarp();
   cluster_sync_all();
+  const int z = group_of(item0), h = item0 % H, cnt = a.rows.cnt[z];
+  // ---- the cluster's partials: CTA `rank` finishes rows [rank * rpc, +rpc) from everybody's shared memory ----
   {
     const int rank = (int)cluster_ctarank();
-    const int rpc = (AU_ROWS + ncl - 1) / ncl;
+    const int rpc = (ROWS + ncl - 1) / ncl;
     const uint32_t ex_local = smem_u32(ex), cml_local = smem_u32(cml);
     uint32_t ex_r[AU_MAX_CLUSTER], cml_r[AU_MAX_CLUSTER];
 #pragma unroll
@@ -522,7 +601,7 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
     }
     for (int it = threadIdx.x; it < rpc * (HD / 4); it += AU_THREADS) {
       const int row = rank * rpc + it / (HD / 4), d = (it % (HD / 4)) * 4;
-      if (row >= AU_ROWS || row0 + row >= cnt) continue;
+      if (row >= ROWS || row >= cnt) continue;
       float2 mlv[AU_MAX_CLUSTER];
       float4 ov[AU_MAX_CLUSTER];
 #pragma unroll
@@ -546,14 +625,15 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const AttnTcArgs a, un
         acc.x += w * ov[s2].x; acc.y += w * ov[s2].y; acc.z += w * ov[s2].z; acc.w += w * ov[s2].w;
       }
       const float inv = 1.f / L;
-      const size_t m = (size_t)b * R + row0 + row;
+      const size_t m = (size_t)z * R + row;
       *reinterpret_cast<uint2*>(a.out + m * H * HD + h * HD + d) =
           make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
     }
   }
-  // nobody leaves while a peer may still read its shared memory
+  // nobody leaves while a peer may still read its shared memory (the values read are in registers by then: nothing to publish)
   __syncwarp();
-  cluster_sync_all();
+  cluster_arrive_relaxed();
+  cluster_wait();
 }
 
 }  // namespace spec

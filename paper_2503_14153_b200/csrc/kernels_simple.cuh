@@ -127,7 +127,8 @@ gather_prompt_ends(const int* __restrict__ end_row, const int* __restrict__ end_
 // that its prompt fills are left alone: clearing the whole pool took 45 us for a 2048-token prompt and 8 layers of the 7B shape.
 __global__ void __launch_bounds__(256)
 clear_free_pages(uint4* __restrict__ pool, const int* __restrict__ offsets, int batch, int pages_per_seq, int max_batch, int page_size,
-                 int pair_vecs, int share) {
+                 int pair_vecs, int share, unsigned int* __restrict__ item_counter) {
+  if (blockIdx.x + blockIdx.y + threadIdx.x == 0) *item_counter = 0u;   // (of attention_umma: an attention that gave up a wait may have left it set)
   // grid (sequences times the CTAs that share one's pages, layers * heads); pool page p * max_batch + b is page p of sequence b
   const int b = blockIdx.x / share, len = b < batch ? offsets[b + 1] - offsets[b] : 0;
   uint4* base = pool + ((size_t)blockIdx.y * pages_per_seq * max_batch + b) * pair_vecs;

@@ -858,8 +858,7 @@ bool attn_long_mode(const spec_ctx* c, int R, int groups, int keys_hi) {
 
 // Key splits of the tcgen05 kernel = its cluster: one CTA per SM, at most a wave of them.
 int attn_umma_splits(const spec_ctx* c, int R, int groups) {
-  const int halves = R > 64 ? (R + 127) / 128 : 1;
-  return std::max(1, std::min(std::min(c->nsplit_attn, AU_MAX_CLUSTER), (SM_SLOTS / 2) / (c->cfg.n_heads * groups * halves)));
+  return std::max(1, std::min(std::min(c->nsplit_attn, AU_MAX_CLUSTER), (SM_SLOTS / 2) / (c->cfg.n_heads * groups)));
 }
 // First positions of a sequence that the attention kernel of such a pass may fetch ahead of its dependency wait, where they
 // lie below the host's lower bound of the committed length. A bound beyond them makes no difference to the kernel.
@@ -896,16 +895,15 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
     // passes of more than 64 rows (prompt chunks, trees of up to 128 nodes): a CTA takes 128 rows and reads the keys once for
     // them; 64 rows or fewer fill the 128-row MMAs twice, with two halves of the keys
     const bool tall = R > 64;
-    const int halves = tall ? (R + 127) / 128 : 1;
     if (B <= ATTN_MAX_SEQS) {
       int idx[ATTN_MAX_SEQS];
       for (int b = 0; b < B; ++b) idx[b] = b;
       std::stable_sort(idx, idx + B, [&](int x, int y) { return len_now[x] > len_now[y]; });
       for (int b = 0; b < B; ++b) a.order[b] = (unsigned char)idx[b];
     }
-    // the key splits of a (sequence, row half, head) are one cluster
+    // the key splits of a (sequence, head) are one cluster; without splits a CTA takes one (sequence, head) after another
     a.nsplit = attn_umma_splits(c, R, B);
-    dim3 grid(H, a.nsplit, B * halves);
+    const dim3 grid = a.nsplit > 1 ? dim3(H, a.nsplit, B) : dim3(std::min(H * B, SM_SLOTS / 2), 1, 1);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     static bool set_dev[kAttrDevices] = {};
     bool& set_ = *attr_flag(set_dev);
@@ -929,7 +927,9 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
       ++n_at;
     }
     cfg.attrs = at; cfg.numAttrs = (unsigned)n_at;
-    cudaError_t e_ = cudaLaunchKernelEx(&cfg, tall ? attention_umma<128, 128> : attention_umma<128, 64>, c->tm_kv, a, c->next_trace("attention_tc"));
+    const CUtensorMap* tq = c->tmap(c->d_q, c->Mcap, (uint64_t)H * D, 64);
+    if (!tq) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (query rows)");
+    cudaError_t e_ = cudaLaunchKernelEx(&cfg, tall ? attention_umma<128, 128> : attention_umma<128, 64>, c->tm_kv, *tq, a, c->next_trace("attention_tc"));
     c->launches++;
     if (e_ != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("attention_umma: ") + cudaGetErrorString(e_));
     return SPEC_OK;
@@ -1409,7 +1409,7 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
     const int lh = f.n_layers * f.n_kv_heads, share = (int)std::max<long long>(1, std::min<long long>(c->pages_per_seq, 8 * SM_SLOTS / ((long long)lh * f.max_batch)));
     for (int lh0 = 0; lh0 < lh; lh0 += 65535)
       clear_free_pages<<<dim3((unsigned)share * (unsigned)f.max_batch, (unsigned)std::min(65535, lh - lh0)), 256, 0, c->stream>>>(
-          static_cast<uint4*>(c->d_pool) + (size_t)lh0 * c->geom.pool_pages() * pair_vecs, c->d_offsets, batch, c->pages_per_seq, f.max_batch, f.page_size, pair_vecs, share);
+          static_cast<uint4*>(c->d_pool) + (size_t)lh0 * c->geom.pool_pages() * pair_vecs, c->d_offsets, batch, c->pages_per_seq, f.max_batch, f.page_size, pair_vecs, share, c->d_attn_arrive);
     LAUNCH_CHECK("clear_free_pages");
   }
   CUDA_OK(cudaMemsetAsync(c->d_pair_arrive, 0, GP_ARRIVE * sizeof(unsigned int), c->stream));   // (a wait that ran out may have left some set)
