@@ -207,3 +207,28 @@ def test_last_layer_of_a_prompt_for_its_last_rows(torch, lens, layers, hd, batch
         k0, v0 = gpu.read_kv(0, layers - 1, len(prompts[0]) + 30, 2)
         assert not k0.any() and not v0.any()          # nothing was written there since the prompts were processed
     gpu.close()
+
+
+@pytest.mark.parametrize("T,heads,kv,batch", [(48, 16, 4, 12), (64, 32, 32, 5), (80, 16, 16, 11), (128, 32, 8, 6)])
+def test_attention_items_one_after_another(torch, T, heads, kv, batch):
+    """Batched passes with more (sequence, head) items than SMs (160 to 192): a CTA of the tcgen05 attention takes several, of one to four
+    key tiles each, so that an item's first tile falls to either softmax group; 64 and 128 rows a CTA, grouped heads. Two
+    sequences against an oracle each; two steps show that the item counter is back at zero."""
+    from oracle.decoder import OracleModel
+    from oracle.spec import OracleSpecDecoder
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    from tests_lockstep import run_lockstep_batch
+    cfg = BASE.with_(n_heads=heads, n_kv_heads=kv, head_dim=128, tree_nodes=T, seed=210 + T)
+    w = draw_weights(cfg)
+    prompts = [draw_prompt(cfg.with_(seed=220 + i), 3 + (97 * i) % 389) for i in range(batch)]
+    tree = build_tree(cfg.topk, T)
+    room = max(len(p) for p in prompts) + 40
+    gpu = SpecDecoder(cfg, upload_weights(cfg, w), tree, room, max_batch=batch, flags=B.FLAG_KEEP_LOGITS)
+    gpu.set_option(B.OPT_LONG_ATTN_KEYS, 1)
+    model = OracleModel(cfg, w)
+    oracles = {b: OracleSpecDecoder(model, tree, room) for b in (1, batch - 1)}
+    reps = run_lockstep_batch(cfg, gpu, oracles, prompts, 2, TOL_BF16, TIE_GAP, tie_from_row_error=True)
+    gpu.close()
+    for b in oracles:
+        assert reps[b].steps == 2
