@@ -9,7 +9,7 @@
 // counter: the query rows (TMA) and the first key tiles of the next item are on their way, and its first scores computed, while the
 // softmax warps finish the last one, and tensor memory and barriers are set up once. What remains exposed of an item is the merge
 // of its streams. A CTA an item spent about 10 us around 8 tiles of 1.4: with this and the merge below, 16 sequences of 64 rows at
-// 128..2048 keys 81 -> 76 us a layer (K and V alone take 44), eight ragged prompts through 4 layers 5.30 -> 5.02 ms; one
+// 128..2048 keys 81 -> 70 us a layer (K and V alone take 44; 76 while an item's last P V waited behind the next one's first scores), eight ragged prompts through 4 layers 5.30 -> 5.02 ms; one
 // sequence of 8192 keys 33.6 -> 32.8.
 // A warp can read only the 32 tensor-memory lanes of
 // its own SM quarter, and lane = MMA row, so to put all four quarters to work the 64 query rows are given
@@ -258,52 +258,42 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
     }
   } else if (warp == 9) {
     if (lane == 0) {
-      // ---- MMA issuer. Order S(0), S(1), then PV(T), S(T + 2) for T = 0, 1, ..., over all items: the scores of the next two tiles
-      // are always out before a group's probabilities are awaited, and no MMA waits behind a load it does not need ----
+      // ---- MMA issuer. Order within an item S(0), S(1), then PV(t), S(t + 2) for t = 0, 1, ...: the scores of the next two tiles are
+      // always out before a group's probabilities are awaited, and no MMA waits behind a load it does not need (an item's last P V
+      // does not wait for the next item's queries; its first scores are computed while the softmax warps merge) ----
       const uint32_t idesc_s = make_idesc_bf16(128, AU_KT);                  // A and B K-major
       const uint32_t idesc_o = make_idesc_bf16(128, HD) | (1u << 16);        // B (V) MN-major
       const uint32_t q_addr = smem_u32(q_s);
       bool ok = true;
-      auto read_item = [&](int k) -> int4 {
-        if (!mbar_wait(&item_full[k % AU_ITEMS], (k / AU_ITEMS) & 1, a.status, 60)) { ok = false; return make_int4(-1, 0, 0, 0); }
-        return items[k % AU_ITEMS];
-      };
-      int s_item = 0, s_t = 0, s_nt = 0, s_T = 0, s_q = 0;
-      bool s_more = true;
-      auto score_next = [&]() {                                              // scores of the next tile, if there is one
-        while (s_more && s_t == s_nt) {
-          const int4 v = read_item(s_item++);
-          if (v.x < 0) { s_more = false; break; }
-          s_nt = tiles_of(v.z, v.w); s_t = 0;
-        }
-        if (!s_more || !ok) return;
-        if (s_t == 0 && !mbar_wait(q_full, s_q++ & 1, a.status, 61)) { ok = false; return; }
-        const int bf = s_T & 1;
-        if (!mbar_wait(&k_full[bf], (s_T >> 1) & 1, a.status, 51)) { ok = false; return; }
-        tc_fence_after();
-        const uint32_t d_addr = tmem + (uint32_t)(bf * 128);
-        const uint32_t k_addr = smem_u32(kv_s + bf * 65536);
-#pragma unroll
-        for (int j = 0; j < HD / 16; ++j) {                                   // k-steps of 16 dims
-          const uint64_t ad = make_kmajor_sw128_desc(q_addr + (j >> 2) * 16384) + 2 * (j & 3);
-          const uint64_t bd = make_kmajor_sw128_desc(k_addr + (j >> 2) * 16384) + 2 * (j & 3);
-          tc_mma_f16(d_addr, ad, bd, idesc_s, j > 0 ? 1u : 0u);
-        }
-        tc_commit(&s_full[bf]);
-        tc_commit(&k_empty[bf]);
-        ++s_T;
-        if (++s_t == s_nt) tc_commit(q_empty);
-      };
-      score_next();
-      score_next();
-      if (ok) trace_mark_max(tr, 3);
-      int T = 0;
+      int T0 = 0, q_items = 0;                                               // tiles and items with tiles so far
       for (int k = 0; ok; ++k) {
-        const int4 v = read_item(k);
+        if (!mbar_wait(&item_full[k % AU_ITEMS], (k / AU_ITEMS) & 1, a.status, 60)) break;
+        const int4 v = items[k % AU_ITEMS];
         if (v.x < 0) break;
         const int nt = tiles_of(v.z, v.w);
-        for (int t = 0; t < nt && ok; ++t, ++T) {
-          const int bf = T & 1;
+        auto mma_s = [&](int t) -> bool {
+          const int T = T0 + t, bf = T & 1;
+          if (t == 0 && !mbar_wait(q_full, q_items & 1, a.status, 61)) return false;
+          if (!mbar_wait(&k_full[bf], (T >> 1) & 1, a.status, 51)) return false;
+          tc_fence_after();
+          const uint32_t d_addr = tmem + (uint32_t)(bf * 128);
+          const uint32_t k_addr = smem_u32(kv_s + bf * 65536);
+#pragma unroll
+          for (int j = 0; j < HD / 16; ++j) {                                 // k-steps of 16 dims
+            const uint64_t ad = make_kmajor_sw128_desc(q_addr + (j >> 2) * 16384) + 2 * (j & 3);
+            const uint64_t bd = make_kmajor_sw128_desc(k_addr + (j >> 2) * 16384) + 2 * (j & 3);
+            tc_mma_f16(d_addr, ad, bd, idesc_s, j > 0 ? 1u : 0u);
+          }
+          tc_commit(&s_full[bf]);
+          tc_commit(&k_empty[bf]);
+          if (t == nt - 1) tc_commit(q_empty);
+          return true;
+        };
+        if (nt > 0) ok = mma_s(0);
+        if (ok && nt > 1) ok = mma_s(1);
+        if (ok && k == 0) trace_mark_max(tr, 3);
+        for (int t = 0; t < nt && ok; ++t) {
+          const int T = T0 + t, bf = T & 1;
           if (!mbar_wait(&p_full[bf], (T >> 1) & 1, a.status, 52) || !mbar_wait(&v_full[bf], (T >> 1) & 1, a.status, 57)) { ok = false; break; }
           tc_fence_after();
           const uint32_t d_addr = tmem + 256u + (uint32_t)(bf * 128);          // the group's accumulator
@@ -316,8 +306,10 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
           }
           tc_commit(&o_done[bf]);
           tc_commit(&v_empty[bf]);
-          score_next();
+          if (t + 2 < nt) ok = mma_s(t + 2);
         }
+        T0 += nt;
+        if (nt > 0) ++q_items;
       }
     }
   } else {
