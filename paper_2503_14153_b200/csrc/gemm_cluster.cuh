@@ -15,7 +15,7 @@
 // semantics where nothing has to be published (now .relaxed); the copies themselves, 48 KB out of the middle CTA with two CTAs an
 // SM, 1.7 us.
 //
-// Three modes (operands swapped as in gemm_stream: 128 weight rows are the MMA's M, the MT activation
+// Four modes (operands swapped as in gemm_stream: 128 weight rows are the MMA's M, the MT activation
 // rows its N; MT covers all rows of the pass):
 //  * GC_RESIDUAL (output and down projections): a cluster of 8 CTAs per 128-row weight tile, CTA r
 //    streaming the r-th eighth of the K chunks. CTA r owns output columns [16 r, 16 r + 16) of the
@@ -26,8 +26,6 @@
 //    2 KC units of the pair are cut into three equal runs, so CTA 0 holds a gate part, CTA 1 a gate
 //    and an up part (two accumulators) and CTA 2 an up part. Each CTA finishes a share of the tile's columns (48, 32 and 48):
 //    gate = G0 + G1, up = U1 + U2, act = bf16(SiLU(gate) * up).
-//  * GC_SWIGLU8 (the same projections where there are few tiles): a cluster of 8 per pair (gate tile t, up tile t), CTAs 0 to 3
-//    streaming a quarter of the gate tile's K chunks each, 4 to 7 the up tile's; columns as in GC_RESIDUAL.
 //  * GC_PLAIN (a projection by itself; lm_head): a cluster of 1 to 8 per tile, CTA r streaming the r-th part of the K chunks, its
 //    first half into one accumulator and its second into another (the error of a running sum grows with its
 //    length), and finishing a block of rows: float32 sums, and where asked each row's largest in the tile.
@@ -47,17 +45,17 @@
 
 namespace spec {
 
-constexpr int GC_RESIDUAL = 0, GC_SWIGLU = 1, GC_ROPE = 2, GC_SWIGLU8 = 3, GC_PLAIN = 4;
+constexpr int GC_RESIDUAL = 0, GC_SWIGLU = 1, GC_ROPE = 2, GC_PLAIN = 3;
 constexpr int GC_THREADS = 320, GC_EPI = GC_THREADS - 64;     // producer, MMA issuer, eight epilogue warps (two per SM quarter)
 constexpr int GC_RES_CLUSTER = 8, GC_GLU_CLUSTER = 3, GC_ROPE_CLUSTER = 2;
 
 struct ClusterGemmParams {
   int M, K, KC;                 // activation rows (<= MT), inner size, K / 64
   int N;                        // weight rows of one matrix (output columns)
-  const uint8_t* packed[3];     // pre-tiled images (GC_RESIDUAL: [0]; GC_SWIGLU(8): gate, up; GC_ROPE: q, k, v) or nullptr -> tensor maps a[i]
+  const uint8_t* packed[3];     // pre-tiled images (GC_RESIDUAL: [0]; GC_SWIGLU: gate, up; GC_ROPE: q, k, v) or nullptr -> tensor maps a[i]
   float* x;                     // GC_RESIDUAL: [M][N] float32 residual stream, updated in place
   float* ss_part;               // GC_RESIDUAL: [M][ceil(N/128) * 8] sums of squares of the updated pieces, or nullptr
-  bf16* act;                    // GC_SWIGLU(8): [M][N] bf16
+  bf16* act;                    // GC_SWIGLU: [M][N] bf16
   // GC_PLAIN: sums to y[M][ldy], columns below N (y may be nullptr), and of every row's sums in this tile the largest and its column (value
   // descending, column ascending) to best_val / best_idx [M][tiles] (may be nullptr); clear: four ints set to zero, or nullptr
   float* y;
@@ -184,9 +182,8 @@ __global__ void __launch_bounds__(GC_THREADS, 2)
 gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) {
   using Cfg = ClusterCfg<MT>;
   constexpr int STAGES = Cfg::STAGES;
-  constexpr bool EIGHT = MODE == GC_RESIDUAL || MODE == GC_SWIGLU8;      // eight CTAs, each finishing 16 columns
   constexpr bool PLAIN = MODE == GC_PLAIN;
-  const int CS = PLAIN ? (int)cluster_nctarank() : (EIGHT ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER));
+  const int CS = PLAIN ? (int)cluster_nctarank() : (MODE == GC_RESIDUAL ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER));
   constexpr int TMEM_COLS = (MODE == GC_SWIGLU || PLAIN ? 2 : 1) * MT < 32 ? 32 : (MODE == GC_SWIGLU || PLAIN ? 2 : 1) * MT;   // 32 to 256
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -211,10 +208,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   // this CTA's runs
   GcSeg seg[2];
   int nseg = 0;
-  if (MODE == GC_SWIGLU8) {
-    seg[0] = GcSeg{rank >> 2, (rank & 3) * KC / 4, ((rank & 3) + 1) * KC / 4};
-    nseg = 1;
-  } else if (PLAIN) {
+  if (PLAIN) {
     const int k0 = rank * KC / CS, k1 = (rank + 1) * KC / CS, mid = (k0 + k1 + 1) >> 1;
     seg[nseg++] = GcSeg{0, k0, mid};
     if (mid < k1) seg[nseg++] = GcSeg{0, mid, k1};
@@ -235,26 +229,26 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   // GC_SWIGLU: the tile's columns in groups of 16, of which CTA 0 finishes 0..2, CTA 1 3 and 4, CTA 2 5..7
   constexpr int GLU_FIRST[4] = {0, 3, 5, 8};
   const int glu_g0 = GLU_FIRST[rank % 3], glu_ng = GLU_FIRST[rank % 3 + 1] - glu_g0;
-  // ... and more than 64 rows in two rounds, because the ring does not hold all of them staged and arriving at once (GC_PLAIN too)
-  constexpr int ROUNDS = (MODE == GC_SWIGLU || PLAIN) && MT > 64 ? 2 : 1, RT = ROUNDS == 2 ? 64 : MT;
+  // GC_PLAIN: more than 64 rows in two rounds, because the ring does not hold all of them staged and arriving at once
+  constexpr int ROUNDS = PLAIN && MT > 64 ? 2 : 1, RT = ROUNDS == 2 ? 64 : MT;
   const int rr = ROUNDS == 2 ? (M + 31) / 32 * 16 : M;       // rows of a round (at most RT)
   // GC_RESIDUAL: rows that travel as bulk copies; the ring of MT = 128 has no room for the staged copy of all rows beside the
   // arriving ones when there are more than about 100, and the others are sent straight from tensor memory
-  const int S = EIGHT ? min(M, (Cfg::RING_BYTES - GC_RES_CLUSTER * M * 64) / ((GC_RES_CLUSTER - 1) * 64) - 1) : rr;
+  const int S = MODE == GC_RESIDUAL ? min(M, (Cfg::RING_BYTES - GC_RES_CLUSTER * M * 64) / ((GC_RES_CLUSTER - 1) * 64) - 1) : rr;
   // GC_PLAIN: CTA r finishes the r-th block of rows of a round
   const int rb = PLAIN ? (rr + CS - 1) / CS : 0;
-  const int in_pitch = EIGHT ? M * 16 : (rr | 1) * 16;       // floats of a group of 16 columns (odd: banks)
+  const int in_pitch = MODE == GC_RESIDUAL ? M * 16 : (rr | 1) * 16;       // floats of a group of 16 columns (odd: banks)
   const int out_pitch = (S | 1) * 16;
   float* in = staging;
-  float* out = staging + (EIGHT ? GC_RES_CLUSTER * in_pitch : MODE == GC_SWIGLU ? 4 * glu_ng * in_pitch : PLAIN ? CS * rb * 128 : 2 * r_rows * 128);
+  float* out = staging + (MODE == GC_RESIDUAL ? GC_RES_CLUSTER * in_pitch : MODE == GC_SWIGLU ? 4 * glu_ng * in_pitch : PLAIN ? CS * rb * 128 : 2 * r_rows * 128);
   static_assert(!PLAIN || Cfg::RING_BYTES >= (2 * RT + 8) * 512, "a round's rows staged, and eight parts of this CTA's block");
-  static_assert(!EIGHT || Cfg::RING_BYTES >= GC_RES_CLUSTER * MT * 64 + (GC_RES_CLUSTER - 1) * 64 * 17, "in, and 16 rows of out");
+  static_assert(MODE != GC_RESIDUAL || Cfg::RING_BYTES >= GC_RES_CLUSTER * MT * 64 + (GC_RES_CLUSTER - 1) * 64 * 17, "in, and 16 rows of out");
   static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 3 + 5) * (RT | 1) * 64, "CTA 0 and 2: four parts of three groups, five groups to send");
   static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 2 + 2 * 6) * (RT | 1) * 64, "CTA 1: four parts of two groups, six groups of two accumulators");
   static_assert(MODE != GC_ROPE || Cfg::RING_BYTES >= 3 * ((MT + 1) / 2) * 512, "own and arriving rows, rows to send");
   // bytes that arrive in a round of `rows` rows
   auto in_bytes = [&](int rows) -> uint32_t {
-    return EIGHT ? (GC_RES_CLUSTER - 1) * S * 64 : MODE == GC_SWIGLU ? (rank == 1 ? 2 : 3) * glu_ng * rows * 64 : PLAIN ? (CS - 1) * max(0, min(rb, rows - rank * rb)) * 512 : r_rows * 512;
+    return MODE == GC_RESIDUAL ? (GC_RES_CLUSTER - 1) * S * 64 : MODE == GC_SWIGLU ? (rank == 1 ? 2 : 3) * glu_ng * rows * 64 : PLAIN ? (CS - 1) * max(0, min(rb, rows - rank * rb)) * 512 : r_rows * 512;
   };
 
   pdl_launch_dependents();
@@ -281,7 +275,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   };
 
   // GC_RESIDUAL: a finishing thread's items (row, group of four columns) and their old values
-  constexpr int X_PER = EIGHT ? (MT * 4 + GC_EPI - 1) / GC_EPI : 1;
+  constexpr int X_PER = MODE == GC_RESIDUAL ? (MT * 4 + GC_EPI - 1) / GC_EPI : 1;
   float4 xo[X_PER];
   bool x_on[X_PER];
 
@@ -447,7 +441,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
     }
     if (epi) {
       tc_fence_after();
-      if (EIGHT) {
+      if (MODE == GC_RESIDUAL) {
         const bool own = grp == rank;
         float* dst = (own ? in + rank * in_pitch : out + (grp - (grp > rank)) * out_pitch) + (w & 15);
         const int rows = own ? M : S;
@@ -493,10 +487,10 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
         if (lane == 0 && n > 0)
           bulk_push(dsmem_addr(smem_u32(in + q * n * 32), (uint32_t)(rank ^ 1)), out + q * n * 32, n * 128, dsmem_addr(smem_u32(part_full), (uint32_t)(rank ^ 1)));
       } else if ((lane & 15) == 0) {
-        const int to = EIGHT ? grp : (grp < GLU_FIRST[1] ? 0 : (grp < GLU_FIRST[2] ? 1 : 2));
+        const int to = MODE == GC_RESIDUAL ? grp : (grp < GLU_FIRST[1] ? 0 : (grp < GLU_FIRST[2] ? 1 : 2));
         if (to != rank) {
           const uint32_t bar = dsmem_addr(smem_u32(part_full), (uint32_t)to), there = dsmem_addr(smem_u32(in), (uint32_t)to);
-          if (EIGHT) {
+          if (MODE == GC_RESIDUAL) {
             bulk_push(there + (uint32_t)(rank * in_pitch * 4), out + (grp - (grp > rank)) * out_pitch, S * 64, bar);
           } else {
             const int g0 = GLU_FIRST[to], ng = GLU_FIRST[to + 1] - g0;
@@ -509,7 +503,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
         }
       }
     }
-    if (EIGHT && S < M) {                                    // (the same in every CTA of the cluster)
+    if (MODE == GC_RESIDUAL && S < M) {                                    // (the same in every CTA of the cluster)
       if (epi) {
         const uint32_t dst = dsmem_addr(smem_u32(in + rank * in_pitch + (w & 15)), (uint32_t)grp);
         tmem_rows<RT>(taddr, hf, M, [&](int m, float v) { if (m >= S && grp != rank) dsmem_st(dst + (uint32_t)(m * 64), v); });
@@ -583,25 +577,6 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
               warp_argmax(bv, bi);
               if (lane == 0) { p.best_val[(size_t)m * tiles_n + t] = bv; p.best_idx[(size_t)m * tiles_n + t] = bi; }
             }
-          }
-        }
-      } else if (MODE == GC_SWIGLU8) {
-        // the four gate parts and the four up parts of columns [16 rank, +16), each in rank order
-#pragma unroll
-        for (int k = 0; k < X_PER; ++k) {
-          const int it = e + GC_EPI * k, m = it >> 2, col = t * 128 + rank * 16 + (it & 3) * 4;
-          if (m < M && col < p.N) {
-            const float* src = in + m * 16 + (it & 3) * 4;
-            float4 ga = *reinterpret_cast<const float4*>(src), ua = *reinterpret_cast<const float4*>(src + 4 * in_pitch);
-#pragma unroll
-            for (int rr8 = 1; rr8 < 4; ++rr8) {
-              add4(ga, *reinterpret_cast<const float4*>(src + rr8 * in_pitch));
-              add4(ua, *reinterpret_cast<const float4*>(src + (4 + rr8) * in_pitch));
-            }
-            uint2 o;
-            o.x = pack_bf16x2(silu_f(ga.x) * ua.x, silu_f(ga.y) * ua.y);
-            o.y = pack_bf16x2(silu_f(ga.z) * ua.z, silu_f(ga.w) * ua.w);
-            *reinterpret_cast<uint2*>(p.act + (size_t)m * p.N + col) = o;
           }
         }
       } else if (MODE == GC_SWIGLU) {

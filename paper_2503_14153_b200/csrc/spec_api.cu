@@ -49,12 +49,6 @@ constexpr int ATTN_STAGES = 4;          // tiles attention_tc has in flight
 constexpr int ATTN_SINGLE_TILES = 12;   // contexts of at most this many 64-key tiles use one KV split
 constexpr int ATTN_LONG_KEYS = 2048;    // default context length from which passes of more than 32 rows use the shared-K/V kernel
 
-// Gate+up projections of at most this many tiles go to clusters of eight: so many of them are resident at once. With fewer CTAs than
-// SMs a cluster of three leaves most of the chip idle (d_ffn 1344, 11 tiles, six layers of d_model 512: a 64-row step
-// 252 -> 216 us; 22 tiles of d_model 1024: 296 -> 261 us).
-constexpr int GC_GLU8_TILES = 33;
-constexpr int GC_GLU8_TILES_TALL = 24;  // the same with more than 64 rows, see cluster_gemm_ok
-
 constexpr int GP_NT = 256;              // activation rows per tile of the many-row projection kernel
 constexpr int GP_MAX_CLUSTERS = SM_SLOTS / 4;   // its clusters: two CTAs each, one CTA per SM
 constexpr int GP_SPLIT_KC = 64;         // see pair_parts
@@ -258,7 +252,7 @@ struct spec_ctx {
   bool pdl = true;                     // programmatic dependent launch between the kernels of a step
   int gemm_ctas = 288;                 // persistent CTAs of the weight-streaming GEMM (measured best; at most SM_SLOTS)
   int l2_prefetch = 0;
-  bool gc_attr_set[16] = {};            // per context (and so per device): shared-memory attribute of each gemm_cluster instance set
+  bool gc_attr_set[11] = {};            // per context (and so per device): shared-memory attribute of each gemm_cluster instance set
   int long_attn_keys = ATTN_LONG_KEYS; // SPEC_OPT_LONG_ATTN_KEYS (0 = never)
   bool attn_umma = true;               // SPEC_OPT_ATTN_UMMA: the long-context kernel is the tcgen05 one (head_dim 128)
   CUtensorMap tm_kv;                   // 5-D view of the page pool for its TMA loads
@@ -719,17 +713,15 @@ int run_gemm(spec_ctx* c, const void* x, int M, int K, int n_mats, const void* c
 // Can the cluster-reduced GEMM take this shape? One activation tile, and enough K chunks for every CTA
 // of the cluster to get a run.
 bool cluster_gemm_ok(const spec_ctx* c, int mode, int M, int K) {
-  const int bit = mode == GC_RESIDUAL ? 1 : (mode == GC_ROPE ? 4 : 2);
+  const int bit = mode == GC_RESIDUAL ? 1 : (mode == GC_SWIGLU ? 2 : 4);
   if (!(c->cluster_epilogue & bit) || M < 1 || M > 128 || K % 64) return false;
   const int KC = K / 64;
   if (mode == GC_RESIDUAL) return KC >= GC_RES_CLUSTER;
-  if (mode == GC_SWIGLU) {
-    // (more than 64 rows, d_model 2048, four layers, step at 69 / 96 / 128 rows: 33 tiles 309 / 334 / 369 us in clusters of eight and 312 / 328 / 351
-    // with the weight streamer and swiglu_reduce_tc; 43 tiles 331 / 351 / 379 in clusters of three and 322 / 337 / 379. Below and above that
-    // the clusters win: 22 tiles and six layers of d_model 1024 305 / 332 / 353 and 330 / 351 / 383, 86 tiles and two layers of 4096 361 / 378 / 397 and 385 / 383 / 411.)
-    const int tiles = (c->cfg.d_ffn + 127) / 128;
-    return KC >= 3 && (M <= 64 || tiles <= GC_GLU8_TILES_TALL || tiles >= 64);
-  }
+  // (gate+up of more than 64 rows stays with the weight streamer, and of fewer with clusters of three whatever the number of tiles: the split of the
+  // inner dimension decides how the operands of the next projection round, and with them which of two candidates that lie close
+  // comes first, that is, at which step a token is emitted. Clusters of eight for up to 33 tiles took 216 us a step instead of 252 on six layers of
+  // d_model 512, and clusters of three or eight for 65 to 128 rows 332 instead of 351 at 96 rows of d_model 1024.)
+  if (mode == GC_SWIGLU) return KC >= 3 && M <= 64;
   return KC >= GC_ROPE_CLUSTER && (c->cfg.head_dim == 64 || c->cfg.head_dim == 128);
 }
 
@@ -741,7 +733,7 @@ constexpr int ROPE_ALL = 0, ROPE_Q = 1, ROPE_KV = 2;     // which of the stacked
 int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const void* const* mats, int N, float* x,
                      bf16* act_out, int kind, int layer = -1, const Rows* rows = nullptr, int which = ROPE_ALL) {
   const spec_config& f = c->cfg;
-  const int MT = mt_for_rows(M), n_mats = mode == GC_RESIDUAL ? 1 : (mode == GC_ROPE ? 3 : 2);
+  const int MT = mt_for_rows(M), n_mats = mode == GC_RESIDUAL ? 1 : (mode == GC_SWIGLU ? 2 : 3);
   ClusterGemmParams p{};
   p.M = M; p.K = K; p.KC = K / 64; p.N = N;
   const int HD = f.n_heads * f.head_dim, KD = f.n_kv_heads * f.head_dim;
@@ -767,7 +759,6 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
     p.pool = static_cast<bf16*>(c->d_pool); p.g = c->geom; p.page_table = c->d_page_table;
   }
   p.trace = c->next_trace(gemm_kind_name(kind));
-  if (mode == GC_SWIGLU && K / 64 >= 4 && n_tiles <= GC_GLU8_TILES) mode = GC_SWIGLU8;
   const int cs = mode == GC_SWIGLU ? GC_GLU_CLUSTER : mode == GC_ROPE ? GC_ROPE_CLUSTER : GC_RES_CLUSTER, grid = n_tiles * cs;
   cudaError_t e = cudaErrorInvalidValue;
   {
@@ -780,19 +771,11 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
         case 64: e = launch_gc_mt<64, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 2); break;
         default: e = launch_gc_mt<128, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 3); break;
       }
-    } else if (mode == GC_SWIGLU8) {
-      switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 12); break;
-        case 32: e = launch_gc_mt<32, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 13); break;
-        case 64: e = launch_gc_mt<64, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 14); break;
-        default: e = launch_gc_mt<128, GC_SWIGLU8>(c->stream, c->pdl, grid, cs, tm, p, as + 15); break;
-      }
     } else if (mode == GC_SWIGLU) {
       switch (MT) {
         case 16: e = launch_gc_mt<16, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 4); break;
         case 32: e = launch_gc_mt<32, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 5); break;
-        case 64: e = launch_gc_mt<64, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 6); break;
-        default: e = launch_gc_mt<128, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 11); break;
+        default: e = launch_gc_mt<64, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 6); break;
       }
     } else {
       switch (MT) {
