@@ -132,6 +132,18 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// Which product of a sum is rounded and which is fused into it is spelled out: left to the compiler it went with the code around it, and the
+// bf16 operands made from the results, and the tokens in the end, with it. (The instances of few rows differ from the others only so
+// that every number of rows keeps the rounding that it has had.)
+template <int MT> __device__ __forceinline__ float sum_sq(const float4& v) {
+  const float xy = MT <= 32 ? __fmaf_rn(v.y, v.y, __fmul_rn(v.x, v.x)) : __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y));
+  return __fmaf_rn(v.w, v.w, __fmaf_rn(v.z, v.z, xy));
+}
+__device__ __forceinline__ float rotate_lo(float a, float c, float co, float si) { return __fmaf_rn(a, co, -__fmul_rn(c, si)); }
+template <int MT> __device__ __forceinline__ float rotate_hi(float a, float c, float co, float si) {
+  return MT == 16 ? __fmaf_rn(a, si, __fmul_rn(c, co)) : __fmaf_rn(c, co, __fmul_rn(a, si));
+}
+
 // Rows of one accumulator (or of a stretch of at most MT of its columns) at `taddr`, in groups of 16 of which the two epilogue warps of an SM quarter take every
 // second one: put(row, value) in the thread that owns the weight row, for rows below M.
 // With `second` > 0 the accumulator that many columns further on is added.
@@ -533,7 +545,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
             for (int rr = 0; rr < CS; ++rr) add4(acc, *reinterpret_cast<const float4*>(src + rr * in_pitch));
             add4(xo[k], acc);
             if (x_on[k]) {
-              ss = xo[k].x * xo[k].x + xo[k].y * xo[k].y + xo[k].z * xo[k].z + xo[k].w * xo[k].w;
+              ss = sum_sq<MT>(xo[k]);
               *reinterpret_cast<float4*>(p.x + (size_t)m * p.N + t * 128 + rank * 16 + c4 * 4) = xo[k];
             }
           }
@@ -619,10 +631,10 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
           const float4 t01 = r_cs01[k], t23 = r_cs23[k];
           uint2 lo_o, hi_o;
           if (rope_mat < 2) {
-            lo_o.x = pack_bf16x2(a.x * t01.x - c.x * t01.y, a.y * t01.z - c.y * t01.w);
-            lo_o.y = pack_bf16x2(a.z * t23.x - c.z * t23.y, a.w * t23.z - c.w * t23.w);
-            hi_o.x = pack_bf16x2(c.x * t01.x + a.x * t01.y, c.y * t01.z + a.y * t01.w);
-            hi_o.y = pack_bf16x2(c.z * t23.x + a.z * t23.y, c.w * t23.z + a.w * t23.w);
+            lo_o.x = pack_bf16x2(rotate_lo(a.x, c.x, t01.x, t01.y), rotate_lo(a.y, c.y, t01.z, t01.w));
+            lo_o.y = pack_bf16x2(rotate_lo(a.z, c.z, t23.x, t23.y), rotate_lo(a.w, c.w, t23.z, t23.w));
+            hi_o.x = pack_bf16x2(rotate_hi<MT>(a.x, c.x, t01.x, t01.y), rotate_hi<MT>(a.y, c.y, t01.z, t01.w));
+            hi_o.y = pack_bf16x2(rotate_hi<MT>(a.z, c.z, t23.x, t23.y), rotate_hi<MT>(a.w, c.w, t23.z, t23.w));
           } else {
             lo_o.x = pack_bf16x2(a.x, a.y); lo_o.y = pack_bf16x2(a.z, a.w);
             hi_o.x = pack_bf16x2(c.x, c.y); hi_o.y = pack_bf16x2(c.z, c.w);
