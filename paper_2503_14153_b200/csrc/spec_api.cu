@@ -816,16 +816,14 @@ int linear_simple(spec_ctx* c, const char* name, const T* x, int n_mats, const v
   return SPEC_OK;
 }
 
-// Passes whose (sequence, head, 16-row block) CTAs fit the SMs in one wave use the kernel that needs no merge across CTAs and no
-// length-dependent launch shape; those of a single row block (trees of at most 16 nodes) only up to ATTN_ROWS_ONE_KEYS positions. Both
-// sides, us a step with 16 nodes at 40 / 500 / 1000 / 1900 positions (attention_tc, which splits the keys and merges the splits, first): 7B
-// width and four layers 456 / 482 / 492 / 504 and 452 / 460 / 477 / 503, grouped heads of 64 and six layers 214 / 247 / 269 / 286 and
-// 199 / 207 / 225 / 257, four sequences of them 265 / 301 / 341 / 385 and 255 / 269 / 288 / 319. A CTA walks its whole context, so the
-// lines cross beyond: at about 3500 positions by their slopes; from 2048 on the tcgen05 kernel takes heads of 128 anyway.
-constexpr int ATTN_ROWS_ONE_KEYS = 2048;
-bool attn_rows_mode(const spec_ctx* c, int R, int groups, int keys_hi) {
+// Passes with several 16-row blocks whose (sequence, head, row block) CTAs fit the SMs in one wave
+// use the kernel that needs no merge across CTAs and no length-dependent launch shape. (A single row block, trees of at most 16 nodes,
+// stays with the kernel that splits the keys: a step with 16 nodes, grouped heads of 64 and six layers takes 247 / 269 / 286 us at 500 /
+// 1000 / 1900 positions with it and 207 / 225 / 257 without splits, but the other order of the sums rounds to other operands, and tokens
+// were emitted at other steps.)
+bool attn_rows_mode(const spec_ctx* c, int R, int groups) {
   const int nw = (R + 15) / 16;
-  return c->cfg.n_heads * groups * nw <= SM_SLOTS / 2 && (nw > 1 || keys_hi <= ATTN_ROWS_ONE_KEYS);
+  return nw > 1 && c->cfg.n_heads * groups * nw <= SM_SLOTS / 2;
 }
 
 // Context length from which a pass of R rows goes to the long-context kernels: the option's value, but at most
@@ -834,7 +832,7 @@ bool attn_rows_mode(const spec_ctx* c, int R, int groups, int keys_hi) {
 constexpr int ATTN_WAVES_KEYS = 512;
 int attn_long_threshold(const spec_ctx* c, int R, int groups) {
   const bool umma = c->attn_umma && c->tm_kv_ok && c->cfg.head_dim == 128;
-  if (c->long_attn_keys > 0 && umma && R > 32 && !attn_rows_mode(c, R, groups, 0)) return std::min(c->long_attn_keys, ATTN_WAVES_KEYS);
+  if (c->long_attn_keys > 0 && umma && R > 32 && !attn_rows_mode(c, R, groups)) return std::min(c->long_attn_keys, ATTN_WAVES_KEYS);
   return c->long_attn_keys;
 }
 // Passes of more than 32 rows (any pass with the tcgen05 kernel) over a context that may exceed that length.
@@ -856,7 +854,7 @@ int attn_fetch_ahead(const spec_ctx* c, int R, int groups, int keys_hi) {
     if (c->attn_umma && c->tm_kv_ok && c->cfg.head_dim == 128) return 2 * attn_umma_splits(c, R, groups) * AU_KT;   // two tiles a split
     if (R > 32) return 0;
   }
-  if (attn_rows_mode(c, R, groups, keys_hi)) return ATTN_ROWS_WARPS * ATTN_ROWS_BUFS * ATTN_ROWS_SUB;
+  if (attn_rows_mode(c, R, groups)) return ATTN_ROWS_WARPS * ATTN_ROWS_BUFS * ATTN_ROWS_SUB;
   return keys_hi <= ATTN_SINGLE_TILES * 64 ? ATTN_STAGES * 64 : 0;
 }
 
@@ -940,7 +938,7 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
     }
     return SPEC_OK;
   }
-  if (attn_rows_mode(c, R, B, tiles_hi * 64)) {
+  if (attn_rows_mode(c, R, B)) {
     // few sequences: a CTA per (head, 16 query rows) walks the whole context, whatever its length
     a.nsplit = 1; a.stages = 2; a.split_tiles = 1;
     dim3 grid(H, nw, B);
@@ -1574,11 +1572,11 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
   std::vector<int> n_hi_plan(B), n_lo_plan(B);
   for (int b = 0; b < B; ++b) {
     // three launch shapes: contexts that may reach the long-context kernel's threshold are planned for any length;
-    // below it the CTA-per-16-rows kernel serves every length up to the threshold (a single row block: up to ATTN_SINGLE_TILES tiles, or
-    // ATTN_ROWS_ONE_KEYS positions), and the split kernel is planned for at most ATTN_SINGLE_TILES tiles or for any length
+    // below it the CTA-per-16-rows kernel serves every length up to the threshold, and the split kernel is planned
+    // for at most ATTN_SINGLE_TILES tiles or for any length
     int bound;
     if (attn_long_mode(c, T_, B, c->n_hi[b] + T_)) bound = c->cap;
-    else if (attn_rows_mode(c, T_, B, c->n_hi[b] + T_)) bound = std::min(attn_long_mode(c, T_, B, 1 << 30) ? attn_long_threshold(c, T_, B) / 64 * 64 : c->cap, T_ > 16 ? c->cap : std::min(c->cap, c->n_hi[b] + T_ <= ATTN_SINGLE_TILES * 64 ? ATTN_SINGLE_TILES * 64 : ATTN_ROWS_ONE_KEYS));
+    else if (attn_rows_mode(c, T_, B)) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(attn_long_threshold(c, T_, B) / 64 * 64, c->cap) : c->cap;
     else if (c->n_hi[b] + T_ > ATTN_SINGLE_TILES * 64) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(std::max(attn_long_threshold(c, T_, B) / 64 * 64, ATTN_SINGLE_TILES * 64), c->cap) : c->cap;
     else bound = std::min(ATTN_SINGLE_TILES * 64, c->cap);
     n_hi_plan[b] = bound - T_;

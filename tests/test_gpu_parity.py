@@ -171,8 +171,8 @@ def test_long_context_attention_kernels_batched_ragged(torch, umma, wide):
 
 @pytest.mark.parametrize("T,hd,prompt_len", [(16, 64, 2026), (16, 128, 2026), (1, 64, 2044), (9, 128, 700)])
 def test_single_row_block_across_its_context_limit(torch, T, hd, prompt_len):
-    """Trees of at most 16 nodes use the attention without key splits up to 2048 positions and another kernel beyond: steps on both
-    sides of the limit (which a recorded step must not outlive), and well below it, against the oracle."""
+    """Trees of at most 16 nodes: steps on both sides of 2048 positions, from where heads of 128 go to another kernel (a limit that a
+    recorded step must not outlive), and of 768, up to which the keys are not split, against the oracle."""
     cfg = SMALL_BF16.with_(name="small_bf16_one_block", n_layers=2, n_heads=256 // hd * 2, n_kv_heads=2, head_dim=hd, tree_nodes=T, seed=81 + T)
     rep = _lockstep(cfg, TOL_BF16, 12, prompt_len=prompt_len, check_kv_every=5)
     assert rep.steps > 0

@@ -28,6 +28,7 @@ BASE = get_config("c0", name="peaked", n_layers=6, d_model=1024, n_heads=16, n_k
 
 # name: (tree nodes, prompt lengths of a batch, batches)
 RUNS = {
+    "rows_16": (16, (100,), 60),
     "rows_23": (23, (100,), 60),
     "rows_64": (64, (100,), 60),
     "rows_100": (100, (100,), 60),
