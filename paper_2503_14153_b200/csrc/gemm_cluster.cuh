@@ -65,7 +65,7 @@ struct ClusterGemmParams {
   int* clear;
   // GC_ROPE: tiles [0, tile0[1]) belong to q, [tile0[1], tile0[2]) to k, the rest to v
   int tile0[3];
-  int tile_first;               // first tile of the launch (a prompt's last layer takes k and v, or q, alone)
+  int tile_first;               // first tile of the launch (a prompt's last layer may take k and v alone)
   int H;                        // query heads
   int layer;
   Rows rows;

@@ -62,6 +62,7 @@ struct PairGemmParams {
   int n_mats;
   int mat_tile0[GS_MAX_MATS + 1];           // first 128-row weight tile of each stacked matrix
   int n_tiles, w_pairs, m_tiles;            // weight tiles (all matrices), pairs of them, activation tiles of NT rows
+  int plan_tiles;                           // host: tiles of the launch whose sharing (parts) this one follows, 0: its own
   int parts;                                // clusters that share a tile's K chunks (1: tiles are whole)
   float* part;                              // parts > 1: [tile][part][CTA of the pair][NT][128] float32
   unsigned int* arrive;                     // parts > 1: [tile][CTA of the pair], zero between launches
@@ -75,6 +76,7 @@ struct PairGemmParams {
   bf16* act;                                // GP_SWIGLU: [M][n_cols]
   // GP_ROPE
   int kind0;                                // what the first matrix is: 0 q, 1 k (a prompt's last layer projects k and v alone)
+  int q_chunk;                              // > 0: row m's query goes to row m * q_chunk + position % q_chunk of q (the last rows of prompts)
   int H, layer;
   Rows rows;
   const float2* cs;                         // [position][head_dim / 2] (cos, sin)
@@ -575,7 +577,8 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
                 const bf16 lo = __float2bfloat16_rn(__fmaf_rn(a, t[j].x, -__fmul_rn(c, t[j].y)));
                 const bf16 hi = __float2bfloat16_rn(__fmaf_rn(c, t[j].x, __fmul_rn(a, t[j].y)));
                 if (kind == 0) {
-                  bf16* dst = p.q + (size_t)(m0 + jb + j) * p.H * D + head * D + di;
+                  const int m = m0 + jb + j;
+                  bf16* dst = p.q + (size_t)(p.q_chunk ? m * p.q_chunk + v.pos % p.q_chunk : m) * p.H * D + head * D + di;
                   dst[0] = lo;
                   dst[half] = hi;
                 } else {

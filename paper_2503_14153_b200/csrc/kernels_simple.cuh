@@ -122,6 +122,19 @@ gather_prompt_ends(const int* __restrict__ end_row, const int* __restrict__ end_
   if (threadIdx.x == 0) n_seq[g] = end_pos[g] + 1;
 }
 
+// Their attention outputs: row end_pos[g] % R of chunk g to row g.
+__global__ void __launch_bounds__(256)
+gather_attention_ends(const int* __restrict__ end_pos, const bf16* __restrict__ attn, bf16* __restrict__ attn_end, int R, int HD, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  const int g = blockIdx.x;
+  const size_t m = (size_t)g * R + end_pos[g] % R;
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  for (int c = threadIdx.x; c < (HD >> 3); c += blockDim.x)
+    reinterpret_cast<uint4*>(attn_end + (size_t)g * HD)[c] = reinterpret_cast<const uint4*>(attn + m * HD)[c];
+}
+
 // Before prompts are processed: zeros in every cache slot that they do not fill, from the page of a sequence's first free slot on
 // (attention reads whole tiles of keys; what lies past a sequence's end has weight zero but must be finite). A sequence's pages
 // that its prompt fills are left alone: clearing the whole pool took 45 us for a 2048-token prompt and 8 layers of the 7B shape.

@@ -594,6 +594,12 @@ int pair_parts(int tiles, int KC, int clusters) {
   return std::min(clusters / tiles, KC >= 2 * GP_SPLIT_KC ? 8 : 4);
 }
 
+// Pairs of weight tiles of the stacked query, key and value projections.
+int qkv_pairs(const spec_config& f) {
+  const int HD = f.n_heads * f.head_dim, KD = f.n_kv_heads * f.head_dim;
+  return ((HD + 127) / 128 + 2 * ((KD + 127) / 128) + 1) / 2;
+}
+
 template <int MODE>
 cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemmParams p, float* part, unsigned int* arrive,
                       int max_clusters = GP_MAX_CLUSTERS) {
@@ -608,7 +614,7 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemm
   }
   const int clusters = std::min(GP_MAX_CLUSTERS, max_clusters);
   const int tiles = p.w_pairs * p.m_tiles;
-  p.parts = MODE != GP_PLAIN && part ? pair_parts(tiles, p.KC, clusters) : 1;
+  p.parts = MODE != GP_PLAIN && part ? pair_parts(p.plan_tiles ? p.plan_tiles : tiles, p.KC, clusters) : 1;
   p.part = part; p.arrive = arrive;
   const int grid = 2 * (p.parts > 1 ? tiles * p.parts : std::min(tiles, clusters));
   auto kernel = gemm_pair<MODE, GP_NT, false>;
@@ -725,13 +731,11 @@ bool cluster_gemm_ok(const spec_ctx* c, int mode, int M, int K) {
   return KC >= GC_ROPE_CLUSTER && (c->cfg.head_dim == 64 || c->cfg.head_dim == 128);
 }
 
-constexpr int ROPE_ALL = 0, ROPE_Q = 1, ROPE_KV = 2;     // which of the stacked projections a GC_ROPE launch takes
-
 // x[M,N] += in[M,K] * W^T (GC_RESIDUAL, mats[0] = W), act_out[M,N] = bf16(SiLU(in W_g^T) * in W_u^T)
 // (GC_SWIGLU, mats = gate, up) or q / cache rows of layer `layer` = RoPE(in [W_q; W_k; W_v]^T) (GC_ROPE, mats =
-// q, k, v; rows = the pass's row bookkeeping), finished inside the kernel. Caller checked cluster_gemm_ok.
+// q, k, v; rows = the pass's row bookkeeping; kv_alone: without q), finished inside the kernel. Caller checked cluster_gemm_ok.
 int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const void* const* mats, int N, float* x,
-                     bf16* act_out, int kind, int layer = -1, const Rows* rows = nullptr, int which = ROPE_ALL) {
+                     bf16* act_out, int kind, int layer = -1, const Rows* rows = nullptr, bool kv_alone = false) {
   const spec_config& f = c->cfg;
   const int MT = mt_for_rows(M), n_mats = mode == GC_RESIDUAL ? 1 : (mode == GC_SWIGLU ? 2 : 3);
   ClusterGemmParams p{};
@@ -753,8 +757,8 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
   if (mode == GC_ROPE) {
     const int tq = (HD + 127) / 128, tk = (KD + 127) / 128;
     p.tile0[0] = 0; p.tile0[1] = tq; p.tile0[2] = tq + tk;
-    p.tile_first = which == ROPE_KV ? tq : 0;
-    n_tiles = which == ROPE_Q ? tq : (which == ROPE_KV ? 2 * tk : tq + 2 * tk);
+    p.tile_first = kv_alone ? tq : 0;
+    n_tiles = (kv_alone ? 0 : tq) + 2 * tk;
     p.H = f.n_heads; p.layer = layer; p.rows = *rows; p.cs = c->d_rope; p.q = static_cast<bf16*>(c->d_q);
     p.pool = static_cast<bf16*>(c->d_pool); p.g = c->geom; p.page_table = c->d_page_table;
   }
@@ -860,10 +864,14 @@ int attn_fetch_ahead(const spec_ctx* c, int R, int groups, int keys_hi) {
 
 // n_hi_pass / n_lo_pass: host bounds of the cached length the pass's rows sit on, per sequence
 // (n_lo_pass may be null: nothing is fetched before the dependency wait).
-// len_now: the lengths as well as the host knows them (what the longest-first order goes by).
-int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pass, const int* n_lo_pass, const int* len_now) {
+// part: the groups of R rows that are computed, where they are not all of the pass's (the kernel and its splits are chosen for the whole
+// pass, so that a row's sums do not depend on which rows are left out).
+// len_now: the computed groups' lengths as well as the host knows them (what the longest-first order goes by).
+int launch_attention_tc(spec_ctx* c, const Rows& pass, int l, const int* n_hi_pass, const int* n_lo_pass, const int* len_now, const Rows* part = nullptr) {
   const spec_config& f = c->cfg;
-  const int H = f.n_heads, D = f.head_dim, R = rows.R, B = rows.B;
+  const int H = f.n_heads, D = f.head_dim, R = pass.R, B = pass.B;
+  const Rows& rows = part ? *part : pass;
+  const int G = rows.B;                                          // groups computed
   AttnTcArgs a{};
   a.q = static_cast<const bf16*>(c->d_q); a.part_o = c->d_part_o; a.part_ml = c->d_part_ml;
   a.pool = static_cast<const bf16*>(c->d_pool); a.g = c->geom; a.page_table = c->d_page_table; a.rows = rows;
@@ -881,15 +889,15 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
     // passes of more than 64 rows (prompt chunks, trees of up to 128 nodes): a CTA takes 128 rows and reads the keys once for
     // them; 64 rows or fewer fill the 128-row MMAs twice, with two halves of the keys
     const bool tall = R > 64;
-    if (B <= ATTN_MAX_SEQS) {
+    if (G <= ATTN_MAX_SEQS) {
       int idx[ATTN_MAX_SEQS];
-      for (int b = 0; b < B; ++b) idx[b] = b;
-      std::stable_sort(idx, idx + B, [&](int x, int y) { return len_now[x] > len_now[y]; });
-      for (int b = 0; b < B; ++b) a.order[b] = (unsigned char)idx[b];
+      for (int b = 0; b < G; ++b) idx[b] = b;
+      std::stable_sort(idx, idx + G, [&](int x, int y) { return len_now[x] > len_now[y]; });
+      for (int b = 0; b < G; ++b) a.order[b] = (unsigned char)idx[b];
     }
     // the key splits of a (sequence, head) are one cluster; without splits a CTA takes one (sequence, head) after another
     a.nsplit = attn_umma_splits(c, R, B);
-    const dim3 grid = a.nsplit > 1 ? dim3(H, a.nsplit, B) : dim3(std::min(H * B, SM_SLOTS / 2), 1, 1);
+    const dim3 grid = a.nsplit > 1 ? dim3(H, a.nsplit, G) : dim3(std::min(H * G, SM_SLOTS / 2), 1, 1);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     static bool set_dev[kAttrDevices] = {};
     bool& set_ = *attr_flag(set_dev);
@@ -925,7 +933,7 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
     const int halves = (R + AS_RB * 16 - 1) / (AS_RB * 16);
     a.nsplit = std::max(1, std::min(c->nsplit_attn, (SM_SLOTS / 2) / (H * B * halves)));
     a.stages = AS_NB; a.split_tiles = AS_SPLIT_SUB;
-    dim3 grid(H, a.nsplit, B * halves);
+    dim3 grid(H, a.nsplit, G * halves);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     static bool set_dev[2][kAttrDevices] = {};
     bool& set_ = *attr_flag(set_dev[D == 128 ? 0 : 1]);
@@ -941,7 +949,7 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
   if (attn_rows_mode(c, R, B)) {
     // few sequences: a CTA per (head, 16 query rows) walks the whole context, whatever its length
     a.nsplit = 1; a.stages = 2; a.split_tiles = 1;
-    dim3 grid(H, nw, B);
+    dim3 grid(H, nw, G);
     ProfScope ps_attn(c, SPEC_PROFILE_ATTENTION);
     if (D == 128) {
       static bool set_dev[kAttrDevices] = {};
@@ -963,7 +971,7 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
   a.nsplit = tiles_hi <= ATTN_SINGLE_TILES ? 1 : slots1;
   a.split_tiles = ATTN_SPLIT_TILES;
   a.stages = ATTN_STAGES;
-  dim3 grid(H, a.nsplit, B);
+  dim3 grid(H, a.nsplit, G);
 #define ATTN_CASE(HDV, NWV, KGV)                                                                         \
   {                                                                                                    \
     size_t sm = attention_tc_smem(HDV, NWV, a.stages);                                                 \
@@ -988,48 +996,70 @@ int launch_attention_tc(spec_ctx* c, const Rows& rows, int l, const int* n_hi_pa
 // Of a prompt-processing pass, the last tokens of prompts that it holds: sequences [seq0, seq0 + count).
 struct PromptEnds {
   int count, seq0;
-  int *row, *pos, *seq, *one;           // device tables by sequence: row within its pass, position, the sequence itself, 1
-  const int* pos_host;
+  // device tables by sequence: row of the last token within its pass, its position, the sequence itself, 1; first position of the
+  // token's chunk and the chunk's rows
+  int *row, *pos, *seq, *one, *start, *cnt;
+  const int* start_host;
   bool* pruned;                         // out: the last layer was computed for these rows alone, their results are in d_h_last / d_hq_last
 };
 
 // The rest of a prompt's last layer once its keys and values are stored: nobody reads the other rows' results, so only the last
-// tokens go on, as a pass of their own with one row a sequence (its own key and value are in the cache; the row sees
-// everything before it and itself). A layer of the 7B shape costs 0.7 ms at 2304 rows and this 0.09: 2048 tokens through 8 layers
-// 7.11 -> 6.39 ms, eight ragged prompts of 128..1024 tokens through 4 layers 7.47 -> 6.02 (with clear_free_pages).
-int finish_prompt_ends(spec_ctx* c, const PromptEnds& e) {
+// tokens go on, through the kernels that the whole pass of M rows would take: their attention with its chunk, the projections
+// with the pass's sharing of the tiles, so that every sum is the whole pass's, bit for bit. On the 7B shape a whole layer takes 0.7 ms at 2304 rows and this
+// 0.25 (the kernels that a pass of so few rows would take by itself, 0.09; but a first token's hidden state that rounds otherwise puts other
+// candidates first).
+int finish_prompt_ends(spec_ctx* c, const Rows& pass, const int* n_hi_pass, const PromptEnds& e) {
   const spec_config& f = c->cfg;
-  const int G = e.count, d = f.d_model, F = f.d_ffn, HD = f.n_heads * f.head_dim, l = f.n_layers - 1;
+  const int G = e.count, d = f.d_model, F = f.d_ffn, HD = f.n_heads * f.head_dim, l = f.n_layers - 1, R = pass.R;
   if (G == 0) return SPEC_OK;
+  const int m_tiles = (pass.B * R + GP_NT - 1) / GP_NT, d_pairs = ((d + 127) / 128 + 1) / 2;
   float* x = c->d_hid;
-  bf16 *u = static_cast<bf16*>(c->d_u), *u_end = static_cast<bf16*>(c->d_hq), *act = static_cast<bf16*>(c->d_act);
-  Rows rows = make_rows(c, 1, true);
-  rows.B = G; rows.seq = e.seq + e.seq0; rows.cnt = e.one;
-  rows.tok = nullptr; rows.pos = rows.slot = rows.n = e.pos + e.seq0;
+  bf16 *u = static_cast<bf16*>(c->d_u), *u_end = static_cast<bf16*>(c->d_hq), *act = static_cast<bf16*>(c->d_act), *attn_end = static_cast<bf16*>(c->d_q);
   KLAUNCH("gather_prompt_ends", gather_prompt_ends, dim3(G), dim3(256), 0, (const int*)(e.row + e.seq0), (const int*)(e.pos + e.seq0), (const float*)c->d_x,
           (const bf16*)u, x, u_end, c->d_n + e.seq0, d);
-  const int n_ss = ((d + 127) / 128) * GC_RES_CLUSTER;
   int r;
   {
-    const void* mats[3] = {c->wq[l], c->wk[l], c->wv[l]};
-    if ((r = run_gemm_cluster(c, GC_ROPE, u_end, G, d, mats, 0, nullptr, nullptr, SPEC_PROFILE_QKV, l, &rows, ROPE_Q))) return r;
+    Rows ends = make_rows(c, 1, true);
+    ends.B = G; ends.seq = e.seq + e.seq0; ends.cnt = e.one;
+    ends.tok = nullptr; ends.pos = ends.slot = ends.n = e.pos + e.seq0;
+    const void* mats[1] = {c->wq[l]};
+    const int rws[1] = {HD};
+    PairGemmParams w{};
+    w.plan_tiles = qkv_pairs(f) * m_tiles;
+    w.H = f.n_heads; w.layer = l; w.rows = ends; w.cs = c->d_rope; w.q = static_cast<bf16*>(c->d_q); w.q_chunk = R;
+    w.pool = static_cast<bf16*>(c->d_pool); w.g = c->geom; w.page_table = c->d_page_table;
+    if ((r = run_gemm_pair(c, GP_ROPE, u_end, G, d, 1, mats, rws, &w, SPEC_PROFILE_QKV))) return r;
   }
-  if ((r = launch_attention_tc(c, rows, l, e.pos_host + e.seq0, nullptr, e.pos_host + e.seq0))) return r;
+  {
+    // (of a chunk's other rows the queries are whatever is there: a row's scores and output depend on no other row)
+    Rows chunks = pass;
+    chunks.B = G; chunks.seq = e.seq + e.seq0; chunks.n = e.start + e.seq0; chunks.cnt = e.cnt + e.seq0;
+    if ((r = launch_attention_tc(c, pass, l, n_hi_pass, nullptr, e.start_host + e.seq0, &chunks))) return r;
+    KLAUNCH("gather_attention_ends", gather_attention_ends, dim3(G), dim3(256), 0, (const int*)(e.pos + e.seq0), static_cast<const bf16*>(c->d_attn), attn_end, R, HD);
+  }
   {
     const void* mats[1] = {c->wo[l]};
-    if ((r = run_gemm_cluster(c, GC_RESIDUAL, c->d_attn, G, HD, mats, d, x, nullptr, SPEC_PROFILE_WO))) return r;
+    const int rws[1] = {d};
+    PairGemmParams w{};
+    w.plan_tiles = d_pairs * m_tiles; w.out = x; w.n_cols = d;
+    if ((r = run_gemm_pair(c, GP_RESIDUAL, attn_end, G, HD, 1, mats, rws, &w, SPEC_PROFILE_WO))) return r;
   }
-  KLAUNCH("norm_reduce_tc", norm_scaled_tc, dim3(G, NORM_CLUSTER), dim3(NORM_THREADS), 0, (const float*)x, (const float*)c->d_ss_part, n_ss, c->fn[l], f.rms_eps, u,
-          (float*)nullptr, d);
+  KLAUNCH("norm_reduce_tc", norm_rows_wide, dim3(G), dim3(NORMW_THREADS), 0, x, PartView{}, c->fn[l], f.rms_eps, u, (float*)nullptr, d);
   {
     const void* mats[2] = {c->wg[l], c->wu[l]};
-    if ((r = run_gemm_cluster(c, GC_SWIGLU, u, G, d, mats, F, nullptr, act, SPEC_PROFILE_GATE_UP))) return r;
+    const int rws[2] = {F, F};
+    PairGemmParams w{};
+    w.plan_tiles = (F + 127) / 128 * m_tiles; w.act = act; w.n_cols = F;
+    if ((r = run_gemm_pair(c, GP_SWIGLU, u, G, d, 2, mats, rws, &w, SPEC_PROFILE_GATE_UP))) return r;
   }
   {
     const void* mats[1] = {c->wd[l]};
-    if ((r = run_gemm_cluster(c, GC_RESIDUAL, act, G, F, mats, d, x, nullptr, SPEC_PROFILE_DOWN))) return r;
+    const int rws[1] = {d};
+    PairGemmParams w{};
+    w.plan_tiles = d_pairs * m_tiles; w.out = x; w.n_cols = d;
+    if ((r = run_gemm_pair(c, GP_RESIDUAL, act, G, F, 1, mats, rws, &w, SPEC_PROFILE_DOWN))) return r;
   }
-  KLAUNCH("norm_reduce_tc", norm_scaled_tc, dim3(G, NORM_CLUSTER), dim3(NORM_THREADS), 0, (const float*)x, (const float*)c->d_ss_part, n_ss, c->final_norm, f.rms_eps,
+  KLAUNCH("norm_reduce_tc", norm_rows_wide, dim3(G), dim3(NORMW_THREADS), 0, x, PartView{}, c->final_norm, f.rms_eps,
           static_cast<bf16*>(c->d_hq_last) + (size_t)e.seq0 * d, c->d_h_last + (size_t)e.seq0 * d, d);
   return SPEC_OK;
 }
@@ -1041,8 +1071,7 @@ bool prompt_ends_alone(const spec_ctx* c, int M, int G) {
   const spec_config& f = c->cfg;
   const int d = f.d_model, HD = f.n_heads * f.head_dim;
   if (G == 0) return pair_gemm_ok(c, M, d) || cluster_gemm_ok(c, GC_ROPE, M, d);
-  return pair_gemm_ok(c, M, d) && cluster_gemm_ok(c, GC_ROPE, G, d) && cluster_gemm_ok(c, GC_RESIDUAL, G, HD) && cluster_gemm_ok(c, GC_SWIGLU, G, d) &&
-         cluster_gemm_ok(c, GC_RESIDUAL, G, f.d_ffn);
+  return pair_gemm_ok(c, M, d) && pair_gemm_ok(c, M, HD) && pair_gemm_ok(c, M, f.d_ffn);
 }
 
 // One pass of the base model over M = groups * R rows whose tokens/positions/slots are prepared and
@@ -1077,13 +1106,13 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
       const bool kv_alone = ends && l == f.n_layers - 1 && prompt_ends_alone(c, M, ends->count);
       if (pair_gemm_ok(c, M, d)) {
         PairGemmParams w{};
-        w.kind0 = kv_alone;
+        w.kind0 = kv_alone; w.plan_tiles = qkv_pairs(f) * ((M + GP_NT - 1) / GP_NT);
         w.H = H; w.layer = l; w.rows = rows; w.cs = c->d_rope; w.q = static_cast<bf16*>(c->d_q);
         w.pool = static_cast<bf16*>(c->d_pool); w.g = c->geom; w.page_table = c->d_page_table;
         if ((r = run_gemm_pair(c, GP_ROPE, u, M, d, 3 - w.kind0, mats + w.kind0, rws + w.kind0, &w, SPEC_PROFILE_QKV))) return r;
       } else if (cluster_gemm_ok(c, GC_ROPE, M, d)) {
         // the clusters rotate q and k and store q and the cache rows themselves
-        if ((r = run_gemm_cluster(c, GC_ROPE, u, M, d, mats, 0, nullptr, nullptr, SPEC_PROFILE_QKV, l, &rows, kv_alone ? ROPE_KV : ROPE_ALL))) return r;
+        if ((r = run_gemm_cluster(c, GC_ROPE, u, M, d, mats, 0, nullptr, nullptr, SPEC_PROFILE_QKV, l, &rows, kv_alone))) return r;
       } else {
         PartView vq{};
         if ((r = run_gemm(c, u, M, d, 3, mats, rws, SPEC_PROFILE_QKV, &vq))) return r;
@@ -1093,7 +1122,7 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
     }
     if (ends && l == f.n_layers - 1 && prompt_ends_alone(c, M, ends->count)) {
       *ends->pruned = true;
-      return finish_prompt_ends(c, *ends);
+      return finish_prompt_ends(c, rows, n_hi_pass, *ends);
     }
     if ((r = launch_attention_tc(c, rows, l, n_hi_pass, n_lo_pass, len_now))) return r;
     PartView vo{};
@@ -1421,17 +1450,19 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   CUDA_OK(cudaMemcpyAsync(c->d_chunk_seq, cseq.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_OK(cudaMemcpyAsync(c->d_chunk_pos, cpos.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   // the prompts' last rows, by sequence (the edge flags of the acceptance step are not in use while prompts are processed)
-  std::vector<int> ends(4 * (size_t)batch);
+  static_assert(PREFILL_ROWS >= 6, "a place of the edge flags a table entry");
+  std::vector<int> ends(6 * (size_t)batch);
   PromptEnds pe{};
   bool pruned = false;
-  pe.row = c->d_edge; pe.pos = pe.row + batch; pe.seq = pe.pos + batch; pe.one = pe.seq + batch;
-  pe.pos_host = ends.data() + batch; pe.pruned = &pruned;
+  pe.row = c->d_edge; pe.pos = pe.row + batch; pe.seq = pe.pos + batch; pe.one = pe.seq + batch; pe.start = pe.one + batch; pe.cnt = pe.start + batch;
+  pe.start_host = ends.data() + 4 * (size_t)batch; pe.pruned = &pruned;
   for (int pass = 0, ch = 0; pass < passes; ++pass) {
     const int g = (chunks - ch + passes - pass - 1) / (passes - pass);
     for (int v = ch; v < ch + g; ++v) {
       const int b = cseq[v], last = off[b + 1] - off[b] - 1;
       if (last >= cpos[v] + R) continue;
-      ends[b] = (v - ch) * R + last - cpos[v]; ends[batch + b] = last; ends[2 * (size_t)batch + b] = b; ends[3 * (size_t)batch + b] = 1;
+      const int entry[6] = {(v - ch) * R + last - cpos[v], last, b, 1, cpos[v], last - cpos[v] + 1};
+      for (int k = 0; k < 6; ++k) ends[(size_t)k * batch + b] = entry[k];
     }
     ch += g;
   }

@@ -1,5 +1,6 @@
 """Passes of more than 128 rows against the oracle: the two-SM projection kernel and its epilogues at the edges of
 their tiles."""
+import numpy as np
 import pytest
 
 from synthetic import draw_prompt, draw_weights, get_config
@@ -207,6 +208,40 @@ def test_last_layer_of_a_prompt_for_its_last_rows(torch, lens, layers, hd, batch
         k0, v0 = gpu.read_kv(0, layers - 1, len(prompts[0]) + 30, 2)
         assert not k0.any() and not v0.any()          # nothing was written there since the prompts were processed
     gpu.close()
+
+
+@pytest.mark.parametrize("lens,hd,kv,d,ffn", [
+    ([300], 128, 4, 512, 1344),                      # one pass, shared K/V attention by key splits
+    ([300], 64, 2, 512, 4160),                       # the down projection's tiles are shared between clusters
+    ([129, 256, 1, 700, 128], 64, 8, 512, 1344),     # ragged: chunks of one row, whole chunks, a lone token
+    ([1600, 40], 128, 1, 512, 1344),                 # longer than 512 positions
+    ([200, 333, 520, 77, 900, 64], 128, 8, 1024, 1344),
+    ([2400, 7], 128, 4, 512, 1344),                  # two passes, the first of which ends no prompt
+    ([256, 129], 128, 32, 4096, 1344),               # query, key and value tiles shared or not by how many there are in all
+    ([250] * 140, 64, 2, 512, 704),                  # more last rows than an activation tile's half, in several passes
+])
+def test_last_rows_as_in_the_whole_layer(torch, lens, hd, kv, d, ffn):
+    """The last layer goes on with the prompts' last rows alone, with the sums of the whole layer bit for bit: with a layer behind it
+    that adds nothing (output and down projections of zeros) it is computed for all rows. Hidden states, first tokens, keys and values."""
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    heads = d // hd
+    two = BASE.with_(n_layers=2, d_model=d, n_heads=heads, n_kv_heads=kv, head_dim=hd, d_ffn=ffn, vocab=1000, tree_nodes=4, seed=170 + len(lens) + ffn)
+    w = draw_weights(two)
+    w["layers.1.wo"][:] = 0
+    w["layers.1.w_down"][:] = 0
+    prompts = [draw_prompt(two.with_(seed=180 + i), n) for i, n in enumerate(lens)]
+    got = []
+    for cfg in (two.with_(n_layers=1), two):
+        dec = SpecDecoder(cfg, upload_weights(cfg, {k: v for k, v in w.items() if cfg.n_layers == 2 or not k.startswith("layers.1.")}),
+                          build_tree(cfg.topk, 4), max(lens) + 20, max_batch=len(lens))
+        dec.prefill(prompts)
+        last = len(lens) - 1
+        got.append([dec.debug(B.DBG_H_LAST).copy(), dec.debug(B.DBG_NEXT_ROOT).copy(), dec.debug(B.DBG_SEQLEN).copy(),
+                    *dec.read_kv(0, 0, 0, lens[0]), *dec.read_kv(last, 0, 0, lens[last])])
+        dec.close()
+    for one, whole in zip(*got):
+        assert np.array_equal(one, whole), int((one != whole).sum())
 
 
 @pytest.mark.parametrize("T,heads,kv,batch", [(48, 16, 4, 12), (64, 32, 32, 5), (80, 16, 16, 11), (128, 32, 8, 6)])

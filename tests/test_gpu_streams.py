@@ -32,6 +32,7 @@ RUNS = {
     "rows_23": (23, (100,), 60),
     "rows_64": (64, (100,), 60),
     "rows_100": (100, (100,), 60),
+    "batch_3": (23, (37, 224, 411), 40),
 }
 STEPS = 16
 
