@@ -479,9 +479,10 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
       // the group's last tile must be through the tensor cores before its accumulator is read
       const int t_last = nt - 1 - ((T0 + nt - 1 - grp) & 1);   // (negative: the group has none)
       if (ok && t_last >= 0 && !mbar_wait(&o_done[grp], ((T0 + t_last) >> 1) & 1, a.status, 58)) ok = false;
-      // ---- the streams of a query row are merged: the two groups' (each thread reads both accumulators of its tensor-memory lane, group
-      // g half of the dims), with 64 rows also the two key halves', which sit in lanes 64 apart, through the diagonal blocks of the P
-      // operands (the others stay zero) ----
+      // ---- the streams of a query row are merged: the two groups' (each thread reads both accumulators of its tensor-memory lane), with
+      // 64 rows also the two key halves', which sit in lanes 64 apart, through the diagonal blocks of the P operands (the others stay
+      // zero). The order of the sums is that of the tiles: the group of the item's first tile before the other group, in each the low keys
+      // before the high ones, whichever group that is and wherever in the CTA's row of items the item stands ----
       // (opaque: the addresses made from them would otherwise be kept in registers through the tiles' loop)
       const int z = item[0], h = item[1], cnt = item[3];       // (read again: registers)
       int mrow_ = mrow, qrow_ = qrow;
@@ -491,44 +492,39 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
       tc_fence_before();
       if (!softmax_and(ok)) break;                             // both groups' sums are there and their accumulators complete
       tc_fence_after();
-      float2 st[4];
+      const int kh_ = ROWS == 64 ? mrow_ >> 6 : 0, first = T0 & 1;                                // group of the item's first tile
+      constexpr int STREAMS = ROWS == 64 ? 4 : 2;
+      float2 st[STREAMS];
 #pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        st[g] = ml(g)[mrow_];
-        st[2 + g] = ROWS == 64 ? ml(g)[mrow_ ^ 64] : make_float2(-INFINITY, 0.f);
+      for (int k = 0; k < 2; ++k) {
+        const float2 own = ml(first ^ k)[mrow_];
+        if (ROWS == 64) {
+          const float2 other = ml(first ^ k)[mrow_ ^ 64];
+          st[2 * k] = kh_ ? other : own;
+          st[STREAMS == 4 ? 2 * k + 1 : 0] = kh_ ? own : other;
+        } else {
+          st[k] = own;
+        }
       }
-      const float mm = fmaxf(fmaxf(st[0].x, st[1].x), fmaxf(st[2].x, st[3].x)), base = mm == -INFINITY ? 0.f : mm;
-      const float w0 = exp2f(st[0].x - base), w1 = exp2f(st[1].x - base);
-      // (the same order of the sum in both halves of a row: low keys first)
-      const float own = w0 * st[0].y + w1 * st[1].y;
-      const float other = ROWS == 64 ? exp2f(st[2].x - base) * st[2].y + exp2f(st[3].x - base) * st[3].y : 0.f;
-      const float L = kh ? other + own : own + other;
-      const bool has0 = nt >= 2 || (nt == 1 && !(T0 & 1)), has1 = nt >= 2 || (nt == 1 && (T0 & 1));   // (a group without a tile has no accumulator)
+      float mm = st[0].x;
+#pragma unroll
+      for (int k = 1; k < STREAMS; ++k) mm = fmaxf(mm, st[k].x);
+      const float base = mm == -INFINITY ? 0.f : mm;
+      float wt[STREAMS], L = 0.f;
+#pragma unroll
+      for (int k = 0; k < STREAMS; ++k) { wt[k] = exp2f(st[k].x - base); L = __fmaf_rn(wt[k], st[k].y, L); }
       // (16 dims at a time, and nothing spilled: with all of the SM's shared memory in use there is hardly any L1 to spill to)
-      auto dims16 = [&](int d, float (&v)[16]) {               // dims [d, +16) of this lane's two streams
-        uint32_t r[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = 0.f;
-        if (has0) {
-          tmem_ld16(tmem + lane_base + 256u + (uint32_t)d, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = w0 * __uint_as_float(r[j]);
-        }
-        if (has1) {
-          tmem_ld16(tmem + lane_base + 384u + (uint32_t)d, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] += w1 * __uint_as_float(r[j]);
-        }
+      auto raw16 = [&](int k, int d, uint32_t (&r)[16]) {      // dims [d, +16) of this lane in the k-th group's accumulator
+        tmem_ld16(tmem + lane_base + 256u + (uint32_t)((first ^ k) * 128 + d), r);
+        tmem_ld_wait();
       };
-      const float inv = 1.f / L;
       auto emit16 = [&](int d, const float (&v)[16]) {         // ... to the output, or to the cluster's exchange
         if (ncl > 1) {
 #pragma unroll
           for (int j = 0; j < 16; j += 4)
             *reinterpret_cast<float4*>(ex + (size_t)qrow_ * AU_EXP + d + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
         } else if (qrow_ < cnt) {
+          const float inv = 1.f / L;
           uint4* dst = reinterpret_cast<uint4*>(a.out + ((size_t)z * R + qrow_) * H * HD + h * HD + d);
 #pragma unroll
           for (int j = 0; j < 2; ++j)
@@ -536,35 +532,58 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
                                 pack_bf16(v[8 * j + 4] * inv, v[8 * j + 5] * inv), pack_bf16(v[8 * j + 6] * inv, v[8 * j + 7] * inv));
         }
       };
-      float v[16];
       if constexpr (ROWS == 128) {
 #pragma unroll 1
         for (int d = grp * 64; d < grp * 64 + 64; d += 16) {
-          dims16(d, v);
+          float v[16] = {};
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            if (nt <= k) break;                                // (a group without a tile has no accumulator)
+            uint32_t r[16];
+            raw16(k, d, r);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = __fmaf_rn(wt[k], __uint_as_float(r[j]), v[j]);
+          }
           emit16(d, v);
         }
       } else {
-        // the thread of key half kh finishes dims [32 kh, +32) of the group's 64 and hands the other 32 over
+        // the thread of key half kh finishes dims [32 kh_, +32) of the group's 64 and hands over what it has of the other 32, 16 at a time
         softmax_bar();                                         // (the sums have been read: they lie in two of the blocks)
         auto at = [&](int half, int c) {                       // 16-byte chunk c of this row in the block for the threads of `half`
           return reinterpret_cast<float4*>(p_s + grp * 32768 + half * (16384 + 8192) + qrow_ * 128 + ((c ^ (qrow_ & 7)) << 4));
         };
+        auto rows_bar = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(3 + grp * 2 + ((mrow_ >> 5) & 1)) : "memory"); };   // the two warps of these rows and this group
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
-          dims16(grp * 64 + (kh ^ 1) * 32 + i * 16, v);
+          if (i) rows_bar();                                   // the first 16 have been read
 #pragma unroll
-          for (int j = 0; j < 4; ++j) *at(kh ^ 1, i * 4 + j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-        }
-        softmax_bar();
-#pragma unroll 1
-        for (int i = 0; i < 2; ++i) {
-          dims16(grp * 64 + kh * 32 + i * 16, v);
+          for (int k = 0; k < 2; ++k) {
+            if (nt <= k) break;                                // (a group without a tile has no accumulator)
+            uint32_t r[16];
+            raw16(k, grp * 64 + (kh_ ^ 1) * 32 + i * 16, r);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float4 o = *at(kh, i * 4 + j);
-            v[4 * j] += o.x; v[4 * j + 1] += o.y; v[4 * j + 2] += o.z; v[4 * j + 3] += o.w;
+            for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(at(kh_ ^ 1, k * 4 + j)) = make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
           }
-          emit16(grp * 64 + kh * 32 + i * 16, v);
+          rows_bar();
+          float v[16] = {};
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            if (nt <= k) break;
+            uint32_t r[16];
+            raw16(k, grp * 64 + kh_ * 32 + i * 16, r);
+            const float w_lo = wt[(2 * k) % STREAMS], w_hi = wt[(2 * k + 1) % STREAMS];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float4 o4 = *at(kh_, k * 4 + j);
+              const float o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+              for (int i4 = 0; i4 < 4; ++i4) {
+                const float own = __uint_as_float(r[4 * j + i4]);
+                v[4 * j + i4] = __fmaf_rn(w_hi, kh_ ? own : o[i4], __fmaf_rn(w_lo, kh_ ? o[i4] : own, v[4 * j + i4]));
+              }
+            }
+          }
+          emit16(grp * 64 + kh_ * 32 + i * 16, v);
         }
       }
       if (ncl > 1 && grp == 0 && kh == 0) *reinterpret_cast<float2*>(cml + qrow * 2) = make_float2(mm, L);

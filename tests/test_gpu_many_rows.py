@@ -267,3 +267,28 @@ def test_attention_items_one_after_another(torch, T, heads, kv, batch):
     gpu.close()
     for b in oracles:
         assert reps[b].steps == 2
+
+
+@pytest.mark.parametrize("T,prompt", [(64, 300), (33, 200), (128, 200), (80, 500)])
+def test_attention_does_not_depend_on_the_place_in_a_batch(torch, T, prompt):
+    """Twelve times the same prompt, 192 (sequence, head) items on the SMs: a CTA's second item begins with an odd tile here (three or
+    five tiles an item), that is, with the other softmax group. Prompt processing and two steps give every sequence the same bits."""
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = BASE.with_(n_heads=16, n_kv_heads=4, head_dim=128, tree_nodes=T, seed=240 + T)
+    dec = SpecDecoder(cfg, upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, T), prompt + 40, max_batch=12)
+    dec.set_option(B.OPT_LONG_ATTN_KEYS, 1)
+    dec.prefill([draw_prompt(cfg, prompt)] * 12)
+
+    def same(a):
+        return (a == a[:1]).all()
+    assert same(dec.debug(B.DBG_H_LAST))
+    for b in (0, 11):
+        k, v = dec.read_kv(b, 1, 0, prompt)
+        first = (k.copy(), v.copy()) if b == 0 else first
+    assert (first[0] == k).all() and (first[1] == v).all()
+    for _ in range(2):
+        toks, counts = dec.step()
+        assert same(counts) and same(toks[:, :counts[0]])
+        assert same(dec.debug(B.DBG_HIDDEN).reshape(12, T, -1)) and same(dec.debug(B.DBG_H_LAST))
+    dec.close()
