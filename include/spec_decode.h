@@ -255,6 +255,9 @@ int spec_debug_read_kv(spec_ctx *ctx, int32_t seq, int32_t layer, int32_t slot0,
  * spec_last_error names place 99), clears the status word, and the context remains usable. Synchronises. */
 int spec_debug_wait_timeout(spec_ctx *ctx, int32_t limit_us);
 
+/* How often the library has asked for pinned host memory on behalf of the stand-alone operations so far in this process. */
+int spec_debug_pinned_allocations(void);
+
 /* ---- single operations of the verify forward, for unit parity tests and profiling ---- */
 
 /* Pre-tiled weights. The paper has no counterpart: it is a storage layout for this library's GEMM.
@@ -282,7 +285,9 @@ int spec_pack_weight(const void *w, int32_t rows, int32_t cols, void *packed, vo
  * two), which write y themselves; of scratch only the status word is used in these cases. float32 runs the CUDA-core row kernel
  * (ctas and scratch ignored).
  * M <= 2048; for bf16 K % 64 == 0, M % 16 == 0, N >= 128, 1 <= ctas <= 1024.
- * Synchronises in bf16 mode. */
+ * Synchronises in bf16 mode. The status is reported through 4 KB of pinned host memory that the first bf16 call of the process
+ * allocates and all later calls share (the last four floats of scratch still get it); where it cannot be had, or 64 calls are
+ * under way at once, through scratch alone, which takes some 10 us more. */
 size_t spec_op_linear_scratch_floats(int32_t M, int32_t N, int32_t K, int32_t ctas);
 int spec_op_linear(int32_t dtype, const void *x, const void *w, float *y, int32_t M, int32_t N,
                    int32_t K, int32_t ctas, float *scratch, void *cuda_stream);
@@ -313,7 +318,7 @@ int spec_build_labels(const int32_t *tokens, int32_t n_seq, int32_t seq_len, int
  * one array: it still holds the previous call's partial sums (the library clears the status
  * word itself), and two calls whose kernels overlap on the GPU - different streams, or
  * different host threads - race on it. Serialise them.
- * Arguments, limits, results and synchronisation are those of spec_op_linear. */
+ * Arguments, limits, results and synchronisation are those of spec_op_linear, whose pinned memory this entry does not use. */
 #define SPEC_STATIC_SCRATCH_FLOATS (2u << 20)
 int spec_op_linear_static(int32_t dtype, const void *x, const void *w, float *y, int32_t M, int32_t N,
                           int32_t K, int32_t ctas, void *cuda_stream);

@@ -563,12 +563,12 @@ topk_slices_tc(const PartView pv, int V, int row0, int slice, int kmax, float* p
   topk_merge_row(pk_val, pk_idx, (int)gridDim.x, row, K, kmax, root_tok, cand_override, cand, zs);
 }
 
-// y[m][n] = sum of the partial slots (logical columns of a single matrix): the stand-alone linear. clear: four ints set to zero.
+// y[m][n] = sum of the partial slots (logical columns of a single matrix): the stand-alone linear. clear: four ints set to zero, or nullptr.
 __global__ void __launch_bounds__(256)
 part_sum_rows(const PartView pv, float* __restrict__ y, int M, int N, int* __restrict__ clear) {
   pdl_launch_dependents();
   pdl_wait();
-  if (blockIdx.x == 0 && threadIdx.x < 4) clear[threadIdx.x] = 0;
+  if (clear && blockIdx.x == 0 && threadIdx.x < 4) clear[threadIdx.x] = 0;
   const int n4 = (N + 3) >> 2;
   const size_t total = (size_t)M * n4;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {

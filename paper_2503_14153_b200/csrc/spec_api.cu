@@ -13,6 +13,7 @@
 
 #include <algorithm>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -2073,40 +2074,80 @@ int spec_debug_read_kv(spec_ctx* c, int32_t seq, int32_t layer, int32_t slot0, i
 }
 
 namespace {
-// The status word of a call lies in pinned host memory, where the kernels report a wait that ran out: nothing has to be cleared
-// before them and nothing copied after them (a memset and a 16-byte copy to pageable memory took 12 of the call's 53 us at 64 rows of 4096 x
-// 11008). A block a thread, given back when the thread ends; a call returns only after its kernels, so no other uses it.
-struct HostStatus {
-  int* word = nullptr;
-  ~HostStatus() { if (word) cudaFreeHost(word); }
-  int* clean() {
-    if (!word && cudaHostAlloc(reinterpret_cast<void**>(&word), 4 * sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-      cudaGetLastError();
-      word = nullptr;
+// Status words of stand-alone calls in pinned host memory, where the kernels report a wait that ran out: nothing has to be cleared before
+// them and nothing copied after them (a memset and a 16-byte copy to pageable memory took 12 of the call's 53 us at 64 rows of 4096 x
+// 11008). One block a process, made by the first call that asks and kept; a word is taken for a call and given back when the call's kernels
+// are through. Where there is none, the caller's words on the device serve.
+class StatusWords {
+ public:
+  int* take(int** dev) {
+    std::lock_guard<std::mutex> lock(m_);
+    if (!block_) {
+      allocations_++;
+      if (cudaHostAlloc(reinterpret_cast<void**>(&block_), (size_t)WORDS * 64, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) block_ = nullptr;
+      busy_ = 0;
     }
-    if (word) memset(word, 0, 4 * sizeof(int));
-    return word;
+    void* d = nullptr;
+    if (block_ && cudaHostGetDevicePointer(&d, block_, 0) != cudaSuccess) block_ = nullptr;   // (the device has been reset: the block went with it)
+    if (!block_ || busy_ == ~0ull) { cudaGetLastError(); return nullptr; }
+    int i = 0;
+    while ((busy_ >> i) & 1) ++i;
+    busy_ |= 1ull << i;
+    *dev = static_cast<int*>(d) + i * 16;
+    memset(block_ + i * 16, 0, 4 * sizeof(int));
+    return block_ + i * 16;
   }
+  void give(const int* word) {
+    std::lock_guard<std::mutex> lock(m_);
+    if (block_ && word >= block_ && word < block_ + WORDS * 16) busy_ &= ~(1ull << ((word - block_) / 16));
+  }
+  int allocations() { std::lock_guard<std::mutex> lock(m_); return allocations_; }
+ private:
+  static constexpr int WORDS = 64;                               // bits of busy_; a word has 64 bytes of the block
+  std::mutex m_;
+  int* block_ = nullptr;
+  unsigned long long busy_ = 0;
+  int allocations_ = 0;
 };
-thread_local HostStatus t_status;
-// Waits for the call's kernels and looks at their status word; `words`, which the kernels have cleared, gets it where it is not zero.
-int op_linear_status(const int* status, int* words, cudaStream_t st) {
-  if (cudaStreamSynchronize(st) != cudaSuccess) return SPEC_E_CUDA;
-  if (*static_cast<const volatile int*>(status) == 0) return SPEC_OK;
-  cudaMemcpy(words, status, 4 * sizeof(int), cudaMemcpyHostToDevice);
-  return SPEC_E_TIMEOUT;
-}
+StatusWords& status_words() { static StatusWords* w = new StatusWords; return *w; }   // (never destroyed: a call may come late in the process's exit)
+
+// The status of one call: four ints `words` of the caller's on the device, which get it, and where `pinned` a host word that the kernels report into.
+class OpStatus {
+ public:
+  OpStatus(int* words, bool pinned, cudaStream_t st) : words_(words), st_(st) {
+    if (pinned) host_ = status_words().take(&dev_);
+    if (!host_) { dev_ = words; ok_ = cudaMemsetAsync(words, 0, 4 * sizeof(int), st) == cudaSuccess; }
+  }
+  ~OpStatus() { if (host_) status_words().give(host_); }
+  OpStatus(const OpStatus&) = delete;
+  OpStatus& operator=(const OpStatus&) = delete;
+  bool ok() const { return ok_; }
+  int* report() const { return dev_; }                           // what the kernels report into
+  int* clear() const { return host_ ? words_ : nullptr; }        // what they set to zero
+  int finish() {                                                 // waits for the call's kernels
+    int st[4] = {};
+    if (!host_ && cudaMemcpyAsync(st, words_, sizeof(st), cudaMemcpyDeviceToHost, st_) != cudaSuccess) return SPEC_E_CUDA;
+    if (cudaStreamSynchronize(st_) != cudaSuccess) return SPEC_E_CUDA;
+    if (!host_) return st[0] == 0 ? SPEC_OK : SPEC_E_TIMEOUT;
+    if (*static_cast<const volatile int*>(host_) == 0) return SPEC_OK;
+    if (cudaMemcpyAsync(words_, host_, sizeof(st), cudaMemcpyHostToDevice, st_) != cudaSuccess || cudaStreamSynchronize(st_) != cudaSuccess) return SPEC_E_CUDA;
+    return SPEC_E_TIMEOUT;
+  }
+ private:
+  int *words_, *dev_ = nullptr, *host_ = nullptr;
+  cudaStream_t st_;
+  bool ok_ = true;
+};
 // Shared body of the two stand-alone linear entry points (bf16): scratch holds the partial
-// sums followed by the four-int status word.
+// sums followed by the four-int status word. pinned: the status may come through pinned host memory.
 int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, int ctas, float* scratch,
-                   size_t scratch_floats, cudaStream_t st) {
+                   size_t scratch_floats, bool pinned, cudaStream_t st) {
   GemmPlan g;
   int rws[1] = {N};
   if (!plan_gemm(M, K, 1, rws, ctas, &g)) return SPEC_E_BADARG;
   StreamTmaps tm{};
-  int* const words = reinterpret_cast<int*>(scratch + scratch_floats);
-  int *const host = t_status.clean(), *status = nullptr;
-  if (!host || cudaHostGetDevicePointer(reinterpret_cast<void**>(&status), host, 0) != cudaSuccess) return SPEC_E_CUDA;
+  OpStatus status(reinterpret_cast<int*>(scratch + scratch_floats), pinned, st);
+  if (!status.ok()) return SPEC_E_CUDA;
   if (M > 128 && (long long)g.p.n_tiles * g.p.seg.m_tiles >= 2LL * g.grid) {
     // many rows: whole tiles on pairs of SMs, finished sums straight into y (at M = 1008, N = 11008, K = 4096 the call takes
     // 112 us; weight streaming, which fetches the weights once per 128 rows, took 127 us, adding up its partial sums 34, the call 204)
@@ -2118,9 +2159,9 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     p.n_tiles = g.p.n_tiles; p.w_pairs = (g.p.n_tiles + 1) / 2; p.m_tiles = (M + GP_NT - 1) / GP_NT;
     for (int i = 1; i <= GS_MAX_MATS; ++i) p.mat_tile0[i] = p.n_tiles;
     p.out = y; p.ld = (size_t)N; p.n_cols = N;
-    p.status = status; p.clear = words;
+    p.status = status.report(); p.clear = status.clear();
     if (launch_gp<GP_PLAIN>(st, false, tm, p, nullptr, nullptr, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
-    return op_linear_status(host, words, st);
+    return status.finish();
   }
   if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, g.MT)) return SPEC_E_CUDA;
   const int cs = M <= 128 ? plain_cluster(g.p.n_tiles, K / 64, ctas) : 0;
@@ -2129,20 +2170,20 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     // runs (few tiles and a long inner dimension): the error of a running sum grows with its length.
     ClusterGemmParams p{};
     p.M = M; p.K = K; p.KC = K / 64; p.N = N; p.y = y; p.ldy = (size_t)N;
-    p.status = status; p.clear = words;
+    p.status = status.report(); p.clear = status.clear();
     if (launch_gc_plain(st, false, g.p.n_tiles, cs, tm, p) != cudaSuccess) return SPEC_E_CUDA;
-    return op_linear_status(host, words, st);
+    return status.finish();
   }
   g.p.part = scratch;
   g.p.slot_stride = (size_t)M * g.p.n_tiles * 128;
   g.p.l2_prefetch = 0;
-  g.p.status = status;
+  g.p.status = status.report();
   // (the partial sums are fully overwritten before they are read)
   if (launch_gs(st, false, g, tm) != cudaSuccess) return SPEC_E_CUDA;
   size_t total = (size_t)M * ((N + 3) / 4);
-  if (launch_k(true, part_sum_rows, dim3((unsigned)std::min<size_t>((total + 255) / 256, 4096)), dim3(256), 0, st, plan_view(g), y, M, N, words) != cudaSuccess)
+  if (launch_k(true, part_sum_rows, dim3((unsigned)std::min<size_t>((total + 255) / 256, 4096)), dim3(256), 0, st, plan_view(g), y, M, N, status.clear()) != cudaSuccess)
     return SPEC_E_CUDA;
-  return op_linear_status(host, words, st);
+  return status.finish();
 }
 int op_linear_f32(const void* x, const void* w, float* y, int M, int N, int K, cudaStream_t st) {
   RowLinear<float> rl{};
@@ -2158,6 +2199,8 @@ bool op_linear_args_ok(int32_t dtype, const void* x, const void* w, const float*
   return dtype == 1 && K % 64 == 0 && M % 16 == 0 && N >= 128 && ctas >= 1 && ctas <= 1024;
 }
 }  // namespace
+
+int spec_debug_pinned_allocations(void) { return status_words().allocations(); }
 
 int spec_build_labels(const int32_t* tokens, int32_t n_seq, int32_t seq_len, int32_t num_heads, int32_t frag_token,
                       int32_t pad_token, int32_t ignore_token, int32_t* labels, void* cuda_stream) {
@@ -2205,7 +2248,7 @@ int spec_op_linear(int32_t dtype, const void* x, const void* w, float* y, int32_
     return op_linear_f32(x, w, y, M, N, K, st);
   }
   if (!scratch) return SPEC_E_BADARG;
-  return op_linear_bf16(x, w, y, M, N, K, ctas, scratch, spec_op_linear_scratch_floats(M, N, K, ctas), st);
+  return op_linear_bf16(x, w, y, M, N, K, ctas, scratch, spec_op_linear_scratch_floats(M, N, K, ctas), true, st);
 }
 
 }  // extern "C"
@@ -2248,8 +2291,8 @@ extern "C" int spec_op_linear_static(int32_t dtype, const void* x, const void* w
     scratch = static_cast<float*>(ptr);
     g_static_scratch_addr[dev] = scratch;
   }
-  // the status word sits at the fixed end of the array
-  int r = op_linear_bf16(x, w, y, M, N, K, ctas, scratch, (size_t)SPEC_STATIC_SCRATCH_FLOATS, st);
+  // the status word sits at the fixed end of the array (not in pinned memory: this entry allocates nothing, on any thread)
+  int r = op_linear_bf16(x, w, y, M, N, K, ctas, scratch, (size_t)SPEC_STATIC_SCRATCH_FLOATS, false, st);
   if (r) g_create_error = "spec_op_linear_static: launch or device status failed";
   return r;
 }

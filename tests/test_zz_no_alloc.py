@@ -79,3 +79,62 @@ def test_static_scratch_linear_refuses_oversize(torch):
     with pytest.raises(SpecError) as ei:
         spec_op_linear_static(x, w, y, ctas)
     assert ei.value.code == -3 and "exceeds the built-in scratch" in str(ei.value)
+
+
+def _call(lib, entry, x, w, y, scratch, stream):
+    M, K, N = x.shape[0], x.shape[1], w.shape[0]
+    args = [1, x.data_ptr(), w.data_ptr(), y.data_ptr(), M, N, K, 296]
+    return getattr(lib, entry)(*args, *([scratch.data_ptr()] if entry == "spec_op_linear" else []), stream.cuda_stream)
+
+
+@pytest.mark.parametrize("entry,most", [("spec_op_linear_static", 0), ("spec_op_linear", 1)])
+def test_no_pinned_memory_for_a_thread(entry, most):
+    """In a process of its own, three threads one after another: the entry without allocations makes no pinned memory either, in no
+    thread, and the other entry one block in all, whatever the number of threads that call it."""
+    import subprocess
+    import sys
+    code = f"""
+import sys, threading
+sys.path[:0] = {[p for p in sys.path if p]!r}
+import torch
+import test_zz_no_alloc as T
+from paper_2503_14153_b200 import load_library
+lib = load_library()
+x, w = T._operands(torch, 64, 1000, 704, 15, torch.bfloat16)
+y, scratch, stream = torch.zeros((64, 1000), device="cuda"), torch.empty(int(lib.spec_op_linear_scratch_floats(64, 1000, 704, 296)) + 4, device="cuda"), torch.cuda.Stream()
+torch.cuda.synchronize()
+for _ in range(3):
+    t = threading.Thread(target=lambda: print(T._call(lib, {entry!r}, x, w, y, scratch, stream), lib.spec_debug_pinned_allocations()))
+    t.start(); t.join()
+"""
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert out.stdout.split() == ["0", str(most)] * 3, out.stdout + out.stderr
+
+
+def test_linear_from_many_threads(torch):
+    """Sixteen threads on streams of their own, ten calls each: every call reports its own status and its own result."""
+    import threading
+    from paper_2503_14153_b200 import load_library
+    lib = load_library()
+    ops = [_operands(torch, 16, 500 + 8 * i, 256, 30 + i, torch.bfloat16) for i in range(16)]
+    outs = [torch.zeros((16, w.shape[0]), device="cuda") for _, w in ops]
+    scratch = [torch.empty(int(lib.spec_op_linear_scratch_floats(16, w.shape[0], 256, 296)) + 4, device="cuda") for _, w in ops]
+    streams = [torch.cuda.Stream() for _ in ops]
+    torch.cuda.synchronize()
+    got = [[] for _ in ops]
+
+    def work(i):
+        torch.cuda.set_device(0)
+        for _ in range(10):
+            got[i].append(_call(lib, "spec_op_linear", *ops[i], outs[i], scratch[i], streams[i]))
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(16)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for i, (x, w) in enumerate(ops):
+        want = x.double() @ w.double().T
+        assert got[i] == [0] * 10
+        assert (outs[i] - want).abs().max().item() / want.abs().max().item() <= TOL
+        assert (scratch[i][-4:].view(torch.int32) == 0).all()
