@@ -255,6 +255,11 @@ int spec_debug_read_kv(spec_ctx *ctx, int32_t seq, int32_t layer, int32_t slot0,
  * spec_last_error names place 99), clears the status word, and the context remains usable. Synchronises. */
 int spec_debug_wait_timeout(spec_ctx *ctx, int32_t limit_us);
 
+/* The same self test through the status of a stand-alone operation: the warp reports into the pinned word that spec_op_linear uses
+ * (pinned != 0) or into `words` (DEVICE, four ints) as spec_op_linear_static does; SPEC_E_TIMEOUT, and words holds the status
+ * (code, place 99, detail) in both cases. Synchronises. */
+int spec_debug_op_wait_timeout(int32_t limit_us, int32_t pinned, int32_t *words, void *cuda_stream);
+
 /* How often the library has asked for pinned host memory on behalf of the stand-alone operations so far in this process. */
 int spec_debug_pinned_allocations(void);
 

@@ -2118,7 +2118,11 @@ class OpStatus {
     if (pinned) host_ = status_words().take(&dev_);
     if (!host_) { dev_ = words; ok_ = cudaMemsetAsync(words, 0, 4 * sizeof(int), st) == cudaSuccess; }
   }
-  ~OpStatus() { if (host_) status_words().give(host_); }
+  ~OpStatus() {
+    if (!host_) return;
+    if (!through_) cudaStreamSynchronize(st_);                   // a call that failed behind its first launch: its kernel may still report
+    status_words().give(host_);
+  }
   OpStatus(const OpStatus&) = delete;
   OpStatus& operator=(const OpStatus&) = delete;
   bool ok() const { return ok_; }
@@ -2128,6 +2132,7 @@ class OpStatus {
     int st[4] = {};
     if (!host_ && cudaMemcpyAsync(st, words_, sizeof(st), cudaMemcpyDeviceToHost, st_) != cudaSuccess) return SPEC_E_CUDA;
     if (cudaStreamSynchronize(st_) != cudaSuccess) return SPEC_E_CUDA;
+    through_ = true;
     if (!host_) return st[0] == 0 ? SPEC_OK : SPEC_E_TIMEOUT;
     if (*static_cast<const volatile int*>(host_) == 0) return SPEC_OK;
     if (cudaMemcpyAsync(words_, host_, sizeof(st), cudaMemcpyHostToDevice, st_) != cudaSuccess || cudaStreamSynchronize(st_) != cudaSuccess) return SPEC_E_CUDA;
@@ -2136,7 +2141,7 @@ class OpStatus {
  private:
   int *words_, *dev_ = nullptr, *host_ = nullptr;
   cudaStream_t st_;
-  bool ok_ = true;
+  bool ok_ = true, through_ = false;
 };
 // Shared body of the two stand-alone linear entry points (bf16): scratch holds the partial
 // sums followed by the four-int status word. pinned: the status may come through pinned host memory.
@@ -2199,6 +2204,16 @@ bool op_linear_args_ok(int32_t dtype, const void* x, const void* w, const float*
   return dtype == 1 && K % 64 == 0 && M % 16 == 0 && N >= 128 && ctas >= 1 && ctas <= 1024;
 }
 }  // namespace
+
+int spec_debug_op_wait_timeout(int32_t limit_us, int32_t pinned, int32_t* words, void* cuda_stream) {
+  if (!words || limit_us < 1 || limit_us > 100000) return SPEC_E_BADARG;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  OpStatus status(words, pinned != 0, st);
+  if (!status.ok()) return SPEC_E_CUDA;
+  wait_probe<<<1, 32, 0, st>>>(status.report(), (unsigned long long)limit_us * 1000ull);
+  if (cudaGetLastError() != cudaSuccess) return SPEC_E_CUDA;
+  return status.finish();
+}
 
 int spec_debug_pinned_allocations(void) { return status_words().allocations(); }
 

@@ -138,3 +138,25 @@ def test_linear_from_many_threads(torch):
         assert got[i] == [0] * 10
         assert (outs[i] - want).abs().max().item() / want.abs().max().item() <= TOL
         assert (scratch[i][-4:].view(torch.int32) == 0).all()
+
+
+@pytest.mark.parametrize("pinned", [1, 0])
+def test_wait_that_runs_out_is_reported(torch, pinned):
+    """A kernel's wait that runs out reaches the caller of a stand-alone operation, through the pinned word as through the caller's own:
+    the code, the status in the caller's words, and a clean call after it, from which nothing of it remains."""
+    from paper_2503_14153_b200 import load_library
+    lib = load_library()
+    stream = torch.cuda.Stream()
+    x, w = _operands(torch, 16, 500, 256, 50, torch.bfloat16)
+    y, scratch = torch.zeros((16, 500), device="cuda"), torch.zeros(int(lib.spec_op_linear_scratch_floats(16, 500, 256, 296)) + 4, device="cuda")
+    words = scratch[-4:]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        assert lib.spec_debug_op_wait_timeout(1000, pinned, words.data_ptr(), stream.cuda_stream) == -6      # SPEC_E_TIMEOUT
+        torch.cuda.synchronize()
+        assert words.view(torch.int32)[:2].tolist() == [1, 99]
+        assert _call(lib, "spec_op_linear", x, w, y, scratch, stream) == 0
+        torch.cuda.synchronize()
+        assert words.view(torch.int32)[0].item() == 0
+        assert (y - x.double() @ w.double().T).abs().max().item() <= TOL * y.abs().max().item()
+    assert lib.spec_debug_op_wait_timeout(0, pinned, words.data_ptr(), stream.cuda_stream) == -1
