@@ -141,6 +141,7 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
   const int item0 = ncl == 1 ? (int)blockIdx.x : (int)(blockIdx.z * H + blockIdx.x);
   auto group_of = [&](int item) { const int zb = item / H; return a.rows.B <= ATTN_MAX_SEQS ? (int)a.order[zb] : zb; };
   auto tiles_of = [&](int n, int cnt) -> int {
+    if (cnt <= 0 && n < 0) return -n;                          // (see announce)
     const int total = cnt > 0 ? (n + cnt + AU_KT - 1) / AU_KT : 0;
     return sp < total ? (total - sp + ncl - 1) / ncl : 0;
   };
@@ -199,11 +200,14 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
   if (warp == 8) {
     if (lane == 0) {
       int T = 0, q_items = 0;
+      // (a group that turns out to have no rows although the loads of its first tiles are out, an error of the pass, goes through all
+      // roles with these tiles and no row that sees a key or is stored: the stages stay in step, and the CTA's further items are computed)
       auto announce = [&](int k, int it) -> int4 {
         int4 v = make_int4(-1, 0, 0, 0);
         if (it < n_items) {
           v.x = group_of(it); v.y = it % H;
           v.z = a.rows.n[v.x]; v.w = a.rows.cnt[v.x];
+          if (k == 0 && v.w <= 0 && pre > 0) v.z = -pre;
         }
         items[k % AU_ITEMS] = v;
         mbar_arrive(&item_full[k % AU_ITEMS]);
@@ -216,22 +220,18 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
         if (k) pre = 0;
         int4 next = make_int4(-1, 0, 0, 0);
         // the next item: from the counter, which the last to ask puts back to zero
-        auto ask = [&](bool go_on) {
+        auto ask = [&]() {
           int it = n_items;
           if (ncl == 1)
             do {
               const unsigned int got = atomicAdd(a.arrive, 1u);
               if (got == (unsigned)(n_items - 1)) *a.arrive = 0u;
               it = (int)(gridDim.x + got);
-            } while (it < n_items && (!go_on || a.rows.cnt[group_of(it)] <= 0));     // (a group without rows has nothing to do)
+            } while (it < n_items && a.rows.cnt[group_of(it)] <= 0);     // (a group without rows has nothing to do)
           next = announce(k + 1, it);
         };
         if (nt == 0) {
-          // a group without rows, or a split without tiles; loads asked for above must have landed before the CTA gives up its
-          // shared memory, and with them its stages are out of step: it takes no further item (an error of the pass)
-          if (pre > 0) { mbar_wait(&k_full[0], 0, a.status, 59); mbar_wait(&v_full[0], 0, a.status, 59); }
-          if (pre > 1) mbar_wait(&k_full[1], 0, a.status, 59);
-          ask(pre == 0);
+          ask();                                               // a group without rows, or a split without tiles
         } else {
           if (q_items > 0 && !mbar_wait(q_empty, (q_items - 1) & 1, a.status, 53)) { ok = false; break; }
           ++q_items;
@@ -245,11 +245,11 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
           if (ok && pre < 2 && nt > 1) ok = load_k(T + 1, 1, seq, lh);
           if (ok && pre < 1) ok = load_v(T, 0, seq, lh);
           // (asking takes two trips to L2, in which this thread issues no loads: not before the second tile's are out)
-          if (nt == 1) ask(true);
+          if (nt == 1) ask();
           for (int t = 1; t < nt && ok; ++t) {
             if (t + 1 < nt) ok = load_k(T + t + 1, t + 1, seq, lh);
             if (ok) ok = load_v(T + t, t, seq, lh);
-            if (t == 1) ask(true);
+            if (t == 1) ask();
           }
           T += nt;
         }

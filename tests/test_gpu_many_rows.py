@@ -292,3 +292,34 @@ def test_attention_does_not_depend_on_the_place_in_a_batch(torch, T, prompt):
         assert same(counts) and same(toks[:, :counts[0]])
         assert same(dec.debug(B.DBG_HIDDEN).reshape(12, T, -1)) and same(dec.debug(B.DBG_H_LAST))
     dec.close()
+
+
+@pytest.mark.parametrize("T", [64, 100])
+def test_a_sequence_without_room_leaves_the_others_alone(torch, T):
+    """192 (sequence, head) items, and the longest sequence, with whose items sixteen CTAs begin and whose first tiles they have asked for,
+    turns out to be beyond its cache (its length on the device is set so): the step says so, and the other eleven sequences
+    get the bits of an undisturbed decoder."""
+    from paper_2503_14153_b200 import SpecDecoder, SpecError, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = BASE.with_(n_heads=16, n_kv_heads=4, head_dim=128, tree_nodes=T, seed=250 + T)
+    dw, tree = upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, T)
+    prompts = [draw_prompt(cfg.with_(seed=260 + i), 420 if i == 3 else 200 + 10 * i) for i in range(12)]
+    got = []
+    for disturbed in (False, True):
+        dec = SpecDecoder(cfg, dw, tree, 480, max_batch=12)
+        dec.set_option(B.OPT_LONG_ATTN_KEYS, 1)
+        dec.prefill(prompts)
+        if disturbed:
+            # (the committed lengths lie behind the status word at the start of the workspace)
+            start = (dec.workspace.data_ptr() + 1023) // 1024 * 1024 - dec.workspace.data_ptr()
+            lengths = dec.workspace[start + 16:start + 16 + 48].view(torch.int32)
+            assert lengths.tolist() == [len(p) for p in prompts]
+            lengths[3] = 100000
+            with pytest.raises(SpecError) as ei:
+                dec.step()
+            assert ei.value.code == -4, ei.value                  # SPEC_E_SEQLEN
+        else:
+            dec.step()
+        got.append(dec.debug(B.DBG_HIDDEN).reshape(12, T, -1)[[b for b in range(12) if b != 3]].copy())
+        dec.close()
+    assert np.array_equal(*got)
