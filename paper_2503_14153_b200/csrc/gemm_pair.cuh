@@ -433,7 +433,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);
         const int live = on && p.out ? p.M - m0 : 0;
 #pragma unroll
-        for (int j = 0; j < HC; ++j) {                         // (a running pointer: 128 separate addresses cost 2-3 us a tile)
+        for (int j = 0; j < HC; ++j) {                         // (a running pointer: separate addresses cost 2-3 us a tile)
           if (j < live) *dst = first[j];
           dst += p.ld;
         }

@@ -38,7 +38,8 @@ constexpr int PREFILL_ROWS = 128;   // rows of one chunk of a prompt (a chunk's 
 // Chunks a prompt-processing pass takes at most on the tensor-core path: 18 chunks = 2304 rows = 9 activation tiles, with
 // which the tiles of all four projections of the 7B shape fill the 74 CTA pairs to 95-97% of whole waves (16 chunks: 86-93%).
 // A 2048-token prompt through 8 layers of that shape: 17.6 ms at 128 rows a pass, 7.1 ms in one; eight ragged prompts of
-// 128..1024 tokens through 4 layers: 14.2 ms in passes of one chunk a prompt (mostly padding at the end), 7.5 ms.
+// 128..1024 tokens through 4 layers: 14.2 ms in passes of one chunk a prompt (mostly padding at the end), 7.5 ms (both with every
+// layer computed whole; they take 6.2 and 6.0 ms since the last one goes on with the prompts' last rows).
 constexpr int PREFILL_CHUNKS = 18;
 constexpr int TRACE_CAP = 1024;     // launches of one step the timeline can hold
 constexpr int SM_SLOTS = 296;       // 148 SMs x 2 co-resident GEMM CTAs
@@ -260,7 +261,7 @@ struct spec_ctx {
   bool tm_kv_ok = false;
   bool wide_gemm = true;               // SPEC_OPT_WIDE_GEMM: passes of more than 128 rows use the two-SM kernel (gemm_pair)
   int cluster_epilogue = 7;            // SPEC_OPT_CLUSTER_EPILOGUE: which projections finish their split-K sums inside a cluster
-                                       // (bits: 1 output/down, 2 gate+up, 4 q/k/v; measured on the 7B shape: only gate+up pays)
+                                       // (bits: 1 output/down, 2 gate+up, 4 q/k/v)
   int small_gemm_ctas = 288;           // CTAs of GEMMs with at most 48 weight tiles (Wo, down); 288 since the weights are pre-tiled (192 before)
   std::vector<int> h_parent, h_depth, h_rank;
   std::vector<int> n_hi, n_lo;         // host upper / lower bounds of the committed lengths
@@ -429,8 +430,8 @@ size_t carve(spec_ctx* c, void* base, int chunk_cap, bool share_tiles) {
   c->keep_logits = !c->tc || (f.flags & SPEC_FLAG_KEEP_LOGITS) || f.accept_mode == 1;
   size_t M = c->Mcap;
 
-  // what a step hands to the host lies side by side, so that one copy brings it: status word, committed lengths, counts,
-  // emitted tokens
+  // what a step hands to the host lies side by side, so that its last kernel writes it to host memory in one go: status word,
+  // committed lengths, counts, emitted tokens
   c->d_result = b.take<int>(4 + (size_t)B * (2 + K + 1));
   c->d_status = c->d_result; c->d_n = c->d_result + 4; c->d_count = c->d_n + B; c->d_out_tok = c->d_count + B;
   c->d_trace = b.take<unsigned long long>((size_t)TRACE_CAP * 4);
@@ -861,6 +862,18 @@ int attn_fetch_ahead(const spec_ctx* c, int R, int groups, int keys_hi) {
   }
   if (attn_rows_mode(c, R, groups)) return ATTN_ROWS_WARPS * ATTN_ROWS_BUFS * ATTN_ROWS_SUB;
   return keys_hi <= ATTN_SINGLE_TILES * 64 ? ATTN_STAGES * 64 : 0;
+}
+
+// Number of positions that a step's launches are planned for where a sequence may reach `keys` of them: the most with which
+// launch_attention_tc takes the kernel and the launch shape that it takes for `keys`.
+int attn_plan_bound(const spec_ctx* c, int R, int groups, int keys) {
+  if (attn_long_mode(c, R, groups, keys)) return c->cap;                       // the long-context kernels: any length
+  const bool may_get_long = attn_long_mode(c, R, groups, 1 << 30);
+  const int below_long = may_get_long ? attn_long_threshold(c, R, groups) / 64 * 64 : c->cap;
+  if (attn_rows_mode(c, R, groups)) return std::min(below_long, c->cap);       // a CTA per 16 rows: any length below the threshold
+  const int single = ATTN_SINGLE_TILES * 64;                                   // one split of the keys up to here, several beyond
+  if (keys <= single) return std::min(single, c->cap);
+  return std::min(may_get_long ? std::max(below_long, single) : c->cap, c->cap);
 }
 
 // n_hi_pass / n_lo_pass: host bounds of the cached length the pass's rows sit on, per sequence
@@ -1444,8 +1457,8 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
     for (int p = 0; p < off[b + 1] - off[b]; p += R) { cseq.push_back(b); cpos.push_back(p); }
   const int chunks = (int)cseq.size();
   // A lone prompt of two chunks goes chunk by chunk, through the projections that stream the weights, in the order of sums that the
-  // prompt of one chunk and a lone sequence's verification steps have. On the 7B shape that takes 8.5 ms instead of 7.1, the
-  // weights being read twice. Nothing more is promised: prompts of more chunks, and any prompt processed together with
+  // prompt of one chunk and a lone sequence's verification steps have; the weights are read twice for that (on the 7B shape 8.5 ms instead
+  // of 7.1 when both forms were measured). Nothing more is promised: prompts of more chunks, and any prompt processed together with
   // others, take the many-row projections, whose order of sums is another one (and, up to 512 rows, depends on the rows).
   const int passes = batch == 1 && chunks == 2 ? 2 : (chunks + cap - 1) / cap;
   CUDA_OK(cudaMemcpyAsync(c->d_chunk_seq, cseq.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
@@ -1598,21 +1611,9 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     CUDA_OK(cudaMemcpyAsync(c->d_cand_ov, cand_override, (size_t)B * K * kmax * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     ov = c->d_cand_ov;
   }
-  // the attention launch shape depends only on whether the context fits ATTN_SINGLE_TILES tiles (the
-  // kernel takes the lengths themselves from the device), so the launches are planned for one of two
-  // length bounds and a recorded step serves every length below its bound
+  // (the kernels take the lengths themselves from the device, so a recorded step serves every length below its bounds)
   std::vector<int> n_hi_plan(B), n_lo_plan(B);
-  for (int b = 0; b < B; ++b) {
-    // three launch shapes: contexts that may reach the long-context kernel's threshold are planned for any length;
-    // below it the CTA-per-16-rows kernel serves every length up to the threshold, and the split kernel is planned
-    // for at most ATTN_SINGLE_TILES tiles or for any length
-    int bound;
-    if (attn_long_mode(c, T_, B, c->n_hi[b] + T_)) bound = c->cap;
-    else if (attn_rows_mode(c, T_, B)) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(attn_long_threshold(c, T_, B) / 64 * 64, c->cap) : c->cap;
-    else if (c->n_hi[b] + T_ > ATTN_SINGLE_TILES * 64) bound = attn_long_mode(c, T_, B, 1 << 30) ? std::min(std::max(attn_long_threshold(c, T_, B) / 64 * 64, ATTN_SINGLE_TILES * 64), c->cap) : c->cap;
-    else bound = std::min(ATTN_SINGLE_TILES * 64, c->cap);
-    n_hi_plan[b] = bound - T_;
-  }
+  for (int b = 0; b < B; ++b) n_hi_plan[b] = attn_plan_bound(c, T_, B, c->n_hi[b] + T_) - T_;
   // a recorded step serves every sequence that is at least as long as the part it fetches ahead
   const int ahead = attn_fetch_ahead(c, T_, B, (*std::max_element(n_hi_plan.begin(), n_hi_plan.end()) + T_ + 63) / 64 * 64);
   for (int b = 0; b < B; ++b) n_lo_plan[b] = std::min(c->n_lo[b], ahead);
@@ -2155,7 +2156,7 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
   if (!status.ok()) return SPEC_E_CUDA;
   if (M > 128 && (long long)g.p.n_tiles * g.p.seg.m_tiles >= 2LL * g.grid) {
     // many rows: whole tiles on pairs of SMs, finished sums straight into y (at M = 1008, N = 11008, K = 4096 the call takes
-    // 112 us; weight streaming, which fetches the weights once per 128 rows, took 127 us, adding up its partial sums 34, the call 204)
+    // 106 us; with weight streaming, which fetches the weights once per 128 rows, 127 us, and adds up partial sums, 34, it took 204)
     // With fewer than two tiles a CTA the streaming kernel is as fast (67 us against 65 in one case) and closer to the exact
     // result, since it cuts the inner dimension into several separately rounded sums where this kernel adds two.
     PairGemmParams p{};

@@ -111,7 +111,7 @@ def test_small_bf16_d512_cluster_epilogues(torch):
 @pytest.mark.parametrize("T,hd", [(1, 128), (2, 64), (17, 128), (33, 64), (63, 128), (65, 128), (75, 64), (96, 128), (97, 128), (103, 64), (128, 128)])
 def test_cluster_projections_at_row_counts(torch, T, hd):
     """The exchange between the CTAs of a cluster goes by the pass's rows: one row (the second CTA of q/k/v has none), odd counts, the
-    edges of a 16-row group and of the tiles, more than 64 rows (gate+up in two rounds, the first up to 48 or 64 rows) and more
+    edges of a 16-row group and of the tiles, more than 64 rows (gate+up by the weight streamer, lm_head in two rounds) and more
     than 100 (some rows of the output and down projections sent straight from tensor memory); T = 128 is a prompt chunk's count too."""
     cfg = SMALL_BF16.with_(name="small_bf16_rows", n_layers=2, d_model=512, n_heads=512 // hd, n_kv_heads=512 // hd // 2, head_dim=hd,
                            d_ffn=1344, n_medusa=4, topk=(10, 4, 2, 2), tree_nodes=T, seed=70 + T)
