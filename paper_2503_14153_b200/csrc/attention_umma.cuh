@@ -30,8 +30,8 @@
 // library places page p of sequence b at pool page p * max_batch + b and keeps the pages of a (layer, head)
 // side by side, so a sequence's pages are a strided dimension of the tensor map --; one thread issues all
 // MMAs. Of the four streams of a row (two groups x two key halves) the groups' two sit in the same tensor-memory
-// lane, so each thread adds them straight from both accumulators; the key halves' are swapped through the blocks of
-// the P operands that are free between items (staging all four streams took 135 KB of shared memory, the next
+// lane, so each thread adds them straight from both accumulators; the key halves hand over their raw sums, 16 dims at a
+// time, through the blocks of the P operands that are free between items (staging all four streams took 135 KB of shared memory, the next
 // item's tiles among it, and 2.3 us). The key
 // splits of a (sequence, head) form one thread-block cluster, split s owning tiles s, s + cluster
 // size, ... (which tiles does not depend on the length, so the first two can be asked for before the
