@@ -198,7 +198,8 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
   float* cml = ex + ROWS * AU_EXP;                             // [ROWS] (reference, sum)
 
   if (warp == 8) {
-    if (lane == 0) {
+    pre = __shfl_sync(0xffffffffu, pre, 0);                    // (counted by its first thread above)
+    if (elect_one()) {
       int T = 0, q_items = 0;
       // (a group that turns out to have no rows although the loads of its first tiles are out, an error of the pass, goes through all
       // roles with these tiles and no row that sees a key or is stored: the stages stay in step, and the CTA's further items are computed)
@@ -257,7 +258,7 @@ attention_umma(const __grid_constant__ CUtensorMap tm_kv, const __grid_constant_
       }
     }
   } else if (warp == 9) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- MMA issuer. Order within an item S(0), S(1), then PV(t), S(t + 2) for t = 0, 1, ...: the scores of the next two tiles are
       // always out before a group's probabilities are awaited, and no MMA waits behind a load it does not need (an item's last P V
       // does not wait for the next item's queries; its first scores are computed while the softmax warps merge) ----

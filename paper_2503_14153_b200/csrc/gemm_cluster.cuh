@@ -342,7 +342,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- producer: weights before the dependency wait, activation tiles after it ----
       const uint64_t wpol = l2_policy_evict_first();
       const int n_pre = n_units < STAGES ? n_units : STAGES;
@@ -384,7 +384,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- MMA issuer: one accumulator per run ----
       const uint32_t idesc = make_idesc_bf16(128, MT);
       bool ok = true;

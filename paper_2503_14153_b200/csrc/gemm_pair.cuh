@@ -206,7 +206,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- producer: this CTA's weight rows and its half of the activation rows ----
       struct At { int i, kc, wp, mt; };
       auto at_tile = [&](At& a) {
@@ -257,7 +257,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       // ---- MMA issuer of the pair ----
       const uint32_t idesc = make_idesc_bf16(256, NT);
       bool ok = true;

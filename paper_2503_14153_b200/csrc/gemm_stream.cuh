@@ -136,7 +136,7 @@ gemm_stream(const __grid_constant__ StreamTmaps tm, const StreamGemmParams p) {
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- TMA producer ----
       const int n_units = hi - lo;
       const uint64_t wpol = l2_policy_evict_first();
@@ -185,7 +185,7 @@ gemm_stream(const __grid_constant__ StreamTmaps tm, const StreamGemmParams p) {
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- MMA issuer ----
       const uint32_t idesc = make_idesc_bf16(128, MT);
       int seg_i = 0;
