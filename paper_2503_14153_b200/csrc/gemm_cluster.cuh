@@ -51,6 +51,7 @@ constexpr int GC_RES_CLUSTER = 8, GC_GLU_CLUSTER = 3, GC_ROPE_CLUSTER = 2;
 
 struct ClusterGemmParams {
   int M, K, KC;                 // activation rows (<= MT), inner size, K / 64
+  int stages;                   // of the ring: ClusterCfg<MT>::STAGES to MAX_STAGES (see cluster_stages)
   int N;                        // weight rows of one matrix (output columns)
   const uint8_t* packed[3];     // pre-tiled images (GC_RESIDUAL: [0]; GC_SWIGLU: gate, up; GC_ROPE: q, k, v) or nullptr -> tensor maps a[i]
   float* x;                     // GC_RESIDUAL: [M][N] float32 residual stream, updated in place
@@ -83,10 +84,22 @@ template <int MT> struct ClusterCfg {
   static constexpr int A_BYTES = 128 * BK * 2;
   static constexpr int B_BYTES = MT * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = (MT <= 32) ? 5 : (MT == 64 ? 4 : 3);
+  static constexpr int STAGES = (MT <= 32) ? 5 : (MT == 64 ? 4 : 3);      // two CTAs an SM
   static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
-  static constexpr int SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
+  static constexpr int EXTRA_BYTES = 1024 /*alignment slack*/ + 256 /*barriers*/;
+  static constexpr int MAX_STAGES = (227 * 1024 - EXTRA_BYTES) / STAGE_BYTES < 12 ? (227 * 1024 - EXTRA_BYTES) / STAGE_BYTES : 12;   // one CTA an SM
+  static constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + EXTRA_BYTES; }
 };
+
+// Stages of a launch of `ctas` CTAs with at most `units` K chunks each. A grid of more than one CTA an SM gets the ring of which two fit.
+// A smaller one (the projections of narrow models: at d_model 1024 q/k/v has 24 CTAs of 8 chunks, gate+up 66 of 11) gets a stage for every
+// chunk as far as shared memory goes, so that all of a CTA's weights are under way before the dependency wait and the chain behind it is
+// activation tiles, MMAs and the exchange. Six layers of d_model 1024, 64 rows: gate+up 10.3 -> 8.4 us, down 6.2 -> 4.9, a step 284 -> 263.
+template <int MT> inline int cluster_stages(int ctas, int units) {
+  using Cfg = ClusterCfg<MT>;
+  if (ctas > 148 || units <= Cfg::STAGES) return Cfg::STAGES;
+  return units < Cfg::MAX_STAGES ? units : Cfg::MAX_STAGES;
+}
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -147,9 +160,9 @@ template <int MT> __device__ __forceinline__ float rotate_hi(float a, float c, f
 // Rows of one accumulator (or of a stretch of at most MT of its columns) at `taddr`, in groups of 16 of which the two epilogue warps of an SM quarter take every
 // second one: put(row, value) in the thread that owns the weight row, for rows below M.
 // With `second` > 0 the accumulator that many columns further on is added.
-template <int MT, typename F>
+template <int MT, int MOST = 2, typename F>
 __device__ __forceinline__ void tmem_rows(uint32_t taddr, int hf, int M, F&& put, int second = 0) {
-  constexpr int NG = MT >= 32 ? MT / 32 : 1, U = NG < 2 ? NG : 2;   // (two groups at a time: registers)
+  constexpr int NG = MT >= 32 ? MT / 32 : 1, U = NG < MOST ? NG : MOST;   // (groups at a time: registers)
   if (MT == 16 && hf) return;
 #pragma unroll
   for (int k0 = 0; k0 < NG; k0 += U) {
@@ -193,19 +206,21 @@ template <int MT, int MODE>
 __global__ void __launch_bounds__(GC_THREADS, 2)
 gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) {
   using Cfg = ClusterCfg<MT>;
-  constexpr int STAGES = Cfg::STAGES;
+  const int stages = p.stages, ring_bytes = stages * Cfg::STAGE_BYTES;
+  const int mma_n = (p.M + 15) & ~15;                        // the MMA's N: only rows that are there are fetched
+  const uint32_t stage_tx = Cfg::A_BYTES + mma_n * Cfg::BK * 2;
   constexpr bool PLAIN = MODE == GC_PLAIN;
   const int CS = PLAIN ? (int)cluster_nctarank() : (MODE == GC_RESIDUAL ? GC_RES_CLUSTER : (MODE == GC_SWIGLU ? GC_GLU_CLUSTER : GC_ROPE_CLUSTER));
   constexpr int TMEM_COLS = (MODE == GC_SWIGLU || PLAIN ? 2 : 1) * MT < 32 ? 32 : (MODE == GC_SWIGLU || PLAIN ? 2 : 1) * MT;   // 32 to 256
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* tiles = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + Cfg::RING_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + ring_bytes);
   uint64_t* full = bars;
-  uint64_t* empty = bars + STAGES;
-  uint64_t* acc_full = bars + 2 * STAGES;
-  uint64_t* part_full = bars + 2 * STAGES + 1;               // the other CTAs' parts of this CTA's outputs have landed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
+  uint64_t* empty = bars + stages;
+  uint64_t* acc_full = bars + 2 * stages;
+  uint64_t* part_full = bars + 2 * stages + 1;               // the other CTAs' parts of this CTA's outputs have landed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * stages + 2);
   float* staging = reinterpret_cast<float*>(tiles);          // reuses the ring once every MMA is complete
 
   KTrace kt(p.trace);
@@ -246,7 +261,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   const int rr = ROUNDS == 2 ? (M + 31) / 32 * 16 : M;       // rows of a round (at most RT)
   // GC_RESIDUAL: rows that travel as bulk copies; the ring of MT = 128 has no room for the staged copy of all rows beside the
   // arriving ones when there are more than about 100, and the others are sent straight from tensor memory
-  const int S = MODE == GC_RESIDUAL ? min(M, (Cfg::RING_BYTES - GC_RES_CLUSTER * M * 64) / ((GC_RES_CLUSTER - 1) * 64) - 1) : rr;
+  const int S = MODE == GC_RESIDUAL ? min(M, (ring_bytes - GC_RES_CLUSTER * M * 64) / ((GC_RES_CLUSTER - 1) * 64) - 1) : rr;
   // GC_PLAIN: CTA r finishes the r-th block of rows of a round
   const int rb = PLAIN ? (rr + CS - 1) / CS : 0;
   const int in_pitch = MODE == GC_RESIDUAL ? M * 16 : (rr | 1) * 16;       // floats of a group of 16 columns (odd: banks)
@@ -266,7 +281,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < stages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(acc_full, 1);
     mbar_init(part_full, 1);
     mbar_fence_init();
@@ -345,7 +360,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
     if (elect_one()) {
       // ---- producer: weights before the dependency wait, activation tiles after it ----
       const uint64_t wpol = l2_policy_evict_first();
-      const int n_pre = n_units < STAGES ? n_units : STAGES;
+      const int n_pre = n_units < stages ? n_units : stages;
       auto load_a = [&](uint8_t* dst, int s, int kc, uint64_t* bar) {
         const int mat = seg[s].mat;
         if (p.packed[mat])
@@ -356,7 +371,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
       for (int i = 0; i < n_pre; ++i) {
         int s, kc;
         unit(i, s, kc);
-        mbar_expect_tx(&full[i], Cfg::STAGE_BYTES);
+        mbar_expect_tx(&full[i], stage_tx);
         load_a(tiles + i * Cfg::STAGE_BYTES, s, kc, &full[i]);
       }
       pdl_wait();
@@ -366,35 +381,34 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
         tma_load_2d(tiles + i * Cfg::STAGE_BYTES + Cfg::A_BYTES, &tm.b, kc * Cfg::BK, 0, &full[i]);
       }
       bool ok = true;
-      int issued = n_pre;
+      int issued = n_pre, st = 0;
+      uint32_t ph = 0;                                       // (a ring that is refilled has been filled once)
       for (; issued < n_units; ++issued) {
-        const int st = issued % STAGES;
-        const uint32_t ph = (issued / STAGES) & 1;
-        if (!mbar_wait(&empty[st], ph ^ 1, p.status, 30)) { ok = false; break; }
+        if (!mbar_wait(&empty[st], ph, p.status, 30)) { ok = false; break; }
         int s, kc;
         unit(issued, s, kc);
         uint8_t* a = tiles + st * Cfg::STAGE_BYTES;
-        mbar_expect_tx(&full[st], Cfg::STAGE_BYTES);
+        mbar_expect_tx(&full[st], stage_tx);
         load_a(a, s, kc, &full[st]);
         tma_load_2d(a + Cfg::A_BYTES, &tm.b, kc * Cfg::BK, 0, &full[st]);
+        if (++st == stages) { st = 0; ph ^= 1; }
       }
       if (!ok) {
-        for (int i = issued > STAGES ? issued - STAGES : 0; i < issued; ++i)
-          mbar_wait(&full[i % STAGES], (i / STAGES) & 1, p.status, 33);
+        for (int i = issued > stages ? issued - stages : 0; i < issued; ++i)
+          mbar_wait(&full[i % stages], (i / stages) & 1, p.status, 33);
       }
     }
   } else if (warp == 1) {
     if (elect_one()) {
       // ---- MMA issuer: one accumulator per run ----
-      const uint32_t idesc = make_idesc_bf16(128, MT);
+      const uint32_t idesc = make_idesc_bf16(128, mma_n);
       bool ok = true;
-      int done = 0;
+      int done = 0, st = 0;
+      uint32_t ph = 0;
       for (int s = 0; s < nseg && ok; ++s) {
         const uint32_t d_addr = tmem_base + (uint32_t)(s * MT);
         const int n = seg[s].kc1 - seg[s].kc0;
         for (int v = 0; v < n; ++v, ++done) {
-          const int st = done % STAGES;
-          const uint32_t ph = (done / STAGES) & 1;
           if (!mbar_wait(&full[st], ph, p.status, 31)) { ok = false; break; }
           if (done == 0) trace_mark_min(p.trace, 2);
           tc_fence_after();
@@ -405,6 +419,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
           for (int k = 0; k < Cfg::BK / 16; ++k)
             tc_mma_f16(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (v > 0 || k > 0) ? 1u : 0u);
           tc_commit(&empty[st]);
+          if (++st == stages) { st = 0; ph ^= 1; }
         }
       }
       if (ok) tc_commit(acc_full);         // arrives once every MMA above is complete (and has read its operands)
@@ -471,7 +486,9 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
         float* mine = in + w;                                  // (block `rank` of `in` starts at row rank * rb)
         float* rest = out + w;
         const int own0 = rank * rb, own1 = own0 + rb;
-        tmem_rows<RT>(taddr + (uint32_t)m0, hf, Mr, [&](int m, float v) { *((m >= own0 && m < own1 ? mine : rest) + m * 128) = v; }, nseg > 1 ? MT : 0);
+        // (in two rounds one group at a time: with two the finishing loop's registers were spilled, to L2 with the L1 given to shared
+        // memory, and lm_head of 69 rows, 32016 x 1024, took 22.7 us instead of 17.7)
+        tmem_rows<RT, ROUNDS == 2 ? 1 : 2>(taddr + (uint32_t)m0, hf, Mr, [&](int m, float v) { *((m >= own0 && m < own1 ? mine : rest) + m * 128) = v; }, nseg > 1 ? MT : 0);
       } else {
         // the other CTA's rows to `out`, its own beside the place where the other's part arrives; both [warp][row][32 columns]
         float* mine = in + (size_t)r_rows * 128 + q * r_rows * 32 + lane;

@@ -196,14 +196,15 @@ cudaError_t launch_gs(cudaStream_t st, bool pdl, const GemmPlan& g, const Stream
 }
 
 template <int MT, int MODE>
-cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int grid, int cluster, const StreamTmaps& tm, const ClusterGemmParams& p, bool* attr_set) {
+cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int grid, int cluster, const StreamTmaps& tm, ClusterGemmParams p, bool* attr_set) {
   if (!*attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_cluster<MT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<MT>::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gemm_cluster<MT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<MT>::smem_bytes(ClusterCfg<MT>::MAX_STAGES));
     if (e != cudaSuccess) return e;
     *attr_set = true;
   }
+  p.stages = cluster_stages<MT>(grid, ((MODE == GC_SWIGLU ? 2 : 1) * p.KC + cluster - 1) / cluster);
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GC_THREADS); cfg.dynamicSmemBytes = (size_t)ClusterCfg<MT>::SMEM_BYTES; cfg.stream = st;
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GC_THREADS); cfg.dynamicSmemBytes = (size_t)ClusterCfg<MT>::smem_bytes(p.stages); cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -751,7 +752,7 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
     if (!t) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (weights)");
     tm.a[i] = *t;
   }
-  const CUtensorMap* tb = c->tmap(in, std::max<size_t>(round_up(M, 16), MT), K, MT);
+  const CUtensorMap* tb = c->tmap(in, round_up(M, 16), K, (uint32_t)round_up(M, 16));
   if (!tb) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (activations)");
   tm.b = *tb;
   p.x = x; p.ss_part = mode == GC_RESIDUAL ? c->d_ss_part : nullptr; p.act = act_out; p.status = c->d_status;
@@ -1302,7 +1303,7 @@ int run_lm_head(spec_ctx* c, const void* x, int M, int cluster, float* y, size_t
     if (!t) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (weights)");
     tm.a[0] = *t;
   }
-  const CUtensorMap* tb = c->tmap(x, std::max<size_t>(round_up(M, 16), MT), d, MT);
+  const CUtensorMap* tb = c->tmap(x, round_up(M, 16), d, (uint32_t)round_up(M, 16));
   if (!tb) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (activations)");
   tm.b = *tb;
   p.trace = c->next_trace(gemm_kind_name(SPEC_PROFILE_OFF));
@@ -2169,9 +2170,10 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     if (launch_gp<GP_PLAIN>(st, false, tm, p, nullptr, nullptr, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
     return status.finish();
   }
-  if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, g.MT)) return SPEC_E_CUDA;
   const int cs = M <= 128 ? plain_cluster(g.p.n_tiles, K / 64, ctas) : 0;
-  if (2LL * g.p.n_tiles * cs >= g.grid) {
+  const bool cluster = 2LL * g.p.n_tiles * cs >= g.grid;
+  if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, cluster ? M : g.MT)) return SPEC_E_CUDA;   // (M % 16 == 0)
+  if (cluster) {
     // few rows: the CTAs of a tile finish its sums on the chip. Not where their half runs would be longer than the streaming kernel's
     // runs (few tiles and a long inner dimension): the error of a running sum grows with its length.
     ClusterGemmParams p{};
