@@ -157,43 +157,29 @@ template <int MT> __device__ __forceinline__ float rotate_hi(float a, float c, f
   return MT == 16 ? __fmaf_rn(a, si, __fmul_rn(c, co)) : __fmaf_rn(c, co, __fmul_rn(a, si));
 }
 
-// Rows of one accumulator (or of a stretch of at most MT of its columns) at `taddr`, in groups of 16 of which the two epilogue warps of an SM quarter take every
+// Rows of one accumulator (or of a stretch of its columns) at `taddr`, in groups of 16 of which the two epilogue warps of an SM quarter take every
 // second one: put(row, value) in the thread that owns the weight row, for rows below M.
-// With `second` > 0 the accumulator that many columns further on is added.
-template <int MT, int MOST = 2, typename F>
+// With `second` > 0 the accumulator that many columns further on is added. One group's code for all of them: a kernel runs through
+// this once, and unrolled over the groups, with a pointer chosen for every row, it waited for its instructions: staging q/k/v of 64 rows took
+// 1.3 us and of 69 rows 3.7 (now 0.6 and 0.7), a step of 69 rows on six layers of d_model 1024 333 us (now 312), and the code of the whole
+// epilogue had lm_head's registers spilled.
+template <typename F>
 __device__ __forceinline__ void tmem_rows(uint32_t taddr, int hf, int M, F&& put, int second = 0) {
-  constexpr int NG = MT >= 32 ? MT / 32 : 1, U = NG < MOST ? NG : MOST;   // (groups at a time: registers)
-  if (MT == 16 && hf) return;
-#pragma unroll
-  for (int k0 = 0; k0 < NG; k0 += U) {
-    uint32_t r[U][16];
-#pragma unroll
-    for (int k = 0; k < U; ++k)
-      if ((2 * (k0 + k) + hf) * 16 < M) tmem_ld16(taddr + (2 * (k0 + k) + hf) * 16, r[k]);      // (the same in the whole warp)
+#pragma unroll 1
+  for (int m0 = hf * 16; m0 < M; m0 += 32) {                 // (the same in the whole warp)
+    uint32_t r[16];
+    tmem_ld16(taddr + m0, r);
     tmem_ld_wait();
     if (second) {
-      uint32_t r2[U][16];
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-        if ((2 * (k0 + k) + hf) * 16 < M) tmem_ld16(taddr + second + (2 * (k0 + k) + hf) * 16, r2[k]);
+      uint32_t r2[16];
+      tmem_ld16(taddr + second + m0, r2);
       tmem_ld_wait();
 #pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int j = 0; j < 16; ++j) r[k][j] = __float_as_uint(__uint_as_float(r[k][j]) + __uint_as_float(r2[k][j]));
+      for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
     }
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int m0 = (2 * (k0 + k) + hf) * 16;
-      if (m0 + 16 <= M) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) put(m0 + j, __uint_as_float(r[k][j]));
-      } else if (m0 < M) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (m0 + j < M) put(m0 + j, __uint_as_float(r[k][j]));
-      }
-    }
+    for (int j = 0; j < 16; ++j)
+      if (m0 + j < M) put(m0 + j, __uint_as_float(r[j]));
   }
 }
 
@@ -405,6 +391,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
       bool ok = true;
       int done = 0, st = 0;
       uint32_t ph = 0;
+      const uint64_t adesc0 = make_kmajor_sw128_desc(smem_u32(tiles)), bdesc0 = make_kmajor_sw128_desc(smem_u32(tiles) + Cfg::A_BYTES);
       for (int s = 0; s < nseg && ok; ++s) {
         const uint32_t d_addr = tmem_base + (uint32_t)(s * MT);
         const int n = seg[s].kc1 - seg[s].kc0;
@@ -412,13 +399,11 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
           if (!mbar_wait(&full[st], ph, p.status, 31)) { ok = false; break; }
           if (done == 0) trace_mark_min(p.trace, 2);
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(tiles + st * Cfg::STAGE_BYTES);
-          const uint64_t adesc = make_kmajor_sw128_desc(a_addr);
-          const uint64_t bdesc = make_kmajor_sw128_desc(a_addr + Cfg::A_BYTES);
+          const uint64_t adesc = adesc0 + (uint64_t)(st * (Cfg::STAGE_BYTES >> 4)), bdesc = bdesc0 + (uint64_t)(st * (Cfg::STAGE_BYTES >> 4));
 #pragma unroll
           for (int k = 0; k < Cfg::BK / 16; ++k)
             tc_mma_f16(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (v > 0 || k > 0) ? 1u : 0u);
-          tc_commit(&empty[st]);
+          if (done + stages < n_units) tc_commit(&empty[st]);     // (a stage that is not filled again needs no announcement)
           if (++st == stages) { st = 0; ph ^= 1; }
         }
       }
@@ -472,29 +457,25 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
         const bool own = grp == rank;
         float* dst = (own ? in + rank * in_pitch : out + (grp - (grp > rank)) * out_pitch) + (w & 15);
         const int rows = own ? M : S;
-        tmem_rows<RT>(taddr, hf, M, [&](int m, float v) { if (MT < 128 || m < rows) dst[m * 16] = v; });
+        tmem_rows(taddr, hf, M, [&](int m, float v) { if (MT < 128 || m < rows) dst[m * 16] = v; });
       } else if (MODE == GC_SWIGLU) {
         const bool own = grp >= glu_g0 && grp < glu_g0 + glu_ng;
         for (int s = 0; s < nseg; ++s) {
           const int slot = seg[s].mat == 0 ? rank : rank + 1;  // gate parts of CTA 0 and 1, up parts of CTA 1 and 2
           float* dst = (own ? in + (slot * glu_ng + grp - glu_g0) * in_pitch
                             : out + (s * (8 - glu_ng) + (grp < glu_g0 ? grp : grp - glu_ng)) * out_pitch) + (w & 15);
-          tmem_rows<RT>(taddr + (uint32_t)(s * MT + m0), hf, Mr, [&](int m, float v) { dst[m * 16] = v; });
+          tmem_rows(taddr + (uint32_t)(s * MT + m0), hf, Mr, [&](int m, float v) { dst[m * 16] = v; });
         }
       } else if (PLAIN) {
         // rows of this CTA's block to its place in `in`, all others to `out`; the two halves of the run are added here
-        float* mine = in + w;                                  // (block `rank` of `in` starts at row rank * rb)
-        float* rest = out + w;
-        const int own0 = rank * rb, own1 = own0 + rb;
-        // (in two rounds one group at a time: with two the finishing loop's registers were spilled, to L2 with the L1 given to shared
-        // memory, and lm_head of 69 rows, 32016 x 1024, took 22.7 us instead of 17.7)
-        tmem_rows<RT, ROUNDS == 2 ? 1 : 2>(taddr + (uint32_t)m0, hf, Mr, [&](int m, float v) { *((m >= own0 && m < own1 ? mine : rest) + m * 128) = v; }, nseg > 1 ? MT : 0);
+        const int own0 = rank * rb, to_out = (int)(out - in);  // (block `rank` of `in` starts at row rank * rb)
+        tmem_rows(taddr + (uint32_t)m0, hf, Mr, [&](int m, float v) { in[((unsigned)(m - own0) < (unsigned)rb ? 0 : to_out) + m * 128 + w] = v; }, nseg > 1 ? MT : 0);
       } else {
         // the other CTA's rows to `out`, its own beside the place where the other's part arrives; both [warp][row][32 columns]
-        float* mine = in + (size_t)r_rows * 128 + q * r_rows * 32 + lane;
-        float* theirs = out + q * (M - r_rows) * 32 + lane;
-        const int there0 = rank ? 0 : r_half;
-        tmem_rows<RT>(taddr, hf, M, [&](int m, float v) { *(((m < r_half) == (rank == 0)) ? mine + (m - r_row0) * 32 : theirs + (m - there0) * 32) = v; });
+        const int mine = (r_rows * 4 + q * r_rows - r_row0) * 32 + lane;
+        const int theirs = (int)(out - in) + (q * (M - r_rows) - (rank ? 0 : r_half)) * 32 + lane;
+        const int below = rank ? theirs : mine, above = rank ? mine : theirs;      // where the rows below r_half and the others go
+        tmem_rows(taddr, hf, M, [&](int m, float v) { in[(m < r_half ? below : above) + m * 32] = v; });
       }
       tc_fence_before();
       fence_smem_async();
@@ -535,7 +516,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
     if (MODE == GC_RESIDUAL && S < M) {                                    // (the same in every CTA of the cluster)
       if (epi) {
         const uint32_t dst = dsmem_addr(smem_u32(in + rank * in_pitch + (w & 15)), (uint32_t)grp);
-        tmem_rows<RT>(taddr, hf, M, [&](int m, float v) { if (m >= S && grp != rank) dsmem_st(dst + (uint32_t)(m * 64), v); });
+        tmem_rows(taddr, hf, M, [&](int m, float v) { if (m >= S && grp != rank) dsmem_st(dst + (uint32_t)(m * 64), v); });
         tc_fence_before();
       }
       __syncwarp();
