@@ -22,6 +22,7 @@
 #include "attention_umma.cuh"
 #include "common.cuh"
 #include "gemm_cluster.cuh"
+#include "gemm_glu.cuh"
 #include "gemm_stream.cuh"
 #include "gemm_pair.cuh"
 #include "glue_tc.cuh"
@@ -585,6 +586,9 @@ int aligned_ctas(int n_tiles, int cap) {
   return cap;
 }
 
+// CTAs of the weight streamer for a launch of n_tiles weight tiles.
+int stream_ctas(const spec_ctx* c, int n_tiles) { return aligned_ctas(n_tiles, n_tiles <= 48 ? std::min(c->gemm_ctas, c->small_gemm_ctas) : c->gemm_ctas); }
+
 // ---- many rows: the two-SM kernel, the step after the projection in its epilogue ----
 bool pair_gemm_ok(const spec_ctx* c, int M, int K) { return c->wide_gemm && M > 128 && K % 64 == 0; }
 
@@ -690,8 +694,7 @@ int run_gemm(spec_ctx* c, const void* x, int M, int K, int n_mats, const void* c
     *view = v;
     return SPEC_OK;
   }
-  const int g_cap = aligned_ctas(tiles_all, tiles_all <= 48 ? std::min(c->gemm_ctas, c->small_gemm_ctas) : c->gemm_ctas);
-  if (!plan_gemm(M, K, n_mats, rows, g_cap, &g))
+  if (!plan_gemm(M, K, n_mats, rows, stream_ctas(c, tiles_all), &g))
     return c->fail(SPEC_E_BADARG, "unsupported linear shape");
   if (plan_part_floats(g) > c->part_floats) return c->fail(SPEC_E_NOMEM, "partial-sum scratch too small");
   StreamTmaps tm{};
@@ -726,10 +729,9 @@ bool cluster_gemm_ok(const spec_ctx* c, int mode, int M, int K) {
   if (!(c->cluster_epilogue & bit) || M < 1 || M > 128 || K % 64) return false;
   const int KC = K / 64;
   if (mode == GC_RESIDUAL) return KC >= GC_RES_CLUSTER;
-  // (gate+up of more than 64 rows stays with the weight streamer, and of fewer with clusters of three whatever the number of tiles: the split of the
-  // inner dimension decides how the operands of the next projection round, and with them which of two candidates that lie close
-  // comes first, that is, at which step a token is emitted. Clusters of eight for up to 33 tiles took 216 us a step instead of 252 on six layers of
-  // d_model 512, and clusters of three or eight for 65 to 128 rows 332 instead of 351 at 96 rows of d_model 1024.)
+  // (gate+up of more than 64 rows keeps the weight streamer's split of the inner dimension, in gemm_glu where that is the same for all tiles, and of
+  // fewer the clusters of three whatever the number of tiles: the split decides how the operands of the next projection round, and with
+  // them which of two candidates that lie close comes first, that is, at which step a token is emitted.)
   if (mode == GC_SWIGLU) return KC >= 3 && M <= 64;
   return KC >= GC_ROPE_CLUSTER && (c->cfg.head_dim == 64 || c->cfg.head_dim == 128);
 }
@@ -795,6 +797,59 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
     c->launches++;
   }
   if (e != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("gemm_cluster launch: ") + cudaGetErrorString(e));
+  return SPEC_OK;
+}
+
+// CTAs that share a (gate tile, up tile) pair in gemm_glu, 0 where the weight streamer and swiglu_reduce_tc serve: the streamer's plan has to cut the K chunks
+// of every tile into the same runs (then it has no run that crosses a tile), at most eight, and all clusters have to fit the chip at one CTA
+// an SM (cudaOccupancyMaxActiveClusters): a second wave would wait for the whole chain of the first.
+int glu_cluster(const spec_ctx* c, int M, int K) {
+  if (!(c->cluster_epilogue & 2) || M <= 64 || M > 128 || K % 64) return 0;
+  const int F = c->cfg.d_ffn, tiles = 2 * ((F + 127) / 128), rows[2] = {F, F};
+  GemmPlan g;
+  if (!plan_gemm(M, K, 2, rows, stream_ctas(c, tiles), &g) || g.grid % tiles) return 0;
+  constexpr int most[GLU_MAX_CLUSTER + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+  const int cs = g.grid / tiles;
+  return cs <= GLU_MAX_CLUSTER && tiles / 2 <= most[cs] ? cs : 0;
+}
+
+int run_gemm_glu(spec_ctx* c, const void* in, int M, int K, int cs, const void* const* mats, bf16* act) {
+  const int F = c->cfg.d_ffn, units = (K / 64 + cs - 1) / cs;
+  GluGemmParams p{};
+  StreamTmaps tm{};
+  p.M = M; p.KC = K / 64; p.N = F; p.stages = std::min(units, GLU_MAX_STAGES); p.act = act; p.status = c->d_status;
+  for (int i = 0; i < 2; ++i) {
+    if (c->packed) { p.packed[i] = static_cast<const uint8_t*>(mats[i]); continue; }
+    const CUtensorMap* t = c->tmap(mats[i], F, K, 128);
+    if (!t) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (weights)");
+    tm.a[i] = *t;
+  }
+  const CUtensorMap* tb = c->tmap(in, round_up(M, 16), K, (uint32_t)round_up(M, 16));
+  if (!tb) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (activations)");
+  tm.b = *tb;
+  p.trace = c->next_trace(gemm_kind_name(SPEC_PROFILE_GATE_UP));
+  static bool attr_set_dev[kAttrDevices] = {};
+  bool& attr_set = *attr_flag(attr_set_dev);
+  if (!attr_set) {
+    CUDA_OK(cudaFuncSetAttribute(gemm_glu, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    attr_set = true;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((F + 127) / 128 * cs); cfg.blockDim = dim3(GLU_THREADS); cfg.dynamicSmemBytes = (size_t)glu_smem_bytes(M, cs, p.stages); cfg.stream = c->stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = c->pdl ? 2 : 1;
+  cudaError_t e;
+  {
+    ProfScope ps(c, SPEC_PROFILE_GATE_UP);
+    e = cudaLaunchKernelEx(&cfg, gemm_glu, tm, p);
+    c->launches++;
+  }
+  if (e != cudaSuccess) return c->fail(SPEC_E_CUDA, std::string("gemm_glu launch: ") + cudaGetErrorString(e));
   return SPEC_OK;
 }
 
@@ -1167,6 +1222,8 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
         if ((r = run_gemm_pair(c, GP_SWIGLU, u, M, d, 2, mats, rws, &w, SPEC_PROFILE_GATE_UP))) return r;
       } else if (cluster_gemm_ok(c, GC_SWIGLU, M, d)) {
         if ((r = run_gemm_cluster(c, GC_SWIGLU, u, M, d, mats, F, nullptr, act, SPEC_PROFILE_GATE_UP))) return r;
+      } else if (const int cs = glu_cluster(c, M, d)) {
+        if ((r = run_gemm_glu(c, u, M, d, cs, mats, act))) return r;
       } else {
         PartView vg{};
         if ((r = run_gemm(c, u, M, d, 2, mats, rws, SPEC_PROFILE_GATE_UP, &vg))) return r;

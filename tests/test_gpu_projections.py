@@ -30,3 +30,52 @@ def test_ring_depths(torch, M, chunks):
     """Grids of at most one CTA an SM get a stage for every K chunk of a CTA (`chunks`, here of a cluster of eight): the ring of which two fit an
     SM and one chunk more, the deepest ring full and run through again, and activation rows that fill the MMA's N only in part."""
     check_linear(torch, M, 1000, 8 * 64 * chunks, 128)
+
+
+def random_decoder(torch, cfg, seed, max_seq):
+    from paper_2503_14153_b200 import FLAG_KEEP_LOGITS, SpecDecoder, build_tree
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    d, F, HD, KD = cfg.d_model, cfg.d_ffn, cfg.n_heads * cfg.head_dim, cfg.n_kv_heads * cfg.head_dim
+
+    def normal(rows, cols, std):
+        return (torch.randn((rows, cols), generator=g, device="cuda") * std).bfloat16()
+
+    w = {"embed": normal(cfg.vocab, d, 1.0), "lm_head": normal(cfg.vocab, d, 0.02), "final_norm": torch.ones(d, device="cuda")}
+    for l in range(cfg.n_layers):
+        p = f"layers.{l}."
+        w.update({p + "wqkv": normal(HD + 2 * KD, d, d ** -0.5), p + "wo": normal(d, HD, HD ** -0.5), p + "w_gate": normal(F, d, d ** -0.5),
+                  p + "w_up": normal(F, d, d ** -0.5), p + "w_down": normal(d, F, F ** -0.5),
+                  p + "attn_norm": torch.ones(d, device="cuda"), p + "ffn_norm": torch.ones(d, device="cuda")})
+    for k in range(cfg.n_medusa):
+        w[f"medusa.{k}.w"] = normal(d, d, 0.01)
+        w[f"medusa.{k}.b"] = normal(1, d, 0.02)[0].contiguous()
+    return SpecDecoder(cfg, w, build_tree(cfg.topk, cfg.tree_nodes), max_seq, max_batch=cfg.batch, flags=FLAG_KEEP_LOGITS)
+
+
+@pytest.mark.parametrize("d,ffn,T", [
+    (512, 1344, 65), (512, 1344, 96), (512, 1344, 97), (512, 2304, 128),      # clusters of eight (the second: too many of them, the streamer serves)
+    (512, 1920, 100), (1024, 2752, 69), (1024, 2752, 128),                    # eight again, six, two rounds
+    (1280, 3200, 77), (1280, 3968, 113),                                      # five, four: a chunk more than stages
+    (2048, 5248, 80), (2048, 7936, 66), (1024, 16000, 112),                   # three (11 chunks a CTA: the ring refilled), two, one
+    (256, 640, 70),                                                           # a run a chunk, fewer CTAs than the cap
+])
+def test_gate_up_in_clusters_as_the_streamer(torch, d, ffn, T):
+    """Gate, up and SwiGLU of 65 to 128 rows in one kernel: a layer's hidden rows, its cache and the logits are those of the weight streamer with the
+    kernel behind it, bit for bit."""
+    import numpy as np
+    from paper_2503_14153_b200 import binding as B
+    from synthetic import get_config
+    cfg = get_config("c0", name="glu", n_layers=2, d_model=d, n_heads=d // 128, n_kv_heads=max(1, d // 256), head_dim=128, d_ffn=ffn, vocab=1000, dtype="bf16",
+                     rope_base=1e6, n_medusa=4, topk=(10, 4, 2, 2), tree_nodes=T)
+    prompt = np.random.default_rng(T).integers(0, 1000, 90).astype(np.int32)
+    seen = {}
+    for mask in (7, 5):
+        gpu = random_decoder(torch, cfg, 5, 160)
+        gpu.set_option(B.OPT_CLUSTER_EPILOGUE, mask)
+        gpu.prefill(prompt)
+        out = [gpu.step() for _ in range(2)]
+        seen[mask] = [np.concatenate([np.append(t[0, :n[0]], n[0]) for t, n in out]), gpu.debug(B.DBG_HIDDEN), gpu.debug(B.DBG_LOGITS), *gpu.read_kv(0, 1, 0, 90 + T)]
+        gpu.close()
+    assert np.isfinite(seen[7][1]).all() and np.abs(seen[7][1]).max() > 0.1
+    for a, b in zip(seen[7], seen[5]):
+        assert a.tobytes() == b.tobytes()
