@@ -57,6 +57,7 @@ struct AttnTcArgs {
   int layer, H;
   int nsplit;           // KV splits launched (gridDim.y); the splits in use are min(nsplit, ceil(tiles / split_tiles))
   int split_tiles;      // fewest KV tiles worth a split of their own
+  int row_parts;        // attention_tc, one split: CTAs that share a (sequence, head), each with its own NW * 16 query rows (1: one has all)
   int stages;           // KV tiles in flight per CTA (2..ATTN_MAX_STAGES, at least KG); sizes the shared memory
   int n_lo[ATTN_MAX_SEQS];   // host's lower bound of each sequence's committed length: keys below it
                              // were written by earlier steps and may be fetched before the dependency wait
@@ -105,8 +106,8 @@ attention_tc(const AttnTcArgs a, unsigned long long* tr) {
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rg = warp % NW, kg = warp / NW;
-  const int h = blockIdx.x, sp = blockIdx.y, b = blockIdx.z;
-  constexpr int row0 = 0;                                        // the CTA owns all query rows of its sequence
+  const int h = blockIdx.x, sp = blockIdx.y, b = blockIdx.z / a.row_parts;
+  const int row0 = (int)(blockIdx.z % a.row_parts) * NW * 16;    // the CTA's first query row
   const int H = a.H, kvh = h / (H / a.g.n_kv_heads);
   const bool single = a.nsplit == 1;          // one split: its tiles start at 0 whatever the length
   const int* pt = a.page_table + a.rows.sequence(b) * a.g.pages_per_seq;
@@ -162,8 +163,8 @@ attention_tc(const AttnTcArgs a, unsigned long long* tr) {
   const int tps = (total_tiles + nsplit - 1) / nsplit;
   t0 = sp * tps;
   const int t1 = min(total_tiles, t0 + tps);
-  if (cnt == 0 || sp >= nsplit) {
-    // inactive sequence or unused split: let the copies already in flight land before the CTA goes away
+  if (cnt <= row0 || sp >= nsplit) {
+    // inactive sequence, no rows here or unused split: let the copies already in flight land before the CTA goes away
     if (threadIdx.x == 0)
       for (int i = 0; i < pre; ++i) mbar_wait(&full[i], 0, a.status, 21);
     return;
