@@ -1236,9 +1236,13 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
       } else {
         PartView vg{};
         if ((r = run_gemm(c, u, M, d, 2, mats, rws, SPEC_PROFILE_GATE_UP, &vg))) return r;
-        size_t total = (size_t)M * (F / 4);
-        unsigned blocks = (unsigned)std::min<size_t>((total + 255) / 256, 2 * SM_SLOTS);
-        KLAUNCH("swiglu_reduce_tc", swiglu_reduce_tc, dim3(blocks), dim3(256), 0, vg, 0, up0, act, M, F);
+        int slots = 0;
+        for (int t = 0; t < 2 * (up0 / 128) * vg.seg.m_tiles; ++t) slots = std::max(slots, vg.seg.nseg(t));
+        if (slots <= 2) {
+          KLAUNCH("swiglu_reduce_tc", swiglu_reduce_tc<SWIGLU_ROWS>, dim3((F / 4 + 255) / 256, (M + SWIGLU_ROWS - 1) / SWIGLU_ROWS), dim3(256), 0, vg, 0, up0, act, M, F);
+        } else {
+          KLAUNCH("swiglu_reduce_tc", swiglu_reduce_tc<1>, dim3((F / 4 + 255) / 256, M), dim3(256), 0, vg, 0, up0, act, M, F);
+        }
       }
     }
     {
