@@ -17,6 +17,11 @@
 // tiles leave some of them idle does not pay: the clusters share the L2's bandwidth, so that fewer of them run faster; at 2048
 // rows the output and down projections took 184 us instead of 120.)
 //
+// The work of a launch is a list of items: tiles of `tile_rows` activation rows (256, or fewer where that fills the waves better or gives a narrow
+// projection to more clusters), of which those from cut_first on, the last wave's, may be cut into slices. The host chooses by a model of the
+// kernel's time (plan_pair); an element's inner dimension runs through in the same order whatever the rows of its item. Fewer rows a stage leave
+// room for more stages: 16 rows, the last tokens of prompts, have eleven.
+//
 // Modes:
 //  * GP_PLAIN     float32 sums to out[m][ld] (columns below n_cols only). The only mode whose sums are results as they stand:
 //                 the two halves of the inner dimension go to the two accumulators and are added in registers, because the error
@@ -61,7 +66,10 @@ struct PairGemmParams {
   int M, KC;                                // activation rows, K / 64
   int n_mats;
   int mat_tile0[GS_MAX_MATS + 1];           // first 128-row weight tile of each stacked matrix
-  int n_tiles, w_pairs, m_tiles;            // weight tiles (all matrices), pairs of them, activation tiles of NT rows
+  int n_tiles, w_pairs, m_tiles;            // weight tiles (all matrices), pairs of them, activation tiles
+  int tile_rows;                            // activation rows of a tile: a multiple of 16, at most NT (parts > 1: NT)
+  int cut_first, cut;                       // tiles from cut_first on are done as `cut` slices of tile_rows / cut activation rows each (a multiple of 16)
+  int stages;                               // of the ring
   int plan_tiles;                           // host: tiles of the launch whose sharing (parts) this one follows, 0: its own
   int parts;                                // clusters that share a tile's K chunks (1: tiles are whole)
   float* part;                              // parts > 1: [tile][part][CTA of the pair][NT][128] float32
@@ -92,12 +100,14 @@ template <int NT> struct PairCfg {
   static constexpr int BK = 64;
   static constexpr int A_BYTES = 128 * BK * 2;
   static constexpr int B_BYTES = (NT / 2) * BK * 2;
-  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = 6;
+  static constexpr int RING_BYTES = 6 * (A_BYTES + B_BYTES);
+  static constexpr int MAX_STAGES = 11;
+  static __host__ __device__ constexpr int stage_bytes(int rows) { return A_BYTES + rows / 2 * BK * 2; }
+  static __host__ __device__ constexpr int stages(int rows) { return RING_BYTES / stage_bytes(rows) < MAX_STAGES ? RING_BYTES / stage_bytes(rows) : MAX_STAGES; }
   static constexpr int EX_COLS = 8;                               // activation rows swapped in one direction at a time
   static constexpr int EX_BYTES = GP_QUARTERS * 2 * 64 * EX_COLS * 4;       // [part][direction][column][64 pairs] float32
   static constexpr int META_BYTES = NT * 16;                      // GP_ROPE: (cache offset, position, swizzle row) of a row
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EX_BYTES + META_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
+  static constexpr int SMEM_BYTES = RING_BYTES + EX_BYTES + META_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
   static constexpr int TMEM_COLS = 2 * NT;
 };
 
@@ -142,6 +152,11 @@ __device__ __forceinline__ bool epilogue_and(bool v) {
   return r != 0;
 }
 
+struct PairTmaps {
+  CUtensorMap a[GS_MAX_MATS];
+  CUtensorMap b, b_cut;                     // boxes of half a tile's and half a slice's activation rows
+};
+
 struct PairRowMeta {
   long long kv;      // element offset of the row's slot within its (layer, head) K|V blocks; -1: row not in use
   int pos, prow;
@@ -150,21 +165,21 @@ struct PairRowMeta {
 // SPLIT: p.parts > 1.
 template <int MODE, int NT, bool SPLIT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
-gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
+gemm_pair(const __grid_constant__ PairTmaps tm, const PairGemmParams p) {
   using Cfg = PairCfg<NT>;
-  constexpr int STAGES = Cfg::STAGES;
+  const int stages = p.stages, stage_bytes = Cfg::stage_bytes(p.tile_rows);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* tiles = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  float* exch = reinterpret_cast<float*>(tiles + STAGES * Cfg::STAGE_BYTES);
-  PairRowMeta* meta = reinterpret_cast<PairRowMeta*>(tiles + STAGES * Cfg::STAGE_BYTES + Cfg::EX_BYTES);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + STAGES * Cfg::STAGE_BYTES + Cfg::EX_BYTES + Cfg::META_BYTES);
+  float* exch = reinterpret_cast<float*>(tiles + Cfg::RING_BYTES);
+  PairRowMeta* meta = reinterpret_cast<PairRowMeta*>(tiles + Cfg::RING_BYTES + Cfg::EX_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + Cfg::RING_BYTES + Cfg::EX_BYTES + Cfg::META_BYTES);
   uint64_t* full = bars;                    // leader's: both CTAs' operands of a stage have landed
-  uint64_t* empty = bars + STAGES;          // each CTA's: the stage has been read
-  uint64_t* acc_full = bars + 2 * STAGES;   // each CTA's
-  uint64_t* acc_empty = bars + 2 * STAGES + 2;   // leader's: drained by the sixteen warps of both CTAs
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
-  volatile uint32_t* last_slot = reinterpret_cast<volatile uint32_t*>(bars + 2 * STAGES + 5);   // this CTA completes a split tile
+  uint64_t* empty = bars + Cfg::MAX_STAGES;          // each CTA's: the stage has been read
+  uint64_t* acc_full = bars + 2 * Cfg::MAX_STAGES;   // each CTA's
+  uint64_t* acc_empty = bars + 2 * Cfg::MAX_STAGES + 2;   // leader's: drained by the sixteen warps of both CTAs
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * Cfg::MAX_STAGES + 4);
+  volatile uint32_t* last_slot = reinterpret_cast<volatile uint32_t*>(bars + 2 * Cfg::MAX_STAGES + 5);   // this CTA completes a split tile
 
   KTrace kt(p.trace);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -173,21 +188,39 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   const int KC = p.KC;
   // this cluster's work: tiles cl, cl + ncl, ..., or with parts > 1 one part of one tile
   const int total_tiles = p.w_pairs * p.m_tiles, parts = SPLIT ? p.parts : 1;
-  const int my_tiles = cl < total_tiles * parts ? (SPLIT ? 1 : (total_tiles - 1 - cl) / ncl + 1) : 0;
+  const int items = SPLIT ? total_tiles * parts : p.cut_first + (total_tiles - p.cut_first) * p.cut;
+  const int my_tiles = cl < items ? (SPLIT ? 1 : (items - 1 - cl) / ncl + 1) : 0;
   const int k_lo = SPLIT ? cl % parts * KC / parts : 0, k_hi = SPLIT ? (cl % parts + 1) * KC / parts : KC;
   static_assert(MODE != GP_PLAIN || !SPLIT, "plain sums are not shared between clusters");
   const int halves = MODE == GP_PLAIN && KC > 1 ? 2 : 1;    // accumulators a tile's inner dimension is cut into
-  auto tile_of = [&](int i) { return SPLIT ? cl / parts : cl + i * ncl; };
+  // this cluster's i-th item: weight pair, first activation row and rows
+  struct Item { int tau, wp, row0, rows; };
+  auto item_of = [&](int i) {
+    Item v;
+    int sub = 0;
+    v.tau = SPLIT ? cl / parts : cl + i * ncl;
+    v.rows = SPLIT ? NT : p.tile_rows;
+    if (!SPLIT && v.tau >= p.cut_first) {
+      const int s = v.tau - p.cut_first;
+      v.rows = p.tile_rows / p.cut;
+      v.tau = p.cut_first + s / p.cut;
+      sub = s % p.cut;
+    }
+    v.wp = v.tau / p.m_tiles;
+    v.row0 = (v.tau - v.wp * p.m_tiles) * (SPLIT ? NT : p.tile_rows) + sub * v.rows;
+    return v;
+  };
 
   pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < stages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(&acc_full[0], 1); mbar_init(&acc_full[1], 1);
     mbar_init(&acc_empty[0], 2 * GP_EPI / 32); mbar_init(&acc_empty[1], 2 * GP_EPI / 32);
     mbar_fence_init();
     for (int i = 0; i < p.n_mats; ++i) tma_prefetch_desc(&tm.a[i]);
     tma_prefetch_desc(&tm.b);
+    if (!SPLIT && p.cut_first < total_tiles) tma_prefetch_desc(&tm.b_cut);
   }
   if (warp == 1) tmem_alloc2(tmem_slot, Cfg::TMEM_COLS);
   tc_fence_before();
@@ -208,12 +241,13 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
   if (warp == 0) {
     if (elect_one()) {
       // ---- producer: this CTA's weight rows and its half of the activation rows ----
-      struct At { int i, kc, wp, mt; };
+      struct At { int i, kc, wp, row0, rows; };
       auto at_tile = [&](At& a) {
-        const int tau = tile_of(a.i);
-        a.wp = tau / p.m_tiles; a.mt = tau - a.wp * p.m_tiles;
+        const Item v = item_of(a.i);
+        a.wp = v.wp; a.row0 = v.row0; a.rows = v.rows;
       };
       auto next = [&](At& a) { if (++a.kc == k_hi) { a.kc = k_lo; ++a.i; at_tile(a); } };
+      auto expect = [&](const At& a, int st) { if (rank == 0) mbar_expect_tx(&full[st], 2 * (Cfg::A_BYTES + a.rows / 2 * Cfg::BK * 2)); };
       auto load_a = [&](uint8_t* dst, const At& a, uint32_t bar) {
         if (MODE == GP_SWIGLU) {
           const int row = (p.packed ? (a.wp * KC + a.kc) * 128 : a.wp * 128) + rank * 64, x = p.packed ? 0 : a.kc * Cfg::BK;
@@ -225,41 +259,41 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         }
       };
       auto load_b = [&](uint8_t* dst, const At& a, uint32_t bar) {
-        tma_load_2d_pair(dst, &tm.b, a.kc * Cfg::BK, a.mt * NT + rank * (NT / 2), bar);
+        tma_load_2d_pair(dst, SPLIT || a.rows == p.tile_rows ? &tm.b : &tm.b_cut, a.kc * Cfg::BK, a.row0 + rank * (a.rows / 2), bar);
       };
       const int n_units = my_tiles * (k_hi - k_lo);
-      const int n_pre = n_units < STAGES ? n_units : STAGES;
+      const int n_pre = n_units < stages ? n_units : stages;
       const uint32_t full0 = dsmem_addr(smem_u32(full), 0);            // the leader's barriers
-      At a{0, k_lo, 0, 0};
+      At a{0, k_lo, 0, 0, 0};
       at_tile(a);
       At b = a;
       // weights do not depend on the kernel before this one
       for (int i = 0; i < n_pre; ++i, next(a)) {
-        if (rank == 0) mbar_expect_tx(&full[i], 2 * Cfg::STAGE_BYTES);
-        load_a(tiles + i * Cfg::STAGE_BYTES, a, full0 + 8 * i);
+        expect(a, i);
+        load_a(tiles + i * stage_bytes, a, full0 + 8 * i);
       }
       pdl_wait();
-      for (int i = 0; i < n_pre; ++i, next(b)) load_b(tiles + i * Cfg::STAGE_BYTES + Cfg::A_BYTES, b, full0 + 8 * i);
+      for (int i = 0; i < n_pre; ++i, next(b)) load_b(tiles + i * stage_bytes + Cfg::A_BYTES, b, full0 + 8 * i);
       bool ok = true;
       int issued = n_pre, st = 0;
       uint32_t ph = 0;
       for (; issued < n_units; ++issued, next(a)) {
         if (!mbar_wait(&empty[st], ph, p.status, 40)) { ok = false; break; }
-        uint8_t* dst = tiles + st * Cfg::STAGE_BYTES;
-        if (rank == 0) mbar_expect_tx(&full[st], 2 * Cfg::STAGE_BYTES);
+        uint8_t* dst = tiles + st * stage_bytes;
+        expect(a, st);
         load_a(dst, a, full0 + 8 * st);
         load_b(dst + Cfg::A_BYTES, a, full0 + 8 * st);
-        if (++st == STAGES) { st = 0; ph ^= 1; }
+        if (++st == stages) { st = 0; ph ^= 1; }
       }
       if (!ok && rank == 0) {
-        for (int i = issued > STAGES ? issued - STAGES : 0; i < issued; ++i)
-          mbar_wait(&full[i % STAGES], (i / STAGES) & 1, p.status, 43);
+        for (int i = issued > stages ? issued - stages : 0; i < issued; ++i)
+          mbar_wait(&full[i % stages], (i / stages) & 1, p.status, 43);
       }
     }
   } else if (warp == 1) {
     if (rank == 0 && elect_one()) {
       // ---- MMA issuer of the pair ----
-      const uint32_t idesc = make_idesc_bf16(256, NT);
+      const uint64_t adesc0 = make_kmajor_sw128_desc(smem_u32(tiles)), bdesc0 = make_kmajor_sw128_desc(smem_u32(tiles) + Cfg::A_BYTES);
       bool ok = true;
       int st = 0;
       uint32_t ph = 0;
@@ -267,21 +301,19 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         const int buf = i & 1;
         if (!mbar_wait(&acc_empty[buf], ((i >> 1) & 1) ^ 1, p.status, 44)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_addr = tmem_base + (uint32_t)(buf * NT);
+        const uint32_t d_addr = tmem_base + (uint32_t)(buf * NT), idesc = make_idesc_bf16(256, item_of(halves == 2 ? i >> 1 : i).rows);
         const int mid = (k_lo + k_hi) >> 1;
         const int k_first = halves == 2 && buf ? mid : k_lo, k_end = halves == 2 && !buf ? mid : k_hi;
         for (int kc = k_first; kc < k_end; ++kc) {
           if (!mbar_wait(&full[st], ph, p.status, 41)) { ok = false; break; }
           if (i == 0 && kc == k_lo) trace_mark_min(p.trace, 2);
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(tiles + st * Cfg::STAGE_BYTES);
-          const uint64_t adesc = make_kmajor_sw128_desc(a_addr);
-          const uint64_t bdesc = make_kmajor_sw128_desc(a_addr + Cfg::A_BYTES);
+          const uint64_t adesc = adesc0 + (uint64_t)(st * (stage_bytes >> 4)), bdesc = bdesc0 + (uint64_t)(st * (stage_bytes >> 4));
 #pragma unroll
           for (int k = 0; k < Cfg::BK / 16; ++k)
             tc_mma_f16_pair(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kc > k_first || k > 0) ? 1u : 0u);
           tc_commit_pair(&empty[st]);
-          if (++st == STAGES) { st = 0; ph ^= 1; }
+          if (++st == stages) { st = 0; ph ^= 1; }
         }
         if (!ok) break;
         tc_commit_pair(&acc_full[buf]);
@@ -290,8 +322,8 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
     }
   } else {
     // ---- epilogue: warp w may touch tensor-memory lanes [32 (w % 4), +32); warps 2..5 take the first quarter of the
-    // tile's activation rows, warps 6..9 the second, ... ----
-    constexpr int HC = NT / GP_QUARTERS;
+    // item's 16-row groups, warps 6..9 the second, ... ----
+    constexpr int HC = NT / GP_QUARTERS;                      // rows of a quarter of the largest tile
     const int q = warp & 3, hf = (warp - 2) >> 2;
     const int wl = q * 32 + lane;                             // weight row within the CTA's 128
     const uint32_t acc_empty0 = dsmem_addr(smem_u32(acc_empty), 0);
@@ -300,11 +332,12 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
     for (int i = 0; i < my_tiles; ++i) {
       const int buf = halves == 2 ? 1 : i & 1;                // the accumulator that completes the tile
       const uint32_t acc_ph = halves == 2 ? i & 1 : (i >> 1) & 1;
-      const int tau = tile_of(i);
-      const int wp = tau / p.m_tiles, mt = tau - wp * p.m_tiles;
+      const Item item = item_of(i);
+      const int tau = item.tau, wp = item.wp, groups = item.rows >> 4;
+      const int g0 = hf * groups / GP_QUARTERS, ng = (hf + 1) * groups / GP_QUARTERS - g0;   // this warp's 16-row groups
       const int nt = 2 * wp + rank;
-      const int m0 = mt * NT + hf * HC;                       // this warp's first activation row
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * NT + hf * HC);
+      const int m0 = item.row0 + g0 * 16;                     // this warp's first activation row
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * NT + g0 * 16);
       constexpr bool split = SPLIT;
       // (what the epilogue needs besides the sums is fetched while the tile's MMAs run)
       // GP_RESIDUAL: old values of the first rows
@@ -320,13 +353,13 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           src += p.n_cols;
         }
       };
-      if (MODE == GP_RESIDUAL && !split) fetch_x(0, xo);
+      if (MODE == GP_RESIDUAL && !split && ng > 0) fetch_x(0, xo);
       // GP_ROPE: the rows' positions and cache slots
-      PairRowMeta* mrow = meta + hf * HC;
+      PairRowMeta* mrow = meta + hf * HC;                     // (a place of its own: the other quarters may be behind, on another item)
       if (MODE == GP_ROPE) {
         const int e = threadIdx.x - 64 - hf * 128;
         group_bar(1 + hf);                                     // everybody is through with the previous tile's rows
-        if (e < HC) {
+        if (e < ng * 16) {
           PairRowMeta v{-1, 0, 0};
           const int m = m0 + e;
           if (m < p.M) {
@@ -351,6 +384,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         if (halves == 2) {
           if (!epilogue_and(mbar_wait(&acc_full[0], acc_ph, p.status, 42))) break;
           tc_fence_after();
+          // (all of a quarter's HC columns, also where the item has fewer: they are this CTA's, and rows that are not its own are not stored)
           uint32_t r[HC / 32][32];
 #pragma unroll
           for (int g = 0; g < HC / 32; ++g) tmem_ld32(taddr - NT + g * 32, r[g]);
@@ -431,7 +465,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * buf);
-        const int live = on && p.out ? p.M - m0 : 0;
+        const int live = on && p.out ? min(p.M - m0, ng * 16) : 0;
 #pragma unroll
         for (int j = 0; j < HC; ++j) {                         // (a running pointer: separate addresses cost 2-3 us a tile)
           if (j < live) *dst = first[j];
@@ -469,7 +503,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
             }
             const int m = m0 + j + lane;
             const float best = first[j];
-            if (nt < p.n_tiles && m < p.M) {
+            if (nt < p.n_tiles && m < p.M && j + lane < ng * 16) {
               p.best_val[(size_t)(nt * 4 + q) * p.M + m] = best == best ? best : -INFINITY;
               p.best_idx[(size_t)(nt * 4 + q) * p.M + m] = best == best ? nt * 128 + q * 32 + from[0] : 0x7fffffff;
             }
@@ -479,10 +513,10 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
       } else if constexpr (MODE == GP_RESIDUAL) {
         // old values of the next 16 rows are fetched while 16 rows are finished
 #pragma unroll 1
-        for (int g = 0; g < HC / 16; ++g) {
+        for (int g = 0; g < ng; ++g) {
           uint32_t r[16];
           float next[16];
-          if (g + 1 < HC / 16) fetch_x(g + 1, next);
+          if (g + 1 < ng) fetch_x(g + 1, next);
           acc(g, r);
           float* dst = p.out + (size_t)(m0 + g * 16) * p.n_cols + rcol;
           const int live = ron ? p.M - m0 - g * 16 : 0;
@@ -508,7 +542,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           const int col = nt * 64 + pr;
           const bool on = col < p.n_cols;
 #pragma unroll 1
-          for (int g = 0; g < HC / 16; ++g) {
+          for (int g = 0; g < ng; ++g) {
             uint32_t r[16];
             acc(g, r);
             if (g) group_bar(1 + hf);
@@ -538,7 +572,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           if (kind == 2) {
             bf16* dst = p.pool + lh + p.g.block_elems();
 #pragma unroll 1
-            for (int g = 0; g < HC / 16; ++g) {
+            for (int g = 0; g < ng; ++g) {
               uint32_t r[16];
               acc(g, r);
 #pragma unroll
@@ -550,7 +584,7 @@ gemm_pair(const __grid_constant__ StreamTmaps tm, const PairGemmParams p) {
           } else {
             const int di = dim & (half - 1);                     // the pair's place in its head
 #pragma unroll 1
-            for (int g = 0; g < HC / 16; ++g) {
+            for (int g = 0; g < ng; ++g) {
               uint32_t r[16];
               const int jb = g * 16 + (lower ? 0 : 8);
               float2 t[8];

@@ -607,9 +607,64 @@ int qkv_pairs(const spec_config& f) {
   return ((HD + 127) / 128 + 2 * ((KD + 127) / 128) + 1) / 2;
 }
 
+// What a launch of `tiles` = w_pairs * ceil(M / rows) tiles takes in microseconds, the tiles of its last wave cut in `cut`. Fitted to 45 kernels of 15 tile
+// heights each (M 384 to 2304 on d_model 4096, 1024 and 512, event-timed at 1.9 GHz; within 10% of most): a K chunk on all clusters takes
+// (0.002 + 0.0013 rows) us, the operands' way out of L2 (0.335 at 256 rows, the same per row from 176 rows on), on few clusters 0.00107 rows, the MMAs,
+// and never less than 0.18, the issue; a tile's epilogue 0.0165 us a row where it adds to the residual stream, 0.028 in the other
+// modes, under the next tile's MMAs, but for the last.
+float pair_cost(int tiles, int rows, int cut, int KC, int clusters, float epilogue) {
+  auto chunk = [&](int h, int n) { return std::max(std::max(0.18f, 0.00107f * h), std::max(0.16f + 0.0004f * h, 0.002f + 0.0013f * h) * n / GP_MAX_CLUSTERS); };
+  auto waves = [&](int items, int h, bool last) {
+    const int full = items / clusters, rest = items % clusters;
+    const float wave = std::max(KC * chunk(h, clusters), epilogue * h) + 1.f;
+    float us = full * wave;
+    if (rest) us += KC * chunk(h, rest) + 1.f;
+    return us + (last ? epilogue * h : 0.f);
+  };
+  if (cut == 1) return waves(tiles, rows, true);
+  const int rest = tiles % clusters;
+  return waves(tiles - rest, rows, rest == 0) + (rest ? waves(rest * cut, rows / cut, true) : 0.f);
+}
+
+// How a launch is cut into items (gemm_pair.cuh), by M, KC, w_pairs and plan_tiles of `p`; with `may_share` the K chunks of few tiles go to several
+// clusters. Otherwise the tile height that pair_cost likes best: 256 rows, less where that fills the last wave better or brings more
+// clusters to work on a narrow projection, or 256 with the last wave's tiles cut. The choice moves no sum: every element's inner dimension
+// runs through as before. 7B shape: q/k/v of 2048 rows 141 -> 127 us (last wave in quarters), output and down projections of 1536 rows 50 -> 40 and
+// 124 -> 95 (176 rows); d_model 1024, 896 rows: 16.6 -> 10.8, 11.6 -> 7.5, gate+up 21.3 -> 16.6, down 18.9 -> 12.3; the last row of a prompt through
+// a 7B layer 166 -> 117 (16 rows, a ring of eleven stages).
+void plan_pair(PairGemmParams* p, int mode, bool may_share, int max_clusters = GP_MAX_CLUSTERS) {
+  const int clusters = std::min(GP_MAX_CLUSTERS, max_clusters), tall = p->w_pairs * ((p->M + GP_NT - 1) / GP_NT);
+  p->tile_rows = GP_NT; p->cut = 1;
+  p->parts = may_share ? pair_parts(p->plan_tiles ? p->plan_tiles : tall, p->KC, clusters) : 1;
+  if (p->parts == 1) {
+    const float epilogue = mode == GP_RESIDUAL ? 0.0165f : 0.028f;
+    // Lower tiles take more bytes out of L2 for the same work, which a launch of several waves pays for in power, and with it in clock: they have to
+    // look better by a tenth (1024 rows in tiles of 176 were 4% faster by themselves and slower in a step of 16 sequences).
+    const int most = std::min(GP_NT, (int)round_up(p->M, 16));
+    auto cost = [&](int rows, int cut) { return pair_cost(p->w_pairs * ((p->M + rows - 1) / rows), rows, cut, p->KC, clusters, epilogue); };
+    float best = cost(most, 1);
+    const float low = 0.9f * best;
+    p->tile_rows = most;
+    if (most == GP_NT)
+      for (int cut = 2; cut <= 4; cut *= 2) {
+        const float us = cost(most, cut);
+        if (us < 0.98f * best) { best = us; p->cut = cut; }
+      }
+    for (int rows = most - 16; rows >= 16; rows -= 16) {
+      const float us = cost(rows, 1);
+      if (us < low && us < 0.99f * best) { best = us; p->tile_rows = rows; p->cut = 1; }
+    }
+  }
+  p->m_tiles = (p->M + p->tile_rows - 1) / p->tile_rows;
+  const int tiles = p->w_pairs * p->m_tiles;
+  p->cut_first = p->cut > 1 ? tiles / clusters * clusters : tiles;
+  if (p->cut_first == tiles) p->cut = 1;
+  p->stages = PairCfg<GP_NT>::stages(p->tile_rows);
+}
+int pair_items(const PairGemmParams& p) { return p.parts > 1 ? p.w_pairs * p.m_tiles * p.parts : p.cut_first + (p.w_pairs * p.m_tiles - p.cut_first) * p.cut; }
+
 template <int MODE>
-cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemmParams p, float* part, unsigned int* arrive,
-                      int max_clusters = GP_MAX_CLUSTERS) {
+cudaError_t launch_gp(cudaStream_t st, bool pdl, const PairTmaps& tm, const PairGemmParams& p, int max_clusters = GP_MAX_CLUSTERS) {
   static bool attr_set_dev[kAttrDevices] = {};
   bool& attr_set = *attr_flag(attr_set_dev);
   if (!attr_set) {
@@ -619,11 +674,7 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemm
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  const int clusters = std::min(GP_MAX_CLUSTERS, max_clusters);
-  const int tiles = p.w_pairs * p.m_tiles;
-  p.parts = MODE != GP_PLAIN && part ? pair_parts(p.plan_tiles ? p.plan_tiles : tiles, p.KC, clusters) : 1;
-  p.part = part; p.arrive = arrive;
-  const int grid = 2 * (p.parts > 1 ? tiles * p.parts : std::min(tiles, clusters));
+  const int items = pair_items(p), grid = 2 * (p.parts > 1 ? items : std::min(items, std::min(GP_MAX_CLUSTERS, max_clusters)));
   auto kernel = gemm_pair<MODE, GP_NT, false>;
   if constexpr (MODE != GP_PLAIN)
     if (p.parts > 1) kernel = gemm_pair<MODE, GP_NT, true>;
@@ -633,7 +684,7 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const StreamTmaps& tm, PairGemm
 // x[M,K] * [mats]^T with the epilogue of `mode`; the caller has filled in the fields its mode uses.
 int run_gemm_pair(spec_ctx* c, int mode, const void* x, int M, int K, int n_mats, const void* const* mats, const int* rows,
                   PairGemmParams* w, int kind) {
-  StreamTmaps tm{};
+  PairTmaps tm{};
   w->M = M; w->KC = K / 64; w->n_mats = n_mats; w->packed = c->packed;
   const uint32_t box = mode == GP_SWIGLU ? 64 : 128;      // SwiGLU: 64 gate rows and 64 up rows make a CTA's tile
   int t0 = 0;
@@ -648,20 +699,25 @@ int run_gemm_pair(spec_ctx* c, int mode, const void* x, int M, int K, int n_mats
   for (int i = n_mats; i <= GS_MAX_MATS; ++i) w->mat_tile0[i] = t0;
   w->n_tiles = mode == GP_SWIGLU ? w->mat_tile0[1] : t0;
   w->w_pairs = mode == GP_SWIGLU ? w->n_tiles : (w->n_tiles + 1) / 2;
-  w->m_tiles = (M + GP_NT - 1) / GP_NT;
-  const CUtensorMap* tb = c->tmap(x, round_up(M, 16), K, GP_NT / 2);
+  const bool may_share = mode != GP_PLAIN && c->part_floats >= GP_PART_FLOATS;   // (a plain projection's sums go to the scratch)
+  plan_pair(w, mode, may_share);
+  w->part = c->d_part; w->arrive = c->d_pair_arrive;
+  const CUtensorMap* tb = c->tmap(x, round_up(M, 16), K, w->tile_rows / 2);
   if (!tb) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (activations)");
   tm.b = *tb;
+  if (w->cut > 1) {
+    if (!(tb = c->tmap(x, round_up(M, 16), K, w->tile_rows / w->cut / 2))) return c->fail(SPEC_E_CUDA, "cuTensorMapEncodeTiled failed (activations)");
+    tm.b_cut = *tb;
+  }
   w->status = c->d_status; w->trace = c->next_trace(gemm_kind_name(kind));
   cudaError_t e;
-  float* part = c->part_floats >= GP_PART_FLOATS ? c->d_part : nullptr;
   {
     ProfScope ps(c, kind);
     switch (mode) {
-      case GP_RESIDUAL: e = launch_gp<GP_RESIDUAL>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
-      case GP_SWIGLU: e = launch_gp<GP_SWIGLU>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
-      case GP_ROPE: e = launch_gp<GP_ROPE>(c->stream, c->pdl, tm, *w, part, c->d_pair_arrive); break;
-      default: e = launch_gp<GP_PLAIN>(c->stream, c->pdl, tm, *w, nullptr, nullptr); break;   // (its sums go to the scratch)
+      case GP_RESIDUAL: e = launch_gp<GP_RESIDUAL>(c->stream, c->pdl, tm, *w); break;
+      case GP_SWIGLU: e = launch_gp<GP_SWIGLU>(c->stream, c->pdl, tm, *w); break;
+      case GP_ROPE: e = launch_gp<GP_ROPE>(c->stream, c->pdl, tm, *w); break;
+      default: e = launch_gp<GP_PLAIN>(c->stream, c->pdl, tm, *w); break;
     }
     c->launches++;
   }
@@ -688,7 +744,7 @@ int run_gemm(spec_ctx* c, const void* x, int M, int K, int n_mats, const void* c
     // the consumers see one finished slot per tile: a dealing of the units with one CTA per (weight tile, activation tile)
     PartView v{};
     v.part = c->d_part; v.slot_stride = (size_t)M * tiles_all * 128; v.ld = tiles_all * 128;
-    v.seg.KC = K / 64; v.seg.m_tiles = w.m_tiles; v.seg.G = w.n_tiles * w.m_tiles; v.seg.total = (int)total;
+    v.seg.KC = K / 64; v.seg.m_tiles = (M + GP_NT - 1) / GP_NT; v.seg.G = w.n_tiles * v.seg.m_tiles; v.seg.total = (int)total;
     v.mt_shift = 8;
     v.single = 1;
     *view = v;
@@ -2231,13 +2287,15 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
     // With fewer than two tiles a CTA the streaming kernel is as fast (67 us against 65 in one case) and closer to the exact
     // result, since it cuts the inner dimension into several separately rounded sums where this kernel adds two.
     PairGemmParams p{};
-    if (!make_tmap(&tm.a[0], w, N, K, 128) || !make_tmap(&tm.b, x, M, K, GP_NT / 2)) return SPEC_E_CUDA;
+    PairTmaps pm{};
     p.M = M; p.KC = K / 64; p.n_mats = 1;
-    p.n_tiles = g.p.n_tiles; p.w_pairs = (g.p.n_tiles + 1) / 2; p.m_tiles = (M + GP_NT - 1) / GP_NT;
+    p.n_tiles = g.p.n_tiles; p.w_pairs = (g.p.n_tiles + 1) / 2;
+    plan_pair(&p, GP_PLAIN, false, std::max(1, ctas / 2));
+    if (!make_tmap(&pm.a[0], w, N, K, 128) || !make_tmap(&pm.b, x, M, K, p.tile_rows / 2) || (p.cut > 1 && !make_tmap(&pm.b_cut, x, M, K, p.tile_rows / p.cut / 2))) return SPEC_E_CUDA;
     for (int i = 1; i <= GS_MAX_MATS; ++i) p.mat_tile0[i] = p.n_tiles;
     p.out = y; p.ld = (size_t)N; p.n_cols = N;
     p.status = status.report(); p.clear = status.clear();
-    if (launch_gp<GP_PLAIN>(st, false, tm, p, nullptr, nullptr, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
+    if (launch_gp<GP_PLAIN>(st, false, pm, p, std::max(1, ctas / 2)) != cudaSuccess) return SPEC_E_CUDA;
     return status.finish();
   }
   const int cs = M <= 128 ? plain_cluster(g.p.n_tiles, K / 64, ctas) : 0;

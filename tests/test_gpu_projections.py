@@ -79,3 +79,36 @@ def test_gate_up_in_clusters_as_the_streamer(torch, d, ffn, T):
     assert np.isfinite(seen[7][1]).all() and np.abs(seen[7][1]).max() > 0.1
     for a, b in zip(seen[7], seen[5]):
         assert a.tobytes() == b.tobytes()
+
+
+@pytest.mark.parametrize("M,N,K,ctas", [
+    (1008, 11008, 512, 296), (1488, 5000, 256, 100),          # the last wave's tiles in halves, on 74 and on 50 pairs of SMs
+    (592, 19008, 256, 296), (2032, 9700, 128, 296),           # in quarters, the last of them without rows; columns that are no multiple of a tile
+    (2032, 4700, 2048, 296), (1040, 2600, 512, 40),           # tiles of 192 and of 208 rows, quarters of 16-row groups that do not divide
+    (144, 19000, 128, 296),                                   # a single tile of fewer rows than 256
+])
+def test_tile_heights(torch, M, N, K, ctas):
+    """Projections of many rows in tiles of other heights, and in slices of tiles."""
+    check_linear(torch, M, N, K, ctas)
+
+
+def test_rows_do_not_depend_on_the_tiles(torch):
+    """The same prompt three times in a pass of 384 rows, sixteen times in one of 2048 and ten times in one of 1280: q/k/v, output, gate+up and down go through tiles of 16
+    to 256 rows and through halves of tiles, and every sequence gets the same bits. (An inner dimension below 64 chunks: no tile is shared.)"""
+    import numpy as np
+    from paper_2503_14153_b200 import binding as B
+    from synthetic import get_config
+    prompt = np.random.default_rng(3).integers(0, 1000, 120).astype(np.int32)
+    first = None
+    for batch in (3, 16, 10):
+        cfg = get_config("c0", name="tiles", n_layers=3, d_model=1024, n_heads=16, n_kv_heads=4, head_dim=64, d_ffn=2752, vocab=1000, dtype="bf16", rope_base=1e6,
+                         n_medusa=4, topk=(10, 4, 2, 2), tree_nodes=4, batch=batch)
+        gpu = random_decoder(torch, cfg, 9, 140)
+        gpu.prefill([prompt] * batch)
+        h = gpu.debug(B.DBG_H_LAST)
+        kv = [np.stack(gpu.read_kv(b, l, 0, 120)) for b in (0, batch // 2, batch - 1) for l in (1, 2)]
+        gpu.close()
+        assert np.isfinite(h).all() and np.abs(h).max() > 0.1
+        first = (h[0], kv[0], kv[1]) if first is None else first
+        assert all((row == first[0]).all() for row in h)
+        assert all((a == first[1 + i % 2]).all() for i, a in enumerate(kv))
