@@ -135,9 +135,46 @@ gather_attention_ends(const int* __restrict__ end_pos, const bf16* __restrict__ 
     reinterpret_cast<uint4*>(attn_end + (size_t)g * HD)[c] = reinterpret_cast<const uint4*>(attn + m * HD)[c];
 }
 
-// Before prompts are processed: zeros in every cache slot that they do not fill, from the page of a sequence's first free slot on
-// (attention reads whole tiles of keys; what lies past a sequence's end has weight zero but must be finite). A sequence's pages
-// that its prompt fills are left alone: clearing the whole pool took 45 us for a 2048-token prompt and 8 layers of the 7B shape.
+// What prompt processing is told by the host, by value: a copy and a memset each for these few hundred ints, and the wait for them, took
+// 50 us before the first kernel of a prompt.
+constexpr int PS_SEQS = 32, PS_CHUNKS = 96;
+struct PrefillSetup {
+  int batch, max_batch, chunks;            // sequences, of which the context has room for, chunks of all prompts
+  int offsets[PS_SEQS + 1];                // first token of a sequence's prompt
+  int page_end[PS_SEQS];                   // of each of max_batch sequences: pages from here on are zero already
+  int chunk_seq[PS_CHUNKS], chunk_pos[PS_CHUNKS];
+  int ends[6 * PS_SEQS];                   // the tables of PromptEnds, batch entries each
+};
+struct PrefillTargets {
+  int *offsets, *chunk_seq, *chunk_pos, *ends, *status, *gen_cnt, *draws;
+  unsigned int *pair_arrive, *item_counter;
+  int n_arrive;
+};
+
+// Before prompts are processed. The first CTA writes the tables and clears the counters (a wait that ran out may have left some set). All of them: zeros
+// in every cache slot that the prompts do not fill, from the page of a sequence's first free slot on, as far as earlier sequences have written
+// (attention reads whole tiles of keys; what lies past a sequence's end has weight zero but must be finite). On the 7B shape clearing the whole pool took
+// 45 us for a 2048-token prompt and 8 layers, and all free pages 55 us for eight prompts of up to 1024 tokens and 4 layers.
+__global__ void __launch_bounds__(256)
+prefill_setup(const __grid_constant__ PrefillSetup s, const PrefillTargets to, uint4* __restrict__ pool, int pages_per_seq, int page_size, int pair_vecs, int share) {
+  const int tid = threadIdx.x;
+  if (to.status && blockIdx.x + blockIdx.y == 0) {
+    if (tid < 4) to.status[tid] = 0;
+    if (tid == 0) *to.item_counter = 0u;
+    for (int i = tid; i < to.n_arrive; i += 256) to.pair_arrive[i] = 0u;
+    for (int i = tid; i < s.batch; i += 256) { to.gen_cnt[i] = 0; to.draws[i] = 0; }
+    for (int i = tid; i <= s.batch; i += 256) to.offsets[i] = s.offsets[i];
+    for (int i = tid; i < s.chunks; i += 256) { to.chunk_seq[i] = s.chunk_seq[i]; to.chunk_pos[i] = s.chunk_pos[i]; }
+    for (int i = tid; i < 6 * s.batch; i += 256) to.ends[i] = s.ends[i];
+  }
+  // grid (sequences times the CTAs that share one's pages, layers * heads); pool page p * max_batch + b is page p of sequence b
+  const int b = blockIdx.x / share, len = b < s.batch ? s.offsets[b + 1] - s.offsets[b] : 0, end = s.page_end[b];
+  uint4* base = pool + ((size_t)blockIdx.y * pages_per_seq * s.max_batch + b) * pair_vecs;
+  for (int p = len / page_size + blockIdx.x % share; p < end; p += share)
+    for (int i = tid; i < pair_vecs; i += 256) base[(size_t)p * s.max_batch * pair_vecs + i] = make_uint4(0, 0, 0, 0);
+}
+
+// The same for more sequences or chunks than that holds, without the tables: all free pages.
 __global__ void __launch_bounds__(256)
 clear_free_pages(uint4* __restrict__ pool, const int* __restrict__ offsets, int batch, int pages_per_seq, int max_batch, int page_size,
                  int pair_vecs, int share, unsigned int* __restrict__ item_counter) {
@@ -720,6 +757,8 @@ struct AcceptArgs {
   const int *parent, *depth;   // tree arrays [R]
   const int* edge_ok;          // typical mode: per-row pass flag; NULL = greedy token match
   int K, frag_token, d, mode;  // mode 0 = verify step, 1 = prefill (row b is sequence b)
+  const int* status;           // mode 1: the status word, which goes to host_status in pinned host memory
+  int* host_status;
   const float* hid;            // [rows][d]
   int *am, *path, *count, *out_tok, *n_old, *root_tok;
   float* h_last;
@@ -745,6 +784,7 @@ __global__ void __launch_bounds__(256) accept_kernel(AcceptArgs a, unsigned long
       a.am[b] = a.root_tok[b] = a.pidx[b];
       a.gen_cnt[b] = 0;
     }
+    if (b == 0 && threadIdx.x < 4) a.host_status[threadIdx.x] = a.status[threadIdx.x];
     return;
   }
   const int cnt = a.rows.cnt[b], m0 = b * R;

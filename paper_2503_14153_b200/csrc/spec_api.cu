@@ -267,6 +267,7 @@ struct spec_ctx {
   int small_gemm_ctas = 288;           // CTAs of GEMMs with at most 48 weight tiles (Wo, down); 288 since the weights are pre-tiled (192 before)
   std::vector<int> h_parent, h_depth, h_rank;
   std::vector<int> n_hi, n_lo;         // host upper / lower bounds of the committed lengths
+  std::vector<int> written;            // [max_batch] cache slots from here on hold zeros (nothing is known of a new workspace)
   std::vector<const void*> wq, wk, wv, wo, wg, wu, wd, mw, mb;
   std::vector<const float*> an, fn;
   const void *embed, *lm_head;
@@ -1524,6 +1525,7 @@ AcceptArgs make_accept(spec_ctx* c, int R, int mode) {
   a.hid = c->d_hid; a.am = c->d_am; a.path = c->d_path; a.count = c->d_count; a.out_tok = c->d_out_tok;
   a.n_old = c->d_n_old; a.root_tok = c->d_root; a.h_last = c->d_h_last;
   a.gen_log = c->d_gen_log; a.gen_cnt = c->d_gen_cnt; a.gen_cap = c->gen_cap;
+  a.status = c->d_status; a.host_status = c->h_result_dev;
   return a;
 }
 
@@ -1557,20 +1559,9 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   c->prefills++;      // a recorded step stays valid while its plan covers the new sequences (step_t looks)
   std::vector<int> off(batch + 1);
   for (int b = 0; b <= batch; ++b) off[b] = offsets[b] - offsets[0];
-  CUDA_OK(cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), c->stream));
-  CUDA_OK(cudaMemcpyAsync(c->d_prompt, tokens + offsets[0], (size_t)off[batch] * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CUDA_OK(cudaMemcpyAsync(c->d_offsets, off.data(), (batch + 1) * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  {
-    const int pair_vecs = (int)(c->geom.block_elems() * 2 * c->esz / 16);   // 16-byte vectors of a page's K and V of one layer and head
-    const int lh = f.n_layers * f.n_kv_heads, share = (int)std::max<long long>(1, std::min<long long>(c->pages_per_seq, 8 * SM_SLOTS / ((long long)lh * f.max_batch)));
-    for (int lh0 = 0; lh0 < lh; lh0 += 65535)
-      clear_free_pages<<<dim3((unsigned)share * (unsigned)f.max_batch, (unsigned)std::min(65535, lh - lh0)), 256, 0, c->stream>>>(
-          static_cast<uint4*>(c->d_pool) + (size_t)lh0 * c->geom.pool_pages() * pair_vecs, c->d_offsets, batch, c->pages_per_seq, f.max_batch, f.page_size, pair_vecs, share, c->d_attn_arrive);
-    LAUNCH_CHECK("clear_free_pages");
-  }
-  CUDA_OK(cudaMemsetAsync(c->d_pair_arrive, 0, GP_ARRIVE * sizeof(unsigned int), c->stream));   // (a wait that ran out may have left some set)
-  CUDA_OK(cudaMemsetAsync(c->d_gen_cnt, 0, batch * sizeof(int), c->stream));
-  CUDA_OK(cudaMemsetAsync(c->d_draws, 0, batch * sizeof(int), c->stream));
+  // (an error on the way leaves it open what has been written)
+  const std::vector<int> before = c->written;
+  c->written.assign(f.max_batch, c->cap);
   // The prompts are cut into chunks of R tokens and the chunks of all prompts, one prompt after another, are dealt to as
   // few passes as the row buffers allow, evenly. A chunk sees the chunks before it in the cache whether they belong to an
   // earlier pass or to this one: a layer stores the keys and values of all its rows before its attention starts.
@@ -1588,8 +1579,6 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   // of 7.1 when both forms were measured). Nothing more is promised: prompts of more chunks, and any prompt processed together with
   // others, take the many-row projections, whose order of sums is another one (and, up to 512 rows, depends on the rows).
   const int passes = batch == 1 && chunks == 2 ? 2 : (chunks + cap - 1) / cap;
-  CUDA_OK(cudaMemcpyAsync(c->d_chunk_seq, cseq.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CUDA_OK(cudaMemcpyAsync(c->d_chunk_pos, cpos.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   // the prompts' last rows, by sequence (the edge flags of the acceptance step are not in use while prompts are processed)
   static_assert(PREFILL_ROWS >= 6, "a place of the edge flags a table entry");
   std::vector<int> ends(6 * (size_t)batch);
@@ -1607,8 +1596,46 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
     }
     ch += g;
   }
-  if (c->tc) CUDA_OK(cudaMemcpyAsync(c->d_edge, ends.data(), ends.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CUDA_OK(cudaStreamSynchronize(c->stream));   // the host staging vectors go out of scope
+  CUDA_OK(cudaMemcpyAsync(c->d_prompt, tokens + offsets[0], (size_t)off[batch] * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  const int pair_vecs = (int)(c->geom.block_elems() * 2 * c->esz / 16);   // 16-byte vectors of a page's K and V of one layer and head
+  const int lh = f.n_layers * f.n_kv_heads, most_share = (int)std::max<long long>(1, std::min<long long>(c->pages_per_seq, 8 * SM_SLOTS / ((long long)lh * f.max_batch)));
+  uint4* pool = static_cast<uint4*>(c->d_pool);
+  const size_t lh_vecs = c->geom.pool_pages() * pair_vecs;
+  if (f.max_batch <= PS_SEQS && chunks <= PS_CHUNKS) {
+    PrefillSetup ps{};
+    ps.batch = batch; ps.max_batch = f.max_batch; ps.chunks = chunks;
+    int pages = 1;                                             // most that a sequence has to clear
+    for (int b = 0; b < f.max_batch; ++b) {
+      ps.page_end[b] = std::min(c->pages_per_seq, (before[b] + f.page_size - 1) / f.page_size);
+      pages = std::max(pages, ps.page_end[b] - (b < batch ? (off[b + 1] - off[b]) / f.page_size : 0));
+    }
+    std::copy(off.begin(), off.end(), ps.offsets);
+    std::copy(cseq.begin(), cseq.end(), ps.chunk_seq);
+    std::copy(cpos.begin(), cpos.end(), ps.chunk_pos);
+    std::copy(ends.begin(), ends.end(), ps.ends);
+    PrefillTargets to{c->d_offsets, c->d_chunk_seq, c->d_chunk_pos, c->d_edge, c->d_status, c->d_gen_cnt, c->d_draws, c->d_pair_arrive, c->d_attn_arrive, GP_ARRIVE};
+    const int share = std::min(most_share, pages);
+    for (int lh0 = 0; lh0 < lh; lh0 += 65535) {
+      prefill_setup<<<dim3((unsigned)share * (unsigned)f.max_batch, (unsigned)std::min(65535, lh - lh0)), 256, 0, c->stream>>>(
+          ps, to, pool + (size_t)lh0 * lh_vecs, c->pages_per_seq, f.page_size, pair_vecs, share);
+      to.status = nullptr;                                     // (the tables are written)
+      LAUNCH_CHECK("prefill_setup");
+    }
+  } else {
+    CUDA_OK(cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), c->stream));
+    CUDA_OK(cudaMemcpyAsync(c->d_offsets, off.data(), (batch + 1) * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    for (int lh0 = 0; lh0 < lh; lh0 += 65535)
+      clear_free_pages<<<dim3((unsigned)most_share * (unsigned)f.max_batch, (unsigned)std::min(65535, lh - lh0)), 256, 0, c->stream>>>(
+          pool + (size_t)lh0 * lh_vecs, c->d_offsets, batch, c->pages_per_seq, f.max_batch, f.page_size, pair_vecs, most_share, c->d_attn_arrive);
+    LAUNCH_CHECK("clear_free_pages");
+    CUDA_OK(cudaMemsetAsync(c->d_pair_arrive, 0, GP_ARRIVE * sizeof(unsigned int), c->stream));
+    CUDA_OK(cudaMemsetAsync(c->d_gen_cnt, 0, batch * sizeof(int), c->stream));
+    CUDA_OK(cudaMemsetAsync(c->d_draws, 0, batch * sizeof(int), c->stream));
+    CUDA_OK(cudaMemcpyAsync(c->d_chunk_seq, cseq.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    CUDA_OK(cudaMemcpyAsync(c->d_chunk_pos, cpos.data(), chunks * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    CUDA_OK(cudaMemcpyAsync(c->d_edge, ends.data(), ends.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    CUDA_OK(cudaStreamSynchronize(c->stream));   // the host staging vectors go out of scope
+  }
   for (int pass = 0, ch = 0; pass < passes; ++pass) {
     const int g = (chunks - ch + passes - pass - 1) / (passes - pass);    // chunks of this pass
     pe.seq0 += pe.count;
@@ -1637,8 +1664,10 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
     KLAUNCH("sample_root", sample_root, dim3(SAMPLE_CLUSTER, batch), dim3(SAMPLE_THREADS), 0, (const float*)c->d_logits, (const float*)c->d_pval2, f.vocab, 1, c->K,
             (const int*)c->d_path, (const int*)c->d_count, f.temperature, f.seed_lo, f.seed_hi, c->d_draws, c->d_root, 1);
   }
-  r = check_status(c);
-  if (r) return r;
+  // (accept_kernel has put the status word into host memory)
+  CUDA_OK(cudaStreamSynchronize(c->stream));
+  if ((r = report_status(c, c->h_result))) return r;
+  for (int b = 0; b < f.max_batch; ++b) c->written[b] = b < batch ? off[b + 1] - off[b] : 0;
   c->n_hi.assign(batch, 0);
   for (int b = 0; b < batch; ++b) c->n_hi[b] = offsets[b + 1] - offsets[b];
   c->n_lo = c->n_hi;
@@ -1738,6 +1767,7 @@ int step_t(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t*
     CUDA_OK(cudaMemcpyAsync(c->d_cand_ov, cand_override, (size_t)B * K * kmax * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     ov = c->d_cand_ov;
   }
+  for (int b = 0; b < B; ++b) c->written[b] = std::max(c->written[b], std::min(c->cap, c->n_hi[b] + T_));
   // (the kernels take the lengths themselves from the device, so a recorded step serves every length below its bounds)
   std::vector<int> n_hi_plan(B), n_lo_plan(B);
   for (int b = 0; b < B; ++b) n_hi_plan[b] = attn_plan_bound(c, T_, B, c->n_hi[b] + T_) - T_;
@@ -1881,6 +1911,7 @@ int spec_create(const spec_config* cfg, const spec_weights* w, const spec_tree* 
   while (need > workspace_bytes && chunks > cfg->max_batch) need = carve(c, workspace, --chunks, true);
   if (need > workspace_bytes) need = carve(c, workspace, chunks, false);
   if (need > workspace_bytes) { g_create_error = "workspace too small"; delete c; return SPEC_E_NOMEM; }
+  c->written.assign(cfg->max_batch, c->cap);
   c->h_parent.assign(tree->parent, tree->parent + c->T);
   c->h_depth.assign(tree->depth, tree->depth + c->T);
   c->h_rank.assign(tree->rank, tree->rank + c->T);

@@ -1,0 +1,55 @@
+"""What prompt processing sets up: tables, counters and the free part of the cache."""
+import numpy as np
+import pytest
+
+from synthetic import get_config
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,max_batch,rounds", [
+    ("bf16", 1, [[300], [20], [170]]),                        # long, then short: what the first left is cleared; two chunks
+    ("bf16", 3, [[100, 31, 260], [16, 5], [40, 50, 7]]),      # a sequence less, and again as many
+    ("fp32", 2, [[90, 40], [12], [33, 60]]),
+    ("bf16", 33, [[9] * 33, [30] * 20]),                      # more sequences than the tables by value hold
+    ("bf16", 1, [[12400], [12300]]),                          # more chunks than they hold
+])
+def test_nothing_left_of_earlier_prompts(dtype, max_batch, rounds):
+    """Prompts after other prompts and steps: first tokens, hidden states and steps as on a fresh context, and zeros in the cache from the page of the
+    first free slot on."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    from synthetic import draw_weights
+    cfg = get_config("c0", name="setup", n_layers=2, d_model=256, n_heads=4, n_kv_heads=2, head_dim=64, d_ffn=704, vocab=1000, dtype=dtype, rope_base=1e6,
+                     n_medusa=3, topk=(4, 2, 2), tree_nodes=9, seed=3)
+    dw = upload_weights(cfg, draw_weights(cfg))
+    tree = build_tree(cfg.topk, 9)
+    room = max(max(r) for r in rounds) + 40
+    rng = np.random.default_rng(1)
+
+    def results(dec, prompts):
+        dec.prefill(prompts)
+        out = [dec.debug(B.DBG_NEXT_ROOT), dec.debug(B.DBG_H_LAST)]
+        for b, p in enumerate(prompts):
+            free = (len(p) + cfg.page_size - 1) // cfg.page_size * cfg.page_size
+            for kv in dec.read_kv(b, 1, free, min(room, free + 400) - free):
+                assert not kv.any()
+        if len(prompts) < dec.max_batch:
+            assert not any(kv.any() for kv in dec.read_kv(dec.max_batch - 1, 0, 0, min(room, 300)))
+        for _ in range(2):
+            t, n = dec.step()
+            out += [n, np.where(np.arange(t.shape[1]) < n[:, None], t, -1)]
+        return out
+
+    used = SpecDecoder(cfg, dw, tree, room, max_batch=max_batch)
+    for lens in rounds:
+        prompts = [rng.integers(0, cfg.vocab, n).astype(np.int32) for n in lens]
+        fresh = SpecDecoder(cfg, dw, tree, room, max_batch=max_batch)
+        a, b = results(used, prompts), results(fresh, prompts)
+        fresh.close()
+        for x, y in zip(a, b):
+            assert x.tobytes() == y.tobytes()
+    used.close()
