@@ -2384,9 +2384,11 @@ int spec_build_labels(const int32_t* tokens, int32_t n_seq, int32_t seq_len, int
   if (n_seq == 0 || seq_len == 0) return SPEC_OK;
   if (!tokens || !labels || n_seq < 0 || seq_len < 0 || num_heads < 0 || num_heads > LABEL_MAX_HEADS || n_seq > 65535)
     return SPEC_E_BADARG;
-  dim3 grid((seq_len + LABEL_THREADS - 1) / LABEL_THREADS, n_seq);
-  build_labels_kernel<<<grid, LABEL_THREADS, 0, static_cast<cudaStream_t>(cuda_stream)>>>(tokens, seq_len, num_heads, frag_token,
-                                                                                        pad_token, ignore_token, labels);
+  const bool vec = seq_len % 4 == 0 && (reinterpret_cast<uintptr_t>(labels) & 15) == 0;
+  const int threads = vec ? LABEL_VEC_THREADS : LABEL_THREADS, cols = vec ? LABEL_VEC_COLS : LABEL_THREADS;
+  auto kernel = vec ? build_labels_vec : build_labels_kernel;
+  kernel<<<dim3((seq_len + cols - 1) / cols, n_seq), threads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(tokens, seq_len, num_heads, frag_token, pad_token,
+                                                                                                        ignore_token, labels);
   return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_E_CUDA;
 }
 
