@@ -5,6 +5,7 @@ decode loop runs inside the shared library's CUDA kernels. There is no CPU fallb
 library is missing, loading raises.
 """
 import ctypes as C
+import functools
 import os
 from typing import Dict, List, Optional, Sequence
 
@@ -127,6 +128,20 @@ def load_library():
     lib.spec_profile_read.argtypes = [C.c_void_p, C.POINTER(C.c_double), C.POINTER(C.c_int64)]
     _lib = lib
     return lib
+
+
+@functools.lru_cache(maxsize=1)
+def _torch():
+    """(torch, a function that gives the current stream of a CUDA device ordinal as a number). The stream without a Stream object around it
+    takes 0.1 us instead of 2 of a call that launches one kernel."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return torch, raw if raw is not None else lambda index: torch.cuda.current_stream(index).cuda_stream
+
+
+@functools.lru_cache(maxsize=1024)
+def _op_linear_scratch(M: int, N: int, K: int, ctas: int) -> int:
+    return int(load_library().spec_op_linear_scratch_floats(M, N, K, ctas))
 
 
 def _i32ptr(a: np.ndarray):
@@ -279,9 +294,11 @@ class SpecDecoder:
             raise SpecError(rc, self.lib.spec_last_error(None).decode())
         self.kmax = int(self.lib.spec_query(self._ctx, Q_KMAX))
         self.batch = max_batch
-        self._out_tok = torch.empty((max_batch, self.K + 1), dtype=torch.int32).pin_memory()
-        self._out_cnt = torch.empty((max_batch,), dtype=torch.int32).pin_memory()
+        self._out_tok = np.empty((max_batch, self.K + 1), dtype=np.int32)
+        self._out_cnt = np.empty((max_batch,), dtype=np.int32)
+        self._out_ptrs = self._out_tok.ctypes.data, self._out_cnt.ctypes.data
         self._ov = torch.empty((max_batch, max(self.K, 1), self.kmax), dtype=torch.int32).pin_memory()
+        self._ov_np, self._ov_ptr = self._ov.numpy(), self._ov.data_ptr()
 
     def _check(self, rc: int):
         if rc != 0:
@@ -312,11 +329,12 @@ class SpecDecoder:
         """One synchronous step; returns (tokens [batch][K+1] int32, counts [batch])."""
         ov = None
         if cand_override is not None:
-            self._ov[: self.batch].copy_(self.torch.from_numpy(
-                np.ascontiguousarray(cand_override, dtype=np.int32).reshape(self.batch, self.K, self.kmax)))
-            ov = self._ov.data_ptr()
-        self._check(self.lib.spec_step(self._ctx, self._out_tok.data_ptr(), self._out_cnt.data_ptr(), ov))
-        return self._out_tok[: self.batch].numpy().copy(), self._out_cnt[: self.batch].numpy().copy()
+            self._ov_np[: self.batch] = np.asarray(cand_override, dtype=np.int32).reshape(self.batch, self.K, self.kmax)
+            ov = self._ov_ptr
+        rc = self.lib.spec_step(self._ctx, *self._out_ptrs, ov)
+        if rc != 0:
+            self._check(rc)
+        return self._out_tok[: self.batch].copy(), self._out_cnt[: self.batch].copy()
 
     def step_async(self):
         """Enqueue one step on the stream without host synchronisation."""
@@ -381,7 +399,7 @@ class SpecDecoder:
                   DBG_NEXT_ROOT: ((self.batch,), np.int32), DBG_H_LAST: ((self.batch, self.cfg.d_model), np.float32),
                   DBG_STATUS: ((4,), np.int32)}
         shape, dt = shapes[what]
-        buf = np.zeros(shape, dtype=dt)
+        buf = np.empty(shape, dtype=dt)                      # (the call fills all of it or fails)
         self._check(self.lib.spec_debug_read(self._ctx, what, buf.ctypes.data, buf.nbytes))
         return buf
 
@@ -394,21 +412,21 @@ class SpecDecoder:
 
 def spec_op_linear(x, w, ctas: int = 296):
     """y = x @ w.T through the library's linear kernel (x, w: CUDA tensors, float32 or bf16)."""
-    import torch
-    lib = load_library()
+    torch, raw_stream = _torch()
+    lib = _lib or load_library()
     M, K = x.shape
     N = w.shape[0]
+    device = x.device
     dtype = 1 if x.dtype == torch.bfloat16 else 0
-    y = torch.empty((M, N), dtype=torch.float32, device=x.device)
+    y = torch.empty((M, N), dtype=torch.float32, device=device)
     scratch = None
     if dtype == 1:
-        need = int(lib.spec_op_linear_scratch_floats(M, N, K, ctas))
+        need = _op_linear_scratch(M, N, K, ctas)
         if need == 0:
             raise SpecError(-1, "spec_op_linear_scratch_floats rejected the shape")
-        scratch = torch.empty(need + 4, dtype=torch.float32, device=x.device)
+        scratch = torch.empty(need + 4, dtype=torch.float32, device=device)
     rc = lib.spec_op_linear(dtype, x.data_ptr(), w.data_ptr(), y.data_ptr(), M, N, K, ctas,
-                            scratch.data_ptr() if scratch is not None else None,
-                            torch.cuda.current_stream(x.device).cuda_stream)
+                            scratch.data_ptr() if scratch is not None else None, raw_stream(device.index))
     if rc != 0:
         raise SpecError(rc, "spec_op_linear failed")
     return y
@@ -416,12 +434,12 @@ def spec_op_linear(x, w, ctas: int = 296):
 
 def spec_build_labels(tokens, num_heads: int, frag: int, pad: int, ignore: int):
     """tokens: CUDA int32 tensor [n_seq, seq_len] -> labels [n_seq, num_heads + 1, seq_len] (Sec. III-C)."""
-    import torch
-    lib = load_library()
+    torch, raw_stream = _torch()
+    lib = _lib or load_library()
     n_seq, seq_len = tokens.shape
-    labels = torch.empty((n_seq, num_heads + 1, seq_len), dtype=torch.int32, device=tokens.device)
-    rc = lib.spec_build_labels(tokens.data_ptr(), n_seq, seq_len, num_heads, frag, pad, ignore, labels.data_ptr(),
-                               torch.cuda.current_stream(tokens.device).cuda_stream)
+    device = tokens.device
+    labels = torch.empty((n_seq, num_heads + 1, seq_len), dtype=torch.int32, device=device)
+    rc = lib.spec_build_labels(tokens.data_ptr(), n_seq, seq_len, num_heads, frag, pad, ignore, labels.data_ptr(), raw_stream(device.index))
     if rc != 0:
         raise SpecError(rc, "spec_build_labels failed")
     return labels
