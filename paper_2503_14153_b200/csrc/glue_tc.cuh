@@ -590,6 +590,117 @@ topk_slices_tc(const PartView pv, int V, int row0, int slice, int kmax, float* p
   topk_merge_row(pk_val, pk_idx, (int)gridDim.x, row, K, kmax, root_tok, cand_override, cand, zs);
 }
 
+// Per-head top-k where the projection left each row's largest in every tile of 128 tokens (best_val / best_idx [row][tiles]) beside the logits: the
+// kmax best lie in tiles whose largest is among the kmax best of those, so a CTA a row reads the maxima and a dozen tiles instead of the vocabulary.
+// Of the maxima of up to 64 groups of tiles (kmax or more of them) the kmax-th largest is a bound that kmax values reach; what reaches it in the tiles that do is
+// ranked (order: value descending, index ascending; NaN never wins). Where more than TOPK_CAP values reach it (many equal ones), kmax
+// rounds over those tiles decide. 4 heads over 32016 tokens: 9.6 us of topk_slices_tc -> 4.1; 64 rows: 22.3 -> 5.2.
+constexpr int TOPK_MAX_TILES = 512;                          // (and at least kmax)
+__global__ void __launch_bounds__(256)
+topk_tiles(const float* __restrict__ z, int ldz, const float* __restrict__ best_val, const int* __restrict__ best_idx, int tiles, int V, int kmax, int K,
+           const int* __restrict__ root_tok, const int* __restrict__ cand_override, int* __restrict__ cand, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  constexpr int NONE = 0x7fffffff, PER = TOPK_MAX_TILES / 256;
+  __shared__ float gv[64], cv[TOPK_CAP];
+  __shared__ int gi[64], ci[TOPK_CAP], list[TOPK_MAX_TILES];
+  __shared__ float tau_v;
+  __shared__ int tau_i, n_list, count;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, row = blockIdx.x, b = row / K, k = row % K;
+  int* out = cand + ((size_t)b * (K + 1) + k + 1) * kmax;
+  const int* ovr = cand_override ? cand_override + ((size_t)b * K + k) * kmax : nullptr;
+  auto emit = [&](int t, int i) {
+    const int o = ovr ? ovr[t] : -1, tok = o >= 0 ? o : i;
+    out[t] = tok == NONE ? 0 : tok;
+  };
+  if (tid == 0) { tau_v = -INFINITY; tau_i = NONE - 1; n_list = count = 0; }   // fewer than kmax groups hold a value: all values pass
+  pdl_wait();
+  if (tid == 0) trace_mark_min(tr, 2);
+  if (k == 0 && tid == 0) cand[(size_t)b * (K + 1) * kmax] = root_tok[b];
+  float tv[PER];
+  int ti[PER];
+  float bv = -INFINITY; int bi = NONE;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int t = tid + j * 256;
+    tv[j] = t < tiles ? __ldcg(best_val + (size_t)row * tiles + t) : -INFINITY;
+    ti[j] = t < tiles ? __ldcg(best_idx + (size_t)row * tiles + t) : NONE;
+    if (better(tv[j], ti[j], bv, bi)) { bv = tv[j]; bi = ti[j]; }
+  }
+  if (tiles <= 64) {
+    if (tid < 64) { gv[tid] = bv; gi[tid] = bi; }            // (a group a tile)
+  } else {
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (better(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+    }
+    if ((tid & 3) == 0) { gv[tid >> 2] = bv; gi[tid >> 2] = bi; }
+  }
+  __syncthreads();
+  if (tid < 64 && gi[tid] != NONE) {
+    const float x = gv[tid]; const int i = gi[tid];
+    int rank = 0;
+#pragma unroll 16
+    for (int j = 0; j < 64; ++j) rank += better(gv[j], gi[j], x, i) ? 1 : 0;
+    if (rank == kmax - 1) { tau_v = x; tau_i = i; }
+  }
+  __syncthreads();
+  const float bound = tau_v; const int bound_i = tau_i;
+  auto reaches = [&](float x, int i) { return x >= bound && i != NONE && !better(bound, bound_i, x, i); };
+#pragma unroll
+  for (int j = 0; j < PER; ++j)
+    if (reaches(tv[j], ti[j])) list[atomicAdd(&n_list, 1)] = tid + j * 256;
+  __syncthreads();
+  const int nl = n_list;
+  const float* zr = z + (size_t)row * ldz;
+  for (int l = warp; l < nl; l += 8) {
+    const int n0 = list[l] * 128 + lane * 4;
+    float x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = -INFINITY;
+    if (n0 < ldz) { const float4 v = __ldcg(reinterpret_cast<const float4*>(zr + n0)); x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }   // (ldz % 4 == 0)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (n0 + j < V && reaches(x[j], n0 + j)) {
+        const int at = atomicAdd(&count, 1);
+        if (at < TOPK_CAP) { cv[at] = x[j]; ci[at] = n0 + j; }
+      }
+  }
+  __syncthreads();
+  const int nc = count;
+  if (nc <= TOPK_CAP) {
+    if (tid < nc) {
+      const float x = cv[tid]; const int i = ci[tid];
+      int rank = 0;
+      for (int j = 0; j < nc; ++j) rank += better(cv[j], ci[j], x, i) ? 1 : 0;
+      if (rank < kmax) emit(rank, i);
+    }
+    if (tid >= nc && tid < kmax) emit(tid, NONE);
+    return;
+  }
+  // many equal values: kmax rounds, each the best below the one before
+  float pv = INFINITY; int pi = -1;
+  for (int t = 0; t < kmax; ++t) {
+    bv = -INFINITY; bi = NONE;
+    for (int c = tid; c < nl * 128; c += 256) {
+      const int n = list[c >> 7] * 128 + (c & 127);
+      if (n >= V) continue;
+      const float x = __ldcg(zr + n);
+      if (better(pv, pi, x, n) && better(x, n, bv, bi)) { bv = x; bi = n; }
+    }
+    warp_argmax(bv, bi);
+    __syncthreads();                                         // (cv / ci of the round before have been read)
+    if (lane == 0) { cv[warp] = bv; ci[warp] = bi; }
+    __syncthreads();
+    bv = cv[0]; bi = ci[0];
+    for (int w = 1; w < 8; ++w) if (better(cv[w], ci[w], bv, bi)) { bv = cv[w]; bi = ci[w]; }
+    if (tid == 0) emit(t, bi);
+    pv = bv; pi = bi;
+  }
+}
+
 // y[m][n] = sum of the partial slots (logical columns of a single matrix): the stand-alone linear. clear: four ints set to zero, or nullptr.
 __global__ void __launch_bounds__(256)
 part_sum_rows(const PartView pv, float* __restrict__ y, int M, int N, int* __restrict__ clear) {

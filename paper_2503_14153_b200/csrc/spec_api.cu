@@ -1460,8 +1460,18 @@ int heads_tc(spec_ctx* c, const int* ov) {
   PartView pl{};
   if (const int cs = lm_head_cluster(c, rows_total)) {
     const int ldz = (int)round_up(f.vocab, 4);                  // (fits: partial sums of this shape would be rows of whole tiles)
-    int r = run_lm_head(c, c->d_r, rows_total, cs, c->d_part, ldz, nullptr, nullptr);
+    const int tiles = (f.vocab + 127) / 128;
+    // (the logits and behind them the tiles' maxima: partial sums of this shape would be rows of whole tiles, in two slots at least)
+    float* val = c->d_part + (size_t)rows_total * ldz;
+    int* idx = reinterpret_cast<int*>(val + (size_t)rows_total * tiles);
+    const bool maxima = tiles >= c->kmax && tiles <= TOPK_MAX_TILES && (size_t)rows_total * (ldz + 2 * (size_t)tiles) <= c->part_floats;
+    int r = run_lm_head(c, c->d_r, rows_total, cs, c->d_part, ldz, maxima ? val : nullptr, maxima ? idx : nullptr);
     if (r) return r;
+    if (maxima) {
+      KLAUNCH("topk_tiles", topk_tiles, dim3(rows_total), dim3(256), 0, (const float*)c->d_part, ldz, (const float*)val, (const int*)idx, tiles, f.vocab, c->kmax, K,
+              (const int*)c->d_root, ov, c->d_cand);
+      return SPEC_OK;
+    }
     pl = plain_view(c->d_part, rows_total, ldz);
   } else {
     const void* mats[1] = {c->lm_head};

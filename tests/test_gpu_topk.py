@@ -1,0 +1,43 @@
+"""Candidate lists out of the tiles' maxima, against the heads' logits in 64 bits."""
+import numpy as np
+import pytest
+
+from synthetic import draw_prompt, draw_weights, get_config
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("vocab,batch,kmax", [
+    (1160, 1, 10), (1290, 3, 10),             # ten and eleven tiles for ten candidates
+    (1000, 1, 10),                            # too few tiles: the slices' kernel
+    (8192, 2, 16), (8200, 2, 16),             # the most tiles that are groups of their own, and one more
+    (32016, 16, 1), (32017, 5, 3), (37888, 1, 16),
+])
+def test_candidates(vocab, batch, kmax):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = get_config("c0", name="topk", dtype="bf16", vocab=vocab, d_ffn=704, n_heads=2, n_kv_heads=2, head_dim=128, n_medusa=1, topk=(kmax,), tree_nodes=kmax + 1, seed=6)
+    w = draw_weights(cfg)
+    dec = SpecDecoder(cfg, upload_weights(cfg, w), build_tree(cfg.topk, kmax + 1), 64, max_batch=batch)
+    dec.prefill([draw_prompt(cfg.with_(seed=30 + b), 5 + b) for b in range(batch)])
+    h = torch.from_numpy(dec.debug(B.DBG_H_LAST)).bfloat16().double()
+    dec.step()
+    cand = dec.debug(B.DBG_CAND)
+    assert dec.kmax == kmax
+    dec.close()
+
+    def operand(a):
+        return torch.from_numpy(np.ascontiguousarray(a)).bfloat16().double()
+    r = (h + torch.nn.functional.silu(h @ operand(w["medusa.0.w"]).T + operand(w["medusa.0.b"]))).bfloat16().double()
+    z = (r @ operand(w["lm_head"]).T).numpy()
+    for b in range(batch):
+        got = cand[b, 1]
+        assert len(set(got.tolist())) == kmax
+        # (a rounding of r that falls the other way moves a logit by 2^-9 of one of its 256 products)
+        tol = 2.0 ** -8 * np.abs(z[b]).max() / 16
+        picked = z[b][got]
+        assert (np.diff(picked) <= tol).all()
+        assert np.delete(z[b], got).max() <= picked[-1] + tol
