@@ -59,6 +59,10 @@
 namespace spec {
 
 constexpr int GP_PLAIN = 0, GP_RESIDUAL = 1, GP_SWIGLU = 2, GP_ROPE = 3;
+// How a launch's sums are made: GP_WHOLE, an element's inner dimension in one run (GP_PLAIN: in halves); GP_SHARED, a tile's chunks on several clusters;
+// GP_RUNS, in the runs and in the order in which the projections of up to 128 rows add it up, a run an accumulator: a prompt of two chunks in one
+// pass over the weights, with the sums of the two passes that it took.
+constexpr int GP_WHOLE = 0, GP_SHARED = 1, GP_RUNS = 2;
 constexpr int GP_EPI = 512, GP_THREADS = 64 + GP_EPI;   // producer, MMA issuer, sixteen epilogue warps (four per SM quarter)
 constexpr int GP_QUARTERS = 4;                          // parts of a tile's activation rows that the epilogue warps share out
 
@@ -70,6 +74,8 @@ struct PairGemmParams {
   int tile_rows;                            // activation rows of a tile: a multiple of 16, at most NT (parts > 1: NT)
   int cut_first, cut;                       // tiles from cut_first on are done as `cut` slices of tile_rows / cut activation rows each (a multiple of 16)
   int stages;                               // of the ring
+  int runs, run_bufs;                       // GP_RUNS: accumulators of an item, at most, and items whose accumulators tensor memory holds (1 or 2)
+  SegMap seg;                               // GP_RUNS, GP_SWIGLU: how the weight streamer deals the stacked gate and up tiles' chunks out
   int plan_tiles;                           // host: tiles of the launch whose sharing (parts) this one follows, 0: its own
   int parts;                                // clusters that share a tile's K chunks (1: tiles are whole)
   float* part;                              // parts > 1: [tile][part][CTA of the pair][NT][128] float32
@@ -162,11 +168,11 @@ struct PairRowMeta {
   int pos, prow;
 };
 
-// SPLIT: p.parts > 1.
-template <int MODE, int NT, bool SPLIT>
+template <int MODE, int NT, int FORM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
 gemm_pair(const __grid_constant__ PairTmaps tm, const PairGemmParams p) {
   using Cfg = PairCfg<NT>;
+  constexpr bool SPLIT = FORM == GP_SHARED, RUNS = FORM == GP_RUNS;
   const int stages = p.stages, stage_bytes = Cfg::stage_bytes(p.tile_rows);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -191,7 +197,10 @@ gemm_pair(const __grid_constant__ PairTmaps tm, const PairGemmParams p) {
   const int items = SPLIT ? total_tiles * parts : p.cut_first + (total_tiles - p.cut_first) * p.cut;
   const int my_tiles = cl < items ? (SPLIT ? 1 : (items - 1 - cl) / ncl + 1) : 0;
   const int k_lo = SPLIT ? cl % parts * KC / parts : 0, k_hi = SPLIT ? (cl % parts + 1) * KC / parts : KC;
-  static_assert(MODE != GP_PLAIN || !SPLIT, "plain sums are not shared between clusters");
+  static_assert(MODE != GP_PLAIN || FORM == GP_WHOLE, "plain sums are results as they stand, in halves");
+  // GP_RUNS: number of runs of a weight pair's tiles and first chunk of the r-th
+  auto runs_of = [&](int wp) { return MODE == GP_SWIGLU ? p.seg.nseg(wp) : p.runs; };
+  auto run_start = [&](int wp, int r) { return MODE == GP_SWIGLU ? (r ? p.seg.lo(p.seg.owner(wp * KC) + r) - wp * KC : 0) : r * KC / p.runs; };
   const int halves = MODE == GP_PLAIN && KC > 1 ? 2 : 1;    // accumulators a tile's inner dimension is cut into
   // this cluster's i-th item: weight pair, first activation row and rows
   struct Item { int tau, wp, row0, rows; };
@@ -297,7 +306,31 @@ gemm_pair(const __grid_constant__ PairTmaps tm, const PairGemmParams p) {
       bool ok = true;
       int st = 0;
       uint32_t ph = 0;
-      for (int i = 0; i < my_tiles * halves && ok; ++i) {        // (accumulator fills: tiles, or halves of tiles in turn)
+      for (int i = 0; RUNS && i < my_tiles && ok; ++i) {
+        const int buf = p.run_bufs == 2 ? i & 1 : 0, use = p.run_bufs == 2 ? i >> 1 : i;
+        if (!mbar_wait(&acc_empty[buf], (use & 1) ^ 1, p.status, 44)) { ok = false; break; }
+        tc_fence_after();
+        const Item item = item_of(i);
+        const uint32_t idesc = make_idesc_bf16(256, item.rows);
+        const int nr = runs_of(item.wp);
+        for (int r = 0; r < nr && ok; ++r) {
+          const uint32_t d_addr = tmem_base + (uint32_t)((buf * p.runs + r) * p.tile_rows);
+          const int k_first = run_start(item.wp, r), k_end = r + 1 < nr ? run_start(item.wp, r + 1) : KC;
+          for (int kc = k_first; kc < k_end; ++kc) {
+            if (!mbar_wait(&full[st], ph, p.status, 41)) { ok = false; break; }
+            if (i == 0 && kc == 0) trace_mark_min(p.trace, 2);
+            tc_fence_after();
+            const uint64_t adesc = adesc0 + (uint64_t)(st * (stage_bytes >> 4)), bdesc = bdesc0 + (uint64_t)(st * (stage_bytes >> 4));
+#pragma unroll
+            for (int k = 0; k < Cfg::BK / 16; ++k)
+              tc_mma_f16_pair(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kc > k_first || k > 0) ? 1u : 0u);
+            tc_commit_pair(&empty[st]);
+            if (++st == stages) { st = 0; ph ^= 1; }
+          }
+        }
+        if (ok) tc_commit_pair(&acc_full[buf]);
+      }
+      for (int i = 0; !RUNS && i < my_tiles * halves && ok; ++i) {   // (accumulator fills: tiles, or halves of tiles in turn)
         const int buf = i & 1;
         if (!mbar_wait(&acc_empty[buf], ((i >> 1) & 1) ^ 1, p.status, 44)) { ok = false; break; }
         tc_fence_after();
@@ -330,14 +363,16 @@ gemm_pair(const __grid_constant__ PairTmaps tm, const PairGemmParams p) {
     pdl_wait();
     if (MODE == GP_PLAIN && p.clear && blockIdx.x == 0 && threadIdx.x < 68) p.clear[threadIdx.x - 64] = 0;
     for (int i = 0; i < my_tiles; ++i) {
-      const int buf = halves == 2 ? 1 : i & 1;                // the accumulator that completes the tile
-      const uint32_t acc_ph = halves == 2 ? i & 1 : (i >> 1) & 1;
+      // the accumulator that completes the tile (GP_RUNS: the accumulators' place)
+      const int buf = RUNS ? (p.run_bufs == 2 ? i & 1 : 0) : (halves == 2 ? 1 : i & 1);
+      const uint32_t acc_ph = RUNS ? (p.run_bufs == 2 ? i >> 1 : i) & 1 : (halves == 2 ? i & 1 : (i >> 1) & 1);
       const Item item = item_of(i);
       const int tau = item.tau, wp = item.wp, groups = item.rows >> 4;
       const int g0 = hf * groups / GP_QUARTERS, ng = (hf + 1) * groups / GP_QUARTERS - g0;   // this warp's 16-row groups
       const int nt = 2 * wp + rank;
       const int m0 = item.row0 + g0 * 16;                     // this warp's first activation row
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * NT + g0 * 16);
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)((RUNS ? buf * p.runs * p.tile_rows : buf * NT) + g0 * 16);
+      const int nr = RUNS ? runs_of(wp) : 1;
       constexpr bool split = SPLIT;
       // (what the epilogue needs besides the sums is fetched while the tile's MMAs run)
       // GP_RESIDUAL: old values of the first rows
@@ -435,6 +470,15 @@ gemm_pair(const __grid_constant__ PairTmaps tm, const PairGemmParams p) {
         if (!split) {
           tmem_ld16(taddr + g * 16, r);
           tmem_ld_wait();
+          if constexpr (RUNS) {
+            for (int k = 1; k < nr; ++k) {
+              uint32_t more[16];
+              tmem_ld16(taddr + k * p.tile_rows + g * 16, more);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(more[j]));
+            }
+          }
           return;
         }
         const float* src = parts_at + g * 16 * 128;

@@ -6,6 +6,7 @@
 // rounding points of the reference path: float32 until the operand is rounded to bf16.
 #pragma once
 #include "common.cuh"
+#include "gemm_cluster.cuh"
 #include "gemm_stream.cuh"
 #include "kernels_simple.cuh"
 
@@ -200,6 +201,64 @@ norm_scaled_tc(const float* __restrict__ x, const float* __restrict__ ss_part, i
     if (c4 < c_hi) emit(c4, keep[k], gk[k]);
   }
   for (int c4 = c_lo + threadIdx.x + NORM_CACHE * NORM_THREADS; c4 < c_hi; c4 += NORM_THREADS)
+    emit(c4, *reinterpret_cast<const float4*>(xr + c4 * 4), *reinterpret_cast<const float4*>(gain + c4 * 4));
+}
+
+// The same sums where no projection has left the pieces' (a prompt of two chunks in one pass): a CTA a row makes them out of x, as the residual epilogue
+// of 128 rows does, and adds them as norm_scaled_tc does. d % 16 == 0, at most NORM_PIECES pieces.
+constexpr int NORM_PIECES = 1024;
+__global__ void __launch_bounds__(NORM_THREADS)
+norm_pieces_tc(const float* __restrict__ x, const float* __restrict__ gain, float eps, bf16* __restrict__ u, int d, unsigned long long* tr) {
+  KTrace kt(tr);
+  pdl_launch_dependents();
+  const int m = blockIdx.x, n4 = d >> 2;
+  const float* xr = x + (size_t)m * d;
+  float4 gk[NORM_CACHE], keep[NORM_CACHE];
+#pragma unroll
+  for (int k = 0; k < NORM_CACHE; ++k) {
+    const int c4 = threadIdx.x + k * NORM_THREADS;
+    gk[k] = c4 < n4 ? *reinterpret_cast<const float4*>(gain + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __shared__ float pieces[NORM_PIECES], red[NORM_THREADS / 32];
+  pdl_wait();
+  if (threadIdx.x == 0) trace_mark_min(tr, 2);
+#pragma unroll
+  for (int k = 0; k < NORM_CACHE; ++k) {
+    const int c4 = threadIdx.x + k * NORM_THREADS;
+    keep[k] = c4 < n4 ? *reinterpret_cast<const float4*>(xr + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // (the four column groups of a piece sit in four neighbouring lanes; n4 is a multiple of four)
+  auto piece = [&](int c4, const float4& v) {
+    float ss = sum_sq<128>(v);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+    if ((threadIdx.x & 3) == 0 && c4 < n4) pieces[c4 >> 2] = ss;
+  };
+#pragma unroll
+  for (int k = 0; k < NORM_CACHE; ++k) piece(threadIdx.x + k * NORM_THREADS, keep[k]);
+  for (int c0 = NORM_CACHE * NORM_THREADS; c0 < n4; c0 += NORM_THREADS) {
+    const int c4 = c0 + threadIdx.x;
+    piece(c4, c4 < n4 ? *reinterpret_cast<const float4*>(xr + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f));
+  }
+  __syncthreads();
+  float ss = 0.f;
+  for (int i = threadIdx.x; i < (n4 >> 2); i += NORM_THREADS) ss += pieces[i];
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < NORM_THREADS / 32; ++w) tot += red[w];
+  const float inv = rsqrtf(tot / (float)d + eps);
+  auto emit = [&](int c4, const float4& v, const float4& g) {
+    *reinterpret_cast<uint2*>(u + (size_t)m * d + c4 * 4) = pack4_bf16(v.x * inv * g.x, v.y * inv * g.y, v.z * inv * g.z, v.w * inv * g.w);
+  };
+#pragma unroll
+  for (int k = 0; k < NORM_CACHE; ++k) {
+    const int c4 = threadIdx.x + k * NORM_THREADS;
+    if (c4 < n4) emit(c4, keep[k], gk[k]);
+  }
+  for (int c4 = threadIdx.x + NORM_CACHE * NORM_THREADS; c4 < n4; c4 += NORM_THREADS)
     emit(c4, *reinterpret_cast<const float4*>(xr + c4 * 4), *reinterpret_cast<const float4*>(gain + c4 * 4));
 }
 

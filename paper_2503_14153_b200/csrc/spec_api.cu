@@ -636,9 +636,17 @@ float pair_cost(int tiles, int rows, int cut, int KC, int clusters, float epilog
 void plan_pair(PairGemmParams* p, int mode, bool may_share, int max_clusters = GP_MAX_CLUSTERS) {
   const int clusters = std::min(GP_MAX_CLUSTERS, max_clusters), tall = p->w_pairs * ((p->M + GP_NT - 1) / GP_NT);
   p->tile_rows = GP_NT; p->cut = 1;
-  p->parts = may_share ? pair_parts(p->plan_tiles ? p->plan_tiles : tall, p->KC, clusters) : 1;
-  if (p->parts == 1) {
-    const float epilogue = mode == GP_RESIDUAL ? 0.0165f : 0.028f;
+  p->parts = may_share && p->runs == 0 ? pair_parts(p->plan_tiles ? p->plan_tiles : tall, p->KC, clusters) : 1;
+  const float epilogue = mode == GP_RESIDUAL ? 0.0165f : 0.028f;
+  if (p->runs > 0) {
+    // a run an accumulator; where tensor memory holds one item's only, its epilogue is not under the next one's MMAs
+    float best = 1e30f;
+    for (int rows = std::min({GP_NT, (int)round_up(p->M, 16), 512 / p->runs / 16 * 16}); rows >= 16; rows -= 16) {
+      const int tiles = p->w_pairs * ((p->M + rows - 1) / rows), bufs = 2 * p->runs * rows <= 512 ? 2 : 1;
+      const float us = pair_cost(tiles, rows, 1, p->KC, clusters, epilogue) + (bufs == 1 ? (tiles - 1) / clusters * epilogue * rows : 0.f);
+      if (us < 0.99f * best) { best = us; p->tile_rows = rows; p->run_bufs = bufs; }
+    }
+  } else if (p->parts == 1) {
     // Lower tiles take more bytes out of L2 for the same work, which a launch of several waves pays for in power, and with it in clock: they have to
     // look better by a tenth (1024 rows in tiles of 176 were 4% faster by themselves and slower in a step of 16 sequences).
     const int most = std::min(GP_NT, (int)round_up(p->M, 16));
@@ -669,16 +677,20 @@ cudaError_t launch_gp(cudaStream_t st, bool pdl, const PairTmaps& tm, const Pair
   static bool attr_set_dev[kAttrDevices] = {};
   bool& attr_set = *attr_flag(attr_set_dev);
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
-    if constexpr (MODE != GP_PLAIN)
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, GP_WHOLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+    if constexpr (MODE != GP_PLAIN) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, GP_SHARED>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair<MODE, GP_NT, GP_RUNS>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<GP_NT>::SMEM_BYTES);
+    }
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   const int items = pair_items(p), grid = 2 * (p.parts > 1 ? items : std::min(items, std::min(GP_MAX_CLUSTERS, max_clusters)));
-  auto kernel = gemm_pair<MODE, GP_NT, false>;
-  if constexpr (MODE != GP_PLAIN)
-    if (p.parts > 1) kernel = gemm_pair<MODE, GP_NT, true>;
+  auto kernel = gemm_pair<MODE, GP_NT, GP_WHOLE>;
+  if constexpr (MODE != GP_PLAIN) {
+    if (p.parts > 1) kernel = gemm_pair<MODE, GP_NT, GP_SHARED>;
+    if (p.runs > 0) kernel = gemm_pair<MODE, GP_NT, GP_RUNS>;
+  }
   return launch_k(pdl, kernel, dim3(grid), dim3(GP_THREADS), (size_t)PairCfg<GP_NT>::SMEM_BYTES, st, tm, p);
 }
 
@@ -1103,7 +1115,7 @@ int launch_attention_tc(spec_ctx* c, const Rows& pass, int l, const int* n_hi_pa
   // positions: 20.1 us a layer on 32 CTAs, 13.2 on 128.)
   a.row_parts = 1;
   if (a.nsplit == 1)
-    while (nw > 2 * a.row_parts && H * B * a.row_parts * 2 <= SM_SLOTS / 2) a.row_parts *= 2;
+    while (nw > 2 * a.row_parts && H * G * a.row_parts * 2 <= SM_SLOTS / 2) a.row_parts *= 2;
   const int nwp = (nw + a.row_parts - 1) / a.row_parts;          // 16-row blocks of a CTA
   dim3 grid(H, a.nsplit, G * a.row_parts);
 #define ATTN_CASE(HDV, NWV, KGV)                                                                         \
@@ -1210,6 +1222,122 @@ bool prompt_ends_alone(const spec_ctx* c, int M, int G) {
   return pair_gemm_ok(c, M, d) && pair_gemm_ok(c, M, HD) && pair_gemm_ok(c, M, f.d_ffn);
 }
 
+// act = SiLU(u W_g^T) * (u W_u^T) of layer l without the many-row kernel.
+int gate_up_act(spec_ctx* c, const bf16* u, int M, int l, bf16* act) {
+  const spec_config& f = c->cfg;
+  const int d = f.d_model, F = f.d_ffn, up0 = (F + 127) / 128 * 128;             // padded column of the up projection in the partial sums
+  const void* mats[2] = {c->wg[l], c->wu[l]};
+  const int rws[2] = {F, F};
+  if (cluster_gemm_ok(c, GC_SWIGLU, M, d)) return run_gemm_cluster(c, GC_SWIGLU, u, M, d, mats, F, nullptr, act, SPEC_PROFILE_GATE_UP);
+  if (const int cs = glu_cluster(c, M, d)) return run_gemm_glu(c, u, M, d, cs, mats, act);
+  PartView vg{};
+  int r = run_gemm(c, u, M, d, 2, mats, rws, SPEC_PROFILE_GATE_UP, &vg);
+  if (r) return r;
+  int slots = 0;
+  for (int t = 0; t < 2 * (up0 / 128) * vg.seg.m_tiles; ++t) slots = std::max(slots, vg.seg.nseg(t));
+  if (slots <= 2) {
+    KLAUNCH("swiglu_reduce_tc", swiglu_reduce_tc<SWIGLU_ROWS>, dim3((F / 4 + 255) / 256, (M + SWIGLU_ROWS - 1) / SWIGLU_ROWS), dim3(256), 0, vg, 0, up0, act, M, F);
+  } else {
+    KLAUNCH("swiglu_reduce_tc", swiglu_reduce_tc<1>, dim3((F / 4 + 255) / 256, M), dim3(256), 0, vg, 0, up0, act, M, F);
+  }
+  return SPEC_OK;
+}
+
+// ---- a lone prompt of two chunks ----
+// Its sums are those of its chunks one after the other, through the projections that stream the weights (see prefill_t). Where those cut every inner dimension
+// into a few runs, the same for a gate tile as for its up tile, both chunks go through the layers together: GP_RUNS adds the runs up in the
+// same order, the norm makes the pieces' sums that the residual clusters leave, and the attention takes the kernel that a chunk by itself
+// takes. The last layer goes on with the second chunk alone, from its attention output on with that chunk's own kernels.
+// On the 7B shape a layer of 256 rows takes 165 us (q/k/v 36, attention 14, output 19, gate+up 49, down 40, norms 7), of two chunks by themselves 224: a prompt through
+// four layers 1.03 -> 0.78 ms with the set-up, what bounds it being the chain of these kernels (weights 62 us, MMAs 65).
+// Fills in how gate and up are dealt out; false: chunk by chunk.
+bool two_chunks_at_once(const spec_ctx* c, SegMap* gate_up, int* gate_up_runs) {
+  const spec_config& f = c->cfg;
+  const int d = f.d_model, F = f.d_ffn, HD = f.n_heads * f.head_dim, R = PREFILL_ROWS, ft = (F + 127) / 128, rows[2] = {F, F};
+  if (!c->tc || c->chunk_cap < 2 || !pair_gemm_ok(c, 2 * R, d) || !pair_gemm_ok(c, 2 * R, HD) || !pair_gemm_ok(c, 2 * R, F) || d > 16 * NORM_PIECES) return false;
+  if (!cluster_gemm_ok(c, GC_ROPE, R, d) || !cluster_gemm_ok(c, GC_RESIDUAL, R, HD) || !cluster_gemm_ok(c, GC_RESIDUAL, R, F)) return false;
+  if (attn_long_mode(c, R, 1, 2 * R)) return false;
+  GemmPlan g;
+  if (!plan_gemm(R, d, 2, rows, stream_ctas(c, 2 * ft), &g)) return false;
+  const SegMap& s = g.p.seg;
+  int most = 0;
+  for (int t = 0; t < ft; ++t) {
+    const int n = s.nseg(t), at = s.owner(t * s.KC), up = s.owner((t + ft) * s.KC);
+    if (s.nseg(t + ft) != n) return false;
+    for (int r = 1; r < n; ++r)
+      if (s.lo(at + r) - t * s.KC != s.lo(up + r) - (t + ft) * s.KC) return false;
+    most = std::max(most, n);
+  }
+  *gate_up = s; *gate_up_runs = most;
+  return most <= 8;
+}
+
+int forward_two_chunks(spec_ctx* c, const Rows& both, int M, const SegMap& gate_up, int gate_up_runs) {
+  const spec_config& f = c->cfg;
+  const int d = f.d_model, F = f.d_ffn, H = f.n_heads, HD = H * f.head_dim, KD = f.n_kv_heads * f.head_dim, R = PREFILL_ROWS;
+  bf16 *u = static_cast<bf16*>(c->d_u), *act = static_cast<bf16*>(c->d_act), *attn = static_cast<bf16*>(c->d_attn);
+  Rows one = both;                           // a chunk by itself, which the attention's kernel is chosen for
+  one.B = 1;
+  const int cached[2] = {0, R};
+  int r;
+  for (int l = 0; l < f.n_layers; ++l) {
+    if (l == 0) {
+      KLAUNCH("norm_reduce_tc", norm_reduce_tc, dim3(M, NORM_CLUSTER), dim3(NORM_THREADS), 0, c->d_x, PartView{}, c->an[l], f.rms_eps, u, (float*)nullptr, d);
+    } else {
+      KLAUNCH("norm_reduce_tc", norm_pieces_tc, dim3(M), dim3(NORM_THREADS), 0, (const float*)c->d_x, c->an[l], f.rms_eps, u, d);
+    }
+    {
+      const void* mats[3] = {c->wq[l], c->wk[l], c->wv[l]};
+      const int rws[3] = {HD, KD, KD};
+      PairGemmParams w{};
+      w.runs = GC_ROPE_CLUSTER;
+      w.H = H; w.layer = l; w.rows = both; w.cs = c->d_rope; w.q = static_cast<bf16*>(c->d_q);
+      w.pool = static_cast<bf16*>(c->d_pool); w.g = c->geom; w.page_table = c->d_page_table;
+      if ((r = run_gemm_pair(c, GP_ROPE, u, M, d, 3, mats, rws, &w, SPEC_PROFILE_QKV))) return r;
+    }
+    if ((r = launch_attention_tc(c, one, l, cached + 1, nullptr, cached, &both))) return r;
+    if (l == f.n_layers - 1) break;
+    {
+      const void* mats[1] = {c->wo[l]};
+      const int rws[1] = {d};
+      PairGemmParams w{};
+      w.runs = GC_RES_CLUSTER; w.out = c->d_x; w.n_cols = d;
+      if ((r = run_gemm_pair(c, GP_RESIDUAL, attn, M, HD, 1, mats, rws, &w, SPEC_PROFILE_WO))) return r;
+    }
+    KLAUNCH("norm_reduce_tc", norm_pieces_tc, dim3(M), dim3(NORM_THREADS), 0, (const float*)c->d_x, c->fn[l], f.rms_eps, u, d);
+    {
+      const void* mats[2] = {c->wg[l], c->wu[l]};
+      const int rws[2] = {F, F};
+      PairGemmParams w{};
+      w.runs = gate_up_runs; w.seg = gate_up; w.act = act; w.n_cols = F;
+      if ((r = run_gemm_pair(c, GP_SWIGLU, u, M, d, 2, mats, rws, &w, SPEC_PROFILE_GATE_UP))) return r;
+    }
+    {
+      const void* mats[1] = {c->wd[l]};
+      const int rws[1] = {d};
+      PairGemmParams w{};
+      w.runs = GC_RES_CLUSTER; w.out = c->d_x; w.n_cols = d;
+      if ((r = run_gemm_pair(c, GP_RESIDUAL, act, M, F, 1, mats, rws, &w, SPEC_PROFILE_DOWN))) return r;
+    }
+  }
+  // the second chunk's rows, whole
+  const int l = f.n_layers - 1, n_ss = ((d + 127) / 128) * GC_RES_CLUSTER;
+  float* x = c->d_x + (size_t)R * d;
+  {
+    const void* mats[1] = {c->wo[l]};
+    if ((r = run_gemm_cluster(c, GC_RESIDUAL, attn + (size_t)R * HD, R, HD, mats, d, x, nullptr, SPEC_PROFILE_WO))) return r;
+  }
+  KLAUNCH("norm_reduce_tc", norm_scaled_tc, dim3(R, NORM_CLUSTER), dim3(NORM_THREADS), 0, (const float*)x, (const float*)c->d_ss_part, n_ss, c->fn[l], f.rms_eps, u, (float*)nullptr, d);
+  if ((r = gate_up_act(c, u, R, l, act))) return r;
+  {
+    const void* mats[1] = {c->wd[l]};
+    if ((r = run_gemm_cluster(c, GC_RESIDUAL, act, R, F, mats, d, x, nullptr, SPEC_PROFILE_DOWN))) return r;
+  }
+  KLAUNCH("norm_reduce_tc", norm_scaled_tc, dim3(R, NORM_CLUSTER), dim3(NORM_THREADS), 0, (const float*)x, (const float*)c->d_ss_part, n_ss, c->final_norm, f.rms_eps,
+          static_cast<bf16*>(c->d_hq), c->d_hid, d);
+  return SPEC_OK;
+}
+
 // One pass of the base model over M = groups * R rows whose tokens/positions/slots are prepared and
 // whose embeddings are in d_x: bf16 tensor-core path. Leaves the final hidden state in d_hid
 // (float32) and d_hq (bf16). ends: of a prompt-processing pass, else null.
@@ -1219,7 +1347,6 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
   bf16* u = static_cast<bf16*>(c->d_u);
   bf16* act = static_cast<bf16*>(c->d_act);
   const int kp0 = (HD + 127) / 128 * 128, vp0 = kp0 + (KD + 127) / 128 * 128;   // padded columns of k and v in the QKV partials
-  const int up0 = (F + 127) / 128 * 128;                                        // and of the up projection
   // (passes of more than 128 rows are bound by bandwidth, not by a row's latency: one plain CTA per row)
   // (after a residual cluster epilogue the pieces' sums of squares exist already: ss_ready)
   bool ss_ready = false;
@@ -1286,20 +1413,8 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
         PairGemmParams w{};
         w.act = act; w.n_cols = F;
         if ((r = run_gemm_pair(c, GP_SWIGLU, u, M, d, 2, mats, rws, &w, SPEC_PROFILE_GATE_UP))) return r;
-      } else if (cluster_gemm_ok(c, GC_SWIGLU, M, d)) {
-        if ((r = run_gemm_cluster(c, GC_SWIGLU, u, M, d, mats, F, nullptr, act, SPEC_PROFILE_GATE_UP))) return r;
-      } else if (const int cs = glu_cluster(c, M, d)) {
-        if ((r = run_gemm_glu(c, u, M, d, cs, mats, act))) return r;
-      } else {
-        PartView vg{};
-        if ((r = run_gemm(c, u, M, d, 2, mats, rws, SPEC_PROFILE_GATE_UP, &vg))) return r;
-        int slots = 0;
-        for (int t = 0; t < 2 * (up0 / 128) * vg.seg.m_tiles; ++t) slots = std::max(slots, vg.seg.nseg(t));
-        if (slots <= 2) {
-          KLAUNCH("swiglu_reduce_tc", swiglu_reduce_tc<SWIGLU_ROWS>, dim3((F / 4 + 255) / 256, (M + SWIGLU_ROWS - 1) / SWIGLU_ROWS), dim3(256), 0, vg, 0, up0, act, M, F);
-        } else {
-          KLAUNCH("swiglu_reduce_tc", swiglu_reduce_tc<1>, dim3((F / 4 + 255) / 256, M), dim3(256), 0, vg, 0, up0, act, M, F);
-        }
+      } else if ((r = gate_up_act(c, u, M, l, act))) {
+        return r;
       }
     }
     {
@@ -1584,9 +1699,8 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
   for (int b = 0; b < batch; ++b)
     for (int p = 0; p < off[b + 1] - off[b]; p += R) { cseq.push_back(b); cpos.push_back(p); }
   const int chunks = (int)cseq.size();
-  // A lone prompt of two chunks goes chunk by chunk, through the projections that stream the weights, in the order of sums that the
-  // prompt of one chunk and a lone sequence's verification steps have; the weights are read twice for that (on the 7B shape 8.5 ms instead
-  // of 7.1 when both forms were measured). Nothing more is promised: prompts of more chunks, and any prompt processed together with
+  // A lone prompt of two chunks has the sums of its chunks one after the other, through the projections that stream the weights: the order of sums that the
+  // prompt of one chunk and a lone sequence's verification steps have. (Both chunks at once where that can be had, see two_chunks_at_once.) Nothing more is promised: prompts of more chunks, and any prompt processed together with
   // others, take the many-row projections, whose order of sums is another one (and, up to 512 rows, depends on the rows).
   const int passes = batch == 1 && chunks == 2 ? 2 : (chunks + cap - 1) / cap;
   // the prompts' last rows, by sequence (the edge flags of the acceptance step are not in use while prompts are processed)
@@ -1646,7 +1760,22 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
     CUDA_OK(cudaMemcpyAsync(c->d_edge, ends.data(), ends.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));   // the host staging vectors go out of scope
   }
-  for (int pass = 0, ch = 0; pass < passes; ++pass) {
+  SegMap gate_up{};
+  int gate_up_runs = 0;
+  const bool at_once = c->tc && batch == 1 && chunks == 2 && two_chunks_at_once(c, &gate_up, &gate_up_runs);
+  if (at_once) {
+    Rows rows = make_rows(c, R, true);
+    rows.B = 2; rows.seq = c->d_chunk_seq; rows.n = c->d_chunk_n; rows.cnt = c->d_chunk_cnt;
+    prepare_prefill_rows<T><<<2 * R, 128, 0, c->stream>>>(rows, c->d_prompt, c->d_offsets, c->d_chunk_pos, static_cast<const T*>(c->embed), c->d_x, f.d_model,
+                                                        f.vocab, c->d_status);
+    LAUNCH_CHECK("prepare_prefill_rows");
+    int r = forward_two_chunks(c, rows, (int)round_up(off[1], 16), gate_up, gate_up_runs);
+    if (r) return r;
+    rows.B = 1; rows.seq += 1; rows.n += 1; rows.cnt += 1;
+    prefill_keep_last<T><<<1, 256, 0, c->stream>>>(rows, c->d_offsets, c->d_chunk_pos + 1, c->d_hid, c->d_h_last, static_cast<T*>(c->d_hq_last), c->d_n, f.d_model);
+    LAUNCH_CHECK("prefill_keep_last");
+  }
+  for (int pass = 0, ch = 0; !at_once && pass < passes; ++pass) {
     const int g = (chunks - ch + passes - pass - 1) / (passes - pass);    // chunks of this pass
     pe.seq0 += pe.count;
     pe.count = 0;

@@ -112,3 +112,32 @@ def test_rows_do_not_depend_on_the_tiles(torch):
         first = (h[0], kv[0], kv[1]) if first is None else first
         assert all((row == first[0]).all() for row in h)
         assert all((a == first[1 + i % 2]).all() for i, a in enumerate(kv))
+
+
+@pytest.mark.parametrize("d,heads,kv,hd,ffn,n", [
+    (512, 4, 4, 128, 1344, 129), (512, 8, 2, 64, 1344, 256),       # eight runs of gate+up; a row, and all, of the second chunk
+    (1024, 16, 4, 64, 2752, 250), (1024, 8, 8, 128, 704, 145),     # six; more than eight: chunk by chunk
+    (2048, 16, 16, 128, 5504, 200),                                # three CTAs to two tiles: runs of other lengths in every second tile
+    (1024, 32, 8, 64, 5248, 177),                                  # three; heads enough for the attention to take several rows' blocks a CTA
+])
+def test_two_chunks_at_once(torch, d, heads, kv, hd, ffn, n):
+    """A lone prompt of two chunks in one pass over the weights: first token, hidden state, cache and the steps that follow are those of its chunks one after
+    the other (to which it goes without the many-row kernel), bit for bit."""
+    import numpy as np
+    from paper_2503_14153_b200 import binding as B
+    from synthetic import get_config
+    cfg = get_config("c0", name="two", n_layers=3, d_model=d, n_heads=heads, n_kv_heads=kv, head_dim=hd, d_ffn=ffn, vocab=1000, dtype="bf16", rope_base=1e6,
+                     n_medusa=4, topk=(10, 4, 2, 2), tree_nodes=20)
+    prompt = np.random.default_rng(n).integers(0, 1000, n).astype(np.int32)
+    seen = {}
+    for wide in (1, 0):
+        gpu = random_decoder(torch, cfg, 5, n + 40)
+        gpu.set_option(B.OPT_WIDE_GEMM, wide)
+        gpu.prefill(prompt)
+        seen[wide] = [gpu.debug(B.DBG_NEXT_ROOT), gpu.debug(B.DBG_H_LAST)] + [a for l in range(3) for a in gpu.read_kv(0, l, 0, n)]
+        for t, c in (gpu.step() for _ in range(2)):
+            seen[wide].append(np.append(t[0, :c[0]], c[0]))
+        gpu.close()
+    assert np.isfinite(seen[1][1]).all() and np.abs(seen[1][1]).max() > 0.1
+    for a, b in zip(seen[1], seen[0]):
+        assert a.tobytes() == b.tobytes()
