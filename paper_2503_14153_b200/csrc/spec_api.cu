@@ -1192,7 +1192,7 @@ int finish_prompt_ends(spec_ctx* c, const Rows& pass, const int* n_hi_pass, cons
     w.plan_tiles = d_pairs * m_tiles; w.out = x; w.n_cols = d;
     if ((r = run_gemm_pair(c, GP_RESIDUAL, attn_end, G, HD, 1, mats, rws, &w, SPEC_PROFILE_WO))) return r;
   }
-  KLAUNCH("norm_reduce_tc", norm_rows_wide, dim3(G), dim3(NORMW_THREADS), 0, x, PartView{}, c->fn[l], f.rms_eps, u, (float*)nullptr, d);
+  KLAUNCH("norm_reduce_tc", norm_rows_wide<false>, dim3(G), dim3(NORMW_THREADS), 0, x, PartView{}, c->fn[l], f.rms_eps, u, (float*)nullptr, d);
   {
     const void* mats[2] = {c->wg[l], c->wu[l]};
     const int rws[2] = {F, F};
@@ -1207,7 +1207,7 @@ int finish_prompt_ends(spec_ctx* c, const Rows& pass, const int* n_hi_pass, cons
     w.plan_tiles = d_pairs * m_tiles; w.out = x; w.n_cols = d;
     if ((r = run_gemm_pair(c, GP_RESIDUAL, act, G, F, 1, mats, rws, &w, SPEC_PROFILE_DOWN))) return r;
   }
-  KLAUNCH("norm_reduce_tc", norm_rows_wide, dim3(G), dim3(NORMW_THREADS), 0, x, PartView{}, c->final_norm, f.rms_eps,
+  KLAUNCH("norm_reduce_tc", norm_rows_wide<false>, dim3(G), dim3(NORMW_THREADS), 0, x, PartView{}, c->final_norm, f.rms_eps,
           static_cast<bf16*>(c->d_hq_last) + (size_t)e.seq0 * d, c->d_h_last + (size_t)e.seq0 * d, d);
   return SPEC_OK;
 }
@@ -1355,7 +1355,11 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
   if (ss_ready && M <= 128) {                                                                            \
     KLAUNCH("norm_reduce_tc", norm_scaled_tc, dim3(M, NORM_CLUSTER), dim3(NORM_THREADS), 0, (const float*)c->d_x, (const float*)c->d_ss_part, n_ss, gain, f.rms_eps, uq, hid, d); \
   } else if (M > 128) {                                                                                         \
-    KLAUNCH("norm_reduce_tc", norm_rows_wide, dim3(M), dim3(NORMW_THREADS), 0, c->d_x, pv, gain, f.rms_eps, uq, hid, d); \
+    if (pv.part) {                                                                                       \
+      KLAUNCH("norm_reduce_tc", norm_rows_wide<true>, dim3(M), dim3(NORMW_THREADS), 0, c->d_x, pv, gain, f.rms_eps, uq, hid, d); \
+    } else {                                                                                             \
+      KLAUNCH("norm_reduce_tc", norm_rows_wide<false>, dim3(M), dim3(NORMW_THREADS), 0, c->d_x, pv, gain, f.rms_eps, uq, hid, d); \
+    }                                                                                                    \
   } else {                                                                                               \
     KLAUNCH("norm_reduce_tc", norm_reduce_tc, dim3(M, NORM_CLUSTER), dim3(NORM_THREADS), 0, c->d_x, pv, gain, f.rms_eps, uq, hid, d); \
   }
