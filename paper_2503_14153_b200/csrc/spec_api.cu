@@ -943,6 +943,13 @@ int linear_simple(spec_ctx* c, const char* name, const T* x, int n_mats, const v
   }
   if (MODE == LR_SWIGLU) groups = (rows[0] + LR_N / 2 - 1) / (LR_N / 2);
   const RowLinearShape sh = linear_rows_shape<T>(groups, M, K);
+  if constexpr (std::is_same<T, float>::value && MODE == LR_PLAIN)
+    if (n_mats == 1 && linear_held(sh, K)) {
+      const dim3 grid = linear_held_grid(sh, M, rows[0]);
+      if (M <= 4) KLAUNCH(name, (linear_rows_held<8, 4>), grid, dim3(LR_WARPS * 32), 0, x, w.w[0], y, ldy, M, rows[0], K, 1);
+      else KLAUNCH(name, (linear_rows_held<4, 8>), grid, dim3(LR_WARPS * 32), 0, x, w.w[0], y, ldy, M, rows[0], K, sh.ms);
+      return SPEC_OK;
+    }
   KLAUNCH(name, (linear_rows<T, MODE>), sh.grid, dim3(LR_WARPS * 32), 0, x, w, y, ldy, act, M, K, groups, sh.ks, sh.ms);
   return SPEC_OK;
 }
@@ -2500,7 +2507,14 @@ int op_linear_f32(const void* x, const void* w, float* y, int M, int N, int K, c
   rl.w[0] = static_cast<const float*>(w); rl.rows[0] = N; rl.n_mats = 1;
   const int groups = (N + LR_N - 1) / LR_N;
   const RowLinearShape sh = linear_rows_shape<float>(groups, M, K);
-  linear_rows<float, LR_PLAIN><<<sh.grid, LR_WARPS * 32, 0, st>>>(static_cast<const float*>(x), rl, y, (size_t)N, nullptr, M, K, groups, sh.ks, sh.ms, nullptr);
+  const float* xf = static_cast<const float*>(x);
+  if (linear_held(sh, K)) {
+    const dim3 grid = linear_held_grid(sh, M, N);
+    if (M <= 4) linear_rows_held<8, 4><<<grid, LR_WARPS * 32, 0, st>>>(xf, rl.w[0], y, (size_t)N, M, N, K, 1, nullptr);
+    else linear_rows_held<4, 8><<<grid, LR_WARPS * 32, 0, st>>>(xf, rl.w[0], y, (size_t)N, M, N, K, sh.ms, nullptr);
+  } else {
+    linear_rows<float, LR_PLAIN><<<sh.grid, LR_WARPS * 32, 0, st>>>(xf, rl, y, (size_t)N, nullptr, M, K, groups, sh.ks, sh.ms, nullptr);
+  }
   return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_E_CUDA;
 }
 bool op_linear_args_ok(int32_t dtype, const void* x, const void* w, const float* y, int M, int N, int K, int ctas) {

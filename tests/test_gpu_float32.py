@@ -44,6 +44,20 @@ def test_rows_do_not_depend_on_the_number_of_rows(torch, N, K):
         assert torch.equal(spec_op_linear(x[:m].contiguous(), w), whole[:m]), m
 
 
+@pytest.mark.parametrize("N,K", [(1, 8), (37, 64), (3001, 128), (2999, 200), (3000, 256), (9600, 248)])
+def test_activations_in_registers(torch, N, K):
+    """Projections of an inner dimension of up to 256, whose warps keep their rows in registers: against 64 bits within the bound of K
+    roundings, whatever the rows beside a row."""
+    from paper_2503_14153_b200 import spec_op_linear
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    x, w = torch.randn((101, K), generator=g, device="cuda"), torch.randn((N, K), generator=g, device="cuda")
+    whole = spec_op_linear(x, w)
+    want, size = x.double() @ w.double().T, x.double().abs() @ w.double().abs().T
+    assert ((whole.double() - want).abs() <= K * 2.0 ** -24 * size).all()
+    for m in (1, 3, 4, 5, 8, 9, 17, 40):
+        assert torch.equal(spec_op_linear(x[:m].contiguous(), w), whole[:m]), m
+
+
 @pytest.mark.parametrize("hd,heads,kv,prompt_len,dtype", [
     (32, 4, 4, 150, "fp32"), (64, 4, 2, 140, "fp32"), (96, 2, 2, 70, "fp32"), (128, 2, 1, 63, "fp32"), (160, 2, 2, 33, "fp32"),
     (256, 2, 2, 100, "fp32"), (256, 1, 1, 1, "fp32"), (64, 4, 2, 140, "bf16"),
