@@ -505,84 +505,101 @@ __global__ void rope_store(const float* __restrict__ qkv, Rows rows,
 
 // ------------------------------------------------------------------ plain tree attention
 // Row i of sequence b sees every cached position < n[b] and row u of the same pass iff bit u of anc[i] is set. A CTA takes
-// AP_ROWS query rows of one head, a warp each, and stages tiles of KT keys and values in shared memory (all of them in
+// ROWS query rows of one head and stages tiles of KT keys and values in shared memory (all of them in
 // one tile for the contexts of the float32 configuration); within a group of 32 keys a lane owns a key for the scores and
 // every 32nd dimension for the values. Two passes over the keys: maximum, then exp / sum / value accumulation with the
 // probabilities rounded to T before the product; with one tile the scores stay in registers in between. (With a warp that
 // walked the keys one by one out of L2, twice, a 16-node step of the two-layer configuration at 60 positions took 320 us in
-// all; with this, the row linear above and their fused steps 138. This kernel is 8.8 us of it per layer.)
-constexpr int AP_ROWS = 8, AP_GROUPS = 4;       // at most AP_GROUPS * 32 keys a tile
-__host__ __device__ inline int attention_plain_tile(int D) { return D <= 64 ? 128 : (D <= 128 ? 64 : 32); }
-inline size_t attention_plain_smem(int D) { return ((size_t)2 * attention_plain_tile(D) * (D + 4) + (size_t)AP_ROWS * D) * sizeof(float); }
+// all; with this, the row linear above and their fused steps 138.) Bound by latency: the chain of loads (length, page, keys), then what a
+// warp has to do for its row. So where that leaves the CTAs resident at once a row gets AP_WARPS / AP_FEW warps, which share its groups of keys and
+// then its dimensions (every sum in the order it has with one warp), and a thread has AP_DEEP key and value loads under way, not one:
+// 16 rows of 4 heads at 60 positions 7.5 -> 3.4 us a layer.
+constexpr int AP_WARPS = 8, AP_GROUPS = 4;      // at most AP_GROUPS * 32 keys a tile
+constexpr int AP_FEW = 2, AP_DEEP = 4;
+__host__ __device__ constexpr int attention_plain_tile(int D) { return D <= 64 ? 128 : (D <= 128 ? 64 : 32); }
+inline size_t attention_plain_smem(int D) { return ((size_t)2 * attention_plain_tile(D) * (D + 4) + (size_t)AP_WARPS * D) * sizeof(float); }
 
-template <typename T, int EPL>
-__global__ void __launch_bounds__(AP_ROWS * 32)
+template <typename T, int EPL, int ROWS>
+__global__ void __launch_bounds__(AP_WARPS * 32)
 attention_plain(const T* __restrict__ q, T* __restrict__ out, const T* __restrict__ pool, KVGeom g,
                 const int* __restrict__ page_table, Rows rows, int layer, int H, float scale, unsigned long long* tr) {
   KTrace kt(tr);
   pdl_launch_dependents();
   extern __shared__ __align__(16) float sm_plain[];
-  constexpr int D = EPL * 32, P = D + 4, KT = D <= 64 ? 128 : (D <= 128 ? 64 : 32);
+  constexpr int D = EPL * 32, P = D + 4, KT = attention_plain_tile(D), groups = KT / 32, PARTS = AP_WARPS / ROWS;
   float* ks = sm_plain;
   float* vs = ks + KT * P;
   float* qs = vs + KT * P;
   __shared__ long long ko[AP_GROUPS * 32];     // a key's offset in the pool, -1 past the end, and its row in its page
   __shared__ int kr_s[AP_GROUPS * 32];
-  __shared__ __align__(16) float ps[AP_ROWS][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.x, b = blockIdx.y, i0 = blockIdx.z * AP_ROWS;
+  __shared__ __align__(16) float ps[ROWS][AP_GROUPS * 32];      // a tile's probabilities, in the operands' type
+  __shared__ float pl[PARTS > 1 ? ROWS : 1][AP_GROUPS * 32];    // ... and as they go into the sum
+  __shared__ float mx_s[ROWS][PARTS];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = warp / PARTS, part = warp % PARTS;
+  const int h = blockIdx.x, b = blockIdx.y, i0 = blockIdx.z * ROWS;
   const int kvh = h / (H / g.n_kv_heads);
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  const int* pt = page_table + rows.sequence(b) * g.pages_per_seq;
+  const int page0 = pt[min((int)threadIdx.x / g.page_size, g.pages_per_seq - 1)];   // of this thread's key of the first tile (with the loads below)
   const int cnt = rows.cnt[b], n = rows.n[b];
   if (i0 >= cnt) return;
   const int S = n + cnt;
-  const int* pt = page_table + rows.sequence(b) * g.pages_per_seq;
-  const int i = i0 + warp;
+  const int i = i0 + row;
   const bool on = i < cnt;
   const size_t m = (size_t)b * rows.R + i;
   uint32_t a[4];
 #pragma unroll
   for (int w = 0; w < 4; ++w) a[w] = on ? rows.anc[i * 4 + w] : 0u;
-  if (on) for (int e = lane; e < D; e += 32) qs[warp * D + e] = to_f<T>(q[m * H * D + h * D + e]);
+  if (on) for (int e = part * 32 + lane; e < D; e += PARTS * 32) qs[row * D + e] = to_f<T>(q[m * H * D + h * D + e]);
   // keys [k0, k0 + KT) and, where asked, their values; rows past the end (up to a whole group of 32) are zeros. The
-  // divisions by the page size are done once a key; D / 4 lanes (or the warp) then copy a row.
+  // divisions by the page size are done once a key; D / 4 lanes (or the warp) then copy a row, AP_DEEP rows under way at a time.
   constexpr int per = D / 4, rpw = per <= 32 ? 32 / per : 1;
   const int sub = per <= 32 ? lane / per : 0, e0 = per <= 32 ? lane - sub * per : lane;
   auto stage = [&](int k0, bool values) {
     const int live = min(KT, (S - k0 + 31) & ~31);
-    for (int r = threadIdx.x; r < live; r += AP_ROWS * 32) {
+    for (int r = threadIdx.x; r < live; r += AP_WARPS * 32) {
       const int j = k0 + r;
       long long o = -1;
       if (j < S) {
         const int pg = j / g.page_size, prow = j - pg * g.page_size;
-        o = (long long)(g.block_offset(pt[pg], layer, 0, kvh) + (size_t)prow * D);
+        o = (long long)(g.block_offset(k0 ? pt[pg] : page0, layer, 0, kvh) + (size_t)prow * D);
         kr_s[r] = prow;
       }
       ko[r] = o;
     }
     __syncthreads();
-    for (int r = warp * rpw + sub; sub < rpw && r < live; r += AP_ROWS * rpw) {
-      const long long o = ko[r];
-      const T* kr = pool + o;
-      const T* vr = kr + g.block_elems();
-      const int prow = kr_s[r];
-      for (int c = e0; c < per; c += 32) {
-        float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
-        if (o >= 0) {
-          const int e = kv_elem<T>(prow, c * 4, D, g.page_size);   // four neighbouring elements stay together
-          if (sizeof(T) == 4) {
-            kv = *reinterpret_cast<const float4*>(kr + e);
-            if (values) vv = *reinterpret_cast<const float4*>(vr + e);
-          } else {
-            kv = make_float4(to_f<T>(kr[e]), to_f<T>(kr[e + 1]), to_f<T>(kr[e + 2]), to_f<T>(kr[e + 3]));
-            if (values) vv = make_float4(to_f<T>(vr[e]), to_f<T>(vr[e + 1]), to_f<T>(vr[e + 2]), to_f<T>(vr[e + 3]));
+    if (sub >= rpw) return;
+    for (int c = e0; c < per; c += 32)
+      for (int r0 = warp * rpw + sub; r0 < live; r0 += AP_DEEP * AP_WARPS * rpw) {
+        float4 kv[AP_DEEP], vv[AP_DEEP];
+#pragma unroll
+        for (int u = 0; u < AP_DEEP; ++u) {
+          const int r = r0 + u * AP_WARPS * rpw;
+          kv[u] = vv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+          const long long o = r < live ? ko[r] : -1;
+          if (o >= 0) {
+            const T* kr = pool + o;
+            const T* vr = kr + g.block_elems();
+            const int e = kv_elem<T>(kr_s[r], c * 4, D, g.page_size);   // four neighbouring elements stay together
+            if (sizeof(T) == 4) {
+              kv[u] = *reinterpret_cast<const float4*>(kr + e);
+              if (values) vv[u] = *reinterpret_cast<const float4*>(vr + e);
+            } else {
+              kv[u] = make_float4(to_f<T>(kr[e]), to_f<T>(kr[e + 1]), to_f<T>(kr[e + 2]), to_f<T>(kr[e + 3]));
+              if (values) vv[u] = make_float4(to_f<T>(vr[e]), to_f<T>(vr[e + 1]), to_f<T>(vr[e + 2]), to_f<T>(vr[e + 3]));
+            }
           }
         }
-        *reinterpret_cast<float4*>(ks + r * P + c * 4) = kv;
-        if (values) *reinterpret_cast<float4*>(vs + r * P + c * 4) = vv;
+#pragma unroll
+        for (int u = 0; u < AP_DEEP; ++u) {
+          const int r = r0 + u * AP_WARPS * rpw;
+          if (r < live) {
+            *reinterpret_cast<float4*>(ks + r * P + c * 4) = kv[u];
+            if (values) *reinterpret_cast<float4*>(vs + r * P + c * 4) = vv[u];
+          }
+        }
       }
-    }
   };
   auto score = [&](int k0, int gr) {
     const int j = k0 + gr * 32 + lane;
@@ -590,7 +607,7 @@ attention_plain(const T* __restrict__ q, T* __restrict__ out, const T* __restric
     const uint32_t word = u < 64 ? (u < 32 ? a[0] : a[1]) : (u < 96 ? a[2] : a[3]);
     const bool vis = on && j < S && (u < 0 || ((word >> (u & 31)) & 1u));
     const float4* kr = reinterpret_cast<const float4*>(ks + (gr * 32 + lane) * P);
-    const float4* qr = reinterpret_cast<const float4*>(qs + warp * D);
+    const float4* qr = reinterpret_cast<const float4*>(qs + row * D);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
     for (int e = 0; e < D / 4; ++e) {
@@ -599,24 +616,32 @@ attention_plain(const T* __restrict__ q, T* __restrict__ out, const T* __restric
     }
     return vis ? ((s.x + s.y) + (s.z + s.w)) * scale : -INFINITY;
   };
-  constexpr int groups = KT / 32;
   const int tiles = (S + KT - 1) / KT;
-  float keep[AP_GROUPS], mx = -INFINITY;
+  constexpr int MINE = (groups + PARTS - 1) / PARTS;              // groups of keys of a tile whose scores are this warp's: part, part + PARTS, ...
+  float keep[MINE], mx = -INFINITY;
   for (int t = 0; t < tiles; ++t) {
     __syncthreads();
     stage(t * KT, tiles == 1);
     __syncthreads();
 #pragma unroll
-    for (int gr = 0; gr < AP_GROUPS; ++gr) {
-      keep[gr] = -INFINITY;
-      if (gr < groups && t * KT + gr * 32 < S) keep[gr] = score(t * KT, gr);
-      mx = fmaxf(mx, keep[gr]);
+    for (int k = 0; k < MINE; ++k) {
+      const int gr = part + k * PARTS;
+      keep[k] = -INFINITY;
+      if (gr < groups && t * KT + gr * 32 < S) keep[k] = score(t * KT, gr);
+      mx = fmaxf(mx, keep[k]);
     }
   }
   mx = warp_max(mx);
-  float l = 0.f, acc[EPL];
+  if (PARTS > 1) {
+    if (lane == 0) mx_s[row][part] = mx;
+    __syncthreads();
 #pragma unroll
-  for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
+    for (int k = 0; k < PARTS; ++k) mx = fmaxf(mx, mx_s[row][k]);
+  }
+  constexpr int DIMS = (EPL + PARTS - 1) / PARTS;                 // and the dimensions lane + 32 * (part, part + PARTS, ...) of the values
+  float l = 0.f, acc[DIMS];
+#pragma unroll
+  for (int e = 0; e < DIMS; ++e) acc[e] = 0.f;
   for (int t = 0; t < tiles; ++t) {
     if (tiles > 1) {
       __syncthreads();
@@ -624,31 +649,42 @@ attention_plain(const T* __restrict__ q, T* __restrict__ out, const T* __restric
       __syncthreads();
     }
 #pragma unroll
-    for (int gr = 0; gr < AP_GROUPS; ++gr) {
+    for (int k = 0; k < MINE; ++k) {
+      const int gr = part + k * PARTS;
       if (gr >= groups || t * KT + gr * 32 >= S) continue;
-      const float s = tiles > 1 ? score(t * KT, gr) : keep[gr];
+      const float s = tiles > 1 ? score(t * KT, gr) : keep[k];
       const float p = s == -INFINITY ? 0.f : expf(s - mx);       // (keys a row does not see carry no weight)
-      l += p;
-      __syncwarp();
-      ps[warp][lane] = quant<T>(p);
-      __syncwarp();
-      const float* vr = vs + gr * 32 * P + lane;
+      ps[row][gr * 32 + lane] = quant<T>(p);
+      if (PARTS > 1) pl[PARTS > 1 ? row : 0][gr * 32 + lane] = p;
+      else l += p;
+    }
+    if (PARTS > 1) __syncthreads();
+    else __syncwarp();
+#pragma unroll
+    for (int gr = 0; gr < groups; ++gr) {
+      if (t * KT + gr * 32 >= S) continue;
+      if (PARTS > 1) l += pl[PARTS > 1 ? row : 0][gr * 32 + lane];
+      if (part >= EPL) continue;
+      const float* vr = vs + gr * 32 * P + lane + part * 32;
 #pragma unroll
       for (int k4 = 0; k4 < 8; ++k4) {
-        const float4 p4 = *reinterpret_cast<const float4*>(&ps[warp][k4 * 4]);
+        const float4 p4 = *reinterpret_cast<const float4*>(&ps[row][gr * 32 + k4 * 4]);
         const float pk[4] = {p4.x, p4.y, p4.z, p4.w};
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-          for (int e = 0; e < EPL; ++e)                          // (a key without weight is left out whatever its values are)
-            acc[e] = fmaf(pk[kk], pk[kk] != 0.f ? vr[(k4 * 4 + kk) * P + e * 32] : 0.f, acc[e]);
+          for (int e = 0; e < DIMS; ++e)                         // (a key without weight is left out whatever its values are)
+            if (EPL % PARTS == 0 || part + e * PARTS < EPL)
+              acc[e] = fmaf(pk[kk], pk[kk] != 0.f ? vr[(k4 * 4 + kk) * P + e * PARTS * 32] : 0.f, acc[e]);
       }
     }
+    if (PARTS == 1) __syncwarp();
   }
   if (!on) return;
   const float inv = 1.f / warp_sum(l);
 #pragma unroll
-  for (int e = 0; e < EPL; ++e) out[m * H * D + h * D + lane + e * 32] = from_f<T>(acc[e] * inv);
+  for (int e = 0; e < DIMS; ++e)
+    if (part + e * PARTS < EPL) out[m * H * D + h * D + lane + (part + e * PARTS) * 32] = from_f<T>(acc[e] * inv);
 }
 
 // ------------------------------------------------------------------ typical acceptance

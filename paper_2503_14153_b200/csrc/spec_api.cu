@@ -1450,16 +1450,22 @@ int forward_layers_tc(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const
   return SPEC_OK;
 }
 
-template <typename T, int EPL>
-int launch_attention_plain(spec_ctx* c, const Rows& rows, int l) {
+template <typename T, int EPL, int ROWS>
+int launch_attention_plain_rows(spec_ctx* c, const Rows& rows, int l) {
   static bool set_dev[kAttrDevices] = {};
   bool& set_ = *attr_flag(set_dev);
   const size_t sm = attention_plain_smem(EPL * 32);
-  if (!set_) { CUDA_OK(cudaFuncSetAttribute(attention_plain<T, EPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); set_ = true; }
-  KLAUNCH("attention_plain", (attention_plain<T, EPL>), dim3(c->cfg.n_heads, rows.B, (rows.R + AP_ROWS - 1) / AP_ROWS), dim3(AP_ROWS * 32), sm,
+  if (!set_) { CUDA_OK(cudaFuncSetAttribute(attention_plain<T, EPL, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); set_ = true; }
+  KLAUNCH("attention_plain", (attention_plain<T, EPL, ROWS>), dim3(c->cfg.n_heads, rows.B, (rows.R + ROWS - 1) / ROWS), dim3(AP_WARPS * 32), sm,
           static_cast<const T*>(c->d_q), static_cast<T*>(c->d_attn), static_cast<const T*>(c->d_pool), c->geom, (const int*)c->d_page_table, rows, l,
           c->cfg.n_heads, 1.0f / sqrtf((float)c->cfg.head_dim));
   return SPEC_OK;
+}
+template <typename T, int EPL>
+int launch_attention_plain(spec_ctx* c, const Rows& rows, int l) {
+  // several warps a row while the SMs take all of the CTAs that makes at once, a warp a row beyond (each CTA stages its head's keys and values for itself)
+  const bool few = (long long)c->cfg.n_heads * rows.B * ((rows.R + AP_FEW - 1) / AP_FEW) <= 2 * 148;
+  return few ? launch_attention_plain_rows<T, EPL, AP_FEW>(c, rows, l) : launch_attention_plain_rows<T, EPL, AP_WARPS>(c, rows, l);
 }
 
 // The same pass with the plain CUDA-core kernels (float32 configurations and the bf16 debug mode).

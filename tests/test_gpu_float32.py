@@ -71,3 +71,15 @@ def test_plain_attention_vs_oracle(torch, hd, heads, kv, prompt_len, dtype):
     rep = run_lockstep(cfg, draw_weights(cfg), build_tree(cfg.topk, cfg.tree_nodes), draw_prompt(cfg, prompt_len), 10,
                        1e-4 if dtype == "fp32" else 2e-2, 1e-2, flags=FLAG_SIMPLE_KERNELS if dtype == "bf16" else 0)
     assert rep.steps > 0
+
+
+@pytest.mark.parametrize("hd,heads,kv,nodes", [(32, 4, 4, 1), (64, 4, 2, 7), (96, 2, 2, 29), (64, 8, 8, 64), (64, 8, 4, 100), (256, 2, 1, 16)])
+def test_warps_of_a_row_vs_oracle(torch, hd, heads, kv, nodes):
+    """Trees whose rows get several warps each in the CUDA-core attention (an odd number of rows among them, more warps than groups of
+    keys or dimensions) and trees beyond that."""
+    from paper_2503_14153_b200 import build_tree
+    from tests_lockstep import run_lockstep
+    cfg = get_config("c0", name="plain", n_heads=heads, n_kv_heads=kv, head_dim=hd, dtype="fp32", vocab=2000, seed=hd, norm_gain="random",
+                     topk=(4, 2, 2) if nodes <= 29 else (10, 4, 2, 2), n_medusa=3 if nodes <= 29 else 4)
+    rep = run_lockstep(cfg, draw_weights(cfg), build_tree(cfg.topk, nodes), draw_prompt(cfg, 50), 8, 1e-4, 1e-2)
+    assert rep.steps > 0
