@@ -651,14 +651,16 @@ topk_slices_tc(const PartView pv, int V, int row0, int slice, int kmax, float* p
   topk_merge_row(pk_val, pk_idx, (int)gridDim.x, row, K, kmax, root_tok, cand_override, cand, zs);
 }
 
-// Per-head top-k where the projection left each row's largest in every tile of 128 tokens (best_val / best_idx [row][tiles]) beside the logits: the
+// Per-head top-k where the projection left each row's largest in every tile of 128 tokens (float32: of `tile` tokens, every tiles-th
+// piece of `piece`; best_val / best_idx [row][tiles]) beside the logits: the
 // kmax best lie in tiles whose largest is among the kmax best of those, so a CTA a row reads the maxima and a dozen tiles instead of the vocabulary.
 // Of the maxima of up to 64 groups of tiles (kmax or more of them) the kmax-th largest is a bound that kmax values reach; what reaches it in the tiles that do is
 // ranked (order: value descending, index ascending; NaN never wins). Where more than TOPK_CAP values reach it (many equal ones), kmax
-// rounds over those tiles decide. 4 heads over 32016 tokens: 9.6 us of topk_slices_tc -> 4.1; 64 rows: 22.3 -> 5.2.
+// rounds over those tiles decide. 4 heads over 32016 tokens: 9.6 us of topk_slices_tc -> 4.1; 64 rows: 22.3 -> 5.2; 3 float32
+// heads 8.6 -> 4.1.
 constexpr int TOPK_MAX_TILES = 512;                          // (and at least kmax)
 __global__ void __launch_bounds__(256)
-topk_tiles(const float* __restrict__ z, int ldz, const float* __restrict__ best_val, const int* __restrict__ best_idx, int tiles, int V, int kmax, int K,
+topk_tiles(const float* __restrict__ z, int ldz, const float* __restrict__ best_val, const int* __restrict__ best_idx, int tiles, int tile, int piece, int V, int kmax, int K,
            const int* __restrict__ root_tok, const int* __restrict__ cand_override, int* __restrict__ cand, unsigned long long* tr) {
   KTrace kt(tr);
   pdl_launch_dependents();
@@ -716,19 +718,21 @@ topk_tiles(const float* __restrict__ z, int ldz, const float* __restrict__ best_
   __syncthreads();
   const int nl = n_list;
   const float* zr = z + (size_t)row * ldz;
-  for (int l = warp; l < nl; l += 8) {
-    const int n0 = list[l] * 128 + lane * 4;
-    float x[4];
+  auto token = [&](int t, int c) { return (c / piece * tiles + t) * piece + c % piece; };
+  for (int l = warp; l < nl; l += 8)
+    for (int c = lane * 4; c < tile; c += 128) {
+      const int n0 = token(list[l], c);
+      float x[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = -INFINITY;
-    if (n0 < ldz) { const float4 v = __ldcg(reinterpret_cast<const float4*>(zr + n0)); x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }   // (ldz % 4 == 0)
+      for (int j = 0; j < 4; ++j) x[j] = -INFINITY;
+      if (n0 < ldz) { const float4 v = __ldcg(reinterpret_cast<const float4*>(zr + n0)); x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }   // (ldz % 4 == piece % 4 == 0)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (n0 + j < V && reaches(x[j], n0 + j)) {
-        const int at = atomicAdd(&count, 1);
-        if (at < TOPK_CAP) { cv[at] = x[j]; ci[at] = n0 + j; }
-      }
-  }
+      for (int j = 0; j < 4; ++j)
+        if (n0 + j < V && reaches(x[j], n0 + j)) {
+          const int at = atomicAdd(&count, 1);
+          if (at < TOPK_CAP) { cv[at] = x[j]; ci[at] = n0 + j; }
+        }
+    }
   __syncthreads();
   const int nc = count;
   if (nc <= TOPK_CAP) {
@@ -745,8 +749,8 @@ topk_tiles(const float* __restrict__ z, int ldz, const float* __restrict__ best_
   float pv = INFINITY; int pi = -1;
   for (int t = 0; t < kmax; ++t) {
     bv = -INFINITY; bi = NONE;
-    for (int c = tid; c < nl * 128; c += 256) {
-      const int n = list[c >> 7] * 128 + (c & 127);
+    for (int c = tid; c < nl * tile; c += 256) {
+      const int n = token(list[c / tile], c % tile);
       if (n >= V) continue;
       const float x = __ldcg(zr + n);
       if (better(pv, pi, x, n) && better(x, n, bv, bi)) { bv = x; bi = n; }

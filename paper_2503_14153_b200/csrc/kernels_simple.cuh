@@ -379,7 +379,8 @@ linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y
 // activations of its M_ rows in registers through all its groups of N_ outputs and fetches a whole group's weights while it reduces the
 // one before; two rows' products are one instruction. linear_rows fetched the activations again for every group (two thirds of its loads) and
 // waited for the second step's weights in each. 32016 outputs of 256: 3 rows in a step 9.4 -> 5.3 us, 16 rows 16.5 -> 13.5, 64 rows 55 -> 42. It is
-// bound by what 12 warps an SM have under way. (Fetching a step's weights as soon as its products are done, not both after them: 14.6 and 45.)
+// bound by what 12 warps an SM have under way. Each row's largest in the columns of a CTA goes to best_val / best_idx [M][gridDim.x] where they are
+// given: what follows reads those instead of the logits. (Fetching a step's weights as soon as its products are done, not both after them: 14.6 and 45.)
 constexpr int LH_STEPS = 2, LH_CTAS = 3;
 using f32x2 = unsigned long long;                              // two float32 in a register pair: one instruction does both products
 __device__ __forceinline__ f32x2 f32x2_of(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
@@ -387,7 +388,8 @@ __device__ __forceinline__ void f32x2_parts(f32x2 v, float& a, float& b) { asm("
 __device__ __forceinline__ f32x2 fma_f32x2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 template <int N_, int M_>
 __global__ void __launch_bounds__(LR_WARPS * 32, LH_CTAS)
-linear_rows_held(const float* __restrict__ x, const float* __restrict__ w, float* __restrict__ y, size_t ldy, int M, int N, int K, int ms, unsigned long long* tr) {
+linear_rows_held(const float* __restrict__ x, const float* __restrict__ w, float* __restrict__ y, size_t ldy, int M, int N, int K, int ms,
+                 float* __restrict__ best_val, int* __restrict__ best_idx, unsigned long long* tr) {
   static_assert(N_ * M_ == 32, "a lane a sum");
   KTrace kt(tr);
   pdl_launch_dependents();
@@ -407,6 +409,8 @@ linear_rows_held(const float* __restrict__ x, const float* __restrict__ w, float
   if (g < groups) load_w(g);
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  float bv = -INFINITY;
+  int bi = 0x7fffffff;
 #pragma unroll
   for (int s = 0; s < LH_STEPS; ++s)
 #pragma unroll
@@ -448,14 +452,36 @@ linear_rows_held(const float* __restrict__ x, const float* __restrict__ w, float
       }
     }
     if (m < M && n < N) y[(size_t)m * ldy + n] = v[0];
+    if (n < N && better(v[0], n, bv, bi)) { bv = v[0]; bi = n; }
   }
+  if (!best_val) return;
+  __shared__ float sv[LR_WARPS][M_];
+  __shared__ int si[LR_WARPS][M_];
+#pragma unroll
+  for (int o = M_; o < 32; o <<= 1) {
+    const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (better(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+  }
+  if (lane < M_) { sv[warp][lane] = bv; si[warp][lane] = bi; }
+  __syncthreads();
+  const int m = m0 + lane;
+  if (warp >= ms || lane >= M_ || m >= M) return;
+  for (int k = warp + ms; k < LR_WARPS; k += ms) if (better(sv[k][lane], si[k][lane], bv, bi)) { bv = sv[k][lane]; bi = si[k][lane]; }
+  best_val[(size_t)m * gridDim.x + blockIdx.x] = bv;
+  best_idx[(size_t)m * gridDim.x + blockIdx.x] = bi;
 }
 inline bool linear_held(const RowLinearShape& s, int K) { return s.ks == 1 && K <= LH_STEPS * 128; }
-// (up to 4 rows: half the loads a sum; the rows of linear_rows's shape otherwise)
-inline dim3 linear_held_grid(const RowLinearShape& s, int M, int N) {
-  const int n = M <= 4 ? 8 : 4, ms = M <= 4 ? 1 : s.ms, per = LR_WARPS / ms;
-  const unsigned y = M <= 4 ? 1u : s.grid.y, all = (unsigned)(((N + n - 1) / n + per - 1) / per);
-  return dim3(std::min(all, std::max(1u, LH_CTAS * 148u / y)), y);
+// (Up to 4 rows: half the loads a sum; the rows of linear_rows's shape otherwise.) A CTA's columns are every grid.x-th piece of `piece`. Neighbouring pieces
+// instead: 3 rows 5.3 -> 6.8 us, 64 rows 42 -> 45.
+struct HeldShape { dim3 grid; int cols, ms, piece; };
+inline HeldShape linear_held_shape(const RowLinearShape& s, int M, int N) {
+  HeldShape h;
+  h.cols = M <= 4 ? 8 : 4; h.ms = M <= 4 ? 1 : s.ms;
+  h.piece = LR_WARPS / h.ms * h.cols;
+  const unsigned y = M <= 4 ? 1u : s.grid.y;
+  h.grid = dim3(std::min((unsigned)((N + h.piece - 1) / h.piece), std::max(1u, LH_CTAS * 148u / y)), y);
+  return h;
 }
 
 // ------------------------------------------------------------------ RoPE + cache store

@@ -931,9 +931,11 @@ int run_gemm_glu(spec_ctx* c, const void* in, int M, int K, int cs, const void* 
 
 // y[M, rows of all matrices] = x * [mats]^T on the CUDA cores, act = SiLU(x W_0^T) * (x W_1^T) (LR_SWIGLU, float32 y unused)
 // or y += x * W_0^T (LR_RESIDUAL). ldy: row pitch of y.
+// best (may be null): set to where each row's largest in every tile (every tiles-th piece of `piece` columns, `tile` of them in all) lies, if the kernel leaves them (in the buffer of the partial sums).
+struct RowBest { float* val; int* idx; int tiles, tile, piece; };
 template <typename T, int MODE>
 int linear_simple(spec_ctx* c, const char* name, const T* x, int n_mats, const void* const* mats, const int* rows, float* y, size_t ldy, T* act,
-                  int M, int K) {
+                  int M, int K, RowBest* best = nullptr) {
   RowLinear<T> w{};
   w.n_mats = n_mats;
   int groups = 0;
@@ -945,9 +947,12 @@ int linear_simple(spec_ctx* c, const char* name, const T* x, int n_mats, const v
   const RowLinearShape sh = linear_rows_shape<T>(groups, M, K);
   if constexpr (std::is_same<T, float>::value && MODE == LR_PLAIN)
     if (n_mats == 1 && linear_held(sh, K)) {
-      const dim3 grid = linear_held_grid(sh, M, rows[0]);
-      if (M <= 4) KLAUNCH(name, (linear_rows_held<8, 4>), grid, dim3(LR_WARPS * 32), 0, x, w.w[0], y, ldy, M, rows[0], K, 1);
-      else KLAUNCH(name, (linear_rows_held<4, 8>), grid, dim3(LR_WARPS * 32), 0, x, w.w[0], y, ldy, M, rows[0], K, sh.ms);
+      const HeldShape h = linear_held_shape(sh, M, rows[0]);
+      RowBest at{};
+      if (best && 2 * (size_t)M * h.grid.x <= c->part_floats)
+        *best = at = RowBest{c->d_part, reinterpret_cast<int*>(c->d_part + (size_t)M * h.grid.x), (int)h.grid.x, (int)round_up(rows[0], h.piece * h.grid.x) / (int)h.grid.x, h.piece};
+      KLAUNCH(name, (h.cols == 8 ? linear_rows_held<8, 4> : linear_rows_held<4, 8>), h.grid, dim3(LR_WARPS * 32), 0, x, w.w[0], y, ldy, M, rows[0], K, h.ms,
+              at.val, at.idx);
       return SPEC_OK;
     }
   KLAUNCH(name, (linear_rows<T, MODE>), sh.grid, dim3(LR_WARPS * 32), 0, x, w, y, ldy, act, M, K, groups, sh.ks, sh.ms);
@@ -1600,7 +1605,7 @@ int heads_tc(spec_ctx* c, const int* ov) {
     int r = run_lm_head(c, c->d_r, rows_total, cs, c->d_part, ldz, maxima ? val : nullptr, maxima ? idx : nullptr);
     if (r) return r;
     if (maxima) {
-      KLAUNCH("topk_tiles", topk_tiles, dim3(rows_total), dim3(256), 0, (const float*)c->d_part, ldz, (const float*)val, (const int*)idx, tiles, f.vocab, c->kmax, K,
+      KLAUNCH("topk_tiles", topk_tiles, dim3(rows_total), dim3(256), 0, (const float*)c->d_part, ldz, (const float*)val, (const int*)idx, tiles, 128, 128, f.vocab, c->kmax, K,
               (const int*)c->d_root, ov, c->d_cand);
       return SPEC_OK;
     }
@@ -1648,8 +1653,13 @@ int lm_head_argmax(spec_ctx* c, const T* src, int M) {
     int r = run_gemm(c, src, M, f.d_model, 1, mats, rws, SPEC_PROFILE_OFF, &pl);
     if (r) return r;
   } else {
-    int r = linear_simple<T, LR_PLAIN>(c, "linear_lm_head", src, 1, mats, rws, c->d_logits, f.vocab, nullptr, M, f.d_model);
+    RowBest best{};
+    int r = linear_simple<T, LR_PLAIN>(c, "linear_lm_head", src, 1, mats, rws, c->d_logits, f.vocab, nullptr, M, f.d_model, &best);
     if (r) return r;
+    if (best.val) {
+      KLAUNCH("argmax_tiles", argmax_tiles, dim3((M + 7) / 8), dim3(256), 0, (const float*)best.val, (const int*)best.idx, M, best.tiles, c->d_pval2, c->d_pidx2);
+      return SPEC_OK;
+    }
     pl = plain_view(c->d_logits, M, f.vocab);
   }
   KLAUNCH("argmax_partials_tc", argmax_partials_tc, dim3(M, c->n_argmax), dim3(256), 0, pl, f.vocab,
@@ -1860,9 +1870,15 @@ int step_body(spec_ctx* c, const int* ov, const int* n_hi_plan, const int* n_lo_
     const int ldz = (int)round_up(f.vocab, 4);
     for (int r0 = 0; r0 < B * K; r0 += c->head_rows) {
       const int rows_now = std::min(c->head_rows, B * K - r0);
+      RowBest best{};
       int r = linear_simple<T, LR_PLAIN>(c, "linear_heads", static_cast<const T*>(c->d_r) + (size_t)r0 * d, 1, mats, &f.vocab, c->d_logits, ldz, nullptr,
-                                         rows_now, d);
+                                         rows_now, d, &best);
       if (r) return r;
+      if (best.val && rows_now == B * K && best.tiles >= kmax && best.tiles <= TOPK_MAX_TILES && best.tile <= 512) {   // (beyond, a tile is much to read again)
+        KLAUNCH("topk_tiles", topk_tiles, dim3(rows_now), dim3(256), 0, (const float*)c->d_logits, ldz, (const float*)best.val, (const int*)best.idx, best.tiles, best.tile, best.piece,
+                f.vocab, kmax, K, (const int*)c->d_root, ov, c->d_cand);
+        break;
+      }
       if ((r = heads_top_k(c, plain_view(c->d_logits, rows_now, ldz), r0, rows_now, ov))) return r;
     }
   } else {
@@ -2515,9 +2531,8 @@ int op_linear_f32(const void* x, const void* w, float* y, int M, int N, int K, c
   const RowLinearShape sh = linear_rows_shape<float>(groups, M, K);
   const float* xf = static_cast<const float*>(x);
   if (linear_held(sh, K)) {
-    const dim3 grid = linear_held_grid(sh, M, N);
-    if (M <= 4) linear_rows_held<8, 4><<<grid, LR_WARPS * 32, 0, st>>>(xf, rl.w[0], y, (size_t)N, M, N, K, 1, nullptr);
-    else linear_rows_held<4, 8><<<grid, LR_WARPS * 32, 0, st>>>(xf, rl.w[0], y, (size_t)N, M, N, K, sh.ms, nullptr);
+    const HeldShape h = linear_held_shape(sh, M, N);
+    (h.cols == 8 ? linear_rows_held<8, 4> : linear_rows_held<4, 8>)<<<h.grid, LR_WARPS * 32, 0, st>>>(xf, rl.w[0], y, (size_t)N, M, N, K, h.ms, nullptr, nullptr, nullptr);
   } else {
     linear_rows<float, LR_PLAIN><<<sh.grid, LR_WARPS * 32, 0, st>>>(xf, rl, y, (size_t)N, nullptr, M, K, groups, sh.ks, sh.ms, nullptr);
   }

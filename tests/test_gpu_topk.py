@@ -41,3 +41,44 @@ def test_candidates(vocab, batch, kmax):
         picked = z[b][got]
         assert (np.diff(picked) <= tol).all()
         assert np.delete(z[b], got).max() <= picked[-1] + tol
+
+
+@pytest.mark.parametrize("vocab,batch,kmax,classes", [
+    (2371, 1, 10, 0), (3001, 2, 5, 0),        # the fewest columns whose warps keep their rows, a ragged end
+    (32016, 3, 4, 0), (32016, 9, 16, 0),      # up to four rows, and two groups of eight
+    (9001, 1, 10, 7), (9001, 6, 16, 7),       # more equal values than the lists hold
+])
+def test_candidates_float32(vocab, batch, kmax, classes):
+    """The same in float32, whose tiles are every so many-th piece of the vocabulary: equal values go by their index."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = get_config("c0", name="topk", vocab=vocab, d_ffn=704, n_heads=2, n_kv_heads=2, n_medusa=1, topk=(kmax,), tree_nodes=kmax + 1, seed=7)
+    w = draw_weights(cfg)
+    if classes:
+        w["lm_head"] = np.ascontiguousarray(w["lm_head"][np.arange(vocab) % classes])
+    dec = SpecDecoder(cfg, upload_weights(cfg, w), build_tree(cfg.topk, kmax + 1), 64, max_batch=batch)
+    dec.prefill([draw_prompt(cfg.with_(seed=30 + b), 5 + b) for b in range(batch)])
+    h = torch.from_numpy(dec.debug(B.DBG_H_LAST)).double()
+    dec.step()
+    cand = dec.debug(B.DBG_CAND)
+    dec.close()
+
+    def operand(a):
+        return torch.from_numpy(np.ascontiguousarray(a)).double()
+    r = h + torch.nn.functional.silu(h @ operand(w["medusa.0.w"]).T + operand(w["medusa.0.b"]))
+    z = (r @ operand(w["lm_head"]).T).numpy()
+    size = (r.abs() @ operand(w["lm_head"]).abs().T).numpy()
+    for b in range(batch):
+        got = cand[b, 1]
+        assert len(set(got.tolist())) == kmax
+        if classes:
+            best = int(np.argmax(z[b, :classes]))
+            assert got.tolist() == [best + classes * i for i in range(kmax)]
+            continue
+        tol = 4 * 256 * 2.0 ** -24 * size[b].max()   # (256 roundings of a sum here, and as many in r, on both sides of a comparison)
+        picked = z[b][got]
+        assert (np.diff(picked) <= tol).all()
+        assert np.delete(z[b], got).max() <= picked[-1] + tol
