@@ -95,8 +95,12 @@ template <int MT> struct ClusterCfg {
 // A smaller one (the projections of narrow models: at d_model 1024 q/k/v has 24 CTAs of 8 chunks, gate+up 66 of 11) gets a stage for every
 // chunk as far as shared memory goes, so that all of a CTA's weights are under way before the dependency wait and the chain behind it is
 // activation tiles, MMAs and the exchange. Six layers of d_model 1024, 64 rows: gate+up 10.3 -> 8.4 us, down 6.2 -> 4.9, a step 284 -> 263.
+// Of more than one CTA an SM with short runs and 16 rows (wo of the 7B shape: 32 clusters of 8 CTAs, 8 chunks each) three fit an SM: the attention
+// before it has 32 CTAs, and with two an SM a few clusters did not find room beside those and began when it ended: wo 9.9 -> 7.5 us.
+// (With 64 rows attention has 128 CTAs and three stages cost more than they give: 10.1 -> 10.8.)
 template <int MT> inline int cluster_stages(int ctas, int units) {
   using Cfg = ClusterCfg<MT>;
+  if (ctas > 148 && MT == 16 && units <= 8) return 4;
   if (ctas > 148 || units <= Cfg::STAGES) return Cfg::STAGES;
   return units < Cfg::MAX_STAGES ? units : Cfg::MAX_STAGES;
 }
