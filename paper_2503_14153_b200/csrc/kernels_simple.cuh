@@ -249,12 +249,26 @@ template <> struct Vec16<bf16> {
 // then come out of L2 once: at lm_head (32016 x 256, 16 rows) the weights crossing L2 are the bound. What follows the
 // projection is done in place of a kernel of its own.
 constexpr int LR_N = 4, LR_M = 8, LR_WARPS = 4;
-constexpr int LR_PLAIN = 0, LR_SWIGLU = 1, LR_RESIDUAL = 2;
+constexpr int LR_PLAIN = 0, LR_SWIGLU = 1, LR_RESIDUAL = 2, LR_ROPE = 3;
 template <typename T> struct RowLinear {
   const T* w[3];          // stacked matrices (LR_SWIGLU: gate, up)
   int rows[3];            // their rows
   int group0[3];          // first group of LR_N outputs of each (LR_SWIGLU: groups of LR_N / 2 columns, one range)
   int n_mats;
+};
+
+// LR_ROPE (q, k, v): rotate-half RoPE (element i pairs with i + D/2, angle pos * base^(-2i/D)) on q and k in registers; q -> T [M][H*D], k and v -> T into the
+// paged cache at the row's slot. A group of q or k is the outputs e, e + 1 and their partners in the other half of the head. A kernel of its own behind the
+// projection took 3 us a layer, nearly all of it a launch and two trips to L2 (the row's slot, its page): the projection makes these while its sums are formed.
+// A request of the two-layer configuration 2.34 -> 2.25 ms. Which product the rotation fuses is fixed, as that kernel had it.
+template <typename T> struct RopeStore {
+  Rows rows;
+  const float2* cs;       // [position][head_dim / 2] (cos, sin)
+  T* q;
+  T* pool;
+  KVGeom g;
+  const int* page_table;
+  int layer, H;
 };
 
 // Warps that share a group of outputs: as many as have a step of the inner dimension each, while 16 rows (the verification
@@ -288,7 +302,7 @@ template <typename T> inline RowLinearShape linear_rows_shape(int groups, int M,
 template <typename T, int MODE>
 __global__ void __launch_bounds__(LR_WARPS * 32, 4)
 linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y, size_t ldy, T* __restrict__ act, int M, int K, int groups, int ks, int ms,
-            unsigned long long* tr) {
+            const RopeStore<T> rs, unsigned long long* tr) {
   KTrace kt(tr);
   pdl_launch_dependents();
   constexpr int VN = Vec16<T>::N;
@@ -298,8 +312,18 @@ linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y
   int g = blockIdx.x * per + warp / (ks * ms);
   // where the current group's outputs are: its matrix, first row there, first column of y
   const T *wa, *wb;
-  int N, n0, col0;
+  int N, n0, col0, up = 2;                                     // (a group's outputs: n0, n0 + 1, n0 + up, n0 + up + 1)
+  const int D = MODE == LR_ROPE ? rs.g.head_dim : 0, half = D >> 1;
   auto locate = [&](int gg) {
+    if (MODE == LR_ROPE) {
+      const int mat = gg >= w.group0[2] ? 2 : (gg >= w.group0[1] ? 1 : 0), gi = gg - (mat == 0 ? 0 : (mat == 1 ? w.group0[1] : w.group0[2]));
+      wa = wb = mat == 0 ? w.w[0] : (mat == 1 ? w.w[1] : w.w[2]);
+      N = mat == 0 ? w.rows[0] : (mat == 1 ? w.rows[1] : w.rows[2]);
+      up = mat == 2 ? 2 : half;
+      n0 = mat == 2 ? gi * LR_N : gi / (half / 2) * D + gi % (half / 2) * 2;
+      col0 = mat;
+      return;
+    }
     if (MODE == LR_SWIGLU) { wa = w.w[0]; wb = w.w[1]; N = w.rows[0]; n0 = gg * (LR_N / 2); col0 = 0; return; }
     const int mat = w.n_mats > 2 && gg >= w.group0[2] ? 2 : (w.n_mats > 1 && gg >= w.group0[1] ? 1 : 0);
     wa = wb = mat == 0 ? w.w[0] : (mat == 1 ? w.w[1] : w.w[2]);
@@ -312,7 +336,7 @@ linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y
   auto load_w = [&](int k) {
 #pragma unroll
     for (int j = 0; j < LR_N; ++j) {
-      const int n = min(MODE == LR_SWIGLU ? n0 + (j & 1) : n0 + j, N - 1);
+      const int n = min(MODE == LR_SWIGLU ? n0 + (j & 1) : (MODE == LR_ROPE ? n0 + (j & 1) + (j >> 1) * up : n0 + j), N - 1);
       Vec16<T>::load((j < 2 ? wa : wb) + (size_t)n * K + k, wv[j]);
     }
   };
@@ -321,11 +345,22 @@ linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y
   if (k0 < K) load_w(k0);
   pdl_wait();
   if (threadIdx.x == 0) trace_mark_min(tr, 2);
+  // LR_ROPE: where this lane's row stands (its sums come last)
+  int pos = -1, page = 0, prow = 0;
+  if (MODE == LR_ROPE && kpart == 0 && m0 + lane % LR_M < M) {
+    const int m = m0 + lane % LR_M, b = m / rs.rows.R;
+    if (m - b * rs.rows.R < rs.rows.cnt[b]) {
+      const int slot = rs.rows.slot[m];
+      pos = rs.rows.pos[m];
+      page = rs.page_table[rs.rows.sequence(b) * rs.g.pages_per_seq + slot / rs.g.page_size];
+      prow = slot % rs.g.page_size;
+    }
+  }
   for (;;) {
     float v[LR_N * LR_M];
 #pragma unroll
     for (int i = 0; i < LR_N * LR_M; ++i) v[i] = 0.f;
-    const int n_this = n0, N_this = N, col_this = col0;
+    const int n_this = n0, N_this = N, col_this = col0, up_this = up;
     g += gridDim.x * per;
     const bool more = g < groups;
     for (int k = k0; k < K;) {
@@ -340,6 +375,8 @@ linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y
       k += ks * 32 * VN;
       if (k < K) load_w(k);
     }
+    float2 t = make_float2(1.f, 0.f);
+    if (MODE == LR_ROPE && pos >= 0 && col_this < 2) t = rs.cs[(size_t)pos * half + n_this % D + ((lane / LR_M) & 1)];
     // the next group's first weights are on their way while this one's sums are reduced
     if (more) { locate(g); if (k0 < K) load_w(k0); }
 #pragma unroll
@@ -359,7 +396,15 @@ linear_rows(const T* __restrict__ x, const RowLinear<T> w, float* __restrict__ y
       for (int i = 1; i < ks; ++i) v[0] += parts[warp + i][lane];
     }
     const int j = lane / LR_M, m = m0 + lane % LR_M;
-    if (MODE == LR_SWIGLU) {
+    if (MODE == LR_ROPE) {
+      const float other = __shfl_xor_sync(0xffffffffu, v[0], 16);
+      const int n = n_this + (j & 1) + (j >> 1) * up_this, head = n / D, e = n - head * D;
+      if (pos >= 0) {
+        const float r = col_this == 2 ? v[0] : (j < 2 ? __fmaf_rn(v[0], t.x, -__fmul_rn(other, t.y)) : __fmaf_rn(v[0], t.x, __fmul_rn(other, t.y)));
+        if (col_this == 0) rs.q[(size_t)m * N_this + n] = from_f<T>(r);
+        else rs.pool[rs.g.block_offset(page, rs.layer, col_this - 1, head) + (size_t)prow * D + kv_elem<T>(prow, e, D, rs.g.page_size)] = from_f<T>(r);
+      }
+    } else if (MODE == LR_SWIGLU) {
       const float up = __shfl_xor_sync(0xffffffffu, v[0], 16);
       const int n = n_this + (j & 1);
       if (j < 2 && m < M && n < N_this) act[(size_t)m * N_this + n] = from_f<T>(silu_f(v[0]) * up);
@@ -482,51 +527,6 @@ inline HeldShape linear_held_shape(const RowLinearShape& s, int M, int N) {
   const unsigned y = M <= 4 ? 1u : s.grid.y;
   h.grid = dim3(std::min((unsigned)((N + h.piece - 1) / h.piece), std::max(1u, LH_CTAS * 148u / y)), y);
   return h;
-}
-
-// ------------------------------------------------------------------ RoPE + cache store
-// qkv: float32 [M][(H+2Hkv)*D]. Rotate-half RoPE (element i pairs with
-// i + D/2, angle pos * base^(-2i/D), table cs[pos][i] = (cos, sin)) on q and k; q -> T
-// [M][H*D]; k, v -> T into the paged cache at the row's slot.
-template <typename T>
-__global__ void rope_store(const float* __restrict__ qkv, Rows rows,
-                           const float2* __restrict__ cs, T* __restrict__ q, T* __restrict__ pool, KVGeom g,
-                           const int* __restrict__ page_table, int layer, int H, unsigned long long* tr) {
-  KTrace kt(tr);
-  pdl_launch_dependents();
-  pdl_wait();
-  if (threadIdx.x == 0) trace_mark_min(tr, 2);
-  int m = blockIdx.x, b = m / rows.R, i = m % rows.R;
-  if (i >= rows.cnt[b]) return;
-  int D = g.head_dim, half = D >> 1, Hkv = g.n_kv_heads;
-  int nq = H * D, nk = Hkv * D, ld = nq + 2 * nk;
-  int pos = rows.pos[m], slot = rows.slot[m];
-  int page = page_table[rows.sequence(b) * g.pages_per_seq + slot / g.page_size], prow = slot % g.page_size;
-  const float* src = qkv + (size_t)m * ld;
-  // q and k pairs
-  int npairs = (H + Hkv) * half;
-  for (int p = threadIdx.x; p < npairs; p += blockDim.x) {
-    int head = p / half, e = p % half;
-    int col = head * D + e;
-    const float a = src[col], c = src[col + half];
-    float2 t = cs[(size_t)pos * half + e];
-    float r0 = a * t.x - c * t.y, r1 = c * t.x + a * t.y;
-    if (head < H) {
-      q[(size_t)m * nq + head * D + e] = from_f<T>(r0);
-      q[(size_t)m * nq + head * D + e + half] = from_f<T>(r1);
-    } else {
-      int kh = head - H;
-      T* dst = pool + g.block_offset(page, layer, 0, kh) + (size_t)prow * D;
-      dst[kv_elem<T>(prow, e, D, g.page_size)] = from_f<T>(r0);
-      dst[kv_elem<T>(prow, e + half, D, g.page_size)] = from_f<T>(r1);
-    }
-  }
-  for (int p = threadIdx.x; p < nk; p += blockDim.x) {
-    int kh = p / D, e = p % D;
-    const float a = src[nq + nk + p];
-    T* dst = pool + g.block_offset(page, layer, 1, kh) + (size_t)prow * D;
-    dst[kv_elem<T>(prow, e, D, g.page_size)] = from_f<T>(a);
-  }
 }
 
 // ------------------------------------------------------------------ plain tree attention

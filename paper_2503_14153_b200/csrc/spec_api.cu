@@ -935,7 +935,7 @@ int run_gemm_glu(spec_ctx* c, const void* in, int M, int K, int cs, const void* 
 struct RowBest { float* val; int* idx; int tiles, tile, piece; };
 template <typename T, int MODE>
 int linear_simple(spec_ctx* c, const char* name, const T* x, int n_mats, const void* const* mats, const int* rows, float* y, size_t ldy, T* act,
-                  int M, int K, RowBest* best = nullptr) {
+                  int M, int K, RowBest* best = nullptr, const RopeStore<T>* rope = nullptr) {
   RowLinear<T> w{};
   w.n_mats = n_mats;
   int groups = 0;
@@ -955,7 +955,7 @@ int linear_simple(spec_ctx* c, const char* name, const T* x, int n_mats, const v
               at.val, at.idx);
       return SPEC_OK;
     }
-  KLAUNCH(name, (linear_rows<T, MODE>), sh.grid, dim3(LR_WARPS * 32), 0, x, w, y, ldy, act, M, K, groups, sh.ks, sh.ms);
+  KLAUNCH(name, (linear_rows<T, MODE>), sh.grid, dim3(LR_WARPS * 32), 0, x, w, y, ldy, act, M, K, groups, sh.ks, sh.ms, rope ? *rope : RopeStore<T>{});
   return SPEC_OK;
 }
 
@@ -1490,10 +1490,9 @@ int forward_layers(spec_ctx* c, const Rows& rows, const int* n_hi_pass, const in
     {
       const void* mats[3] = {c->wq[l], c->wk[l], c->wv[l]};
       const int rws[3] = {HD, KD, KD};
-      if ((r = linear_simple<T, LR_PLAIN>(c, "linear_qkv", u, 3, mats, rws, c->d_part, c->Nqkv, nullptr, M, d))) return r;
+      const RopeStore<T> rs{rows, c->d_rope, q, pool, c->geom, c->d_page_table, l, H};
+      if ((r = linear_simple<T, LR_ROPE>(c, "linear_qkv", u, 3, mats, rws, nullptr, 0, nullptr, M, d, nullptr, &rs))) return r;
     }
-    KLAUNCH("rope_store", rope_store<T>, dim3(M), dim3(256), 0, (const float*)c->d_part, rows, (const float2*)c->d_rope, q, pool, c->geom,
-            (const int*)c->d_page_table, l, H);
     switch (D / 32) {
       case 1: r = launch_attention_plain<T, 1>(c, rows, l); break;
       case 2: r = launch_attention_plain<T, 2>(c, rows, l); break;
@@ -2534,7 +2533,7 @@ int op_linear_f32(const void* x, const void* w, float* y, int M, int N, int K, c
     const HeldShape h = linear_held_shape(sh, M, N);
     (h.cols == 8 ? linear_rows_held<8, 4> : linear_rows_held<4, 8>)<<<h.grid, LR_WARPS * 32, 0, st>>>(xf, rl.w[0], y, (size_t)N, M, N, K, h.ms, nullptr, nullptr, nullptr);
   } else {
-    linear_rows<float, LR_PLAIN><<<sh.grid, LR_WARPS * 32, 0, st>>>(xf, rl, y, (size_t)N, nullptr, M, K, groups, sh.ks, sh.ms, nullptr);
+    linear_rows<float, LR_PLAIN><<<sh.grid, LR_WARPS * 32, 0, st>>>(xf, rl, y, (size_t)N, nullptr, M, K, groups, sh.ks, sh.ms, RopeStore<float>{}, nullptr);
   }
   return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_E_CUDA;
 }

@@ -83,3 +83,26 @@ def test_warps_of_a_row_vs_oracle(torch, hd, heads, kv, nodes):
                      topk=(4, 2, 2) if nodes <= 29 else (10, 4, 2, 2), n_medusa=3 if nodes <= 29 else 4)
     rep = run_lockstep(cfg, draw_weights(cfg), build_tree(cfg.topk, nodes), draw_prompt(cfg, 50), 8, 1e-4, 1e-2)
     assert rep.steps > 0
+
+
+@pytest.mark.parametrize("hd,heads,kv", [(32, 4, 2), (64, 4, 4), (160, 2, 1)])
+def test_rows_of_ragged_prompts(torch, hd, heads, kv):
+    """Queries, keys and values out of one projection for prompts that leave rows of the pass empty: every prompt as by itself, bit for bit."""
+    import numpy as np
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = get_config("c0", name="ragged", n_heads=heads, n_kv_heads=kv, head_dim=hd, vocab=2000, seed=hd, norm_gain="random")
+    w = upload_weights(cfg, draw_weights(cfg))
+    prompts = [draw_prompt(cfg.with_(seed=40 + i), n) for i, n in enumerate((1, 37, 150))]
+
+    def run(ps):
+        dec = SpecDecoder(cfg, w, build_tree(cfg.topk, cfg.tree_nodes), 256, max_batch=len(ps))
+        dec.prefill(ps)
+        for _ in range(3):
+            dec.step()
+        h = np.array(dec.debug(B.DBG_H_LAST))
+        dec.close()
+        return h
+    together = run(prompts)
+    for i, p in enumerate(prompts):
+        assert np.array_equal(run([p])[0], together[i]), i
