@@ -2178,8 +2178,11 @@ int spec_prefill(spec_ctx* c, int32_t batch, const int32_t* tokens, const int32_
 int spec_step(spec_ctx* c, int32_t* out_tokens, int32_t* out_counts, const int32_t* cand_override) {
   if (!c) return SPEC_E_BADARG;
   if (!c->prefilled) return c->fail(SPEC_E_STATE, "spec_step before spec_prefill");
-  return c->cfg.dtype == 1 ? step_t<bf16>(c, out_tokens, out_counts, cand_override)
-                           : step_t<float>(c, out_tokens, out_counts, cand_override);
+  const int r = c->cfg.dtype == 1 ? step_t<bf16>(c, out_tokens, out_counts, cand_override)
+                                  : step_t<float>(c, out_tokens, out_counts, cand_override);
+  // (a failed step may have moved the device's lengths on while the host's bounds stay: what later ones write is not known here)
+  if (r != SPEC_OK) c->written.assign(c->cfg.max_batch, c->cap);
+  return r;
 }
 
 int spec_read_generated(spec_ctx* c, int32_t seq, int32_t* out, int32_t max_tokens, int32_t* n_generated) {

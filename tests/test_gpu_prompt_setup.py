@@ -53,3 +53,28 @@ def test_nothing_left_of_earlier_prompts(dtype, max_batch, rounds):
         for x, y in zip(a, b):
             assert x.tobytes() == y.tobytes()
     used.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_nothing_left_of_failed_steps(dtype):
+    """Steps that report an error (a candidate outside the vocabulary) move a sequence on all the same: the next prompt clears what all of them have
+    written, not what the first one could have."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2503_14153_b200 import SpecDecoder, SpecError, build_tree, upload_weights
+    from synthetic import draw_weights
+    cfg = get_config("c0", name="setup", n_layers=2, d_model=256, n_heads=4, n_kv_heads=2, head_dim=64, d_ffn=704, vocab=1000, dtype=dtype, rope_base=1e6,
+                     n_medusa=3, topk=(4, 2, 2), tree_nodes=9, seed=3)
+    dec = SpecDecoder(cfg, upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, 9), 400, max_batch=1)
+    rng = np.random.default_rng(2)
+    dec.prefill(rng.integers(0, cfg.vocab, 300).astype(np.int32))
+    outside = np.full((1, cfg.n_medusa, dec.kmax), cfg.vocab, np.int32)
+    for _ in range(40):
+        with pytest.raises(SpecError):
+            dec.step(outside)
+    assert any(kv.any() for kv in dec.read_kv(0, 1, 336, 12))             # (beyond the page that a step at the prompt's end reaches)
+    dec.prefill(rng.integers(0, cfg.vocab, 20).astype(np.int32))
+    for kv in dec.read_kv(0, 1, 32, 368):
+        assert not kv.any()
+    dec.close()
