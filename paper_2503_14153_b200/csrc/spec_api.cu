@@ -1694,6 +1694,13 @@ int check_status(spec_ctx* c) {
   return report_status(c, c->h_result);
 }
 
+// Waits for a stream at the end of its scope, unless that has been done.
+struct StreamWait {
+  cudaStream_t st;
+  bool through = false;
+  ~StreamWait() { if (!through) cudaStreamSynchronize(st); }
+};
+
 template <typename T>
 int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offsets) {
   const spec_config& f = c->cfg;
@@ -1746,6 +1753,7 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
     }
     ch += g;
   }
+  StreamWait wait{c->stream};     // (page-locked tokens are read until their copy is through, which a return with an error must not leave behind)
   CUDA_OK(cudaMemcpyAsync(c->d_prompt, tokens + offsets[0], (size_t)off[batch] * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   const int pair_vecs = (int)(c->geom.block_elems() * 2 * c->esz / 16);   // 16-byte vectors of a page's K and V of one layer and head
   const int lh = f.n_layers * f.n_kv_heads, most_share = (int)std::max<long long>(1, std::min<long long>(c->pages_per_seq, 8 * SM_SLOTS / ((long long)lh * f.max_batch)));
@@ -1830,6 +1838,7 @@ int prefill_t(spec_ctx* c, int batch, const int32_t* tokens, const int32_t* offs
             (const int*)c->d_path, (const int*)c->d_count, f.temperature, f.seed_lo, f.seed_hi, c->d_draws, c->d_root, 1);
   }
   // (accept_kernel has put the status word into host memory)
+  wait.through = true;
   CUDA_OK(cudaStreamSynchronize(c->stream));
   if ((r = report_status(c, c->h_result))) return r;
   for (int b = 0; b < f.max_batch; ++b) c->written[b] = b < batch ? off[b + 1] - off[b] : 0;

@@ -78,3 +78,31 @@ def test_nothing_left_of_failed_steps(dtype):
     for kv in dec.read_kv(0, 1, 32, 368):
         assert not kv.any()
     dec.close()
+
+
+def test_failed_prompt_waits_for_its_copies():
+    """A prompt whose processing ends with an error on the host (here a lm_head that no tensor map takes, after the layers have been enqueued) is
+    returned from when the stream is through: page-locked tokens are the caller's again."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from synthetic import draw_weights
+    cfg = get_config("c0", name="setup", n_layers=2, d_model=256, n_heads=4, n_kv_heads=2, head_dim=64, d_ffn=704, vocab=1000, dtype="bf16", rope_base=1e6,
+                     n_medusa=3, topk=(4, 2, 2), tree_nodes=9, seed=3)
+    w = upload_weights(cfg, draw_weights(cfg))
+    odd = torch.zeros(cfg.vocab * cfg.d_model + 1, dtype=torch.bfloat16, device="cuda")
+    odd[1:] = w["lm_head"].reshape(-1)
+    w["lm_head"] = odd[1:].view(cfg.vocab, cfg.d_model)                   # two bytes off the boundary
+    dec = SpecDecoder(cfg, w, build_tree(cfg.topk, 9), 100, packed=False)
+    tokens, offsets = torch.zeros(30, dtype=torch.int32).pin_memory(), np.array([0, 30], np.int32)
+    a = torch.randn((8192, 8192), device="cuda").bfloat16()
+    assert dec.lib.spec_prefill(dec._ctx, 1, tokens.data_ptr(), offsets.ctypes.data) != 0     # (a kernel's first launch loads it, which may wait by itself)
+    a @ a
+    torch.cuda.synchronize()
+    for _ in range(60):                                                   # some 40 ms of work before the prompt's
+        a @ a
+    assert not dec.stream.query()
+    assert dec.lib.spec_prefill(dec._ctx, 1, tokens.data_ptr(), offsets.ctypes.data) != 0
+    assert dec.stream.query()
+    dec.close()
