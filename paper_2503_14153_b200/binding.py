@@ -31,7 +31,7 @@ EXPORTS = ["spec_workspace_bytes", "spec_create", "spec_prefill", "spec_step", "
            "spec_op_linear", "spec_op_linear_scratch_floats", "spec_op_linear_static", "spec_packed_weight_bytes",
            "spec_pack_weight", "spec_set_option", "spec_trace_read", "spec_build_labels", "spec_last_step_phase_ms", "spec_profile_kernel",
            "spec_profile_read", "spec_debug_wait_timeout", "spec_debug_pinned_allocations",
-           "spec_debug_op_wait_timeout"]
+           "spec_debug_op_wait_timeout", "spec_debug_cluster_residency"]
 
 
 class SpecError(RuntimeError):
@@ -122,6 +122,8 @@ def load_library():
     lib.spec_debug_op_wait_timeout.argtypes = [C.c_int32, C.c_int32, C.c_void_p, C.c_void_p]
     lib.spec_debug_pinned_allocations.restype = C.c_int
     lib.spec_debug_pinned_allocations.argtypes = []
+    lib.spec_debug_cluster_residency.restype = C.c_int
+    lib.spec_debug_cluster_residency.argtypes = [C.c_int32] * 5 + [C.c_void_p]
     lib.spec_profile_kernel.restype = C.c_int
     lib.spec_profile_kernel.argtypes = [C.c_void_p, C.c_int32]
     lib.spec_profile_read.restype = C.c_int

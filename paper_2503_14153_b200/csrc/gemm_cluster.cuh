@@ -91,18 +91,23 @@ template <int MT> struct ClusterCfg {
   static constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + EXTRA_BYTES; }
 };
 
-// Stages of a launch of `ctas` CTAs with at most `units` K chunks each. A grid of more than one CTA an SM gets the ring of which two fit.
-// A smaller one (the projections of narrow models: at d_model 1024 q/k/v has 24 CTAs of 8 chunks, gate+up 66 of 11) gets a stage for every
-// chunk as far as shared memory goes, so that all of a CTA's weights are under way before the dependency wait and the chain behind it is
-// activation tiles, MMAs and the exchange. Six layers of d_model 1024, 64 rows: gate+up 10.3 -> 8.4 us, down 6.2 -> 4.9, a step 284 -> 263.
+// Clusters of `size` CTAs that the chip holds at one CTA an SM (cudaOccupancyMaxActiveClusters): a cluster lies within a group of neighbouring SMs, so
+// 15 clusters of eight fit, not 18.
+constexpr int CLUSTERS_ALONE[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+
+// Stages of a launch of `tiles` clusters of `cluster` CTAs with at most `units` K chunks each. Where all clusters fit at one CTA an SM (the projections
+// of narrow models: at d_model 1024 q/k/v has 24 CTAs of 8 chunks, gate+up 66 of 11) a CTA gets a stage for every
+// chunk as far as shared memory goes, so that all of its weights are under way before the dependency wait and the chain behind it is
+// activation tiles, MMAs and the exchange: a 64-row step of six layers of d_model 1024 284 -> 263 us. The others get the ring of which two fit an SM:
+// with the deep one the last clusters run when the first ones are through (eight layers of 64 rows, d_model 2048, ffn 6144, down in 16 clusters of
+// eight: 468 us with the deep ring, 399 with the shallow one).
 // Of more than one CTA an SM with short runs and 16 rows (wo of the 7B shape: 32 clusters of 8 CTAs, 8 chunks each) three fit an SM: the attention
 // before it has 32 CTAs, and with two an SM a few clusters did not find room beside those and began when it ended: wo 9.9 -> 7.5 us.
 // (With 64 rows attention has 128 CTAs and three stages cost more than they give: 10.1 -> 10.8.)
-template <int MT> inline int cluster_stages(int ctas, int units) {
+template <int MT> inline int cluster_stages(int tiles, int cluster, int units) {
   using Cfg = ClusterCfg<MT>;
-  if (ctas > 148 && MT == 16 && units <= 8) return 4;
-  if (ctas > 148 || units <= Cfg::STAGES) return Cfg::STAGES;
-  return units < Cfg::MAX_STAGES ? units : Cfg::MAX_STAGES;
+  if (tiles > CLUSTERS_ALONE[cluster]) return MT == 16 && tiles * cluster > 148 && units <= 8 ? 4 : Cfg::STAGES;
+  return units <= Cfg::STAGES ? Cfg::STAGES : (units < Cfg::MAX_STAGES ? units : Cfg::MAX_STAGES);
 }
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {

@@ -196,24 +196,48 @@ cudaError_t launch_gs(cudaStream_t st, bool pdl, const GemmPlan& g, const Stream
   }
 }
 
+// The launch of gemm_cluster<MT, MODE> over `tiles` clusters of `cluster` CTAs with a ring of `stages`.
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[2];
+  ClusterLaunch(cudaStream_t st, bool pdl, int tiles, int cluster, size_t smem) {
+    cfg.gridDim = dim3(tiles * cluster); cfg.blockDim = dim3(GC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 2 : 1;
+  }
+};
+template <int MT, int MODE> cudaError_t allow_deepest_ring() {
+  return cudaFuncSetAttribute(gemm_cluster<MT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<MT>::smem_bytes(ClusterCfg<MT>::MAX_STAGES));
+}
+template <int MODE> int cluster_units(int KC, int cluster) { return ((MODE == GC_SWIGLU ? 2 : 1) * KC + cluster - 1) / cluster; }   // K chunks of a CTA, at most
+
 template <int MT, int MODE>
-cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int grid, int cluster, const StreamTmaps& tm, ClusterGemmParams p, bool* attr_set) {
+cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int tiles, int cluster, const StreamTmaps& tm, ClusterGemmParams p, bool* attr_set) {
   if (!*attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_cluster<MT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<MT>::smem_bytes(ClusterCfg<MT>::MAX_STAGES));
+    cudaError_t e = allow_deepest_ring<MT, MODE>();
     if (e != cudaSuccess) return e;
     *attr_set = true;
   }
-  p.stages = cluster_stages<MT>(grid, ((MODE == GC_SWIGLU ? 2 : 1) * p.KC + cluster - 1) / cluster);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GC_THREADS); cfg.dynamicSmemBytes = (size_t)ClusterCfg<MT>::smem_bytes(p.stages); cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, gemm_cluster<MT, MODE>, tm, p);
+  p.stages = cluster_stages<MT>(tiles, cluster, cluster_units<MODE>(p.KC, cluster));
+  ClusterLaunch l(st, pdl, tiles, cluster, (size_t)ClusterCfg<MT>::smem_bytes(p.stages));
+  return cudaLaunchKernelEx(&l.cfg, gemm_cluster<MT, MODE>, tm, p);
+}
+
+// Stages that such a launch takes, and the clusters that the device holds at once with them and with the ring of which two CTAs fit an SM.
+template <int MT, int MODE>
+cudaError_t cluster_residency(int tiles, int cluster, int KC, int* out) {
+  cudaError_t e = allow_deepest_ring<MT, MODE>();
+  out[0] = cluster_stages<MT>(tiles, cluster, cluster_units<MODE>(KC, cluster));
+  const int stages[2] = {out[0], ClusterCfg<MT>::STAGES};
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+    ClusterLaunch l(nullptr, false, tiles, cluster, (size_t)ClusterCfg<MT>::smem_bytes(stages[i]));
+    e = cudaOccupancyMaxActiveClusters(&out[1 + i], gemm_cluster<MT, MODE>, &l.cfg);
+  }
+  return e;
 }
 
 // CTAs that share each tile of a GC_PLAIN launch: as many as let all clusters be resident at once (96 KB of shared memory a CTA) and have
@@ -228,10 +252,10 @@ int plain_cluster(int tiles, int KC, int max_ctas) {
 cudaError_t launch_gc_plain(cudaStream_t st, bool pdl, int tiles, int cluster, const StreamTmaps& tm, const ClusterGemmParams& p) {
   static bool set[4][kAttrDevices] = {};
   switch (mt_for_rows(p.M)) {
-    case 16: return launch_gc_mt<16, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[0]));
-    case 32: return launch_gc_mt<32, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[1]));
-    case 64: return launch_gc_mt<64, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[2]));
-    default: return launch_gc_mt<128, GC_PLAIN>(st, pdl, tiles * cluster, cluster, tm, p, attr_flag(set[3]));
+    case 16: return launch_gc_mt<16, GC_PLAIN>(st, pdl, tiles, cluster, tm, p, attr_flag(set[0]));
+    case 32: return launch_gc_mt<32, GC_PLAIN>(st, pdl, tiles, cluster, tm, p, attr_flag(set[1]));
+    case 64: return launch_gc_mt<64, GC_PLAIN>(st, pdl, tiles, cluster, tm, p, attr_flag(set[2]));
+    default: return launch_gc_mt<128, GC_PLAIN>(st, pdl, tiles, cluster, tm, p, attr_flag(set[3]));
   }
 }
 
@@ -837,30 +861,30 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
     p.pool = static_cast<bf16*>(c->d_pool); p.g = c->geom; p.page_table = c->d_page_table;
   }
   p.trace = c->next_trace(gemm_kind_name(kind));
-  const int cs = mode == GC_SWIGLU ? GC_GLU_CLUSTER : mode == GC_ROPE ? GC_ROPE_CLUSTER : GC_RES_CLUSTER, grid = n_tiles * cs;
+  const int cs = mode == GC_SWIGLU ? GC_GLU_CLUSTER : mode == GC_ROPE ? GC_ROPE_CLUSTER : GC_RES_CLUSTER;
   cudaError_t e = cudaErrorInvalidValue;
   {
     ProfScope ps(c, kind);
     bool* as = c->gc_attr_set;
     if (mode == GC_RESIDUAL) {
       switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 0); break;
-        case 32: e = launch_gc_mt<32, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 1); break;
-        case 64: e = launch_gc_mt<64, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 2); break;
-        default: e = launch_gc_mt<128, GC_RESIDUAL>(c->stream, c->pdl, grid, cs, tm, p, as + 3); break;
+        case 16: e = launch_gc_mt<16, GC_RESIDUAL>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 0); break;
+        case 32: e = launch_gc_mt<32, GC_RESIDUAL>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 1); break;
+        case 64: e = launch_gc_mt<64, GC_RESIDUAL>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 2); break;
+        default: e = launch_gc_mt<128, GC_RESIDUAL>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 3); break;
       }
     } else if (mode == GC_SWIGLU) {
       switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 4); break;
-        case 32: e = launch_gc_mt<32, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 5); break;
-        default: e = launch_gc_mt<64, GC_SWIGLU>(c->stream, c->pdl, grid, cs, tm, p, as + 6); break;
+        case 16: e = launch_gc_mt<16, GC_SWIGLU>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 4); break;
+        case 32: e = launch_gc_mt<32, GC_SWIGLU>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 5); break;
+        default: e = launch_gc_mt<64, GC_SWIGLU>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 6); break;
       }
     } else {
       switch (MT) {
-        case 16: e = launch_gc_mt<16, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 7); break;
-        case 32: e = launch_gc_mt<32, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 8); break;
-        case 64: e = launch_gc_mt<64, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 9); break;
-        default: e = launch_gc_mt<128, GC_ROPE>(c->stream, c->pdl, grid, cs, tm, p, as + 10); break;
+        case 16: e = launch_gc_mt<16, GC_ROPE>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 7); break;
+        case 32: e = launch_gc_mt<32, GC_ROPE>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 8); break;
+        case 64: e = launch_gc_mt<64, GC_ROPE>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 9); break;
+        default: e = launch_gc_mt<128, GC_ROPE>(c->stream, c->pdl, n_tiles, cs, tm, p, as + 10); break;
       }
     }
     c->launches++;
@@ -871,15 +895,14 @@ int run_gemm_cluster(spec_ctx* c, int mode, const void* in, int M, int K, const 
 
 // CTAs that share a (gate tile, up tile) pair in gemm_glu, 0 where the weight streamer and swiglu_reduce_tc serve: the streamer's plan has to cut the K chunks
 // of every tile into the same runs (then it has no run that crosses a tile), at most eight, and all clusters have to fit the chip at one CTA
-// an SM (cudaOccupancyMaxActiveClusters): a second wave would wait for the whole chain of the first.
+// an SM: a second wave would wait for the whole chain of the first.
 int glu_cluster(const spec_ctx* c, int M, int K) {
   if (!(c->cluster_epilogue & 2) || M <= 64 || M > 128 || K % 64) return 0;
   const int F = c->cfg.d_ffn, tiles = 2 * ((F + 127) / 128), rows[2] = {F, F};
   GemmPlan g;
   if (!plan_gemm(M, K, 2, rows, stream_ctas(c, tiles), &g) || g.grid % tiles) return 0;
-  constexpr int most[GLU_MAX_CLUSTER + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
   const int cs = g.grid / tiles;
-  return cs <= GLU_MAX_CLUSTER && tiles / 2 <= most[cs] ? cs : 0;
+  return cs <= GLU_MAX_CLUSTER && tiles / 2 <= CLUSTERS_ALONE[cs] ? cs : 0;
 }
 
 int run_gemm_glu(spec_ctx* c, const void* in, int M, int K, int cs, const void* const* mats, bf16* act) {
@@ -2564,6 +2587,29 @@ int spec_debug_op_wait_timeout(int32_t limit_us, int32_t pinned, int32_t* words,
   wait_probe<<<1, 32, 0, st>>>(status.report(), (unsigned long long)limit_us * 1000ull);
   if (cudaGetLastError() != cudaSuccess) return SPEC_E_CUDA;
   return status.finish();
+}
+
+int spec_debug_cluster_residency(int32_t mode, int32_t rows, int32_t tiles, int32_t cluster, int32_t chunks, int32_t* out) {
+  constexpr int size[4] = {GC_RES_CLUSTER, GC_GLU_CLUSTER, GC_ROPE_CLUSTER, 0};
+  if (!out || mode < 0 || mode > 3 || rows < 1 || rows > (mode == GC_SWIGLU ? 64 : 128) || tiles < 1 || tiles > 1024 || chunks < 1 || chunks > 4096) return SPEC_E_BADARG;
+  if (cluster < 1 || cluster > 8 || (size[mode] && cluster != size[mode])) return SPEC_E_BADARG;
+  cudaError_t e = cudaErrorInvalidValue;
+#define MODES(MT)                                                                       \
+  switch (mode) {                                                                       \
+    case GC_RESIDUAL: e = cluster_residency<MT, GC_RESIDUAL>(tiles, cluster, chunks, out); break; \
+    case GC_ROPE: e = cluster_residency<MT, GC_ROPE>(tiles, cluster, chunks, out); break;         \
+    case GC_PLAIN: e = cluster_residency<MT, GC_PLAIN>(tiles, cluster, chunks, out); break;       \
+    default:                                                                            \
+      if constexpr (MT < 128) e = cluster_residency<MT, GC_SWIGLU>(tiles, cluster, chunks, out);  \
+  }
+  switch (mt_for_rows(rows)) {
+    case 16: MODES(16) break;
+    case 32: MODES(32) break;
+    case 64: MODES(64) break;
+    default: MODES(128) break;
+  }
+#undef MODES
+  return e == cudaSuccess ? SPEC_OK : SPEC_E_CUDA;
 }
 
 int spec_debug_pinned_allocations(void) { return status_words().allocations(); }
