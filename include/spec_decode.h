@@ -265,8 +265,8 @@ int spec_debug_pinned_allocations(void);
 
 /* How a cluster projection is launched (mode 0: output and down, clusters of 8; 1: gate+up of at most 64 rows, of 3; 2: q/k/v, of 2; 3: a projection by
  * itself, of 1 to 8) over `rows` <= 128 activation rows, `tiles` clusters and `chunks` K chunks of 64: out[0] stages of the weight ring, out[1] clusters that
- * the device holds at once with it, out[2] with the ring of which two CTAs fit an SM. Launches nothing. */
-int spec_debug_cluster_residency(int32_t mode, int32_t rows, int32_t tiles, int32_t cluster, int32_t chunks, int32_t *out /* HOST [3] */);
+ * the device holds at once at one CTA an SM. Launches nothing. */
+int spec_debug_cluster_residency(int32_t mode, int32_t rows, int32_t tiles, int32_t cluster, int32_t chunks, int32_t *out /* HOST [2] */);
 
 /* ---- single operations of the verify forward, for unit parity tests and profiling ---- */
 

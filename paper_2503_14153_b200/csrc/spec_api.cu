@@ -227,17 +227,15 @@ cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int tiles, int cluster, cons
   return cudaLaunchKernelEx(&l.cfg, gemm_cluster<MT, MODE>, tm, p);
 }
 
-// Stages that such a launch takes, and the clusters that the device holds at once with them and with the ring of which two CTAs fit an SM.
+// Stages that such a launch takes, and the clusters of it that the device holds at once at one CTA an SM. (At two an SM the runtime does not tell: for
+// kernels with tensor memory it answers one CTA an SM whatever their shared memory.)
 template <int MT, int MODE>
 cudaError_t cluster_residency(int tiles, int cluster, int KC, int* out) {
   cudaError_t e = allow_deepest_ring<MT, MODE>();
+  if (e != cudaSuccess) return e;
   out[0] = cluster_stages<MT>(tiles, cluster, cluster_units<MODE>(KC, cluster));
-  const int stages[2] = {out[0], ClusterCfg<MT>::STAGES};
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-    ClusterLaunch l(nullptr, false, tiles, cluster, (size_t)ClusterCfg<MT>::smem_bytes(stages[i]));
-    e = cudaOccupancyMaxActiveClusters(&out[1 + i], gemm_cluster<MT, MODE>, &l.cfg);
-  }
-  return e;
+  ClusterLaunch l(nullptr, false, tiles, cluster, (size_t)ClusterCfg<MT>::smem_bytes(ClusterCfg<MT>::MAX_STAGES));
+  return cudaOccupancyMaxActiveClusters(&out[1], gemm_cluster<MT, MODE>, &l.cfg);
 }
 
 // CTAs that share each tile of a GC_PLAIN launch: as many as let all clusters be resident at once (96 KB of shared memory a CTA) and have

@@ -34,21 +34,18 @@ def test_ring_depths(torch, M, chunks):
 
 @pytest.mark.parametrize("mode,cluster", [(0, 8), (1, 3), (2, 2), (3, 1), (3, 2), (3, 3), (3, 4), (3, 6), (3, 8)])
 def test_rings_leave_no_cluster_waiting(torch, mode, cluster):
-    """Whatever the number of weight tiles, as many clusters of a launch are on the chip at once as with the ring of which two CTAs fit an SM; the deep ring is
-    taken as long as all of them are with one CTA an SM."""
+    """A ring that fills an SM is taken as long as all clusters of the launch are on the chip at once with it, the one of which two fit an SM beyond."""
     import ctypes as C
     from paper_2503_14153_b200 import load_library
-    lib, out = load_library(), (C.c_int32 * 3)()
+    lib, out = load_library(), (C.c_int32 * 2)()
 
     def launch(rows, tiles, chunks):
         assert lib.spec_debug_cluster_residency(mode, rows, tiles, cluster, chunks, out) == 0
         return list(out)
     for rows in (1, 16, 17, 64) + ((65, 128) if mode != 1 else ()):
         two_an_sm = 5 if rows <= 32 else (4 if rows <= 64 else 3)
-        alone = launch(rows, 1, 16 * cluster)[1]              # (16 chunks a CTA, of gate and up 32: more than the deepest ring has stages)
-        for tiles in range(1, 160 // cluster + 2):
-            stages, now, shallow = launch(rows, tiles, 16 * cluster)
-            assert now >= min(tiles, shallow), (rows, tiles, stages, now, shallow)
+        for tiles in range(1, 160 // cluster + 2):            # (16 chunks a CTA, of gate and up 32: more than the deepest ring has stages)
+            stages, alone = launch(rows, tiles, 16 * cluster)
             assert (stages > two_an_sm) == (tiles <= alone), (rows, tiles, stages, alone)
 
 
