@@ -51,7 +51,7 @@ constexpr int GC_RES_CLUSTER = 8, GC_GLU_CLUSTER = 3, GC_ROPE_CLUSTER = 2;
 
 struct ClusterGemmParams {
   int M, K, KC;                 // activation rows (<= MT), inner size, K / 64
-  int stages;                   // of the ring: ClusterCfg<MT>::STAGES to MAX_STAGES (see cluster_stages)
+  int stages;                   // of the ring: ClusterCfg<MT>::FEWEST_STAGES to MAX_STAGES (see cluster_stages)
   int N;                        // weight rows of one matrix (output columns)
   const uint8_t* packed[3];     // pre-tiled images (GC_RESIDUAL: [0]; GC_SWIGLU: gate, up; GC_ROPE: q, k, v) or nullptr -> tensor maps a[i]
   float* x;                     // GC_RESIDUAL: [M][N] float32 residual stream, updated in place
@@ -85,7 +85,7 @@ template <int MT> struct ClusterCfg {
   static constexpr int B_BYTES = MT * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = (MT <= 32) ? 5 : (MT == 64 ? 4 : 3);      // two CTAs an SM
-  static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
+  static constexpr int FEWEST_STAGES = MT == 16 ? 4 : STAGES;             // three (GC_RESIDUAL)
   static constexpr int EXTRA_BYTES = 1024 /*alignment slack*/ + 256 /*barriers*/;
   static constexpr int MAX_STAGES = (227 * 1024 - EXTRA_BYTES) / STAGE_BYTES < 12 ? (227 * 1024 - EXTRA_BYTES) / STAGE_BYTES : 12;   // one CTA an SM
   static constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + EXTRA_BYTES; }
@@ -101,12 +101,12 @@ constexpr int CLUSTERS_ALONE[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
 // activation tiles, MMAs and the exchange: a 64-row step of six layers of d_model 1024 284 -> 263 us. The others get the ring of which two fit an SM:
 // with the deep one the last clusters run when the first ones are through (eight layers of 64 rows, d_model 2048, ffn 6144, down in 16 clusters of
 // eight: 468 us with the deep ring, 399 with the shallow one).
-// Of more than one CTA an SM with short runs and 16 rows (wo of the 7B shape: 32 clusters of 8 CTAs, 8 chunks each) three fit an SM: the attention
-// before it has 32 CTAs, and with two an SM a few clusters did not find room beside those and began when it ended: wo 9.9 -> 7.5 us.
-// (With 64 rows attention has 128 CTAs and three stages cost more than they give: 10.1 -> 10.8.)
-template <int MT> inline int cluster_stages(int tiles, int cluster, int units) {
+// The output and down projections of up to 16 rows in more clusters than that, with short runs (wo of the 7B shape: 32 clusters of 8 CTAs, 8 chunks
+// each), have a ring of which three fit an SM: the attention before wo has 32 CTAs, and with two an SM a few clusters did not find room beside those and
+// began when it ended: wo 9.9 -> 7.5 us. (With 64 rows attention has 128 CTAs and three stages cost more than they give: 10.1 -> 10.8.)
+template <int MT, int MODE> inline int cluster_stages(int tiles, int cluster, int units) {
   using Cfg = ClusterCfg<MT>;
-  if (tiles > CLUSTERS_ALONE[cluster]) return MT == 16 && tiles * cluster > 148 && units <= 8 ? 4 : Cfg::STAGES;
+  if (tiles > CLUSTERS_ALONE[cluster]) return MODE == GC_RESIDUAL && MT == 16 && tiles * cluster > 148 && units <= 8 ? Cfg::FEWEST_STAGES : Cfg::STAGES;
   return units <= Cfg::STAGES ? Cfg::STAGES : (units < Cfg::MAX_STAGES ? units : Cfg::MAX_STAGES);
 }
 
@@ -245,6 +245,7 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   const int n_units = (seg[0].kc1 - seg[0].kc0) + (nseg > 1 ? seg[1].kc1 - seg[1].kc0 : 0);
 
   // ---- layout of the exchange, in the ring: `in`, the parts of this CTA's outputs, then `out`, what it sends ----
+  constexpr int LEAST_BYTES = (MODE == GC_RESIDUAL ? Cfg::FEWEST_STAGES : Cfg::STAGES) * Cfg::STAGE_BYTES;   // of a ring
   const int M = p.M;
   // GC_ROPE: CTA 0 finishes activation rows [0, r_half), CTA 1 the rest
   const int r_half = (M + 1) / 2, r_row0 = rank * r_half, r_rows = MODE == GC_ROPE ? (rank ? M - r_half : r_half) : 0;
@@ -263,11 +264,11 @@ gemm_cluster(const __grid_constant__ StreamTmaps tm, const ClusterGemmParams p) 
   const int out_pitch = (S | 1) * 16;
   float* in = staging;
   float* out = staging + (MODE == GC_RESIDUAL ? GC_RES_CLUSTER * in_pitch : MODE == GC_SWIGLU ? 4 * glu_ng * in_pitch : PLAIN ? CS * rb * 128 : 2 * r_rows * 128);
-  static_assert(!PLAIN || Cfg::RING_BYTES >= (2 * RT + 8) * 512, "a round's rows staged, and eight parts of this CTA's block");
-  static_assert(MODE != GC_RESIDUAL || Cfg::RING_BYTES >= GC_RES_CLUSTER * MT * 64 + (GC_RES_CLUSTER - 1) * 64 * 17, "in, and 16 rows of out");
-  static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 3 + 5) * (RT | 1) * 64, "CTA 0 and 2: four parts of three groups, five groups to send");
-  static_assert(MODE != GC_SWIGLU || Cfg::RING_BYTES >= (4 * 2 + 2 * 6) * (RT | 1) * 64, "CTA 1: four parts of two groups, six groups of two accumulators");
-  static_assert(MODE != GC_ROPE || Cfg::RING_BYTES >= 3 * ((MT + 1) / 2) * 512, "own and arriving rows, rows to send");
+  static_assert(!PLAIN || LEAST_BYTES >= (2 * RT + 8) * 512, "a round's rows staged, and eight parts of this CTA's block");
+  static_assert(MODE != GC_RESIDUAL || LEAST_BYTES >= GC_RES_CLUSTER * MT * 64 + (GC_RES_CLUSTER - 1) * 64 * 17, "in, and 16 rows of out");
+  static_assert(MODE != GC_SWIGLU || LEAST_BYTES >= (4 * 3 + 5) * (RT | 1) * 64, "CTA 0 and 2: four parts of three groups, five groups to send");
+  static_assert(MODE != GC_SWIGLU || LEAST_BYTES >= (4 * 2 + 2 * 6) * (RT | 1) * 64, "CTA 1: four parts of two groups, six groups of two accumulators");
+  static_assert(MODE != GC_ROPE || LEAST_BYTES >= 3 * ((MT + 1) / 2) * 512, "own and arriving rows, rows to send");
   // bytes that arrive in a round of `rows` rows
   auto in_bytes = [&](int rows) -> uint32_t {
     return MODE == GC_RESIDUAL ? (GC_RES_CLUSTER - 1) * S * 64 : MODE == GC_SWIGLU ? (rank == 1 ? 2 : 3) * glu_ng * rows * 64 : PLAIN ? (CS - 1) * max(0, min(rb, rows - rank * rb)) * 512 : r_rows * 512;

@@ -222,7 +222,7 @@ cudaError_t launch_gc_mt(cudaStream_t st, bool pdl, int tiles, int cluster, cons
     if (e != cudaSuccess) return e;
     *attr_set = true;
   }
-  p.stages = cluster_stages<MT>(tiles, cluster, cluster_units<MODE>(p.KC, cluster));
+  p.stages = cluster_stages<MT, MODE>(tiles, cluster, cluster_units<MODE>(p.KC, cluster));
   ClusterLaunch l(st, pdl, tiles, cluster, (size_t)ClusterCfg<MT>::smem_bytes(p.stages));
   return cudaLaunchKernelEx(&l.cfg, gemm_cluster<MT, MODE>, tm, p);
 }
@@ -233,7 +233,7 @@ template <int MT, int MODE>
 cudaError_t cluster_residency(int tiles, int cluster, int KC, int* out) {
   cudaError_t e = allow_deepest_ring<MT, MODE>();
   if (e != cudaSuccess) return e;
-  out[0] = cluster_stages<MT>(tiles, cluster, cluster_units<MODE>(KC, cluster));
+  out[0] = cluster_stages<MT, MODE>(tiles, cluster, cluster_units<MODE>(KC, cluster));
   ClusterLaunch l(nullptr, false, tiles, cluster, (size_t)ClusterCfg<MT>::smem_bytes(ClusterCfg<MT>::MAX_STAGES));
   return cudaOccupancyMaxActiveClusters(&out[1], gemm_cluster<MT, MODE>, &l.cfg);
 }

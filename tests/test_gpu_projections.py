@@ -34,7 +34,8 @@ def test_ring_depths(torch, M, chunks):
 
 @pytest.mark.parametrize("mode,cluster", [(0, 8), (1, 3), (2, 2), (3, 1), (3, 2), (3, 3), (3, 4), (3, 6), (3, 8)])
 def test_rings_leave_no_cluster_waiting(torch, mode, cluster):
-    """A ring that fills an SM is taken as long as all clusters of the launch are on the chip at once with it, the one of which two fit an SM beyond."""
+    """A ring that fills an SM is taken as long as all clusters of the launch are on the chip at once with it, the one of which two fit an SM beyond, and the
+    one of which three do for output and down projections alone."""
     import ctypes as C
     from paper_2503_14153_b200 import load_library
     lib, out = load_library(), (C.c_int32 * 2)()
@@ -47,6 +48,7 @@ def test_rings_leave_no_cluster_waiting(torch, mode, cluster):
         for tiles in range(1, 160 // cluster + 2):            # (16 chunks a CTA, of gate and up 32: more than the deepest ring has stages)
             stages, alone = launch(rows, tiles, 16 * cluster)
             assert (stages > two_an_sm) == (tiles <= alone), (rows, tiles, stages, alone)
+        assert launch(rows, 296 // cluster, 4 * cluster)[0] == (4 if mode == 0 and rows <= 16 else two_an_sm)
 
 
 @pytest.mark.parametrize("N,chunks", [(1920, 90), (2048, 90), (2304, 96), (2944, 70), (4480, 50), (6144, 36)])
