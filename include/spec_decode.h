@@ -159,7 +159,7 @@ const char *spec_last_error(const spec_ctx *ctx);
 enum { SPEC_Q_KMAX = 0, SPEC_Q_KERNEL_LAUNCHES = 1, SPEC_Q_N_NODES = 2, SPEC_Q_BATCH = 3,
        SPEC_Q_ALGO_BYTES_PER_STEP = 4 /* weights + lm_head (twice) + heads, in KiB */,
        SPEC_Q_GRAPH_CAPTURES = 5 /* times a step was recorded into a CUDA graph */,
-       SPEC_Q_CLUSTER_GATE_UP = 6 /* 1 if a step's gate+up projection runs as the cluster kernel with the SwiGLU inside */,
+       SPEC_Q_CLUSTER_GATE_UP = 6 /* 1 if a step's gate+up projection runs as a cluster kernel with the SwiGLU inside */,
        SPEC_Q_WIDE_GEMM = 7 /* 1 if passes of more than 128 rows use the kernel that runs a tile on two SMs */ };
 int64_t spec_query(const spec_ctx *ctx, int32_t what);
 
@@ -182,7 +182,8 @@ int64_t spec_query(const spec_ctx *ctx, int32_t what);
  * those boundaries: about 0.03 ms of a 7B step). SPEC_OPT_CLUSTER_EPILOGUE [7]: bit mask of the projections
  * that, in passes of at most 128 rows, run as thread-block clusters which add their split-K sums through
  * distributed shared memory and apply the step that follows themselves: 1 = output and down projections
- * (residual add in place), 2 = gate+up (SwiGLU, passes of at most 64 rows), 4 = q/k/v (RoPE and cache
+ * (residual add in place), 2 = gate+up (SwiGLU; passes of at most 64 rows, of up to 128 where the weight streamer would cut all tiles into the same
+ * runs and all clusters fit the chip, with the streamer's sums), 4 = q/k/v (RoPE and cache
  * store). A projection whose bit is clear leaves partial sums for a separate kernel (other summation
  * order, same rounding points). All three are on by default: on the 7B shape they shorten a step by 2.2%,
  * 2% and 4.4%. SPEC_OPT_WIDE_GEMM [1]: passes of more than

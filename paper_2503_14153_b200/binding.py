@@ -386,7 +386,7 @@ class SpecDecoder:
         m = self.batch * self.T
         mt = 16 if m <= 16 else (32 if m <= 32 else (64 if m <= 64 else 128))
         if self.query(Q_CLUSTER_GATE_UP):
-            return f"gemm_cluster<{mt},swiglu>"
+            return f"gemm_cluster<{mt},swiglu>" if m <= 64 else "gemm_glu"
         return "gemm_pair<swiglu>" if m > 128 and self.query(Q_WIDE_GEMM) else f"gemm_stream<{mt}>"
 
     def query(self, what: int) -> int:

@@ -2263,7 +2263,7 @@ int64_t spec_query(const spec_ctx* c, int32_t what) {
     case SPEC_Q_BATCH: return c->B;
     case SPEC_Q_GRAPH_CAPTURES: return c->graph_captures;
     case SPEC_Q_WIDE_GEMM: return c->tc && c->wide_gemm ? 1 : 0;
-    case SPEC_Q_CLUSTER_GATE_UP: return c->tc && cluster_gemm_ok(c, GC_SWIGLU, c->B * c->T, f.d_model) ? 1 : 0;
+    case SPEC_Q_CLUSTER_GATE_UP: return c->tc && (cluster_gemm_ok(c, GC_SWIGLU, c->B * c->T, f.d_model) || glu_cluster(c, c->B * c->T, f.d_model)) ? 1 : 0;
     case SPEC_Q_ALGO_BYTES_PER_STEP: {
       double d = f.d_model, F = f.d_ffn, V = f.vocab, HD = (double)f.n_heads * f.head_dim, KD = (double)f.n_kv_heads * f.head_dim;
       double layer = d * HD + 2 * d * KD + HD * d + 3 * d * F;

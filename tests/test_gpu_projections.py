@@ -167,3 +167,24 @@ def test_two_chunks_at_once(torch, d, heads, kv, hd, ffn, n):
     assert np.isfinite(seen[1][1]).all() and np.abs(seen[1][1]).max() > 0.1
     for a, b in zip(seen[1], seen[0]):
         assert a.tobytes() == b.tobytes()
+
+
+@pytest.mark.parametrize("d,ffn,T,batch,kernel", [
+    (1024, 2752, 69, 1, "gemm_glu"), (1024, 2752, 23, 3, "gemm_glu"), (512, 2304, 128, 1, "gemm_stream<128>"),
+    (1024, 2752, 64, 1, "gemm_cluster<64,swiglu>"), (1024, 2752, 43, 3, "gemm_pair<swiglu>"),
+])
+def test_gate_up_kernel_name(torch, d, ffn, T, batch, kernel):
+    """The kernel that a decoder names for a step's gate and up projections is the one that runs: the streamer alone leaves the SwiGLU to another."""
+    import numpy as np
+    from paper_2503_14153_b200 import binding as B
+    from synthetic import get_config
+    cfg = get_config("c0", name="names", n_layers=1, d_model=d, n_heads=d // 128, n_kv_heads=d // 128, head_dim=128, d_ffn=ffn, vocab=1000, dtype="bf16",
+                     rope_base=1e6, n_medusa=4, topk=(10, 4, 2, 2), tree_nodes=T, batch=batch)
+    gpu = random_decoder(torch, cfg, 5, 160)
+    gpu.prefill([np.arange(20 + b, dtype=np.int32) for b in range(batch)])
+    gpu.set_option(B.OPT_TRACE, 1)
+    gpu.step()
+    ran = [r[0] for r in gpu.trace()]
+    assert gpu.gate_up_kernel_name() == kernel and gpu.query(B.Q_CLUSTER_GATE_UP) == (kernel[:8] in ("gemm_glu", "gemm_clu"))
+    assert ("swiglu_reduce_tc" in ran) == (kernel[:8] == "gemm_str")
+    gpu.close()
