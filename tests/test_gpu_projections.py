@@ -79,7 +79,7 @@ def random_decoder(torch, cfg, seed, max_seq):
 
 
 @pytest.mark.parametrize("d,ffn,T", [
-    (512, 1344, 65), (512, 1344, 96), (512, 1344, 97), (512, 2304, 128),      # clusters of eight (the second: too many of them, the streamer serves)
+    (512, 1344, 65), (512, 1344, 96), (512, 1344, 97), (512, 2304, 128),      # clusters of eight (the last: too many of them, the streamer serves)
     (512, 1920, 100), (1024, 2752, 69), (1024, 2752, 128),                    # eight again, six, two rounds
     (1280, 3200, 77), (1280, 3968, 113),                                      # five, four: a chunk more than stages
     (2048, 5248, 80), (2048, 7936, 66), (1024, 16000, 112),                   # three (11 chunks a CTA: the ring refilled), two, one
@@ -94,14 +94,17 @@ def test_gate_up_in_clusters_as_the_streamer(torch, d, ffn, T):
     cfg = get_config("c0", name="glu", n_layers=2, d_model=d, n_heads=d // 128, n_kv_heads=max(1, d // 256), head_dim=128, d_ffn=ffn, vocab=1000, dtype="bf16",
                      rope_base=1e6, n_medusa=4, topk=(10, 4, 2, 2), tree_nodes=T)
     prompt = np.random.default_rng(T).integers(0, 1000, 90).astype(np.int32)
-    seen = {}
+    seen, launches = {}, {}
     for mask in (7, 5):
         gpu = random_decoder(torch, cfg, 5, 160)
         gpu.set_option(B.OPT_CLUSTER_EPILOGUE, mask)
         gpu.prefill(prompt)
+        before = gpu.query(B.Q_KERNEL_LAUNCHES)
         out = [gpu.step() for _ in range(2)]
+        launches[mask] = gpu.query(B.Q_KERNEL_LAUNCHES) - before
         seen[mask] = [np.concatenate([np.append(t[0, :n[0]], n[0]) for t, n in out]), gpu.debug(B.DBG_HIDDEN), gpu.debug(B.DBG_LOGITS), *gpu.read_kv(0, 1, 0, 90 + T)]
         gpu.close()
+    assert launches[5] - launches[7] == (0 if ffn == 2304 else 2 * 2)         # a kernel less in each layer of both steps: the two paths are two
     assert np.isfinite(seen[7][1]).all() and np.abs(seen[7][1]).max() > 0.1
     for a, b in zip(seen[7], seen[5]):
         assert a.tobytes() == b.tobytes()
@@ -155,15 +158,18 @@ def test_two_chunks_at_once(torch, d, heads, kv, hd, ffn, n):
     cfg = get_config("c0", name="two", n_layers=3, d_model=d, n_heads=heads, n_kv_heads=kv, head_dim=hd, d_ffn=ffn, vocab=1000, dtype="bf16", rope_base=1e6,
                      n_medusa=4, topk=(10, 4, 2, 2), tree_nodes=20)
     prompt = np.random.default_rng(n).integers(0, 1000, n).astype(np.int32)
-    seen = {}
+    seen, launches = {}, {}
     for wide in (1, 0):
         gpu = random_decoder(torch, cfg, 5, n + 40)
         gpu.set_option(B.OPT_WIDE_GEMM, wide)
+        before = gpu.query(B.Q_KERNEL_LAUNCHES)
         gpu.prefill(prompt)
+        launches[wide] = gpu.query(B.Q_KERNEL_LAUNCHES) - before
         seen[wide] = [gpu.debug(B.DBG_NEXT_ROOT), gpu.debug(B.DBG_H_LAST)] + [a for l in range(3) for a in gpu.read_kv(0, l, 0, n)]
         for t, c in (gpu.step() for _ in range(2)):
             seen[wide].append(np.append(t[0, :c[0]], c[0]))
         gpu.close()
+    assert launches[1] == launches[0] if ffn == 704 else launches[1] < 0.7 * launches[0]      # (one pass over the layers, not two)
     assert np.isfinite(seen[1][1]).all() and np.abs(seen[1][1]).max() > 0.1
     for a, b in zip(seen[1], seen[0]):
         assert a.tobytes() == b.tobytes()
