@@ -272,7 +272,7 @@ struct spec_ctx {
   int T, K, kmax, B;                   // tree nodes, heads, candidates per head, current batch
   bool tc;                             // bf16 tensor-core path
   size_t esz;                          // operand element size
-  int Mcap, cap, pages_per_seq, gen_cap, nsplit_attn, Nqkv, n_argmax, topk_slice, topk_blocks;
+  int Mcap, cap, pages_per_seq, gen_cap, nsplit_attn, n_argmax, topk_slice, topk_blocks;
   bool qkv_fused, keep_logits;
   bool packed = false;                 // linear weights are pre-tiled images (SPEC_FLAG_PACKED_WEIGHTS)
   bool pdl = true;                     // programmatic dependent launch between the kernels of a step
@@ -430,6 +430,12 @@ int full_chunk_cap(const spec_ctx* c) {
   return c->tc ? std::max(c->cfg.max_batch, std::min(PREFILL_CHUNKS, max_prompt_chunks(c->cfg))) : c->cfg.max_batch;
 }
 
+// Floats of the row maxima that a float32 projection [M, K] x [N, K] leaves (RowBest), 0 where it leaves none.
+size_t held_best_floats(int M, int N, int K) {
+  const RowLinearShape sh = linear_rows_shape<float>((N + LR_N - 1) / LR_N, M, K);
+  return linear_held(sh, K) ? 2 * (size_t)M * linear_held_shape(sh, M, N).grid.x : 0;
+}
+
 // Lays the workspace out; with base == nullptr only measures it. chunk_cap: prompt chunks of a pass, at least one a sequence;
 // share_tiles: with scratch for the partial sums of gemm_pair's shared tiles even if no other use asks for that much.
 size_t carve(spec_ctx* c, void* base, int chunk_cap, bool share_tiles) {
@@ -437,7 +443,6 @@ size_t carve(spec_ctx* c, void* base, int chunk_cap, bool share_tiles) {
   Bump b(base);
   int B = f.max_batch, T = c->T, K = c->K, d = f.d_model, F = f.d_ffn, V = f.vocab;
   int HD = f.n_heads * f.head_dim;
-  c->Nqkv = HD + 2 * f.n_kv_heads * f.head_dim;
   const int max_chunks = max_prompt_chunks(f);
   c->chunk_cap = chunk_cap;
   // a workspace with less than full room: buffers that are never in use at the same time share their place
@@ -508,10 +513,11 @@ size_t carve(spec_ctx* c, void* base, int chunk_cap, bool share_tiles) {
         if (plan_gemm((int)m, d, 1, r_lm, SM_SLOTS, &g)) pf = std::max(pf, plan_part_floats(g));
         int r_hd[GS_MAX_MATS] = {d, d, d, d};
         if (plan_gemm((int)m, d, GS_MAX_MATS, r_hd, SM_SLOTS, &g)) pf = std::max(pf, plan_part_floats(g));
-      } else {
-        pf = std::max(pf, m * (size_t)c->Nqkv);
       }
     }
+    // (float32: each row's largest out of lm_head, whatever the number of rows)
+    if (f.dtype == 0)
+      for (int m = 1; m <= B * std::max(T, K); ++m) pf = std::max(pf, held_best_floats(m, V, d));
   }
   // (split tiles of the many-row projections leave their partial sums here too)
   if (share_tiles && c->tc && c->Mcap > 128 && std::max(d, std::max(HD, F)) >= 64 * GP_SPLIT_KC) pf = std::max(pf, GP_PART_FLOATS);

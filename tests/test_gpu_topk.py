@@ -24,7 +24,9 @@ def test_candidates(vocab, batch, kmax):
     dec = SpecDecoder(cfg, upload_weights(cfg, w), build_tree(cfg.topk, kmax + 1), 64, max_batch=batch)
     dec.prefill([draw_prompt(cfg.with_(seed=30 + b), 5 + b) for b in range(batch)])
     h = torch.from_numpy(dec.debug(B.DBG_H_LAST)).bfloat16().double()
+    dec.set_option(B.OPT_TRACE, 1)
     dec.step()
+    assert (("topk_tiles" if vocab > 1000 else "topk_slices_tc") in [r[0] for r in dec.trace()])
     cand = dec.debug(B.DBG_CAND)
     assert dec.kmax == kmax
     dec.close()
@@ -62,7 +64,9 @@ def test_candidates_float32(vocab, batch, kmax, classes):
     dec = SpecDecoder(cfg, upload_weights(cfg, w), build_tree(cfg.topk, kmax + 1), 64, max_batch=batch)
     dec.prefill([draw_prompt(cfg.with_(seed=30 + b), 5 + b) for b in range(batch)])
     h = torch.from_numpy(dec.debug(B.DBG_H_LAST)).double()
+    dec.set_option(B.OPT_TRACE, 1)
     dec.step()
+    assert "topk_tiles" in [r[0] for r in dec.trace()]
     cand = dec.debug(B.DBG_CAND)
     dec.close()
 
@@ -82,3 +86,21 @@ def test_candidates_float32(vocab, batch, kmax, classes):
         picked = z[b][got]
         assert (np.diff(picked) <= tol).all()
         assert np.delete(z[b], got).max() <= picked[-1] + tol
+
+
+@pytest.mark.parametrize("heads,hd,T,batch", [(1, 32, 20, 1), (1, 32, 29, 3), (4, 64, 16, 2)])
+def test_row_maxima_have_room(heads, hd, T, batch):
+    """The float32 argmax reads the row maxima that lm_head leaves, whatever the width of the queries."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2503_14153_b200 import SpecDecoder, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    cfg = get_config("c0", name="room", vocab=32016, d_ffn=704, n_heads=heads, n_kv_heads=heads, head_dim=hd, topk=(4, 2, 2), tree_nodes=T, seed=7)
+    dec = SpecDecoder(cfg, upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, T), 64, max_batch=batch)
+    dec.prefill([draw_prompt(cfg.with_(seed=30 + b), 5 + b) for b in range(batch)])
+    dec.set_option(B.OPT_TRACE, 1)
+    dec.step()
+    ran = [r[0] for r in dec.trace()]
+    dec.close()
+    assert "topk_tiles" in ran and "argmax_tiles" in ran and "argmax_partials_tc" not in ran
