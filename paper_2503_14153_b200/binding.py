@@ -324,8 +324,9 @@ class SpecDecoder:
         toks = np.ascontiguousarray(np.concatenate([np.asarray(p, dtype=np.int32) for p in prompts]))
         offs = np.zeros(len(prompts) + 1, dtype=np.int32)
         offs[1:] = np.cumsum([len(p) for p in prompts])
-        self.batch = len(prompts)
-        self._check(self.lib.spec_prefill(self._ctx, self.batch, toks.ctypes.data, offs.ctypes.data))
+        rc = self.lib.spec_prefill(self._ctx, len(prompts), toks.ctypes.data, offs.ctypes.data)
+        self.batch = self.query(Q_BATCH)                     # (prompts that are refused leave the sequences as they were)
+        self._check(rc)
 
     def step(self, cand_override: Optional[np.ndarray] = None):
         """One synchronous step; returns (tokens [batch][K+1] int32, counts [batch])."""

@@ -106,3 +106,26 @@ def test_failed_prompt_waits_for_its_copies():
     assert dec.lib.spec_prefill(dec._ctx, 1, tokens.data_ptr(), offsets.ctypes.data) != 0
     assert dec.stream.query()
     dec.close()
+
+
+def test_refused_prompts_leave_the_batch():
+    """More prompts than the decoder has room for, or a prompt that is too long, are refused: steps and debug reads go on with the sequences that were there."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2503_14153_b200 import SpecDecoder, SpecError, build_tree, upload_weights
+    from paper_2503_14153_b200 import binding as B
+    from synthetic import draw_weights
+    cfg = get_config("c0", name="setup", n_layers=1, d_model=256, n_heads=4, n_kv_heads=2, head_dim=64, d_ffn=704, vocab=1000, n_medusa=3, topk=(4, 2, 2),
+                     tree_nodes=9, seed=3)
+    dec = SpecDecoder(cfg, upload_weights(cfg, draw_weights(cfg)), build_tree(cfg.topk, 9), 100, max_batch=3)
+    prompts = [np.arange(20 + b, dtype=np.int32) for b in range(2)]
+    dec.prefill(prompts)
+    first = dec.debug(B.DBG_H_LAST)
+    for refused in ([prompts[0]] * 4, [np.zeros(100, np.int32)] * 3):
+        with pytest.raises(SpecError):
+            dec.prefill(refused)
+        assert np.array_equal(dec.debug(B.DBG_H_LAST), first)
+        tokens, counts = dec.step() if len(refused) == 3 else (first, first)
+        assert len(tokens) == len(counts) == 2
+    dec.close()
