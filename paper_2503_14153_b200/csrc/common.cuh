@@ -148,9 +148,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
   return true;
 }
 
-// True in one lane of a converged warp. A branch on this, unlike one on the lane's number, tells the compiler that a single thread goes on,
-// which the instructions that take their descriptors and barriers from uniform registers (tcgen05.mma, tcgen05.commit, TMA) need: issuing the
-// four MMAs of a 64-wide K chunk behind a completed barrier, with their commit, takes 250 cycles instead of 500 (the MMAs alone: 170 at N = 16, 256 at N = 128).
+// True in one lane of a converged warp. Timed with clock stamps: the four MMAs of a 64-wide K chunk behind a completed barrier, with their commit, take
+// 250 cycles to issue behind a branch on this and 500 behind one on the lane's number (the MMAs alone: 170 at N = 16, 256 at N = 128).
 __device__ __forceinline__ bool elect_one() {
   uint32_t r;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(r));

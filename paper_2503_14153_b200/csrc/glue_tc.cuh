@@ -413,7 +413,7 @@ rope_store_tc(const PartView pv, int qp0, int kp0, int vp0, Rows rows, const flo
 // act[m][f] = bf16(SiLU(gate) * up), gate / up = sums of the partial slots of the gate and up
 // matrices (padded columns gp0 + f and up0 + f). F % 4 == 0. Bound by L2. ROWS = SWIGLU_ROWS, where no tile has more than two slots (7B shape): a
 // thread has four columns of that many rows, fetches all their slots before it uses the first and finds the tile's slots, which takes
-// divisions, once; 128 rows of 2 x 11008 take 6.0 us behind the projection (12.3 with an item a thread after the other). ROWS = 1: more slots.
+// divisions, once; 128 rows of 2 x 11008 take 5.3 us behind the projection (12.5 with an item a thread after the other). ROWS = 1: more slots.
 constexpr int SWIGLU_ROWS = 4;                               // (divides the activation tiles of the streamer)
 template <int ROWS>
 __global__ void __launch_bounds__(256)

@@ -659,8 +659,8 @@ float pair_cost(int tiles, int rows, int cut, int KC, int clusters, float epilog
 // clusters. Otherwise the tile height that pair_cost likes best: 256 rows, less where that fills the last wave better or brings more
 // clusters to work on a narrow projection, or 256 with the last wave's tiles cut. The choice moves no sum: every element's inner dimension
 // runs through as before. 7B shape: q/k/v of 2048 rows 141 -> 127 us (last wave in quarters), output and down projections of 1536 rows 50 -> 40 and
-// 124 -> 95 (176 rows); d_model 1024, 896 rows: 16.6 -> 10.8, 11.6 -> 7.5, gate+up 21.3 -> 16.6, down 18.9 -> 12.3; the last row of a prompt through
-// a 7B layer 166 -> 117 (16 rows, a ring of eleven stages).
+// 124 -> 95 (176 rows). Inside a step, from the end of the kernel before: d_model 1024, 896 rows 16.2 -> 10.4, 12.1 -> 8.5, gate+up 21.5 -> 17.1, down
+// 20.2 -> 13.3; from the output to the down projection of a prompt's last row on the 7B shape 149 -> 97 (16 rows, a ring of eleven stages).
 void plan_pair(PairGemmParams* p, int mode, bool may_share, int max_clusters = GP_MAX_CLUSTERS) {
   const int clusters = std::min(GP_MAX_CLUSTERS, max_clusters), tall = p->w_pairs * ((p->M + GP_NT - 1) / GP_NT);
   p->tile_rows = GP_NT; p->cut = 1;
@@ -2523,10 +2523,11 @@ int op_linear_bf16(const void* x, const void* w, float* y, int M, int N, int K, 
   OpStatus status(reinterpret_cast<int*>(scratch + scratch_floats), pinned, st);
   if (!status.ok()) return SPEC_E_CUDA;
   if (M > 128 && (long long)g.p.n_tiles * g.p.seg.m_tiles >= 2LL * g.grid) {
-    // many rows: whole tiles on pairs of SMs, finished sums straight into y (at M = 1008, N = 11008, K = 4096 the call takes
-    // 106 us; with weight streaming, which fetches the weights once per 128 rows, 127 us, and adds up partial sums, 34, it took 204)
-    // With fewer than two tiles a CTA the streaming kernel is as fast (67 us against 65 in one case) and closer to the exact
-    // result, since it cuts the inner dimension into several separately rounded sums where this kernel adds two.
+    // many rows: whole tiles on pairs of SMs, finished sums straight into y (M = 1008, N = 11008, K = 4096: 94 us a call; weight streaming fetches the
+    // weights once per 128 rows and adds up partial sums: 204). With few tiles a CTA the streaming kernel is closer to the exact result, since it cuts
+    // the inner dimension into more separately rounded sums than the two that this kernel adds: 256 x 4096 x 4096 (0.2 tiles a CTA) 8.1e-7 off
+    // 64-bit products against 2.1e-6, 52 us against 47. The line was drawn at two tiles a CTA when the kernel had one tile height; with the heights it
+    // has, it is the more exact one from about 0.7 on (512 x 11008 x 4096, 1.2 a CTA: 3.3e-6 and 117 us here, 2.1e-6 and 66 there).
     PairGemmParams p{};
     PairTmaps pm{};
     p.M = M; p.KC = K / 64; p.n_mats = 1;
